@@ -390,14 +390,15 @@ struct TcGemm {
   int passes;            // 1 or 3 tf32 passes on fp32 operands; 0: A and B are 16-bit arrays (one kind::f16 pass);
                          // 6: 16-bit high and low parts, three kind::f16 passes
   int fp16;              // passes 0 / 6: the 16-bit type is fp16 (1) or bf16 (0)
+  int mn_major;          // passes 0: A and B are [K][M] and [K][N] arrays (lda, ldb: distance of two k)
   const float* row_scale; const float* col_scale;   // both or neither: C = acc * row_scale[m] * col_scale[n]
   int64_t k_segment;     // K extent accumulated in tensor memory before it is folded into C (0: all of K)
   int accumulate;        // C += (read-modify-write) instead of C =
   int symmetric_lower;   // only the lower triangle (tiles with n0 <= m0, elements with column <= row) is computed (M == N)
   const float* d1; const float* d2;  // optional dot operands (ld = ldc)
-  double* part1; double* part2;      // [tiles] partial sums
+  double* part1; double* part2;      // partial sums, launch_tc_gemm says how many
 };
-armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_tiles, cudaStream_t s);
+armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStream_t s);
 bool tc_gemm_shape_ok(int64_t M, int64_t N, int64_t K);
 // the 2:4 core on the sparse tensor cores (sparse_tcgen05.cu)
 bool tc_sparse_ok(const armor_ctx* c);

@@ -68,11 +68,11 @@ armor_status rmul_H(armor_ctx* c, const float* in, const float* H, float* out, i
     g.k_segment = (g.passes >= 3) ? K_SEGMENT : 0;   // one-pass tf32 rounding (2^-11) dwarfs the accumulator drift
     g.part1 = d1 ? c->partials : nullptr;
     g.part2 = d2 ? c->partials + 8 * c->npart : nullptr;
-    int tiles = 0;
-    armor_status st = launch_tc_gemm(c, g, &tiles, s);
+    int n_part = 0;
+    armor_status st = launch_tc_gemm(c, g, &n_part, s);
     if (st != ARMOR_OK) return st;
-    if (d1) reduce_partials_to(c, c->partials, 8 * tiles, out1, s);
-    if (d2) reduce_partials_to(c, c->partials + 8 * c->npart, 8 * tiles, out2, s);
+    if (d1) reduce_partials_to(c, c->partials, n_part, out1, s);
+    if (d2) reduce_partials_to(c, c->partials + 8 * c->npart, n_part, out2, s);
     return ARMOR_OK;
   }
   if (d1) dot_to_ptr(c, out, d1, rows * d_in, out1, s);
@@ -99,6 +99,27 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
       g.M = (int)d_in; g.N = (int)d_in; g.K = (int)n; g.batch = 1; g.alpha = 1.f; g.beta = 1.f;
       launch_bgemm(c, g, s);
     }
+    return ARMOR_OK;
+  }
+  if (bf16 && ldx % 8 == 0 && reinterpret_cast<uintptr_t>(Xv) % 16 == 0 && d_in % 32 == 0) {
+    // bf16 activations go to the tensor cores as they lie in memory: X is an operand of X^T X that is contiguous along
+    // the channels, products of two bf16 values are exact in fp32, so nothing is scaled, transposed or staged.  (A
+    // leading dimension or base that TMA does not take leaves the staged path below.)
+    // One launch per gram_rows tokens, as in the staged path: a long call sums like a sequence of shorter ones.
+    for (int64_t r0 = 0; r0 < n_rows; r0 += c->gram_rows) {
+      TcGemm g{};
+      g.A = static_cast<const char*>(Xv) + (size_t)(r0 * ldx) * 2; g.lda = ldx;
+      g.B = g.A; g.ldb = ldx;
+      g.C = H; g.ldc = d_in;
+      g.M = d_in; g.N = d_in; g.K = n_rows - r0 < c->gram_rows ? n_rows - r0 : c->gram_rows;
+      g.passes = 0; g.mn_major = 1;
+      g.accumulate = 1;
+      g.symmetric_lower = 1;
+      g.k_segment = K_SEGMENT;
+      const armor_status st = launch_tc_gemm(c, g, nullptr, s);
+      if (st != ARMOR_OK) return st;
+    }
+    launch_mirror_lower(c, H, d_in, s);
     return ARMOR_OK;
   }
   if (c->cfg.precision == ARMOR_PREC_FP16X3) {

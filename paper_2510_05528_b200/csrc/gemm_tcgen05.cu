@@ -4,13 +4,18 @@
 // paper; both operands are the transposed, staged chunk of X) and the right-multiplications by the
 // symmetric Gram, E.H, T.H and V.H (H[n][k] = H[k][n], so H itself is the K-major B operand).
 //
-// Design: persistent kernel, one CTA per SM, 192 threads:
-//   warp 0   : TMA producer  (cp.async.bulk.tensor.2d, 128-byte swizzle, mbarrier complete_tx)
-//   warp 1   : MMA issuer    (one thread issues tcgen05.mma kind::tf32, 128 x 256 x 8 per instruction,
-//                             accumulators in tensor memory, two accumulator buffers of 256 columns)
+// Design: persistent kernel on pairs of CTAs (cluster of two, cta_group::2), a 256 x 256 tile of C per pair:
+//   warp 0   : TMA producer  (cp.async.bulk.tensor.2d, 128-byte swizzle; each CTA loads its 128 rows of A and its
+//                             128 rows of B and signals the even CTA's barrier)
+//   warp 1   : MMA issuer    (one thread of the even CTA issues tcgen05.mma.cta_group::2, 256 x 256 x 16 (x 8 for
+//                             tf32); every SM holds its own 128 rows of the accumulator in tensor memory, two
+//                             accumulator buffers of 256 columns)
 //   warps 2-9: epilogue      (tcgen05.ld 32 lanes x 32 columns; the K segments of a tile are summed in registers,
 //                             then one fused C-update / dot products; a symmetric product writes its lower
 //                             triangle only, the caller mirrors it once at the end)
+// Why pairs: per 64 columns of K one SM fetches 32 KB (64 KB with split operands) for its 128 x 256 outputs, where a
+// CTA of its own fetches 48 KB (96 KB).  With one MMA per product the single CTA was bound by what L2 delivers
+// (8.7 TB/s into shared memory at 720 TFLOP/s), not by the tensor pipe.
 // passes == 3: every operand is given as a tf32-exact high part and an fp32 low part; the three products
 // hi*hi, lo*hi, hi*lo are accumulated into the same fp32 accumulator (error-compensated tf32, fp32-grade).
 // passes == 6: the same three products on fp16 high and low parts (kind::f16, twice the tf32 issue rate, half
@@ -26,30 +31,41 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BN = 256, BK = 32;          // BK fp32 = 128 bytes = one swizzle row
+constexpr int BMP = 256, BM = 128, BN = 256, BK = 32;   // pair tile rows, rows per CTA, columns; BK fp32 = 128 bytes
+constexpr int BNH = BN / 2;                         // rows of B each CTA of the pair holds
 constexpr int NTHREADS = 320;                       // TMA warp, MMA warp, eight epilogue warps
-constexpr int RB = 8;                               // rows of C an epilogue lane keeps in flight
 constexpr int EPI_COLS = 128;                       // accumulator columns per epilogue warp
-constexpr int TB_LD = 17;                           // padded row length of an epilogue warp's 32 x 16 staging tile
+constexpr int EPI_BYTES = 32 * 32 * 4;              // an epilogue warp's 32 x 32 staging tile
 constexpr uint32_t TMEM_COLS = 512;                 // two accumulator buffers of BN columns
 constexpr int A_BYTES = BM * BK * 4;                // 16 KiB
-constexpr int B_BYTES = BN * BK * 4;                // 32 KiB
+constexpr int B_BYTES = BNH * BK * 4;               // 16 KiB
+constexpr int MN_BOX = 64 * 64 * 2;                 // 64 k x 64 rows of a 16-bit operand that is contiguous along M / N
+
+// stages of the shared-memory ring: 3 x 64 KiB with split operands, 6 x 32 KiB otherwise
+template <int PASSES>
+struct Ring {
+  static constexpr int BYTES = (PASSES == 3 || PASSES == 6 ? 2 : 1) * (A_BYTES + B_BYTES);
+  static constexpr int STAGES = PASSES == 3 || PASSES == 6 ? 3 : 6;
+};
+
+constexpr int PARTS = 16;                           // partial dot products per tile: one per epilogue warp of the pair
 
 struct Params {
   float* C; int64_t ldc;
   int64_t M, N, K;
   int m_tiles, n_tiles, n_tiles_total;
   int accumulate, symmetric_lower;
+  int c_vec;             // rows of C start on 16-byte boundaries
   int kt_seg;            // k-tiles accumulated in tensor memory before the epilogue folds them into C
   const float* d1; const float* d2;
   double* part1; double* part2;
   const float* row_scale; const float* col_scale;   // optional powers of two the accumulator is multiplied by
   int f16;               // 16-bit operands are fp16 (1) or bf16 (0)
   int32_t* status;
-  // Tail split: tiles [split_first, n_tiles_total) are cut into split_parts pieces along K, each piece a work
-  // item of its own that writes a 128 x 256 slab of partial sums; a second kernel adds the slabs.  This fills
-  // the last, partly empty wave of tiles.
-  int split_first, split_parts, n_items;
+  // Tail split: tiles [split_first, n_tiles_total) are cut into split_parts pieces of split_kt k-tiles (the last one
+  // may be shorter), each piece a work item of its own that writes a 256 x 256 slab of partial sums; a second kernel
+  // adds the slabs.  This fills the last, partly empty wave of tiles.
+  int split_first, split_parts, split_kt, n_items;
   float* slabs;
 };
 
@@ -64,34 +80,48 @@ __device__ __forceinline__ uint64_t smem_desc_k_sw128(uint32_t addr) {
   return d;
 }
 
-// tcgen05.mma with the accumulate flag set (the constant predicate costs no instruction)
+// The other form of a 16-bit operand: contiguous along M / N (a row-major X is such an operand of X^T X).  A k-row
+// holds 64 elements (128 bytes), groups of 8 k-rows are 1024 bytes apart, the next 64 elements one box further.
+__device__ __forceinline__ uint64_t smem_desc_mn_sw128(uint32_t addr) { return smem_desc_sw128(addr, MN_BOX, 1024); }
+
+// tcgen05.mma of the pair; ACC: the accumulate flag is a constant, which costs no instruction
 template <bool F16>
 __device__ __forceinline__ void umma_acc(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
   if (F16)
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
   else
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
+                 "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc) : "memory");
+}
+template <bool F16>
+__device__ __forceinline__ void umma_first(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
+  if (F16)
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
+  else
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::2.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(acc) : "memory");
 }
 
-// fp32 accumulate, both operands K-major, M = 128, N = 256; operand format 0: fp16, 1: bf16 (both kind::f16),
-// 2: tf32 (kind::tf32).
-__device__ __forceinline__ uint32_t instr_desc(uint32_t fmt) {
+// fp32 accumulate, M = 256 (the pair), N = 256; operand format 0: fp16, 1: bf16 (both kind::f16), 2: tf32
+// (kind::tf32); mn: both operands are contiguous along M / N instead of K.
+__device__ __forceinline__ uint32_t instr_desc(uint32_t fmt, uint32_t mn) {
   uint32_t d = 0;
   d |= 1u << 4;                   // D format: F32
   d |= fmt << 7;                  // A format
   d |= fmt << 10;                 // B format
+  d |= mn << 15;
+  d |= mn << 16;
   d |= (uint32_t)(BN >> 3) << 17; // N
-  d |= (uint32_t)(BM >> 4) << 24; // M
+  d |= (uint32_t)(BMP >> 4) << 24; // M
   return d;
 }
 
-// tile index -> (m tile, n tile).  Groups of GROUP_M m tiles; inside a group m runs fastest, then n: the 148 tiles
-// in flight are about 16 x 9, which minimises what a wave reads (16 A panels + 9 B panels, a B panel being twice
-// an A panel) -- with m running over all m tiles every wave read up to 148 A panels, and on the large shapes
-// (operands far beyond L2) the product became DRAM-bound.
-constexpr int GROUP_M = 16;
+// tile index -> (m tile, n tile).  Groups of GROUP_M m tiles; inside a group m runs fastest, then n: the 74 tiles
+// in flight are about 8 x 9, which minimises what a wave reads -- with m running over all m tiles every wave read up
+// to 74 A panels, and on the large shapes (operands far beyond L2) the product became DRAM-bound.
+constexpr int GROUP_M = 8;
 __device__ __forceinline__ void tile_coords(const Params& p, int tile, int& mt, int& nt) {
   if (!p.symmetric_lower) {
     const int per_group = GROUP_M * p.n_tiles;
@@ -101,13 +131,13 @@ __device__ __forceinline__ void tile_coords(const Params& p, int tile, int& mt, 
     nt = r / gm;
     return;
   }
-  // only tiles that hold an element with column <= row: m tile >= 2 * n tile.  Same grouping: bands of GROUP_M
+  // only tiles that hold an element with column <= row: m tile >= n tile.  Same grouping: bands of GROUP_M
   // m tiles, inside a band the n tile is the outer index and m runs fastest
   int rem = tile;
   for (int m0 = 0; m0 < p.m_tiles; m0 += GROUP_M) {
     const int m1 = min(m0 + GROUP_M, p.m_tiles);
-    for (nt = 0; 2 * nt < m1 && nt < p.n_tiles; ++nt) {
-      const int lo = max(m0, 2 * nt);
+    for (nt = 0; nt < m1 && nt < p.n_tiles; ++nt) {
+      const int lo = max(m0, nt);
       const int cnt = m1 - lo;
       if (rem < cnt) { mt = lo + rem; return; }
       rem -= cnt;
@@ -125,57 +155,71 @@ __device__ __forceinline__ void item_decode(const Params& p, int item, int kt_to
     const int idx = item - p.split_first;
     tile = p.split_first + idx / p.split_parts;
     part = idx % p.split_parts;
-    const int per = kt_total / p.split_parts;
-    kt_begin = part * per; kt_end = kt_begin + per;
+    kt_begin = part * p.split_kt; kt_end = min(kt_total, kt_begin + p.split_kt);
   }
 }
 
-// One epilogue warp's 32 rows x 128 columns of finished sums (lane = row) go out through shared memory, 16
-// columns at a time, so that every store instruction writes two rows of 64 contiguous bytes.  Optional:
-// power-of-two scales, C += (read-modify-write), lower triangle only, partial dot products with d1 / d2.
-__device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float* tilebuf, int lane, float* C, int64_t ldc,
+// four floats of C: one access where every row of C starts on a 16-byte boundary (vec)
+__device__ __forceinline__ float4 load4(const float* q, int vec) {
+  return vec ? *reinterpret_cast<const float4*>(q) : make_float4(q[0], q[1], q[2], q[3]);
+}
+__device__ __forceinline__ void store4(float* q, const float4& v, int vec) {
+  if (vec) { *reinterpret_cast<float4*>(q) = v; return; }
+  q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
+}
+
+// One epilogue warp's 32 rows x 128 columns of finished sums (lane = row) go out through a 32 x 32 staging tile in
+// shared memory (16-byte units, swizzled by the row: no bank conflicts either way), so that every access to C writes or
+// reads four rows of 128 contiguous bytes.  Optional: power-of-two scales, C += (read-modify-write), chunks of 32 x 32
+// above the diagonal left out, partial dot products with d1 / d2.
+__device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* stg, int lane, float* C, int64_t ldc, int vec,
                                           int64_t row_base, int64_t col_base, int64_t M, int64_t N, bool accum, bool sym,
                                           const float* rs, const float* cs, const float* d1, const float* d2, int64_t ldd,
                                           double& dot1, double& dot2) {
   if (row_base >= M) return;                                  // warp-uniform
-  const int rr = lane >> 4, cc = lane & 15;
+  const int rr = lane >> 3, cc = lane & 7;
+  const float rscale = (rs && row_base + lane < M) ? rs[row_base + lane] : 1.f;
 #pragma unroll
-  for (int c16 = 0; c16 < EPI_COLS / 16; ++c16) {
-    const int64_t col0 = col_base + c16 * 16;
+  for (int ch = 0; ch < EPI_COLS / 32; ++ch) {
+    const int64_t col0 = col_base + ch * 32;
     if (col0 >= N) continue;                                   // warp-uniform (N is a multiple of 32)
     if (sym && col0 > row_base + 31) continue;                 // chunk lies above the diagonal
 #pragma unroll
-    for (int i = 0; i < 16; ++i) tilebuf[lane * TB_LD + i] = acc[c16 * 16 + i];
+    for (int j = 0; j < 8; ++j)
+      stg[lane * 8 + (j ^ (lane & 7))] = make_float4(acc[ch * 32 + 4 * j] * rscale, acc[ch * 32 + 4 * j + 1] * rscale,
+                                                     acc[ch * 32 + 4 * j + 2] * rscale, acc[ch * 32 + 4 * j + 3] * rscale);
     __syncwarp();
-    const int64_t col = col0 + cc;
-    const float cscale = cs ? cs[col] : 1.f;
+    const int64_t col = col0 + 4 * cc;
+    const float4 sc4 = cs ? *reinterpret_cast<const float4*>(cs + col) : make_float4(1.f, 1.f, 1.f, 1.f);
     float f1 = 0.f, f2 = 0.f;
-#pragma unroll 1
-    for (int r0 = 0; r0 < 32; r0 += 2 * RB) {
-      float x[RB], o[RB];
-      bool keep[RB];
 #pragma unroll
-      for (int j = 0; j < RB; ++j) {
-        const int r = r0 + 2 * j + rr;
+    for (int h = 0; h < 2; ++h) {
+      float4 o[4];
+      if (accum) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int64_t grow = row_base + 16 * h + 4 * i + rr;
+          o[i] = grow < M ? load4(C + grow * ldc + col, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = 16 * h + 4 * i + rr;
         const int64_t grow = row_base + r;
-        keep[j] = grow < M && (!sym || col <= grow);
-        x[j] = tilebuf[r * TB_LD + cc];
-        if (rs) x[j] *= (grow < M ? rs[grow] : 1.f) * cscale;
-        o[j] = (accum && keep[j]) ? C[grow * ldc + col] : 0.f;
+        if (grow >= M) continue;
+        float4 x = stg[r * 8 + (cc ^ (r & 7))];
+        x.x *= sc4.x; x.y *= sc4.y; x.z *= sc4.z; x.w *= sc4.w;
+        if (accum) { x.x += o[i].x; x.y += o[i].y; x.z += o[i].z; x.w += o[i].w; }
+        if (d1) {
+          const float4 w = *reinterpret_cast<const float4*>(d1 + grow * ldd + col);
+          f1 += x.x * w.x + x.y * w.y + x.z * w.z + x.w * w.w;
+        }
+        if (d2) {
+          const float4 w = *reinterpret_cast<const float4*>(d2 + grow * ldd + col);
+          f2 += x.x * w.x + x.y * w.y + x.z * w.z + x.w * w.w;
+        }
+        store4(C + grow * ldc + col, x, vec);
       }
-      if (d1) {
-#pragma unroll
-        for (int j = 0; j < RB; ++j)
-          if (keep[j]) f1 = fmaf(x[j] + o[j], d1[(row_base + r0 + 2 * j + rr) * ldd + col], f1);
-      }
-      if (d2) {
-#pragma unroll
-        for (int j = 0; j < RB; ++j)
-          if (keep[j]) f2 = fmaf(x[j] + o[j], d2[(row_base + r0 + 2 * j + rr) * ldd + col], f2);
-      }
-#pragma unroll
-      for (int j = 0; j < RB; ++j)
-        if (keep[j]) C[(row_base + r0 + 2 * j + rr) * ldc + col] = x[j] + o[j];
     }
     dot1 += (double)f1;
     dot2 += (double)f2;
@@ -183,14 +227,15 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float* t
   }
 }
 
-template <int PASSES>
+// MN: both operands are 16-bit arrays contiguous along M / N (PASSES 0 only)
+template <int PASSES, bool MN>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapAlo,
                const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo, const Params p) {
   constexpr bool SPLIT = (PASSES == 3 || PASSES == 6);   // operands come as high and low parts
   constexpr bool H16 = (PASSES == 0 || PASSES == 6);     // 16-bit operands (kind::f16)
-  constexpr int STAGE_BYTES = (SPLIT ? 2 : 1) * (A_BYTES + B_BYTES);
-  constexpr int STAGES = SPLIT ? 2 : 4;
+  constexpr int STAGE_BYTES = Ring<PASSES>::BYTES;
+  constexpr int STAGES = Ring<PASSES>::STAGES;
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte alignment for the swizzled tiles
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -199,72 +244,85 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = smem_u32(&bars[2 * STAGES + 2]);
   constexpr int BKE = H16 ? 64 : 32;                // elements of K per 128-byte row: 16-bit or fp32
   const int kt_total = (int)((p.K + BKE - 1) / BKE);
 
+  // full, empty of the stages; tfull, tempty of the accumulator buffers.  full and tempty are used in the even CTA
+  // only (both CTAs' loads and epilogue warps signal it there), empty and tfull in both (commits reach the pair).
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 8); }
+    for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 16); }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
                  "r"(TMEM_COLS)
                  : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();                                  // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
   if (warp == 0) {
-    // ------------------------------------------------------------ TMA producer
+    // ------------------------------------------------------------ TMA producer (both CTAs)
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0; long long issued = 0;
       bool ok = true;
-      for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+      for (int item = pair; item < p.n_items && ok; item += n_pairs) {
         int tile, part, kt_begin, kt_end, mt, nt;
         item_decode(p, item, kt_total, tile, part, kt_begin, kt_end);
         tile_coords(p, tile, mt, nt);
+        const int arow = mt * BMP + (int)rank * BM, brow = nt * BN + (int)rank * BNH;
         for (int kt = kt_begin; kt < kt_end; ++kt) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
-          const uint32_t fb = full0 + 8 * stage;
-          mbar_expect_tx(fb, STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * STAGE_BYTES);
+          const uint32_t fb = map_to_cta(full0 + 8 * stage, 0);
           uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          tma_load_2d(dst, &mapA, kt * BKE, mt * BM, fb);
-          dst += A_BYTES;
-          if (SPLIT) { tma_load_2d(dst, &mapAlo, kt * BKE, mt * BM, fb); dst += A_BYTES; }
-          tma_load_2d(dst, &mapB, kt * BKE, nt * BN, fb);
-          dst += B_BYTES;
-          if (SPLIT) tma_load_2d(dst, &mapBlo, kt * BKE, nt * BN, fb);
+          if (MN) {
+            // x = row of the operand (a channel), y = k (a token); rows and k beyond the operand are zero-filled
+            tma_load_2d_pair(dst, &mapA, arow, kt * BKE, fb);
+            tma_load_2d_pair(dst + MN_BOX, &mapA, arow + 64, kt * BKE, fb);
+            tma_load_2d_pair(dst + A_BYTES, &mapB, brow, kt * BKE, fb);
+            tma_load_2d_pair(dst + A_BYTES + MN_BOX, &mapB, brow + 64, kt * BKE, fb);
+          } else {
+            tma_load_2d_pair(dst, &mapA, kt * BKE, arow, fb);
+            dst += A_BYTES;
+            if (SPLIT) { tma_load_2d_pair(dst, &mapAlo, kt * BKE, arow, fb); dst += A_BYTES; }
+            tma_load_2d_pair(dst, &mapB, kt * BKE, brow, fb);
+            dst += B_BYTES;
+            if (SPLIT) tma_load_2d_pair(dst, &mapBlo, kt * BKE, brow, fb);
+          }
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
-      if (!ok) {
-        // leave no bulk copy in flight: wait (bounded) for the stages armed most recently
-        for (int back = 1; back <= STAGES && back <= issued; ++back) {
-          int s = stage - back; uint32_t ph = phase;
-          if (s < 0) { s += STAGES; ph ^= 1; }
-          const long long t0 = clock64();
-          while (!mbar_try(full0 + 8 * s, ph) && clock64() - t0 < 20000000ll) {}
-        }
+      // tail: the MMAs that read the stages issued last have finished (their commits reach both CTAs), so nothing is
+      // in flight towards this CTA's shared memory when it leaves
+      for (int back = 1; back <= STAGES && back <= issued; ++back) {
+        int s = stage - back; uint32_t ph = phase;
+        if (s < 0) { s += STAGES; ph ^= 1; }
+        const long long t0 = clock64();
+        while (!mbar_try(empty0 + 8 * s, ph) && clock64() - t0 < (ok ? WAIT_CYCLES : 20000000ll)) {}
       }
     }
   } else if (warp == 1) {
-    // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
-      const uint32_t idesc = instr_desc(H16 ? (p.f16 ? 0u : 1u) : 2u);
-      const uint64_t d0 = smem_desc_k_sw128(smem_u32(smem));
+    // ------------------------------------------------------------ MMA issuer (even CTA)
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = instr_desc(H16 ? (p.f16 ? 0u : 1u) : 2u, MN ? 1u : 0u);
+      const uint64_t d0 = MN ? smem_desc_mn_sw128(smem_u32(smem)) : smem_desc_k_sw128(smem_u32(smem));
       int stage = 0; uint32_t phase = 0;
       int local = 0;   // (tile, K segment) items handled so far: selects the accumulator buffer
       bool ok = true;
-      for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+      for (int item = pair; item < p.n_items && ok; item += n_pairs) {
         int tile, part, kt_begin, kt_end;
         item_decode(p, item, kt_total, tile, part, kt_begin, kt_end);
         for (int kt0 = kt_begin; kt0 < kt_end && ok; kt0 += p.kt_seg, ++local) {
@@ -285,46 +343,41 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
             const uint64_t dbm = da + (((SPLIT ? 2 : 1) * A_BYTES) >> 4);
             const uint64_t dbl = dbm + (B_BYTES >> 4);
             const uint32_t acc = (uint32_t)(kt > kt0);
-            if (PASSES == 3) {
-              umma_tf32(tacc, dal, dbm, idesc, acc);
-              umma_acc<false>(tacc, da, dbl, idesc);
-              umma_acc<false>(tacc, da, dbm, idesc);
-            } else if (PASSES == 6) {
-              umma_bf16(tacc, dal, dbm, idesc, acc);
-              umma_acc<true>(tacc, da, dbl, idesc);
-              umma_acc<true>(tacc, da, dbm, idesc);
-            } else if (PASSES == 0) {
-              umma_bf16(tacc, da, dbm, idesc, acc);
+            if (SPLIT) {
+              umma_first<H16>(tacc, dal, dbm, idesc, acc);
+              umma_acc<H16>(tacc, da, dbl, idesc);
+              umma_acc<H16>(tacc, da, dbm, idesc);
             } else {
-              umma_tf32(tacc, da, dbm, idesc, acc);
+              umma_first<H16>(tacc, da, dbm, idesc, acc);
             }
 #pragma unroll
             for (int k = 1; k < BK / 8; ++k) {
-              const uint64_t ko = (uint64_t)(k * (32 >> 4));   // 8 fp32 (16 halves) of K: 32 bytes along the row
+              // 8 fp32 (16 halves) of K: 32 bytes along the row, or 16 k-rows of 128 bytes
+              const uint64_t ko = (uint64_t)(MN ? k * (2048 >> 4) : k * (32 >> 4));
               if (SPLIT) {
                 umma_acc<H16>(tacc, dal + ko, dbm + ko, idesc);
                 umma_acc<H16>(tacc, da + ko, dbl + ko, idesc);
               }
               umma_acc<H16>(tacc, da + ko, dbm + ko, idesc);
             }
-            umma_commit(empty0 + 8 * stage);   // frees the stage once these MMAs have read it
+            umma_commit_pair(empty0 + 8 * stage);   // frees the stage in both CTAs once these MMAs have read it
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
           }
-          if (ok) umma_commit(tfull0 + 8 * as);
+          if (ok) umma_commit_pair(tfull0 + 8 * as);
         }
       }
     }
   } else {
-    // ------------------------------------------------------------ epilogue warps
+    // ------------------------------------------------------------ epilogue warps (both CTAs)
     // Eight warps: warp w reads TMEM lanes 32 (w % 4) .. and one half (128 columns) of the accumulator, one
     // row per lane.  The K segments of a tile are summed in registers (ordinary round-to-nearest adds), so the
     // accumulator buffer is handed back right after it has been read and C is touched once per tile.
     const int q = warp & 3;
     const int half = (warp - 2) >> 2;
-    float* tilebuf = reinterpret_cast<float*>(smem + (size_t)STAGES * STAGE_BYTES) + (warp - 2) * (32 * TB_LD);
+    float4* stg = reinterpret_cast<float4*>(smem + (size_t)STAGES * STAGE_BYTES + (size_t)(warp - 2) * EPI_BYTES);
     int local = 0;
     bool ok = true;
-    for (int item = blockIdx.x; item < p.n_items && ok; item += gridDim.x) {
+    for (int item = pair; item < p.n_items && ok; item += n_pairs) {
       int tile, part, kt_begin, kt_end, mt, nt;
       item_decode(p, item, kt_total, tile, part, kt_begin, kt_end);
       tile_coords(p, tile, mt, nt);
@@ -345,55 +398,56 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(tempty0 + 8 * as);
+        if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty0 + 8 * as, 0));
       }
       if (!ok) break;
       if (part >= 0) {
         // a piece of a split tile: its partial sums go, plainly, to this item's slab
-        float* slab = p.slabs + ((int64_t)(tile - p.split_first) * p.split_parts + part) * (BM * BN);
+        float* slab = p.slabs + (((int64_t)(tile - p.split_first) * p.split_parts + part) * 2 + rank) * (BM * BN);
         double u1 = 0.0, u2 = 0.0;
-        write_out(acc, tilebuf, lane, slab, BN, q * 32, half * EPI_COLS, BM, BN, false, false, nullptr, nullptr, nullptr,
+        write_out(acc, stg, lane, slab, BN, 1, q * 32, half * EPI_COLS, BM, BN, false, false, nullptr, nullptr, nullptr,
                   nullptr, 0, u1, u2);
         continue;
       }
       double dot1 = 0.0, dot2 = 0.0;
-      write_out(acc, tilebuf, lane, p.C, p.ldc, (int64_t)mt * BM + q * 32, (int64_t)nt * BN + half * EPI_COLS, p.M, p.N,
-                p.accumulate != 0, p.symmetric_lower != 0, p.row_scale, p.col_scale, p.d1, p.d2, p.ldc, dot1, dot2);
+      write_out(acc, stg, lane, p.C, p.ldc, p.c_vec, (int64_t)mt * BMP + rank * BM + q * 32, (int64_t)nt * BN + half * EPI_COLS, p.M,
+                p.N, p.accumulate != 0, p.symmetric_lower != 0, p.row_scale, p.col_scale, p.d1, p.d2, p.ldc, dot1, dot2);
       if (p.part1 || p.part2) {
         for (int o = 16; o > 0; o >>= 1) {
           dot1 += __shfl_down_sync(0xffffffffu, dot1, o);
           dot2 += __shfl_down_sync(0xffffffffu, dot2, o);
         }
         if (lane == 0) {
-          if (p.part1) p.part1[(int64_t)tile * 8 + half * 4 + q] = dot1;
-          if (p.part2) p.part2[(int64_t)tile * 8 + half * 4 + q] = dot2;
+          if (p.part1) p.part1[(int64_t)tile * PARTS + rank * 8 + half * 4 + q] = dot1;
+          if (p.part2) p.part2[(int64_t)tile * PARTS + rank * 8 + half * 4 + q] = dot2;
         }
       }
     }
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();                                  // neither CTA leaves while its partner may still signal it
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
   }
 }
 
 // Adds the slabs of every split tile into C (+ what C held, if the product accumulates) and forms the tile's
-// share of the fused dot products.  Four CTAs per split tile (32 rows each); fixed order.
+// share of the fused dot products.  Eight CTAs per split tile (32 rows each); fixed order.
 __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
-  const int tile = p.split_first + blockIdx.x / 4, qq = blockIdx.x % 4;
+  const int tile = p.split_first + blockIdx.x / 8, half = (blockIdx.x >> 2) & 1, qq = blockIdx.x % 4;
   int mt, nt;
   tile_coords(p, tile, mt, nt);
-  const float* slab0 = p.slabs + (int64_t)(blockIdx.x / 4) * p.split_parts * (BM * BN);
+  const float* slab0 = p.slabs + ((int64_t)(blockIdx.x / 8) * p.split_parts * 2 + half) * (BM * BN);
   double d1 = 0.0, d2 = 0.0;
   for (int e = threadIdx.x; e < 32 * BN / 4; e += 256) {
     const int r = qq * 32 + e / (BN / 4), c4 = (e % (BN / 4)) * 4;
-    const int64_t grow = (int64_t)mt * BM + r, gcol = (int64_t)nt * BN + c4;
-    if (grow >= p.M || gcol >= p.N) continue;
+    const int64_t grow = (int64_t)mt * BMP + half * BM + r, gcol = (int64_t)nt * BN + c4;
+    if (grow >= p.M || gcol >= p.N || (p.symmetric_lower && gcol > grow)) continue;
     float4 v = *reinterpret_cast<const float4*>(slab0 + (int64_t)r * BN + c4);
     for (int k = 1; k < p.split_parts; ++k) {
-      const float4 w = *reinterpret_cast<const float4*>(slab0 + (int64_t)k * (BM * BN) + (int64_t)r * BN + c4);
+      const float4 w = *reinterpret_cast<const float4*>(slab0 + (int64_t)k * (2 * BM * BN) + (int64_t)r * BN + c4);
       v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
     }
     if (p.row_scale) {
@@ -403,10 +457,10 @@ __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
     }
     float* cp = p.C + grow * p.ldc + gcol;
     if (p.accumulate) {
-      const float4 o = *reinterpret_cast<const float4*>(cp);
+      const float4 o = load4(cp, p.c_vec);
       v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
     }
-    *reinterpret_cast<float4*>(cp) = v;
+    store4(cp, v, p.c_vec);
     if (p.d1) {
       const float4 w = *reinterpret_cast<const float4*>(p.d1 + grow * p.ldc + gcol);
       d1 += (double)(v.x * w.x + v.y * w.y) + (double)(v.z * w.z + v.w * w.w);
@@ -426,21 +480,23 @@ __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
   if (threadIdx.x == 0) {
     double t1 = 0.0, t2 = 0.0;
     for (int w = 0; w < 8; ++w) { t1 += red1[w]; t2 += red2[w]; }
-    // eight slots per tile (the GEMM's eight epilogue warps); this kernel fills four and clears the rest
-    if (p.part1) { p.part1[(int64_t)tile * 8 + qq] = t1; p.part1[(int64_t)tile * 8 + 4 + qq] = 0.0; }
-    if (p.part2) { p.part2[(int64_t)tile * 8 + qq] = t2; p.part2[(int64_t)tile * 8 + 4 + qq] = 0.0; }
+    // sixteen slots per tile (the epilogue warps of the pair); this kernel fills eight and clears the rest
+    const int64_t slot = (int64_t)tile * PARTS + half * 8 + qq;
+    if (p.part1) { p.part1[slot] = t1; p.part1[slot + 4] = 0.0; }
+    if (p.part2) { p.part2[slot] = t2; p.part2[slot + 4] = 0.0; }
   }
 }
 
 // ------------------------------------------------------------------ host side
 // [rows][K] fp32, leading dimension ld: box = BK x box_rows, 128-byte swizzle, zero fill out of bounds.
 // bits16: 0 fp32 elements, 1 bf16, 2 fp16
-bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows, int bits16 = 0) {
+// mn: the array is [K][rows] of 16-bit elements (contiguous along the rows of the operand): box = 64 rows x 64 k
+bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows, int bits16, bool mn) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
   if (!enc) return false;
-  cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
+  cuuint64_t dims[2] = {(cuuint64_t)(mn ? rows : K), (cuuint64_t)(mn ? K : rows)};
   cuuint64_t strides[1] = {(cuuint64_t)ld * (bits16 ? 2 : 4)};
-  cuuint32_t box[2] = {(cuuint32_t)(bits16 ? 64 : BK), (cuuint32_t)box_rows};
+  cuuint32_t box[2] = {(cuuint32_t)(bits16 ? 64 : BK), (cuuint32_t)(mn ? 64 : box_rows)};
   cuuint32_t estr[2] = {1, 1};
   const CUtensorMapDataType dt = bits16 == 0 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
                                  : bits16 == 1 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
@@ -450,51 +506,60 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64
   return r == CUDA_SUCCESS;
 }
 
-template <int PASSES>
+template <int PASSES, bool MN>
 armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s) {
   CUtensorMap mA, mAlo, mB, mBlo;
   constexpr bool SPLIT = (PASSES == 3 || PASSES == 6);
   constexpr bool H16 = (PASSES == 0 || PASSES == 6);
   const int bits16 = H16 ? (g.fp16 ? 2 : 1) : 0;
-  if (!make_map(&mA, g.A, g.M, g.K, g.lda, BM, bits16)) return ARMOR_ERR_CUDA;
-  if (!make_map(&mB, g.B, g.N, g.K, g.ldb, BN, bits16)) return ARMOR_ERR_CUDA;
+  if (!make_map(&mA, g.A, g.M, g.K, g.lda, BM, bits16, MN)) return ARMOR_ERR_CUDA;
+  if (!make_map(&mB, g.B, g.N, g.K, g.ldb, BNH, bits16, MN)) return ARMOR_ERR_CUDA;
   if (SPLIT) {
-    if (!make_map(&mAlo, g.Alo, g.M, g.K, g.lda, BM, bits16)) return ARMOR_ERR_CUDA;
-    if (!make_map(&mBlo, g.Blo, g.N, g.K, g.ldb, BN, bits16)) return ARMOR_ERR_CUDA;
+    if (!make_map(&mAlo, g.Alo, g.M, g.K, g.lda, BM, bits16, MN)) return ARMOR_ERR_CUDA;
+    if (!make_map(&mBlo, g.Blo, g.N, g.K, g.ldb, BNH, bits16, MN)) return ARMOR_ERR_CUDA;
   } else {
     mAlo = mA;
     mBlo = mB;
   }
-  constexpr int STAGE_BYTES = (SPLIT ? 2 : 1) * (A_BYTES + B_BYTES);
-  constexpr int STAGES = SPLIT ? 2 : 4;
-  constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 8 * 32 * TB_LD * sizeof(float);
+  constexpr size_t SMEM = (size_t)Ring<PASSES>::STAGES * Ring<PASSES>::BYTES + 1024 + 8 * EPI_BYTES;
   static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
-  const int n_sm = c->n_sm;
+  if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES, MN>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  const int n_pairs = c->n_sm / 2;
+  if (n_pairs < 1) return ARMOR_ERR_UNSUPPORTED;
   // tail split: the tiles of the last, partly filled wave are cut along K so that their pieces fill the wave
-  p.split_first = p.n_tiles_total; p.split_parts = 1; p.n_items = p.n_tiles_total; p.slabs = c->gemm_slabs;
+  p.split_first = p.n_tiles_total; p.split_parts = 1; p.split_kt = 0; p.n_items = p.n_tiles_total; p.slabs = c->gemm_slabs;
   const int kt_total = (int)((p.K + (H16 ? 64 : BK) - 1) / (H16 ? 64 : BK));
-  const int rem = p.n_tiles_total % n_sm;
-  if (c->gemm_slabs && !p.symmetric_lower && rem > 0 && p.ldc % 4 == 0 && p.N % 4 == 0) {
-    int parts = n_sm / rem;
-    if (parts > 4) parts = 4;
-    // a piece must be whole K segments (or lie inside one) so that issuer and epilogue agree on the segments
-    while (parts > 1 && (kt_total % parts || kt_total / parts < 8 ||
-                         ((kt_total / parts) % p.kt_seg && p.kt_seg < kt_total / parts)))
-      --parts;
-    if (parts > 1 && (int64_t)rem * parts <= c->gemm_slab_count) {
-      p.split_first = p.n_tiles_total - rem;
-      p.split_parts = parts;
-      p.n_items = p.split_first + rem * parts;
+  const int rem = p.n_tiles_total % n_pairs;
+  if (c->gemm_slabs && rem > 0) {
+    int parts = n_pairs / rem;
+    const int64_t room = c->gemm_slab_count / (2 * rem);         // a slab holds 128 x 256 sums, a piece writes two
+    if (parts > room) parts = (int)room;
+    // A piece writes 256 KB of sums and the second kernel reads them: about 6 us, 8 k-tiles with three MMAs per
+    // product (0.8 us each) or 24 with one, which the shorter wave has to give back
+    const int worth = SPLIT ? 8 : 24;
+    if (parts > 1) {
+      const int per = (kt_total + parts - 1) / parts;
+      if (kt_total - per >= worth) {
+        p.split_kt = per;
+        p.split_parts = (kt_total + per - 1) / per;
+        p.split_first = p.n_tiles_total - rem;
+        p.n_items = p.split_first + rem * p.split_parts;
+      }
     }
   }
-  const int grid = p.n_items < n_sm ? p.n_items : n_sm;
+  const int pairs = p.n_items < n_pairs ? p.n_items : n_pairs;
   {
     KTimer kt(c, ARMOR_KC_GEMM, p.symmetric_lower ? (double)p.M * (double)(p.N + BM) * (double)p.K
                                                   : 2.0 * (double)p.M * (double)p.N * (double)p.K, s);
-    tc_gemm_kernel<PASSES><<<grid, NTHREADS, SMEM, s>>>(mA, mAlo, mB, mBlo, p);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = SMEM; cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at; cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
-      tc_gemm_fixup_kernel<<<4 * (p.n_tiles_total - p.split_first), 256, 0, s>>>(p);
+      tc_gemm_fixup_kernel<<<8 * (p.n_tiles_total - p.split_first), 256, 0, s>>>(p);
       c->launches++;
     }
   }
@@ -508,36 +573,33 @@ bool tc_gemm_shape_ok(int64_t M, int64_t N, int64_t K) {
   return M > 0 && N > 0 && K > 0 && (N % 32 == 0) && (K % 4 == 0);
 }
 
-armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_tiles, cudaStream_t s) {
-  if (!tc_gemm_shape_ok(g.M, g.N, g.K)) return ARMOR_ERR_UNSUPPORTED;
+armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStream_t s) {
+  if (!tc_gemm_shape_ok(g.M, g.N, g.mn_major ? 4 : g.K)) return ARMOR_ERR_UNSUPPORTED;   // (k beyond K reads as zero)
   const bool h16 = (g.passes == 0 || g.passes == 6);
   if ((g.lda % (h16 ? 8 : 4)) || (g.ldb % (h16 ? 8 : 4)) || (g.ldc % 4)) return ARMOR_ERR_UNSUPPORTED;
   if ((g.row_scale == nullptr) != (g.col_scale == nullptr)) return ARMOR_ERR_INVALID_ARG;
   if (g.symmetric_lower && g.M != g.N) return ARMOR_ERR_INVALID_ARG;
   Params p{};
   p.C = g.C; p.ldc = g.ldc; p.M = g.M; p.N = g.N; p.K = g.K;
-  p.m_tiles = (int)((g.M + BM - 1) / BM);
+  p.m_tiles = (int)((g.M + BMP - 1) / BMP);
   p.n_tiles = (int)((g.N + BN - 1) / BN);
-  if (g.symmetric_lower) {
-    int tot = 0;
-    for (int nt = 0; nt < p.n_tiles; ++nt) {
-      const int cnt = p.m_tiles - 2 * nt;
-      if (cnt > 0) tot += cnt;
-    }
-    p.n_tiles_total = tot;
-  } else {
-    p.n_tiles_total = p.m_tiles * p.n_tiles;
-  }
+  p.n_tiles_total = g.symmetric_lower ? p.m_tiles * (p.m_tiles + 1) / 2 : p.m_tiles * p.n_tiles;
   p.accumulate = g.accumulate; p.symmetric_lower = g.symmetric_lower;
   p.d1 = g.d1; p.d2 = g.d2; p.part1 = g.part1; p.part2 = g.part2;
   p.row_scale = g.row_scale; p.col_scale = g.col_scale; p.f16 = g.fp16;
   p.status = c->status;
+  p.c_vec = (reinterpret_cast<uintptr_t>(g.C) % 16 == 0) ? 1 : 0;   // (ldc is a multiple of 4)
   const int bke = h16 ? 64 : BK;
   p.kt_seg = g.k_segment > 0 ? (int)((g.k_segment + bke - 1) / bke) : (int)((g.K + bke - 1) / bke);
   if (p.kt_seg < 1) p.kt_seg = 1;
-  if (n_tiles) *n_tiles = p.n_tiles_total;
-  if (g.passes == 3) return launch_impl<3>(c, g, p, s);
-  if (g.passes == 6) return launch_impl<6>(c, g, p, s);
-  if (g.passes == 0) return launch_impl<0>(c, g, p, s);
-  return launch_impl<1>(c, g, p, s);
+  if (n_part) *n_part = PARTS * p.n_tiles_total;
+  if (g.mn_major) {
+    // a map's rows start at multiples of 64 elements; the base and the leading dimension must be multiples of 16 bytes
+    if (g.passes != 0 || reinterpret_cast<uintptr_t>(g.A) % 16 || reinterpret_cast<uintptr_t>(g.B) % 16) return ARMOR_ERR_UNSUPPORTED;
+    return launch_impl<0, true>(c, g, p, s);
+  }
+  if (g.passes == 3) return launch_impl<3, false>(c, g, p, s);
+  if (g.passes == 6) return launch_impl<6, false>(c, g, p, s);
+  if (g.passes == 0) return launch_impl<0, false>(c, g, p, s);
+  return launch_impl<1, false>(c, g, p, s);
 }

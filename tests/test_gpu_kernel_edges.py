@@ -1,0 +1,60 @@
+"""Kernels at the sizes where their tiling can go wrong: tile edges, remainders, the smallest and largest of a range."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+def _ctx(*a, **k):
+    from paper_2510_05528_b200 import binding as Bd
+    return Bd.ArmorContext(*a, device=DEV, **k)
+
+
+def _gen(seed):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(seed)
+    return g
+
+
+@pytest.mark.parametrize("d_in,tokens", [(128, 1), (128, 4095), (256, 63), (384, 65), (640, 1024), (1024, 1025),
+                                         (256, 16384 + 77)])
+@pytest.mark.parametrize("form", ["plain", "strided", "unaligned_x", "unaligned_h"])
+def test_bf16_gram_as_it_lies_in_memory(d_in, tokens, form):
+    """X is read where it lies (any leading dimension that is a multiple of 8); a base or leading dimension that TMA does
+    not take goes through the staged path; H may start on any 4-byte boundary.  Sums of exact products in fp32: segments
+    of 1,024 terms that truncate (2^-23 per 16 terms: below 64 x 2^-23 = 8e-6 of sum |x_i x_j|), then rounded sums."""
+    lead = {"plain": d_in, "strided": d_in + 24, "unaligned_x": d_in + 3, "unaligned_h": d_in}[form]
+    buf = torch.randn(tokens * lead + 1, device=DEV, generator=_gen(tokens + d_in)).to(torch.bfloat16)
+    off = 1 if form == "unaligned_x" else 0
+    X = buf[off: off + tokens * lead].view(tokens, lead)[:, :d_in]
+    ctx = _ctx(128, d_in, 128)
+    store = torch.ones(d_in * d_in + 1, device=DEV)
+    H = store[1:].view(d_in, d_in) if form == "unaligned_h" else store[:-1].view(d_in, d_in)
+    ctx.gram(X, H)
+    Xd = X.double()
+    err = (H.double() - 1.0 - Xd.t() @ Xd).abs()
+    assert torch.equal(H, H.t())
+    assert (err <= 8e-6 * (1.0 + Xd.abs().t() @ Xd.abs())).all()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in", [(128, 128), (128, 384), (384, 256), (640, 1152), (1024, 2560)])
+@pytest.mark.parametrize("precision", ["FP16X3", "FP32X3", "TF32"])
+def test_dense_product_with_h_at_tile_edges(d_out, d_in, precision):
+    """W H through one iteration's loss: L = <E H, E> with E = W - A S B at the initialisation, tiles of 256 x 256 cut by
+    the matrix's edge, with and without the contraction split over several pairs of CTAs."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + d_in)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    X = torch.randn(2 * d_in, d_in, device=DEV, generator=g)
+    H = (X.double().t() @ X.double()).float()
+    ctx = _ctx(d_out, d_in, 128, precision=getattr(Bd, "PREC_" + precision))
+    st = ctx.init(W, H)
+    loss = ctx.proxy_loss(st, H).item()
+    E = (W - st.S).double()
+    ref = ((E @ H.double()) * E).sum().item()
+    assert abs(loss - ref) <= (2e-2 if precision == "TF32" else 1e-5) * ref
+    assert np.isfinite(ref) and ctx.device_status()[:4] == [0, 0, 0, 0]
