@@ -858,6 +858,13 @@ armor_status armor_apply_layer(armor_ctx* c, const void* d_packed, const void* d
   cudaStream_t s = cs(stream);
   const char* buf = static_cast<const char*>(d_packed);
   const int64_t d_out = c->d_out, d_in = c->d_in;
+  if (n_tokens <= ARMOR_SMALL_TOKENS) {
+    int pieces = 0;
+    armor_status st = launch_fwd_small(c, d_x, 0, buf + layer_off_B(c), c->T, n_tokens, d_in, s);               // z1 = (r1 . x) B^T
+    if (st == ARMOR_OK) st = launch_tc_sparse_small(c, buf, buf + tc_sparse_values_bytes(c), c->T, c->E, n_tokens, &pieces, s);
+    if (st == ARMOR_OK) st = launch_fwd_small(c, c->E, pieces, buf + layer_off_A(c), d_y, n_tokens, d_out, s);  // y = r2 . (z2 A^T)
+    return st == ARMOR_OK ? finish_call(c) : st;
+  }
   const int64_t chunk = d_out < d_in ? d_out : d_in;   // bf16 z1 [chunk, d_in] and z2 [chunk, d_out] fit W-shaped scratch
   for (int64_t t0 = 0; t0 < n_tokens; t0 += chunk) {
     const int64_t n = (n_tokens - t0 < chunk) ? n_tokens - t0 : chunk;

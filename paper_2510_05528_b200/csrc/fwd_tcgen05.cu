@@ -200,6 +200,81 @@ fwd_block_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant
   }
 }
 
+// The same product for few tokens: one CTA per 16 tokens x 128 columns, eight warps of 16 columns.  At this size only
+// latency counts, and the persistent kernel above pays for tensor memory, barriers and 128-row tiles that are mostly
+// padding (4.6 us a launch at one token); here a warp requests its wrapper rows before it waits for the kernel before
+// (programmatic dependent launch), the tokens go through shared memory once, and mma.sync m16n8k16 (tokens on the M side)
+// does the rest.  The order of k inside an instruction is free as long as both operands agree, so a lane takes eight
+// consecutive k (16 bytes) of its rows as the operands of two instructions; the columns of the two n-tiles are dealt out so
+// that a lane ends with four neighbouring ones.
+// SUM: the tokens come as `pieces` arrays of fp32 partial sums [rows][d], added in order and rounded to bf16 once.
+__device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
+                                         uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+template <int DB, bool SUM>
+__global__ void __launch_bounds__(256)
+fwd_small_kernel(const void* __restrict__ X, int pieces, const __nv_bfloat16* __restrict__ Q, __nv_bfloat16* __restrict__ out,
+                 int rows, int64_t d) {
+  constexpr int LD = DB * 2 + 64;                     // bytes per staged token: eight lanes of a phase hit eight banks
+  __shared__ __align__(16) uint8_t tok[16 * LD];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  const int64_t n0 = (int64_t)blockIdx.x * 128 + warp * 16;
+  const int64_t kbase = (int64_t)blockIdx.x * 128 / DB * DB;   // first column of X of the block these columns belong to
+  const int r0 = blockIdx.y * 16;
+  grid_launch_dependents();
+  uint4 w[2][DB / 32];
+#pragma unroll
+  for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+    for (int ch = 0; ch < DB / 32; ++ch)
+      w[nt][ch] = __ldg(reinterpret_cast<const uint4*>(Q + (n0 + 4 * (g >> 1) + 2 * nt + (g & 1)) * DB + ch * 32 + 8 * t));
+  if (SUM) grid_dependency_wait();
+#pragma unroll
+  for (int e = threadIdx.x; e < 16 * DB / 8; e += 256) {
+    const int r = e / (DB / 8), c8 = e % (DB / 8);
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (r0 + r < rows) {
+      const int64_t o = (int64_t)(r0 + r) * d + kbase + 8 * c8;
+      if (SUM) {
+        const float* z = static_cast<const float*>(X) + o;
+        float4 a = *reinterpret_cast<const float4*>(z), b = *reinterpret_cast<const float4*>(z + 4);
+#pragma unroll 4
+        for (int k = 1; k < pieces; ++k) {
+          z += (int64_t)rows * d;
+          const float4 a2 = *reinterpret_cast<const float4*>(z), b2 = *reinterpret_cast<const float4*>(z + 4);
+          a.x += a2.x; a.y += a2.y; a.z += a2.z; a.w += a2.w;
+          b.x += b2.x; b.y += b2.y; b.z += b2.z; b.w += b2.w;
+        }
+        v = make_uint4(pack_bf16(a.x, a.y), pack_bf16(a.z, a.w), pack_bf16(b.x, b.y), pack_bf16(b.z, b.w));
+      } else {
+        v = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(X) + o);
+      }
+    }
+    *reinterpret_cast<uint4*>(tok + r * LD + 16 * c8) = v;
+  }
+  __syncthreads();
+  float acc[2][4] = {};
+#pragma unroll
+  for (int ch = 0; ch < DB / 32; ++ch) {
+    const uint4 a0 = *reinterpret_cast<const uint4*>(tok + g * LD + ch * 64 + t * 16);
+    const uint4 a1 = *reinterpret_cast<const uint4*>(tok + (g + 8) * LD + ch * 64 + t * 16);
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      mma_bf16(acc[nt], a0.x, a1.x, a0.y, a1.y, w[nt][ch].x, w[nt][ch].y);
+      mma_bf16(acc[nt], a0.z, a1.z, a0.w, a1.w, w[nt][ch].z, w[nt][ch].w);
+    }
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+    if (r0 + g + 8 * h < rows)
+      *reinterpret_cast<uint2*>(out + (int64_t)(r0 + g + 8 * h) * d + n0 + 4 * t) =
+          make_uint2(pack_bf16(acc[0][2 * h], acc[0][2 * h + 1]), pack_bf16(acc[1][2 * h], acc[1][2 * h + 1]));
+}
+
 // Q[i][m][k] = rowscale[i*db + m] * colscale[i*db + k] * P[i][m][k], rounded to bf16 (either scale may be null)
 __global__ void __launch_bounds__(256)
 pack_blocks_kernel(const float* __restrict__ P, const float* __restrict__ rowscale, const float* __restrict__ colscale,
@@ -263,4 +338,28 @@ armor_status launch_fwd_block(armor_ctx* c, const void* X, const void* Q, void* 
   fwd_block_kernel<<<grid, NTHREADS, SMEM, s>>>(mX, mQ, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+}
+
+// The same for up to ARMOR_SMALL_TOKENS rows.  pieces == 0: X is bf16 [rows][d]; otherwise X holds that many fp32 arrays
+// [rows][d] whose sum, rounded to bf16, is the operand, and the launch may overlap the kernel that writes them.
+armor_status launch_fwd_small(armor_ctx* c, const void* X, int pieces, const void* Q, void* out, int64_t rows, int64_t d,
+                              cudaStream_t s) {
+  if (!fwd_block_ok(c) || rows <= 0 || rows > ARMOR_SMALL_TOKENS || d % 128) return ARMOR_ERR_UNSUPPORTED;
+  KTimer kt(c, ARMOR_KC_FORWARD, 4.0 * (double)rows * (double)d, s);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(d / 128), (unsigned)((rows + 15) / 16)); cfg.blockDim = dim3(256); cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = pieces > 0 ? 1 : 0;
+  const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(Q);
+  __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out);
+  const int n = (int)rows;
+  cudaError_t e;
+  if (c->db == 128) e = pieces > 0 ? cudaLaunchKernelEx(&cfg, fwd_small_kernel<128, true>, X, pieces, q, o, n, d)
+                                   : cudaLaunchKernelEx(&cfg, fwd_small_kernel<128, false>, X, 0, q, o, n, d);
+  else e = pieces > 0 ? cudaLaunchKernelEx(&cfg, fwd_small_kernel<256, true>, X, pieces, q, o, n, d)
+                      : cudaLaunchKernelEx(&cfg, fwd_small_kernel<256, false>, X, 0, q, o, n, d);
+  c->launches++;
+  return e == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }

@@ -429,6 +429,140 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
   }
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// The same product for few tokens (up to 128, one tile of BNS tokens), where reading S is the whole cost and the tiles
+// above leave most of the chip idle (one 256 x 256 tile per pair: 32 of 148 SMs at 4096 x 4096, 21 us).  The contraction
+// is cut into pieces so that (row tiles) x (pieces) fills two CTAs per SM; a CTA keeps up to 72 KiB of S in flight, sums
+// its piece in tensor memory and writes it as fp32, and the kernel that multiplies with A adds the pieces in a fixed
+// order (fwd_small_kernel).  S does not depend on the kernel before: its first stages are requested before the wait for
+// that kernel's z1 (programmatic dependent launch).
+template <int BNS>
+struct SmallN {
+  static constexpr int BH = BNS * 64 * 2;                       // one half (64 k) of the Z1 stage
+  static constexpr int STAGE = A_BYTES + 2 * BH + E_BYTES;
+  static constexpr int STAGES = BNS <= 32 ? 4 : (BNS == 64 ? 3 : 2);   // two CTAs share an SM's shared memory
+  static constexpr uint32_t COLS = BNS <= 32 ? 64 : (BNS == 64 ? 128 : 256);   // accumulator, then 4 columns per stage
+  static constexpr size_t SMEM = (size_t)STAGES * STAGE + 1024;
+};
+
+template <int BNS>
+__global__ void __launch_bounds__(NTHREADS, 2)
+tc_sparse_small_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
+                       const __grid_constant__ CUtensorMap mapE, const SParams p, int k_per_piece) {
+  using T = SmallN<BNS>;
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t bars[2 * T::STAGES + 1];
+  __shared__ uint32_t tmem_base_holder;
+  __shared__ int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[T::STAGES]), tfull = smem_u32(&bars[2 * T::STAGES]);
+  const int mt = blockIdx.x;
+  const int k0 = blockIdx.y * k_per_piece, k1 = min(p.k_tiles, k0 + k_per_piece);
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < T::STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+    mbar_init(tfull, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
+                 "r"(T::COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  grid_launch_dependents();
+  const uint32_t tmem_base = tmem_base_holder;
+  volatile int* abortp = &abort_flag;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      auto load_s = [&](int kt, int stage) {
+        const uint32_t dst = smem_u32(smem + (size_t)stage * T::STAGE), fb = full0 + 8 * stage;
+        mbar_expect_tx(fb, T::STAGE);
+        tma_load_2d(dst, &mapA, kt * 64, mt * BM, fb);
+        tma_load_2d(dst + A_BYTES + 2 * T::BH, &mapE, 0, (mt * p.k_tiles + kt) * 128, fb);
+      };
+      auto load_z = [&](int kt, int stage) {
+        const uint32_t dst = smem_u32(smem + (size_t)stage * T::STAGE) + A_BYTES, fb = full0 + 8 * stage;
+        tma_load_2d(dst, &mapB, kt * BKL, 0, fb);
+        tma_load_2d(dst + T::BH, &mapB, kt * BKL + 64, 0, fb);
+      };
+      const int pre = min(T::STAGES, k1 - k0);
+      for (int i = 0; i < pre; ++i) load_s(k0 + i, i);
+      grid_dependency_wait();
+      for (int i = 0; i < pre; ++i) load_z(k0 + i, i);
+      int stage = pre % T::STAGES; uint32_t phase = pre == T::STAGES ? 1 : 0;
+      long long issued = pre;
+      bool ok = true;
+      for (int kt = k0 + pre; kt < k1; ++kt) {
+        if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
+        load_s(kt, stage);
+        load_z(kt, stage);
+        ++issued;
+        if (++stage == T::STAGES) { stage = 0; phase ^= 1; }
+      }
+      if (!ok) {
+        for (int back = 1; back <= T::STAGES && back <= issued; ++back) {
+          int s = stage - back; uint32_t ph = phase;
+          if (s < 0) { s += T::STAGES; ph ^= 1; }
+          const long long t0 = clock64();
+          while (!mbar_try(full0 + 8 * s, ph) && clock64() - t0 < 20000000ll) {}
+        }
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = (instr_desc_sp(0) & ~(0x3Fu << 17)) | ((uint32_t)(BNS >> 3) << 17);
+      int stage = 0; uint32_t phase = 0;
+      bool ok = true;
+      for (int kt = k0; kt < k1; ++kt) {
+        if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+        tc_fence_after();
+        const uint32_t sa = smem_u32(smem + (size_t)stage * T::STAGE);
+        const uint32_t sb = sa + A_BYTES;
+        const uint32_t meta = tmem_base + BNS + (uint32_t)(4 * stage);
+        tmem_cp_e(meta, smem_desc_e(sb + 2 * T::BH));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const uint64_t da = smem_desc_k(sa + j * 32);
+          const uint64_t dbm = smem_desc_k(sb + (j >> 1) * T::BH + (j & 1) * 64);
+          umma_bf16_sp(tmem_base, da, dbm, meta + (uint32_t)(j & ~1), idesc | (uint32_t)(j & 1), (uint32_t)((kt > k0) | (j != 0)));
+        }
+        umma_commit(empty0 + 8 * stage);
+        if (++stage == T::STAGES) { stage = 0; phase ^= 1; }
+      }
+      if (ok) umma_commit(tfull);
+    }
+  } else {
+    const int q = warp & 3;
+    if (mbar_wait(tfull, 0, abortp, p.status)) {
+      tc_fence_after();
+      const int64_t row = (int64_t)mt * BM + q * 32 + lane;
+      float* Z = p.Z + (int64_t)blockIdx.y * p.N * p.ldz + row;          // this piece's sums, [tokens][d_out]
+#pragma unroll 1
+      for (int ch = 0; ch < BNS / 16; ++ch) {
+        uint32_t r[16];
+        tmem_ld16(tmem_base + (uint32_t)(ch * 16) + ((uint32_t)(q * 32) << 16), r);
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+          if (ch * 16 + i < p.N) Z[(int64_t)(ch * 16 + i) * p.ldz] = __uint_as_float(r[i]);
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(T::COLS) : "memory");
+  }
+}
+
 // One thread per 32-bit word of positions: 2 rows x 16 k.  Writes the word and the eight pairs of kept values.
 // A group whose mask byte keeps fewer than two positions is padded with unkept positions (their values are
 // written as zeros); more than two kept positions cannot be represented: the first two are taken and the
@@ -478,17 +612,41 @@ compress_24_kernel(const float* __restrict__ S, const uint8_t* __restrict__ Mk, 
   if (bad) atomicAdd(&status[ST_SPARSE_BAD_GROUPS], 1);
 }
 
-bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld) {
+bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows = 128) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {64, 128};
+  cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+bool make_map_e(CUtensorMap* map, const void* base, int64_t rows);
+
+template <int BNS>
+armor_status launch_small(armor_ctx* c, const void* Sc, const void* E, const void* z1, SParams p, int pieces, int per,
+                          cudaStream_t s) {
+  CUtensorMap mA, mB, mE;
+  if (!make_map_bf16(&mA, Sc, c->d_out, c->d_in / 2, c->d_in / 2)) return ARMOR_ERR_CUDA;
+  if (!make_map_bf16(&mB, z1, p.N, c->d_in, c->d_in, BNS)) return ARMOR_ERR_CUDA;
+  if (!make_map_e(&mE, E, (c->d_out / 128) * (c->d_in / 128) * 128)) return ARMOR_ERR_CUDA;
+  static PerDeviceOnce attr;
+  if (ensure_dynamic_smem(attr, c->device, tc_sparse_small_kernel<BNS>, SmallN<BNS>::SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)p.M * (double)p.N * (double)p.K, s);   // dense-equivalent flops
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)p.m_tiles, (unsigned)pieces); cfg.blockDim = dim3(NTHREADS);
+  cfg.dynamicSmemBytes = SmallN<BNS>::SMEM; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, tc_sparse_small_kernel<BNS>, mA, mB, mE, p, per) != cudaSuccess) return ARMOR_ERR_CUDA;
+  c->launches++;
+  return ARMOR_OK;
 }
 
 // positions: [rows of 16 bytes], box = 128 rows, no swizzle
@@ -564,4 +722,24 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
   }
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+}
+
+// Zp[piece][n][d_out] = the pieces of Z1[n][d_in] * S^T (bf16 operands, fp32 sums) for n <= ARMOR_SMALL_TOKENS tokens;
+// their number goes to *pieces.  pieces * n <= d_in, so Zp fits a W-shaped fp32 buffer.
+armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E, const void* z1_bf16, float* Zp, int64_t n,
+                                    int* pieces, cudaStream_t s) {
+  if (!tc_sparse_ok(c) || n <= 0 || n > ARMOR_SMALL_TOKENS) return ARMOR_ERR_UNSUPPORTED;
+  SParams p{};
+  p.Z = Zp; p.ldz = c->d_out; p.M = c->d_out; p.N = n; p.K = c->d_in;
+  p.m_tiles = (int)(c->d_out / BM); p.n_tiles = 1; p.k_tiles = (int)(c->d_in / BKL);
+  p.status = c->status;
+  int want = 2 * c->n_sm / p.m_tiles;
+  if (want < 1) want = 1;
+  if (want > p.k_tiles) want = p.k_tiles;
+  const int per = (p.k_tiles + want - 1) / want;
+  *pieces = (p.k_tiles + per - 1) / per;
+  if (n <= 16) return launch_small<16>(c, Sc, E, z1_bf16, p, *pieces, per, s);
+  if (n <= 32) return launch_small<32>(c, Sc, E, z1_bf16, p, *pieces, per, s);
+  if (n <= 64) return launch_small<64>(c, Sc, E, z1_bf16, p, *pieces, per, s);
+  return launch_small<128>(c, Sc, E, z1_bf16, p, *pieces, per, s);
 }

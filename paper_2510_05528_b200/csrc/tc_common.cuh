@@ -133,6 +133,16 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
 }
 
 
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
 // registers -> tensor memory: lane l of the warp writes r[0..31] to 32 consecutive columns of TMEM lane (base lane + l);
 // the caller issues tcgen05.wait::st before it signals the consumer
 __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* r) {
@@ -185,6 +195,11 @@ __device__ __forceinline__ uint32_t instr_desc_tf32_mn(int M, int N, int a_mn, i
   d |= (uint32_t)(M >> 4) << 24;
   return d;
 }
+
+// ---- programmatic dependent launch: a kernel launched with the attribute starts once every CTA of the kernel before it
+// has called grid_launch_dependents (or has ended); what that kernel wrote may be read after grid_dependency_wait
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // ---- pairs of CTAs (cluster of two, cta_group::2)
 __device__ __forceinline__ uint32_t cluster_ctarank() {

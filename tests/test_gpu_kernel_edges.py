@@ -58,3 +58,34 @@ def test_dense_product_with_h_at_tile_edges(d_out, d_in, precision):
     ref = ((E @ H.double()) * E).sum().item()
     assert abs(loss - ref) <= (2e-2 if precision == "TF32" else 1e-5) * ref
     assert np.isfinite(ref) and ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(128, 128, 128), (384, 512, 128), (512, 256, 256), (4096, 1152, 128),
+                                                (19072, 2048, 128)])
+def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
+    """The packed layer at every token tile of the split product (16, 32, 64, 128) and beside its edges, against the rows
+    of a batch that takes the persistent kernels.  Integer operands: every fp32 sum is exact in any order, so the
+    roundings to bf16 are the same and the outputs agree bit for bit."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out * 7 + d_in)
+    ctx = _ctx(d_out, d_in, d_block)
+
+    def ints(lo, hi, *shape):
+        return torch.randint(lo, hi + 1, shape, device=DEV, generator=g).float()
+    S = ints(-2, 2, d_out, d_in)
+    grp = S.view(d_out, d_in // 4, 4)
+    keep = torch.zeros_like(grp, dtype=torch.bool).scatter_(2, torch.rand(grp.shape, device=DEV, generator=g).topk(2, 2).indices, True)
+    grp.mul_(keep)
+    M = (keep * torch.tensor([1, 2, 4, 8], device=DEV)).sum(2).to(torch.uint8)
+    st = Bd.LayerState(Wbar=S, A=ints(-1, 1, d_out // d_block, d_block, d_block), B=ints(-1, 1, d_in // d_block, d_block, d_block),
+                       S=S, M=M)
+    packed = ctx.pack_layer(st)
+    x = ints(-1, 1, 300, d_in).to(torch.bfloat16)
+    big = ctx.apply_layer(packed, x)
+    z1 = torch.einsum("tjk,jmk->tjm", x.float().view(300, -1, d_block), st.B).reshape(300, d_in).to(torch.bfloat16)
+    z2 = (z1.double() @ S.double().t()).to(torch.bfloat16)
+    y = torch.einsum("tjk,jmk->tjm", z2.double().view(300, -1, d_block), st.A.double()).reshape(300, d_out).float().to(torch.bfloat16)
+    assert torch.equal(big, y)
+    for n in (1, 15, 16, 17, 32, 33, 63, 64, 65, 127, 128, 129):
+        assert torch.equal(ctx.apply_layer(packed, x[:n].contiguous()), big[:n]), n
+    assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
