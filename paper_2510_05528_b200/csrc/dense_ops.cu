@@ -11,6 +11,13 @@
 // contraction into running sums held by its epilogue warps (ordinary round-to-nearest fp32 adds).
 static const int64_t K_SEGMENT = 1024;
 
+// Products this small run on the fp32 lanes: one launch instead of the operand split, the tensor-core product and the sum
+// of its pieces, whose fixed costs (tensor memory, cluster launch, a second pass over the operand) exceed the arithmetic.
+static bool dense_on_lanes(const armor_ctx* c, int64_t rows) {
+  if (c->cfg.precision == ARMOR_PREC_SIMT) return true;
+  return c->cfg.precision != ARMOR_PREC_TF32 && rows * c->d_in * c->d_in <= (1 << 25);
+}
+
 armor_status prepare_H(armor_ctx* c, const float* H, cudaStream_t s) {
   launch_extract_hblocks(c, H, s);
   if (c->cfg.h_mode == ARMOR_H_FULL && c->cfg.precision == ARMOR_PREC_FP32X3)
@@ -37,7 +44,7 @@ armor_status rmul_H(armor_ctx* c, const float* in, const float* H, float* out, i
   }
   if (c->cfg.h_mode == ARMOR_H_DIAG) {
     launch_colscale(c, in, c->hdiag, out, rows, d_in, s);
-  } else if (c->cfg.precision == ARMOR_PREC_SIMT) {
+  } else if (dense_on_lanes(c, rows)) {
     BGemm g{};
     g.A = in; g.sAm = d_in; g.sAk = 1;
     g.B = H; g.sBk = d_in; g.sBn = 1;

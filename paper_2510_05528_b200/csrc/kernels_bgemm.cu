@@ -231,6 +231,117 @@ __global__ void __launch_bounds__(NT, 2) bgemm_tile_kernel(BGemm g, float* __res
   }
 }
 
+// ------------------------------------------------------------------------------ small products
+// 32 x 32 tiles for products that would leave most SMs without a 128 x 128 tile (the wrapper products of small blocks, the
+// [nb, d_block, d_block] products).  They are bound by latency: eight warps fetch 128 k of both operands at once (the next
+// 128 are in flight meanwhile), every pair of warps multiplies a quarter of them, 4 x 4 sums per thread, and the four
+// quarters are added in a fixed order at the end.  Same operand forms as above; K a multiple of 16.
+constexpr int SM_T = 32, SM_K = 128;
+// position of 16-byte unit u of k-row k: swizzled so that neither the writes along k nor the reads along a row conflict
+__device__ __forceinline__ int sm_unit(int k, int u) { return k * SM_T + 4 * (u ^ ((k >> 2) & 7)); }
+
+template <bool A_KFAST, bool B_NFAST>
+__global__ void __launch_bounds__(NT) bgemm_small_kernel(BGemm g) {
+  __shared__ __align__(16) float As[SM_K * SM_T];
+  __shared__ __align__(16) float Bs[SM_K * SM_T];
+  const int m0 = blockIdx.y * SM_T, n0 = blockIdx.x * SM_T;
+  int64_t oa, ob, oc, od;
+  batch_offsets(g, blockIdx.z, oa, ob, oc, od);
+  const float* __restrict__ A = g.A + oa;
+  const float* __restrict__ B = g.B + ob;
+  const int tid = threadIdx.x;
+  float4 ra[4], rb[4];
+  // 32 x 128 floats of either operand: four float4 per thread, along whichever index is contiguous
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int f = tid + e * NT;
+      ra[e] = rb[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (A_KFAST) {
+        const int m = tid >> 3, k = k0 + 32 * e + 4 * (tid & 7);
+        if (m0 + m < g.M && k < g.K) ra[e] = *reinterpret_cast<const float4*>(A + (int64_t)(m0 + m) * g.sAm + k);
+      } else {
+        const int k = k0 + (f >> 3), m = m0 + 4 * (f & 7);
+        if (m < g.M && k < g.K) ra[e] = *reinterpret_cast<const float4*>(A + (int64_t)k * g.sAk + m);
+      }
+      if (B_NFAST) {
+        const int k = k0 + (f >> 3), n = n0 + 4 * (f & 7);
+        if (n < g.N && k < g.K) rb[e] = *reinterpret_cast<const float4*>(B + (int64_t)k * g.sBk + n);
+      } else {
+        const int n = tid >> 3, k = k0 + 32 * e + 4 * (tid & 7);
+        if (n0 + n < g.N && k < g.K) rb[e] = *reinterpret_cast<const float4*>(B + (int64_t)(n0 + n) * g.sBn + k);
+      }
+    }
+  };
+  auto stash_one = [&](float* T, const float4& v, int e, bool kfast) {
+    if (kfast) {
+      const int x = tid >> 3, k = 32 * e + 4 * (tid & 7);
+      float* q = T + sm_unit(k, x >> 2) + (x & 3);        // the four k share a swizzle
+      q[0] = v.x; q[SM_T] = v.y; q[2 * SM_T] = v.z; q[3 * SM_T] = v.w;
+    } else {
+      const int f = tid + e * NT;
+      *reinterpret_cast<float4*>(T + sm_unit(f >> 3, f & 7)) = v;
+    }
+  };
+  const int grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
+  float acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  fetch(0);
+  for (int k0 = 0; k0 < g.K; k0 += SM_K) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { stash_one(As, ra[e], e, A_KFAST); stash_one(Bs, rb[e], e, !B_NFAST); }
+    __syncthreads();
+    if (k0 + SM_K < g.K) fetch(k0 + SM_K);
+    const int kn = min(SM_K, g.K - k0) >> 2;              // k of this step per group: a multiple of 4
+    const int kb = grp * kn;
+#pragma unroll 4
+    for (int k = 0; k < kn; ++k) {
+      const float4 a4 = *reinterpret_cast<const float4*>(As + sm_unit(kb + k, ty));
+      const float4 b4 = *reinterpret_cast<const float4*>(Bs + sm_unit(kb + k, tx));
+      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  // sums of the four groups, in group order; then one float4 of a row per thread
+  float* part = As;                                       // [4][32][32]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    *reinterpret_cast<float4*>(part + (grp * SM_T + 4 * ty + i) * SM_T + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  __syncthreads();
+  const int r = tid >> 3, c4 = 4 * (tid & 7);
+  const int m = m0 + r, n = n0 + c4;
+  if (m >= g.M || n >= g.N) return;
+  float4 v = *reinterpret_cast<const float4*>(part + r * SM_T + c4);
+#pragma unroll
+  for (int q = 1; q < 4; ++q) {
+    const float4 w = *reinterpret_cast<const float4*>(part + (q * SM_T + r) * SM_T + c4);
+    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+  }
+  v = make_float4(g.alpha * v.x, g.alpha * v.y, g.alpha * v.z, g.alpha * v.w);
+  if (g.D) {
+    const float4 d = *reinterpret_cast<const float4*>(g.D + od + (int64_t)m * g.sDm + n);
+    v.x = fmaf(g.beta, d.x, v.x); v.y = fmaf(g.beta, d.y, v.y);
+    v.z = fmaf(g.beta, d.z, v.z); v.w = fmaf(g.beta, d.w, v.w);
+  }
+  *reinterpret_cast<float4*>(g.C + oc + (int64_t)m * g.sCm + n) = v;
+}
+
+// The share of the chip's lanes that 128 x 128 tiles would keep busy: tiles per SM, times the part of a tile that holds
+// elements.  Below a half the small tiles are faster.
+inline bool small_tiles_better(const BGemm& g) {
+  const int64_t tiles = (int64_t)((g.M + FM - 1) / FM) * ((g.N + FN - 1) / FN) * g.batch * (g.ksplit > 1 ? g.ksplit : 1);
+  const int64_t elems = (int64_t)g.M * g.N * g.batch * (g.ksplit > 1 ? g.ksplit : 1);
+  const int64_t slots = tiles > 148 ? tiles : 148;
+  return 2 * elems < slots * FM * FN;
+}
+
 // out[b][m][n] = alpha * sum_ks part[ks][b][m][n]  (fixed order), scattered to the strided destination
 __global__ void __launch_bounds__(NT) bgemm_splitsum_kernel(BGemm g, const float* __restrict__ part,
                                                             int64_t part_stride) {
@@ -279,6 +390,15 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
   if (g.ksplit > 1 && (g.D || !c->gpart || (int64_t)g.ksplit * g.batch * g.M * g.N > c->gpart_floats)) g.ksplit = 1;
   bool a_kfast = false, b_nfast = false;
   if (g.ksplit > 1 && !tile_kernel_ok(g, a_kfast, b_nfast)) g.ksplit = 1;
+  if (tile_kernel_ok(g, a_kfast, b_nfast) && small_tiles_better(g)) {
+    dim3 grid((g.N + SM_T - 1) / SM_T, (g.M + SM_T - 1) / SM_T, g.batch);
+    if (a_kfast && b_nfast) bgemm_small_kernel<true, true><<<grid, NT, 0, s>>>(g);
+    else if (a_kfast && !b_nfast) bgemm_small_kernel<true, false><<<grid, NT, 0, s>>>(g);
+    else if (!a_kfast && b_nfast) bgemm_small_kernel<false, true><<<grid, NT, 0, s>>>(g);
+    else bgemm_small_kernel<false, false><<<grid, NT, 0, s>>>(g);
+    c->launches++;
+    return;
+  }
   if (tile_kernel_ok(g, a_kfast, b_nfast)) {
     const int ks = g.ksplit > 1 ? g.ksplit : 1;
     dim3 grid((g.N + FN - 1) / FN, (g.M + FM - 1) / FM, g.batch * ks);

@@ -89,3 +89,31 @@ def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
     for n in (1, 15, 16, 17, 32, 33, 63, 64, 65, 127, 128, 129):
         assert torch.equal(ctx.apply_layer(packed, x[:n].contiguous()), big[:n]), n
     assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(32, 64, 32), (96, 256, 32), (256, 256, 32), (320, 128, 64), (120, 200, 8),
+                                                (48, 144, 16), (1024, 512, 64), (160, 96, 32)])
+@pytest.mark.parametrize("side", [0, 1])
+@pytest.mark.parametrize("transpose", [0, 1])
+def test_small_wrapper_products(d_out, d_in, d_block, side, transpose):
+    """Products with small wrapper blocks (32 x 32 tiles on fp32 lanes), plain and with an addend, in every operand order;
+    an fp32 sum of d_block terms: below d_block * 2^-24 of the sum of magnitudes, plus the addend's rounding."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + 3 * d_in + d_block)
+    ctx = _ctx(d_out, d_in, d_block, precision=Bd.PREC_SIMT, h_mode=Bd.H_DIAG)
+    X = torch.randn(d_out, d_in, device=DEV, generator=g)
+    D = torch.randn(d_out, d_in, device=DEV, generator=g)
+    nb = (d_out if side else d_in) // d_block
+    Q = torch.randn(nb, d_block, d_block, device=DEV, generator=g)
+    Qd = (Q.transpose(1, 2) if transpose else Q).double()
+    if side:
+        ref = (Qd @ X.double().view(nb, d_block, d_in)).view(d_out, d_in)
+        mag = (Qd.abs() @ X.double().abs().view(nb, d_block, d_in)).view(d_out, d_in)
+    else:
+        ref = torch.einsum("rjk,jkm->rjm", X.double().view(d_out, nb, d_block), Qd).reshape(d_out, d_in)
+        mag = torch.einsum("rjk,jkm->rjm", X.double().abs().view(d_out, nb, d_block), Qd.abs()).reshape(d_out, d_in)
+    out = torch.empty_like(X)
+    Bd.armor_block_product(ctx.ctx, side, transpose, Q, X, out, 1.0, None, 0.0, 0)
+    assert ((out.double() - ref).abs() <= d_block * 2.0 ** -24 * mag + 1e-30).all()
+    Bd.armor_block_product(ctx.ctx, side, transpose, Q, X, out, -1.0, D, 1.0, 0)
+    assert ((out.double() - (D.double() - ref)).abs() <= (d_block + 2) * 2.0 ** -24 * (mag + D.double().abs())).all()
