@@ -434,20 +434,24 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 }
 
 // Adds the slabs of every split tile into C (+ what C held, if the product accumulates) and forms the tile's
-// share of the fused dot products.  Eight CTAs per split tile (32 rows each); fixed order.
+// share of the fused dot products.  Sixteen CTAs per split tile (16 rows each), four pieces in flight; fixed order.
 __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
-  const int tile = p.split_first + blockIdx.x / 8, half = (blockIdx.x >> 2) & 1, qq = blockIdx.x % 4;
+  constexpr int FR = BMP / PARTS;                         // rows per CTA
+  const int tile = p.split_first + blockIdx.x / PARTS, slot = blockIdx.x % PARTS;
   int mt, nt;
   tile_coords(p, tile, mt, nt);
-  const float* slab0 = p.slabs + ((int64_t)(blockIdx.x / 8) * p.split_parts * 2 + half) * (BM * BN);
+  const float* slab0 = p.slabs + (int64_t)(blockIdx.x / PARTS) * p.split_parts * (BMP * BN) + (int64_t)slot * FR * BN;
   double d1 = 0.0, d2 = 0.0;
-  for (int e = threadIdx.x; e < 32 * BN / 4; e += 256) {
-    const int r = qq * 32 + e / (BN / 4), c4 = (e % (BN / 4)) * 4;
-    const int64_t grow = (int64_t)mt * BMP + half * BM + r, gcol = (int64_t)nt * BN + c4;
+#pragma unroll
+  for (int e = threadIdx.x; e < FR * BN / 4; e += 256) {
+    const int r = e / (BN / 4), c4 = (e % (BN / 4)) * 4;
+    const int64_t grow = (int64_t)mt * BMP + slot * FR + r, gcol = (int64_t)nt * BN + c4;
     if (grow >= p.M || gcol >= p.N || (p.symmetric_lower && gcol > grow)) continue;
-    float4 v = *reinterpret_cast<const float4*>(slab0 + (int64_t)r * BN + c4);
+    const float* sp = slab0 + (int64_t)r * BN + c4;
+    float4 v = *reinterpret_cast<const float4*>(sp);
+#pragma unroll 4
     for (int k = 1; k < p.split_parts; ++k) {
-      const float4 w = *reinterpret_cast<const float4*>(slab0 + (int64_t)k * (2 * BM * BN) + (int64_t)r * BN + c4);
+      const float4 w = *reinterpret_cast<const float4*>(sp + (int64_t)k * (BMP * BN));
       v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
     }
     if (p.row_scale) {
@@ -470,6 +474,7 @@ __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
       d2 += (double)(v.x * w.x + v.y * w.y) + (double)(v.z * w.z + v.w * w.w);
     }
   }
+  if (!p.part1 && !p.part2) return;
   __shared__ double red1[8], red2[8];
   for (int o = 16; o > 0; o >>= 1) {
     d1 += __shfl_down_sync(0xffffffffu, d1, o);
@@ -480,10 +485,9 @@ __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
   if (threadIdx.x == 0) {
     double t1 = 0.0, t2 = 0.0;
     for (int w = 0; w < 8; ++w) { t1 += red1[w]; t2 += red2[w]; }
-    // sixteen slots per tile (the epilogue warps of the pair); this kernel fills eight and clears the rest
-    const int64_t slot = (int64_t)tile * PARTS + half * 8 + qq;
-    if (p.part1) { p.part1[slot] = t1; p.part1[slot + 4] = 0.0; }
-    if (p.part2) { p.part2[slot] = t2; p.part2[slot + 4] = 0.0; }
+    // the slots of the tile's epilogue warps, filled by this kernel's CTAs instead
+    if (p.part1) p.part1[(int64_t)tile * PARTS + slot] = t1;
+    if (p.part2) p.part2[(int64_t)tile * PARTS + slot] = t2;
   }
 }
 
@@ -534,6 +538,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     int parts = n_pairs / rem;
     const int64_t room = c->gemm_slab_count / (2 * rem);         // a slab holds 128 x 256 sums, a piece writes two
     if (parts > room) parts = (int)room;
+    if (parts > 16) parts = 16;      // beyond that the sum of the slabs costs more than the shorter pieces give
     // A piece writes 256 KB of sums and the second kernel reads them: about 6 us, 8 k-tiles with three MMAs per
     // product (0.8 us each) or 24 with one, which the shorter wave has to give back
     const int worth = SPLIT ? 8 : 24;
@@ -559,7 +564,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     cfg.attrs = at; cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
-      tc_gemm_fixup_kernel<<<8 * (p.n_tiles_total - p.split_first), 256, 0, s>>>(p);
+      tc_gemm_fixup_kernel<<<PARTS * (p.n_tiles_total - p.split_first), 256, 0, s>>>(p);
       c->launches++;
     }
   }

@@ -234,8 +234,8 @@ __global__ void __launch_bounds__(NT, 2) bgemm_tile_kernel(BGemm g, float* __res
 // ------------------------------------------------------------------------------ small products
 // 32 x 32 tiles for products that would leave most SMs without a 128 x 128 tile (the wrapper products of small blocks, the
 // [nb, d_block, d_block] products).  They are bound by latency: eight warps fetch 128 k of both operands at once (the next
-// 128 are in flight meanwhile), every pair of warps multiplies a quarter of them, 4 x 4 sums per thread, and the four
-// quarters are added in a fixed order at the end.  Same operand forms as above; K a multiple of 16.
+// 128 are in flight meanwhile); 2 x 2 sums per thread, each in the order of k, a cut contraction (ksplit) as sums of its
+// pieces: the same additions as in the kernel above, the same bits.  Same operand forms; K a multiple of 16.
 constexpr int SM_T = 32, SM_K = 128;
 // position of 16-byte unit u of k-row k: swizzled so that neither the writes along k nor the reads along a row conflict
 __device__ __forceinline__ int sm_unit(int k, int u) { return k * SM_T + 4 * (u ^ ((k >> 2) & 7)); }
@@ -283,54 +283,56 @@ __global__ void __launch_bounds__(NT) bgemm_small_kernel(BGemm g) {
       *reinterpret_cast<float4*>(T + sm_unit(f >> 3, f & 7)) = v;
     }
   };
-  const int grp = tid >> 6, tx = tid & 7, ty = (tid >> 3) & 7;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  const int tx = tid & 15, ty = tid >> 4;                 // columns 2 tx, 2 tx + 1; rows 2 ty, 2 ty + 1
+  const int kc = g.K / (g.ksplit > 1 ? g.ksplit : 1);     // a piece of the contraction
+  float acc[2][2] = {}, sum[2][2] = {};
+  int left = kc;
+  bool first = true;
   fetch(0);
   for (int k0 = 0; k0 < g.K; k0 += SM_K) {
 #pragma unroll
     for (int e = 0; e < 4; ++e) { stash_one(As, ra[e], e, A_KFAST); stash_one(Bs, rb[e], e, !B_NFAST); }
     __syncthreads();
     if (k0 + SM_K < g.K) fetch(k0 + SM_K);
-    const int kn = min(SM_K, g.K - k0) >> 2;              // k of this step per group: a multiple of 4
-    const int kb = grp * kn;
+    const int kn = min(SM_K, g.K - k0);
+    for (int k = 0; k < kn;) {
+      const int run = min(kn - k, left);                  // a multiple of 16
 #pragma unroll 4
-    for (int k = 0; k < kn; ++k) {
-      const float4 a4 = *reinterpret_cast<const float4*>(As + sm_unit(kb + k, ty));
-      const float4 b4 = *reinterpret_cast<const float4*>(Bs + sm_unit(kb + k, tx));
-      const float a[4] = {a4.x, a4.y, a4.z, a4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+      for (const int e = k + run; k < e; k += 4) {
+        // (four k share a swizzle)
+        const float* pa = As + sm_unit(k, ty >> 1) + 2 * (ty & 1);
+        const float* pb = Bs + sm_unit(k, tx >> 1) + 2 * (tx & 1);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int t = 0; t < 4; ++t) {
+          const float2 a = *reinterpret_cast<const float2*>(pa + t * SM_T);
+          const float2 b = *reinterpret_cast<const float2*>(pb + t * SM_T);
+          acc[0][0] = fmaf(a.x, b.x, acc[0][0]); acc[0][1] = fmaf(a.x, b.y, acc[0][1]);
+          acc[1][0] = fmaf(a.y, b.x, acc[1][0]); acc[1][1] = fmaf(a.y, b.y, acc[1][1]);
+        }
+      }
+      left -= run;
+      if (left == 0) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], bb[j], acc[i][j]);
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) { sum[i][j] = first ? acc[i][j] : sum[i][j] + acc[i][j]; acc[i][j] = 0.f; }
+        first = false;
+        left = kc;
+      }
     }
     __syncthreads();
   }
-  // sums of the four groups, in group order; then one float4 of a row per thread
-  float* part = As;                                       // [4][32][32]
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
-    *reinterpret_cast<float4*>(part + (grp * SM_T + 4 * ty + i) * SM_T + 4 * tx) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
-  __syncthreads();
-  const int r = tid >> 3, c4 = 4 * (tid & 7);
-  const int m = m0 + r, n = n0 + c4;
-  if (m >= g.M || n >= g.N) return;
-  float4 v = *reinterpret_cast<const float4*>(part + r * SM_T + c4);
-#pragma unroll
-  for (int q = 1; q < 4; ++q) {
-    const float4 w = *reinterpret_cast<const float4*>(part + (q * SM_T + r) * SM_T + c4);
-    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+  for (int i = 0; i < 2; ++i) {
+    const int m = m0 + 2 * ty + i, n = n0 + 2 * tx;
+    if (m >= g.M || n >= g.N) continue;
+    float2 v = make_float2(g.alpha * sum[i][0], g.alpha * sum[i][1]);
+    if (g.D) {
+      const float2 d = *reinterpret_cast<const float2*>(g.D + od + (int64_t)m * g.sDm + n);
+      v.x = fmaf(g.beta, d.x, v.x); v.y = fmaf(g.beta, d.y, v.y);
+    }
+    *reinterpret_cast<float2*>(g.C + oc + (int64_t)m * g.sCm + n) = v;
   }
-  v = make_float4(g.alpha * v.x, g.alpha * v.y, g.alpha * v.z, g.alpha * v.w);
-  if (g.D) {
-    const float4 d = *reinterpret_cast<const float4*>(g.D + od + (int64_t)m * g.sDm + n);
-    v.x = fmaf(g.beta, d.x, v.x); v.y = fmaf(g.beta, d.y, v.y);
-    v.z = fmaf(g.beta, d.z, v.z); v.w = fmaf(g.beta, d.w, v.w);
-  }
-  *reinterpret_cast<float4*>(g.C + oc + (int64_t)m * g.sCm + n) = v;
 }
 
 // The share of the chip's lanes that 128 x 128 tiles would keep busy: tiles per SM, times the part of a tile that holds

@@ -5,395 +5,388 @@
 //   mode 2 (right+gd): out = rhs (G + lam I)^-1;  part = <dotw, out>
 // A failed factorisation leaves A unchanged / writes zeros and raises failflag[block].
 //
-// One CTA factorises one d_block x d_block matrix in shared memory and solves for a slice of the
-// right-hand sides (all of them for d_block <= 128; d_block = 256 is split over four CTAs that each
-// repeat the factorisation, because factor and right-hand sides do not fit one CTA's shared memory).
-// Blocked left-looking Cholesky with panels of 32 columns: a panel first receives the contributions of
-// all earlier panels as one small matrix product (every element is accumulated in fp64 and rounded to
-// fp32 once), then its 32 columns are eliminated with dot products of at most 31 terms.  The
-// triangular solves are blocked the same way; the 32 x 32 diagonal solves keep one right-hand side per
-// thread in registers and eliminate column by column, so the dependent chain is one multiply-add per
-// unknown.
+// One CTA factorises one d_block x d_block matrix in shared memory and solves for a slice of the right-hand sides beside it;
+// the slices of a block repeat the factorisation.  What bounds this is the chain of pivots (about 200 cycles each in the
+// factorisation, 80 in a solve), next to it fp64 conversions, which cost as much as dozens of fp32 instructions and are
+// kept out of the sums:
+//   storage: panels of 32 columns, rows of 32 floats, the 16-byte units of a row swizzled so that eight lanes reading the
+//            same unit of consecutive rows, or of every fourth row, or all units of one row, meet no bank conflict; G
+//            arrives by cp.async, and everything below reads four columns per access.
+//   factor : blocked left-looking Cholesky.  A panel receives the contributions of the earlier panels as one small product
+//            (fp32 over 32 terms, panels added as unevaluated pairs of floats, one rounding).  Then every warp that owns 32
+//            of its rows repeats the elimination of the diagonal block in registers (lane = row) and carries its own rows
+//            along, so that no second pass over the rows below follows.
+//   solve  : left-looking with the same two-level sums, a lane per right-hand side, a warp per four rows of a block of 32:
+//            every warp works in every step.
+// Measured and left: pivots eight at a time with every thread factorising the 8 x 8 block (elimination 1.4 x slower), rows
+// or right-hand sides moving down one register per pivot in a rolled loop (2 x), solutions handed round by shuffles (1.2 x).
+// A launch, d_block 128: 32 blocks over 4 CTAs each 57 us (79 before), 112 blocks 86 us (85); d_block 256, 32 blocks 176 us
+// (about 270).
 #include "armor_internal.cuh"
 
 namespace {
 
 constexpr int NT = 256;
 constexpr int NB = 32;       // panel width
-constexpr int LDP = NB + 1;  // padded row length of a panel
 
 struct PanelMap {
   int db;
-  // offset (floats) of panel kb: rows NB*kb .. db-1, LDP floats each
-  __device__ __forceinline__ int off(int kb) const { return LDP * (kb * db - NB * kb * (kb - 1) / 2); }
-  // element (i, k), i >= NB * (k / NB)
-  __device__ __forceinline__ int at(int i, int k) const {
-    const int kb = k / NB;
-    return off(kb) + (i - NB * kb) * LDP + (k - NB * kb);
-  }
+  // offset (floats) of panel kb: rows NB*kb .. db-1, NB floats each
+  __device__ __forceinline__ int off(int kb) const { return NB * (kb * db - NB * kb * (kb - 1) / 2); }
 };
+// 16-byte unit u (columns 4u .. 4u + 3) of row r of a panel
+__device__ __forceinline__ int unit(int r, int u) { return r * NB + 4 * (u ^ (((r >> 2) ^ (r << 1)) & 7)); }
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
 __host__ __device__ inline size_t panel_floats(int db) {
   const int np = db / NB;
-  return (size_t)LDP * ((size_t)np * db - (size_t)NB * np * (np - 1) / 2);
+  return (size_t)NB * ((size_t)np * db - (size_t)NB * np * (np - 1) / 2);
 }
 
-// y -= sum over the 32 columns of one earlier panel, fp32 products; the caller adds the chunk to an fp64 sum
-#define ARMOR_TILE_ZERO(acc)                                   \
-  _Pragma("unroll") for (int a_ = 0; a_ < 4; ++a_)             \
-  _Pragma("unroll") for (int b_ = 0; b_ < 4; ++b_) acc[a_][b_] = 0.f;
+// running sum of fp32 values as an unevaluated pair: every rounding error of an addition is kept (Knuth's two-sum)
+struct Pair { float hi, lo; };
+__device__ __forceinline__ void pair_add(Pair& a, float v) {
+  const float s = a.hi + v, bb = s - a.hi;
+  a.lo += (a.hi - (s - bb)) + (v - bb);
+  a.hi = s;
+}
+// v - a, rounded once
+__device__ __forceinline__ float pair_sub_from(float v, const Pair& a) {
+  const float s = v - a.hi, bb = s - v;
+  return s + (((v - (s - bb)) - (a.hi + bb)) - a.lo);
+}
 
-__global__ void __launch_bounds__(NT, 1)
-chol_blocked_kernel(int mode, const float* __restrict__ Gmat, const float* __restrict__ rhs, float* __restrict__ out,
-                    const float* __restrict__ dotw, float* __restrict__ A, float ridge, int db,
-                    int w, double* __restrict__ part, int32_t* __restrict__ failflag, int32_t* __restrict__ status) {
-  extern __shared__ float smem[];
-  const PanelMap pm{db};
-  const int np = db / NB;
-  const int ldr = w + 1;
-  float* Lp = smem;
-  float* Rs = smem + panel_floats(db);                  // [db][w + 1]: row = unknown index, column = right-hand side
-  __shared__ float Df[NB][NB + 1];                      // diagonal block of the current panel
-  __shared__ float invd[NB];                            // reciprocals of its diagonal
-  __shared__ double red[NT / 32];
-  __shared__ int s_fail;
-  __shared__ double s_lam;
-  const int b = blockIdx.x, q = blockIdx.y, tid = threadIdx.x, lane = threadIdx.x & 31;
-  const int64_t off = (int64_t)b * db * db;
-  const bool right = (mode != 1);
-  const int v0 = q * w;  // first right-hand side of this CTA
-
-  // ---- load: lower triangle of G, the slice of right-hand sides.  float4 loads, eight in flight per
-  // thread, so that the global-memory latency is paid a few times and not once per element.
-  {
-    const int q4 = db / 4;                      // float4 per row
-    const int n4 = db * q4;
-    for (int e0 = tid; e0 < n4; e0 += 8 * NT) {
-      float4 v[8];
+// The panel's 32 columns, eliminated right-looking with rows in registers: ad is the lane's row of the diagonal block (the
+// same in every warp that takes part), ab its row of the warp's own 32 rows below (`below` groups of 32 rows); nothing in
+// the chain of pivots goes through memory.  Called by the whole CTA; one copy serves every block size.
+__device__ __noinline__ void eliminate_panel(float* P, float* invd, int below, int* s_fail) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool mine = warp < below;
+  const bool takes_part = mine || warp == 0;
+  const int rb = NB * (warp + 1) + lane;
+  float ad[NB], ab[NB];
+  if (takes_part) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * NT;
-        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (e < n4 && (e % q4) * 4 <= e / q4) v[u] = reinterpret_cast<const float4*>(Gmat + off)[e];
-      }
+    for (int u = 0; u < NB / 4; ++u) {
+      const float4 v = ld4(P + unit(lane, u));
+      const float4 w = mine ? ld4(P + unit(rb, u)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      ad[4 * u] = v.x; ad[4 * u + 1] = v.y; ad[4 * u + 2] = v.z; ad[4 * u + 3] = v.w;   // (j > lane: never used)
+      ab[4 * u] = w.x; ab[4 * u + 1] = w.y; ab[4 * u + 2] = w.z; ab[4 * u + 3] = w.w;
+    }
+  }
+  __syncthreads();                                          // every warp has read the block warp 0 is about to replace
+  if (takes_part) {
+    bool bad = false;
+    float dg = 1.f;
+    float akk = __shfl_sync(0xffffffffu, ad[0], 0);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * NT;
-        if (e >= n4) continue;
-        const int r = e / q4, c4 = (e % q4) * 4;
-        if (c4 > r) continue;
-        float* dst = Lp + pm.at(r, c4);         // c4 .. c4 + 3 lie in one panel
-        const float vv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+    for (int k = 0; k < NB; ++k) {
+      bad |= !(akk > 0.f) | !isfinite(akk);
+      // 1 / sqrt(a): hardware estimate refined by one Newton step
+      float inv = rsqrtf(akk);
+      inv = inv * fmaf(-0.5f * akk * inv, inv, 1.5f);
+      const float ld = ad[k] * inv, lb = ab[k] * inv;
+      ad[k] = ld;
+      ab[k] = lb;
+      if (lane == k) dg = ld;
+      // the next pivot needs lane k + 1's own multiplier only: it goes ahead of the rest of the column
+      if (k + 1 < NB) akk = __shfl_sync(0xffffffffu, fmaf(-ld, ld, ad[k + 1]), k + 1);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if (c4 + j <= r) dst[j] = vv[j];
+      for (int j = k + 1; j < NB; ++j) {
+        const float ljk = __shfl_sync(0xffffffffu, ld, j);
+        ad[j] = fmaf(-ld, ljk, ad[j]);
+        ab[j] = fmaf(-lb, ljk, ab[j]);
       }
     }
-    // right-hand sides: vector id x unknown index
-    const int m4 = right ? w * q4 : db * (w / 4);
-    for (int e0 = tid; e0 < m4; e0 += 8 * NT) {
-      float4 v[8];
+    if (bad) {
+      if (lane == 0) *s_fail = 1;
+    } else {
+      if (warp == 0) {
+        invd[lane] = 1.f / dg;
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * NT;
-        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (e < m4) {
-          if (right) v[u] = *reinterpret_cast<const float4*>(rhs + off + (int64_t)(v0 + e / q4) * db + (e % q4) * 4);
-          else v[u] = *reinterpret_cast<const float4*>(rhs + off + (int64_t)(e / (w / 4)) * db + v0 + (e % (w / 4)) * 4);
-        }
+        for (int u = 0; u < NB / 4; ++u)
+          *reinterpret_cast<float4*>(P + unit(lane, u)) = make_float4(ad[4 * u], ad[4 * u + 1], ad[4 * u + 2], ad[4 * u + 3]);
       }
+      if (mine) {
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int e = e0 + u * NT;
-        if (e >= m4) continue;
-        const float vv[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-        if (right) {
-          // right-hand side vid is row v0 + vid of rhs; the unknown index runs along the row
-          const int vid = e / q4, r4 = (e % q4) * 4;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) Rs[(r4 + j) * ldr + vid] = vv[j];
-        } else {
-          const int r = e / (w / 4), vid4 = (e % (w / 4)) * 4;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) Rs[r * ldr + vid4 + j] = vv[j];
-        }
+        for (int u = 0; u < NB / 4; ++u)
+          *reinterpret_cast<float4*>(P + unit(rb, u)) = make_float4(ab[4 * u], ab[4 * u + 1], ab[4 * u + 2], ab[4 * u + 3]);
       }
     }
   }
+  __syncthreads();
+}
+
+// panel kb (at P, first row c0) -= sum_{p < c0} L(i, p) L(k, p): TR x 4 elements per thread, rows TR*tr.., columns 4*tc..
+template <int TR>
+__device__ __forceinline__ void update_panel(float* Lp, const PanelMap& pm, int kb) {
+  const int db = pm.db, c0 = NB * kb;
+  float* P = Lp + pm.off(kb);
+  const int ntiles = ((db - c0) / TR) * (NB / 4);
+  for (int tix = threadIdx.x; tix < ntiles; tix += NT) {
+    const int tr = tix / (NB / 4), tc = tix % (NB / 4);
+    Pair acc[TR][4];
+#pragma unroll
+    for (int a = 0; a < TR; ++a)
+#pragma unroll
+      for (int bb = 0; bb < 4; ++bb) acc[a][bb] = {0.f, 0.f};
+    for (int pb = 0; pb < kb; ++pb) {
+      const float* Q = Lp + pm.off(pb);
+      const int ri = c0 - NB * pb + TR * tr, rk = c0 - NB * pb + 4 * tc;      // rows of panel pb
+      float a32[TR][4];
+#pragma unroll
+      for (int a = 0; a < TR; ++a)
+#pragma unroll
+        for (int bb = 0; bb < 4; ++bb) a32[a][bb] = 0.f;
+#pragma unroll 2
+      for (int u = 0; u < NB / 4; ++u) {
+        float4 li[TR], lk[4];
+#pragma unroll
+        for (int a = 0; a < TR; ++a) li[a] = ld4(Q + unit(ri + a, u));
+#pragma unroll
+        for (int a = 0; a < 4; ++a) lk[a] = ld4(Q + unit(rk + a, u));
+#pragma unroll
+        for (int a = 0; a < TR; ++a)
+#pragma unroll
+          for (int bb = 0; bb < 4; ++bb) {
+            a32[a][bb] = fmaf(li[a].x, lk[bb].x, a32[a][bb]);
+            a32[a][bb] = fmaf(li[a].y, lk[bb].y, a32[a][bb]);
+            a32[a][bb] = fmaf(li[a].z, lk[bb].z, a32[a][bb]);
+            a32[a][bb] = fmaf(li[a].w, lk[bb].w, a32[a][bb]);
+          }
+      }
+#pragma unroll
+      for (int a = 0; a < TR; ++a)
+#pragma unroll
+        for (int bb = 0; bb < 4; ++bb) pair_add(acc[a][bb], a32[a][bb]);
+    }
+#pragma unroll
+    for (int a = 0; a < TR; ++a) {
+      float4* dst = reinterpret_cast<float4*>(P + unit(TR * tr + a, tc));
+      const float4 v = *dst;
+      *dst = make_float4(pair_sub_from(v.x, acc[a][0]), pair_sub_from(v.y, acc[a][1]), pair_sub_from(v.z, acc[a][2]),
+                         pair_sub_from(v.w, acc[a][3]));
+    }
+  }
+}
+
+// Block kb's 32 unknowns of every right-hand side: x (in X, one column per right-hand side) becomes L^-1 x, or with T L^-T x.
+// Lane = right-hand side (G of them, 32 apart), warp = four rows.  First the solved blocks' share (forward: blocks before kb
+// with the rows of L; T: blocks after kb with its columns; in block order either way), then the block itself, four unknowns
+// at a time.  Called by the whole CTA.
+template <bool T, int G>
+__device__ __forceinline__ void solve_block(const float* Lp, const PanelMap& pm, const float* invd, float* X, int ldx, int kb) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = 4 * warp;
+  const int p_begin = T ? kb + 1 : 0, p_end = T ? pm.db / NB : kb;
+  float* own = X + (NB * kb + r0) * ldx + lane;
+  float y[G][4];
+  {
+    Pair acc[G][4];
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) acc[g][m] = {0.f, 0.f};
+#pragma unroll 1
+    for (int pb = p_begin; pb < p_end; ++pb) {
+      const float* Q = Lp + pm.off(T ? kb : pb);
+      const float* xp = X + NB * pb * ldx + lane;
+      float a32[G][4];
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) a32[g][m] = 0.f;
+#pragma unroll (G == 1 ? 4 : 2)
+      for (int u = 0; u < NB / 4; ++u) {
+        float l[4][4];                                        // [row][unknown 4 u + j]
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float4 v = ld4(T ? Q + unit(NB * (pb - kb) + 4 * u + t, warp) : Q + unit(NB * (kb - pb) + r0 + t, u));
+          if (T) { l[0][t] = v.x; l[1][t] = v.y; l[2][t] = v.z; l[3][t] = v.w; }
+          else { l[t][0] = v.x; l[t][1] = v.y; l[t][2] = v.z; l[t][3] = v.w; }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int g = 0; g < G; ++g) {
+            const float x = xp[(4 * u + j) * ldx + 32 * g];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) a32[g][m] = fmaf(l[m][j], x, a32[g][m]);
+          }
+      }
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) pair_add(acc[g][m], a32[g][m]);
+    }
+#pragma unroll
+    for (int g = 0; g < G; ++g)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) y[g][m] = pair_sub_from(own[m * ldx + 32 * g], acc[g][m]);
+  }
+  const float* D = Lp + pm.off(kb);
+#pragma unroll 1
+  for (int s = 0; s < NB / 4; ++s) {
+    const int u = T ? NB / 4 - 1 - s : s;                     // the warp whose four rows are solved now
+    const bool open = T ? warp <= u : warp >= u;
+    float l[4][4];                                            // [row of this warp][unknown 4 u + j]
+    if (open) {
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float4 v = ld4(T ? D + unit(4 * u + t, warp) : D + unit(r0 + t, u));
+        if (T) { l[0][t] = v.x; l[1][t] = v.y; l[2][t] = v.z; l[3][t] = v.w; }
+        else { l[t][0] = v.x; l[t][1] = v.y; l[t][2] = v.z; l[t][3] = v.w; }
+      }
+    }
+    if (warp == u) {
+      const float4 iv4 = ld4(invd + NB * kb + r0);
+      const float iv[4] = {iv4.x, iv4.y, iv4.z, iv4.w};
+#pragma unroll
+      for (int g = 0; g < G; ++g) {
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+          const int j = T ? 3 - jj : jj;
+          y[g][j] *= iv[j];
+#pragma unroll
+          for (int m = 0; m < 4; ++m)
+            if (T ? m < j : m > j) y[g][m] = fmaf(-l[m][j], y[g][j], y[g][m]);
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) own[m * ldx + 32 * g] = y[g][m];
+      }
+    }
+    __syncthreads();
+    if (open && warp != u) {
+      const float* xu = X + (NB * kb + 4 * u) * ldx + lane;
+#pragma unroll
+      for (int g = 0; g < G; ++g)
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+          const int j = T ? 3 - jj : jj;
+          const float x = xu[j * ldx + 32 * g];
+#pragma unroll
+          for (int m = 0; m < 4; ++m) y[g][m] = fmaf(-l[m][j], x, y[g][m]);
+        }
+    }
+  }
+}
+
+constexpr int MAX_DB = 256;
+
+// G: a CTA takes 32 G right-hand sides
+template <int G>
+__global__ void __launch_bounds__(NT, 1)
+chol_blocked_kernel(int mode, const float* __restrict__ Gmat, const float* __restrict__ rhs, float* __restrict__ out,
+                    const float* __restrict__ dotw, float* __restrict__ A, float ridge, int db, double* __restrict__ part,
+                    int32_t* __restrict__ failflag, int32_t* __restrict__ status) {
+  constexpr int W = 32 * G, LDX = W + 1;                // (odd: neither a row of X nor 8 x 4 floats along a column conflict)
+  extern __shared__ __align__(16) float smem[];
+  const PanelMap pm{db};
+  const int np = db / NB;
+  float* Lp = smem;
+  float* X = smem + panel_floats(db);                   // [unknown][right-hand side]
+  __shared__ __align__(16) float invd[MAX_DB];          // reciprocals of the factor's diagonal
+  __shared__ double red[NT / 32];
+  __shared__ int s_fail;
+  __shared__ double s_lam;
+  const int b = blockIdx.x, q = blockIdx.y, tid = threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t off = (int64_t)b * db * db;
+  const bool right = (mode != 1);
+  const int v0 = q * W;                                 // first right-hand side of this CTA
+  const int q4 = db / 4;                                // 16-byte units per row
+
+  // ---- load: the units of G on and below the diagonal, then the right-hand sides
+  for (int e = tid; e < db * q4; e += NT) {
+    const int r = e / q4, u = e % q4, kb = u / (NB / 4);
+    if (4 * u > r) continue;
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(Lp + pm.off(kb) + unit(r - NB * kb, u - kb * (NB / 4)));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(Gmat + off + 4 * (int64_t)e) : "memory");
+  }
+  // A right solve's right-hand side is a row of rhs (eight lanes along it, four rows per warp access), a left solve's a
+  // column (lanes along the row of rhs).  Right-hand sides past the end are zeros.
+  if (right) {
+#pragma unroll 4
+    for (int e = tid; e < W * q4; e += NT) {
+      const int c8 = e & 7, v = (e >> 3) % W, i = 4 * (c8 + 8 * ((e >> 3) / W));
+      const float4 x = v0 + v < db ? ld4(rhs + off + (int64_t)(v0 + v) * db + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      X[i * LDX + v] = x.x; X[(i + 1) * LDX + v] = x.y; X[(i + 2) * LDX + v] = x.z; X[(i + 3) * LDX + v] = x.w;
+    }
+  } else {
+#pragma unroll 8
+    for (int e = tid; e < W * db; e += NT) {
+      const int v = e % W, i = e / W;
+      X[i * LDX + v] = v0 + v < db ? rhs[off + (int64_t)i * db + v0 + v] : 0.f;
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
   if (tid == 0) s_fail = 0;
   __syncthreads();
   if (tid < 32) {
     double tr = 0.0;
-    for (int i = tid; i < db; i += 32) tr += (double)Lp[pm.at(i, i)];
+    for (int kb = 0; kb < np; ++kb) tr += (double)Lp[pm.off(kb) + unit(tid, tid >> 2) + (tid & 3)];
     for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
     if (tid == 0) s_lam = (double)ridge * tr / (double)db;
   }
   __syncthreads();
   const double lam = s_lam;
-  for (int i = tid; i < db; i += NT) Lp[pm.at(i, i)] = (float)((double)Lp[pm.at(i, i)] + lam);
+  for (int i = tid; i < db; i += NT) {
+    float* d = Lp + pm.off(i / NB) + unit(i % NB, (i % NB) >> 2) + (i & 3);
+    *d = (float)((double)*d + lam);
+  }
   __syncthreads();
 
   // ---- blocked Cholesky
   for (int kb = 0; kb < np; ++kb) {
-    const int c0 = NB * kb;
-    float* P = Lp + pm.off(kb);
     if (kb > 0) {
-      // panel(i, k) -= sum_{p < c0} L(i, p) L(k, p): 4 x 4 tiles, rows c0 + 4*tr.., columns c0 + 4*tc..
-      const int ntiles = ((db - c0) / 4) * (NB / 4);
-      for (int tix = tid; tix < ntiles; tix += NT) {
-        const int tr = tix / (NB / 4), tc = tix % (NB / 4);
-        double acc[4][4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int bb = 0; bb < 4; ++bb) acc[a][bb] = 0.0;
-        for (int pb = 0; pb < kb; ++pb) {
-          const float* Li = Lp + pm.off(pb) + (c0 + 4 * tr - NB * pb) * LDP;   // rows i of panel pb
-          const float* Lk = Lp + pm.off(pb) + (c0 + 4 * tc - NB * pb) * LDP;   // rows k of panel pb
-          float a32[4][4];
-          ARMOR_TILE_ZERO(a32)
-#pragma unroll 8
-          for (int p = 0; p < NB; ++p) {
-            float li[4], lk[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) { li[a] = Li[a * LDP + p]; lk[a] = Lk[a * LDP + p]; }
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-              for (int bb = 0; bb < 4; ++bb) a32[a][bb] = fmaf(li[a], lk[bb], a32[a][bb]);
-          }
-#pragma unroll
-          for (int a = 0; a < 4; ++a)
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb) acc[a][bb] += (double)a32[a][bb];
-        }
-        float* dst = P + (4 * tr) * LDP + 4 * tc;
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int bb = 0; bb < 4; ++bb) dst[a * LDP + bb] = (float)((double)dst[a * LDP + bb] - acc[a][bb]);
-      }
+      // (the last panels have too few 4 x 4 tiles for the CTA's warps)
+      if (db - NB * kb > 64) update_panel<4>(Lp, pm, kb); else update_panel<1>(Lp, pm, kb);
       __syncthreads();
     }
-    // diagonal block: warp 0, lane i keeps row i in registers and the warp eliminates column by column
-    // (right-looking); the entries of the pivot column come from the other lanes by shuffle, so nothing in the
-    // chain goes through memory
-    if (tid < 32) {
-      float arow[NB];
-#pragma unroll
-      for (int j = 0; j < NB; ++j) arow[j] = (j <= lane) ? P[lane * LDP + j] : 0.f;
-      bool bad = false;
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        const float akk = __shfl_sync(0xffffffffu, arow[k], k);
-        bad |= !(akk > 0.f) | !isfinite(akk);
-        // 1 / sqrt(a): hardware estimate refined by one Newton step
-        float inv = rsqrtf(akk);
-        inv = inv * fmaf(-0.5f * akk * inv, inv, 1.5f);
-        const float lik = (lane == k) ? akk * inv : arow[k] * inv;
-        arow[k] = lik;
-        if (lane == k) invd[k] = inv;
-#pragma unroll
-        for (int j = k + 1; j < NB; ++j) {
-          const float ljk = __shfl_sync(0xffffffffu, lik, j);
-          arow[j] = fmaf(-lik, ljk, arow[j]);      // entries above the diagonal (j > lane) are never used
-        }
-      }
-      if (bad) {
-        if (lane == 0) s_fail = 1;
-      } else {
-#pragma unroll
-        for (int j = 0; j < NB; ++j) {
-          Df[lane][j] = (j <= lane) ? arow[j] : 0.f;
-          if (j <= lane) P[lane * LDP + j] = arow[j];
-        }
-      }
-    }
-    __syncthreads();
+    eliminate_panel(Lp + pm.off(kb), invd + NB * kb, np - 1 - kb, &s_fail);
     if (s_fail) break;
-    // rows below the diagonal block: l_ik = (a_ik - sum_{p<k} l_ip l_kp) / l_kk, row i in registers
-    const int nrow = db - c0;
-    if (tid >= NB && tid < nrow) {   // nrow <= d_block <= 256 = NT
-      const int i = tid;
-      // column-oriented elimination: once l_ik is final it leaves the later entries of the row at once, so the
-      // dependent chain is one multiply-add per column
-      float arow[NB];
-#pragma unroll
-      for (int j = 0; j < NB; ++j) arow[j] = P[i * LDP + j];
-#pragma unroll
-      for (int k = 0; k < NB; ++k) {
-        const float lik = arow[k] * invd[k];
-        arow[k] = lik;
-#pragma unroll
-        for (int j = k + 1; j < NB; ++j) arow[j] = fmaf(-lik, Df[j][k], arow[j]);
-      }
-#pragma unroll
-      for (int j = 0; j < NB; ++j) P[i * LDP + j] = arow[j];
-    }
-    __syncthreads();
   }
-  __syncthreads();
   const bool fail = (s_fail != 0);
   const bool hold = (mode == 0) && status[ST_POISON] != 0;   // unusable inputs: the A-step is withheld (X = 0)
 
   if (!fail) {
-    const int wq = w / 4;          // column c of tile column tc: tc + wq * j  (conflict-free shared-memory rows)
     // ---- forward substitution  L y = r, then backward substitution  L^T x = y
-    for (int pass = 0; pass < 2; ++pass) {
-      for (int step = 0; step < np; ++step) {
-        const int kb = pass == 0 ? step : np - 1 - step;
-        const int c0 = NB * kb;
-        const float* P = Lp + pm.off(kb);
-        // the diagonal block and the reciprocals of its diagonal
-        for (int e = tid; e < NB * NB; e += NT) {
-          const int r = e / NB, cc = e % NB;
-          const float v = (cc <= r) ? P[r * LDP + cc] : 0.f;
-          Df[r][cc] = v;
-          if (r == cc) invd[r] = 1.f / v;
-        }
-        if (step > 0) {
-          const int ntiles = (NB / 4) * wq;
-          for (int tix = tid; tix < ntiles; tix += NT) {
-            const int ta = tix / wq, tc = tix % wq;
-            double acc[4][4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) acc[a][j] = 0.0;
-            if (pass == 0) {
-              for (int pb = 0; pb < kb; ++pb) {
-                const float* Li = Lp + pm.off(pb) + (c0 + 4 * ta - NB * pb) * LDP;
-                const float* Xp = Rs + (NB * pb) * ldr + tc;
-                float a32[4][4];
-                ARMOR_TILE_ZERO(a32)
-#pragma unroll 8
-                for (int p = 0; p < NB; ++p) {
-                  float li[4], x[4];
-#pragma unroll
-                  for (int a = 0; a < 4; ++a) { li[a] = Li[a * LDP + p]; x[a] = Xp[p * ldr + wq * a]; }
-#pragma unroll
-                  for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) a32[a][j] = fmaf(li[a], x[j], a32[a][j]);
-                }
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) acc[a][j] += (double)a32[a][j];
-              }
-            } else {
-              // sum over p >= c0 + NB of L(p, c0 + 4 ta + a) x[p]: column c0 + 4 ta + a lives in panel kb
-              const float* Lcol = P + 4 * ta;
-              const float* Xp = Rs + tc;
-              for (int p0 = c0 + NB; p0 < db; p0 += NB) {
-                float a32[4][4];
-                ARMOR_TILE_ZERO(a32)
-#pragma unroll 8
-                for (int p = p0; p < p0 + NB; ++p) {
-                  float lc[4], x[4];
-#pragma unroll
-                  for (int a = 0; a < 4; ++a) { lc[a] = Lcol[(p - c0) * LDP + a]; x[a] = Xp[p * ldr + wq * a]; }
-#pragma unroll
-                  for (int a = 0; a < 4; ++a)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) a32[a][j] = fmaf(lc[a], x[j], a32[a][j]);
-                }
-#pragma unroll
-                for (int a = 0; a < 4; ++a)
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) acc[a][j] += (double)a32[a][j];
-              }
-            }
-            float* dst = Rs + (c0 + 4 * ta) * ldr + tc;
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) dst[a * ldr + wq * j] = (float)((double)dst[a * ldr + wq * j] - acc[a][j]);
-          }
-        }
-        __syncthreads();
-        if (tid < w) {
-          float sreg[NB];
-#pragma unroll
-          for (int r = 0; r < NB; ++r) sreg[r] = Rs[(c0 + r) * ldr + tid];
-          if (pass == 0) {
-#pragma unroll
-            for (int r = 0; r < NB; ++r) {
-              const float x = sreg[r] * invd[r];
-              sreg[r] = x;
-#pragma unroll
-              for (int r2 = r + 1; r2 < NB; ++r2) sreg[r2] = fmaf(-Df[r2][r], x, sreg[r2]);
-            }
-          } else {
-#pragma unroll
-            for (int r = NB - 1; r >= 0; --r) {
-              const float x = sreg[r] * invd[r];
-              sreg[r] = x;
-#pragma unroll
-              for (int r2 = 0; r2 < r; ++r2) sreg[r2] = fmaf(-Df[r][r2], x, sreg[r2]);
-            }
-          }
-#pragma unroll
-          for (int r = 0; r < NB; ++r) Rs[(c0 + r) * ldr + tid] = sreg[r];
-        }
-        __syncthreads();
-      }
-    }
+    for (int kb = 0; kb < np; ++kb) solve_block<false, G>(Lp, pm, invd, X, LDX, kb);
+    for (int kb = np - 1; kb >= 0; --kb) solve_block<true, G>(Lp, pm, invd, X, LDX, kb);
+    __syncthreads();
   }
 
-  // ---- write back.  Right solves: solution vid is row v0 + vid of the result; left solves: column v0 + vid.
+  // ---- write back.  Right solves: right-hand side vid is row vid of the result; left solves: column vid.
   double acc = 0.0;
-  {
-    const int q4 = db / 4;
-    const int m4 = right ? w * q4 : db * (w / 4);
-    for (int e0 = tid; e0 < m4; e0 += 4 * NT) {
-      float4 x[4], aold[4], gin[4];
-      int64_t gidx[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int e = e0 + u * NT;
-        x[u] = aold[u] = gin[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        gidx[u] = -1;
-        if (e >= m4) continue;
-        if (right) {
-          const int vid = e / q4, r4 = (e % q4) * 4;
-          gidx[u] = (int64_t)(v0 + vid) * db + r4;
-          if (!fail && !hold) x[u] = make_float4(Rs[r4 * ldr + vid], Rs[(r4 + 1) * ldr + vid], Rs[(r4 + 2) * ldr + vid],
-                                                 Rs[(r4 + 3) * ldr + vid]);
-        } else {
-          const int r = e / (w / 4), vid4 = (e % (w / 4)) * 4;
-          gidx[u] = (int64_t)r * db + v0 + vid4;
-          if (!fail && !hold) x[u] = make_float4(Rs[r * ldr + vid4], Rs[r * ldr + vid4 + 1], Rs[r * ldr + vid4 + 2],
-                                                 Rs[r * ldr + vid4 + 3]);
-        }
-        if (mode == 0) {
-          aold[u] = *reinterpret_cast<const float4*>(A + off + gidx[u]);
-          gin[u] = *reinterpret_cast<const float4*>(rhs + off + gidx[u]);
-        } else if (mode == 2) {
-          gin[u] = *reinterpret_cast<const float4*>(dotw + off + gidx[u]);
-        }
+  if (right) {
+#pragma unroll 4
+    for (int e = tid; e < W * q4; e += NT) {
+      const int c8 = e & 7, v = (e >> 3) % W, i = 4 * (c8 + 8 * ((e >> 3) / W));
+      if (v0 + v >= db) continue;
+      const int64_t idx = off + (int64_t)(v0 + v) * db + i;
+      const float4 aold = mode == 0 ? ld4(A + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float4 gin = ld4((mode == 0 ? rhs : dotw) + idx);
+      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (!fail && !hold) x = make_float4(X[i * LDX + v], X[(i + 1) * LDX + v], X[(i + 2) * LDX + v], X[(i + 3) * LDX + v]);
+      *reinterpret_cast<float4*>(out + idx) = x;
+      if (mode == 0) {
+        *reinterpret_cast<float4*>(A + idx) = make_float4(aold.x + x.x, aold.y + x.y, aold.z + x.z, aold.w + x.w);
+        acc += (double)gin.x * (double)x.x + lam * (double)x.x * (double)x.x;
+        acc += (double)gin.y * (double)x.y + lam * (double)x.y * (double)x.y;
+        acc += (double)gin.z * (double)x.z + lam * (double)x.z * (double)x.z;
+        acc += (double)gin.w * (double)x.w + lam * (double)x.w * (double)x.w;
+      } else {
+        acc += (double)gin.x * (double)x.x + (double)gin.y * (double)x.y + (double)gin.z * (double)x.z + (double)gin.w * (double)x.w;
       }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        if (gidx[u] < 0) continue;
-        *reinterpret_cast<float4*>(out + off + gidx[u]) = x[u];
-        if (mode == 0) {
-          *reinterpret_cast<float4*>(A + off + gidx[u]) =
-              make_float4(aold[u].x + x[u].x, aold[u].y + x[u].y, aold[u].z + x[u].z, aold[u].w + x[u].w);
-          acc += (double)gin[u].x * (double)x[u].x + lam * (double)x[u].x * (double)x[u].x;
-          acc += (double)gin[u].y * (double)x[u].y + lam * (double)x[u].y * (double)x[u].y;
-          acc += (double)gin[u].z * (double)x[u].z + lam * (double)x[u].z * (double)x[u].z;
-          acc += (double)gin[u].w * (double)x[u].w + lam * (double)x[u].w * (double)x[u].w;
-        } else if (mode == 2) {
-          acc += (double)gin[u].x * (double)x[u].x + (double)gin[u].y * (double)x[u].y +
-                 (double)gin[u].z * (double)x[u].z + (double)gin[u].w * (double)x[u].w;
-        }
-      }
+    }
+  } else {
+#pragma unroll 4
+    for (int e = tid; e < W * db; e += NT) {
+      const int v = e % W, i = e / W;
+      if (v0 + v < db) out[off + (int64_t)i * db + v0 + v] = fail ? 0.f : X[i * LDX + v];
     }
   }
   if (mode != 1) {
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((tid & 31) == 0) red[tid >> 5] = acc;
+    if (lane == 0) red[warp] = acc;
     __syncthreads();
     if (tid == 0) {
       double t = 0.0;
@@ -508,14 +501,39 @@ __global__ void chol_kernel(int mode, const float* __restrict__ Gmat, const floa
 
 }  // namespace
 
-// Right-hand sides of one block are split over this many CTAs (each repeats the factorisation).  d_block 256
-// needs 4 for its shared memory; smaller blocks are split while that still fits one wave of CTAs.
+namespace {
+
+// right-hand sides per CTA in units of 32: as few as still give one wave of CTAs (d_block > 128: what fits beside the factor)
+int chol_groups(int db, int nb) {
+  if (db > 128) return 2;
+  for (int g = 1; g < 4; g *= 2)
+    if ((int64_t)nb * ((db + 32 * g - 1) / (32 * g)) <= 148 || 32 * g >= db) return g;
+  return 4;
+}
+
+template <int G>
+armor_status launch_blocked(armor_ctx* c, int mode, const float* Gm, const float* rhs, float* out, const float* dotw, float* A,
+                            int nb, double* part, cudaStream_t s) {
+  const int db = c->db;
+  const size_t smem = (panel_floats(db) + (size_t)db * (32 * G + 1)) * sizeof(float);
+  const int widest = G == 2 ? MAX_DB : 128;
+  static PerDeviceOnce attr;
+  if (ensure_dynamic_smem(attr, c->device, chol_blocked_kernel<G>,
+                          (panel_floats(widest) + (size_t)widest * (32 * G + 1)) * sizeof(float)) != ARMOR_OK)
+    return ARMOR_ERR_CUDA;
+  chol_blocked_kernel<G><<<dim3(nb, (db + 32 * G - 1) / (32 * G)), NT, smem, s>>>(mode, Gm, rhs, out, dotw, A, c->cfg.ridge, db,
+                                                                                  part, c->failflag, c->status);
+  c->launches++;
+  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+}
+
+}  // namespace
+
+// The right-hand sides of one block are dealt to this many CTAs (at most four), each of which repeats the factorisation.
 int chol_parts_per_block(int db, int nb) {
   if (db % NB) return 1;
-  if (db > 128) return db / 64;
-  int parts = 1;
-  while (parts < 4 && 2 * parts * nb <= 148 && db / (2 * parts) >= 32) parts *= 2;
-  return parts;
+  const int w = 32 * chol_groups(db, nb);
+  return (db + w - 1) / w;
 }
 
 armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float* rhs, float* out, const float* dotw,
@@ -523,21 +541,10 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
   const int db = c->db;
   KTimer kt(c, ARMOR_KC_CHOLESKY, (double)nb * (7.0 / 3.0) * (double)db * (double)db * (double)db, s);   // flops
   if (db % NB == 0) {
-    const int slices = chol_parts_per_block(db, nb);
-    const int w = db / slices;
-    const size_t smem = (panel_floats(db) + (size_t)db * (w + 1)) * sizeof(float);
-    static size_t attr_bytes[64] = {};   // per device: the limit set so far
-    const int dv = (c->device >= 0 && c->device < 64) ? c->device : 0;
-    if (smem > attr_bytes[dv] || c->device != dv) {
-      if (cudaFuncSetAttribute(chol_blocked_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-          cudaSuccess)
-        return ARMOR_ERR_CUDA;
-      attr_bytes[dv] = smem;
-    }
-    chol_blocked_kernel<<<dim3(nb, slices), NT, smem, s>>>(mode, Gmat, rhs, out, dotw, A, c->cfg.ridge, db, w,
-                                                          part, c->failflag, c->status);
-    c->launches++;
-    return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+    const int g = chol_groups(db, nb);
+    if (g == 1) return launch_blocked<1>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
+    if (g == 2) return launch_blocked<2>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
+    return launch_blocked<4>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
   }
   const size_t smem = 2 * (size_t)db * (db + 1) * sizeof(float);
   static PerDeviceOnce attr_set;

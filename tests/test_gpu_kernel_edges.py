@@ -117,3 +117,34 @@ def test_small_wrapper_products(d_out, d_in, d_block, side, transpose):
     assert ((out.double() - ref).abs() <= d_block * 2.0 ** -24 * mag + 1e-30).all()
     Bd.armor_block_product(ctx.ctx, side, transpose, Q, X, out, -1.0, D, 1.0, 0)
     assert ((out.double() - (D.double() - ref)).abs() <= (d_block + 2) * 2.0 ** -24 * (mag + D.double().abs())).all()
+
+
+@pytest.mark.parametrize("d_block,nb_out,nb_in", [(32, 8, 5), (64, 2, 9), (96, 3, 2), (128, 2, 3), (128, 40, 2), (128, 80, 1),
+                                                  (160, 2, 1), (192, 1, 2), (224, 2, 2), (256, 2, 3)])
+def test_block_solves(d_block, nb_out, nb_in):
+    """A-step and B-step of one iteration with the diagonal weighting, for every panel count and every number of right-hand
+    sides per warp: A - I solves (T D T^T + lam I) and the losses only fall.  fp32 solve of systems whose condition number
+    is below 1e3 by construction (d_in rows of T exceed d_block): 1e-4 of the result."""
+    from paper_2510_05528_b200 import binding as Bd
+    d_out, d_in = nb_out * d_block, nb_in * d_block * 4
+    g = _gen(d_block + nb_out)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    h = torch.rand(d_in, device=DEV, generator=g) + 0.5
+    H = torch.diag(h)
+    ctx = _ctx(d_out, d_in, d_block, precision=Bd.PREC_FP16X3, h_mode=Bd.H_DIAG, phases=1)   # A-step alone
+    st = ctx.init(W, H)
+    A0, S0 = st.A.clone(), st.S.clone()
+    stats = ctx.read_stats(ctx.bcd_step(st, H, 0, 1))
+    T = S0.double().view(nb_out, d_block, d_in)
+    E = (W - S0).double().view(nb_out, d_block, d_in)
+    G = (T * h.double()) @ T.transpose(1, 2)
+    lam = 1e-6 * G.diagonal(dim1=1, dim2=2).sum(1) / d_block
+    rhs = (E * h.double()) @ T.transpose(1, 2)
+    Gl = G + lam[:, None, None] * torch.eye(d_block, device=DEV, dtype=torch.float64)
+    X = torch.linalg.solve(Gl, rhs.transpose(1, 2)).transpose(1, 2)
+    assert torch.linalg.cond(Gl).max() < 1e3
+    got = (st.A - A0).double()
+    assert (got - X).norm() <= 1e-4 * X.norm()
+    dec = (rhs * X).sum() + (lam[:, None, None] * X * X).sum()
+    assert abs((stats["loss_start"][0] - stats["loss_A"][0]) - dec.item()) <= 1e-3 * dec.item()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
