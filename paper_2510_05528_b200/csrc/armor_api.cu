@@ -494,10 +494,11 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       if (st != ARMOR_OK) return st;
       launch_stage(c, is, 0, nullptr, 0, 0, s);
     } else {
-    bd_right(c, S, B, false, c->T, d_out, d_in, 1.f, nullptr, 0.f, s);              // T = S B
     if (first || !carry_P) {
-      st = rmul_H(c, c->T, H, c->P, d_out, nullptr, nullptr, nullptr, nullptr, s);   // P = T H_w
+      st = bd_right_H(c, S, B, H, c->T, c->P, s);                                    // T = S B, P = T H_w
       if (st != ARMOR_OK) return st;
+    } else {
+      bd_right(c, S, B, false, c->T, d_out, d_in, 1.f, nullptr, 0.f, s);             // T = S B
     }
     bd_left(c, A, false, c->P, c->EH, d_out, d_in, -1.f, c->WH, 1.f, s);             // E H_w = W H_w - A P
     if (fresh_loss) {
@@ -574,8 +575,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
         launch_delta_finish(c, c->Delta, c->GamB, c->partblk, s);                    // part_j = <Gamma_j, Delta_j>
       }
       // direction in B: V = A R with R = S Delta; R H_w serves both V H_w = A (R H_w) and the carried P
-      bd_right(c, S, c->Delta, false, c->Tmp, d_out, d_in, 1.f, nullptr, 0.f, s);    // R = S Delta
-      st = rmul_H(c, c->Tmp, H, c->E, d_out, nullptr, nullptr, nullptr, nullptr, s); // R H_w
+      st = bd_right_H(c, S, c->Delta, H, c->Tmp, c->E, s);                           // R = S Delta, R H_w
       if (st != ARMOR_OK) return st;
       // V H_w = A (R H_w) and q = <V H_w, V> with V = A R (summed by the stage; V itself is needed nowhere else)
       int nq = 0;
@@ -591,11 +591,16 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
 
     // ---- S-step: exact line search along Gamma (.) M ------------------------------------------
     if (!adam && (ph & ARMOR_PHASE_S)) {
-      core_gradient(c, A, B, s);
       double* nrm_part = c->partials + 8 * c->npart;                                 // kept until the stage below
-      launch_masked_copy(c, c->Gam, M, c->U, nrm_part, s);                           // U = Gamma (.) M, |U|^2
-      bd_right(c, c->U, B, false, c->Tmp, d_out, d_in, 1.f, nullptr, 0.f, s);        // R = Gamma_M B
-      st = rmul_H(c, c->Tmp, H, c->E, d_out, nullptr, nullptr, nullptr, nullptr, s); // R H_w
+      int n_nrm = 0;
+      // U = Gamma (.) M, |U|^2: the mask is applied where the gradient leaves tensor memory, or in a pass of its own
+      if (!(c->tc_blocks == 3 && tc_block2_ok(c, d_out, d_in) &&
+            tc_done(c, tc_two_sided(c, A, true, c->EH, B, true, c->U, d_out, d_in, 1.f, s, M, nrm_part, &n_nrm)))) {
+        core_gradient(c, A, B, s);
+        launch_masked_copy(c, c->Gam, M, c->U, nrm_part, s);
+        n_nrm = ARMOR_DOT_BLOCKS;
+      }
+      st = bd_right_H(c, c->U, B, H, c->Tmp, c->E, s);                               // R = Gamma_M B, R H_w
       if (st != ARMOR_OK) return st;
       // V H_w = A (R H_w) and q = <V H_w, V> with V = A Gamma_M B
       int nq = 0;
@@ -618,7 +623,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
         }
       }
       launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S,
-                   nrm_part, ARMOR_DOT_BLOCKS, SC_NRM_S);
+                   nrm_part, n_nrm, SC_NRM_S);
       // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
       launch_axpy_multi(c, S, c->U, 1.f, c->EH, c->VH, -1.f, carry_P ? c->P : nullptr, c->E, 1.f, c->wn, SC_TAU_S, s);
     } else if (!adam) {
@@ -639,8 +644,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
             if (carry_P) {
               launch_mask_carry_P(c, c->P, s);                                       // P += dS B H_w (if accepted)
             } else {
-              bd_right(c, S, B, false, c->T, d_out, d_in, 1.f, nullptr, 0.f, s);     // T = S B
-              st = rmul_H(c, c->T, H, c->P, d_out, nullptr, nullptr, nullptr, nullptr, s);
+              st = bd_right_H(c, S, B, H, c->T, c->P, s);                            // T = S B, P = T H_w
               if (st != ARMOR_OK) return st;
             }
             bd_left(c, A, false, c->P, c->EH, d_out, d_in, -1.f, c->WH, 1.f, s);     // E H_w = W H_w - A P

@@ -125,9 +125,9 @@ struct armor_ctx {
   int n_sm;             // its number of SMs
   int tc_blocks;        // 1, 2, 3: block products and per-block Grams on the tensor cores where the shape allows.
                         // 1: the streaming kernel for every product; 2: with d_block = 128 the kernel that keeps the
-                        // wrapper block in tensor memory for every product; 3 (default): that kernel for the dual
-                        // product, where it halves the shared-memory traffic, and the streaming kernel elsewhere
-                        // (the two measure equal on single products at 4096 x 4096);
+                        // wrapper block in tensor memory (products and dual products); 3 (default): that kernel for
+                        // left and dual products and for right products with the column-scaled second output, the
+                        // streaming kernel for other right products, the two-sided kernel where both wrappers apply;
                         // 0: always the fp32 CUDA-core kernels (exact products with 0 and 1)
   int gram_pairs;       // 1: the two per-block Grams of a step in one launch (shared operand read once)
   armor_status host_err;   // first launch failure inside the running call that no fallback covers
@@ -203,6 +203,9 @@ void bd_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, flo
               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
 void bd_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
              int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
+// out = in Bdiag and outH = out H_w for the layer's shape [d_out, d_in] (one launch with the diagonal weighting where the
+// tensor-core kernel takes d_block)
+armor_status bd_right_H(armor_ctx* c, const float* in, const float* Bblk, const float* H, float* out, float* outH, cudaStream_t s);
 // out = alpha * Lop X Rop with both wrappers (Lop_i = Lblk[i] or its transpose, Rop_j likewise): one fused launch on
 // the tensor cores where the shape allows (d_block 128; the intermediate stays in tensor memory), else the two
 // one-sided products through tmp
@@ -227,7 +230,8 @@ armor_status tc_bd_left_dual(armor_ctx* c, const float* Ablk, bool transA, const
 // both wrappers in one launch (block2_tcgen05.cu); d_block = 128
 bool tc_block2_ok(const armor_ctx* c, int64_t rows, int64_t cols);
 armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const float* X, const float* Rblk, bool transR,
-                          float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s);
+                          float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s, const uint8_t* mask = nullptr,
+                          double* norm_part = nullptr, int* n_norm = nullptr);
 
 // E = add - Ablk in, EH = E diag(colw), partial sums of <E, EH> at part: one launch
 armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* in, const float* add, const float* colw,
@@ -236,7 +240,8 @@ armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* i
 // the same with the wrapper block held in tensor memory (blockres_tcgen05.cu); d_block = 128
 bool tc_blockres_ok(const armor_ctx* c);
 armor_status tc_blockres_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
-                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
+                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s,
+                               const float* colw = nullptr, float* out2 = nullptr);
 armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
 

@@ -48,6 +48,10 @@ struct P2Params {
   int64_t c_rows, c_cols;
   float alpha;
   int32_t* status;
+  // not null: only the entries that the N:M mask keeps are written, the others as zeros, and norm_part takes 4 partial sums
+  // per tile (one per epilogue warp, in the order of the work items) of their squares
+  const uint8_t* mask; int m_group;      // one byte per m_group entries of a row
+  double* norm_part;
 };
 
 
@@ -71,6 +75,13 @@ __device__ __forceinline__ void schedule_step(int o, int n, bool& second, int& t
   if (m == 2 * n - 2) { second = true; t = n - 1; return; }
   second = (m & 1) != 0;
   t = second ? (m >> 1) : (m >> 1) + 1;
+}
+
+// the low four bits of each byte, side by side
+__device__ __forceinline__ uint32_t low_nibbles(uint32_t v) {
+  v &= 0x0f0f0f0fu;
+  v = (v | (v >> 4)) & 0x00ff00ffu;
+  return (v | (v >> 8)) & 0xffffu;
 }
 
 __device__ __forceinline__ uint64_t op_desc(uint32_t base, int mn) {
@@ -271,6 +282,21 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
       const int i = item / p.nbj, j = item - i * p.nbj;
       const int64_t row_base = (int64_t)TILE * i + q * 32;
       const int64_t col_tile = (int64_t)TILE * j;
+      // the mask of the lane's row: four bits per 16-byte cell, one word per box
+      uint32_t keep[4] = {0u, 0u, 0u, 0u};
+      double norm = 0.0;
+      if (p.mask) {
+        const uint8_t* mrow = p.mask + ((row_base + lane) * p.c_cols + col_tile) / p.m_group;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          if (p.m_group == 8) {
+            keep[g] = *reinterpret_cast<const uint32_t*>(mrow + 4 * g);
+          } else {
+            const uint2 v = *reinterpret_cast<const uint2*>(mrow + 8 * g);
+            keep[g] = low_nibbles(v.x) | (low_nibbles(v.y) << 16);
+          }
+        }
+      }
       // The warp's 32 x 128 slab goes through shared memory in two halves of 64 columns (two 32 x 32 boxes).
 #pragma unroll 1
       for (int hf = 0; hf < 2 && ok; ++hf) {
@@ -289,8 +315,16 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
 #pragma unroll
           for (int cq = 0; cq < 8; ++cq) {
             float4* cell = reinterpret_cast<float4*>(rowp + ((cq ^ (lane & 7)) << 4));
-            *cell = make_float4(p.alpha * __uint_as_float(r[4 * cq]), p.alpha * __uint_as_float(r[4 * cq + 1]),
-                                p.alpha * __uint_as_float(r[4 * cq + 2]), p.alpha * __uint_as_float(r[4 * cq + 3]));
+            float4 v = make_float4(p.alpha * __uint_as_float(r[4 * cq]), p.alpha * __uint_as_float(r[4 * cq + 1]),
+                                   p.alpha * __uint_as_float(r[4 * cq + 2]), p.alpha * __uint_as_float(r[4 * cq + 3]));
+            if (p.mask) {
+              const uint32_t m = (hf ? (ch ? keep[3] : keep[2]) : (ch ? keep[1] : keep[0])) >> (4 * cq);
+              v.x = (m & 1u) ? v.x : 0.f; v.y = (m & 2u) ? v.y : 0.f; v.z = (m & 4u) ? v.z : 0.f; v.w = (m & 8u) ? v.w : 0.f;
+              float sq = v.x * v.x;
+              sq = fmaf(v.y, v.y, sq); sq = fmaf(v.z, v.z, sq); sq = fmaf(v.w, v.w, sq);
+              norm += (double)sq;
+            }
+            *cell = v;
           }
         }
         if (hf == 1) tc_fence_before();             // all reads of the accumulator are done
@@ -302,6 +336,12 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
             tma_store_2d(&mapC, (int)(col_tile + 64 * hf + 32 * ch), (int)row_base, buf_u32 + ch * 4096);
           tma_store_commit();
         }
+      }
+      if (p.mask) {
+        // lanes in a fixed order
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) norm += __shfl_xor_sync(0xffffffffu, norm, o);
+        if (ok && lane == 0) p.norm_part[(size_t)item * 4 + q] = norm;
       }
     }
     if (lane == 0) tma_store_wait_read();           // shared memory stays valid until the stores have read it
@@ -348,10 +388,13 @@ bool tc_block2_ok(const armor_ctx* c, int64_t rows, int64_t cols) {
 }
 
 // out[i-th block row, j-th block column] = alpha * Lop_i * X_ij * Rop_j,  Lop_i = Lblk[i] or its transpose, Rop_j = Rblk[j]
-// or its transpose; X and out are [rows, cols] and must not overlap
+// or its transpose; X and out are [rows, cols] and must not overlap.  With mask only the kept entries of out are written (the
+// others as zeros), and *n_norm partial sums of their squares go to norm_part.
 armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const float* X, const float* Rblk, bool transR,
-                          float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s) {
+                          float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s, const uint8_t* mask,
+                          double* norm_part, int* n_norm) {
   if (!ptr_ok(Lblk) || !ptr_ok(X) || !ptr_ok(Rblk) || !ptr_ok(out)) return ARMOR_ERR_UNSUPPORTED;
+  if (mask && !ptr_ok(mask)) return ARMOR_ERR_UNSUPPORTED;
   P2Params p{};
   p.l_mn = transL ? 1 : 0;
   p.r_mn = transR ? 0 : 1;
@@ -359,6 +402,8 @@ armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const fl
   p.c_rows = rows; p.c_cols = cols;
   p.alpha = alpha;
   p.status = c->status;
+  p.mask = mask; p.m_group = c->cfg.m_group; p.norm_part = norm_part;
+  if (n_norm) *n_norm = 4 * p.nbi * p.nbj;
   CUtensorMap mL, mX, mR, mC;
   if (!make_map_2d(&mL, Lblk, TILE, rows, TILE, 32, p.l_mn ? 32 : TILE, p.l_mn != 0)) return ARMOR_ERR_CUDA;
   if (!make_map_2d(&mX, X, cols, rows, cols, 32, 32, true)) return ARMOR_ERR_CUDA;

@@ -441,6 +441,16 @@ void bd_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, flo
   launch_bgemm(c, g, s);
 }
 
+armor_status bd_right_H(armor_ctx* c, const float* in, const float* Bblk, const float* H, float* out, float* outH, cudaStream_t s) {
+  const int64_t rows = c->d_out, cols = c->d_in;
+  // diagonal weighting: the column scale is a second output of the product's epilogue (same multiplications)
+  if (c->cfg.h_mode == ARMOR_H_DIAG && c->tc_blocks > 1 && tc_block_ok(c, rows, cols) && tc_blockres_ok(c) &&
+      tc_done(c, tc_blockres_right(c, in, Bblk, false, out, rows, cols, 1.f, nullptr, 0.f, s, c->hdiag, outH)))
+    return ARMOR_OK;
+  bd_right(c, in, Bblk, false, out, rows, cols, 1.f, nullptr, 0.f, s);
+  return rmul_H(c, out, H, outH, rows, nullptr, nullptr, nullptr, nullptr, s);
+}
+
 void bd_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
              int64_t cols, float alpha, const float* add, float beta, cudaStream_t s) {
   if (c->tc_blocks && tc_block_ok(c, rows, cols) &&

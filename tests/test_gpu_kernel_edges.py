@@ -148,3 +148,33 @@ def test_block_solves(d_block, nb_out, nb_in):
     dec = (rhs * X).sum() + (lam[:, None, None] * X * X).sum()
     assert abs((stats["loss_start"][0] - stats["loss_A"][0]) - dec.item()) <= 1e-3 * dec.item()
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("n_keep,m_group", [(2, 4), (4, 8), (6, 8)])
+@pytest.mark.parametrize("mode", ["diag", "full"])
+@pytest.mark.parametrize("d_out,d_in", [(128, 128), (384, 256), (2688, 1024)])
+def test_core_step_with_the_mask_applied_in_the_gradient(n_keep, m_group, mode, d_out, d_in):
+    """S-step alone from a state off the initialisation: S moves along Gamma (.) M by |Gamma_M|^2 / tr(V H V^T), the other
+    entries stay zero.  Three-pass products of 128 terms behind one with d_in terms: 2e-5 of the move."""
+    from paper_2510_05528_b200 import binding as Bd
+    db = 128
+    g = _gen(d_out + d_in + m_group)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    X = torch.randn(2 * d_in, d_in, device=DEV, generator=g)
+    H = torch.diag(torch.rand(d_in, device=DEV, generator=g) + 0.5) if mode == "diag" else (X.double().t() @ X.double()).float()
+    ctx = _ctx(d_out, d_in, db, n_keep=n_keep, m_group=m_group, phases=4, h_mode=Bd.H_DIAG if mode == "diag" else Bd.H_FULL)
+    st = ctx.init(W, H)
+    st.A.add_(torch.randn(st.A.shape, device=DEV, generator=g) * 0.05)
+    st.B.add_(torch.randn(st.B.shape, device=DEV, generator=g) * 0.05)
+    S0 = st.S.clone()
+    keep = torch.stack([(st.M.int() >> k) & 1 for k in range(m_group)], -1).view(d_out, d_in).bool()
+    Ad, Bd64 = torch.block_diag(*st.A.double()), torch.block_diag(*st.B.double())
+    Hd = H.double()
+    Gm = (Ad.t() @ (W.double() - Ad @ S0.double() @ Bd64) @ Hd @ Bd64.t()) * keep
+    V = Ad @ Gm @ Bd64
+    tau = (Gm * Gm).sum() / ((V @ Hd) * V).sum()
+    ctx.bcd_step(st, H, 0, 1)
+    move = (st.S - S0).double()
+    assert (st.S[~keep] == 0).all()
+    assert (move - tau * Gm).norm() <= 2e-5 * (tau * Gm).norm() + 2.0 ** -24 * S0.double().norm()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
