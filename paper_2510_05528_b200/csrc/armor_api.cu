@@ -485,7 +485,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
   armor_iter_stats* const is = d_stats;   // base of the records; the kernels add the device counter
   auto body = [&](bool first, bool fresh_loss, bool t_zero, cudaStream_t s) -> armor_status {
     armor_status st = ARMOR_OK;
-    launch_zero_scalars(c, !fresh_loss, is, s);      // with a carried loss this also opens the iteration's record
+    launch_zero_scalars(c, !first, !fresh_loss, is, s);      // with a carried loss this also opens the iteration's record
     if (adam) {
       // Adam normalises every entry's move, so a gradient that is exactly zero (the kept entries of the core at
       // the initialisation, where E vanishes on them) must come out as zero: E H_w is formed from E itself, not
@@ -552,7 +552,6 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
 
     // ---- B-step: block-Newton directions, one exact step --------------------------------------
     if (!adam && (ph & ARMOR_PHASE_B)) {
-      launch_zero_flags(c, s);
       bd_left(c, A, false, S, c->U, d_out, d_in, 1.f, nullptr, 0.f, s);              // U = A S
       colblock_grams(c, c->U, c->U, c->EH, c->C, c->GamB, s);   // C_j = U_j^T U_j, Gamma_j = U_j^T (E H_w)_j
       const bool b_gd = (c->cfg.ab_step == ARMOR_AB_GD);
@@ -581,10 +580,10 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       int nq = 0;
       bd_left_dual(c, A, c->Tmp, c->E, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
       if (b_gd) launch_stage(c, is, 8, nullptr, 0, 0, s, c->partials, nq, SC_Q_B);
-      else launch_stage(c, is, 2, c->partblk, nbi, nbi, s, c->partials, nq, SC_Q_B);
-      launch_axpy_slot(c, B, c->Delta, (int64_t)nbi * db * db, SC_TAU_B, 1.f, s);    // B += tau Delta
-      // EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
-      launch_axpy_multi(c, c->EH, c->VH, -1.f, carry_P ? c->P : nullptr, c->E, 1.f, nullptr, nullptr, 0.f, c->wn, SC_TAU_B, s);
+      else launch_stage(c, is, 2, c->partblk, DELTA_PARTS * nbi, nbi, s, c->partials, nq, SC_Q_B);
+      // B += tau Delta, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
+      launch_axpy_multi(c, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
+                        (int64_t)nbi * db * db, SC_TAU_B, s);
     } else if (!adam) {
       launch_stage(c, is, 2, nullptr, 0, 0, s);
     }
@@ -625,7 +624,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S,
                    nrm_part, n_nrm, SC_NRM_S);
       // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
-      launch_axpy_multi(c, S, c->U, 1.f, c->EH, c->VH, -1.f, carry_P ? c->P : nullptr, c->E, 1.f, c->wn, SC_TAU_S, s);
+      launch_axpy_multi(c, S, c->U, 1.f, c->wn, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, c->E, 1.f, c->wn, SC_TAU_S, s);
     } else if (!adam) {
       launch_stage(c, is, 3, nullptr, 0, 0, s);
     }
@@ -660,7 +659,6 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
     } else {
       launch_stage(c, is, 5, nullptr, 0, 0, s);
     }
-    launch_advance_iteration(c, s);
     return ARMOR_OK;
   };
 

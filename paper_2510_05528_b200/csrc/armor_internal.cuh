@@ -108,7 +108,7 @@ struct armor_ctx {
   unsigned long long* tab_g;   // its global group index
   int32_t* status;    // [ST_COUNT]
   int32_t* screen;    // [4] per-call counters of the input screening
-  int64_t* it_dev;    // iteration index inside the running armor_bcd_step call (advanced by the last kernel of an iteration)
+  int64_t* it_dev;    // iteration index inside the running armor_bcd_step call (advanced by the first kernel of an iteration)
   int use_graphs;     // 1: repeated iterations of a call are replayed from a CUDA graph
   cudaStream_t cap_stream;   // the context's own stream, used only to capture that graph
   // Capture in pieces (while the dense products are being timed with events, which a graph cannot replay): every
@@ -322,13 +322,13 @@ void launch_masked_copy(armor_ctx* c, const float* Gam, const uint8_t* M, float*
                         cudaStream_t s);              // out = Gam (.) M; ARMOR_DOT_BLOCKS partial sums of ||out||^2
 void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slot, float sign,
                       cudaStream_t s);
-void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, float* y1, const float* x1, float s1, float* y2,
-                       const float* x2, float s2, int64_t n, int slot, cudaStream_t s);                                       // y += sign * sc[slot] * x
+void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64_t n0, float* y1, const float* x1, float s1,
+                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s);                                       // y += sign * sc[slot] * x
 void launch_init(armor_ctx* c, const float* W, const float* H, float* Wbar, float* r1, float* r2,
                  float* A, float* B, float* S, uint8_t* M, cudaStream_t s);
 // st: base of the iteration records (the kernels add c->it_dev), or null
-void launch_zero_scalars(armor_ctx* c, bool carry_loss, armor_iter_stats* st, cudaStream_t s);
-void launch_advance_iteration(armor_ctx* c, cudaStream_t s);   // ++*c->it_dev
+// advance: ++*c->it_dev first
+void launch_zero_scalars(armor_ctx* c, bool advance, bool carry_loss, armor_iter_stats* st, cudaStream_t s);
 // Input screening at the top of a call: counts non-finite entries of W and H and negative / zero diagonal
 // entries of H into the status words and sets or clears ST_POISON for the call.
 armor_status launch_screen_inputs(armor_ctx* c, const float* W, const float* H, cudaStream_t s);
@@ -339,7 +339,6 @@ void launch_adam(armor_ctx* c, float* theta, const float* gamma, float* m, float
 // part[b] = weight_b * || X_b ||_F for the nblk blocks of db x db floats in X; weight_b = 1, or the Euclidean
 // norm of hdiag over the (b % nbi)-th block of columns; out = sum of the parts (fixed order)
 void launch_block_fro_sum(armor_ctx* c, const float* X, int nblk, const float* hdiag, double* out, cudaStream_t s);
-void launch_zero_flags(armor_ctx* c, cudaStream_t s);
 // per-iteration bookkeeping on the device: stage 0 start, 1 after A, 2 after B, 3 after S, 4 mask accept
 // (p1, n1, slot1), (p2, n2, slot2): partial sums the stage first adds up into sc[slot] (a preceding dot product)
 void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, int nflag,
@@ -365,7 +364,8 @@ int chol_parts_per_block(int db, int nb);
 // (H_jj + mu I)^-1 for every column block into c->Hinv (H_jj does not change inside a call), failures into c->hinv_fail
 armor_status launch_hjj_inverse(armor_ctx* c, cudaStream_t s);
 // after Delta = Y Hinv: zeroes the blocks whose H_jj was not positive definite (raising their failflag, as a failed
-// solve would) and writes part[j] = <dotw_j, Delta_j>
+// solve would) and writes DELTA_PARTS partial sums of <dotw_j, Delta_j> per block
+static const int DELTA_PARTS = 4;
 void launch_delta_finish(armor_ctx* c, float* Delta, const float* dotw, double* part, cudaStream_t s);
 armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float* rhs, float* out, const float* dotw,
                          float* A, int nb, double* part, cudaStream_t s);

@@ -655,13 +655,16 @@ armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* i
 
 namespace {
 
-// out[e] = sum over the slabs, in slab order
+// out[e] = sum over the slabs, in slab order; blockIdx.y 1: the same for the second Gram of a pair, n_slab slabs further on
 __global__ void __launch_bounds__(256) sum_slabs_kernel(const float4* __restrict__ part, int64_t n4, int n_slab,
-                                                        float4* __restrict__ out) {
+                                                        float4* __restrict__ out0, float4* __restrict__ out1) {
+  const float4* p = part + (int64_t)blockIdx.y * n_slab * n4;
+  float4* out = blockIdx.y ? out1 : out0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (int64_t)gridDim.x * 256) {
-    float4 acc = part[i];
+    float4 acc = p[i];
+#pragma unroll 4
     for (int k = 1; k < n_slab; ++k) {
-      const float4 v = part[(int64_t)k * n4 + i];
+      const float4 v = p[(int64_t)k * n4 + i];
       acc.x += v.x; acc.y += v.y; acc.z += v.z; acc.w += v.w;
     }
     out[i] = acc;
@@ -696,7 +699,7 @@ armor_status gram_launch(armor_ctx* c, const HostOp& A, const HostOp& B, float* 
   int64_t blocks = (slab / 4 + 255) / 256;
   if (blocks > 148 * 8) blocks = 148 * 8;
   sum_slabs_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
-                                                   reinterpret_cast<float4*>(G));
+                                                   reinterpret_cast<float4*>(G), nullptr);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
@@ -725,11 +728,9 @@ armor_status gram_pair_launch(armor_ctx* c, const HostOp& A, const HostOp& B, co
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
   int64_t blocks = (slab / 4 + 255) / 256;
   if (blocks > 148 * 8) blocks = 148 * 8;
-  sum_slabs_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
-                                                   reinterpret_cast<float4*>(G));
-  sum_slabs_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(c->gpart + ks * slab), slab / 4, ks,
-                                                   reinterpret_cast<float4*>(G2));
-  c->launches += 2;
+  sum_slabs_kernel<<<dim3((unsigned)blocks, 2), 256, 0, s>>>(reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
+                                                            reinterpret_cast<float4*>(G), reinterpret_cast<float4*>(G2));
+  c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
 

@@ -568,18 +568,23 @@ __global__ void save_flags_kernel(const int32_t* __restrict__ failflag, int32_t*
   if (i < n) saved[i] = failflag[i];
 }
 
-// one CTA per block: Delta_j = 0 and failflag[j] = 1 where the inverse does not exist; part[j] = <dotw_j, Delta_j>
+// DELTA_PARTS CTAs per block: Delta_j = 0 and failflag[j] = 1 where the inverse does not exist; partial sums of
+// <dotw_j, Delta_j>
 __global__ void __launch_bounds__(NT) delta_finish_kernel(float* __restrict__ Delta, const float* __restrict__ dotw,
                                                           const int32_t* __restrict__ hinv_fail,
                                                           int32_t* __restrict__ failflag, double* __restrict__ part,
                                                           int db) {
-  const int j = blockIdx.x;
+  const int j = blockIdx.x / DELTA_PARTS, q = blockIdx.x % DELTA_PARTS;
   const int64_t off = (int64_t)j * db * db;
+  const int n4 = db * db / 4, e1 = n4 * (q + 1) / DELTA_PARTS;
   const bool bad = hinv_fail[j] != 0;
   double acc = 0.0;
-  for (int e = threadIdx.x; e < db * db; e += NT) {
-    if (bad) Delta[off + e] = 0.f;
-    else acc += (double)dotw[off + e] * (double)Delta[off + e];
+#pragma unroll 4
+  for (int e = n4 * q / DELTA_PARTS + threadIdx.x; e < e1; e += NT) {
+    float4* d = reinterpret_cast<float4*>(Delta + off) + e;
+    if (bad) { *d = make_float4(0.f, 0.f, 0.f, 0.f); continue; }
+    const float4 w = *(reinterpret_cast<const float4*>(dotw + off) + e), v = *d;
+    acc += (double)w.x * (double)v.x + (double)w.y * (double)v.y + (double)w.z * (double)v.z + (double)w.w * (double)v.w;
   }
   __shared__ double red[NT / 32];
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
@@ -588,7 +593,7 @@ __global__ void __launch_bounds__(NT) delta_finish_kernel(float* __restrict__ De
   if (threadIdx.x == 0) {
     double t = 0.0;
     for (int w = 0; w < NT / 32; ++w) t += red[w];
-    part[j] = t;
+    part[blockIdx.x] = t;
     if (bad) failflag[j] = 1;
   }
 }
@@ -613,7 +618,7 @@ armor_status launch_hjj_inverse(armor_ctx* c, cudaStream_t s) {
 
 void launch_delta_finish(armor_ctx* c, float* Delta, const float* dotw, double* part, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  delta_finish_kernel<<<c->nbi, NT, 0, s>>>(Delta, dotw, c->hinv_fail, c->failflag, part, c->db);
+  delta_finish_kernel<<<DELTA_PARTS * c->nbi, NT, 0, s>>>(Delta, dotw, c->hinv_fail, c->failflag, part, c->db);
   c->launches++;
 }
 

@@ -80,16 +80,25 @@ __global__ void __launch_bounds__(NT) rowcolscale_kernel(const float* __restrict
 }
 
 // ---- H diagonal and diagonal blocks -------------------------------------------------------------
-__global__ void extract_hblocks_kernel(const float* __restrict__ H, float* __restrict__ hdiag,
-                                       float* __restrict__ Hjj, int64_t d_in, int db, int diag_only) {
-  const int j = blockIdx.x;
-  for (int e = threadIdx.x; e < db * db; e += blockDim.x) {
-    int a = e / db, b = e % db;
+// (eight rows of a block per CTA: with a CTA per block the dependent loads of 16,384 elements took 33 us)
+constexpr int HB_ROWS = 8;
+__global__ void __launch_bounds__(NT) extract_hblocks_kernel(const float* __restrict__ H, float* __restrict__ hdiag,
+                                                             float* __restrict__ Hjj, int64_t d_in, int db, int diag_only) {
+  const int j = blockIdx.x, a0 = blockIdx.y * HB_ROWS;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < HB_ROWS * db; e += NT) {
+    const int a = a0 + e / db, b = e % db;
+    if (a >= db) break;
     float v = H[(int64_t)(j * db + a) * d_in + (j * db + b)];
     if (diag_only && a != b) v = 0.f;
-    Hjj[(int64_t)j * db * db + e] = v;
+    Hjj[((int64_t)j * db + a) * db + b] = v;
     if (a == b) hdiag[j * db + a] = v;
   }
+}
+
+__global__ void __launch_bounds__(NT) diag_kernel(const float* __restrict__ H, float* __restrict__ hdiag, int64_t d_in) {
+  const int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x;
+  if (k < d_in) hdiag[k] = H[k * d_in + k];
 }
 
 // ---- Gamma_M = Gamma (.) M and its squared norm -------------------------------------------------
@@ -128,8 +137,8 @@ __global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* __restrict__ y, c
   }
 }
 
-// the same for up to three arrays of one length that move by the same step: one launch
-struct AxpyTerm { float4* y; const float4* x; float sign; };
+// the same for up to three arrays that move by the same step: one launch
+struct AxpyTerm { float4* y; const float4* x; float sign; int64_t n4; };
 __global__ void __launch_bounds__(NT) axpy_multi_slot_kernel(AxpyTerm t0, AxpyTerm t1, AxpyTerm t2, int n_terms, int64_t n4,
                                                              const double* __restrict__ sc, int slot) {
   const float a = (float)sc[slot];
@@ -139,6 +148,7 @@ __global__ void __launch_bounds__(NT) axpy_multi_slot_kernel(AxpyTerm t0, AxpyTe
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       if (k >= n_terms) break;
+      if (i >= t[k].n4) continue;
       const float ak = t[k].sign * a;
       const float4 u = t[k].y[i], v = t[k].x[i];
       t[k].y[i] = make_float4(fmaf(ak, v.x, u.x), fmaf(ak, v.y, u.y), fmaf(ak, v.z, u.z), fmaf(ak, v.w, u.w));
@@ -170,17 +180,35 @@ __global__ void __launch_bounds__(NT) colnorm_final_kernel(const double* __restr
   float r = (float)sqrt(acc);
   r1[col] = (r == 0.f) ? 1.f : r;
 }
+// The row norm of W / r1 to more than double the digits of fp32, without fp64 in the loop (a division in fp64 per element
+// took this pass to three times its memory time): 1 / r1 as a pair of floats, product and square with their rounding errors,
+// the sum as an unevaluated pair per thread, fp64 across threads.
 __global__ void __launch_bounds__(NT) rownorm_scale_kernel(const float* __restrict__ W, const float* __restrict__ r1,
                                                            float* __restrict__ r2, float* __restrict__ Wbar,
                                                            int64_t cols) {
   const int64_t row = blockIdx.x;
   const float* w = W + row * cols;
-  double acc = 0.0;
+  float hi = 0.f, lo = 0.f;
+#pragma unroll 2
   for (int64_t c = threadIdx.x; c < cols; c += NT) {
-    double v = (double)w[c] / (double)r1[c];
-    acc += v * v;
+    const float d = r1[c], x = w[c];
+    const float ih = 1.f / d, il = fmaf(-d, ih, 1.f) * ih;             // 1 / d = ih + il
+    const float vh = x * ih, vl = fmaf(x, ih, -vh) + x * il;           // x / d
+    const float qh = vh * vh, ql = fmaf(vh, vh, -qh) + 2.f * vh * vl;  // its square
+    const float s = hi + qh, bb = s - hi;
+    lo += (hi - (s - bb)) + (qh - bb) + ql;
+    hi = (d > 1e-30f && d < 1e30f) ? s : __int_as_float(0x7fc00000);   // (else the pair of 1 / d loses digits)
   }
   __shared__ float r2s;
+  double acc = (double)hi + (double)lo;
+  if (!isfinite(acc) || acc < 1e-30) {
+    // out of the range in which the pairs carry their digits: every term in fp64
+    acc = 0.0;
+    for (int64_t c = threadIdx.x; c < cols; c += NT) {
+      const double v = (double)w[c] / (double)r1[c];
+      acc += v * v;
+    }
+  }
   acc = block_reduce_sum(acc);
   if (threadIdx.x == 0) {
     float r = (float)sqrt(acc);
@@ -190,37 +218,60 @@ __global__ void __launch_bounds__(NT) rownorm_scale_kernel(const float* __restri
   }
   __syncthreads();
   const float rr = r2s;
+#pragma unroll 4
   for (int64_t c = threadIdx.x; c < cols; c += NT) Wbar[row * cols + c] = (w[c] / r1[c]) / rr;
 }
 
 // ---- initialisation (Eq. init): top-n_keep of each group of MG by W^2 * H_jj ---------------------
 // Position p is kept iff fewer than n_keep positions beat it; q beats p if its score is larger, or equal
 // with q < p (ties keep the lower column).
+// The order is the one of the scores in fp64.  Scores in fp32 (two roundings, 2^-23 relative) give the same order unless two
+// of a group lie within 5e-7 of each other, are all below the range where fp32 keeps its digits, or are not finite: only
+// such a group is scored again in fp64, whose instructions otherwise took this pass to three times its memory time.
 template <int MG>
-__global__ void __launch_bounds__(NT) init_core_kernel(const float* __restrict__ W, const float* __restrict__ H,
-                                                       int64_t d_in, float* __restrict__ S, uint8_t* __restrict__ M,
+__global__ void __launch_bounds__(NT) init_core_kernel(const float* __restrict__ W, const float* __restrict__ hdiag,
+                                                       float* __restrict__ S, uint8_t* __restrict__ M,
                                                        int64_t ngroups, int groups_per_row, int n_keep) {
   for (int64_t g = (int64_t)blockIdx.x * NT + threadIdx.x; g < ngroups; g += (int64_t)gridDim.x * NT) {
     const int64_t c0 = (g % groups_per_row) * MG;
-    float wv[MG];
+    float wv[MG], hv[MG], sc[MG];
 #pragma unroll
     for (int h = 0; h < MG / 4; ++h) {
       const float4 w = *reinterpret_cast<const float4*>(W + g * MG + 4 * h);
+      const float4 d = __ldg(reinterpret_cast<const float4*>(hdiag + c0 + 4 * h));
       wv[4 * h] = w.x; wv[4 * h + 1] = w.y; wv[4 * h + 2] = w.z; wv[4 * h + 3] = w.w;
+      hv[4 * h] = d.x; hv[4 * h + 1] = d.y; hv[4 * h + 2] = d.z; hv[4 * h + 3] = d.w;
     }
-    double sc[MG];
 #pragma unroll
-    for (int p = 0; p < MG; ++p) {
-      const double h = (double)H[(c0 + p) * d_in + (c0 + p)];
-      sc[p] = (double)wv[p] * (double)wv[p] * h;
-    }
+    for (int p = 0; p < MG; ++p) sc[p] = wv[p] * (wv[p] * hv[p]);
+    bool clear = true;
+#pragma unroll
+    for (int p = 0; p < MG; ++p)
+#pragma unroll
+      for (int q = p + 1; q < MG; ++q) {
+        const float big = fmaxf(fabsf(sc[p]), fabsf(sc[q]));
+        clear &= big > 1e-30f && fabsf(sc[p] - sc[q]) > 5e-7f * big;     // (false for NaN and for two infinities)
+      }
     unsigned m = 0;
+    if (clear) {
 #pragma unroll
-    for (int p = 0; p < MG; ++p) {
-      int beaten = 0;
+      for (int p = 0; p < MG; ++p) {
+        int beaten = 0;
 #pragma unroll
-      for (int q = 0; q < MG; ++q) beaten += (q != p) && (sc[q] > sc[p] || (sc[q] == sc[p] && q < p));
-      if (beaten < n_keep) m |= 1u << p;
+        for (int q = 0; q < MG; ++q) beaten += (q != p) && sc[q] > sc[p];
+        if (beaten < n_keep) m |= 1u << p;
+      }
+    } else {
+      double sd[MG];
+#pragma unroll
+      for (int p = 0; p < MG; ++p) sd[p] = (double)wv[p] * (double)wv[p] * (double)hv[p];
+#pragma unroll
+      for (int p = 0; p < MG; ++p) {
+        int beaten = 0;
+#pragma unroll
+        for (int q = 0; q < MG; ++q) beaten += (q != p) && (sd[q] > sd[p] || (sd[q] == sd[p] && q < p));
+        if (beaten < n_keep) m |= 1u << p;
+      }
     }
     M[g] = (uint8_t)m;
 #pragma unroll
@@ -252,24 +303,28 @@ __device__ __forceinline__ void start_record(armor_iter_stats* st, double loss) 
   st->reserved = 0;
 }
 
+// advance: the iteration counter moves on first (every iteration of a call but its first).
 // carry_loss: the running loss of the previous iteration becomes this iteration's starting loss, and the
 // iteration's record is opened here (no loss evaluation follows)
+static_assert(SC_COUNT == 32, "one scalar per lane");
 __global__ void zero_scalars_kernel(double* sc, int32_t* failflag, int nflag, int carry_loss, armor_iter_stats* st_base,
-                                    const int64_t* __restrict__ it_dev) {
-  armor_iter_stats* st = st_base ? st_base + *it_dev : nullptr;
+                                    int64_t* it_dev, int advance) {
   const double carried = sc[SC_LOSS];
   __syncthreads();
   for (int i = threadIdx.x; i < SC_COUNT; i += blockDim.x)
     sc[i] = (carry_loss && (i == SC_L0 || i == SC_LOSS)) ? carried : 0.0;
   for (int i = threadIdx.x; i < nflag; i += blockDim.x) failflag[i] = 0;
-  if (carry_loss && st && threadIdx.x == 0) start_record(st, carried);
+  if (threadIdx.x == 0) {
+    const int64_t it = *it_dev + advance;
+    if (advance) *it_dev = it;
+    if (carry_loss && st_base) start_record(st_base + it, carried);
+  }
 }
 
 // Fixed-order sums by the CTA of the bookkeeping kernel (STAGE_NT threads): thread t adds entries t, t + STAGE_NT, ...
-// (eight loads in flight), a shuffle tree per warp, then the warps in order.  All threads get the sum.  The line
-// searches hand over thousands of partial sums (four or eight per tile); one warp took 14 us over them.
-constexpr int STAGE_NT = 256;
-__device__ __forceinline__ double stage_sum_f64(const double* __restrict__ p, int n, double* scratch) {
+// (eight loads in flight).  The line searches hand over thousands of partial sums (four or eight per tile).
+constexpr int STAGE_NT = 1024;
+__device__ __forceinline__ double stage_thread_sum(const double* __restrict__ p, int n) {
   double v = 0.0;
   int i = threadIdx.x;
   for (; i + 7 * STAGE_NT < n; i += 8 * STAGE_NT) {
@@ -279,46 +334,14 @@ __device__ __forceinline__ double stage_sum_f64(const double* __restrict__ p, in
 #pragma unroll
     for (int u = 0; u < 8; ++u) v += t[u];
   }
+#pragma unroll 4
   for (; i < n; i += STAGE_NT) v += p[i];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < STAGE_NT / 32; ++w) t += scratch[w];
-  __syncthreads();
-  return t;
-}
-__device__ __forceinline__ int stage_count_flags(const int32_t* __restrict__ f, int n, double* scratch) {
-  int v = 0;
-  for (int i = threadIdx.x; i < n; i += STAGE_NT) v += f[i] ? 1 : 0;
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0) scratch[threadIdx.x >> 5] = (double)v;
-  __syncthreads();
-  int t = 0;
-  for (int w = 0; w < STAGE_NT / 32; ++w) t += (int)scratch[w];
-  __syncthreads();
-  return t;
+  return v;
 }
 
-// stage 0: start, 1: after A, 2: after B, 3 / 6: after S, 4: mask accept, 5: mask phase off.  One CTA of STAGE_NT threads.
-// Up to two arrays of partial sums (p1, p2) are first added, in a fixed order, into the scalars slot1 / slot2: the
-// reductions of the dot products that precede the stage need no launch of their own.
-__global__ void advance_iteration_kernel(int64_t* it_dev) { *it_dev += 1; }
-
-__global__ void stage_kernel(double* sc, armor_iter_stats* st_base, const int64_t* __restrict__ it_dev, int stage,
-                             const int32_t* failflag, int nflag,
-                             const double* partA, int nA, int32_t* status, const double* p1, int n1, int slot1,
-                             const double* p2, int n2, int slot2) {
-  armor_iter_stats* st = st_base ? st_base + *it_dev : nullptr;
-  __shared__ double scratch[STAGE_NT / 32];
-  if (p1) { const double v = stage_sum_f64(p1, n1, scratch); if (threadIdx.x == 0) sc[slot1] = v; }
-  if (p2) { const double v = stage_sum_f64(p2, n2, scratch); if (threadIdx.x == 0) sc[slot2] = v; }
-  double psum = 0.0;
-  int nf = 0;
-  if (stage == 1 || stage == 2 || stage == 4) psum = stage_sum_f64(partA, nA, scratch);
-  if (stage == 1 || stage == 2) nf = stage_count_flags(failflag, nflag, scratch);
-  if (threadIdx.x != 0) return;
-  const bool poisoned = status[ST_POISON] != 0;   // unusable inputs: every step length is zero, nothing is accepted
+// One thread's part of a stage: step lengths, accept flag, running loss, the iteration's record.
+__device__ __forceinline__ void stage_scalars(double* sc, armor_iter_stats* st, int stage, double psum, int nf, int32_t* status,
+                                              bool poisoned) {
   if (stage == 0) {
     sc[SC_LOSS] = sc[SC_L0];
     if (st) start_record(st, sc[SC_L0]);
@@ -376,6 +399,59 @@ __global__ void stage_kernel(double* sc, armor_iter_stats* st_base, const int64_
     sc[SC_DL_M] = 0.0;
     if (st) st->loss_mask = sc[SC_LOSS];
   }
+}
+
+// stage 0: start, 1: after A, 2: after B, 3 / 6: after S, 4: mask accept, 5: mask phase off.  One CTA of STAGE_NT threads.
+// Up to two arrays of partial sums (p1, p2) are first added, in a fixed order, into the scalars slot1 / slot2: the
+// reductions of the dot products that precede the stage need no launch of their own.
+// All sums of a call go through one shuffle tree and one barrier; the scalars and the record thread 0 will need are on their
+// way meanwhile (the kernel is nothing but latency: as a chain of separate sums it took 4 to 6 us, four times an iteration).
+__global__ void __launch_bounds__(STAGE_NT)
+stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* __restrict__ it_dev, int stage, int32_t* failflag,
+             int nflag, int nflag_clear, const double* partA, int nA, int32_t* status, const double* p1, int n1, int slot1,
+             const double* p2, int n2, int slot2) {
+  __shared__ double sc[SC_COUNT];
+  __shared__ double sums[3][STAGE_NT / 32];
+  __shared__ int flags[STAGE_NT / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double mine = threadIdx.x < SC_COUNT ? sc_g[threadIdx.x] : 0.0;
+  armor_iter_stats* st = nullptr;
+  bool poisoned = false;                  // unusable inputs: every step length is zero, nothing is accepted
+  if (threadIdx.x == 0) {
+    if (st_base) st = st_base + *it_dev;
+    poisoned = status[ST_POISON] != 0;
+  }
+  double v[3] = {0.0, 0.0, 0.0};
+  int nf = 0;
+  if (p1) v[0] = stage_thread_sum(p1, n1);
+  if (p2) v[1] = stage_thread_sum(p2, n2);
+  if (stage == 1 || stage == 2 || stage == 4) v[2] = stage_thread_sum(partA, nA);
+  if (stage == 1 || stage == 2)
+    for (int i = threadIdx.x; i < nflag; i += STAGE_NT) nf += failflag[i] ? 1 : 0;
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    nf += __shfl_xor_sync(0xffffffffu, nf, o);
+  }
+  if (threadIdx.x < SC_COUNT) sc[threadIdx.x] = mine;
+  if (lane == 0) { sums[0][warp] = v[0]; sums[1][warp] = v[1]; sums[2][warp] = v[2]; flags[warp] = nf; }
+  __syncthreads();
+  // (the flags have been counted: the next solves raise them again)
+  for (int i = threadIdx.x; i < nflag_clear; i += STAGE_NT) failflag[i] = 0;
+  if (warp != 0) return;
+  v[0] = sums[0][lane]; v[1] = sums[1][lane]; v[2] = sums[2][lane]; nf = flags[lane];
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
+    nf += __shfl_xor_sync(0xffffffffu, nf, o);
+  }
+  if (lane == 0) {
+    if (p1) sc[slot1] = v[0];
+    if (p2) sc[slot2] = v[1];
+    stage_scalars(sc, st, stage, v[2], nf, status, poisoned);
+  }
+  __syncwarp();
+  sc_g[lane] = sc[lane];                  // SC_COUNT == 32
 }
 
 // ---- input screening -----------------------------------------------------------------------------
@@ -581,11 +657,6 @@ void reduce_partials_to(armor_ctx* c, const double* part, int n, double* out, cu
   c->launches++;
 }
 
-void launch_zero_flags(armor_ctx* c, cudaStream_t s) {
-  const int nflag = c->nbo > c->nbi ? c->nbo : c->nbi;
-  cudaMemsetAsync(c->failflag, 0, (size_t)nflag * sizeof(int32_t), s);
-}
-
 void launch_colscale(armor_ctx* c, const float* in, const float* h, float* out, int64_t rows, int64_t cols,
                      cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_AXPY, 8.0 * (double)rows * (double)cols, s);
@@ -603,7 +674,7 @@ void launch_scale_rows_cols(armor_ctx* c, const float* in, const float* colscale
 
 void launch_extract_hblocks(armor_ctx* c, const float* H, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  extract_hblocks_kernel<<<c->nbi, NT, 0, s>>>(H, c->hdiag, c->Hjj, c->d_in, c->db, c->cfg.h_mode == ARMOR_H_DIAG);
+  extract_hblocks_kernel<<<dim3(c->nbi, (c->db + HB_ROWS - 1) / HB_ROWS), NT, 0, s>>>(H, c->hdiag, c->Hjj, c->d_in, c->db, c->cfg.h_mode == ARMOR_H_DIAG);
   c->launches++;
 }
 
@@ -620,18 +691,21 @@ void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slo
   c->launches++;
 }
 
-// y_k += sign_k * sc[slot] * x_k for up to three pairs of length n (a pair with y == nullptr is skipped)
-void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, float* y1, const float* x1, float s1, float* y2,
-                       const float* x2, float s2, int64_t n, int slot, cudaStream_t s) {
+// y_k += sign_k * sc[slot] * x_k for up to three pairs of lengths n_k (a pair with y == nullptr is skipped)
+void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64_t n0, float* y1, const float* x1, float s1,
+                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s) {
   AxpyTerm t[3];
   int k = 0;
-  if (y0) t[k++] = {(float4*)y0, (const float4*)x0, s0};
-  if (y1) t[k++] = {(float4*)y1, (const float4*)x1, s1};
-  if (y2) t[k++] = {(float4*)y2, (const float4*)x2, s2};
+  if (y0) t[k++] = {(float4*)y0, (const float4*)x0, s0, n0 / 4};
+  if (y1) t[k++] = {(float4*)y1, (const float4*)x1, s1, n1 / 4};
+  if (y2) t[k++] = {(float4*)y2, (const float4*)x2, s2, n2 / 4};
   if (k == 0) return;
+  int64_t n4 = 0;
+  double elems = 0.0;
+  for (int j = 0; j < k; ++j) { n4 = t[j].n4 > n4 ? t[j].n4 : n4; elems += 4.0 * (double)t[j].n4; }
   for (int j = k; j < 3; ++j) t[j] = t[0];
-  KTimer kt(c, n >= (1 << 22) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * (double)n * k, s);
-  axpy_multi_slot_kernel<<<grid_for(n / 4), NT, 0, s>>>(t[0], t[1], t[2], k, n / 4, c->sc, slot);
+  KTimer kt(c, n4 >= (1 << 20) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * elems, s);
+  axpy_multi_slot_kernel<<<grid_for(n4), NT, 0, s>>>(t[0], t[1], t[2], k, n4, c->sc, slot);
   c->launches++;
 }
 
@@ -653,15 +727,16 @@ void launch_init(armor_ctx* c, const float* W, const float* H, float* Wbar, floa
     c->launches++;
   }
   const int mg = c->cfg.m_group;
+  diag_kernel<<<(unsigned)((cols + NT - 1) / NT), NT, 0, s>>>(H, c->hdiag, cols);
   if (mg == 8)
-    init_core_kernel<8><<<grid_for(c->wn / 8), NT, 0, s>>>(Wbar, H, cols, S, M, c->wn / 8, (int)(cols / 8),
+    init_core_kernel<8><<<grid_for(c->wn / 8), NT, 0, s>>>(Wbar, c->hdiag, S, M, c->wn / 8, (int)(cols / 8),
                                                           c->cfg.n_keep);
   else
-    init_core_kernel<4><<<grid_for(c->wn / 4), NT, 0, s>>>(Wbar, H, cols, S, M, c->wn / 4, (int)(cols / 4),
+    init_core_kernel<4><<<grid_for(c->wn / 4), NT, 0, s>>>(Wbar, c->hdiag, S, M, c->wn / 4, (int)(cols / 4),
                                                           c->cfg.n_keep);
   identity_blocks_kernel<<<c->nbo, NT, 0, s>>>(A, c->db);
   identity_blocks_kernel<<<c->nbi, NT, 0, s>>>(B, c->db);
-  c->launches += 3;
+  c->launches += 4;
 }
 
 armor_status launch_screen_inputs(armor_ctx* c, const float* W, const float* H, cudaStream_t s) {
@@ -676,24 +751,19 @@ armor_status launch_screen_inputs(armor_ctx* c, const float* W, const float* H, 
   return ARMOR_OK;
 }
 
-void launch_zero_scalars(armor_ctx* c, bool carry_loss, armor_iter_stats* st, cudaStream_t s) {
+void launch_zero_scalars(armor_ctx* c, bool advance, bool carry_loss, armor_iter_stats* st, cudaStream_t s) {
   const int nflag = c->nbo > c->nbi ? c->nbo : c->nbi;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  zero_scalars_kernel<<<1, NT, 0, s>>>(c->sc, c->failflag, nflag, carry_loss ? 1 : 0, st, c->it_dev);
-  c->launches++;
-}
-
-void launch_advance_iteration(armor_ctx* c, cudaStream_t s) {
-  KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  advance_iteration_kernel<<<1, 1, 0, s>>>(c->it_dev);
+  zero_scalars_kernel<<<1, NT, 0, s>>>(c->sc, c->failflag, nflag, carry_loss ? 1 : 0, st, c->it_dev, advance ? 1 : 0);
   c->launches++;
 }
 
 void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, int nflag,
                   cudaStream_t s, const double* p1, int n1, int slot1, const double* p2, int n2, int slot2) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  stage_kernel<<<1, STAGE_NT, 0, s>>>(c->sc, st, c->it_dev, stage, c->failflag, nflag, part, npart, c->status, p1, n1, slot1,
-                               p2, n2, slot2);
+  const int nflag_clear = stage == 1 ? (c->nbo > c->nbi ? c->nbo : c->nbi) : 0;     // the B-step's solves start afresh
+  stage_kernel<<<1, STAGE_NT, 0, s>>>(c->sc, st, c->it_dev, stage, c->failflag, nflag, nflag_clear, part, npart, c->status, p1,
+                                      n1, slot1, p2, n2, slot2);
   c->launches++;
 }
 

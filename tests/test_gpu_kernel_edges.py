@@ -178,3 +178,46 @@ def test_core_step_with_the_mask_applied_in_the_gradient(n_keep, m_group, mode, 
     assert (st.S[~keep] == 0).all()
     assert (move - tau * Gm).norm() <= 2e-5 * (tau * Gm).norm() + 2.0 ** -24 * S0.double().norm()
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("m_group,n_keep", [(4, 2), (8, 4), (8, 6)])
+def test_initial_mask_orders_scores_as_fp64_does(m_group, n_keep):
+    """Scores that fp32 cannot tell apart (equal magnitudes, one ulp apart, products that underflow, overflow or vanish)
+    are ordered by their fp64 values, ties to the lower column."""
+    d_out, d_in, db = 64, 256, 16
+    g = _gen(m_group + n_keep)
+    from paper_2510_05528_b200 import binding as Bd
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    W[8:16] = W[8:16].sign()
+    W[16:24] = W[16:24].sign() * torch.nextafter(torch.ones(1, device=DEV), torch.full((1,), 2.0, device=DEV)) ** \
+        torch.randint(0, 3, (8, d_in), device=DEV, generator=g).float()
+    W[24:32] *= 1e-25
+    W[32:40] *= 1e19
+    W[40:44] = 0.0
+    h = torch.exp(2 * torch.randn(d_in, device=DEV, generator=g))
+    h[:64] = 1.0
+    h[64:72] = 0.0
+    ctx = _ctx(d_out, d_in, db, precision=Bd.PREC_SIMT, h_mode=Bd.H_DIAG, m_group=m_group, n_keep=n_keep)
+    st = ctx.init(W, torch.diag(h))
+    sc = (W.double() * W.double() * h.double()).view(d_out, -1, m_group)
+    order = torch.argsort(sc, dim=2, descending=True, stable=True)[:, :, :n_keep]
+    keep = torch.zeros_like(sc, dtype=torch.bool).scatter_(2, order, True)
+    bits = (keep * (1 << torch.arange(m_group, device=DEV))).sum(2).to(torch.uint8)
+    assert torch.equal(st.M, bits)
+
+
+@pytest.mark.parametrize("scale", [1.0, 1e-18, 1e16])
+def test_row_norms_of_the_normalisation(scale):
+    """r2 against fp64 to one rounding (2^-23 relative covers the rounding of r1 in the quotient's place: r1 itself is
+    taken as stored), for widths below and above a CTA's stride, with a zero row and a zero column."""
+    from paper_2510_05528_b200 import binding as Bd
+    for d_in in (64, 1024, 4352):
+        g = _gen(d_in)
+        W = torch.randn(96, d_in, device=DEV, generator=g) * torch.exp(3 * torch.randn(d_in, device=DEV, generator=g)) * scale
+        W[5] = 0.0
+        W[:, 7] = 0.0
+        ctx = _ctx(96, d_in, 32, precision=Bd.PREC_SIMT, h_mode=Bd.H_DIAG, normalize=1)
+        st = ctx.init(W, torch.eye(d_in, device=DEV))
+        r2 = (W.double() / st.r1.double()).norm(dim=1)
+        r2[5] = 1.0
+        assert ((st.r2.double() - r2).abs() <= 2.0 ** -23 * r2).all()
