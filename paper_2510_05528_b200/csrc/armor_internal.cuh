@@ -248,6 +248,16 @@ armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, cons
 armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* out,
                                    int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
 
+// products and per-block Grams of 256 x 256 blocks on pairs of CTAs (blockpair_tcgen05.cu)
+bool tc_blockpair_ok(const armor_ctx* c);
+armor_status tc_blockpair_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
+                                int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
+armor_status tc_blockpair_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
+                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s,
+                               const float* in2 = nullptr, double* part = nullptr, int* n_part = nullptr);
+armor_status tc_blockpair_gram(armor_ctx* c, const float* P, const float* T, bool by_rows, float* G, int n_split, cudaStream_t s,
+                               const float* P2 = nullptr, float* G2 = nullptr);
+
 // per-block Grams over a long contraction on the tensor cores
 bool tc_gram_ok(const armor_ctx* c);
 armor_status tc_rowblock_gram(armor_ctx* c, const float* P, const float* T, float* G, cudaStream_t s);
@@ -300,6 +310,11 @@ armor_status gram_accumulate(armor_ctx* c, const void* X, int x_dtype, int64_t n
 // z2 [n, d_out] = z1 [n, d_in] * S^T
 armor_status apply_core(armor_ctx* c, const float* z1, const float* S, const void* packed, float* z2, int64_t n,
                         bool bf16, cudaStream_t s);
+
+// the same in the three-pass fp16 mode with S split beforehand (once per call), up to gram_rows tokens at a time
+bool core_f16_ok(const armor_ctx* c);
+void core_f16_split_S(armor_ctx* c, const float* S, cudaStream_t s);
+armor_status core_f16_product(armor_ctx* c, const float* z1, float* z2, int64_t n, cudaStream_t s);
 
 // operand preparation of the three-pass fp16 mode (split_f16.cu)
 void launch_f16_prepare_H(armor_ctx* c, const float* H, cudaStream_t s);   // hpow, scaled H as fp16 hi | lo in Hlo
