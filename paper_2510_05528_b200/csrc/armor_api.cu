@@ -737,7 +737,15 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
                                cudaStream_t s) {
   const size_t esz = bf16 ? 2 : 4;
   const int64_t d_out = c->d_out, d_in = c->d_in;
-  const int64_t chunk = d_out < d_in ? d_out : d_in;   // z1 [chunk, d_in] and z2 [chunk, d_out] fit W-shaped scratch
+  // fp32 activations in the three-pass fp16 mode: the W-shaped buffers that lie side by side take z1 (T, E, EH, P) and
+  // z2 (V to WH: five), the Gram's staging buffer takes the split z1, S is split once (U).  A chunk of four times the tokens
+  // needs a quarter of the splits of S and leaves no short chunk behind (8,195 tokens of a 4096 x 4096 layer came as 4,096,
+  // 4,096 and 3).
+  const bool wide = !bf16 && !packed && c->cfg.precision == ARMOR_PREC_FP16X3 && core_f16_ok(c);
+  int64_t chunk = d_out < d_in ? d_out : d_in;   // z1 [chunk, d_in] and z2 [chunk, d_out] fit W-shaped scratch
+  if (wide) chunk = 4 * chunk < c->gram_rows ? 4 * chunk : c->gram_rows;
+  float* const z2 = wide ? c->V : c->E;
+  if (wide) core_f16_split_S(c, S, s);
   for (int64_t t0 = 0; t0 < n_tokens; t0 += chunk) {
     const int64_t n = (n_tokens - t0 < chunk) ? n_tokens - t0 : chunk;
     const float* xc;
@@ -752,18 +760,19 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
       xc = static_cast<const float*>(d_x) + t0 * d_in;
       yc = static_cast<float*>(d_y) + t0 * d_out;
       if (r1) {
-        launch_scale_rows_cols(c, xc, r1, nullptr, c->Tmp, n, d_in, s);
-        xc = c->Tmp;
+        float* xs = wide ? c->V : c->Tmp;      // (z2 takes its place after z1 is formed)
+        launch_scale_rows_cols(c, xc, r1, nullptr, xs, n, d_in, s);
+        xc = xs;
       }
     }
     // the bf16 forward rounds z1, S and y to 8 bits: its wrapper products take one tf32 pass (11 bits)
     c->block_one_pass = bf16 ? 1 : 0;
     bd_right(c, xc, B, true, c->T, n, d_in, 1.f, nullptr, 0.f, s);                   // z1 = x B^T
     c->block_one_pass = 0;
-    armor_status st = apply_core(c, c->T, S, packed, c->E, n, bf16, s);              // z2 = z1 S^T
+    armor_status st = wide ? core_f16_product(c, c->T, z2, n, s) : apply_core(c, c->T, S, packed, z2, n, bf16, s);   // z2 = z1 S^T
     if (st != ARMOR_OK) return st;
     c->block_one_pass = bf16 ? 1 : 0;
-    bd_right(c, c->E, A, true, yc, n, d_out, 1.f, nullptr, 0.f, s);                  // y = z2 A^T
+    bd_right(c, z2, A, true, yc, n, d_out, 1.f, nullptr, 0.f, s);                    // y = z2 A^T
     c->block_one_pass = 0;
     if (bf16) launch_f32_to_bf16(c, yc, r2, static_cast<char*>(d_y) + (size_t)(t0 * d_out) * esz, n, d_out, s);
     else if (r2) launch_scale_rows_cols(c, yc, r2, nullptr, yc, n, d_out, s);

@@ -204,6 +204,33 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
   return ARMOR_OK;
 }
 
+// The core product of the fp32 forward in the three-pass fp16 mode: rows of z1 (tokens) and rows of S (outputs) each scaled
+// by their own power of two.  S is split once for all chunks of a call, into U; z1 into the Gram's staging buffer, whose
+// gram_rows x d_in words hold the two parts of up to gram_rows tokens, with the scales in the normalisation's scratch (128
+// d_in floats).
+bool core_f16_ok(const armor_ctx* c) {
+  return c->cfg.precision == ARMOR_PREC_FP16X3 && c->d_out % 32 == 0 && c->d_in % 8 == 0;
+}
+void core_f16_split_S(armor_ctx* c, const float* S, cudaStream_t s) {
+  __half* shi = reinterpret_cast<__half*>(c->U);
+  launch_f16_split_rows(c, S, c->d_in, c->d_out, c->d_in, nullptr, 1.f, shi, shi + c->wn, c->rowscale2, s);
+}
+armor_status core_f16_product(armor_ctx* c, const float* z1, float* z2, int64_t n, cudaStream_t s) {
+  const int64_t d_in = c->d_in, d_out = c->d_out;
+  __half* ahi = reinterpret_cast<__half*>(c->Xt_hi);
+  __half* shi = reinterpret_cast<__half*>(c->U);
+  float* scales = reinterpret_cast<float*>(c->colpart);         // 64 d_in doubles
+  launch_f16_split_rows(c, z1, d_in, n, d_in, nullptr, 1.f, ahi, ahi + n * d_in, scales, s);
+  TcGemm g{};
+  g.lda = d_in; g.ldb = d_in; g.ldc = d_out;
+  g.M = n; g.N = d_out; g.K = d_in;
+  g.C = z2;
+  g.A = ahi; g.Alo = ahi + n * d_in; g.B = shi; g.Blo = shi + c->wn; g.passes = 6; g.fp16 = 1;
+  g.row_scale = scales; g.col_scale = c->rowscale2;
+  g.k_segment = K_SEGMENT;
+  return launch_tc_gemm(c, g, nullptr, s);
+}
+
 armor_status apply_core(armor_ctx* c, const float* z1, const float* S, const void* packed, float* z2, int64_t n,
                         bool bf16, cudaStream_t s) {
   const int64_t d_in = c->d_in, d_out = c->d_out;
@@ -244,14 +271,11 @@ armor_status apply_core(armor_ctx* c, const float* z1, const float* S, const voi
     launch_split_hilo(c, z1, nullptr, c->Lo, n * d_in, s);
     launch_split_hilo(c, S, nullptr, c->U, c->wn, s);
     g.A = z1; g.Alo = c->Lo; g.B = S; g.Blo = c->U; g.passes = 3;
+  } else if (core_f16_ok(c)) {
+    core_f16_split_S(c, S, s);
+    return core_f16_product(c, z1, z2, n, s);
   } else if (c->cfg.precision == ARMOR_PREC_FP16X3) {
-    // rows of z1 (tokens) and rows of S (outputs) each scaled by their own power of two
-    __half* ahi = reinterpret_cast<__half*>(c->Lo);
-    __half* shi = reinterpret_cast<__half*>(c->U);
-    launch_f16_split_rows(c, z1, d_in, n, d_in, nullptr, 1.f, ahi, ahi + n * d_in, c->rowscale, s);
-    launch_f16_split_rows(c, S, d_in, d_out, d_in, nullptr, 1.f, shi, shi + c->wn, c->rowscale2, s);
-    g.A = ahi; g.Alo = ahi + n * d_in; g.B = shi; g.Blo = shi + c->wn; g.passes = 6; g.fp16 = 1;
-    g.row_scale = c->rowscale; g.col_scale = c->rowscale2;
+    return ARMOR_ERR_UNSUPPORTED;
   } else {
     g.A = z1; g.B = S; g.passes = 1;
   }

@@ -94,7 +94,10 @@ __global__ void __launch_bounds__(NT) split_H_kernel(const float4* __restrict__ 
 }
 
 // One CTA per row of `in` [rows, cols] (leading dimension ld): the row times the column scales, brought into
-// range by a power of two of its own; out_scale[row] = post / that power.
+// range by a power of two of its own; out_scale[row] = post / that power.  KEEP float4 per thread stay in registers between
+// the maximum and the split (0: the row is read again).  The scaling is a product with a power of two: exact, or rounded
+// once where the result is subnormal.
+template <int KEEP>
 __global__ void __launch_bounds__(NT) split_rows_kernel(const float* __restrict__ in, int64_t ld, int64_t cols,
                                                         const float* __restrict__ colscale, float post,
                                                         __half2* __restrict__ hi, __half2* __restrict__ lo,
@@ -103,27 +106,48 @@ __global__ void __launch_bounds__(NT) split_rows_kernel(const float* __restrict_
   const float4* src = reinterpret_cast<const float4*>(in + row * ld);
   const float4* cs4 = reinterpret_cast<const float4*>(colscale);
   const int64_t c4n = cols / 4;
-  float mx = 0.f;
-  for (int64_t i = threadIdx.x; i < c4n; i += NT) {
+  auto fetch = [&](int64_t i) {
     float4 v = src[i];
-    if (colscale) { const float4 d = cs4[i]; v.x *= d.x; v.y *= d.y; v.z *= d.z; v.w *= d.w; }
-    mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w))));
+    if (colscale) { const float4 d = __ldg(cs4 + i); v.x *= d.x; v.y *= d.y; v.z *= d.z; v.w *= d.w; }
+    return v;
+  };
+  auto larger = [](float m, const float4& v) { return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
+  float4 kept[KEEP > 0 ? KEEP : 1];
+  float mx = 0.f;
+  if (KEEP > 0) {
+#pragma unroll
+    for (int u = 0; u < KEEP; ++u) {
+      const int64_t i = threadIdx.x + (int64_t)u * NT;
+      kept[u] = i < c4n ? fetch(i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int u = 0; u < KEEP; ++u) mx = larger(mx, kept[u]);
+  } else {
+    for (int64_t i = threadIdx.x; i < c4n; i += NT) mx = larger(mx, fetch(i));
   }
   mx = block_max(mx);
   const int e = scale_exp(mx);
+  const float p = scalbnf(1.f, e);
   if (threadIdx.x == 0) out_scale[row] = scalbnf(post, -e);
-  __half2* dh = hi + row * (cols / 2);
-  __half2* dl = lo + row * (cols / 2);
-  for (int64_t i = threadIdx.x; i < c4n; i += NT) {
-    float4 v = src[i];
-    if (colscale) { const float4 d = cs4[i]; v.x *= d.x; v.y *= d.y; v.z *= d.z; v.w *= d.w; }
-    __half h0, h1, h2, h3, l0, l1, l2, l3;
-    split2(scalbnf(v.x, e), h0, l0);
-    split2(scalbnf(v.y, e), h1, l1);
-    split2(scalbnf(v.z, e), h2, l2);
-    split2(scalbnf(v.w, e), h3, l3);
-    dh[2 * i] = __halves2half2(h0, h1); dh[2 * i + 1] = __halves2half2(h2, h3);
-    dl[2 * i] = __halves2half2(l0, l1); dl[2 * i + 1] = __halves2half2(l2, l3);
+  uint2* dh = reinterpret_cast<uint2*>(hi + row * (cols / 2));
+  uint2* dl = reinterpret_cast<uint2*>(lo + row * (cols / 2));
+  auto put = [&](int64_t i, const float4& v) {
+    __half2 h[2], l[2];
+    split2(v.x * p, h[0].x, l[0].x);
+    split2(v.y * p, h[0].y, l[0].y);
+    split2(v.z * p, h[1].x, l[1].x);
+    split2(v.w * p, h[1].y, l[1].y);
+    dh[i] = *reinterpret_cast<const uint2*>(h);
+    dl[i] = *reinterpret_cast<const uint2*>(l);
+  };
+  if (KEEP > 0) {
+#pragma unroll
+    for (int u = 0; u < KEEP; ++u) {
+      const int64_t i = threadIdx.x + (int64_t)u * NT;
+      if (i < c4n) put(i, kept[u]);
+    }
+  } else {
+    for (int64_t i = threadIdx.x; i < c4n; i += NT) put(i, fetch(i));
   }
 }
 
@@ -211,8 +235,12 @@ void launch_f16_prepare_H(armor_ctx* c, const float* H, cudaStream_t s) {
 void launch_f16_split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t rows, int64_t cols, const float* colscale,
                            float post, void* hi, void* lo, float* out_scale, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 8.0 * (double)rows * (double)cols, s);
-  split_rows_kernel<<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, static_cast<__half2*>(hi),
-                                                  static_cast<__half2*>(lo), out_scale);
+  __half2 *h = static_cast<__half2*>(hi), *l = static_cast<__half2*>(lo);
+  // a row in registers up to 8,192 columns: one read of it instead of two (from L1 or L2)
+  if (cols <= 4 * NT) split_rows_kernel<1><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
+  else if (cols <= 16 * NT) split_rows_kernel<4><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
+  else if (cols <= 32 * NT) split_rows_kernel<8><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
+  else split_rows_kernel<0><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
   c->launches++;
 }
 

@@ -221,3 +221,81 @@ def test_row_norms_of_the_normalisation(scale):
         r2 = (W.double() / st.r1.double()).norm(dim=1)
         r2[5] = 1.0
         assert ((st.r2.double() - r2).abs() <= 2.0 ** -23 * r2).all()
+
+
+@pytest.mark.parametrize("rows,cols", [(256, 256), (200, 768), (1025, 512), (512, 260), (2560, 2048)])
+@pytest.mark.parametrize("side,transpose", [(0, 0), (0, 1), (1, 0), (1, 1)])
+def test_products_with_blocks_of_256_on_pairs_of_ctas(rows, cols, side, transpose):
+    """The kernel for pairs of CTAs gives the bits of the streaming kernel (path 1): same operand parts, same order of MMAs;
+    ragged rows of a right product and columns of a left one, with an addend, in place."""
+    from paper_2510_05528_b200 import binding as Bd
+    if (cols if side == 0 else rows) % 256:
+        pytest.skip("not a shape of this side")
+    g = _gen(rows + cols)
+    ctx = _ctx(2560, 2048, 256)
+    X = torch.randn(rows, cols, device=DEV, generator=g)
+    D = torch.randn(rows, cols, device=DEV, generator=g)
+    Q = torch.randn((rows if side else cols) // 256, 256, 256, device=DEV, generator=g)
+    out = {}
+    for path in (1, -1):
+        a, b = torch.full_like(X, 7.0), D.clone()
+        Bd.armor_block_product(ctx.ctx, side, transpose, Q, X, a, 1.5, None, 0.0, path)
+        Bd.armor_block_product(ctx.ctx, side, transpose, Q, X, b, -1.0, b, 1.0, path)
+        out[path] = (a, b)
+    assert torch.equal(out[1][0], out[-1][0]) and torch.equal(out[1][1], out[-1][1])
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in", [(256, 256), (512, 2304), (4864, 768)])
+def test_dual_product_and_grams_with_blocks_of_256(d_out, d_in):
+    """Dual product: the bits of the streaming kernel, the dot product to the order of its fp64 partial sums; A- and B-step of
+    one iteration (both Grams of either) likewise against a run on the streaming kernels' results in fp64."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + d_in)
+    ctx = _ctx(d_out, d_in, 256)
+    Q = torch.randn(d_out // 256, 256, 256, device=DEV, generator=g) / 16
+    X1, X2 = (torch.randn(d_out, d_in, device=DEV, generator=g) for _ in range(2))
+    a, b = torch.empty_like(X1), torch.empty_like(X1)
+    d1 = Bd.armor_block_product_dual(ctx.ctx, Q, X1, X2, a, path=1)
+    d2 = Bd.armor_block_product_dual(ctx.ctx, Q, X1, X2, b, path=-1)
+    assert torch.equal(a, b)
+    V1, V2 = (torch.matmul(Q.double(), X.double().view(-1, 256, d_in)) for X in (X1, X2))
+    for d in (d1, d2):
+        assert abs(d - (V1 * V2).sum().item()) <= 2e-6 * (V1.norm() * V2.norm()).item()
+    # A-step alone with the diagonal weighting: X = E D T^T (T D T^T + lam I)^-1 per row block
+    h = torch.rand(d_in, device=DEV, generator=g) + 0.5
+    ctx = _ctx(d_out, d_in, 256, h_mode=Bd.H_DIAG, phases=1)
+    st = ctx.init(X1, torch.diag(h))
+    A0, S0 = st.A.clone().double(), st.S.clone()
+    ctx.bcd_step(st, torch.diag(h), 0, 1)
+    T, E = (M.double().view(-1, 256, d_in) for M in (S0, X1 - S0))
+    G = (T * h.double()) @ T.transpose(1, 2)
+    G = G + 1e-6 * G.diagonal(dim1=1, dim2=2).mean(1)[:, None, None] * torch.eye(256, device=DEV, dtype=torch.float64)
+    X = torch.linalg.solve(G, ((E * h.double()) @ T.transpose(1, 2)).transpose(1, 2)).transpose(1, 2)
+    cond = torch.linalg.cond(G).max().item()
+    assert (st.A.double() - A0 - X).norm() <= max(1e-4, 1e-6 * cond) * X.norm()
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(64, 64, 32), (256, 128, 128), (384, 1280, 128), (512, 256, 256)])
+@pytest.mark.parametrize("normalize", [0, 1])
+def test_fp32_forward_over_chunk_edges(d_out, d_in, d_block, normalize):
+    """y = A S B x in fp32 for token counts below, at and above a chunk (four times the smaller dimension).  Bound: each of the three
+    products adds at most 3 x 128 / 8 truncated sums of its wrapper's (the core's: one segment's) accumulator, 48 x 2^-24 =
+    2.9e-6 of the result each, beside 2^-21 for the parts left out: 1e-5 in all."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + d_in + normalize)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    ctx = _ctx(d_out, d_in, d_block, h_mode=Bd.H_DIAG, normalize=normalize)
+    st = ctx.init(W, torch.eye(d_in, device=DEV))
+    st.A.add_(torch.randn(st.A.shape, device=DEV, generator=g) * 0.1)
+    st.B.add_(torch.randn(st.B.shape, device=DEV, generator=g) * 0.1)
+    Wh = torch.block_diag(*st.A.double()) @ st.S.double() @ torch.block_diag(*st.B.double())
+    if normalize:
+        Wh = st.r2.double()[:, None] * Wh * st.r1.double()[None, :]
+    chunk = min(4 * min(d_out, d_in), 16384)
+    for n in (1, 3, chunk - 1, chunk, chunk + 1, 2 * chunk + 77):
+        x = torch.randn(n, d_in, device=DEV, generator=g)
+        y = ctx.apply(st, x, denormalize=bool(normalize)).double()
+        ref = x.double() @ Wh.t()
+        assert (y - ref).norm() <= 1e-5 * ref.norm(), n
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
