@@ -90,7 +90,7 @@ struct armor_ctx {
   float *hpow, *rowscale, *rowscale2, *gscale;
   float* gscale2;       // output scales of the chunk staged in Xt_hi2
   unsigned* gmax;
-  // Gram staging (transposed, split chunk of X)
+  // Gram staging (split chunk of X; transposed in the tf32 modes)
   float *Xt_hi, *Xt_lo;
   float* Xt_hi2;        // second staging buffer (FP16X3): chunk p + 1 is staged on side_stream while chunk p is contracted
   cudaStream_t side_stream;
@@ -322,7 +322,7 @@ void launch_f16_split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t ro
                            float post, void* hi, void* lo, float* out_scale, cudaStream_t s);
 float f16_H_post_scale();
 armor_status launch_f16_gram_stage(armor_ctx* c, const void* X, int x_dtype, int64_t ldx, int64_t rows, int64_t cols,
-                                   void* Thi, void* Tlo, int64_t ldt, float* gscale, cudaStream_t s);
+                                   void* Thi, void* Tlo, float* gscale, cudaStream_t s);
 
 // deterministic reductions (two stages, fixed order)
 void dot_to_ptr(armor_ctx* c, const float* x, const float* y, int64_t n, double* out, cudaStream_t s);
@@ -410,7 +410,7 @@ struct TcGemm {
   int passes;            // 1 or 3 tf32 passes on fp32 operands; 0: A and B are 16-bit arrays (one kind::f16 pass);
                          // 6: 16-bit high and low parts, three kind::f16 passes
   int fp16;              // passes 0 / 6: the 16-bit type is fp16 (1) or bf16 (0)
-  int mn_major;          // passes 0: A and B are [K][M] and [K][N] arrays (lda, ldb: distance of two k)
+  int mn_major;          // passes 0 / 6: A and B (and their low parts) are [K][M] and [K][N] arrays (lda, ldb: distance of two k)
   const float* row_scale; const float* col_scale;   // both or neither: C = acc * row_scale[m] * col_scale[n]
   int64_t k_segment;     // K extent accumulated in tensor memory before it is folded into C (0: all of K)
   int accumulate;        // C += (read-modify-write) instead of C =

@@ -154,21 +154,20 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
       float* gscale = b ? c->gscale2 : c->gscale;
       cudaStream_t ss = overlap ? c->side_stream : s;
       const int64_t n = n_rows - r0 < c->gram_rows ? n_rows - r0 : c->gram_rows;
-      const int64_t kpad = (n + 63) / 64 * 64;
       // buffer b was last read by the contraction of chunk p - 2
       if (overlap && p >= 2 && cudaStreamWaitEvent(ss, c->ev_used[b], 0) != cudaSuccess) return ARMOR_ERR_CUDA;
       armor_status st = launch_f16_gram_stage(c, static_cast<const char*>(Xv) + (size_t)(r0 * ldx) * esz, x_dtype, ldx, n,
-                                              d_in, thi, tlo, kpad, gscale, ss);
+                                              d_in, thi, tlo, gscale, ss);
       if (st != ARMOR_OK) return st;
       if (overlap && (cudaEventRecord(c->ev_staged[b], ss) != cudaSuccess ||
                       cudaStreamWaitEvent(s, c->ev_staged[b], 0) != cudaSuccess))
         return ARMOR_ERR_CUDA;
       TcGemm g{};
-      g.A = thi; g.Alo = tlo; g.lda = kpad;
-      g.B = thi; g.Blo = tlo; g.ldb = kpad;
+      g.A = thi; g.Alo = tlo; g.lda = d_in;
+      g.B = thi; g.Blo = tlo; g.ldb = d_in;
       g.C = H; g.ldc = d_in;
-      g.M = d_in; g.N = d_in; g.K = kpad;
-      g.passes = bf16 ? 0 : 6; g.fp16 = 1;
+      g.M = d_in; g.N = d_in; g.K = n;
+      g.passes = bf16 ? 0 : 6; g.fp16 = 1; g.mn_major = 1;
       g.row_scale = gscale; g.col_scale = gscale;
       g.accumulate = 1;
       g.symmetric_lower = 1;

@@ -227,7 +227,7 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* 
   }
 }
 
-// MN: both operands are 16-bit arrays contiguous along M / N (PASSES 0 only)
+// MN: both operands are 16-bit arrays contiguous along M / N (PASSES 0 and 6)
 template <int PASSES, bool MN>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapAlo,
@@ -289,10 +289,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
           uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
           if (MN) {
             // x = row of the operand (a channel), y = k (a token); rows and k beyond the operand are zero-filled
-            tma_load_2d_pair(dst, &mapA, arow, kt * BKE, fb);
-            tma_load_2d_pair(dst + MN_BOX, &mapA, arow + 64, kt * BKE, fb);
-            tma_load_2d_pair(dst + A_BYTES, &mapB, brow, kt * BKE, fb);
-            tma_load_2d_pair(dst + A_BYTES + MN_BOX, &mapB, brow + 64, kt * BKE, fb);
+#pragma unroll
+            for (int part = 0; part < (SPLIT ? 2 : 1); ++part) {
+              const CUtensorMap* ma = part ? &mapAlo : &mapA;
+              const CUtensorMap* mb = part ? &mapBlo : &mapB;
+              const uint32_t da = dst + part * A_BYTES, db = dst + (SPLIT ? 2 : 1) * A_BYTES + part * B_BYTES;
+              tma_load_2d_pair(da, ma, arow, kt * BKE, fb);
+              tma_load_2d_pair(da + MN_BOX, ma, arow + 64, kt * BKE, fb);
+              tma_load_2d_pair(db, mb, brow, kt * BKE, fb);
+              tma_load_2d_pair(db + MN_BOX, mb, brow + 64, kt * BKE, fb);
+            }
           } else {
             tma_load_2d_pair(dst, &mapA, kt * BKE, arow, fb);
             dst += A_BYTES;
@@ -600,8 +606,8 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
   if (n_part) *n_part = PARTS * p.n_tiles_total;
   if (g.mn_major) {
     // a map's rows start at multiples of 64 elements; the base and the leading dimension must be multiples of 16 bytes
-    if (g.passes != 0 || reinterpret_cast<uintptr_t>(g.A) % 16 || reinterpret_cast<uintptr_t>(g.B) % 16) return ARMOR_ERR_UNSUPPORTED;
-    return launch_impl<0, true>(c, g, p, s);
+    if (!h16 || reinterpret_cast<uintptr_t>(g.A) % 16 || reinterpret_cast<uintptr_t>(g.B) % 16) return ARMOR_ERR_UNSUPPORTED;
+    return g.passes == 6 ? launch_impl<6, true>(c, g, p, s) : launch_impl<0, true>(c, g, p, s);
   }
   if (g.passes == 3) return launch_impl<3, false>(c, g, p, s);
   if (g.passes == 6) return launch_impl<6, false>(c, g, p, s);

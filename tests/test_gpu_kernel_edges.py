@@ -299,3 +299,23 @@ def test_fp32_forward_over_chunk_edges(d_out, d_in, d_block, normalize):
         ref = x.double() @ Wh.t()
         assert (y - ref).norm() <= 1e-5 * ref.norm(), n
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_in,tokens", [(128, 1), (384, 63), (640, 1025), (256, 16384 + 77)])
+@pytest.mark.parametrize("form", ["plain", "strided", "unaligned"])
+def test_fp32_gram_staged_as_it_lies(d_in, tokens, form):
+    """Three-pass Gram of fp32 activations with channels of very different scales: the staged parts hold 22 bits below a
+    channel's largest entry, the sums truncate as in the bf16 Gram: (8e-6 + 2^-21) of the products of the channels' norms."""
+    lead = {"plain": d_in, "strided": d_in + 20, "unaligned": d_in + 3}[form]
+    g = _gen(tokens + d_in)
+    buf = torch.randn(tokens * lead + 1, device=DEV, generator=g)
+    off = 1 if form == "unaligned" else 0
+    X = buf[off: off + tokens * lead].view(tokens, lead)[:, :d_in]
+    X.mul_(torch.exp(4 * torch.randn(d_in, device=DEV, generator=g)))
+    ctx = _ctx(128, d_in, 128)
+    H = ctx.new_gram()
+    ctx.gram(X, H)
+    Xd = X.double()
+    nrm = Xd.norm(dim=0)
+    assert torch.equal(H, H.t())
+    assert ((H.double() - Xd.t() @ Xd).abs() <= (8e-6 + 2.0 ** -21) * nrm[:, None] * nrm[None, :]).all()
