@@ -552,20 +552,49 @@ __global__ void __launch_bounds__(NT) f32_to_bf16_kernel(const float* __restrict
   }
 }
 
-// H[r][c] = H[c][r] for c > r: the upper triangle from the lower one, 32 x 32 tiles through shared memory
-__global__ void mirror_lower_kernel(float* __restrict__ H, int64_t n) {
-  if (blockIdx.x < blockIdx.y) return;   // blockIdx.x: tile column of the destination, blockIdx.y: its tile row
-  __shared__ float tile[32][33];
-  const int64_t c0 = (int64_t)blockIdx.x * 32, r0 = (int64_t)blockIdx.y * 32;
-  // source tile: rows c0.., columns r0..
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int64_t sr = c0 + j, sc = r0 + threadIdx.x;
-    tile[j][threadIdx.x] = (sr < n && sc < n) ? H[sr * n + sc] : 0.f;
+// H[r][c] = H[c][r] for c > r: the upper triangle from the lower one, 64 x 64 tiles through shared memory, 16 bytes an access
+// (VEC: rows start on 16-byte boundaries and n is a multiple of 4); a CTA per tile on or below the diagonal.
+constexpr int MIR = 64;
+template <bool VEC>
+__global__ void __launch_bounds__(NT) mirror_lower_kernel(float* __restrict__ H, int64_t n) {
+  // blockIdx.x counts the tiles (i, j), j <= i, of the lower triangle row by row
+  int i = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+  while ((int64_t)(i + 1) * (i + 2) / 2 <= (int64_t)blockIdx.x) ++i;
+  while ((int64_t)i * (i + 1) / 2 > (int64_t)blockIdx.x) --i;
+  const int j = (int)((int64_t)blockIdx.x - (int64_t)i * (i + 1) / 2);
+  __shared__ float tile[MIR][MIR + 1];
+  const int64_t r0 = (int64_t)i * MIR, c0 = (int64_t)j * MIR;            // source tile
+  const int q = threadIdx.x & 15, w = threadIdx.x >> 4;
+  float4 v[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int64_t r = r0 + w + 16 * k, c = c0 + 4 * q;
+    v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r >= n) continue;
+    if (VEC) { if (c < n) v[k] = *reinterpret_cast<const float4*>(H + r * n + c); }
+    else {
+      float* f = &v[k].x;
+      for (int t = 0; t < 4; ++t) if (c + t < n) f[t] = H[r * n + c + t];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float* t = &tile[w + 16 * k][4 * q];
+    t[0] = v[k].x; t[1] = v[k].y; t[2] = v[k].z; t[3] = v[k].w;
   }
   __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += blockDim.y) {
-    const int64_t dr = r0 + j, dc = c0 + threadIdx.x;
-    if (dr < n && dc < n && dc > dr) H[dr * n + dc] = tile[threadIdx.x][j];
+  // row c0 + w + 16 k of the upper triangle, columns r0 + 4 q ..
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int64_t r = c0 + w + 16 * k, c = r0 + 4 * q;
+    if (r >= n) continue;
+    const float f[4] = {tile[4 * q][w + 16 * k], tile[4 * q + 1][w + 16 * k], tile[4 * q + 2][w + 16 * k], tile[4 * q + 3][w + 16 * k]};
+    if (VEC && i != j) {
+      if (c < n) *reinterpret_cast<float4*>(H + r * n + c) = make_float4(f[0], f[1], f[2], f[3]);
+    } else {
+      for (int t = 0; t < 4; ++t)
+        if (c + t < n && c + t > r) H[r * n + c + t] = f[t];
+    }
   }
 }
 
@@ -786,9 +815,11 @@ void launch_transpose_split(armor_ctx* c, const void* X, int x_dtype, int64_t ld
 }
 
 void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s) {
-  const unsigned t = (unsigned)((n + 31) / 32);
+  const int64_t t = (n + MIR - 1) / MIR;
+  const unsigned tiles = (unsigned)(t * (t + 1) / 2);
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  mirror_lower_kernel<<<dim3(t, t), dim3(32, 8), 0, s>>>(H, n);
+  if (n % 4 == 0 && reinterpret_cast<uintptr_t>(H) % 16 == 0) mirror_lower_kernel<true><<<tiles, NT, 0, s>>>(H, n);
+  else mirror_lower_kernel<false><<<tiles, NT, 0, s>>>(H, n);
   c->launches++;
 }
 
