@@ -411,7 +411,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         // a piece of a split tile: its partial sums go, plainly, to this item's slab
         float* slab = p.slabs + (((int64_t)(tile - p.split_first) * p.split_parts + part) * 2 + rank) * (BM * BN);
         double u1 = 0.0, u2 = 0.0;
-        write_out(acc, stg, lane, slab, BN, 1, q * 32, half * EPI_COLS, BM, BN, false, false, nullptr, nullptr, nullptr,
+        const int64_t rows = p.M - ((int64_t)mt * BMP + rank * BM);          // (rows past the end are not read back)
+        write_out(acc, stg, lane, slab, BN, 1, q * 32, half * EPI_COLS, rows < BM ? rows : BM, BN, false, false, nullptr, nullptr, nullptr,
                   nullptr, 0, u1, u2);
         continue;
       }
@@ -536,26 +537,34 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
   if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES, MN>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int n_pairs = c->n_sm / 2;
   if (n_pairs < 1) return ARMOR_ERR_UNSUPPORTED;
-  // tail split: the tiles of the last, partly filled wave are cut along K so that their pieces fill the wave
+  // Tail split: the tiles of the last, partly filled wave are cut along K so that their pieces fill the wave.  Where the
+  // contraction is summed in segments, the pieces are the segments themselves (the slabs are then added in the order in which
+  // an uncut tile adds its segments: the same bits), except that the tiles of a general product are cut in two to four equal
+  // pieces where these are whole segments or lie within one: fewer slabs.  One-pass products without segments: any pieces.
   p.split_first = p.n_tiles_total; p.split_parts = 1; p.split_kt = 0; p.n_items = p.n_tiles_total; p.slabs = c->gemm_slabs;
   const int kt_total = (int)((p.K + (H16 ? 64 : BK) - 1) / (H16 ? 64 : BK));
   const int rem = p.n_tiles_total % n_pairs;
   if (c->gemm_slabs && rem > 0) {
-    int parts = n_pairs / rem;
-    const int64_t room = c->gemm_slab_count / (2 * rem);         // a slab holds 128 x 256 sums, a piece writes two
-    if (parts > room) parts = (int)room;
-    if (parts > 16) parts = 16;      // beyond that the sum of the slabs costs more than the shorter pieces give
     // A piece writes 256 KB of sums and the second kernel reads them: about 6 us, 8 k-tiles with three MMAs per
     // product (0.8 us each) or 24 with one, which the shorter wave has to give back
     const int worth = SPLIT ? 8 : 24;
-    if (parts > 1) {
-      const int per = (kt_total + parts - 1) / parts;
-      if (kt_total - per >= worth) {
-        p.split_kt = per;
-        p.split_parts = (kt_total + per - 1) / per;
-        p.split_first = p.n_tiles_total - rem;
-        p.n_items = p.split_first + rem * p.split_parts;
-      }
+    const int fill = n_pairs / rem;                                // pieces per tile that still fit the wave
+    int per = kt_total;
+    if (!SPLIT && p.kt_seg >= kt_total) {
+      if (fill > 1) per = (kt_total + (fill < 16 ? fill : 16) - 1) / (fill < 16 ? fill : 16);
+    } else {
+      for (int parts = fill < 4 ? fill : 4; parts > 1 && !p.symmetric_lower && per == kt_total; --parts)
+        if (kt_total % parts == 0 && kt_total / parts >= 8 && ((kt_total / parts) % p.kt_seg == 0 || kt_total / parts <= p.kt_seg))
+          per = kt_total / parts;
+      if (per == kt_total && fill > 1 && p.kt_seg < kt_total) per = p.kt_seg;
+    }
+    const int parts = (kt_total + per - 1) / per;
+    // (a slab holds 128 x 256 sums, a piece writes two)
+    if (parts > 1 && kt_total - per >= worth && (int64_t)rem * parts * 2 <= c->gemm_slab_count) {
+      p.split_kt = per;
+      p.split_parts = parts;
+      p.split_first = p.n_tiles_total - rem;
+      p.n_items = p.split_first + rem * parts;
     }
   }
   const int pairs = p.n_items < n_pairs ? p.n_items : n_pairs;
