@@ -563,7 +563,8 @@ armor_status tc_bd_right(armor_ctx* c, const float* in, const float* Bblk, bool 
   // (by default this kernel: a CTA of the other one stays with one column block and so reads 512 bytes of every row, which
   // costs more than the saved shared-memory traffic: 45 us against 42 at 4096 x 4096)
   if (c->tc_blocks == 2 && tc_blockres_ok(c)) return tc_blockres_right(c, in, Bblk, transB, out, rows, cols, alpha, add, beta, s);
-  if (c->tc_blocks != 1 && tc_blockpair_ok(c)) return tc_blockpair_right(c, in, Bblk, transB, out, rows, cols, alpha, add, beta, s);
+  if (c->tc_blocks != 1 && tc_blockpair_ok(c, ((rows + 255) / 256) * (cols / 256)))
+    return tc_blockpair_right(c, in, Bblk, transB, out, rows, cols, alpha, add, beta, s);
   const int db = c->db;
   const int nb = (int)(cols / db);
   if (!ptr_ok(in) || !ptr_ok(Bblk) || !ptr_ok(out)) return ARMOR_ERR_UNSUPPORTED;
@@ -587,7 +588,8 @@ armor_status tc_bd_left(armor_ctx* c, const float* Ablk, bool transA, const floa
                         int64_t cols, float alpha, const float* add, float beta, cudaStream_t s) {
   // (39 us against 42 at 4096 x 4096, 47 against 55 with an addend)
   if (c->tc_blocks != 1 && tc_blockres_ok(c)) return tc_blockres_left(c, Ablk, transA, in, out, rows, cols, alpha, add, beta, s);
-  if (c->tc_blocks != 1 && tc_blockpair_ok(c)) return tc_blockpair_left(c, Ablk, transA, in, out, rows, cols, alpha, add, beta, s);
+  if (c->tc_blocks != 1 && tc_blockpair_ok(c, (rows / 256) * ((cols + 255) / 256)))
+    return tc_blockpair_left(c, Ablk, transA, in, out, rows, cols, alpha, add, beta, s);
   const int db = c->db;
   const int nb = (int)(rows / db);
   if (!ptr_ok(in) || !ptr_ok(Ablk) || !ptr_ok(out)) return ARMOR_ERR_UNSUPPORTED;
@@ -613,7 +615,7 @@ armor_status tc_bd_left_dual(armor_ctx* c, const float* Ablk, bool transA, const
   // instruction (half the shared-memory traffic of two passes through the streaming kernel)
   if (c->tc_blocks != 1 && !transA && tc_blockres_ok(c))
     return tc_blockres_left_dual(c, Ablk, in1, in2, out, rows, cols, part, n_part, s);
-  if (c->tc_blocks != 1 && tc_blockpair_ok(c))
+  if (c->tc_blocks != 1 && tc_blockpair_ok(c, (rows / 256) * ((cols + 255) / 256)))
     return tc_blockpair_left(c, Ablk, transA, in1, out, rows, cols, 1.f, nullptr, 0.f, s, in2, part, n_part);
   const int db = c->db;
   const int nb = (int)(rows / db);
@@ -697,7 +699,7 @@ armor_status gram_launch(armor_ctx* c, const HostOp& A, const HostOp& B, bool by
   p.m_tiles = db / TILE; p.n_tiles = db / TILE; p.batch = nb; p.k_chunks = (int)(chunks / ks); p.n_split = ks;
   p.alpha = 1.f; p.beta = 0.f; p.m_valid = 1 << 30;
   // two W-shaped operands are read once each
-  armor_status st = c->tc_blocks != 1 && tc_blockpair_ok(c) ? tc_blockpair_gram(c, A.base, B.base, by_rows, p.C, ks, s)
+  armor_status st = c->tc_blocks != 1 && tc_blockpair_ok(c, 2 * (int64_t)nb * ks) ? tc_blockpair_gram(c, A.base, B.base, by_rows, p.C, ks, s)
                                                             : launch(c, A, B, p, ARMOR_KC_BLOCK_GRAM, 8.0 * (double)c->wn, s);
   if (st != ARMOR_OK || ks == 1) return st;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
@@ -728,7 +730,7 @@ armor_status gram_pair_launch(armor_ctx* c, const HostOp& A, const HostOp& B, co
   p.alpha = 1.f; p.beta = 0.f; p.m_valid = 1 << 30;
   p.pair = pair;
   // three (pair 1) or two (pair 2) W-shaped operands are read once each
-  armor_status st = pair == 1 && c->tc_blocks != 1 && tc_blockpair_ok(c)
+  armor_status st = pair == 1 && c->tc_blocks != 1 && tc_blockpair_ok(c, 2 * (int64_t)nb * ks)
                         ? tc_blockpair_gram(c, A.base, B.base, true, p.C, ks, s, A2, C2)
                         : launch(c, A, B, p, ARMOR_KC_BLOCK_GRAM, (pair == 1 ? 12.0 : 8.0) * (double)c->wn, s, A2, C2);
   if (st != ARMOR_OK || ks == 1) return st;

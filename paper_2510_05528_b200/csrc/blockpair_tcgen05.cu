@@ -402,7 +402,12 @@ inline bool ptr_ok(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15)
 
 }  // namespace
 
-bool tc_blockpair_ok(const armor_ctx* c) { return c->db == BLK && c->n_sm >= 2; }
+// Two waves of tiles at least: with fewer, 128 x 128 tiles on single CTAs spread better (3840 x 6400, 148 tokens: 64 us against
+// 76 for a forward).  Products that round their operands to one pass are bound by neither fetching nor splitting (23808 x
+// 3072, 2,292 tokens: 397 us against 428).
+bool tc_blockpair_ok(const armor_ctx* c, int64_t tiles) {
+  return c->db == BLK && !c->block_one_pass && c->n_sm >= 2 && tiles >= c->n_sm;
+}
 
 // out[:, j-th block] = alpha * in[:, j-th block] * Q_j (+ beta * add[:, j-th block]),  Q_j = Bblk[j] or its transpose
 armor_status tc_blockpair_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,

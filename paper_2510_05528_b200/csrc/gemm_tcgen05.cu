@@ -551,7 +551,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     const int fill = n_pairs / rem;                                // pieces per tile that still fit the wave
     int per = kt_total;
     if (!SPLIT && p.kt_seg >= kt_total) {
-      if (fill > 1) per = (kt_total + (fill < 16 ? fill : 16) - 1) / (fill < 16 ? fill : 16);
+      if (fill > 1) per = (kt_total + (fill < 4 ? fill : 4) - 1) / (fill < 4 ? fill : 4);
     } else {
       for (int parts = fill < 4 ? fill : 4; parts > 1 && !p.symmetric_lower && per == kt_total; --parts)
         if (kt_total % parts == 0 && kt_total / parts >= 8 && ((kt_total / parts) % p.kt_seg == 0 || kt_total / parts <= p.kt_seg))

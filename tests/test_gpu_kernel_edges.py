@@ -223,10 +223,10 @@ def test_row_norms_of_the_normalisation(scale):
         assert ((st.r2.double() - r2).abs() <= 2.0 ** -23 * r2).all()
 
 
-@pytest.mark.parametrize("rows,cols", [(256, 256), (200, 768), (1025, 512), (512, 260), (2560, 2048)])
+@pytest.mark.parametrize("rows,cols", [(256, 256), (1025, 512), (4864, 2048), (4801, 2048), (4864, 2052), (2560, 4096)])
 @pytest.mark.parametrize("side,transpose", [(0, 0), (0, 1), (1, 0), (1, 1)])
 def test_products_with_blocks_of_256_on_pairs_of_ctas(rows, cols, side, transpose):
-    """The kernel for pairs of CTAs gives the bits of the streaming kernel (path 1): same operand parts, same order of MMAs;
+    """The kernel for pairs of CTAs (from 148 tiles on) gives the bits of the streaming kernel (path 1): same operand parts, same order of MMAs;
     ragged rows of a right product and columns of a left one, with an addend, in place."""
     from paper_2510_05528_b200 import binding as Bd
     if (cols if side == 0 else rows) % 256:
@@ -246,7 +246,7 @@ def test_products_with_blocks_of_256_on_pairs_of_ctas(rows, cols, side, transpos
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
 
 
-@pytest.mark.parametrize("d_out,d_in", [(256, 256), (512, 2304), (4864, 768)])
+@pytest.mark.parametrize("d_out,d_in", [(512, 2304), (4864, 2304), (18944, 512)])
 def test_dual_product_and_grams_with_blocks_of_256(d_out, d_in):
     """Dual product: the bits of the streaming kernel, the dot product to the order of its fp64 partial sums; A- and B-step of
     one iteration (both Grams of either) likewise against a run on the streaming kernels' results in fp64."""
@@ -320,3 +320,29 @@ def test_fp32_gram_staged_as_it_lies(d_in, tokens, form):
     nrm = Xd.norm(dim=0)
     assert torch.equal(H, H.t())
     assert ((H.double() - Xd.t() @ Xd).abs() <= (192 * 2.0 ** -23 + 2.0 ** -21) * nrm[:, None] * nrm[None, :]).all()
+
+
+def test_few_token_forward_in_a_captured_graph():
+    """The dependent launches of the few-token forward are captured and replayed like any others."""
+    from paper_2510_05528_b200 import binding as Bd
+    d_out, d_in = 1024, 768
+    g = _gen(3)
+    ctx = _ctx(d_out, d_in, 128)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    st = ctx.init(W, torch.eye(d_in, device=DEV))
+    packed = ctx.pack_layer(st)
+    for n in (1, 50, 300):
+        x = torch.randn(n, d_in, device=DEV, generator=g).to(torch.bfloat16)
+        want = ctx.apply_layer(packed, x).clone()
+        y = torch.zeros_like(want)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            Bd.armor_apply_layer(ctx.ctx, packed, x, y)
+        for _ in range(3):
+            y.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(y, want), n
+        del graph
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
