@@ -441,19 +441,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 }
 
 // Adds the slabs of every split tile into C (+ what C held, if the product accumulates) and forms the tile's
-// share of the fused dot products.  Sixteen CTAs per split tile (16 rows each), four pieces in flight; fixed order.
-__global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
+// share of the fused dot products.  Sixteen CTAs per split tile, 16 rows each, one float4 per thread (the kernel is nothing
+// but latency), four pieces in flight; fixed order.
+constexpr int FIX_NT = BMP / PARTS * BN / 4;
+__global__ void __launch_bounds__(FIX_NT) tc_gemm_fixup_kernel(const Params p) {
   constexpr int FR = BMP / PARTS;                         // rows per CTA
   const int tile = p.split_first + blockIdx.x / PARTS, slot = blockIdx.x % PARTS;
   int mt, nt;
   tile_coords(p, tile, mt, nt);
   const float* slab0 = p.slabs + (int64_t)(blockIdx.x / PARTS) * p.split_parts * (BMP * BN) + (int64_t)slot * FR * BN;
   double d1 = 0.0, d2 = 0.0;
-#pragma unroll
-  for (int e = threadIdx.x; e < FR * BN / 4; e += 256) {
-    const int r = e / (BN / 4), c4 = (e % (BN / 4)) * 4;
-    const int64_t grow = (int64_t)mt * BMP + slot * FR + r, gcol = (int64_t)nt * BN + c4;
-    if (grow >= p.M || gcol >= p.N || (p.symmetric_lower && gcol > grow)) continue;
+  const int r = threadIdx.x / (BN / 4), c4 = (threadIdx.x % (BN / 4)) * 4;
+  const int64_t grow = (int64_t)mt * BMP + slot * FR + r, gcol = (int64_t)nt * BN + c4;
+  if (grow < p.M && gcol < p.N && !(p.symmetric_lower && gcol > grow)) {
     const float* sp = slab0 + (int64_t)r * BN + c4;
     float4 v = *reinterpret_cast<const float4*>(sp);
 #pragma unroll 4
@@ -482,7 +482,7 @@ __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
     }
   }
   if (!p.part1 && !p.part2) return;
-  __shared__ double red1[8], red2[8];
+  __shared__ double red1[FIX_NT / 32], red2[FIX_NT / 32];
   for (int o = 16; o > 0; o >>= 1) {
     d1 += __shfl_down_sync(0xffffffffu, d1, o);
     d2 += __shfl_down_sync(0xffffffffu, d2, o);
@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(256) tc_gemm_fixup_kernel(const Params p) {
   __syncthreads();
   if (threadIdx.x == 0) {
     double t1 = 0.0, t2 = 0.0;
-    for (int w = 0; w < 8; ++w) { t1 += red1[w]; t2 += red2[w]; }
+    for (int w = 0; w < FIX_NT / 32; ++w) { t1 += red1[w]; t2 += red2[w]; }
     // the slots of the tile's epilogue warps, filled by this kernel's CTAs instead
     if (p.part1) p.part1[(int64_t)tile * PARTS + slot] = t1;
     if (p.part2) p.part2[(int64_t)tile * PARTS + slot] = t2;
@@ -579,7 +579,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     cfg.attrs = at; cfg.numAttrs = 1;
     if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
-      tc_gemm_fixup_kernel<<<PARTS * (p.n_tiles_total - p.split_first), 256, 0, s>>>(p);
+      tc_gemm_fixup_kernel<<<PARTS * (p.n_tiles_total - p.split_first), FIX_NT, 0, s>>>(p);
       c->launches++;
     }
   }

@@ -493,60 +493,53 @@ __global__ void mask_commit_kernel(const SelRec* __restrict__ sel, int nblocks, 
 }
 
 // The accepted group updates change T H_w = S B H_w by the rows (delta^T B_j[group rows, :]) H_w[j-th block
-// row, :] = y_ij, added to row r_ij.  Groups of one row-block may share a row, so one CTA walks the column
-// blocks j in order (deterministic sums); the grid is (row-block, chunk of 1024 columns).
+// row, :] = y_ij, added to row r_ij.  Groups of one row-block may share a row; its additions happen in the order of the column
+// blocks (deterministic sums), all of them by the CTA that holds the first.  The grid is (row-block, chunk of 1024 columns,
+// CARRY_PICKS column blocks): one CTA walking all column blocks in batches took 20 us for 50 MB, a chain of batches with few
+// CTAs in flight.
+constexpr int CARRY_PICKS = 4;
 __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* __restrict__ sel, const float* __restrict__ Y,
                                                         float* __restrict__ P, const double* __restrict__ sc,
                                                         int64_t d_in, int nbo_pad, int nbv) {
+  extern __shared__ int row_of[];                          // [nbv] row of every column block's group, -1: none
+  __shared__ int earlier, later;                           // bit u: pick j0 + u shares its row with an earlier / a later one
   if (sc[SC_ACCEPT] == 0.0) return;
-  const int bi = blockIdx.x;
+  const int bi = blockIdx.x, j0 = blockIdx.z * CARRY_PICKS;
+  for (int j = threadIdx.x; j < nbv; j += NT) {
+    const SelRec* rec = sel + (int64_t)bi * nbv + j;
+    row_of[j] = rec->valid ? rec->row : -1;
+  }
+  if (threadIdx.x == 0) earlier = later = 0;
+  __syncthreads();
+  for (int j = threadIdx.x; j < nbv; j += NT)
+#pragma unroll
+    for (int u = 0; u < CARRY_PICKS; ++u)
+      if (j0 + u < nbv && j != j0 + u && row_of[j] >= 0 && row_of[j] == row_of[j0 + u]) atomicOr(j < j0 + u ? &earlier : &later, 1 << u);
+  __syncthreads();
   const int64_t c4 = (int64_t)blockIdx.y * 1024 + 4 * threadIdx.x;
   if (c4 >= d_in) return;
-  // Virtual column blocks in order, eight at a time.  The eight rows are almost always distinct: then their loads are
-  // independent and issued together (a chain of 32 dependent read-modify-writes was the whole cost of this kernel);
-  // a batch in which two groups share a row is walked one by one, so that every element of P sees its additions in
-  // the order of the column blocks (deterministic sums).
-  for (int j0 = 0; j0 < nbv; j0 += 8) {
-    int row[8];
-    bool val[8];
+  float4 v[CARRY_PICKS], y[CARRY_PICKS];
+  bool mine[CARRY_PICKS];
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      val[u] = false; row[u] = 0;
-      if (j0 + u < nbv) {
-        const SelRec* rec = sel + (bi * nbv + j0 + u);
-        val[u] = rec->valid != 0;
-        row[u] = rec->row;
+  for (int u = 0; u < CARRY_PICKS; ++u) {
+    mine[u] = j0 + u < nbv && row_of[j0 + u] >= 0 && !((earlier >> u) & 1);
+    if (!mine[u]) continue;
+    v[u] = *reinterpret_cast<const float4*>(P + (int64_t)row_of[j0 + u] * d_in + c4);
+    y[u] = *reinterpret_cast<const float4*>(Y + ((int64_t)(j0 + u) * nbo_pad + bi) * d_in + c4);
+  }
+#pragma unroll
+  for (int u = 0; u < CARRY_PICKS; ++u) {
+    if (!mine[u]) continue;
+    const int r = row_of[j0 + u];
+    float4 x = v[u];
+    x.x += y[u].x; x.y += y[u].y; x.z += y[u].z; x.w += y[u].w;
+    if ((later >> u) & 1)
+      for (int j = j0 + u + 1; j < nbv; ++j) {
+        if (row_of[j] != r) continue;
+        const float4 w = *reinterpret_cast<const float4*>(Y + ((int64_t)j * nbo_pad + bi) * d_in + c4);
+        x.x += w.x; x.y += w.y; x.z += w.z; x.w += w.w;
       }
-    }
-    bool shared_row = false;
-#pragma unroll
-    for (int u = 1; u < 8; ++u)
-#pragma unroll
-      for (int w = 0; w < u; ++w) shared_row |= val[u] && val[w] && row[u] == row[w];
-    if (!shared_row) {
-      float4 y[8], v[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (val[u]) {
-          y[u] = *reinterpret_cast<const float4*>(Y + ((int64_t)(j0 + u) * nbo_pad + bi) * d_in + c4);
-          v[u] = *reinterpret_cast<const float4*>(P + (int64_t)row[u] * d_in + c4);
-        }
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (val[u]) {
-          v[u].x += y[u].x; v[u].y += y[u].y; v[u].z += y[u].z; v[u].w += y[u].w;
-          *reinterpret_cast<float4*>(P + (int64_t)row[u] * d_in + c4) = v[u];
-        }
-    } else {
-      for (int u = 0; u < 8; ++u) {
-        if (!val[u]) continue;
-        const float4 y = *reinterpret_cast<const float4*>(Y + ((int64_t)(j0 + u) * nbo_pad + bi) * d_in + c4);
-        float4* dst = reinterpret_cast<float4*>(P + (int64_t)row[u] * d_in + c4);
-        float4 v = *dst;
-        v.x += y.x; v.y += y.y; v.z += y.z; v.w += y.w;
-        *dst = v;
-      }
-    }
+    *reinterpret_cast<float4*>(P + (int64_t)r * d_in + c4) = x;
   }
 }
 
@@ -554,8 +547,9 @@ __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* __restrict
 
 void launch_mask_carry_P(armor_ctx* c, float* P, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  mask_carry_kernel<<<dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024)), NT, 0, s>>>(c->sel, c->Ysel, P, c->sc, c->d_in,
-                                                                                   c->nbo_pad, c->nbi * c->kg);
+  const int nbv = c->nbi * c->kg;
+  mask_carry_kernel<<<dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)((nbv + CARRY_PICKS - 1) / CARRY_PICKS)), NT,
+                      (size_t)nbv * sizeof(int), s>>>(c->sel, c->Ysel, P, c->sc, c->d_in, c->nbo_pad, nbv);
   c->launches++;
 }
 

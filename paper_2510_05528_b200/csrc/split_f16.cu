@@ -69,6 +69,11 @@ __global__ void hpow_kernel(const float* __restrict__ hdiag, float* __restrict__
   hpow[k] = scalbnf(1.f, e);
 }
 
+// 2^shift / d for a power of two d = 2^e, |e| < 100: arithmetic on the exponent field instead of a division per entry
+__device__ __forceinline__ float over_pow2(float d, int shift) {
+  return __uint_as_float((uint32_t)((254 + shift) << 23) - __float_as_uint(d));
+}
+
 // Hhi + Hlo = H_kn / (d_k d_n) * 2^H_SHIFT, four columns per thread
 __global__ void __launch_bounds__(NT) split_H_kernel(const float4* __restrict__ H, const float* __restrict__ hpow,
                                                      __half2* __restrict__ hi, __half2* __restrict__ lo, int64_t n,
@@ -76,10 +81,11 @@ __global__ void __launch_bounds__(NT) split_H_kernel(const float4* __restrict__ 
   const int64_t n4 = n / 4;
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n * n4; i += (int64_t)gridDim.x * NT) {
     const int64_t k = i / n4, c4 = (i % n4) * 4;
-    const float rk = scalbnf(1.f / hpow[k], H_SHIFT);     // reciprocal of a power of two: exact
+    const float rk = over_pow2(hpow[k], H_SHIFT);
     const float4 v = H[i];
-    const float4 d = *reinterpret_cast<const float4*>(hpow + c4);
-    const float x0 = v.x * rk / d.x, x1 = v.y * rk / d.y, x2 = v.z * rk / d.z, x3 = v.w * rk / d.w;
+    const float4 d = __ldg(reinterpret_cast<const float4*>(hpow + c4));
+    const float x0 = v.x * rk * over_pow2(d.x, 0), x1 = v.y * rk * over_pow2(d.y, 0), x2 = v.z * rk * over_pow2(d.z, 0),
+                x3 = v.w * rk * over_pow2(d.w, 0);
     const int over = (fabsf(x0) > 65504.f && isfinite(x0)) + (fabsf(x1) > 65504.f && isfinite(x1)) +
                      (fabsf(x2) > 65504.f && isfinite(x2)) + (fabsf(x3) > 65504.f && isfinite(x3));
     if (over) atomicAdd(&status[ST_H_RANGE], over);
