@@ -6,8 +6,8 @@
 // A failed factorisation leaves A unchanged / writes zeros and raises failflag[block].
 //
 // One CTA factorises one d_block x d_block matrix in shared memory and solves for a slice of the right-hand sides beside it;
-// the slices of a block repeat the factorisation.  What bounds this is the chain of pivots (about 200 cycles each in the
-// factorisation, 80 in a solve), next to it fp64 conversions, which cost as much as dozens of fp32 instructions and are
+// the slices of a block repeat the factorisation.  What bounds this is the chain of pivots (about 150 cycles each in the
+// factorisation, 140 in a solve), next to it fp64 conversions, which cost as much as dozens of fp32 instructions and are
 // kept out of the sums:
 //   storage: panels of 32 columns, rows of 32 floats, the 16-byte units of a row swizzled so that eight lanes reading the
 //            same unit of consecutive rows, or of every fourth row, or all units of one row, meet no bank conflict; G
@@ -18,10 +18,11 @@
 //            along, so that no second pass over the rows below follows.
 //   solve  : left-looking with the same two-level sums, a lane per right-hand side, a warp per four rows of a block of 32:
 //            every warp works in every step.
-// Measured and left: pivots eight at a time with every thread factorising the 8 x 8 block (elimination 1.4 x slower), rows
-// or right-hand sides moving down one register per pivot in a rolled loop (2 x), solutions handed round by shuffles (1.2 x).
-// A launch, d_block 128: 32 blocks over 4 CTAs each 57 us (79 before), 112 blocks 86 us (85); d_block 256, 32 blocks 176 us
-// (about 270).
+// Measured and left: pivots eight at a time with every thread factorising the 8 x 8 block (elimination 2 x slower), rows
+// or right-hand sides moving down one register per pivot in a rolled loop (3 x and 1.4 x), solutions handed round by shuffles
+// (1.2 x).
+// A launch, d_block 128: 32 blocks over 4 CTAs each 57 us (79 before), 112 blocks 86 us (85); d_block 256, a 28672 x 8192
+// layer's launches of 112 and 32 blocks 469 us on average (545).
 #include "armor_internal.cuh"
 
 namespace {
