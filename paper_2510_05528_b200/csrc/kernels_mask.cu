@@ -495,51 +495,58 @@ __global__ void mask_commit_kernel(const SelRec* __restrict__ sel, int nblocks, 
 // The accepted group updates change T H_w = S B H_w by the rows (delta^T B_j[group rows, :]) H_w[j-th block
 // row, :] = y_ij, added to row r_ij.  Groups of one row-block may share a row; its additions happen in the order of the column
 // blocks (deterministic sums), all of them by the CTA that holds the first.  The grid is (row-block, chunk of 1024 columns,
-// CARRY_PICKS column blocks): one CTA walking all column blocks in batches took 20 us for 50 MB, a chain of batches with few
-// CTAs in flight.
+// CARRY_PICKS column blocks at a time): one CTA walking all column blocks in batches took 20 us for 50 MB, a chain of batches
+// with few CTAs in flight.  Which pick is a row's first and which its last is found once per CTA in a table of the block's
+// rows (d_block <= 256), so that neither shared memory nor, with at most CARRY_CTAS along the picks, the work grows faster
+// than their number (thousands with small blocks and several draws).
 constexpr int CARRY_PICKS = 4;
+constexpr int CARRY_CTAS = 64;
+constexpr int CARRY_TAB = 2048;                            // picks whose rows are kept in shared memory
+__device__ __forceinline__ int carry_row(const SelRec& rec, int row0) { return rec.valid ? rec.row - row0 : -1; }
 __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* __restrict__ sel, const float* __restrict__ Y,
                                                         float* __restrict__ P, const double* __restrict__ sc,
-                                                        int64_t d_in, int nbo_pad, int nbv) {
-  extern __shared__ int row_of[];                          // [nbv] row of every column block's group, -1: none
-  __shared__ int earlier, later;                           // bit u: pick j0 + u shares its row with an earlier / a later one
+                                                        int64_t d_in, int db, int nbo_pad, int nbv) {
+  __shared__ int row_of[CARRY_TAB];                        // row inside the block, -1: no group
+  __shared__ int first[256], last[256];                    // picks of a row
   if (sc[SC_ACCEPT] == 0.0) return;
-  const int bi = blockIdx.x, j0 = blockIdx.z * CARRY_PICKS;
-  for (int j = threadIdx.x; j < nbv; j += NT) {
-    const SelRec* rec = sel + (int64_t)bi * nbv + j;
-    row_of[j] = rec->valid ? rec->row : -1;
-  }
-  if (threadIdx.x == 0) earlier = later = 0;
+  const int bi = blockIdx.x, row0 = bi * db;
+  const SelRec* mine_sel = sel + (int64_t)bi * nbv;
+  for (int r = threadIdx.x; r < db; r += NT) { first[r] = nbv; last[r] = -1; }
   __syncthreads();
-  for (int j = threadIdx.x; j < nbv; j += NT)
-#pragma unroll
-    for (int u = 0; u < CARRY_PICKS; ++u)
-      if (j0 + u < nbv && j != j0 + u && row_of[j] >= 0 && row_of[j] == row_of[j0 + u]) atomicOr(j < j0 + u ? &earlier : &later, 1 << u);
+  for (int j = threadIdx.x; j < nbv; j += NT) {
+    const int r = carry_row(mine_sel[j], row0);
+    if (j < CARRY_TAB) row_of[j] = r;
+    if (r >= 0) { atomicMin(&first[r], j); atomicMax(&last[r], j); }
+  }
   __syncthreads();
   const int64_t c4 = (int64_t)blockIdx.y * 1024 + 4 * threadIdx.x;
   if (c4 >= d_in) return;
-  float4 v[CARRY_PICKS], y[CARRY_PICKS];
-  bool mine[CARRY_PICKS];
+  auto row_at = [&](int j) { return j < CARRY_TAB ? row_of[j] : carry_row(mine_sel[j], row0); };
+  for (int j0 = blockIdx.z * CARRY_PICKS; j0 < nbv; j0 += gridDim.z * CARRY_PICKS) {
+    float4 v[CARRY_PICKS], y[CARRY_PICKS];
+    int row[CARRY_PICKS];                                  // -1: nothing to do for this pick
 #pragma unroll
-  for (int u = 0; u < CARRY_PICKS; ++u) {
-    mine[u] = j0 + u < nbv && row_of[j0 + u] >= 0 && !((earlier >> u) & 1);
-    if (!mine[u]) continue;
-    v[u] = *reinterpret_cast<const float4*>(P + (int64_t)row_of[j0 + u] * d_in + c4);
-    y[u] = *reinterpret_cast<const float4*>(Y + ((int64_t)(j0 + u) * nbo_pad + bi) * d_in + c4);
-  }
+    for (int u = 0; u < CARRY_PICKS; ++u) {
+      const int j = j0 + u;
+      row[u] = j < nbv ? row_at(j) : -1;
+      if (row[u] >= 0 && first[row[u]] != j) row[u] = -1;
+      if (row[u] < 0) continue;
+      v[u] = *reinterpret_cast<const float4*>(P + (int64_t)(row0 + row[u]) * d_in + c4);
+      y[u] = *reinterpret_cast<const float4*>(Y + ((int64_t)j * nbo_pad + bi) * d_in + c4);
+    }
 #pragma unroll
-  for (int u = 0; u < CARRY_PICKS; ++u) {
-    if (!mine[u]) continue;
-    const int r = row_of[j0 + u];
-    float4 x = v[u];
-    x.x += y[u].x; x.y += y[u].y; x.z += y[u].z; x.w += y[u].w;
-    if ((later >> u) & 1)
-      for (int j = j0 + u + 1; j < nbv; ++j) {
-        if (row_of[j] != r) continue;
+    for (int u = 0; u < CARRY_PICKS; ++u) {
+      if (row[u] < 0) continue;
+      float4 x = v[u];
+      x.x += y[u].x; x.y += y[u].y; x.z += y[u].z; x.w += y[u].w;
+      const int end = last[row[u]];
+      for (int j = j0 + u + 1; j <= end; ++j) {
+        if (row_at(j) != row[u]) continue;
         const float4 w = *reinterpret_cast<const float4*>(Y + ((int64_t)j * nbo_pad + bi) * d_in + c4);
         x.x += w.x; x.y += w.y; x.z += w.z; x.w += w.w;
       }
-    *reinterpret_cast<float4*>(P + (int64_t)r * d_in + c4) = x;
+      *reinterpret_cast<float4*>(P + (int64_t)(row0 + row[u]) * d_in + c4) = x;
+    }
   }
 }
 
@@ -548,8 +555,10 @@ __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* __restrict
 void launch_mask_carry_P(armor_ctx* c, float* P, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
   const int nbv = c->nbi * c->kg;
-  mask_carry_kernel<<<dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)((nbv + CARRY_PICKS - 1) / CARRY_PICKS)), NT,
-                      (size_t)nbv * sizeof(int), s>>>(c->sel, c->Ysel, P, c->sc, c->d_in, c->nbo_pad, nbv);
+  int groups = (nbv + CARRY_PICKS - 1) / CARRY_PICKS;
+  if (groups > CARRY_CTAS) groups = CARRY_CTAS;
+  mask_carry_kernel<<<dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s>>>(
+      c->sel, c->Ysel, P, c->sc, c->d_in, c->db, c->nbo_pad, nbv);
   c->launches++;
 }
 

@@ -346,3 +346,35 @@ def test_few_token_forward_in_a_captured_graph():
             assert torch.equal(y, want), n
         del graph
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_block,d_in,draws", [(4, 1024, 8), (4, 1152, 8), (32, 1024, 4), (128, 1280, 1), (4, 6272, 8)])
+def test_carried_product_over_many_column_blocks_and_draws(d_block, d_in, draws):
+    """Group updates alone, from a core that was halved: the carried P = S B H_w takes a row from every draw of every column
+    block (up to 12,544 here, on rows that thousands of them share), and the next iteration starts from it.  One call of
+    three iterations against three calls, each of which forms P anew: the two differ by the rounding of P, sums of up to
+    1,568 rows, sqrt(1568) x 2^-24 = 2.4e-6 of P, and by nothing else (the draws cover every group of a small block; the
+    masks keep their margins)."""
+    from paper_2510_05528_b200 import binding as Bd
+    d_out = 128
+    g = _gen(d_in + draws)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    v = torch.randn(d_in, device=DEV, generator=g)
+    H = torch.eye(d_in, device=DEV) + 0.3 * torch.outer(v, v) / v.square().sum()
+    got = {}
+    for calls in (1, 3):
+        ctx = _ctx(d_out, d_in, d_block, mask_groups=draws, phases=8, seed=3)
+        st = ctx.init(W, H)
+        st.S.mul_(0.5)
+        acc = []
+        for t in range(calls):
+            acc.append(ctx.read_stats(ctx.bcd_step(st, H, t * (3 // calls), 3 // calls)))
+        assert acc[0]["mask_accepted"][0] == 1 and acc[0]["delta_L_mask"][0] < 0
+        loss = ctx.proxy_loss(st, H).item()
+        assert abs(acc[-1]["loss_mask"][-1] - loss) <= 1e-5 * loss
+        assert ctx.device_status()[:4] == [0, 0, 0, 0]
+        got[calls] = (st.S.clone(), st.M.clone(), loss)
+        del ctx, st
+    assert torch.equal(got[1][1], got[3][1])
+    assert (got[1][0] - got[3][0]).norm() <= 1e-5 * got[3][0].norm()
+    assert abs(got[1][2] - got[3][2]) <= 1e-5 * got[3][2]
