@@ -462,9 +462,10 @@ __global__ void __launch_bounds__(FIX_NT) tc_gemm_fixup_kernel(const Params p) {
       v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
     }
     if (p.row_scale) {
+      // one scale after the other, as write_out applies them: their product may leave fp32's range where the result does not
       const float rs = p.row_scale[grow];
       const float4 cs = *reinterpret_cast<const float4*>(p.col_scale + gcol);
-      v.x *= rs * cs.x; v.y *= rs * cs.y; v.z *= rs * cs.z; v.w *= rs * cs.w;
+      v.x = v.x * rs * cs.x; v.y = v.y * rs * cs.y; v.z = v.z * rs * cs.z; v.w = v.w * rs * cs.w;
     }
     float* cp = p.C + grow * p.ldc + gcol;
     if (p.accumulate) {

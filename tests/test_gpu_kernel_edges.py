@@ -378,3 +378,24 @@ def test_carried_product_over_many_column_blocks_and_draws(d_block, d_in, draws)
     assert torch.equal(got[1][1], got[3][1])
     assert (got[1][0] - got[3][0]).norm() <= 1e-5 * got[3][0].norm()
     assert abs(got[1][2] - got[3][2]) <= 1e-5 * got[3][2]
+
+
+@pytest.mark.parametrize("tokens", [1000, 4100, 16384 + 3000])
+def test_fp32_gram_of_tiny_and_huge_channels(tokens):
+    """Channels between 1e-20 and 1e16 side by side, in tiles that are cut along the tokens (256 channels: the only tile) and in
+    whole ones (1,000 tokens): every scaling is a power of two, so an entry keeps the accuracy of its channels however
+    small they are (the bound of test_fp32_gram_staged_as_it_lies, and 2^-149 where the entry itself is subnormal)."""
+    d_in = 256
+    g = _gen(tokens)
+    scale = 10.0 ** torch.linspace(-20.0, 16.0, d_in, device=DEV, dtype=torch.float64)
+    scale = scale[torch.randperm(d_in, device=DEV, generator=g)]
+    X = (torch.randn(tokens, d_in, device=DEV, generator=g).double() * scale).float()
+    ctx = _ctx(128, d_in, 128)
+    H = ctx.new_gram()
+    ctx.gram(X, H)
+    Xd = X.double()
+    nrm = Xd.norm(dim=0)
+    err = (H.double() - Xd.t() @ Xd).abs()
+    assert torch.isfinite(H).all()
+    assert (err <= (192 * 2.0 ** -23 + 2.0 ** -21) * nrm[:, None] * nrm[None, :] + 2.0 ** -149).all()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
