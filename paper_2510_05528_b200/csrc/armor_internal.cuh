@@ -364,7 +364,11 @@ void launch_scale_rows_cols(armor_ctx* c, const float* in, const float* colscale
 void launch_split_hilo(armor_ctx* c, const float* in, float* hi, float* lo, int64_t n, cudaStream_t s);
 void launch_transpose_split(armor_ctx* c, const void* X, int x_dtype, int64_t ldx, int64_t rows, int64_t cols,
                             float* Thi, float* Tlo, int64_t ldt, cudaStream_t s);
-void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s);
+void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s, const void* X_bf16 = nullptr, int64_t ldx = 0,
+                         int64_t n_rows = 0, const float* in_range = nullptr);
+// in_range[k] = 0 for a channel of X (bf16, [n_rows][ldx], rows on 16-byte boundaries) that is not all zeros and nowhere reaches
+// 2^-57 in magnitude, else 1
+void launch_gram_range(armor_ctx* c, const void* X_bf16, int64_t ldx, int64_t n_rows, float* in_range, cudaStream_t s);
 void launch_bf16_to_f32(armor_ctx* c, const void* in, const float* colscale, float* out, int64_t rows, int64_t cols,
                         cudaStream_t s);
 void launch_f32_to_bf16(armor_ctx* c, const float* in, const float* colscale, void* out, int64_t rows, int64_t cols,
@@ -412,6 +416,7 @@ struct TcGemm {
   int fp16;              // passes 0 / 6: the 16-bit type is fp16 (1) or bf16 (0)
   int mn_major;          // passes 0 / 6: A and B (and their low parts) are [K][M] and [K][N] arrays (lda, ldb: distance of two k)
   const float* row_scale; const float* col_scale;   // both or neither: C = acc * row_scale[m] * col_scale[n]
+  int dependent;         // programmatic dependent launch behind the kernel that writes the scales (only they are waited for)
   int64_t k_segment;     // K extent accumulated in tensor memory before it is folded into C (0: all of K)
   int accumulate;        // C += (read-modify-write) instead of C =
   int symmetric_lower;   // only the lower triangle (tiles with n0 <= m0, elements with column <= row) is computed (M == N)

@@ -60,6 +60,7 @@ struct Params {
   const float* d1; const float* d2;
   double* part1; double* part2;
   const float* row_scale; const float* col_scale;   // optional powers of two the accumulator is multiplied by
+  int dependent;         // launched beside the kernel that writes the scales: the epilogue waits for it
   int f16;               // 16-bit operands are fp16 (1) or bf16 (0)
   int32_t* status;
   // Tail split: tiles [split_first, n_tiles_total) are cut into split_parts pieces of split_kt k-tiles (the last one
@@ -383,6 +384,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
     float4* stg = reinterpret_cast<float4*>(smem + (size_t)STAGES * STAGE_BYTES + (size_t)(warp - 2) * EPI_BYTES);
     int local = 0;
     bool ok = true;
+    if (p.dependent) grid_dependency_wait();
     for (int item = pair; item < p.n_items && ok; item += n_pairs) {
       int tile, part, kt_begin, kt_end, mt, nt;
       item_decode(p, item, kt_total, tile, part, kt_begin, kt_end);
@@ -574,10 +576,12 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
                                                   : 2.0 * (double)p.M * (double)p.N * (double)p.K, s);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = SMEM; cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at; cfg.numAttrs = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at; cfg.numAttrs = p.dependent ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
       tc_gemm_fixup_kernel<<<PARTS * (p.n_tiles_total - p.split_first), FIX_NT, 0, s>>>(p);
@@ -607,7 +611,7 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
   p.n_tiles_total = g.symmetric_lower ? p.m_tiles * (p.m_tiles + 1) / 2 : p.m_tiles * p.n_tiles;
   p.accumulate = g.accumulate; p.symmetric_lower = g.symmetric_lower;
   p.d1 = g.d1; p.d2 = g.d2; p.part1 = g.part1; p.part2 = g.part2;
-  p.row_scale = g.row_scale; p.col_scale = g.col_scale; p.f16 = g.fp16;
+  p.row_scale = g.row_scale; p.col_scale = g.col_scale; p.dependent = g.dependent; p.f16 = g.fp16;
   p.status = c->status;
   p.c_vec = (reinterpret_cast<uintptr_t>(g.C) % 16 == 0) ? 1 : 0;   // (ldc is a multiple of 4)
   const int bke = h16 ? 64 : BK;

@@ -554,9 +554,12 @@ __global__ void __launch_bounds__(NT) f32_to_bf16_kernel(const float* __restrict
 
 // H[r][c] = H[c][r] for c > r: the upper triangle from the lower one, 64 x 64 tiles through shared memory, 16 bytes an access
 // (VEC: rows start on 16-byte boundaries and n is a multiple of 4); a CTA per tile on or below the diagonal.
+// in_range not null: H is the Gram of a bf16 X [n_rows][ldx] whose product left out the channels with in_range 0: their entries
+// are added first, a warp per entry, in fp64 (a channel of values below 2^-57 throughout: time does not count).
 constexpr int MIR = 64;
 template <bool VEC>
-__global__ void __launch_bounds__(NT) mirror_lower_kernel(float* __restrict__ H, int64_t n) {
+__global__ void __launch_bounds__(NT) mirror_lower_kernel(float* H, int64_t n, const __nv_bfloat16* __restrict__ X, int64_t ldx,
+                                                          int64_t n_rows, const float* __restrict__ in_range) {
   // blockIdx.x counts the tiles (i, j), j <= i, of the lower triangle row by row
   int i = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
   while ((int64_t)(i + 1) * (i + 2) / 2 <= (int64_t)blockIdx.x) ++i;
@@ -564,6 +567,22 @@ __global__ void __launch_bounds__(NT) mirror_lower_kernel(float* __restrict__ H,
   const int j = (int)((int64_t)blockIdx.x - (int64_t)i * (i + 1) / 2);
   __shared__ float tile[MIR][MIR + 1];
   const int64_t r0 = (int64_t)i * MIR, c0 = (int64_t)j * MIR;            // source tile
+  if (in_range) {
+    const int64_t k = (threadIdx.x < MIR ? r0 : c0 - MIR) + threadIdx.x;
+    if (__syncthreads_or(threadIdx.x < 2 * MIR && k < n && in_range[k] == 0.f)) {
+      const int lane = threadIdx.x & 31;
+      for (int e = threadIdx.x >> 5; e < MIR * MIR; e += NT / 32) {
+        const int64_t r = r0 + e / MIR, c = c0 + e % MIR;
+        if (r >= n || c > r || (in_range[r] != 0.f && in_range[c] != 0.f)) continue;
+        double acc = 0.0;
+        for (int64_t t = lane; t < n_rows; t += 32)
+          acc += (double)__bfloat162float(X[t * ldx + r]) * (double)__bfloat162float(X[t * ldx + c]);
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (lane == 0) H[r * n + c] = (float)((double)H[r * n + c] + acc);
+      }
+      __syncthreads();
+    }
+  }
   const int q = threadIdx.x & 15, w = threadIdx.x >> 4;
   float4 v[4];
 #pragma unroll
@@ -814,12 +833,14 @@ void launch_transpose_split(armor_ctx* c, const void* X, int x_dtype, int64_t ld
   c->launches++;
 }
 
-void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s) {
+void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s, const void* X_bf16, int64_t ldx, int64_t n_rows,
+                         const float* in_range) {
   const int64_t t = (n + MIR - 1) / MIR;
   const unsigned tiles = (unsigned)(t * (t + 1) / 2);
+  const __nv_bfloat16* X = static_cast<const __nv_bfloat16*>(X_bf16);
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  if (n % 4 == 0 && reinterpret_cast<uintptr_t>(H) % 16 == 0) mirror_lower_kernel<true><<<tiles, NT, 0, s>>>(H, n);
-  else mirror_lower_kernel<false><<<tiles, NT, 0, s>>>(H, n);
+  if (n % 4 == 0 && reinterpret_cast<uintptr_t>(H) % 16 == 0) mirror_lower_kernel<true><<<tiles, NT, 0, s>>>(H, n, X, ldx, n_rows, in_range);
+  else mirror_lower_kernel<false><<<tiles, NT, 0, s>>>(H, n, X, ldx, n_rows, in_range);
   c->launches++;
 }
 

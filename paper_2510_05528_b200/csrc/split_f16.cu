@@ -16,6 +16,7 @@
 #include <cuda_fp16.h>
 
 #include "armor_internal.cuh"
+#include "tc_common.cuh"
 
 namespace {
 
@@ -231,6 +232,48 @@ __global__ void __launch_bounds__(NT) split_columns_kernel(const TIn* __restrict
   }
 }
 
+// Which channels of a bf16 X are in range for a Gram without scaling: 64 channels per CTA, 128 rows at a time until each of
+// them has shown a value that is large enough -- one batch as a rule, so that the kernel is over before the product beside
+// it (a dependent launch) needs the answer; a channel of zeros is read to its end.  256 threads of few registers: a CTA of the
+// product finds room beside one.
+constexpr unsigned RANGE_BITS = (127 - 57) << 7;           // 2^-57
+__global__ void __launch_bounds__(NT) gram_range_kernel(const uint16_t* __restrict__ X, int64_t ldx, int64_t rows, int64_t cols,
+                                                        float* __restrict__ in_range) {
+  __shared__ unsigned big[8], nonzero[8];                  // a bit per channel
+  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
+  const int64_t col = (int64_t)blockIdx.x * 64 + 8 * tx;
+  tc::grid_launch_dependents();
+  if (threadIdx.x < 8) { big[threadIdx.x] = 0u; nonzero[threadIdx.x] = 0u; }
+  __syncthreads();
+  const bool mine = col < cols;                            // (a multiple of 8)
+  bool open = mine;
+  for (int64_t r0 = 0; r0 < rows; r0 += 128) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t r = r0 + ty + 32 * u;
+      v[u] = open && r < rows ? __ldg(reinterpret_cast<const uint4*>(X + r * ldx + col)) : make_uint4(0u, 0u, 0u, 0u);
+    }
+    unsigned b = 0u, z = 0u;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const unsigned w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const unsigned lo = w[k] & 0x7fffu, hi = (w[k] >> 16) & 0x7fffu;      // magnitudes compare like their bits
+        b |= (unsigned)(lo >= RANGE_BITS) << (2 * k) | (unsigned)(hi >= RANGE_BITS) << (2 * k + 1);
+        z |= (unsigned)(lo != 0u) << (2 * k) | (unsigned)(hi != 0u) << (2 * k + 1);
+      }
+    }
+    if (b) atomicOr(&big[tx], b);
+    if (z) atomicOr(&nonzero[tx], z);
+    __syncthreads();
+    open = mine && big[tx] != 0xffu;
+    if (!__syncthreads_or(open)) break;
+  }
+  if (mine && ty < 8) in_range[col + ty] = ((nonzero[tx] & ~big[tx]) >> ty) & 1u ? 0.f : 1.f;
+}
+
 inline unsigned grid_for(int64_t n) {
   int64_t b = (n + NT - 1) / NT;
   return (unsigned)(b < 148 * 8 ? (b < 1 ? 1 : b) : 148 * 8);
@@ -292,4 +335,10 @@ armor_status launch_f16_gram_stage(armor_ctx* c, const void* X, int x_dtype, int
   gram_scale_kernel<<<(unsigned)((cols + 255) / 256), 256, 0, s>>>(c->gmax, gscale, cols);
   c->launches += 3;
   return ARMOR_OK;
+}
+
+void launch_gram_range(armor_ctx* c, const void* X, int64_t ldx, int64_t n_rows, float* in_range, cudaStream_t s) {
+  KTimer kt(c, ARMOR_KC_GRAM_STAGING, 0.0, s);
+  gram_range_kernel<<<(unsigned)((c->d_in + 63) / 64), NT, 0, s>>>(static_cast<const uint16_t*>(X), ldx, n_rows, c->d_in, in_range);
+  c->launches++;
 }

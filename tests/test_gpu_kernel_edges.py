@@ -399,3 +399,49 @@ def test_fp32_gram_of_tiny_and_huge_channels(tokens):
     assert torch.isfinite(H).all()
     assert (err <= (192 * 2.0 ** -23 + 2.0 ** -21) * nrm[:, None] * nrm[None, :] + 2.0 ** -149).all()
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_in,tokens", [(32, 1), (96, 129), (160, 1000), (256, 4100), (640, 16384 + 3000), (1056, 127)])
+def test_bf16_gram_of_tiny_channels(d_in, tokens):
+    """Channels down to 1e-22 beside ordinary ones and channels of zeros, channels that show their size in the last token only,
+    and numbers of channels that leave a tile's box, or a CTA's half of it, over the edge.  Bound of
+    test_bf16_gram_as_it_lies_in_memory, beside 2^-24 of the product of the channels' norms (sums of multiples of 2^-149
+    of channels above 2^-57), and the rounding of an entry that is itself subnormal, once per call."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(tokens + d_in)
+    sizes = torch.tensor([1.0, 1e-17, 1e-19, 10 ** -20.5, 1e-21, 0.0, 10 ** -21.5, 1e-22], dtype=torch.float64, device=DEV)
+    scale = sizes[torch.randint(0, 8, (d_in,), device=DEV, generator=g)]
+    X = (torch.randn(tokens, d_in, device=DEV, generator=g).double() * scale).to(torch.bfloat16)
+    X[:, 3], X[-1, 3] = 0.0, 1e-19
+    X[:, 5], X[-1, 5] = X[:, 5] * 0.0 + 1e-21, 1.0
+    ctx = _ctx(128, d_in, 32, h_mode=Bd.H_DIAG)
+    H = ctx.new_gram()
+    ctx.gram(X, H)
+    Xd = X.double()
+    nrm = Xd.norm(dim=0)
+    ref = Xd.t() @ Xd
+    assert torch.equal(H, H.t())
+    assert ((H.double() - ref).abs() <= 8e-6 * (Xd.abs().t() @ Xd.abs()) + 2.0 ** -24 * nrm[:, None] * nrm[None, :] + 2.0 ** -149).all()
+    ctx.gram(X, H)                       # on top of what is there
+    assert ((H.double() - 2 * ref).abs() <= 2 * (8e-6 * (Xd.abs().t() @ Xd.abs()) + 2.0 ** -24 * nrm[:, None] * nrm[None, :] + 2.0 ** -149)).all()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("d_in,tokens,at", [(96, 65, 64), (640, 5000, 17), (256, 16384 + 9, 16384 + 8)])
+def test_gram_with_a_value_that_is_not_finite(d_in, tokens, at, dtype, bad):
+    """One Inf or NaN stays in its channel's row and column and is visible there; the other entries are those of the clean X."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(tokens + d_in)
+    X = torch.randn(tokens, d_in, device=DEV, generator=g).to(dtype)
+    ctx = _ctx(128, d_in, 32, h_mode=Bd.H_DIAG)
+    clean, H = ctx.new_gram(), ctx.new_gram()
+    ctx.gram(X, clean)
+    k = d_in // 3
+    X[at, k] = bad
+    ctx.gram(X, H)
+    others = torch.arange(d_in, device=DEV) != k
+    assert not torch.isfinite(H[k, k])
+    assert not torch.isfinite(H[k]).any() and not torch.isfinite(H[:, k]).any()
+    assert torch.equal(H[others][:, others], clean[others][:, others])
