@@ -113,10 +113,11 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
     // the channels, products of two bf16 values have 16 significant bits, so nothing is scaled, transposed or staged.  (A
     // leading dimension or base that TMA does not take leaves the staged path below.)
     // The accumulator rounds to multiples of 2^-149: about 2^-139 in a sum of 16,384 tokens, which counts only between two
-    // channels whose norms multiply to less than 2^-115.  A channel that nowhere reaches 2^-57 is therefore left out of the
-    // product (its scale is 0) and its entries are summed in fp64 before the mirroring.
+    // channels whose norms multiply to less than 2^-115.  In the mode that scales its operands a channel that nowhere reaches
+    // 2^-57 is therefore left out of the product (its scale is 0) and its entries are summed in fp64 before the mirroring.
     // One launch per gram_rows tokens, as in the staged path: a long call sums like a sequence of shorter ones.
-    launch_gram_range(c, Xv, ldx, n_rows, c->gscale, s);
+    float* const in_range = c->cfg.precision == ARMOR_PREC_FP16X3 ? c->gscale : nullptr;
+    if (in_range) launch_gram_range(c, Xv, ldx, n_rows, in_range, s);
     for (int64_t r0 = 0; r0 < n_rows; r0 += c->gram_rows) {
       TcGemm g{};
       g.A = static_cast<const char*>(Xv) + (size_t)(r0 * ldx) * 2; g.lda = ldx;
@@ -124,15 +125,15 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
       g.C = H; g.ldc = d_in;
       g.M = d_in; g.N = d_in; g.K = n_rows - r0 < c->gram_rows ? n_rows - r0 : c->gram_rows;
       g.passes = 0; g.mn_major = 1;
-      g.row_scale = g.col_scale = c->gscale;
-      g.dependent = r0 == 0;
+      g.row_scale = g.col_scale = in_range;
+      g.dependent = in_range && r0 == 0;
       g.accumulate = 1;
       g.symmetric_lower = 1;
       g.k_segment = K_SEGMENT;
       const armor_status st = launch_tc_gemm(c, g, nullptr, s);
       if (st != ARMOR_OK) return st;
     }
-    launch_mirror_lower(c, H, d_in, s, Xv, ldx, n_rows, c->gscale);
+    launch_mirror_lower(c, H, d_in, s, Xv, ldx, n_rows, in_range);
     return ARMOR_OK;
   }
   if (c->cfg.precision == ARMOR_PREC_FP16X3) {

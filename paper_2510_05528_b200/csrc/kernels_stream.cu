@@ -567,6 +567,22 @@ __global__ void __launch_bounds__(NT) mirror_lower_kernel(float* H, int64_t n, c
   const int j = (int)((int64_t)blockIdx.x - (int64_t)i * (i + 1) / 2);
   __shared__ float tile[MIR][MIR + 1];
   const int64_t r0 = (int64_t)i * MIR, c0 = (int64_t)j * MIR;            // source tile
+  const int q = threadIdx.x & 15, w = threadIdx.x >> 4;
+  float4 v[4];
+  auto fetch = [&]() {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int64_t r = r0 + w + 16 * k, c = c0 + 4 * q;
+      v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r >= n) continue;
+      if (VEC) { if (c < n) v[k] = *reinterpret_cast<const float4*>(H + r * n + c); }
+      else {
+        float* f = &v[k].x;
+        for (int t = 0; t < 4; ++t) if (c + t < n) f[t] = H[r * n + c + t];
+      }
+    }
+  };
+  fetch();
   if (in_range) {
     const int64_t k = (threadIdx.x < MIR ? r0 : c0 - MIR) + threadIdx.x;
     if (__syncthreads_or(threadIdx.x < 2 * MIR && k < n && in_range[k] == 0.f)) {
@@ -581,19 +597,7 @@ __global__ void __launch_bounds__(NT) mirror_lower_kernel(float* H, int64_t n, c
         if (lane == 0) H[r * n + c] = (float)((double)H[r * n + c] + acc);
       }
       __syncthreads();
-    }
-  }
-  const int q = threadIdx.x & 15, w = threadIdx.x >> 4;
-  float4 v[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const int64_t r = r0 + w + 16 * k, c = c0 + 4 * q;
-    v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r >= n) continue;
-    if (VEC) { if (c < n) v[k] = *reinterpret_cast<const float4*>(H + r * n + c); }
-    else {
-      float* f = &v[k].x;
-      for (int t = 0; t < 4; ++t) if (c + t < n) f[t] = H[r * n + c + t];
+      fetch();
     }
   }
 #pragma unroll
