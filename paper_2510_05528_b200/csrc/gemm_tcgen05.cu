@@ -335,12 +335,12 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         for (int kt0 = kt_begin; kt0 < kt_end && ok; kt0 += p.kt_seg, ++local) {
           const int as = local & 1;
           const uint32_t aphase = (uint32_t)(local >> 1) & 1u;
-          if (!mbar_wait(tempty0 + 8 * as, aphase ^ 1, abortp, p.status)) { ok = false; break; }
+          if (!mbar_wait_cluster(tempty0 + 8 * as, aphase ^ 1, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t tacc = tmem_base + (uint32_t)(as * BN);
           const int kt1 = min(kt_end, kt0 + p.kt_seg);
           for (int kt = kt0; kt < kt1; ++kt) {
-            if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+            if (!mbar_wait_cluster(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
             tc_fence_after();
             // One thread issues every MMA: the descriptors of stage 0 are formed once and only their address field
             // moves, and every MMA but a tile's first carries a constant accumulate flag, so that the instructions

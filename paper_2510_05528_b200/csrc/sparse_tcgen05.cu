@@ -375,10 +375,10 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
       int local = 0;
       bool ok = true;
       for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs, ++local) {
-        if (!mbar_wait(tempty, ((uint32_t)local & 1u) ^ 1u, abortp, p.status)) { ok = false; break; }
+        if (!mbar_wait_cluster(tempty, ((uint32_t)local & 1u) ^ 1u, abortp, p.status)) { ok = false; break; }
         tc_fence_after();
         for (int kt = 0; kt < p.k_tiles; ++kt) {
-          if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+          if (!mbar_wait_cluster(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t sa = smem_u32(smem + (size_t)stage * STAGE_BYTES);
           const uint32_t sb = sa + A_BYTES;
