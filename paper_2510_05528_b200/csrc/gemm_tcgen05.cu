@@ -23,6 +23,9 @@
 // so the caller scales rows of the operands by powers of two into the fp16 range beforehand and the epilogue
 // multiplies the accumulator by the inverse scales (a per-row and a per-column vector): every scaling is
 // exact, the result is fp32-grade.
+// Few rows (FEW, the bf16 core product of up to 512 tokens): the operands change sides.  256 columns of C are the M side of an
+// instruction and the rows of a tile, only as many as there are, its N side, so that neither the MMAs nor the fetched bytes
+// are spent on rows that do not exist (a 256 x 256 tile of one row took 43 us of MMAs for 21 us of reading at 8192 x 8192).
 // Every wait is bounded: a wait that runs out raises a status word and the CTA leaves through the common
 // exit that frees its tensor memory.
 #include "tc_common.cuh"
@@ -67,6 +70,7 @@ struct Params {
   // may be shorter), each piece a work item of its own that writes a 256 x 256 slab of partial sums; a second kernel
   // adds the slabs.  This fills the last, partly empty wave of tiles.
   int split_first, split_parts, split_kt, n_items;
+  int tile_m;            // rows of C per tile: 256; FEW: the rows dealt evenly to one or two tiles, a multiple of 32
   float* slabs;
 };
 
@@ -107,14 +111,14 @@ __device__ __forceinline__ void umma_first(uint32_t tmem_d, uint64_t adesc, uint
 
 // fp32 accumulate, M = 256 (the pair), N = 256; operand format 0: fp16, 1: bf16 (both kind::f16), 2: tf32
 // (kind::tf32); mn: both operands are contiguous along M / N instead of K.
-__device__ __forceinline__ uint32_t instr_desc(uint32_t fmt, uint32_t mn) {
+__device__ __forceinline__ uint32_t instr_desc(uint32_t fmt, uint32_t mn, uint32_t n = BN) {
   uint32_t d = 0;
   d |= 1u << 4;                   // D format: F32
   d |= fmt << 7;                  // A format
   d |= fmt << 10;                 // B format
   d |= mn << 15;
   d |= mn << 16;
-  d |= (uint32_t)(BN >> 3) << 17; // N
+  d |= (n >> 3) << 17;            // N
   d |= (uint32_t)(BMP >> 4) << 24; // M
   return d;
 }
@@ -228,8 +232,8 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* 
   }
 }
 
-// MN: both operands are 16-bit arrays contiguous along M / N (PASSES 0 and 6)
-template <int PASSES, bool MN>
+// MN: both operands are 16-bit arrays contiguous along M / N (PASSES 0 and 6).  FEW: PASSES 0, K-major, C = A B^T and nothing else.
+template <int PASSES, bool MN, bool FEW>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapAlo,
                const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo, const Params p) {
@@ -270,6 +274,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   __syncthreads();
   cluster_sync_all();                                  // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
+  if (PASSES == 0 && !MN) grid_launch_dependents();    // (the kernel that adds the pieces of cut tiles, see launch_impl)
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -285,10 +290,13 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         const int arow = mt * BMP + (int)rank * BM, brow = nt * BN + (int)rank * BNH;
         for (int kt = kt_begin; kt < kt_end; ++kt) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, FEW ? 2 * (A_BYTES + (p.tile_m / 2) * 128) : 2 * STAGE_BYTES);
           const uint32_t fb = map_to_cta(full0 + 8 * stage, 0);
           uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          if (MN) {
+          if (FEW) {
+            tma_load_2d_pair(dst, &mapB, kt * BKE, brow, fb);
+            tma_load_2d_pair(dst + A_BYTES, &mapA, kt * BKE, mt * p.tile_m + (int)rank * (p.tile_m / 2), fb);
+          } else if (MN) {
             // x = row of the operand (a channel), y = k (a token); rows and k beyond the operand are zero-filled
 #pragma unroll
             for (int part = 0; part < (SPLIT ? 2 : 1); ++part) {
@@ -324,7 +332,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA)
     if (lane == 0 && rank == 0) {
-      const uint32_t idesc = instr_desc(H16 ? (p.f16 ? 0u : 1u) : 2u, MN ? 1u : 0u);
+      const uint32_t idesc = instr_desc(H16 ? (p.f16 ? 0u : 1u) : 2u, MN ? 1u : 0u, FEW ? (uint32_t)p.tile_m : BN);
       const uint64_t d0 = MN ? smem_desc_mn_sw128(smem_u32(smem)) : smem_desc_k_sw128(smem_u32(smem));
       int stage = 0; uint32_t phase = 0;
       int local = 0;   // (tile, K segment) items handled so far: selects the accumulator buffer
@@ -399,6 +407,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         tc_fence_after();
 #pragma unroll
         for (int ch = 0; ch < EPI_COLS / 32; ++ch) {
+          if (FEW && half * EPI_COLS + ch * 32 >= p.tile_m) continue;    // warp-uniform
           uint32_t r[32];
           tmem_ld32(tmem_base + (uint32_t)(as * BN + half * EPI_COLS + ch * 32) + ((uint32_t)(q * 32) << 16), r);
 #pragma unroll
@@ -409,6 +418,22 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty0 + 8 * as, 0));
       }
       if (!ok) break;
+      if (FEW) {
+        // lane = column of C, accumulator column = row: 128 bytes of a row per store; a piece into its slab, [row][column]
+        const int64_t col = (int64_t)nt * BN + rank * BM + q * 32 + lane, row0 = (int64_t)mt * p.tile_m;
+        float* out = part < 0 ? p.C + row0 * p.ldc + col
+                              : p.slabs + ((int64_t)(tile - p.split_first) * p.split_parts + part) * (BMP * BN) + rank * BM + q * 32 + lane;
+        const int64_t ld = part < 0 ? p.ldc : BN;
+        const int64_t left = p.M - row0;
+        const int rows = (int)(left < p.tile_m ? left : p.tile_m) - half * EPI_COLS;
+        out += (int64_t)half * EPI_COLS * ld;
+        if (col < p.N) {                                                 // warp-uniform (N is a multiple of 32)
+#pragma unroll
+          for (int i = 0; i < EPI_COLS; ++i)
+            if (i < rows) out[i * ld] = acc[i];
+        }
+        continue;
+      }
       if (part >= 0) {
         // a piece of a split tile: its partial sums go, plainly, to this item's slab
         float* slab = p.slabs + (((int64_t)(tile - p.split_first) * p.split_parts + part) * 2 + rank) * (BM * BN);
@@ -448,14 +473,16 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 constexpr int FIX_NT = BMP / PARTS * BN / 4;
 __global__ void __launch_bounds__(FIX_NT) tc_gemm_fixup_kernel(const Params p) {
   constexpr int FR = BMP / PARTS;                         // rows per CTA
-  const int tile = p.split_first + blockIdx.x / PARTS, slot = blockIdx.x % PARTS;
+  grid_dependency_wait();                                 // (where it is launched beside the product's tail)
+  const int slots = gridDim.x / (p.n_tiles_total - p.split_first);       // PARTS, or those that hold rows
+  const int tile = p.split_first + blockIdx.x / slots, slot = blockIdx.x % slots;
   int mt, nt;
   tile_coords(p, tile, mt, nt);
-  const float* slab0 = p.slabs + (int64_t)(blockIdx.x / PARTS) * p.split_parts * (BMP * BN) + (int64_t)slot * FR * BN;
+  const float* slab0 = p.slabs + (int64_t)(blockIdx.x / slots) * p.split_parts * (BMP * BN) + (int64_t)slot * FR * BN;
   double d1 = 0.0, d2 = 0.0;
   const int r = threadIdx.x / (BN / 4), c4 = (threadIdx.x % (BN / 4)) * 4;
-  const int64_t grow = (int64_t)mt * BMP + slot * FR + r, gcol = (int64_t)nt * BN + c4;
-  if (grow < p.M && gcol < p.N && !(p.symmetric_lower && gcol > grow)) {
+  const int64_t grow = (int64_t)mt * p.tile_m + slot * FR + r, gcol = (int64_t)nt * BN + c4;
+  if (slot * FR + r < p.tile_m && grow < p.M && gcol < p.N && !(p.symmetric_lower && gcol > grow)) {
     const float* sp = slab0 + (int64_t)r * BN + c4;
     float4 v = *reinterpret_cast<const float4*>(sp);
 #pragma unroll 4
@@ -520,13 +547,13 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64
   return r == CUDA_SUCCESS;
 }
 
-template <int PASSES, bool MN>
+template <int PASSES, bool MN, bool FEW = false>
 armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s) {
   CUtensorMap mA, mAlo, mB, mBlo;
   constexpr bool SPLIT = (PASSES == 3 || PASSES == 6);
   constexpr bool H16 = (PASSES == 0 || PASSES == 6);
   const int bits16 = H16 ? (g.fp16 ? 2 : 1) : 0;
-  if (!make_map(&mA, g.A, g.M, g.K, g.lda, BM, bits16, MN)) return ARMOR_ERR_CUDA;
+  if (!make_map(&mA, g.A, g.M, g.K, g.lda, FEW ? p.tile_m / 2 : BM, bits16, MN)) return ARMOR_ERR_CUDA;
   if (!make_map(&mB, g.B, g.N, g.K, g.ldb, BNH, bits16, MN)) return ARMOR_ERR_CUDA;
   if (SPLIT) {
     if (!make_map(&mAlo, g.Alo, g.M, g.K, g.lda, BM, bits16, MN)) return ARMOR_ERR_CUDA;
@@ -537,7 +564,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
   }
   constexpr size_t SMEM = (size_t)Ring<PASSES>::STAGES * Ring<PASSES>::BYTES + 1024 + 8 * EPI_BYTES;
   static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES, MN>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES, MN, FEW>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int n_pairs = c->n_sm / 2;
   if (n_pairs < 1) return ARMOR_ERR_UNSUPPORTED;
   // Tail split: the tiles of the last, partly filled wave are cut along K so that their pieces fill the wave.  Where the
@@ -554,7 +581,9 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     const int fill = n_pairs / rem;                                // pieces per tile that still fit the wave
     int per = kt_total;
     if (!SPLIT && p.kt_seg >= kt_total) {
-      if (fill > 1) per = (kt_total + (fill < 4 ? fill : 4) - 1) / (fill < 4 ? fill : 4);
+      // (more pieces are more slabs to add, at most four; eight where few rows of a slab exist: 1,024 x 5,120, 600 tokens 80 -> 78 us)
+      const int most = PASSES == 0 && !MN ? 8 : 4;
+      if (fill > 1) per = (kt_total + (fill < most ? fill : most) - 1) / (fill < most ? fill : most);
     } else {
       for (int parts = fill < 4 ? fill : 4; parts > 1 && !p.symmetric_lower && per == kt_total; --parts)
         if (kt_total % parts == 0 && kt_total / parts >= 8 && ((kt_total / parts) % p.kt_seg == 0 || kt_total / parts <= p.kt_seg))
@@ -582,9 +611,16 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = p.dependent ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN, FEW>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
-      tc_gemm_fixup_kernel<<<PARTS * (p.n_tiles_total - p.split_first), FIX_NT, 0, s>>>(p);
+      // 16 rows per CTA; the slots of rows that do not exist are launched only where each has a partial sum to write
+      const int64_t rows = p.M < p.tile_m ? p.M : p.tile_m;
+      const int slots = (p.part1 || p.part2) ? PARTS : (int)((rows + BMP / PARTS - 1) / (BMP / PARTS));
+      cudaLaunchConfig_t fc{};
+      fc.gridDim = dim3(slots * (p.n_tiles_total - p.split_first)); fc.blockDim = dim3(FIX_NT); fc.stream = s;
+      // behind the bf16 product it is a dependent launch: with a handful of tokens its launch counts
+      fc.attrs = &at[1]; fc.numAttrs = PASSES == 0 && !MN ? 1 : 0;
+      if (cudaLaunchKernelEx(&fc, tc_gemm_fixup_kernel, p) != cudaSuccess) return ARMOR_ERR_CUDA;
       c->launches++;
     }
   }
@@ -617,6 +653,7 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
   const int bke = h16 ? 64 : BK;
   p.kt_seg = g.k_segment > 0 ? (int)((g.k_segment + bke - 1) / bke) : (int)((g.K + bke - 1) / bke);
   if (p.kt_seg < 1) p.kt_seg = 1;
+  p.tile_m = BMP;
   if (n_part) *n_part = PARTS * p.n_tiles_total;
   if (g.mn_major) {
     // a map's rows start at multiples of 64 elements; the base and the leading dimension must be multiples of 16 bytes
@@ -625,6 +662,15 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
   }
   if (g.passes == 3) return launch_impl<3, false>(c, g, p, s);
   if (g.passes == 6) return launch_impl<6, false>(c, g, p, s);
-  if (g.passes == 0) return launch_impl<0, false>(c, g, p, s);
+  if (g.passes == 0) {
+    // Few rows: dealt evenly to one or two tiles.  (The core product of a forward with them, whole pass at 8192 x 8192: 1 token
+    // 156 -> 142 us, 300 186 -> 176, 512 198 -> 191; from three tiles on the two forms are alike.)
+    const int even = (int)((g.M + p.m_tiles - 1) / p.m_tiles + 31) / 32 * 32;
+    if (p.m_tiles <= 2 && !g.row_scale && !g.accumulate && !g.symmetric_lower && !g.d1 && !g.d2) {
+      p.tile_m = even;
+      return launch_impl<0, false, true>(c, g, p, s);
+    }
+    return launch_impl<0, false>(c, g, p, s);
+  }
   return launch_impl<1, false>(c, g, p, s);
 }

@@ -445,3 +445,30 @@ def test_gram_with_a_value_that_is_not_finite(d_in, tokens, at, dtype, bad):
     assert not torch.isfinite(H[k, k])
     assert not torch.isfinite(H[k]).any() and not torch.isfinite(H[:, k]).any()
     assert torch.equal(H[others][:, others], clean[others][:, others])
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(128, 128, 128), (160, 96, 32), (640, 2560, 128), (1024, 6144, 256), (4096, 4096, 128),
+                                                (19072, 2048, 128)])
+def test_bf16_forward_of_few_tokens_with_the_dense_core(d_out, d_in, d_block):
+    """Token counts at the edges of the narrow tiles (32, 64, .. per tile, one tile up to 256, two up to 512, whole tiles beyond),
+    core products cut along d_in and not.  Integer operands: every fp32 sum is exact in any order and every value on the way
+    is an integer below 2^8 or rounded to bf16 in one place, so the result is that of fp64, bit for bit."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + 5 * d_in)
+    ctx = _ctx(d_out, d_in, d_block, h_mode=Bd.H_DIAG)
+
+    def sparse_ints(hi, density, *shape):
+        return torch.randint(-hi, hi + 1, shape, device=DEV, generator=g).float() * (torch.rand(shape, device=DEV, generator=g) < density)
+    S = sparse_ints(3, 0.5, d_out, d_in)
+    A = sparse_ints(1, 4.0 / d_block, d_out // d_block, d_block, d_block)
+    B = sparse_ints(1, 4.0 / d_block, d_in // d_block, d_block, d_block)
+    st = Bd.LayerState(Wbar=S, A=A, B=B, S=S, M=torch.zeros(d_out, d_in // 4, dtype=torch.uint8, device=DEV))
+    x = sparse_ints(2, 0.5, 600, d_in).to(torch.bfloat16)
+    z1 = torch.einsum("tjk,jmk->tjm", x.double().view(600, -1, d_block), B.double()).reshape(600, d_in)
+    assert z1.abs().max() < 256
+    z2 = z1 @ S.double().t()
+    assert z2.abs().max() < 2 ** 11                      # exact as one tf32 operand of the last product
+    y = torch.einsum("tjk,jmk->tjm", z2.view(600, -1, d_block), A.double()).reshape(600, d_out).float().to(torch.bfloat16)
+    for n in (1, 2, 31, 32, 33, 64, 65, 127, 128, 129, 224, 225, 255, 256, 257, 300, 448, 449, 511, 512, 513, 600):
+        assert torch.equal(ctx.apply(st, x[:n].contiguous()), y[:n]), n
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
