@@ -196,9 +196,9 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* 
     __syncwarp();
     const int64_t col = col0 + 4 * cc;
     const float4 sc4 = cs ? *reinterpret_cast<const float4*>(cs + col) : make_float4(1.f, 1.f, 1.f, 1.f);
-    float f1 = 0.f, f2 = 0.f;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
+      float f1 = 0.f, f2 = 0.f;                                // 16 terms in fp32, then fp64
       float4 o[4];
       if (accum) {
 #pragma unroll
@@ -225,9 +225,9 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* 
         }
         store4(C + grow * ldc + col, x, vec);
       }
+      dot1 += (double)f1;
+      dot2 += (double)f2;
     }
-    dot1 += (double)f1;
-    dot2 += (double)f2;
     __syncwarp();
   }
 }
@@ -581,7 +581,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     const int fill = n_pairs / rem;                                // pieces per tile that still fit the wave
     int per = kt_total;
     if (!SPLIT && p.kt_seg >= kt_total) {
-      // (more pieces are more slabs to add, at most four; eight where few rows of a slab exist: 1,024 x 5,120, 600 tokens 80 -> 78 us)
+      // (more pieces are more slabs to add: at most four, eight of the bf16 product: 1,024 x 5,120, 600 tokens 80 -> 78 us)
       const int most = PASSES == 0 && !MN ? 8 : 4;
       if (fill > 1) per = (kt_total + (fill < most ? fill : most) - 1) / (fill < most ? fill : most);
     } else {

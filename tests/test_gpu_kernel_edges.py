@@ -472,3 +472,22 @@ def test_bf16_forward_of_few_tokens_with_the_dense_core(d_out, d_in, d_block):
     for n in (1, 2, 31, 32, 33, 64, 65, 127, 128, 129, 224, 225, 255, 256, 257, 300, 448, 449, 511, 512, 513, 600):
         assert torch.equal(ctx.apply(st, x[:n].contiguous()), y[:n]), n
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("precision", ["FP16X3", "FP32X3"])
+@pytest.mark.parametrize("d_out,d_in", [(256, 512), (4096, 4096)])
+def test_fused_dot_product_keeps_small_terms(d_out, d_in, precision):
+    """L = <E H, E> of an E with rows of 1024 and rows of 7 / 16 in turns of 16, H = I: every product and every sum of the 16
+    terms that a lane adds in fp32 is exact (2^20 or 49 / 256 each), and a lane's two runs meet in fp64.  Summed in fp32 across
+    the runs the small rows vanish (2^24 + 0.77), 1.8e-7 of the loss."""
+    from paper_2510_05528_b200 import binding as Bd
+    ctx = _ctx(d_out, d_in, 128, precision=getattr(Bd, "PREC_" + precision))
+    W = torch.full((d_out, d_in), 1024.0, device=DEV)
+    W.view(-1, 2, 16, d_in)[:, 1] = 0.4375
+    H = torch.eye(d_in, device=DEV)
+    st = ctx.init(W, H)
+    st.S.zero_()
+    loss = ctx.proxy_loss(st, H).item()
+    ref = W.double().square().sum().item()
+    assert abs(loss - ref) <= 1e-9 * ref
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
