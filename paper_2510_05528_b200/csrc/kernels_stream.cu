@@ -554,11 +554,12 @@ __global__ void __launch_bounds__(NT) f32_to_bf16_kernel(const float* __restrict
 
 // H[r][c] = H[c][r] for c > r: the upper triangle from the lower one, 64 x 64 tiles through shared memory, 16 bytes an access
 // (VEC: rows start on 16-byte boundaries and n is a multiple of 4); a CTA per tile on or below the diagonal.
-// in_range not null: H is the Gram of a bf16 X [n_rows][ldx] whose product left out the channels with in_range 0: their entries
-// are added first, a warp per entry, in fp64 (a channel of values below 2^-57 throughout: time does not count).
+// LEFT_OUT: H is the Gram of a bf16 X [n_rows][ldx] whose product left out the channels with in_range 0: their entries are added
+// first, a warp per entry, in fp64 (a channel of values below 2^-57 throughout: time does not count).  Eight CTAs per SM in
+// either form: with five, the 409 MB of 10,112 channels took 12 us more.
 constexpr int MIR = 64;
-template <bool VEC>
-__global__ void __launch_bounds__(NT) mirror_lower_kernel(float* H, int64_t n, const __nv_bfloat16* __restrict__ X, int64_t ldx,
+template <bool VEC, bool LEFT_OUT>
+__global__ void __launch_bounds__(NT, 8) mirror_lower_kernel(float* H, int64_t n, const __nv_bfloat16* __restrict__ X, int64_t ldx,
                                                           int64_t n_rows, const float* __restrict__ in_range) {
   // blockIdx.x counts the tiles (i, j), j <= i, of the lower triangle row by row
   int i = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(NT) mirror_lower_kernel(float* H, int64_t n, c
     }
   };
   fetch();
-  if (in_range) {
+  if (LEFT_OUT) {
     const int64_t k = (threadIdx.x < MIR ? r0 : c0 - MIR) + threadIdx.x;
     if (__syncthreads_or(threadIdx.x < 2 * MIR && k < n && in_range[k] == 0.f)) {
       const int lane = threadIdx.x & 31;
@@ -843,8 +844,14 @@ void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s, cons
   const unsigned tiles = (unsigned)(t * (t + 1) / 2);
   const __nv_bfloat16* X = static_cast<const __nv_bfloat16*>(X_bf16);
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  if (n % 4 == 0 && reinterpret_cast<uintptr_t>(H) % 16 == 0) mirror_lower_kernel<true><<<tiles, NT, 0, s>>>(H, n, X, ldx, n_rows, in_range);
-  else mirror_lower_kernel<false><<<tiles, NT, 0, s>>>(H, n, X, ldx, n_rows, in_range);
+  const bool vec = n % 4 == 0 && reinterpret_cast<uintptr_t>(H) % 16 == 0;
+  if (in_range) {
+    if (vec) mirror_lower_kernel<true, true><<<tiles, NT, 0, s>>>(H, n, X, ldx, n_rows, in_range);
+    else mirror_lower_kernel<false, true><<<tiles, NT, 0, s>>>(H, n, X, ldx, n_rows, in_range);
+  } else {
+    if (vec) mirror_lower_kernel<true, false><<<tiles, NT, 0, s>>>(H, n, nullptr, 0, 0, nullptr);
+    else mirror_lower_kernel<false, false><<<tiles, NT, 0, s>>>(H, n, nullptr, 0, 0, nullptr);
+  }
   c->launches++;
 }
 
