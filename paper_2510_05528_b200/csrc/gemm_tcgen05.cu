@@ -176,7 +176,9 @@ __device__ __forceinline__ void store4(float* q, const float4& v, int vec) {
 // One epilogue warp's 32 rows x 128 columns of finished sums (lane = row) go out through a 32 x 32 staging tile in
 // shared memory (16-byte units, swizzled by the row: no bank conflicts either way), so that every access to C writes or
 // reads four rows of 128 contiguous bytes.  Optional: power-of-two scales, C += (read-modify-write), chunks of 32 x 32
-// above the diagonal left out, partial dot products with d1 / d2.
+// above the diagonal left out, partial dot products with d1 / d2 (DOTS; without, the code for them is not there: fp64 conversions
+// of nothing cost a Gram of few tokens 3 %).
+template <bool DOTS>
 __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* stg, int lane, float* C, int64_t ldc, int vec,
                                           int64_t row_base, int64_t col_base, int64_t M, int64_t N, bool accum, bool sym,
                                           const float* rs, const float* cs, const float* d1, const float* d2, int64_t ldd,
@@ -196,9 +198,9 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* 
     __syncwarp();
     const int64_t col = col0 + 4 * cc;
     const float4 sc4 = cs ? *reinterpret_cast<const float4*>(cs + col) : make_float4(1.f, 1.f, 1.f, 1.f);
+    float f1[2] = {0.f, 0.f}, f2[2] = {0.f, 0.f};              // 16 terms each in fp32, then fp64
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      float f1 = 0.f, f2 = 0.f;                                // 16 terms in fp32, then fp64
       float4 o[4];
       if (accum) {
 #pragma unroll
@@ -215,25 +217,28 @@ __device__ __forceinline__ void write_out(const float (&acc)[EPI_COLS], float4* 
         float4 x = stg[r * 8 + (cc ^ (r & 7))];
         x.x *= sc4.x; x.y *= sc4.y; x.z *= sc4.z; x.w *= sc4.w;
         if (accum) { x.x += o[i].x; x.y += o[i].y; x.z += o[i].z; x.w += o[i].w; }
-        if (d1) {
+        if (DOTS && d1) {
           const float4 w = *reinterpret_cast<const float4*>(d1 + grow * ldd + col);
-          f1 += x.x * w.x + x.y * w.y + x.z * w.z + x.w * w.w;
+          f1[h] += x.x * w.x + x.y * w.y + x.z * w.z + x.w * w.w;
         }
-        if (d2) {
+        if (DOTS && d2) {
           const float4 w = *reinterpret_cast<const float4*>(d2 + grow * ldd + col);
-          f2 += x.x * w.x + x.y * w.y + x.z * w.z + x.w * w.w;
+          f2[h] += x.x * w.x + x.y * w.y + x.z * w.z + x.w * w.w;
         }
         store4(C + grow * ldc + col, x, vec);
       }
-      dot1 += (double)f1;
-      dot2 += (double)f2;
+    }
+    if (DOTS) {
+      dot1 += (double)f1[0] + (double)f1[1];
+      dot2 += (double)f2[0] + (double)f2[1];
     }
     __syncwarp();
   }
 }
 
 // MN: both operands are 16-bit arrays contiguous along M / N (PASSES 0 and 6).  FEW: PASSES 0, K-major, C = A B^T and nothing else.
-template <int PASSES, bool MN, bool FEW>
+// DOTS: with dot products.
+template <int PASSES, bool MN, bool FEW, bool DOTS>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapAlo,
                const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo, const Params p) {
@@ -439,14 +444,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
         float* slab = p.slabs + (((int64_t)(tile - p.split_first) * p.split_parts + part) * 2 + rank) * (BM * BN);
         double u1 = 0.0, u2 = 0.0;
         const int64_t rows = p.M - ((int64_t)mt * BMP + rank * BM);          // (rows past the end are not read back)
-        write_out(acc, stg, lane, slab, BN, 1, q * 32, half * EPI_COLS, rows < BM ? rows : BM, BN, false, false, nullptr, nullptr, nullptr,
+        write_out<false>(acc, stg, lane, slab, BN, 1, q * 32, half * EPI_COLS, rows < BM ? rows : BM, BN, false, false, nullptr, nullptr, nullptr,
                   nullptr, 0, u1, u2);
         continue;
       }
       double dot1 = 0.0, dot2 = 0.0;
-      write_out(acc, stg, lane, p.C, p.ldc, p.c_vec, (int64_t)mt * BMP + rank * BM + q * 32, (int64_t)nt * BN + half * EPI_COLS, p.M,
-                p.N, p.accumulate != 0, p.symmetric_lower != 0, p.row_scale, p.col_scale, p.d1, p.d2, p.ldc, dot1, dot2);
-      if (p.part1 || p.part2) {
+      write_out<DOTS>(acc, stg, lane, p.C, p.ldc, p.c_vec, (int64_t)mt * BMP + rank * BM + q * 32, (int64_t)nt * BN + half * EPI_COLS, p.M,
+                      p.N, p.accumulate != 0, p.symmetric_lower != 0, p.row_scale, p.col_scale, p.d1, p.d2, p.ldc, dot1, dot2);
+      if (DOTS) {
         for (int o = 16; o > 0; o >>= 1) {
           dot1 += __shfl_down_sync(0xffffffffu, dot1, o);
           dot2 += __shfl_down_sync(0xffffffffu, dot2, o);
@@ -547,7 +552,7 @@ bool make_map(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64
   return r == CUDA_SUCCESS;
 }
 
-template <int PASSES, bool MN, bool FEW = false>
+template <int PASSES, bool MN, bool FEW = false, bool DOTS = false>
 armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s) {
   CUtensorMap mA, mAlo, mB, mBlo;
   constexpr bool SPLIT = (PASSES == 3 || PASSES == 6);
@@ -564,7 +569,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
   }
   constexpr size_t SMEM = (size_t)Ring<PASSES>::STAGES * Ring<PASSES>::BYTES + 1024 + 8 * EPI_BYTES;
   static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES, MN, FEW>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  if (ensure_dynamic_smem(attr, c->device, tc_gemm_kernel<PASSES, MN, FEW, DOTS>, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int n_pairs = c->n_sm / 2;
   if (n_pairs < 1) return ARMOR_ERR_UNSUPPORTED;
   // Tail split: the tiles of the last, partly filled wave are cut along K so that their pieces fill the wave.  Where the
@@ -611,7 +616,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at; cfg.numAttrs = p.dependent ? 2 : 1;
-    if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN, FEW>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
+    if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN, FEW, DOTS>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
       // 16 rows per CTA; the slots of rows that do not exist are launched only where each has a partial sum to write
       const int64_t rows = p.M < p.tile_m ? p.M : p.tile_m;
@@ -655,10 +660,17 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
   if (p.kt_seg < 1) p.kt_seg = 1;
   p.tile_m = BMP;
   if (n_part) *n_part = PARTS * p.n_tiles_total;
+  const bool dots = g.part1 || g.part2;
   if (g.mn_major) {
     // a map's rows start at multiples of 64 elements; the base and the leading dimension must be multiples of 16 bytes
-    if (!h16 || reinterpret_cast<uintptr_t>(g.A) % 16 || reinterpret_cast<uintptr_t>(g.B) % 16) return ARMOR_ERR_UNSUPPORTED;
+    if (!h16 || dots || reinterpret_cast<uintptr_t>(g.A) % 16 || reinterpret_cast<uintptr_t>(g.B) % 16) return ARMOR_ERR_UNSUPPORTED;
     return g.passes == 6 ? launch_impl<6, true>(c, g, p, s) : launch_impl<0, true>(c, g, p, s);
+  }
+  if (dots) {
+    if (g.passes == 3) return launch_impl<3, false, false, true>(c, g, p, s);
+    if (g.passes == 6) return launch_impl<6, false, false, true>(c, g, p, s);
+    if (g.passes == 1) return launch_impl<1, false, false, true>(c, g, p, s);
+    return ARMOR_ERR_UNSUPPORTED;
   }
   if (g.passes == 3) return launch_impl<3, false>(c, g, p, s);
   if (g.passes == 6) return launch_impl<6, false>(c, g, p, s);
@@ -666,7 +678,7 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
     // Few rows: dealt evenly to one or two tiles.  (The core product of a forward with them, whole pass at 8192 x 8192: 1 token
     // 156 -> 142 us, 300 186 -> 176, 512 198 -> 191; from three tiles on the two forms are alike.)
     const int even = (int)((g.M + p.m_tiles - 1) / p.m_tiles + 31) / 32 * 32;
-    if (p.m_tiles <= 2 && !g.row_scale && !g.accumulate && !g.symmetric_lower && !g.d1 && !g.d2) {
+    if (p.m_tiles <= 2 && !g.row_scale && !g.accumulate && !g.symmetric_lower) {
       p.tile_m = even;
       return launch_impl<0, false, true>(c, g, p, s);
     }
