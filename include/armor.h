@@ -135,10 +135,12 @@ armor_status armor_destroy(armor_ctx* ctx);
  * dimension ldx (elements).  The caller zeroes d_H before the first chunk.
  * x_dtype: ARMOR_DTYPE_F32 or ARMOR_DTYPE_BF16 (bf16 values are exact tensor-core
  * operands, so their Gram needs one pass in every tensor-core precision; not
- * available with ARMOR_PREC_SIMT).  n_rows == 0 is a no-op.  A chunk is worked through in pieces of 16,384 rows
- * (transposed, scaled and split into a staging buffer, then contracted); with ARMOR_PREC_FP16X3 a call of several
- * pieces stages piece p + 1 on a stream of the context's own while piece p is contracted on `stream` (the result does
- * not depend on it; the call returns with all of its work ordered before later work on `stream`, as always). */
+ * available with ARMOR_PREC_SIMT).  n_rows == 0 is a no-op.  A chunk is worked through in pieces of 16,384 rows.
+ * bf16 rows that start on 16-byte boundaries are contracted where they lie; other pieces go through a staging buffer
+ * first (ARMOR_PREC_FP16X3: scaled per channel and split as they lie; tf32 modes: transposed, with ARMOR_PREC_FP32X3
+ * also split).  With ARMOR_PREC_FP16X3 a call of several staged pieces prepares piece p + 1 on a stream of the context's
+ * own while piece p is contracted on `stream` (the result does not depend on it; the call returns with all of its work
+ * ordered before later work on `stream`, as always). */
 armor_status armor_gram(armor_ctx* ctx, const void* d_X, int32_t x_dtype, int64_t n_rows, int64_t ldx,
                         float* d_H, armor_stream_t stream);
 
@@ -286,7 +288,7 @@ enum {
   ARMOR_KC_MASK_SELECT = 7,    /* scoring, selection and mask sweep: one read of Gamma, 4 B / element */
   ARMOR_KC_MASK_GUARD = 8,     /* the other kernels of the sparse-core update (vectors, thin product with H, commit, carry) */
   ARMOR_KC_OPERAND_SPLIT = 9,  /* high / low parts of a dense product's operands: 8 B / element */
-  ARMOR_KC_GRAM_STAGING = 10,  /* channel maxima, transposition and split of a chunk of activations */
+  ARMOR_KC_GRAM_STAGING = 10,  /* staging of a chunk of activations (channel maxima, split; tf32 modes: transposition); channels of a bf16 chunk out of range */
   ARMOR_KC_INIT = 11,          /* normalisation, initial masks and core, input screening */
   ARMOR_KC_SMALL = 12,         /* reductions, bookkeeping, small block products */
   ARMOR_KC_FORWARD = 13,       /* conversions, packing and wrapper products of the deployment form */

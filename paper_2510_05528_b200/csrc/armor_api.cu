@@ -6,7 +6,7 @@
 namespace {
 
 constexpr int LOSS_REFRESH = 64;      // iterations of a call between two evaluations of the loss from the residual
-constexpr int64_t GRAM_ROWS = 16384;  // rows of X staged (transposed, split) per tensor-core Gram pass
+constexpr int64_t GRAM_ROWS = 16384;  // rows of X staged and contracted per tensor-core Gram pass
 
 struct Layout {
   size_t total = 0;

@@ -249,13 +249,13 @@ armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float*
                                    int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
 
 // products and per-block Grams of 256 x 256 blocks on pairs of CTAs (blockpair_tcgen05.cu)
-bool tc_blockpair_ok(const armor_ctx* c, int64_t tiles);   // tiles of 256 x 256 (Grams: pieces of a tile)
+bool tc_blockpair_ok(const armor_ctx* c, int64_t tiles);   // tiles of 256 x 256
 armor_status tc_blockpair_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
                                 int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
 armor_status tc_blockpair_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
                                int64_t cols, float alpha, const float* add, float beta, cudaStream_t s,
                                const float* in2 = nullptr, double* part = nullptr, int* n_part = nullptr);
-armor_status tc_blockpair_gram(armor_ctx* c, const float* P, const float* T, bool by_rows, float* G, int n_split, cudaStream_t s,
+armor_status tc_blockpair_gram(armor_ctx* c, const float* P, const float* T, bool by_rows, float* G, cudaStream_t s,
                                const float* P2 = nullptr, float* G2 = nullptr);
 
 // per-block Grams over a long contraction on the tensor cores

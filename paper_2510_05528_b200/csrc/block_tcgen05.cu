@@ -699,7 +699,8 @@ armor_status gram_launch(armor_ctx* c, const HostOp& A, const HostOp& B, bool by
   p.m_tiles = db / TILE; p.n_tiles = db / TILE; p.batch = nb; p.k_chunks = (int)(chunks / ks); p.n_split = ks;
   p.alpha = 1.f; p.beta = 0.f; p.m_valid = 1 << 30;
   // two W-shaped operands are read once each
-  armor_status st = c->tc_blocks != 1 && tc_blockpair_ok(c, 2 * (int64_t)nb * ks) ? tc_blockpair_gram(c, A.base, B.base, by_rows, p.C, ks, s)
+  // (on pairs of CTAs from 74 blocks on, none of which is then cut: ks == 1)
+  armor_status st = ks == 1 && c->tc_blocks != 1 && tc_blockpair_ok(c, 2 * (int64_t)nb) ? tc_blockpair_gram(c, A.base, B.base, by_rows, p.C, s)
                                                             : launch(c, A, B, p, ARMOR_KC_BLOCK_GRAM, 8.0 * (double)c->wn, s);
   if (st != ARMOR_OK || ks == 1) return st;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
@@ -730,8 +731,8 @@ armor_status gram_pair_launch(armor_ctx* c, const HostOp& A, const HostOp& B, co
   p.alpha = 1.f; p.beta = 0.f; p.m_valid = 1 << 30;
   p.pair = pair;
   // three (pair 1) or two (pair 2) W-shaped operands are read once each
-  armor_status st = pair == 1 && c->tc_blocks != 1 && tc_blockpair_ok(c, 2 * (int64_t)nb * ks)
-                        ? tc_blockpair_gram(c, A.base, B.base, true, p.C, ks, s, A2, C2)
+  armor_status st = pair == 1 && ks == 1 && c->tc_blocks != 1 && tc_blockpair_ok(c, 2 * (int64_t)nb)
+                        ? tc_blockpair_gram(c, A.base, B.base, true, p.C, s, A2, C2)
                         : launch(c, A, B, p, ARMOR_KC_BLOCK_GRAM, (pair == 1 ? 12.0 : 8.0) * (double)c->wn, s, A2, C2);
   if (st != ARMOR_OK || ks == 1) return st;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);

@@ -43,12 +43,11 @@ struct PParams {
   OpCoord a, b;
   const float* D;                   // addend or nullptr
   int64_t c_rows, c_cols;           // extent of C (stores are guarded)
-  int64_t r_b, c_b, r_s;            // tile origin: row = r_b * batch + 256 * tm + r_s * split, column = c_b * batch + 256 * tn
-  int m_tiles, n_tiles, batch, k_chunks, n_split;   // tiles of 256; k_chunks: chunks of 32 per work item
+  int64_t r_b, c_b;                 // tile origin: row = r_b * batch + 256 * tm, column = c_b * batch + 256 * tn
+  int m_tiles, n_tiles, batch, k_chunks;            // tiles of 256; k_chunks: chunks of 32 per work item
   int batch_fastest;                // 1: consecutive work items are consecutive batches (neighbouring column blocks)
   float alpha, beta;
   int32_t* status;
-  int one_pass;                     // 1: operands as they are, no low parts
   int dual;                         // two N-side operands (mapB, mapB2); C = alpha * A.B2, dot_part = <A.B1, A.B2>
   double* dot_part;                 // dual: 16 partial sums per tile (one per epilogue warp of the pair)
   int two;                          // two products with the same N side: C = A.B and, for the odd work items, C2 = A2.B (A2
@@ -67,20 +66,18 @@ __device__ __forceinline__ void load_operand(uint32_t dst, const CUtensorMap* ma
   }
 }
 
-__device__ __forceinline__ void item_decode(const PParams& p, int item, int& tn, int& tm, int& b, int& ks, int& which) {
+__device__ __forceinline__ void item_decode(const PParams& p, int item, int& tn, int& tm, int& b, int& which) {
   which = p.two ? item & 1 : 0;
   if (p.two) item >>= 1;
   if (p.batch_fastest) {
     b = item % p.batch;
     const int rest = item / p.batch;
     tn = rest % p.n_tiles;
-    tm = (rest / p.n_tiles) % p.m_tiles;
-    ks = rest / (p.n_tiles * p.m_tiles);
+    tm = rest / p.n_tiles;
   } else {
     tn = item % p.n_tiles;
     tm = (item / p.n_tiles) % p.m_tiles;
-    b = (item / (p.n_tiles * p.m_tiles)) % p.batch;
-    ks = item / (p.n_tiles * p.m_tiles * p.batch);
+    b = item / (p.n_tiles * p.m_tiles);
   }
 }
 
@@ -117,7 +114,7 @@ tc_blockpair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
   const uint32_t full0 = smem_u32(&bars[0]), split0 = smem_u32(&bars[STAGES]), empty0 = smem_u32(&bars[2 * STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[3 * STAGES]), tempty0 = smem_u32(&bars[3 * STAGES + 2]);
   const uint32_t dfull0 = smem_u32(&bars[3 * STAGES + 4]);
-  const int n_items = p.batch * p.m_tiles * p.n_tiles * p.n_split * (p.two ? 2 : 1);
+  const int n_items = p.batch * p.m_tiles * p.n_tiles * (p.two ? 2 : 1);
   const int n_sub = p.dual ? 2 : 1;
 
   if (threadIdx.x == 0) {
@@ -150,16 +147,16 @@ tc_blockpair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
       int stage = 0; uint32_t phase = 0; long long issued = 0;
       bool ok = true;
       for (int item = pair; item < n_items && ok; item += n_pairs) {
-        int tn, tm, b, ks, which;
-        item_decode(p, item, tn, tm, b, ks, which);
+        int tn, tm, b, which;
+        item_decode(p, item, tn, tm, b, which);
         for (int sub = 0; sub < n_sub && ok; ++sub)
           for (int kc = 0; kc < p.k_chunks; ++kc) {
             if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
             const uint32_t fb = full0 + 8 * stage;
             mbar_expect_tx(fb, 2 * OP_BYTES);
             const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-            load_operand(dst, which ? &mapB2 : &mapA, p.a, b, 2 * tm + rank, ks * p.k_chunks + kc, fb);
-            load_operand(dst + 2 * OP_BYTES, sub ? &mapB2 : &mapB, p.b, b, 2 * tn + rank, ks * p.k_chunks + kc, fb);
+            load_operand(dst, which ? &mapB2 : &mapA, p.a, b, 2 * tm + rank, kc, fb);
+            load_operand(dst + 2 * OP_BYTES, sub ? &mapB2 : &mapB, p.b, b, 2 * tn + rank, kc, fb);
             ++issued;
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
           }
@@ -197,20 +194,14 @@ tc_blockpair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
             const uint64_t da = da0 + so, dal = da + (OP_BYTES >> 4);
             const uint64_t dbm = db0 + so, dbl = dbm + (OP_BYTES >> 4);
             const uint32_t first = (uint32_t)(kc > 0);
-            if (p.one_pass) {
-              umma_pair(tacc, da, dbm, idesc, first);
+            umma_pair(tacc, dal, dbm, idesc, first);
+            umma_pair_acc(tacc, da, dbl, idesc);
+            umma_pair_acc(tacc, da, dbm, idesc);
 #pragma unroll
-              for (int k = 1; k < BK / 8; ++k) umma_pair_acc(tacc, da + k * kinc_a, dbm + k * kinc_b, idesc);
-            } else {
-              umma_pair(tacc, dal, dbm, idesc, first);
-              umma_pair_acc(tacc, da, dbl, idesc);
-              umma_pair_acc(tacc, da, dbm, idesc);
-#pragma unroll
-              for (int k = 1; k < BK / 8; ++k) {
-                umma_pair_acc(tacc, dal + k * kinc_a, dbm + k * kinc_b, idesc);
-                umma_pair_acc(tacc, da + k * kinc_a, dbl + k * kinc_b, idesc);
-                umma_pair_acc(tacc, da + k * kinc_a, dbm + k * kinc_b, idesc);
-              }
+            for (int k = 1; k < BK / 8; ++k) {
+              umma_pair_acc(tacc, dal + k * kinc_a, dbm + k * kinc_b, idesc);
+              umma_pair_acc(tacc, da + k * kinc_a, dbl + k * kinc_b, idesc);
+              umma_pair_acc(tacc, da + k * kinc_a, dbm + k * kinc_b, idesc);
             }
             umma_commit_pair(empty0 + 8 * stage);   // frees the stage in both CTAs once these MMAs have read it
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
@@ -227,22 +218,20 @@ tc_blockpair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
       for (int kc = 0; kc < n_sub * p.k_chunks; ++kc) {
         if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
         float4* base = reinterpret_cast<float4*>(smem + (size_t)stage * STAGE_BYTES);
-        if (!p.one_pass) {
 #pragma unroll
-          for (int op = 0; op < 2; ++op) {
-            float4* hi = base + op * (2 * OP_BYTES / 16);
-            float4* lo = hi + OP_BYTES / 16;
+        for (int op = 0; op < 2; ++op) {
+          float4* hi = base + op * (2 * OP_BYTES / 16);
+          float4* lo = hi + OP_BYTES / 16;
 #pragma unroll
-            for (int e = 0; e < OP_BYTES / 16 / 128; ++e) {
-              const int idx = t + e * 128;
-              const float4 v = hi[idx];
-              float4 h;
-              h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
-              h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
-              h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
-              h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
-              lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
-            }
+          for (int e = 0; e < OP_BYTES / 16 / 128; ++e) {
+            const int idx = t + e * 128;
+            const float4 v = hi[idx];
+            float4 h;
+            h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
+            h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
+            h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
+            h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
+            lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
           }
         }
         // make the generic-proxy writes visible to the tensor-core (async proxy) reads of the pair
@@ -263,10 +252,10 @@ tc_blockpair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
     uint32_t local = 0, d_loads = 0;
     bool ok = true;
     for (int item = pair; item < n_items && ok; item += n_pairs, ++local) {
-      int tn, tm, b, ks, which;
-      item_decode(p, item, tn, tm, b, ks, which);
+      int tn, tm, b, which;
+      item_decode(p, item, tn, tm, b, which);
       const uint32_t as = p.dual ? 0u : (local & 1u), aphase = (p.dual ? local : local >> 1) & 1u;
-      const int64_t row = p.r_b * b + p.r_s * ks + (int64_t)tm * BLK + rank * HALF + q * 32;
+      const int64_t row = p.r_b * b + (int64_t)tm * BLK + rank * HALF + q * 32;
       const int64_t col = p.c_b * b + (int64_t)tn * BLK + half * HALF;
       double dot = 0.0;
       bool got = false;
@@ -381,10 +370,9 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, PParams p, f
   }
   p.a = A.c; p.b = B.c;
   p.status = c->status;
-  p.one_pass = c->block_one_pass;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_blockpair_kernel, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
-  const int n_items = p.batch * p.m_tiles * p.n_tiles * p.n_split * (p.two ? 2 : 1);
+  const int n_items = p.batch * p.m_tiles * p.n_tiles * (p.two ? 2 : 1);
   const int pairs = n_items < c->n_sm / 2 ? n_items : c->n_sm / 2;
   KTimer kt(c, kclass, kbytes, s);
   cudaLaunchConfig_t cfg{};
@@ -421,7 +409,7 @@ armor_status tc_blockpair_right(armor_ctx* c, const float* in, const float* Bblk
   PParams p{};
   p.D = add; p.c_rows = rows; p.c_cols = cols;
   p.c_b = BLK;
-  p.m_tiles = (int)((rows + BLK - 1) / BLK); p.n_tiles = 1; p.batch = nb; p.k_chunks = BLK / BK; p.n_split = 1;
+  p.m_tiles = (int)((rows + BLK - 1) / BLK); p.n_tiles = 1; p.batch = nb; p.k_chunks = BLK / BK;
   p.batch_fastest = 1;
   p.alpha = alpha; p.beta = add ? beta : 0.f;
   return launch(c, A, B, p, out, cols, ARMOR_KC_BLOCK_PRODUCT, (add ? 12.0 : 8.0) * (double)rows * (double)cols, s);
@@ -441,7 +429,7 @@ armor_status tc_blockpair_left(armor_ctx* c, const float* Ablk, bool transA, con
   PParams p{};
   p.D = add; p.c_rows = rows; p.c_cols = cols;
   p.r_b = BLK;
-  p.m_tiles = 1; p.n_tiles = (int)((cols + BLK - 1) / BLK); p.batch = nb; p.k_chunks = BLK / BK; p.n_split = 1;
+  p.m_tiles = 1; p.n_tiles = (int)((cols + BLK - 1) / BLK); p.batch = nb; p.k_chunks = BLK / BK;
   p.alpha = alpha; p.beta = add ? beta : 0.f;
   if (in2) {
     p.dual = 1; p.dot_part = part;
@@ -451,22 +439,19 @@ armor_status tc_blockpair_left(armor_ctx* c, const float* Ablk, bool transA, con
 }
 
 // by_rows: G_i = P_i T_i^T over the row blocks (contraction over d_in); else G_j = P_j^T T_j over the column blocks
-// (contraction over d_out).  The contraction is cut into n_split pieces, piece k to G + k * (number of blocks) * 256 * 256.
-// P2: G2 likewise with P2 in the place of P, in the same launch.
-armor_status tc_blockpair_gram(armor_ctx* c, const float* P, const float* T, bool by_rows, float* G, int n_split, cudaStream_t s,
+// (contraction over d_out).  P2: G2 likewise with P2 in the place of P, in the same launch.
+armor_status tc_blockpair_gram(armor_ctx* c, const float* P, const float* T, bool by_rows, float* G, cudaStream_t s,
                                const float* P2, float* G2) {
   if (!ptr_ok(P) || !ptr_ok(T) || !ptr_ok(G) || (P2 && (!ptr_ok(P2) || !ptr_ok(G2)))) return ARMOR_ERR_UNSUPPORTED;
   const int nb = by_rows ? c->nbo : c->nbi;
-  const int chunks = (int)((by_rows ? c->d_in : c->d_out) / BK);
-  if (chunks % n_split) return ARMOR_ERR_UNSUPPORTED;
   OpCoord o;
   if (by_rows) o = {0, 0, 0, BK, BLK, HALF, 0};         // [m][k] = P[256 i + m][k]: K-major
   else         o = {1, BLK, HALF, 0, 0, 0, BK};         // [m][k] = P[k][256 j + m]: M-major
   HostOp A{P, c->d_in, c->d_out, c->d_in, o}, B{T, c->d_in, c->d_out, c->d_in, o};
   PParams p{};
-  p.c_rows = (int64_t)n_split * nb * BLK; p.c_cols = BLK;
-  p.r_b = BLK; p.r_s = (int64_t)nb * BLK;
-  p.m_tiles = 1; p.n_tiles = 1; p.batch = nb; p.k_chunks = chunks / n_split; p.n_split = n_split;
+  p.c_rows = (int64_t)nb * BLK; p.c_cols = BLK;
+  p.r_b = BLK;
+  p.m_tiles = 1; p.n_tiles = 1; p.batch = nb; p.k_chunks = (int)((by_rows ? c->d_in : c->d_out) / BK);
   p.alpha = 1.f;
   return launch(c, A, B, p, G, BLK, ARMOR_KC_BLOCK_GRAM, (P2 ? 12.0 : 8.0) * (double)c->wn, s, nullptr, P2, G2);
 }

@@ -1,5 +1,5 @@
 // Products with the block-diagonal wrappers (Section 3.1 of the paper) for d_block = 128, with the wrapper block
-// held in TENSOR MEMORY as the M-side operand of tcgen05.mma and 128 x 256 accumulators.
+// held in TENSOR MEMORY as the M-side operand of tcgen05.mma.
 //
 // The streaming kernel of block_tcgen05.cu reads both operands of every MMA from shared memory: 8 KiB per
 // 128 x 128 x 8 instruction, which at the instruction's 65 cycles is the whole shared-memory bandwidth of the SM.
@@ -49,7 +49,6 @@ template <bool DUAL> struct Geo {
   static constexpr int LSTAGES = 4 / CH;          // low-part chunks
   static constexpr int STAGE_BYTES = CH * OP_BYTES;
   static constexpr int PIECES = 4 / CH;           // stages a wrapper block takes
-  static constexpr int N_ACC = DUAL ? 1 : 2;
 };
 constexpr uint32_t TMEM_COLS = 512;               // accumulators 0..255, wrapper high part 256..383, low part 384..511
 constexpr uint32_t W_HI = 256, W_LO = 384;

@@ -277,11 +277,8 @@ armor_status apply_core(armor_ctx* c, const float* z1, const float* S, const voi
     launch_split_hilo(c, z1, nullptr, c->Lo, n * d_in, s);
     launch_split_hilo(c, S, nullptr, c->U, c->wn, s);
     g.A = z1; g.Alo = c->Lo; g.B = S; g.Blo = c->U; g.passes = 3;
-  } else if (core_f16_ok(c)) {
-    core_f16_split_S(c, S, s);
-    return core_f16_product(c, z1, z2, n, s);
   } else if (c->cfg.precision == ARMOR_PREC_FP16X3) {
-    return ARMOR_ERR_UNSUPPORTED;
+    return ARMOR_ERR_UNSUPPORTED;          // (fp32 activations of every shape the mode takes: core_f16_product)
   } else {
     g.A = z1; g.B = S; g.passes = 1;
   }

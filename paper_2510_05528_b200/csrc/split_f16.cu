@@ -158,7 +158,6 @@ __global__ void __launch_bounds__(NT) split_rows_kernel(const float* __restrict_
   }
 }
 
-__device__ __forceinline__ float to_f32(float v) { return v; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
 
 // Four neighbouring elements of a row: one access where every row starts on a boundary of four elements (VEC)
