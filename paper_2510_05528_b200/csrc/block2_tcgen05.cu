@@ -127,6 +127,7 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -415,7 +416,7 @@ armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const fl
   const int grid = n_items < c->n_sm ? n_items : c->n_sm;
   // one W-shaped read, one W-shaped write
   KTimer kt(c, ARMOR_KC_BLOCK_PRODUCT, 8.0 * (double)rows * (double)cols, s);
-  tc_block2_kernel<<<grid, NTHREADS, SMEM_BYTES, s>>>(mL, mX, mR, mC, p);
+  launch_dependent(tc_block2_kernel, grid, NTHREADS, SMEM_BYTES, s, mL, mX, mR, mC, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }

@@ -152,6 +152,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -543,8 +544,8 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, i
   const int n_items = p.batch * p.m_tiles * p.n_tiles * p.n_split;
   const int grid = n_items < n_sm ? n_items : n_sm;
   KTimer kt(c, kclass, kbytes, s);
-  if (p.pair == 1) tc_block_kernel<3><<<grid, NTHREADS, smem_bytes<3>(), s>>>(mA, mB, mB2, mC, mD, p);
-  else tc_block_kernel<2><<<grid, NTHREADS, smem_bytes<2>(), s>>>(mA, mB, mB2, mC, mD, p);
+  if (p.pair == 1) launch_dependent(tc_block_kernel<3>, grid, NTHREADS, smem_bytes<3>(), s, mA, mB, mB2, mC, mD, p);
+  else launch_dependent(tc_block_kernel<2>, grid, NTHREADS, smem_bytes<2>(), s, mA, mB, mB2, mC, mD, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
@@ -662,8 +663,9 @@ armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* i
 namespace {
 
 // out[e] = sum over the slabs, in slab order; blockIdx.y 1: the same for the second Gram of a pair, n_slab slabs further on
-__global__ void __launch_bounds__(256) sum_slabs_kernel(const float4* __restrict__ part, int64_t n4, int n_slab,
+__global__ void __launch_bounds__(256) sum_slabs_kernel(const float4* part, int64_t n4, int n_slab,
                                                         float4* __restrict__ out0, float4* __restrict__ out1) {
+  grid_begin();
   const float4* p = part + (int64_t)blockIdx.y * n_slab * n4;
   float4* out = blockIdx.y ? out1 : out0;
   for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n4; i += (int64_t)gridDim.x * 256) {
@@ -706,7 +708,7 @@ armor_status gram_launch(armor_ctx* c, const HostOp& A, const HostOp& B, bool by
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
   int64_t blocks = (slab / 4 + 255) / 256;
   if (blocks > 148 * 8) blocks = 148 * 8;
-  sum_slabs_kernel<<<(unsigned)blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
+  launch_dependent(sum_slabs_kernel, (unsigned)blocks, 256, 0, s, reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
                                                    reinterpret_cast<float4*>(G), nullptr);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
@@ -738,7 +740,7 @@ armor_status gram_pair_launch(armor_ctx* c, const HostOp& A, const HostOp& B, co
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
   int64_t blocks = (slab / 4 + 255) / 256;
   if (blocks > 148 * 8) blocks = 148 * 8;
-  sum_slabs_kernel<<<dim3((unsigned)blocks, 2), 256, 0, s>>>(reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
+  launch_dependent(sum_slabs_kernel, dim3((unsigned)blocks, 2), 256, 0, s, reinterpret_cast<const float4*>(c->gpart), slab / 4, ks,
                                                             reinterpret_cast<float4*>(G), reinterpret_cast<float4*>(G2));
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;

@@ -138,6 +138,7 @@ tc_blockpair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_const
   __syncthreads();
   cluster_sync_all();                               // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
+  grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -377,10 +378,12 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, PParams p, f
   KTimer kt(c, kclass, kbytes, s);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = s;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = 2;
   if (cudaLaunchKernelEx(&cfg, tc_blockpair_kernel, mA, mB, mB2, mC, mD, p) != cudaSuccess) return ARMOR_ERR_CUDA;
   c->launches++;
   return ARMOR_OK;

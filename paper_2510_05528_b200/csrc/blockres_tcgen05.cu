@@ -140,6 +140,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -595,7 +596,7 @@ armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, 
   const int64_t n_items = (int64_t)p.batch * p.tiles;
   const int grid = (int)(n_items < c->n_sm ? n_items : c->n_sm);
   KTimer kt(c, ARMOR_KC_BLOCK_PRODUCT, ((p.D || X2) ? 12.0 : 8.0) * (double)rows * (double)cols, s);
-  tc_blockres_kernel<DUAL><<<grid, NTHREADS, SMEM_BYTES, s>>>(mX, mX2, mQ, mC, mD, p);
+  launch_dependent(tc_blockres_kernel<DUAL>, grid, NTHREADS, SMEM_BYTES, s, mX, mX2, mQ, mC, mD, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }

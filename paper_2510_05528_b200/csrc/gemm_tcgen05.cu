@@ -279,7 +279,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   __syncthreads();
   cluster_sync_all();                                  // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
-  if (PASSES == 0 && !MN) grid_launch_dependents();    // (the kernel that adds the pieces of cut tiles, see launch_impl)
+  // (tensor memory is this CTA's before the next kernel's CTAs start; a Gram's product waits where its scales are read)
+  if (!MN) grid_begin();
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -485,7 +486,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
 constexpr int FIX_NT = BMP / PARTS * BN / 4;
 __global__ void __launch_bounds__(FIX_NT) tc_gemm_fixup_kernel(const Params p) {
   constexpr int FR = BMP / PARTS;                         // rows per CTA
-  grid_dependency_wait();                                 // (where it is launched beside the product's tail)
+  grid_begin();
   const int slots = gridDim.x / (p.n_tiles_total - p.split_first);       // PARTS, or those that hold rows
   const int tile = p.split_first + blockIdx.x / slots, slot = blockIdx.x % slots;
   int mt, nt;
@@ -622,7 +623,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
     at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
     at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at; cfg.numAttrs = p.dependent ? 2 : 1;
+    cfg.attrs = at; cfg.numAttrs = !MN || p.dependent ? 2 : 1;
     if (cudaLaunchKernelEx(&cfg, tc_gemm_kernel<PASSES, MN, FEW, DOTS>, mA, mAlo, mB, mBlo, p) != cudaSuccess) return ARMOR_ERR_CUDA;
     if (p.split_parts > 1) {
       // 16 rows per CTA; the slots of rows that do not exist are launched only where each has a partial sum to write
@@ -630,8 +631,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
       const int slots = (p.part1 || p.part2) ? PARTS : (int)((rows + BMP / PARTS - 1) / (BMP / PARTS));
       cudaLaunchConfig_t fc{};
       fc.gridDim = dim3(slots * (p.n_tiles_total - p.split_first)); fc.blockDim = dim3(FIX_NT); fc.stream = s;
-      // behind the bf16 product it is a dependent launch: with a handful of tokens its launch counts
-      fc.attrs = &at[1]; fc.numAttrs = PASSES == 0 && !MN ? 1 : 0;
+      fc.attrs = &at[1]; fc.numAttrs = MN ? 0 : 1;
       if (cudaLaunchKernelEx(&fc, tc_gemm_fixup_kernel, p) != cudaSuccess) return ARMOR_ERR_CUDA;
       c->launches++;
     }

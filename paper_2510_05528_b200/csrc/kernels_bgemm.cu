@@ -28,14 +28,15 @@ __device__ __forceinline__ void batch_offsets(const BGemm& g, int b, int64_t& oa
 }
 
 __global__ void __launch_bounds__(NT) bgemm_kernel(BGemm g) {
+  grid_begin();
   __shared__ float As[BK][BM + 4];
   __shared__ float Bs[BK][BN + 4];
   const int b = blockIdx.z;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   int64_t oa, ob, oc, od;
   batch_offsets(g, b, oa, ob, oc, od);
-  const float* __restrict__ A = g.A + oa;
-  const float* __restrict__ B = g.B + ob;
+  const float* A = g.A + oa;
+  const float* B = g.B + ob;
   const int tid = threadIdx.x;
   const int tx = tid % 16, ty = tid / 16;
   // which index runs fastest over consecutive threads when a tile is fetched: the unit-stride one
@@ -106,6 +107,7 @@ constexpr int FM = 128, FN = 128, FK = 16, FLD = FM + 4;
 // strides and all batch strides multiples of 4, 16-byte aligned bases, sCn == sDn == 1.
 template <bool A_KFAST, bool B_NFAST>
 __global__ void __launch_bounds__(NT, 2) bgemm_tile_kernel(BGemm g, float* __restrict__ part_out, int64_t part_stride) {
+  grid_begin();
   __shared__ __align__(16) float As[2][FK][FLD];
   __shared__ __align__(16) float Bs[2][FK][FLD];
   const int ksplit = g.ksplit > 1 ? g.ksplit : 1;
@@ -114,8 +116,8 @@ __global__ void __launch_bounds__(NT, 2) bgemm_tile_kernel(BGemm g, float* __res
   int64_t oa, ob, oc, od;
   batch_offsets(g, b, oa, ob, oc, od);
   const int kc = g.K / ksplit;
-  const float* __restrict__ A = g.A + oa + (int64_t)ks * kc * g.sAk;
-  const float* __restrict__ B = g.B + ob + (int64_t)ks * kc * g.sBk;
+  const float* A = g.A + oa + (int64_t)ks * kc * g.sAk;
+  const float* B = g.B + ob + (int64_t)ks * kc * g.sBk;
   const int tid = threadIdx.x;
   const int tx = tid % 16, ty = tid / 16;
 
@@ -242,13 +244,14 @@ __device__ __forceinline__ int sm_unit(int k, int u) { return k * SM_T + 4 * (u 
 
 template <bool A_KFAST, bool B_NFAST>
 __global__ void __launch_bounds__(NT) bgemm_small_kernel(BGemm g) {
+  grid_begin();
   __shared__ __align__(16) float As[SM_K * SM_T];
   __shared__ __align__(16) float Bs[SM_K * SM_T];
   const int m0 = blockIdx.y * SM_T, n0 = blockIdx.x * SM_T;
   int64_t oa, ob, oc, od;
   batch_offsets(g, blockIdx.z, oa, ob, oc, od);
-  const float* __restrict__ A = g.A + oa;
-  const float* __restrict__ B = g.B + ob;
+  const float* A = g.A + oa;
+  const float* B = g.B + ob;
   const int tid = threadIdx.x;
   float4 ra[4], rb[4];
   // 32 x 128 floats of either operand: four float4 per thread, along whichever index is contiguous
@@ -345,8 +348,9 @@ inline bool small_tiles_better(const BGemm& g) {
 }
 
 // out[b][m][n] = alpha * sum_ks part[ks][b][m][n]  (fixed order), scattered to the strided destination
-__global__ void __launch_bounds__(NT) bgemm_splitsum_kernel(BGemm g, const float* __restrict__ part,
+__global__ void __launch_bounds__(NT) bgemm_splitsum_kernel(BGemm g, const float* part,
                                                             int64_t part_stride) {
+  grid_begin();
   const int64_t per = (int64_t)g.M * g.N;
   const int64_t n4 = (int64_t)g.batch * per / 4;
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) {
@@ -394,10 +398,10 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
   if (g.ksplit > 1 && !tile_kernel_ok(g, a_kfast, b_nfast)) g.ksplit = 1;
   if (tile_kernel_ok(g, a_kfast, b_nfast) && small_tiles_better(g)) {
     dim3 grid((g.N + SM_T - 1) / SM_T, (g.M + SM_T - 1) / SM_T, g.batch);
-    if (a_kfast && b_nfast) bgemm_small_kernel<true, true><<<grid, NT, 0, s>>>(g);
-    else if (a_kfast && !b_nfast) bgemm_small_kernel<true, false><<<grid, NT, 0, s>>>(g);
-    else if (!a_kfast && b_nfast) bgemm_small_kernel<false, true><<<grid, NT, 0, s>>>(g);
-    else bgemm_small_kernel<false, false><<<grid, NT, 0, s>>>(g);
+    if (a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<true, true>, grid, NT, 0, s, g);
+    else if (a_kfast && !b_nfast) launch_dependent(bgemm_small_kernel<true, false>, grid, NT, 0, s, g);
+    else if (!a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<false, true>, grid, NT, 0, s, g);
+    else launch_dependent(bgemm_small_kernel<false, false>, grid, NT, 0, s, g);
     c->launches++;
     return;
   }
@@ -405,22 +409,22 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
     const int ks = g.ksplit > 1 ? g.ksplit : 1;
     dim3 grid((g.N + FN - 1) / FN, (g.M + FM - 1) / FM, g.batch * ks);
     const int64_t pstride = (int64_t)g.batch * g.M * g.N;
-    if (a_kfast && b_nfast) bgemm_tile_kernel<true, true><<<grid, NT, 0, s>>>(g, c->gpart, pstride);
-    else if (a_kfast && !b_nfast) bgemm_tile_kernel<true, false><<<grid, NT, 0, s>>>(g, c->gpart, pstride);
-    else if (!a_kfast && b_nfast) bgemm_tile_kernel<false, true><<<grid, NT, 0, s>>>(g, c->gpart, pstride);
-    else bgemm_tile_kernel<false, false><<<grid, NT, 0, s>>>(g, c->gpart, pstride);
+    if (a_kfast && b_nfast) launch_dependent(bgemm_tile_kernel<true, true>, grid, NT, 0, s, g, c->gpart, pstride);
+    else if (a_kfast && !b_nfast) launch_dependent(bgemm_tile_kernel<true, false>, grid, NT, 0, s, g, c->gpart, pstride);
+    else if (!a_kfast && b_nfast) launch_dependent(bgemm_tile_kernel<false, true>, grid, NT, 0, s, g, c->gpart, pstride);
+    else launch_dependent(bgemm_tile_kernel<false, false>, grid, NT, 0, s, g, c->gpart, pstride);
     c->launches++;
     if (ks > 1) {
       const int64_t n4 = pstride / 4;
       int64_t blocks = (n4 + NT - 1) / NT;
       if (blocks > 148 * 8) blocks = 148 * 8;
-      bgemm_splitsum_kernel<<<(unsigned)blocks, NT, 0, s>>>(g, c->gpart, pstride);
+      launch_dependent(bgemm_splitsum_kernel, (unsigned)blocks, NT, 0, s, g, c->gpart, pstride);
       c->launches++;
     }
     return;
   }
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-  bgemm_kernel<<<grid, NT, 0, s>>>(g);
+  launch_dependent(bgemm_kernel, grid, NT, 0, s, g);
   c->launches++;
 }
 

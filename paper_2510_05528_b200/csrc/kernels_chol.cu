@@ -276,9 +276,10 @@ constexpr int MAX_DB = 256;
 // G: a CTA takes 32 G right-hand sides
 template <int G>
 __global__ void __launch_bounds__(NT, 1)
-chol_blocked_kernel(int mode, const float* __restrict__ Gmat, const float* __restrict__ rhs, float* __restrict__ out,
-                    const float* __restrict__ dotw, float* __restrict__ A, float ridge, int db, double* __restrict__ part,
+chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __restrict__ out,
+                    const float* dotw, float* __restrict__ A, float ridge, int db, double* __restrict__ part,
                     int32_t* __restrict__ failflag, int32_t* __restrict__ status) {
+  grid_begin();
   constexpr int W = 32 * G, LDX = W + 1;                // (odd: neither a row of X nor 8 x 4 floats along a column conflict)
   extern __shared__ __align__(16) float smem[];
   const PanelMap pm{db};
@@ -402,10 +403,11 @@ chol_blocked_kernel(int mode, const float* __restrict__ Gmat, const float* __res
 }
 
 // Unblocked variant for block sizes that are not a multiple of 32: thread i owns row i.
-__global__ void chol_kernel(int mode, const float* __restrict__ Gmat, const float* __restrict__ rhs,
-                            float* __restrict__ out, const float* __restrict__ dotw, float* __restrict__ A,
+__global__ void chol_kernel(int mode, const float* Gmat, const float* rhs,
+                            float* __restrict__ out, const float* dotw, float* __restrict__ A,
                             float ridge, int db, double* __restrict__ part,
                             int32_t* __restrict__ failflag, int32_t* __restrict__ status) {
+  grid_begin();
   extern __shared__ float smem[];
   const int ld = db + 1;
   float* L = smem;
@@ -522,7 +524,7 @@ armor_status launch_blocked(armor_ctx* c, int mode, const float* Gm, const float
   if (ensure_dynamic_smem(attr, c->device, chol_blocked_kernel<G>,
                           (panel_floats(widest) + (size_t)widest * (32 * G + 1)) * sizeof(float)) != ARMOR_OK)
     return ARMOR_ERR_CUDA;
-  chol_blocked_kernel<G><<<dim3(nb, (db + 32 * G - 1) / (32 * G)), NT, smem, s>>>(mode, Gm, rhs, out, dotw, A, c->cfg.ridge, db,
+  launch_dependent(chol_blocked_kernel<G>, dim3(nb, (db + 32 * G - 1) / (32 * G)), NT, smem, s, mode, Gm, rhs, out, dotw, A, c->cfg.ridge, db,
                                                                                   part, c->failflag, c->status);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
@@ -551,7 +553,7 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
   static PerDeviceOnce attr_set;
   if (ensure_dynamic_smem(attr_set, c->device, chol_kernel, 2 * 128 * 129 * 4) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int nt = ((db + 31) / 32) * 32;
-  chol_kernel<<<nb, nt < 64 ? 64 : nt, smem, s>>>(mode, Gmat, rhs, out, dotw, A, c->cfg.ridge, db, part,
+  launch_dependent(chol_kernel, nb, nt < 64 ? 64 : nt, smem, s, mode, Gmat, rhs, out, dotw, A, c->cfg.ridge, db, part,
                                                  c->failflag, c->status);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
@@ -560,21 +562,24 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
 namespace {
 
 __global__ void identity_rhs_kernel(float* __restrict__ X, int db) {
+  grid_begin();
   float* Xb = X + (int64_t)blockIdx.x * db * db;
   for (int e = threadIdx.x; e < db * db; e += blockDim.x) Xb[e] = (e / db == e % db) ? 1.f : 0.f;
 }
 
-__global__ void save_flags_kernel(const int32_t* __restrict__ failflag, int32_t* __restrict__ saved, int n) {
+__global__ void save_flags_kernel(const int32_t* failflag, int32_t* __restrict__ saved, int n) {
+  grid_begin();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) saved[i] = failflag[i];
 }
 
 // DELTA_PARTS CTAs per block: Delta_j = 0 and failflag[j] = 1 where the inverse does not exist; partial sums of
 // <dotw_j, Delta_j>
-__global__ void __launch_bounds__(NT) delta_finish_kernel(float* __restrict__ Delta, const float* __restrict__ dotw,
-                                                          const int32_t* __restrict__ hinv_fail,
+__global__ void __launch_bounds__(NT) delta_finish_kernel(float* __restrict__ Delta, const float* dotw,
+                                                          const int32_t* hinv_fail,
                                                           int32_t* __restrict__ failflag, double* __restrict__ part,
                                                           int db) {
+  grid_begin();
   const int j = blockIdx.x / DELTA_PARTS, q = blockIdx.x % DELTA_PARTS;
   const int64_t off = (int64_t)j * db * db;
   const int n4 = db * db / 4, e1 = n4 * (q + 1) / DELTA_PARTS;
@@ -606,20 +611,20 @@ armor_status launch_hjj_inverse(armor_ctx* c, cudaStream_t s) {
   if (cudaMemsetAsync(c->failflag, 0, (size_t)nbi * sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
   {
     KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-    identity_rhs_kernel<<<nbi, NT, 0, s>>>(c->Ktmp, c->db);
+    launch_dependent(identity_rhs_kernel, nbi, NT, 0, s, c->Ktmp, c->db);
     c->launches++;
   }
   armor_status st = launch_chol(c, 1, c->Hjj, c->Ktmp, c->Hinv, nullptr, nullptr, nbi, nullptr, s);
   if (st != ARMOR_OK) return st;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  save_flags_kernel<<<(nbi + 255) / 256, 256, 0, s>>>(c->failflag, c->hinv_fail, nbi);
+  launch_dependent(save_flags_kernel, (nbi + 255) / 256, 256, 0, s, c->failflag, c->hinv_fail, nbi);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
 
 void launch_delta_finish(armor_ctx* c, float* Delta, const float* dotw, double* part, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  delta_finish_kernel<<<DELTA_PARTS * c->nbi, NT, 0, s>>>(Delta, dotw, c->hinv_fail, c->failflag, part, c->db);
+  launch_dependent(delta_finish_kernel, DELTA_PARTS * c->nbi, NT, 0, s, Delta, dotw, c->hinv_fail, c->failflag, part, c->db);
   c->launches++;
 }
 

@@ -25,7 +25,8 @@ __device__ __forceinline__ float neg_log_uniform(uint32_t k24) {
 
 // alpha[r] = || A[:, r] ||^2 : column r of the block that owns row r of the core.
 // blockDim = (32 columns, 8 row slices); grid = (nbo, db / 32).
-__global__ void alpha_kernel(const float* __restrict__ A, float* __restrict__ alpha, int db) {
+__global__ void alpha_kernel(const float* A, float* __restrict__ alpha, int db) {
+  grid_begin();
   const int i = blockIdx.x;
   const int r = blockIdx.y * 32 + threadIdx.x;
   const float* Ai = A + (int64_t)i * db * db;
@@ -121,15 +122,16 @@ __device__ __forceinline__ bool chol_small(int n, const double (&Kin)[NKM][NKM],
 // side by side: PHASE 1 is pass 1 alone (the block's winner goes to best_key / best_g), PHASE 2 is pass 2
 // alone (one warp per block for groups of four, 256 threads for groups of eight).
 template <int MG, int NKM, bool MULTI, int PHASE>
-__global__ void __launch_bounds__(NT) mask_select_kernel(const float* __restrict__ Gam, const float* __restrict__ S,
-                                                         const uint8_t* __restrict__ M, const float* __restrict__ alpha,
-                                                         const float* __restrict__ Kfull, SelRec* __restrict__ sel,
+__global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const float* S,
+                                                         const uint8_t* M, const float* alpha,
+                                                         const float* Kfull, SelRec* __restrict__ sel,
                                                          double* __restrict__ part, int64_t d_in, int db, int nbi,
                                                          int n_keep, int select_mode, uint64_t seed, uint64_t t_base,
-                                                         uint64_t t_mul, const int64_t* __restrict__ it_dev,
+                                                         uint64_t t_mul, const int64_t* it_dev,
                                                          uint64_t n_groups_total, int kg_arg,
                                                          float* __restrict__ tab_key,
                                                          unsigned long long* __restrict__ tab_g) {
+  grid_begin();
   const uint64_t t = t_base + t_mul * (uint64_t)(*it_dev);   // selection counter of this run of Algorithm 3
   const int kg = MULTI ? kg_arg : 1;                       // one draw: the loop and the key cache compile away
   const int bi = blockIdx.x / nbi, bj = blockIdx.x % nbi;
@@ -406,10 +408,11 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* __restrict
 // with a_ij = A_i[:, r_ij] and z_ij = delta_ij^T B_j[rows of the group, :]: row-blocks decouple because A is
 // block diagonal.  mask_vectors_kernel gathers a and z, a batched product forms y_ij = z_ij H_w[j-th block
 // row, :], and mask_quad_kernel sums the pairs in a fixed order.
-__global__ void __launch_bounds__(NT) mask_vectors_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                          const SelRec* __restrict__ sel, float* __restrict__ Zsel,
+__global__ void __launch_bounds__(NT) mask_vectors_kernel(const float* A, const float* B,
+                                                          const SelRec* sel, float* __restrict__ Zsel,
                                                           float* __restrict__ Acol, int db, int nbo_pad, int nbi, int mg,
                                                           int nbv) {
+  grid_begin();
   const int blk = blockIdx.x;                  // (row block, virtual column block v = draw * nbi + column block)
   const int bi = blk / nbv, v = blk % nbv, bj = v % nbi;
   const SelRec rec = sel[blk];
@@ -429,10 +432,11 @@ __global__ void __launch_bounds__(NT) mask_vectors_kernel(const float* __restric
 
 // One CTA per block (i, j), one warp per pair (j, j') at a time.  Y == nullptr: diagonal weighting, only the
 // j == j' pair contributes and y = z (.) hdiag.
-__global__ void __launch_bounds__(NT) mask_quad_kernel(const float* __restrict__ Zsel, const float* __restrict__ Acol,
-                                                       const float* __restrict__ Y, const float* __restrict__ hdiag,
+__global__ void __launch_bounds__(NT) mask_quad_kernel(const float* Zsel, const float* Acol,
+                                                       const float* Y, const float* hdiag,
                                                        double* __restrict__ part, int64_t d_in, int db, int nbo_pad,
                                                        int nbi, int nbv) {
+  grid_begin();
   const int bi = blockIdx.x / nbv, j = blockIdx.x % nbv;      // j, j2: virtual column blocks (draw * nbi + column block)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = NT / 32;
   double acc = 0.0;
@@ -466,9 +470,10 @@ __global__ void __launch_bounds__(NT) mask_quad_kernel(const float* __restrict__
   }
 }
 
-__global__ void mask_commit_kernel(const SelRec* __restrict__ sel, int nblocks, float* __restrict__ S,
-                                   uint8_t* __restrict__ M, int64_t d_in, int mg, const double* __restrict__ sc,
-                                   armor_iter_stats* st_base, const int64_t* __restrict__ it_dev) {
+__global__ void mask_commit_kernel(const SelRec* sel, int nblocks, float* __restrict__ S,
+                                   uint8_t* __restrict__ M, int64_t d_in, int mg, const double* sc,
+                                   armor_iter_stats* st_base, const int64_t* it_dev) {
+  grid_begin();
   armor_iter_stats* st = st_base ? st_base + *it_dev : nullptr;
   __shared__ int changed;
   if (threadIdx.x == 0) changed = 0;
@@ -503,9 +508,10 @@ constexpr int CARRY_PICKS = 4;
 constexpr int CARRY_CTAS = 64;
 constexpr int CARRY_TAB = 2048;                            // picks whose rows are kept in shared memory
 __device__ __forceinline__ int carry_row(const SelRec& rec, int row0) { return rec.valid ? rec.row - row0 : -1; }
-__global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* __restrict__ sel, const float* __restrict__ Y,
-                                                        float* __restrict__ P, const double* __restrict__ sc,
+__global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* sel, const float* Y,
+                                                        float* __restrict__ P, const double* sc,
                                                         int64_t d_in, int db, int nbo_pad, int nbv) {
+  grid_begin();
   __shared__ int row_of[CARRY_TAB];                        // row inside the block, -1: no group
   __shared__ int first[256], last[256];                    // picks of a row
   if (sc[SC_ACCEPT] == 0.0) return;
@@ -557,14 +563,14 @@ void launch_mask_carry_P(armor_ctx* c, float* P, cudaStream_t s) {
   const int nbv = c->nbi * c->kg;
   int groups = (nbv + CARRY_PICKS - 1) / CARRY_PICKS;
   if (groups > CARRY_CTAS) groups = CARRY_CTAS;
-  mask_carry_kernel<<<dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s>>>(
+  launch_dependent(mask_carry_kernel, dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s, 
       c->sel, c->Ysel, P, c->sc, c->d_in, c->db, c->nbo_pad, nbv);
   c->launches++;
 }
 
 void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  alpha_kernel<<<dim3(c->nbo, (c->db + 31) / 32), dim3(32, 8), 0, s>>>(A, c->alpha, c->db);
+  launch_dependent(alpha_kernel, dim3(c->nbo, (c->db + 31) / 32), dim3(32, 8), 0, s, A, c->alpha, c->db);
   c->launches++;
 }
 
@@ -573,9 +579,10 @@ void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s) {
 // Y = B_j H_jj comes from a block product.  CTAs [0, n_kc): one warp per group, lane l takes columns l, l + 32, ..;
 // the remaining CTAs compute alpha.
 template <int MG>
-__global__ void __launch_bounds__(NT) mask_prep_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                       const float* __restrict__ Y, float* __restrict__ Kfull,
+__global__ void __launch_bounds__(NT) mask_prep_kernel(const float* A, const float* B,
+                                                       const float* Y, float* __restrict__ Kfull,
                                                        float* __restrict__ alpha, int db, int nbi, int n_kc) {
+  grid_begin();
   if ((int)blockIdx.x < n_kc) {
     const int gpb = db / MG;
     const int wg = blockIdx.x * (NT / 32) + (threadIdx.x >> 5);       // (column block, group)
@@ -636,8 +643,8 @@ void launch_mask_prep(armor_ctx* c, const float* A, const float* B, const float*
   const int n_kc = (c->nbi * (db / mg) + NT / 32 - 1) / (NT / 32);
   const int n_al = c->nbo * ((db + 31) / 32);
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  if (mg == 8) mask_prep_kernel<8><<<n_kc + n_al, NT, 0, s>>>(A, B, Y, c->Kfull, c->alpha, db, c->nbi, n_kc);
-  else mask_prep_kernel<4><<<n_kc + n_al, NT, 0, s>>>(A, B, Y, c->Kfull, c->alpha, db, c->nbi, n_kc);
+  if (mg == 8) launch_dependent(mask_prep_kernel<8>, n_kc + n_al, NT, 0, s, A, B, Y, c->Kfull, c->alpha, db, c->nbi, n_kc);
+  else launch_dependent(mask_prep_kernel<4>, n_kc + n_al, NT, 0, s, A, B, Y, c->Kfull, c->alpha, db, c->nbi, n_kc);
   c->launches++;
 }
 
@@ -655,10 +662,10 @@ void launch_mask_select(armor_ctx* c, const float* Gam, const float* S, const ui
       if (smem > 48 * 1024)                                                                                             \
         cudaFuncSetAttribute(mask_select_kernel<MGV, NKV, MULTIV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                              (int)smem);                                                                                \
-      mask_select_kernel<MGV, NKV, MULTIV, 0><<<c->nbo * c->nbi, NT, smem, s>>>(ARMOR_SELECT_ARGS);                     \
+      launch_dependent(mask_select_kernel<MGV, NKV, MULTIV, 0>, c->nbo * c->nbi, NT, smem, s, ARMOR_SELECT_ARGS);                     \
     } else {                                                                                                            \
-      mask_select_kernel<MGV, NKV, false, 1><<<c->nbo * c->nbi, NT, 0, s>>>(ARMOR_SELECT_ARGS);                         \
-      mask_select_kernel<MGV, NKV, false, 2><<<c->nbo * c->nbi, MGV == 4 ? 32 : NT, 0, s>>>(ARMOR_SELECT_ARGS);         \
+      launch_dependent(mask_select_kernel<MGV, NKV, false, 1>, c->nbo * c->nbi, NT, 0, s, ARMOR_SELECT_ARGS);                         \
+      launch_dependent(mask_select_kernel<MGV, NKV, false, 2>, c->nbo * c->nbi, MGV == 4 ? 32 : NT, 0, s, ARMOR_SELECT_ARGS);         \
       c->launches++;                                                                                                    \
     }                                                                                                                   \
   } while (0)
@@ -676,7 +683,7 @@ void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const f
   const int db = c->db, nbo = c->nbo, nbi = c->nbi, nbo_pad = c->nbo_pad, kg = c->kg, nbv = nbi * kg;
   {
     KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-    mask_vectors_kernel<<<nbo * nbv, NT, 0, s>>>(A, B, c->sel, c->Zsel, c->Acol, db, nbo_pad, nbi, c->cfg.m_group, nbv);
+    launch_dependent(mask_vectors_kernel, nbo * nbv, NT, 0, s, A, B, c->sel, c->Zsel, c->Acol, db, nbo_pad, nbi, c->cfg.m_group, nbv);
   }
   c->launches++;
   const float* Y = nullptr;
@@ -699,7 +706,7 @@ void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const f
   double* part = c->quadpart;
   {
     KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-    mask_quad_kernel<<<nbo * nbv, NT, 0, s>>>(c->Zsel, c->Acol, Y, c->hdiag, part, c->d_in, db, nbo_pad, nbi, nbv);
+    launch_dependent(mask_quad_kernel, nbo * nbv, NT, 0, s, c->Zsel, c->Acol, Y, c->hdiag, part, c->d_in, db, nbo_pad, nbi, nbv);
   }
   c->launches++;
   // (the caller's stage kernel adds the nbo * nbv terms up into sc[SC_Q_M])
@@ -707,7 +714,7 @@ void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const f
 
 void launch_mask_commit(armor_ctx* c, float* S, uint8_t* M, armor_iter_stats* st, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  mask_commit_kernel<<<1, 256, 0, s>>>(c->sel, c->nbo * c->nbi * c->kg, S, M, c->d_in, c->cfg.m_group, c->sc, st,
+  launch_dependent(mask_commit_kernel, 1, 256, 0, s, c->sel, c->nbo * c->nbi * c->kg, S, M, c->d_in, c->cfg.m_group, c->sc, st,
                                        c->it_dev);
   c->launches++;
 }

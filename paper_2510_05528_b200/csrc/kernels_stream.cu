@@ -23,9 +23,10 @@ __device__ __forceinline__ double block_reduce_sum(double v) {
 }
 
 // ---- deterministic two-stage dot product: fixed grid, fixed order --------------------------------
-__global__ void __launch_bounds__(NT) dot_partial_kernel(const float4* __restrict__ x,
-                                                         const float4* __restrict__ y, int64_t n4,
+__global__ void __launch_bounds__(NT) dot_partial_kernel(const float4* x,
+                                                         const float4* y, int64_t n4,
                                                          double* __restrict__ part) {
+  grid_begin();
   double acc = 0.0;
   const int64_t stride = (int64_t)gridDim.x * NT;
   // four independent pairs of loads in flight per thread; the order of the additions is fixed by the grid
@@ -50,8 +51,9 @@ __global__ void __launch_bounds__(NT) dot_partial_kernel(const float4* __restric
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
-__global__ void __launch_bounds__(NT) reduce_final_kernel(const double* __restrict__ part, int n,
+__global__ void __launch_bounds__(NT) reduce_final_kernel(const double* part, int n,
                                                           double* __restrict__ out) {
+  grid_begin();
   double acc = 0.0;
   for (int i = threadIdx.x; i < n; i += NT) acc += part[i];
   acc = block_reduce_sum(acc);
@@ -59,17 +61,19 @@ __global__ void __launch_bounds__(NT) reduce_final_kernel(const double* __restri
 }
 
 // ---- column scale: out = in * diag(h) -----------------------------------------------------------
-__global__ void __launch_bounds__(NT) colscale_kernel(const float4* __restrict__ in, const float4* __restrict__ h,
+__global__ void __launch_bounds__(NT) colscale_kernel(const float4* in, const float4* h,
                                                       float4* __restrict__ out, int64_t n4, int cols4) {
+  grid_begin();
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) {
     float4 a = in[i], s = h[i % cols4];
     out[i] = make_float4(a.x * s.x, a.y * s.y, a.z * s.z, a.w * s.w);
   }
 }
 
-__global__ void __launch_bounds__(NT) rowcolscale_kernel(const float* __restrict__ in, const float* __restrict__ cs,
-                                                         const float* __restrict__ rs, float* __restrict__ out,
+__global__ void __launch_bounds__(NT) rowcolscale_kernel(const float* in, const float* cs,
+                                                         const float* rs, float* __restrict__ out,
                                                          int64_t rows, int64_t cols) {
+  grid_begin();
   const int64_t n = rows * cols;
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
     float v = in[i];
@@ -82,8 +86,9 @@ __global__ void __launch_bounds__(NT) rowcolscale_kernel(const float* __restrict
 // ---- H diagonal and diagonal blocks -------------------------------------------------------------
 // (eight rows of a block per CTA: with a CTA per block the dependent loads of 16,384 elements took 33 us)
 constexpr int HB_ROWS = 8;
-__global__ void __launch_bounds__(NT) extract_hblocks_kernel(const float* __restrict__ H, float* __restrict__ hdiag,
+__global__ void __launch_bounds__(NT) extract_hblocks_kernel(const float* H, float* __restrict__ hdiag,
                                                              float* __restrict__ Hjj, int64_t d_in, int db, int diag_only) {
+  grid_begin();
   const int j = blockIdx.x, a0 = blockIdx.y * HB_ROWS;
 #pragma unroll 4
   for (int e = threadIdx.x; e < HB_ROWS * db; e += NT) {
@@ -96,39 +101,57 @@ __global__ void __launch_bounds__(NT) extract_hblocks_kernel(const float* __rest
   }
 }
 
-__global__ void __launch_bounds__(NT) diag_kernel(const float* __restrict__ H, float* __restrict__ hdiag, int64_t d_in) {
+__global__ void __launch_bounds__(NT) diag_kernel(const float* H, float* __restrict__ hdiag, int64_t d_in) {
+  grid_begin();
   const int64_t k = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (k < d_in) hdiag[k] = H[k * d_in + k];
 }
 
 // ---- Gamma_M = Gamma (.) M and its squared norm -------------------------------------------------
 // One float4 per thread step; a mask byte covers m_group / 4 consecutive float4 (q4 = 1 or 2).
-__global__ void __launch_bounds__(NT) masked_copy_kernel(const float4* __restrict__ gam, const uint8_t* __restrict__ M,
+__global__ void __launch_bounds__(NT) masked_copy_kernel(const float4* gam, const uint8_t* M,
                                                          float4* __restrict__ out, int64_t n4, int q4,
                                                          double* __restrict__ part) {
+  grid_begin();
   double acc = 0.0;
-  for (int64_t g = (int64_t)blockIdx.x * NT + threadIdx.x; g < n4; g += (int64_t)gridDim.x * NT) {
-    float4 v = gam[g];
-    const unsigned m = (q4 == 1) ? M[g] : ((unsigned)M[g >> 1] >> (4 * (int)(g & 1)));
-    v.x = (m & 1u) ? v.x : 0.f;
-    v.y = (m & 2u) ? v.y : 0.f;
-    v.z = (m & 4u) ? v.z : 0.f;
-    v.w = (m & 8u) ? v.w : 0.f;
-    out[g] = v;
-    float s = v.x * v.x;
-    s = fmaf(v.y, v.y, s);
-    s = fmaf(v.z, v.z, s);
-    s = fmaf(v.w, v.w, s);
-    acc += (double)s;
+  const int64_t stride = (int64_t)gridDim.x * NT;
+  for (int64_t g0 = (int64_t)blockIdx.x * NT + threadIdx.x; g0 < n4; g0 += 4 * stride) {
+    float4 v4[4];
+    unsigned m4[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t g = g0 + u * stride;
+      v4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      m4[u] = 0u;
+      if (g < n4) { v4[u] = gam[g]; m4[u] = (q4 == 1) ? M[g] : ((unsigned)M[g >> 1] >> (4 * (int)(g & 1))); }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t g = g0 + u * stride;
+      if (g >= n4) break;
+      const unsigned m = m4[u];
+      float4 v = v4[u];
+      v.x = (m & 1u) ? v.x : 0.f;
+      v.y = (m & 2u) ? v.y : 0.f;
+      v.z = (m & 4u) ? v.z : 0.f;
+      v.w = (m & 8u) ? v.w : 0.f;
+      out[g] = v;
+      float s = v.x * v.x;
+      s = fmaf(v.y, v.y, s);
+      s = fmaf(v.z, v.z, s);
+      s = fmaf(v.w, v.w, s);
+      acc += (double)s;
+    }
   }
   acc = block_reduce_sum(acc);
   if (threadIdx.x == 0) part[blockIdx.x] = acc;
 }
 
 // ---- y += sign * sc[slot] * x -------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* __restrict__ y, const float4* __restrict__ x,
-                                                       int64_t n4, const double* __restrict__ sc, int slot,
+__global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* __restrict__ y, const float4* x,
+                                                       int64_t n4, const double* sc, int slot,
                                                        float sign) {
+  grid_begin();
   const float a = sign * (float)sc[slot];
   if (a == 0.f) return;                 // a zero step (also what withheld updates look like): y stays bit for bit
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) {
@@ -140,7 +163,8 @@ __global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* __restrict__ y, c
 // the same for up to three arrays that move by the same step: one launch
 struct AxpyTerm { float4* y; const float4* x; float sign; int64_t n4; };
 __global__ void __launch_bounds__(NT) axpy_multi_slot_kernel(AxpyTerm t0, AxpyTerm t1, AxpyTerm t2, int n_terms, int64_t n4,
-                                                             const double* __restrict__ sc, int slot) {
+                                                             const double* sc, int slot) {
+  grid_begin();
   const float a = (float)sc[slot];
   if (a == 0.f) return;
   const AxpyTerm t[3] = {t0, t1, t2};
@@ -158,8 +182,9 @@ __global__ void __launch_bounds__(NT) axpy_multi_slot_kernel(AxpyTerm t0, AxpyTe
 
 // ---- normalisation (Section 3.2): r1 = column norms, r2 = row norms of W / r1 -------------------
 constexpr int COLSUM_CHUNKS = 64;
-__global__ void __launch_bounds__(NT) colsumsq_partial_kernel(const float* __restrict__ W, int64_t rows, int64_t cols,
+__global__ void __launch_bounds__(NT) colsumsq_partial_kernel(const float* W, int64_t rows, int64_t cols,
                                                               double* __restrict__ part) {
+  grid_begin();
   const int64_t col = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (col >= cols) return;
   const int64_t per = (rows + COLSUM_CHUNKS - 1) / COLSUM_CHUNKS;
@@ -171,8 +196,9 @@ __global__ void __launch_bounds__(NT) colsumsq_partial_kernel(const float* __res
   }
   part[(int64_t)blockIdx.y * cols + col] = acc;
 }
-__global__ void __launch_bounds__(NT) colnorm_final_kernel(const double* __restrict__ part, int64_t cols,
+__global__ void __launch_bounds__(NT) colnorm_final_kernel(const double* part, int64_t cols,
                                                            float* __restrict__ r1) {
+  grid_begin();
   const int64_t col = (int64_t)blockIdx.x * NT + threadIdx.x;
   if (col >= cols) return;
   double acc = 0.0;
@@ -183,9 +209,10 @@ __global__ void __launch_bounds__(NT) colnorm_final_kernel(const double* __restr
 // The row norm of W / r1 to more than double the digits of fp32, without fp64 in the loop (a division in fp64 per element
 // took this pass to three times its memory time): 1 / r1 as a pair of floats, product and square with their rounding errors,
 // the sum as an unevaluated pair per thread, fp64 across threads.
-__global__ void __launch_bounds__(NT) rownorm_scale_kernel(const float* __restrict__ W, const float* __restrict__ r1,
+__global__ void __launch_bounds__(NT) rownorm_scale_kernel(const float* W, const float* r1,
                                                            float* __restrict__ r2, float* __restrict__ Wbar,
                                                            int64_t cols) {
+  grid_begin();
   const int64_t row = blockIdx.x;
   const float* w = W + row * cols;
   float hi = 0.f, lo = 0.f;
@@ -229,16 +256,17 @@ __global__ void __launch_bounds__(NT) rownorm_scale_kernel(const float* __restri
 // of a group lie within 5e-7 of each other, are all below the range where fp32 keeps its digits, or are not finite: only
 // such a group is scored again in fp64, whose instructions otherwise took this pass to three times its memory time.
 template <int MG>
-__global__ void __launch_bounds__(NT) init_core_kernel(const float* __restrict__ W, const float* __restrict__ hdiag,
+__global__ void __launch_bounds__(NT) init_core_kernel(const float* W, const float* hdiag,
                                                        float* __restrict__ S, uint8_t* __restrict__ M,
                                                        int64_t ngroups, int groups_per_row, int n_keep) {
+  grid_begin();
   for (int64_t g = (int64_t)blockIdx.x * NT + threadIdx.x; g < ngroups; g += (int64_t)gridDim.x * NT) {
     const int64_t c0 = (g % groups_per_row) * MG;
     float wv[MG], hv[MG], sc[MG];
 #pragma unroll
     for (int h = 0; h < MG / 4; ++h) {
       const float4 w = *reinterpret_cast<const float4*>(W + g * MG + 4 * h);
-      const float4 d = __ldg(reinterpret_cast<const float4*>(hdiag + c0 + 4 * h));
+      const float4 d = *reinterpret_cast<const float4*>(hdiag + c0 + 4 * h);
       wv[4 * h] = w.x; wv[4 * h + 1] = w.y; wv[4 * h + 2] = w.z; wv[4 * h + 3] = w.w;
       hv[4 * h] = d.x; hv[4 * h + 1] = d.y; hv[4 * h + 2] = d.z; hv[4 * h + 3] = d.w;
     }
@@ -283,11 +311,13 @@ __global__ void __launch_bounds__(NT) init_core_kernel(const float* __restrict__
 }
 
 __global__ void identity_blocks_kernel(float* __restrict__ A, int db) {
+  grid_begin();
   const int64_t off = (int64_t)blockIdx.x * db * db;
   for (int e = threadIdx.x; e < db * db; e += blockDim.x) A[off + e] = (e / db == e % db) ? 1.f : 0.f;
 }
 
-__global__ void copy_kernel(const float4* __restrict__ in, float4* __restrict__ out, int64_t n4) {
+__global__ void copy_kernel(const float4* in, float4* __restrict__ out, int64_t n4) {
+  grid_begin();
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) out[i] = in[i];
 }
 
@@ -309,6 +339,7 @@ __device__ __forceinline__ void start_record(armor_iter_stats* st, double loss) 
 static_assert(SC_COUNT == 32, "one scalar per lane");
 __global__ void zero_scalars_kernel(double* sc, int32_t* failflag, int nflag, int carry_loss, armor_iter_stats* st_base,
                                     int64_t* it_dev, int advance) {
+  grid_begin();
   const double carried = sc[SC_LOSS];
   __syncthreads();
   for (int i = threadIdx.x; i < SC_COUNT; i += blockDim.x)
@@ -324,7 +355,7 @@ __global__ void zero_scalars_kernel(double* sc, int32_t* failflag, int nflag, in
 // Fixed-order sums by the CTA of the bookkeeping kernel (STAGE_NT threads): thread t adds entries t, t + STAGE_NT, ...
 // (eight loads in flight).  The line searches hand over thousands of partial sums (four or eight per tile).
 constexpr int STAGE_NT = 1024;
-__device__ __forceinline__ double stage_thread_sum(const double* __restrict__ p, int n) {
+__device__ __forceinline__ double stage_thread_sum(const double* p, int n) {
   double v = 0.0;
   int i = threadIdx.x;
   for (; i + 7 * STAGE_NT < n; i += 8 * STAGE_NT) {
@@ -407,9 +438,10 @@ __device__ __forceinline__ void stage_scalars(double* sc, armor_iter_stats* st, 
 // All sums of a call go through one shuffle tree and one barrier; the scalars and the record thread 0 will need are on their
 // way meanwhile (the kernel is nothing but latency: as a chain of separate sums it took 4 to 6 us, four times an iteration).
 __global__ void __launch_bounds__(STAGE_NT)
-stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* __restrict__ it_dev, int stage, int32_t* failflag,
+stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* it_dev, int stage, int32_t* failflag,
              int nflag, int nflag_clear, const double* partA, int nA, int32_t* status, const double* p1, int n1, int slot1,
              const double* p2, int n2, int slot2) {
+  grid_begin();
   __shared__ double sc[SC_COUNT];
   __shared__ double sums[3][STAGE_NT / 32];
   __shared__ int flags[STAGE_NT / 32];
@@ -458,10 +490,11 @@ stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* __restrict_
 __device__ __forceinline__ int bad4(const float4 v) {
   return (isfinite(v.x) ? 0 : 1) + (isfinite(v.y) ? 0 : 1) + (isfinite(v.z) ? 0 : 1) + (isfinite(v.w) ? 0 : 1);
 }
-__global__ void __launch_bounds__(NT) screen_count_kernel(const float4* __restrict__ W, int64_t wn4,
-                                                          const float4* __restrict__ H, int64_t hn4,
-                                                          const float* __restrict__ Hs, int64_t d_in,
+__global__ void __launch_bounds__(NT) screen_count_kernel(const float4* W, int64_t wn4,
+                                                          const float4* H, int64_t hn4,
+                                                          const float* Hs, int64_t d_in,
                                                           int32_t* __restrict__ scr) {
+  grid_begin();
   int bw = 0, bh = 0, neg = 0, zero = 0;
   const int64_t stride = (int64_t)gridDim.x * NT, i0 = (int64_t)blockIdx.x * NT + threadIdx.x;
   for (int64_t i = i0; i < wn4; i += stride) bw += bad4(W[i]);
@@ -482,7 +515,8 @@ __global__ void __launch_bounds__(NT) screen_count_kernel(const float4* __restri
     if (zero) atomicAdd(&scr[3], zero);
   }
 }
-__global__ void screen_final_kernel(const int32_t* __restrict__ scr, int32_t* __restrict__ status) {
+__global__ void screen_final_kernel(const int32_t* scr, int32_t* __restrict__ status) {
+  grid_begin();
   status[ST_NONFINITE_W] += scr[0];
   status[ST_NONFINITE_H] += scr[1];
   status[ST_NEG_DIAG_H] += scr[2];
@@ -493,8 +527,9 @@ __global__ void screen_final_kernel(const int32_t* __restrict__ scr, int32_t* __
 }
 
 // ---- operand split for the three-pass tensor-core mode ------------------------------------------
-__global__ void __launch_bounds__(NT) split_hilo_kernel(const float4* __restrict__ in, float4* __restrict__ hi,
+__global__ void __launch_bounds__(NT) split_hilo_kernel(const float4* in, float4* __restrict__ hi,
                                                         float4* __restrict__ lo, int64_t n4) {
+  grid_begin();
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) {
     float4 v = in[i];
     float4 h;
@@ -534,17 +569,19 @@ __global__ void transpose_split_kernel(const TIn* __restrict__ X, int64_t ldx, i
 }
 
 // bf16 <-> fp32 with an optional per-column scale (the denormalisation of the deployment form)
-__global__ void __launch_bounds__(NT) bf16_to_f32_kernel(const __nv_bfloat16* __restrict__ in,
-                                                         const float* __restrict__ cs, float* __restrict__ out,
+__global__ void __launch_bounds__(NT) bf16_to_f32_kernel(const __nv_bfloat16* in,
+                                                         const float* cs, float* __restrict__ out,
                                                          int64_t n, int64_t cols) {
+  grid_begin();
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
     float v = __bfloat162float(in[i]);
     if (cs) v *= cs[i % cols];
     out[i] = v;
   }
 }
-__global__ void __launch_bounds__(NT) f32_to_bf16_kernel(const float* __restrict__ in, const float* __restrict__ cs,
+__global__ void __launch_bounds__(NT) f32_to_bf16_kernel(const float* in, const float* cs,
                                                          __nv_bfloat16* __restrict__ out, int64_t n, int64_t cols) {
+  grid_begin();
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
     float v = in[i];
     if (cs) v *= cs[i % cols];
@@ -623,9 +660,10 @@ __global__ void __launch_bounds__(NT, 8) mirror_lower_kernel(float* H, int64_t n
 }
 
 // part[b] = weight * || X_b ||_F for block b of db x db floats (the terms of beta_A and beta_B, Eq. lrA / lrB)
-__global__ void __launch_bounds__(NT) block_fro_kernel(const float4* __restrict__ X, int n4_per_block,
-                                                       const float* __restrict__ hdiag, int db, int nbi,
+__global__ void __launch_bounds__(NT) block_fro_kernel(const float4* X, int n4_per_block,
+                                                       const float* hdiag, int db, int nbi,
                                                        double* __restrict__ part) {
+  grid_begin();
   const float4* xb = X + (int64_t)blockIdx.x * n4_per_block;
   double acc = 0.0;
   for (int i = threadIdx.x; i < n4_per_block; i += NT) {
@@ -647,11 +685,12 @@ __global__ void __launch_bounds__(NT) block_fro_kernel(const float4* __restrict_
 }
 
 // ---- Adam (Kingma & Ba, Algorithm 1, with bias correction) ----------------------------------------------
-__global__ void __launch_bounds__(NT) adam_kernel(float4* __restrict__ theta, const float4* __restrict__ gamma,
+__global__ void __launch_bounds__(NT) adam_kernel(float4* __restrict__ theta, const float4* gamma,
                                                   float4* __restrict__ m, float4* __restrict__ v, int64_t n4,
-                                                  const uint8_t* __restrict__ M, int q4, float lr, float b1, float b2,
-                                                  float eps, int64_t step_base, const int64_t* __restrict__ it_dev,
-                                                  const int32_t* __restrict__ status) {
+                                                  const uint8_t* M, int q4, float lr, float b1, float b2,
+                                                  float eps, int64_t step_base, const int64_t* it_dev,
+                                                  const int32_t* status) {
+  grid_begin();
   if (status[ST_POISON] != 0) return;   // unusable inputs: parameters and moments stay as they are
   // bias corrections 1 / (1 - beta^step), step = step_base + the iteration counter: once per block
   __shared__ float s_bc[2];
@@ -692,28 +731,28 @@ inline int grid_for(int64_t n) {
 
 void dot_to_ptr(armor_ctx* c, const float* x, const float* y, int64_t n, double* out, cudaStream_t s) {
   KTimer kt(c, n >= (1 << 22) ? ARMOR_KC_DOT : ARMOR_KC_SMALL, 8.0 * (double)n, s);
-  dot_partial_kernel<<<ARMOR_DOT_BLOCKS, NT, 0, s>>>((const float4*)x, (const float4*)y, n / 4, c->partials);
-  reduce_final_kernel<<<1, NT, 0, s>>>(c->partials, ARMOR_DOT_BLOCKS, out);
+  launch_dependent(dot_partial_kernel, ARMOR_DOT_BLOCKS, NT, 0, s, (const float4*)x, (const float4*)y, n / 4, c->partials);
+  launch_dependent(reduce_final_kernel, 1, NT, 0, s, c->partials, ARMOR_DOT_BLOCKS, out);
   c->launches += 2;
 }
 
 // partial sums of <x, y> only (ARMOR_DOT_BLOCKS entries at `part`); the consumer adds them up
 void dot_partials(armor_ctx* c, const float* x, const float* y, int64_t n, double* part, cudaStream_t s) {
   KTimer kt(c, n >= (1 << 22) ? ARMOR_KC_DOT : ARMOR_KC_SMALL, 8.0 * (double)n, s);
-  dot_partial_kernel<<<ARMOR_DOT_BLOCKS, NT, 0, s>>>((const float4*)x, (const float4*)y, n / 4, part);
+  launch_dependent(dot_partial_kernel, ARMOR_DOT_BLOCKS, NT, 0, s, (const float4*)x, (const float4*)y, n / 4, part);
   c->launches++;
 }
 
 void reduce_partials_to(armor_ctx* c, const double* part, int n, double* out, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  reduce_final_kernel<<<1, NT, 0, s>>>(part, n, out);
+  launch_dependent(reduce_final_kernel, 1, NT, 0, s, part, n, out);
   c->launches++;
 }
 
 void launch_colscale(armor_ctx* c, const float* in, const float* h, float* out, int64_t rows, int64_t cols,
                      cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_AXPY, 8.0 * (double)rows * (double)cols, s);
-  colscale_kernel<<<grid_for(rows * cols / 4), NT, 0, s>>>((const float4*)in, (const float4*)h, (float4*)out,
+  launch_dependent(colscale_kernel, grid_for(rows * cols / 4), NT, 0, s, (const float4*)in, (const float4*)h, (float4*)out,
                                                           rows * cols / 4, (int)(cols / 4));
   c->launches++;
 }
@@ -721,26 +760,26 @@ void launch_colscale(armor_ctx* c, const float* in, const float* h, float* out, 
 void launch_scale_rows_cols(armor_ctx* c, const float* in, const float* colscale, const float* rowscale, float* out,
                             int64_t rows, int64_t cols, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_FORWARD, 8.0 * (double)rows * (double)cols, s);
-  rowcolscale_kernel<<<grid_for(rows * cols), NT, 0, s>>>(in, colscale, rowscale, out, rows, cols);
+  launch_dependent(rowcolscale_kernel, grid_for(rows * cols), NT, 0, s, in, colscale, rowscale, out, rows, cols);
   c->launches++;
 }
 
 void launch_extract_hblocks(armor_ctx* c, const float* H, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  extract_hblocks_kernel<<<dim3(c->nbi, (c->db + HB_ROWS - 1) / HB_ROWS), NT, 0, s>>>(H, c->hdiag, c->Hjj, c->d_in, c->db, c->cfg.h_mode == ARMOR_H_DIAG);
+  launch_dependent(extract_hblocks_kernel, dim3(c->nbi, (c->db + HB_ROWS - 1) / HB_ROWS), NT, 0, s, H, c->hdiag, c->Hjj, c->d_in, c->db, c->cfg.h_mode == ARMOR_H_DIAG);
   c->launches++;
 }
 
 void launch_masked_copy(armor_ctx* c, const float* Gam, const uint8_t* M, float* out, double* part, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASKED_COPY, (8.0 + 1.0 / c->cfg.m_group) * (double)c->wn, s);
-  masked_copy_kernel<<<ARMOR_DOT_BLOCKS, NT, 0, s>>>((const float4*)Gam, M, (float4*)out, c->wn / 4,
+  launch_dependent(masked_copy_kernel, ARMOR_DOT_BLOCKS, NT, 0, s, (const float4*)Gam, M, (float4*)out, c->wn / 4,
                                                     c->cfg.m_group / 4, part);
   c->launches++;
 }
 
 void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slot, float sign, cudaStream_t s) {
   KTimer kt(c, n >= (1 << 22) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * (double)n, s);
-  axpy_slot_kernel<<<grid_for(n / 4), NT, 0, s>>>((float4*)y, (const float4*)x, n / 4, c->sc, slot, sign);
+  launch_dependent(axpy_slot_kernel, grid_for(n / 4), NT, 0, s, (float4*)y, (const float4*)x, n / 4, c->sc, slot, sign);
   c->launches++;
 }
 
@@ -758,7 +797,7 @@ void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64
   for (int j = 0; j < k; ++j) { n4 = t[j].n4 > n4 ? t[j].n4 : n4; elems += 4.0 * (double)t[j].n4; }
   for (int j = k; j < 3; ++j) t[j] = t[0];
   KTimer kt(c, n4 >= (1 << 20) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * elems, s);
-  axpy_multi_slot_kernel<<<grid_for(n4), NT, 0, s>>>(t[0], t[1], t[2], k, n4, c->sc, slot);
+  launch_dependent(axpy_multi_slot_kernel, grid_for(n4), NT, 0, s, t[0], t[1], t[2], k, n4, c->sc, slot);
   c->launches++;
 }
 
@@ -771,24 +810,24 @@ void launch_init(armor_ctx* c, const float* W, const float* H, float* Wbar, floa
   if (c->cfg.normalize) {
     double* part = c->colpart;
     dim3 g1((unsigned)((cols + NT - 1) / NT), COLSUM_CHUNKS);
-    colsumsq_partial_kernel<<<g1, NT, 0, s>>>(W, rows, cols, part);
-    colnorm_final_kernel<<<(unsigned)((cols + NT - 1) / NT), NT, 0, s>>>(part, cols, r1);
-    rownorm_scale_kernel<<<(unsigned)rows, NT, 0, s>>>(W, r1, r2, Wbar, cols);
+    launch_dependent(colsumsq_partial_kernel, g1, NT, 0, s, W, rows, cols, part);
+    launch_dependent(colnorm_final_kernel, (unsigned)((cols + NT - 1) / NT), NT, 0, s, part, cols, r1);
+    launch_dependent(rownorm_scale_kernel, (unsigned)rows, NT, 0, s, W, r1, r2, Wbar, cols);
     c->launches += 3;
   } else if (Wbar != W) {
-    copy_kernel<<<grid_for(c->wn / 4), NT, 0, s>>>((const float4*)W, (float4*)Wbar, c->wn / 4);
+    launch_dependent(copy_kernel, grid_for(c->wn / 4), NT, 0, s, (const float4*)W, (float4*)Wbar, c->wn / 4);
     c->launches++;
   }
   const int mg = c->cfg.m_group;
-  diag_kernel<<<(unsigned)((cols + NT - 1) / NT), NT, 0, s>>>(H, c->hdiag, cols);
+  launch_dependent(diag_kernel, (unsigned)((cols + NT - 1) / NT), NT, 0, s, H, c->hdiag, cols);
   if (mg == 8)
-    init_core_kernel<8><<<grid_for(c->wn / 8), NT, 0, s>>>(Wbar, c->hdiag, S, M, c->wn / 8, (int)(cols / 8),
+    launch_dependent(init_core_kernel<8>, grid_for(c->wn / 8), NT, 0, s, Wbar, c->hdiag, S, M, c->wn / 8, (int)(cols / 8),
                                                           c->cfg.n_keep);
   else
-    init_core_kernel<4><<<grid_for(c->wn / 4), NT, 0, s>>>(Wbar, c->hdiag, S, M, c->wn / 4, (int)(cols / 4),
+    launch_dependent(init_core_kernel<4>, grid_for(c->wn / 4), NT, 0, s, Wbar, c->hdiag, S, M, c->wn / 4, (int)(cols / 4),
                                                           c->cfg.n_keep);
-  identity_blocks_kernel<<<c->nbo, NT, 0, s>>>(A, c->db);
-  identity_blocks_kernel<<<c->nbi, NT, 0, s>>>(B, c->db);
+  launch_dependent(identity_blocks_kernel, c->nbo, NT, 0, s, A, c->db);
+  launch_dependent(identity_blocks_kernel, c->nbi, NT, 0, s, B, c->db);
   c->launches += 4;
 }
 
@@ -796,10 +835,10 @@ armor_status launch_screen_inputs(armor_ctx* c, const float* W, const float* H, 
   if (cudaMemsetAsync(c->screen, 0, 4 * sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
   const int64_t wn4 = c->wn / 4, hn4 = c->d_in * c->d_in / 4;
   KTimer kt(c, ARMOR_KC_INIT, 4.0 * ((double)c->wn + (double)c->d_in * (double)c->d_in), s);
-  screen_count_kernel<<<grid_for(wn4 > hn4 ? wn4 : hn4), NT, 0, s>>>(reinterpret_cast<const float4*>(W), wn4,
+  launch_dependent(screen_count_kernel, grid_for(wn4 > hn4 ? wn4 : hn4), NT, 0, s, reinterpret_cast<const float4*>(W), wn4,
                                                                      reinterpret_cast<const float4*>(H), hn4, H, c->d_in,
                                                                      c->screen);
-  screen_final_kernel<<<1, 1, 0, s>>>(c->screen, c->status);
+  launch_dependent(screen_final_kernel, 1, 1, 0, s, c->screen, c->status);
   c->launches += 2;
   return ARMOR_OK;
 }
@@ -807,7 +846,7 @@ armor_status launch_screen_inputs(armor_ctx* c, const float* W, const float* H, 
 void launch_zero_scalars(armor_ctx* c, bool advance, bool carry_loss, armor_iter_stats* st, cudaStream_t s) {
   const int nflag = c->nbo > c->nbi ? c->nbo : c->nbi;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  zero_scalars_kernel<<<1, NT, 0, s>>>(c->sc, c->failflag, nflag, carry_loss ? 1 : 0, st, c->it_dev, advance ? 1 : 0);
+  launch_dependent(zero_scalars_kernel, 1, NT, 0, s, c->sc, c->failflag, nflag, carry_loss ? 1 : 0, st, c->it_dev, advance ? 1 : 0);
   c->launches++;
 }
 
@@ -815,14 +854,14 @@ void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* p
                   cudaStream_t s, const double* p1, int n1, int slot1, const double* p2, int n2, int slot2) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
   const int nflag_clear = stage == 1 ? (c->nbo > c->nbi ? c->nbo : c->nbi) : 0;     // the B-step's solves start afresh
-  stage_kernel<<<1, STAGE_NT, 0, s>>>(c->sc, st, c->it_dev, stage, c->failflag, nflag, nflag_clear, part, npart, c->status, p1,
+  launch_dependent(stage_kernel, 1, STAGE_NT, 0, s, c->sc, st, c->it_dev, stage, c->failflag, nflag, nflag_clear, part, npart, c->status, p1,
                                       n1, slot1, p2, n2, slot2);
   c->launches++;
 }
 
 void launch_split_hilo(armor_ctx* c, const float* in, float* hi, float* lo, int64_t n, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 8.0 * (double)n, s);
-  split_hilo_kernel<<<grid_for(n / 4), NT, 0, s>>>((const float4*)in, (float4*)hi, (float4*)lo, n / 4);
+  launch_dependent(split_hilo_kernel, grid_for(n / 4), NT, 0, s, (const float4*)in, (float4*)hi, (float4*)lo, n / 4);
   c->launches++;
 }
 
@@ -857,8 +896,8 @@ void launch_mirror_lower(armor_ctx* c, float* H, int64_t n, cudaStream_t s, cons
 
 void launch_block_fro_sum(armor_ctx* c, const float* X, int nblk, const float* hdiag, double* out, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  block_fro_kernel<<<nblk, NT, 0, s>>>((const float4*)X, c->db * c->db / 4, hdiag, c->db, c->nbi, c->quadpart);
-  reduce_final_kernel<<<1, NT, 0, s>>>(c->quadpart, nblk, out);
+  launch_dependent(block_fro_kernel, nblk, NT, 0, s, (const float4*)X, c->db * c->db / 4, hdiag, c->db, c->nbi, c->quadpart);
+  launch_dependent(reduce_final_kernel, 1, NT, 0, s, c->quadpart, nblk, out);
   c->launches += 2;
 }
 
@@ -869,7 +908,7 @@ void launch_adam(armor_ctx* c, float* theta, const float* gamma, float* m, float
   const float b2 = c->cfg.adam_beta2 > 0.f ? c->cfg.adam_beta2 : 0.999f;
   const float eps = c->cfg.adam_eps > 0.f ? c->cfg.adam_eps : 1e-8f;
   KTimer kt(c, n >= (1 << 22) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 28.0 * (double)n, s);
-  adam_kernel<<<grid_for(n / 4), NT, 0, s>>>((float4*)theta, (const float4*)gamma, (float4*)m, (float4*)v, n / 4, M,
+  launch_dependent(adam_kernel, grid_for(n / 4), NT, 0, s, (float4*)theta, (const float4*)gamma, (float4*)m, (float4*)v, n / 4, M,
                                             c->cfg.m_group / 4, lr, b1, b2, eps, step_base, c->it_dev, c->status);
   c->launches++;
 }
@@ -877,7 +916,7 @@ void launch_adam(armor_ctx* c, float* theta, const float* gamma, float* m, float
 void launch_bf16_to_f32(armor_ctx* c, const void* in, const float* colscale, float* out, int64_t rows, int64_t cols,
                         cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_FORWARD, 6.0 * (double)rows * (double)cols, s);
-  bf16_to_f32_kernel<<<grid_for(rows * cols), NT, 0, s>>>(static_cast<const __nv_bfloat16*>(in), colscale, out,
+  launch_dependent(bf16_to_f32_kernel, grid_for(rows * cols), NT, 0, s, static_cast<const __nv_bfloat16*>(in), colscale, out,
                                                          rows * cols, cols);
   c->launches++;
 }
@@ -885,7 +924,7 @@ void launch_bf16_to_f32(armor_ctx* c, const void* in, const float* colscale, flo
 void launch_f32_to_bf16(armor_ctx* c, const float* in, const float* colscale, void* out, int64_t rows, int64_t cols,
                         cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_FORWARD, 6.0 * (double)rows * (double)cols, s);
-  f32_to_bf16_kernel<<<grid_for(rows * cols), NT, 0, s>>>(in, colscale, static_cast<__nv_bfloat16*>(out), rows * cols,
+  launch_dependent(f32_to_bf16_kernel, grid_for(rows * cols), NT, 0, s, in, colscale, static_cast<__nv_bfloat16*>(out), rows * cols,
                                                          cols);
   c->launches++;
 }

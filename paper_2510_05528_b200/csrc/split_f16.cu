@@ -57,7 +57,8 @@ __device__ __forceinline__ float block_max(float v) {
 }
 
 // hpow[k] = 2^floor(log2 sqrt(H_kk)) (1 for a dead channel)
-__global__ void hpow_kernel(const float* __restrict__ hdiag, float* __restrict__ hpow, int64_t n) {
+__global__ void hpow_kernel(const float* hdiag, float* __restrict__ hpow, int64_t n) {
+  grid_begin();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const float h = hdiag[k];
@@ -76,15 +77,16 @@ __device__ __forceinline__ float over_pow2(float d, int shift) {
 }
 
 // Hhi + Hlo = H_kn / (d_k d_n) * 2^H_SHIFT, four columns per thread
-__global__ void __launch_bounds__(NT) split_H_kernel(const float4* __restrict__ H, const float* __restrict__ hpow,
+__global__ void __launch_bounds__(NT) split_H_kernel(const float4* H, const float* hpow,
                                                      __half2* __restrict__ hi, __half2* __restrict__ lo, int64_t n,
                                                      int32_t* __restrict__ status) {
+  grid_begin();
   const int64_t n4 = n / 4;
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n * n4; i += (int64_t)gridDim.x * NT) {
     const int64_t k = i / n4, c4 = (i % n4) * 4;
     const float rk = over_pow2(hpow[k], H_SHIFT);
     const float4 v = H[i];
-    const float4 d = __ldg(reinterpret_cast<const float4*>(hpow + c4));
+    const float4 d = *reinterpret_cast<const float4*>(hpow + c4);
     const float x0 = v.x * rk * over_pow2(d.x, 0), x1 = v.y * rk * over_pow2(d.y, 0), x2 = v.z * rk * over_pow2(d.z, 0),
                 x3 = v.w * rk * over_pow2(d.w, 0);
     const int over = (fabsf(x0) > 65504.f && isfinite(x0)) + (fabsf(x1) > 65504.f && isfinite(x1)) +
@@ -105,17 +107,18 @@ __global__ void __launch_bounds__(NT) split_H_kernel(const float4* __restrict__ 
 // the maximum and the split (0: the row is read again).  The scaling is a product with a power of two: exact, or rounded
 // once where the result is subnormal.
 template <int KEEP>
-__global__ void __launch_bounds__(NT) split_rows_kernel(const float* __restrict__ in, int64_t ld, int64_t cols,
-                                                        const float* __restrict__ colscale, float post,
+__global__ void __launch_bounds__(NT) split_rows_kernel(const float* in, int64_t ld, int64_t cols,
+                                                        const float* colscale, float post,
                                                         __half2* __restrict__ hi, __half2* __restrict__ lo,
                                                         float* __restrict__ out_scale) {
+  grid_begin();
   const int64_t row = blockIdx.x;
   const float4* src = reinterpret_cast<const float4*>(in + row * ld);
   const float4* cs4 = reinterpret_cast<const float4*>(colscale);
   const int64_t c4n = cols / 4;
   auto fetch = [&](int64_t i) {
     float4 v = src[i];
-    if (colscale) { const float4 d = __ldg(cs4 + i); v.x *= d.x; v.y *= d.y; v.z *= d.z; v.w *= d.w; }
+    if (colscale) { const float4 d = cs4[i]; v.x *= d.x; v.y *= d.y; v.z *= d.z; v.w *= d.w; }
     return v;
   };
   auto larger = [](float m, const float4& v) { return fmaxf(m, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
@@ -283,9 +286,9 @@ inline unsigned grid_for(int64_t n) {
 void launch_f16_prepare_H(armor_ctx* c, const float* H, cudaStream_t s) {
   const int64_t n = c->d_in;
   KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 8.0 * (double)n * (double)n, s);
-  hpow_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(c->hdiag, c->hpow, n);
+  launch_dependent(hpow_kernel, (unsigned)((n + 255) / 256), 256, 0, s, c->hdiag, c->hpow, n);
   __half* hi = reinterpret_cast<__half*>(c->Hlo);
-  split_H_kernel<<<grid_for(n * n / 4), NT, 0, s>>>(reinterpret_cast<const float4*>(H), c->hpow,
+  launch_dependent(split_H_kernel, grid_for(n * n / 4), NT, 0, s, reinterpret_cast<const float4*>(H), c->hpow,
                                                     reinterpret_cast<__half2*>(hi), reinterpret_cast<__half2*>(hi + n * n), n, c->status);
   c->launches += 2;
 }
@@ -295,10 +298,10 @@ void launch_f16_split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t ro
   KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 8.0 * (double)rows * (double)cols, s);
   __half2 *h = static_cast<__half2*>(hi), *l = static_cast<__half2*>(lo);
   // a row in registers up to 8,192 columns: one read of it instead of two (from L1 or L2)
-  if (cols <= 4 * NT) split_rows_kernel<1><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
-  else if (cols <= 16 * NT) split_rows_kernel<4><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
-  else if (cols <= 32 * NT) split_rows_kernel<8><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
-  else split_rows_kernel<0><<<(unsigned)rows, NT, 0, s>>>(in, ld, cols, colscale, post, h, l, out_scale);
+  if (cols <= 4 * NT) launch_dependent(split_rows_kernel<1>, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale);
+  else if (cols <= 16 * NT) launch_dependent(split_rows_kernel<4>, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale);
+  else if (cols <= 32 * NT) launch_dependent(split_rows_kernel<8>, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale);
+  else launch_dependent(split_rows_kernel<0>, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale);
   c->launches++;
 }
 
