@@ -292,6 +292,8 @@ bool tc_gram_ok(const armor_ctx* c);
 armor_status tc_rowblock_gram(armor_ctx* c, const float* P, const float* T, float* G, cudaStream_t s);
 armor_status tc_colblock_gram(armor_ctx* c, const float* U, const float* Y, float* Cm, cudaStream_t s);
 // two Grams with a shared operand in one launch (the shared chunks are read once)
+armor_status tc_gram_launch(armor_ctx* c, const float* A, const float* A2, const float* B, bool by_rows, bool self, float* C, float* C2,
+                            int n_split, cudaStream_t s);
 armor_status tc_rowblock_gram_pair(armor_ctx* c, const float* P, const float* P2, const float* T, float* G, float* G2,
                                    cudaStream_t s);
 armor_status tc_colblock_gram_self_pair(armor_ctx* c, const float* U, const float* Y, float* Cm, float* Cm2, cudaStream_t s);
