@@ -97,7 +97,7 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const uint32_t full0 = smem_u32(&bars[0]), split0 = smem_u32(&bars[STAGES]), empty0 = smem_u32(&bars[2 * STAGES]);
   const uint32_t d1full0 = smem_u32(&bars[3 * STAGES]), convdone = d1full0 + 16;
   const uint32_t d2full = d1full0 + 24, d2empty = d1full0 + 32;
@@ -128,7 +128,7 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
   __syncthreads();
   tc_fence_after();
   grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
-  const uint32_t tmem_base = tmem_base_holder;
+  const uint32_t tmem_base = uniform(tmem_base_holder);
   volatile int* abortp = &abort_flag;
 
   if (warp == 0) {
@@ -171,7 +171,8 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {
+      const uint32_t leader = elect_lane();
       const uint32_t idesc1 = instr_desc_tf32_mn(TILE, TILE, p.l_mn, 1);
       const uint32_t idesc2 = instr_desc_tf32_mn(TILE, TILE, 0, p.r_mn);
       // descriptors of stage 0; only their address field moves
@@ -189,51 +190,53 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
         const uint32_t d1 = tmem_base + T_D1 + (uint32_t)((t & 1) * TILE);
         if (!second) {
           // ---- product 1 of tile t: D1[t % 2] = Lop_i X_ij  (low part of Lop first, as in the one-sided kernel).  The
-          // buffer was last read by product 2 of tile t - 2, which precedes this point in the pipe's order.
+          // buffer was last read by product 2 of tile t - 2, which has to be complete: instructions with different
+          // accumulators are not ordered among each other.
+          if (t >= 2 && !mbar_wait_warp(d2full, (uint32_t)t & 1u, abortp, p.status)) { ok = false; break; }
           for (int kc = 0; kc < 4; ++kc) {
-            if (!mbar_wait(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+            if (!mbar_wait_warp(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
             tc_fence_after();
             const uint64_t so = (uint64_t)(uint32_t)(stage * (STAGE_BYTES >> 4));
             const uint64_t da = da0 + so, dal = da + (OP_BYTES >> 4), dx = dx0 + so, dxl = dx + (OP_BYTES >> 4);
-            umma_tf32(d1, dal, dx, idesc1, (uint32_t)(kc > 0));
-            umma_tf32_acc(d1, da, dxl, idesc1);
-            umma_tf32_acc(d1, da, dx, idesc1);
+            umma_tf32_w(leader, d1, dal, dx, idesc1, (uint32_t)(kc > 0));
+            umma_tf32_w(leader, d1, da, dxl, idesc1, 1u);
+            umma_tf32_w(leader, d1, da, dx, idesc1, 1u);
 #pragma unroll
             for (int k = 1; k < BK / 8; ++k) {
-              umma_tf32_acc(d1, dal + k * kinc_a, dx + k * kinc_x, idesc1);
-              umma_tf32_acc(d1, da + k * kinc_a, dxl + k * kinc_x, idesc1);
-              umma_tf32_acc(d1, da + k * kinc_a, dx + k * kinc_x, idesc1);
+              umma_tf32_w(leader, d1, dal + k * kinc_a, dx + k * kinc_x, idesc1, 1u);
+              umma_tf32_w(leader, d1, da + k * kinc_a, dxl + k * kinc_x, idesc1, 1u);
+              umma_tf32_w(leader, d1, da + k * kinc_a, dx + k * kinc_x, idesc1, 1u);
             }
-            umma_commit(empty0 + 8 * stage);
+            umma_commit_w(leader, empty0 + 8 * stage);
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
           }
           if (!ok) break;
-          umma_commit(d1full0 + 8 * (t & 1));
+          umma_commit_w(leader, d1full0 + 8 * (t & 1));
         } else {
           // ---- product 2 of tile t: D2 = D1[t % 2] Rop_j, D1 from tensor memory (its low part first: the M side of this
           // product).  Warps 10-13 have split D1; the epilogue has drained D2 of tile t - 1.
-          if (!mbar_wait(convdone, (uint32_t)t & 1u, abortp, p.status)) { ok = false; break; }
-          if (t > 0 && !mbar_wait(d2empty, (uint32_t)(t - 1) & 1u, abortp, p.status)) { ok = false; break; }
+          if (!mbar_wait_warp(convdone, (uint32_t)t & 1u, abortp, p.status)) { ok = false; break; }
+          if (t > 0 && !mbar_wait_warp(d2empty, (uint32_t)(t - 1) & 1u, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
           for (int kc = 0; kc < 4; ++kc) {
-            if (!mbar_wait(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+            if (!mbar_wait_warp(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
             tc_fence_after();
             const uint64_t dr = dr0 + (uint64_t)(uint32_t)(stage * (STAGE_BYTES >> 4)), drl = dr + (OP_BYTES >> 4);
             const uint32_t a_hi = d1 + (uint32_t)(kc * BK), a_lo = d1lo + (uint32_t)(kc * BK);
-            umma_tf32_ta(d2, a_lo, dr, idesc2, (uint32_t)(kc > 0));
-            umma_tf32_ta_acc(d2, a_hi, drl, idesc2);
-            umma_tf32_ta_acc(d2, a_hi, dr, idesc2);
+            umma_tf32_ta_w(leader, d2, a_lo, dr, idesc2, (uint32_t)(kc > 0));
+            umma_tf32_ta_w(leader, d2, a_hi, drl, idesc2, 1u);
+            umma_tf32_ta_w(leader, d2, a_hi, dr, idesc2, 1u);
 #pragma unroll
             for (int k = 1; k < BK / 8; ++k) {
-              umma_tf32_ta_acc(d2, a_lo + 8 * k, dr + k * kinc_r, idesc2);
-              umma_tf32_ta_acc(d2, a_hi + 8 * k, drl + k * kinc_r, idesc2);
-              umma_tf32_ta_acc(d2, a_hi + 8 * k, dr + k * kinc_r, idesc2);
+              umma_tf32_ta_w(leader, d2, a_lo + 8 * k, dr + k * kinc_r, idesc2, 1u);
+              umma_tf32_ta_w(leader, d2, a_hi + 8 * k, drl + k * kinc_r, idesc2, 1u);
+              umma_tf32_ta_w(leader, d2, a_hi + 8 * k, dr + k * kinc_r, idesc2, 1u);
             }
-            umma_commit(empty0 + 8 * stage);
+            umma_commit_w(leader, empty0 + 8 * stage);
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
           }
           if (!ok) break;
-          umma_commit(d2full);      // D2 is complete; the low part of D1 may be overwritten
+          umma_commit_w(leader, d2full);      // D2 is complete; the low part of D1 may be overwritten
         }
       }
     }

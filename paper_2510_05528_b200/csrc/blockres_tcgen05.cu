@@ -10,8 +10,8 @@
 //   one product : 128 x 128 x 8 instructions into two accumulators in turn, four epilogue warps for each, so that the
 //                 MMAs of a tile run while the tile before is stored.  (With one accumulator of 256 columns, two tiles per
 //                 instruction, the MMAs waited for the epilogue and the pass was no faster than the streaming kernel.)
-//                 Left at 4096 x 4096: 39 us, 47 with an addend, against 42 and 55.  With neither MMAs nor split nor
-//                 store it takes 29 us: what is left is the loads with their head and tail.
+//                 Left at 4096 x 4096: 31 us, 38 with an addend, against 37 and 44 there and 25 for a copy; with operands formed
+//                 in front of every MMA by one lane (tc_common.cuh, umma_tf32_ta_w) it took 34 and 40.
 //   dual product: A.X1 and A.X2 of a tile in one 128 x 256 x 8 instruction.
 //   side "left":   out[128 b + m][n]  = alpha * sum_k Qop_b[m][k] * X[128 b + k][n]  (+ beta * add)
 //   side "right":  out[r][128 b + n]  = alpha * sum_k X[r][128 b + k] * Qop_b[k][n]  (+ beta * add)
@@ -106,7 +106,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_flag;
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
   const uint32_t full0 = smem_u32(&bars[0]), split0 = smem_u32(&bars[STAGES]), empty0 = smem_u32(&bars[2 * STAGES]);
   const uint32_t lfree0 = smem_u32(&bars[3 * STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[3 * STAGES + LSTAGES]), tempty0 = tfull0 + 16;   // per accumulator
@@ -141,7 +141,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   __syncthreads();
   tc_fence_after();
   grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
-  const uint32_t tmem_base = tmem_base_holder;
+  const uint32_t tmem_base = uniform(tmem_base_holder);
   volatile int* abortp = &abort_flag;
 
   if (warp == 0) {
@@ -198,7 +198,8 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    {
+      const uint32_t leader = elect_lane();
       const uint32_t idesc = instr_desc_tf32_mn(TILE, CH * TILE, 0, p.x.mn_major);
       const uint64_t dx0 = x_desc(smem_u32(smem), p.x.mn_major, 0), dl0 = x_desc(smem_u32(smem + LO_OFF), p.x.mn_major, 0);
       const uint64_t kinc = p.x.mn_major ? (1024u >> 4) : (32u >> 4);     // one k-step of 8 in the address field
@@ -211,60 +212,58 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       Unit u;
       for (int item = i0; ok && next_unit(item, i1, p.tiles, u); ++local) {
         if (u.b != cur_b) {
-          if (!mbar_wait(wfull, w_loads & 1u, abortp, p.status)) { ok = false; break; }
+          if (!mbar_wait_warp(wfull, w_loads & 1u, abortp, p.status)) { ok = false; break; }
           ++w_loads;
           cur_b = u.b;
           for (int piece = 0; piece < G::PIECES; ++piece)   // the block's pieces went through the ring
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
         const uint32_t as = DUAL ? 0u : (local & 1u), aphase = (DUAL ? local : local >> 1) & 1u;
-        if (!mbar_wait(tempty0 + 8 * as, aphase ^ 1u, abortp, p.status)) { ok = false; break; }
+        if (!mbar_wait_warp(tempty0 + 8 * as, aphase ^ 1u, abortp, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t tacc = tmem_base + as * (uint32_t)TILE;
         for (int kc = 0; kc < TILE / BK; ++kc) {
-          if (!mbar_wait(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+          if (!mbar_wait_warp(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
-          // One thread issues every MMA, so the instructions around each tcgen05.mma are what bounds the rate (a
-          // descriptor built from scratch per MMA costs more than the MMA takes to execute): the descriptors of
-          // stage 0 are formed once and only their address field moves.
+          // the descriptors of stage 0 are formed once and only their address field moves
           const uint64_t dx = dx0 + (uint64_t)(uint32_t)(stage * (STAGE_BYTES >> 4));
           const uint64_t dxl = dl0 + (uint64_t)(uint32_t)(lst * (STAGE_BYTES >> 4));
           const uint32_t w_hi = w_hi0 + (uint32_t)(kc * BK), w_lo = w_lo0 + (uint32_t)(kc * BK);
           if (p.one_pass) {
-            umma_tf32_ta(tacc, w_hi, dx, idesc, (uint32_t)(kc > 0));
+            umma_tf32_ta_w(leader, tacc, w_hi, dx, idesc, (uint32_t)(kc > 0));
 #pragma unroll
-            for (int k = 1; k < BK / 8; ++k) umma_tf32_ta_acc(tacc, w_hi + 8 * k, dx + k * kinc, idesc);
+            for (int k = 1; k < BK / 8; ++k) umma_tf32_ta_w(leader, tacc, w_hi + 8 * k, dx + k * kinc, idesc, 1u);
           } else if (p.right) {
             // low part of X (the M side of the untransposed product) first
-            umma_tf32_ta(tacc, w_hi, dxl, idesc, (uint32_t)(kc > 0));
-            umma_tf32_ta_acc(tacc, w_lo, dx, idesc);
-            umma_tf32_ta_acc(tacc, w_hi, dx, idesc);
+            umma_tf32_ta_w(leader, tacc, w_hi, dxl, idesc, (uint32_t)(kc > 0));
+            umma_tf32_ta_w(leader, tacc, w_lo, dx, idesc, 1u);
+            umma_tf32_ta_w(leader, tacc, w_hi, dx, idesc, 1u);
 #pragma unroll
             for (int k = 1; k < BK / 8; ++k) {
-              umma_tf32_ta_acc(tacc, w_hi + 8 * k, dxl + k * kinc, idesc);
-              umma_tf32_ta_acc(tacc, w_lo + 8 * k, dx + k * kinc, idesc);
-              umma_tf32_ta_acc(tacc, w_hi + 8 * k, dx + k * kinc, idesc);
+              umma_tf32_ta_w(leader, tacc, w_hi + 8 * k, dxl + k * kinc, idesc, 1u);
+              umma_tf32_ta_w(leader, tacc, w_lo + 8 * k, dx + k * kinc, idesc, 1u);
+              umma_tf32_ta_w(leader, tacc, w_hi + 8 * k, dx + k * kinc, idesc, 1u);
             }
           } else {
-            umma_tf32_ta(tacc, w_lo, dx, idesc, (uint32_t)(kc > 0));
-            umma_tf32_ta_acc(tacc, w_hi, dxl, idesc);
-            umma_tf32_ta_acc(tacc, w_hi, dx, idesc);
+            umma_tf32_ta_w(leader, tacc, w_lo, dx, idesc, (uint32_t)(kc > 0));
+            umma_tf32_ta_w(leader, tacc, w_hi, dxl, idesc, 1u);
+            umma_tf32_ta_w(leader, tacc, w_hi, dx, idesc, 1u);
 #pragma unroll
             for (int k = 1; k < BK / 8; ++k) {
-              umma_tf32_ta_acc(tacc, w_lo + 8 * k, dx + k * kinc, idesc);
-              umma_tf32_ta_acc(tacc, w_hi + 8 * k, dxl + k * kinc, idesc);
-              umma_tf32_ta_acc(tacc, w_hi + 8 * k, dx + k * kinc, idesc);
+              umma_tf32_ta_w(leader, tacc, w_lo + 8 * k, dx + k * kinc, idesc, 1u);
+              umma_tf32_ta_w(leader, tacc, w_hi + 8 * k, dxl + k * kinc, idesc, 1u);
+              umma_tf32_ta_w(leader, tacc, w_hi + 8 * k, dx + k * kinc, idesc, 1u);
             }
           }
-          umma_commit(empty0 + 8 * stage);   // frees the raw chunk and the low-part chunk once these MMAs have read them
-          umma_commit(lfree0 + 8 * lst);
+          umma_commit_w(leader, empty0 + 8 * stage);   // frees the raw chunk and the low-part chunk once these MMAs have read them
+          umma_commit_w(leader, lfree0 + 8 * lst);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
           if (++lst == LSTAGES) { lst = 0; lphase ^= 1; }
         }
         if (!ok) break;
-        umma_commit(tfull0 + 8 * as);
+        umma_commit_w(leader, tfull0 + 8 * as);
         // the last tiles of this wrapper block: tensor memory may be rewritten once these MMAs have read it
-        if (item < i1 && item / p.tiles != u.b) umma_commit(wfree);
+        if (item < i1 && item / p.tiles != u.b) umma_commit_w(leader, wfree);
       }
       (void)lphase;
     }
