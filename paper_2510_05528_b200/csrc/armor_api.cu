@@ -469,6 +469,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
   const bool adam = (c->cfg.ab_step == ARMOR_AB_ADAM);
   const int sweeps = c->cfg.mask_sweeps > 0 ? c->cfg.mask_sweeps : 1;
   const bool carry_P = (c->cfg.h_mode == ARMOR_H_FULL) && !adam;
+  const bool late_P = carry_P && (ph & ARMOR_PHASE_B) && (ph & ARMOR_PHASE_S);   // P's moves of the B-step and the S-step together
   if (!adam && c->cfg.ab_step == ARMOR_AB_EXACT && (ph & ARMOR_PHASE_B) && n_iters > 0) {
     st = launch_hjj_inverse(c, s);
     if (st != ARMOR_OK) return st;
@@ -581,8 +582,9 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       bd_left_dual(c, A, c->Tmp, c->E, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
       if (b_gd) launch_stage(c, is, 8, nullptr, 0, 0, s, c->partials, nq, SC_Q_B);
       else launch_stage(c, is, 2, c->partblk, DELTA_PARTS * nbi, nbi, s, c->partials, nq, SC_Q_B);
-      // B += tau Delta, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
-      launch_axpy_multi(c, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
+      // B += tau Delta, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch.  (With a core step P moves
+      // there by both steps: nothing reads it in between.)
+      launch_axpy_multi(c, c->EH, c->VH, -1.f, c->wn, carry_P && !late_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
                         (int64_t)nbi * db * db, SC_TAU_B, s);
     } else if (!adam) {
       launch_stage(c, is, 2, nullptr, 0, 0, s);
@@ -599,11 +601,13 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
         launch_masked_copy(c, c->Gam, M, c->U, nrm_part, s);
         n_nrm = ARMOR_DOT_BLOCKS;
       }
-      st = bd_right_H(c, c->U, B, H, c->Tmp, c->E, s);                               // R = Gamma_M B, R H_w
+      // (the B-step's R H_w stays in E until P has moved by it; T is free from the A-step on)
+      float* const RH = late_P ? c->T : c->E;
+      st = bd_right_H(c, c->U, B, H, c->Tmp, RH, s);                                 // R = Gamma_M B, R H_w
       if (st != ARMOR_OK) return st;
       // V H_w = A (R H_w) and q = <V H_w, V> with V = A Gamma_M B
       int nq = 0;
-      bd_left_dual(c, A, c->Tmp, c->E, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
+      bd_left_dual(c, A, c->Tmp, RH, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
       const bool beta_step = (c->cfg.s_step == ARMOR_S_BETA);
       if (beta_step) {
         // the paper's step size (Eq. lrWprime): |A^T A|_F and |B H_w B^T|_F  (these dot products reuse the
@@ -624,7 +628,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S,
                    nrm_part, n_nrm, SC_NRM_S);
       // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
-      launch_axpy_multi(c, S, c->U, 1.f, c->wn, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, c->E, 1.f, c->wn, SC_TAU_S, s);
+      launch_axpy_multi(c, S, c->U, 1.f, c->wn, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, RH, 1.f, c->wn, SC_TAU_S, s,
+                        late_P ? c->E : nullptr, SC_TAU_B);
     } else if (!adam) {
       launch_stage(c, is, 3, nullptr, 0, 0, s);
     }

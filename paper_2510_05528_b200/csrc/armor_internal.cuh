@@ -369,7 +369,7 @@ void launch_masked_copy(armor_ctx* c, const float* Gam, const uint8_t* M, float*
 void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slot, float sign,
                       cudaStream_t s);
 void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64_t n0, float* y1, const float* x1, float s1,
-                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s);                                       // y += sign * sc[slot] * x
+                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s, const float* x2_before = nullptr, int slot_before = 0);                                       // y += sign * sc[slot] * x
 void launch_init(armor_ctx* c, const float* W, const float* H, float* Wbar, float* r1, float* r2,
                  float* A, float* B, float* S, uint8_t* M, cudaStream_t s);
 // st: base of the iteration records (the kernels add c->it_dev), or null

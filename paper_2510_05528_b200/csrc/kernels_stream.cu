@@ -160,22 +160,35 @@ __global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* __restrict__ y, c
   }
 }
 
-// the same for up to three arrays that move by the same step: one launch
+// the same for up to three arrays that move by the same step: one launch.  The last may make an earlier step on the way
+// (y += sc[slot_before] x_before first): the two moves of an array that nothing reads in between cost one read and one write of
+// it less.
 struct AxpyTerm { float4* y; const float4* x; float sign; int64_t n4; };
-__global__ void __launch_bounds__(NT) axpy_multi_slot_kernel(AxpyTerm t0, AxpyTerm t1, AxpyTerm t2, int n_terms, int64_t n4,
-                                                             const double* sc, int slot) {
+__device__ __forceinline__ float4 axpy4(float a, const float4 v, const float4 u) {
+  return make_float4(fmaf(a, v.x, u.x), fmaf(a, v.y, u.y), fmaf(a, v.z, u.z), fmaf(a, v.w, u.w));
+}
+template <int TERMS, bool BEFORE>
+__global__ void __launch_bounds__(NT) axpy_multi_slot_kernel(AxpyTerm t0, AxpyTerm t1, AxpyTerm t2, int64_t n4, const double* sc,
+                                                             int slot, const float4* x_before, int slot_before) {
   grid_begin();
-  const float a = (float)sc[slot];
-  if (a == 0.f) return;
+  const float a = (float)sc[slot], ab = BEFORE ? (float)sc[slot_before] : 0.f;
+  if (a == 0.f && ab == 0.f) return;               // (a zero step: y stays bit for bit)
   const AxpyTerm t[3] = {t0, t1, t2};
   for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) {
+    float4 u[TERMS], v[TERMS], w = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      if (k >= n_terms) break;
+    for (int k = 0; k < TERMS; ++k) {
+      u[k] = v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i < t[k].n4) { u[k] = t[k].y[i]; v[k] = t[k].x[i]; }
+    }
+    if (BEFORE && i < t[TERMS - 1].n4) w = x_before[i];
+#pragma unroll
+    for (int k = 0; k < TERMS; ++k) {
       if (i >= t[k].n4) continue;
-      const float ak = t[k].sign * a;
-      const float4 u = t[k].y[i], v = t[k].x[i];
-      t[k].y[i] = make_float4(fmaf(ak, v.x, u.x), fmaf(ak, v.y, u.y), fmaf(ak, v.z, u.z), fmaf(ak, v.w, u.w));
+      const bool before = BEFORE && k == TERMS - 1 && ab != 0.f;
+      if (before) u[k] = axpy4(ab, w, u[k]);
+      if (a != 0.f) u[k] = axpy4(t[k].sign * a, v[k], u[k]);
+      if (a != 0.f || before) t[k].y[i] = u[k];
     }
   }
 }
@@ -783,9 +796,11 @@ void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slo
   c->launches++;
 }
 
-// y_k += sign_k * sc[slot] * x_k for up to three pairs of lengths n_k (a pair with y == nullptr is skipped)
+// y_k += sign_k * sc[slot] * x_k for up to three pairs of lengths n_k (a pair with y == nullptr is skipped); with x2_before the
+// third, which then exists, takes y2 += sc[slot_before] * x2_before first
 void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64_t n0, float* y1, const float* x1, float s1,
-                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s) {
+                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s,
+                       const float* x2_before, int slot_before) {
   AxpyTerm t[3];
   int k = 0;
   if (y0) t[k++] = {(float4*)y0, (const float4*)x0, s0, n0 / 4};
@@ -796,8 +811,12 @@ void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64
   double elems = 0.0;
   for (int j = 0; j < k; ++j) { n4 = t[j].n4 > n4 ? t[j].n4 : n4; elems += 4.0 * (double)t[j].n4; }
   for (int j = k; j < 3; ++j) t[j] = t[0];
-  KTimer kt(c, n4 >= (1 << 20) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * elems, s);
-  launch_dependent(axpy_multi_slot_kernel, grid_for(n4), NT, 0, s, t[0], t[1], t[2], k, n4, c->sc, slot);
+  KTimer kt(c, n4 >= (1 << 20) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * elems + (x2_before ? 4.0 * (double)n2 : 0.0), s);
+  const float4* xb = reinterpret_cast<const float4*>(x2_before);
+  if (xb) launch_dependent(axpy_multi_slot_kernel<3, true>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
+  else if (k == 3) launch_dependent(axpy_multi_slot_kernel<3, false>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
+  else if (k == 2) launch_dependent(axpy_multi_slot_kernel<2, false>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
+  else launch_dependent(axpy_multi_slot_kernel<1, false>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
   c->launches++;
 }
 
