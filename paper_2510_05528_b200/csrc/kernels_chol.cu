@@ -6,23 +6,22 @@
 // A failed factorisation leaves A unchanged / writes zeros and raises failflag[block].
 //
 // One CTA factorises one d_block x d_block matrix in shared memory and solves for a slice of the right-hand sides beside it;
-// the slices of a block repeat the factorisation.  What bounds this is the chain of pivots (about 150 cycles each in the
-// factorisation, 140 in a solve), next to it fp64 conversions, which cost as much as dozens of fp32 instructions and are
-// kept out of the sums:
+// the slices of a block repeat the factorisation.  What bounds this is the chain of pivots (130 to 190 cycles each in the
+// factorisation, 70 in a solve), what shared memory returns to the small products (a 16-byte broadcast costs four cycles), and
+// fetching instructions: a launch meets its code cold, about 100 cycles a line of eight, so the loops stay rolled.  fp64
+// conversions cost as much as dozens of fp32 instructions and are kept out of the sums:
 //   storage: panels of 32 columns, rows of 32 floats, the 16-byte units of a row swizzled so that eight lanes reading the
 //            same unit of consecutive rows, or of every fourth row, or all units of one row, meet no bank conflict; G
 //            arrives by cp.async, and everything below reads four columns per access.
 //   factor : blocked left-looking Cholesky.  A panel receives the contributions of the earlier panels as one small product
-//            (fp32 over 32 terms, panels added as unevaluated pairs of floats, one rounding).  Then every warp that owns 32
-//            of its rows repeats the elimination of the diagonal block in registers (lane = row) and carries its own rows
-//            along, so that no second pass over the rows below follows.
-//   solve  : left-looking with the same two-level sums, a lane per right-hand side, a warp per four rows of a block of 32:
-//            every warp works in every step.
+//            (fp32 over 32 terms, panels added as unevaluated pairs of floats, one rounding), then eliminate_panel.
+//   solve  : left-looking with the same two-level sums, see solve_block.
 // Measured and left: pivots eight at a time with every thread factorising the 8 x 8 block (elimination 2 x slower), rows
-// or right-hand sides moving down one register per pivot in a rolled loop (3 x and 1.4 x), solutions handed round by shuffles
-// (1.2 x).
-// A launch, d_block 128: 32 blocks over 4 CTAs each 57 us (79 before), 112 blocks 86 us (85); d_block 256, a 28672 x 8192
-// layer's launches of 112 and 32 blocks 469 us on average (545).
+// or right-hand sides moving down one register per pivot in a rolled loop (3 x and 1.4 x); two CTAs per SM with fewer right-hand
+// sides each (40 blocks: 59 us a launch against 52).
+// A launch, d_block 128: 32 blocks over 4 CTAs each 48.6 us (62.2 with the panel's elimination unrolled), 40 blocks over 2 to 4 CTAs
+// 51.7 (65.1), 112 and 32 blocks 60.4 on average (74.4); d_block 32, 8 blocks 16 k cycles (22 k); d_block 256, a 28672 x 8192
+// layer's launches of 112 and 32 blocks 480 to 505 us on average.
 #include "armor_internal.cuh"
 
 namespace {
@@ -57,63 +56,77 @@ __device__ __forceinline__ float pair_sub_from(float v, const Pair& a) {
   return s + (((v - (s - bb)) - (a.hi + bb)) - a.lo);
 }
 
-// The panel's 32 columns, eliminated right-looking with rows in registers: ad is the lane's row of the diagonal block (the
-// same in every warp that takes part), ab its row of the warp's own 32 rows below (`below` groups of 32 rows); nothing in
-// the chain of pivots goes through memory.  Called by the whole CTA; one copy serves every block size.
-__device__ __noinline__ void eliminate_panel(float* P, float* invd, int below, int* s_fail) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool mine = warp < below;
-  const bool takes_part = mine || warp == 0;
-  const int rb = NB * (warp + 1) + lane;
-  float ad[NB], ab[NB];
-  if (takes_part) {
+// The panel's 32 columns, eliminated right-looking, eight at a time.  Warp 0 holds the eight columns of the diagonal block in
+// registers (lane = row) and takes the pivots; behind a barrier warp w > 0 does the same to the 32 rows below it that it owns
+// (group w - 1 of `below`), with the factors and reciprocals that warp 0 has left, and every warp brings the panel's later
+// columns of its rows up to date.  An element meets the pivots in ascending order, one fused multiply-add each.  Rolled over
+// the four groups of eight and over the columns behind them, because what bounded this was fetching instructions: with all 32
+// columns in registers and 32 pivots unrolled (30 KB of code) a launch's first panel took 31 k cycles and the others 5.5 k.
+__device__ __forceinline__ void later_columns(float* P, int row, int c0, const float (&l)[8]) {
+#pragma unroll 1
+  for (int u = c0 / 4 + 2; u < NB / 4; ++u) {
+    float4* dst = reinterpret_cast<float4*>(P + unit(row, u));
+    const float4 v = *dst;
+    float w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int u = 0; u < NB / 4; ++u) {
-      const float4 v = ld4(P + unit(lane, u));
-      const float4 w = mine ? ld4(P + unit(rb, u)) : make_float4(0.f, 0.f, 0.f, 0.f);
-      ad[4 * u] = v.x; ad[4 * u + 1] = v.y; ad[4 * u + 2] = v.z; ad[4 * u + 3] = v.w;   // (j > lane: never used)
-      ab[4 * u] = w.x; ab[4 * u + 1] = w.y; ab[4 * u + 2] = w.z; ab[4 * u + 3] = w.w;
+    for (int q = 0; q < 4; ++q) {
+      const float4 a = ld4(P + unit(4 * u + q, c0 / 4)), b = ld4(P + unit(4 * u + q, c0 / 4 + 1));
+      const float m[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int k = 0; k < 8; ++k) w[q] = fmaf(-l[k], m[k], w[q]);
     }
+    *dst = make_float4(w[0], w[1], w[2], w[3]);
   }
-  __syncthreads();                                          // every warp has read the block warp 0 is about to replace
-  if (takes_part) {
-    bool bad = false;
-    float dg = 1.f;
-    float akk = __shfl_sync(0xffffffffu, ad[0], 0);
-#pragma unroll
-    for (int k = 0; k < NB; ++k) {
-      bad |= !(akk > 0.f) | !isfinite(akk);
-      // 1 / sqrt(a): hardware estimate refined by one Newton step
-      float inv = rsqrtf(akk);
-      inv = inv * fmaf(-0.5f * akk * inv, inv, 1.5f);
-      const float ld = ad[k] * inv, lb = ab[k] * inv;
-      ad[k] = ld;
-      ab[k] = lb;
-      if (lane == k) dg = ld;
-      // the next pivot needs lane k + 1's own multiplier only: it goes ahead of the rest of the column
-      if (k + 1 < NB) akk = __shfl_sync(0xffffffffu, fmaf(-ld, ld, ad[k + 1]), k + 1);
-#pragma unroll
-      for (int j = k + 1; j < NB; ++j) {
-        const float ljk = __shfl_sync(0xffffffffu, ld, j);
-        ad[j] = fmaf(-ld, ljk, ad[j]);
-        ab[j] = fmaf(-lb, ljk, ab[j]);
-      }
+}
+__device__ __noinline__ void eliminate_panel(float* P, float* invd, int below, int* s_fail) {
+  __shared__ float s_inv[NB];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int row = NB * warp + lane;
+  bool bad = false;
+  float dg = 1.f;
+#pragma unroll 1
+  for (int c0 = 0; c0 < NB; c0 += 8) {
+    float l[8];
+    if (warp <= below) {
+      const float4 a = ld4(P + unit(row, c0 / 4)), b = ld4(P + unit(row, c0 / 4 + 1));
+      l[0] = a.x; l[1] = a.y; l[2] = a.z; l[3] = a.w; l[4] = b.x; l[5] = b.y; l[6] = b.z; l[7] = b.w;
     }
-    if (bad) {
-      if (lane == 0) *s_fail = 1;
-    } else {
-      if (warp == 0) {
-        invd[lane] = 1.f / dg;
+    if (warp == 0) {
+      float akk = __shfl_sync(0xffffffffu, l[0], c0);
 #pragma unroll
-        for (int u = 0; u < NB / 4; ++u)
-          *reinterpret_cast<float4*>(P + unit(lane, u)) = make_float4(ad[4 * u], ad[4 * u + 1], ad[4 * u + 2], ad[4 * u + 3]);
-      }
-      if (mine) {
+      for (int k = 0; k < 8; ++k) {
+        bad |= !(akk > 0.f) | !isfinite(akk);
+        // 1 / sqrt(a): hardware estimate refined by one Newton step
+        float inv = rsqrtf(akk);
+        inv = inv * fmaf(-0.5f * akk * inv, inv, 1.5f);
+        const float ld = l[k] * inv;
+        l[k] = ld;
+        if (lane == c0 + k) { dg = ld; s_inv[lane] = inv; }
+        // the next pivot needs lane k + 1's own multiplier only: it goes ahead of the rest of the column
+        if (k < 7) akk = __shfl_sync(0xffffffffu, fmaf(-ld, ld, l[k + 1]), c0 + k + 1);
 #pragma unroll
-        for (int u = 0; u < NB / 4; ++u)
-          *reinterpret_cast<float4*>(P + unit(rb, u)) = make_float4(ab[4 * u], ab[4 * u + 1], ab[4 * u + 2], ab[4 * u + 3]);
+        for (int j = k + 1; j < 8; ++j) l[j] = fmaf(-ld, __shfl_sync(0xffffffffu, ld, c0 + j), l[j]);
       }
+      *reinterpret_cast<float4*>(P + unit(row, c0 / 4)) = make_float4(l[0], l[1], l[2], l[3]);
+      *reinterpret_cast<float4*>(P + unit(row, c0 / 4 + 1)) = make_float4(l[4], l[5], l[6], l[7]);
     }
+    __syncthreads();
+    if (warp > 0 && warp <= below) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        l[k] *= s_inv[c0 + k];
+#pragma unroll
+        for (int j = k + 1; j < 8; ++j) l[j] = fmaf(-l[k], P[unit(c0 + j, (c0 + k) / 4) + (k & 3)], l[j]);
+      }
+      *reinterpret_cast<float4*>(P + unit(row, c0 / 4)) = make_float4(l[0], l[1], l[2], l[3]);
+      *reinterpret_cast<float4*>(P + unit(row, c0 / 4 + 1)) = make_float4(l[4], l[5], l[6], l[7]);
+    }
+    if (warp <= below) later_columns(P, row, c0, l);
+    __syncwarp();
+  }
+  if (warp == 0) {
+    if (bad) { if (lane == 0) *s_fail = 1; }
+    else invd[lane] = 1.f / dg;
   }
   __syncthreads();
 }
@@ -172,9 +185,12 @@ __device__ __forceinline__ void update_panel(float* Lp, const PanelMap& pm, int 
 }
 
 // Block kb's 32 unknowns of every right-hand side: x (in X, one column per right-hand side) becomes L^-1 x, or with T L^-T x.
-// Lane = right-hand side (G of them, 32 apart), warp = four rows.  First the solved blocks' share (forward: blocks before kb
-// with the rows of L; T: blocks after kb with its columns; in block order either way), then the block itself, four unknowns
-// at a time.  Called by the whole CTA.
+// First the solved blocks' share (forward: blocks before kb with the rows of L; T: blocks after kb with its columns; in block
+// order either way): lane = right-hand side (G of them, 32 apart), warp = four rows.  Then the block itself.  G 1: lane = unknown,
+// a warp takes four right-hand sides side by side and hands every solution round by a shuffle, without a barrier in the
+// chain of 32.  More right-hand sides: lanes and warps as before, four unknowns at a time with a barrier behind them (32 and
+// more shuffles an unknown cost more: 12 and 20 k cycles a CTA of 64 and 128 right-hand sides against 10.6 and 17.7, while 32 take
+// 16.9 against 18.5).  Called by the whole CTA.
 template <bool T, int G>
 __device__ __forceinline__ void solve_block(const float* Lp, const PanelMap& pm, const float* invd, float* X, int ldx, int kb) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, r0 = 4 * warp;
@@ -225,6 +241,44 @@ __device__ __forceinline__ void solve_block(const float* Lp, const PanelMap& pm,
       for (int m = 0; m < 4; ++m) y[g][m] = pair_sub_from(own[m * ldx + 32 * g], acc[g][m]);
   }
   const float* D = Lp + pm.off(kb);
+  if constexpr (G == 1) {
+    if (p_begin < p_end) {
+#pragma unroll
+      for (int m = 0; m < 4; ++m) own[m * ldx] = y[0][m];
+      __syncthreads();
+    }
+    float* x0 = X + (NB * kb + lane) * ldx + 4 * warp;
+    const float iv = invd[NB * kb + lane];
+    float z[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) z[i] = x0[i];
+#pragma unroll 1
+    for (int s = 0; s < NB / 4; ++s) {
+      const int u = T ? NB / 4 - 1 - s : s;
+      float l[4];                                               // what unknown 4 u + j contributes to this lane's
+      if (T) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) l[j] = D[unit(4 * u + j, lane >> 2) + (lane & 3)];
+      } else {
+        const float4 v = ld4(D + unit(lane, u));
+        l[0] = v.x; l[1] = v.y; l[2] = v.z; l[3] = v.w;
+      }
+#pragma unroll
+      for (int jj = 0; jj < 4; ++jj) {
+        const int j = T ? 3 - jj : jj, k = 4 * u + j;
+        const bool open = T ? lane < k : lane > k;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float x = __shfl_sync(0xffffffffu, z[i] * iv, k);
+          if (open) z[i] = fmaf(-l[j], x, z[i]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x0[i] = z[i] * iv;
+    __syncthreads();
+    return;
+  }
 #pragma unroll 1
   for (int s = 0; s < NB / 4; ++s) {
     const int u = T ? NB / 4 - 1 - s : s;                     // the warp whose four rows are solved now
