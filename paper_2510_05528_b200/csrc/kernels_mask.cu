@@ -171,13 +171,14 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
     {
       const bool lane_on = rl0 < rstep;
       float wbound = INFINITY;                                   // warp-uniform: the smallest key any lane holds
+      int best_rl = -1;                                          // row in the block of the thread's best group: it meets its
+                                                                 // groups in ascending order, so a tie stays with the first
       const int n_steps = (db + U * rstep - 1) / (U * rstep);    // the same for every lane: the shuffles below need all 32
       const int64_t row0 = (int64_t)bi * db + (lane_on ? rl0 : 0);
       const int64_t cg = (int64_t)bj * gpb + cl;
       const float* gp = Gam + row0 * d_in + cg * MG;
       const float* ap = alpha + row0;
-      uint64_t g = (uint64_t)row0 * (uint64_t)ng_row + (uint64_t)cg;
-      uint64_t ctr = t * n_groups_total + g;
+      uint64_t ctr = t * n_groups_total + (uint64_t)row0 * (uint64_t)ng_row + (uint64_t)cg;
       const uint64_t gstep = (uint64_t)rstep * (uint64_t)ng_row;
       const int64_t pstep = (int64_t)rstep * d_in;
       for (int step = 0, rl = rl0; step < n_steps; ++step, rl += U * rstep) {
@@ -215,7 +216,6 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
             if (select_mode == ARMOR_SELECT_L2_RANDOM) score = sqrtf(sq);
             else if (select_mode == ARMOR_SELECT_UNIFORM_RANDOM) score = 1.f;
             if (!(al[u] > 0.f)) score = 0.f;
-            const uint64_t gu = g + (uint64_t)u * gstep;
             float key = INFINITY;
             if (score > 0.f) {
               if (select_mode != ARMOR_SELECT_L1_GREEDY) {
@@ -229,20 +229,19 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
               } else {
                 key = -score;
               }
-              if (key < best_key || (key == best_key && gu < best_g)) { best_key = key; best_g = gu; }
+              if (key < best_key) { best_key = key; best_rl = rl + u * rstep; }
             }
             if (MULTI) s_keys[(rl + u * rstep) * gpb + cl] = key;
           }
         }
         gp += U * pstep;
         ap += U * rstep;
-        g += U * gstep;
         ctr += U * gstep;
         if (!MULTI) {
-          wbound = best_key;
-          for (int o = 16; o > 0; o >>= 1) wbound = fminf(wbound, __shfl_xor_sync(0xffffffffu, wbound, o));
+          asm volatile("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(wbound) : "f"(best_key));
         }
       }
+      if (best_rl >= 0) best_g = (uint64_t)((int64_t)bi * db + best_rl) * (uint64_t)ng_row + (uint64_t)cg;
     }
   }
   // arg-min over the CTA; ties go to the lower group index
@@ -470,31 +469,28 @@ __global__ void __launch_bounds__(NT) mask_quad_kernel(const float* Zsel, const 
   }
 }
 
-__global__ void mask_commit_kernel(const SelRec* sel, int nblocks, float* __restrict__ S,
-                                   uint8_t* __restrict__ M, int64_t d_in, int mg, const double* sc,
-                                   armor_iter_stats* st_base, const int64_t* it_dev) {
+// A thread per block (one CTA walking 3,584 blocks took 21 us).
+constexpr int COMMIT_NT = 64;
+__global__ void __launch_bounds__(COMMIT_NT) mask_commit_kernel(const SelRec* sel, int nblocks, float* __restrict__ S,
+                                                                uint8_t* __restrict__ M, int64_t d_in, int mg, const double* sc,
+                                                                armor_iter_stats* st_base, const int64_t* it_dev) {
   grid_begin();
-  armor_iter_stats* st = st_base ? st_base + *it_dev : nullptr;
-  __shared__ int changed;
-  if (threadIdx.x == 0) changed = 0;
-  __syncthreads();
-  const bool accept = sc[SC_ACCEPT] != 0.0;
-  int mine = 0;
-  if (accept) {
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-      const SelRec rec = sel[b];
-      if (!rec.valid) continue;
+  if (sc[SC_ACCEPT] == 0.0) return;
+  const int b = blockIdx.x * COMMIT_NT + threadIdx.x;
+  bool changed = false;
+  if (b < nblocks) {
+    const SelRec rec = sel[b];
+    if (rec.valid) {
       float* sp = S + (int64_t)rec.row * d_in + (int64_t)rec.cgrp * mg;
       for (int h = 0; h < mg / 4; ++h)
         *reinterpret_cast<float4*>(sp + 4 * h) =
             make_float4(rec.new_val[4 * h], rec.new_val[4 * h + 1], rec.new_val[4 * h + 2], rec.new_val[4 * h + 3]);
       M[(int64_t)rec.row * (d_in / mg) + rec.cgrp] = (uint8_t)rec.new_mask;
-      mine += (rec.new_mask != rec.old_mask) ? 1 : 0;
+      changed = rec.new_mask != rec.old_mask;
     }
   }
-  atomicAdd(&changed, mine);
-  __syncthreads();
-  if (threadIdx.x == 0 && st) st->groups_changed += changed;   // summed over the sweeps of the iteration
+  const int n = __popc(__ballot_sync(0xffffffffu, changed));
+  if (st_base && n && (threadIdx.x & 31) == 0) atomicAdd(&st_base[*it_dev].groups_changed, n);   // summed over the sweeps of the iteration
 }
 
 // The accepted group updates change T H_w = S B H_w by the rows (delta^T B_j[group rows, :]) H_w[j-th block
@@ -714,7 +710,8 @@ void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const f
 
 void launch_mask_commit(armor_ctx* c, float* S, uint8_t* M, armor_iter_stats* st, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  launch_dependent(mask_commit_kernel, 1, 256, 0, s, c->sel, c->nbo * c->nbi * c->kg, S, M, c->d_in, c->cfg.m_group, c->sc, st,
+  const int n = c->nbo * c->nbi * c->kg;
+  launch_dependent(mask_commit_kernel, (n + COMMIT_NT - 1) / COMMIT_NT, COMMIT_NT, 0, s, c->sel, n, S, M, c->d_in, c->cfg.m_group, c->sc, st,
                                        c->it_dev);
   c->launches++;
 }
