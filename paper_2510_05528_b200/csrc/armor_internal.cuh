@@ -161,10 +161,11 @@ __device__ __forceinline__ void grid_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
-// Kernels of more CTAs than this start behind their predecessor as ever: CTAs of a streaming kernel that wait in their
-// hundreds beside the products slow those down (a 4096 x 4096 layer's diagonal Adam iterations 6,561 us with this limit,
-// 6,775 without, 6,626 with no dependent launches; limits of 1, 148 and 1,100 CTAs: 256 x 256 layer 2,886, 2,767 and 2,746 us).
-constexpr int64_t DEPENDENT_CTAS = 592;
+// Kernels of more threads than this start behind their predecessor as ever: CTAs of a streaming kernel that wait in their
+// hundreds beside the products slow those down (a 4096 x 4096 layer's diagonal Adam iterations with a limit of 592 CTAs of 256
+// threads 6,561 us, 6,775 without a limit, 6,626 with no dependent launches; limits of 1, 148 and 1,100 CTAs: 256 x 256 layer 2,886,
+// 2,767 and 2,746 us).
+constexpr int64_t DEPENDENT_THREADS = 592 * 256;
 template <typename... Params, typename... Args>
 inline void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
   cudaLaunchConfig_t cfg{};
@@ -172,7 +173,7 @@ inline void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, s
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z <= DEPENDENT_CTAS ? 1 : 0;
+  cfg.attrs = at; cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z * block.x * block.y <= DEPENDENT_THREADS ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, Params(args)...);   // (an error is found by the call's cudaGetLastError)
 }
 

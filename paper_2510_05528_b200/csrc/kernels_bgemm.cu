@@ -338,6 +338,109 @@ __global__ void __launch_bounds__(NT) bgemm_small_kernel(BGemm g) {
   }
 }
 
+// The same tiles where several share an SM: 64 threads with 4 x 4 sums, 32 k at once.  A sum then takes half as much of shared
+// memory's 128 bytes a cycle (16 cycles a k and tile against 32), which is what bounds it there.  The same additions again.
+constexpr int MID_NT = 64, MID_K = 32;
+
+template <bool A_KFAST, bool B_NFAST>
+__global__ void __launch_bounds__(MID_NT) bgemm_mid_kernel(BGemm g) {
+  grid_begin();
+  __shared__ __align__(16) float As[MID_K * SM_T];
+  __shared__ __align__(16) float Bs[MID_K * SM_T];
+  const int m0 = blockIdx.y * SM_T, n0 = blockIdx.x * SM_T;
+  int64_t oa, ob, oc, od;
+  batch_offsets(g, blockIdx.z, oa, ob, oc, od);
+  const float* A = g.A + oa;
+  const float* B = g.B + ob;
+  const int tid = threadIdx.x;
+  float4 ra[4], rb[4];
+  // element e of a thread of a 32 x 32 piece, along whichever index is contiguous: row (or column) x, four k or four x from there
+  auto place = [&](int e, bool kfast, int& x, int& k) {
+    const int hi = (tid >> 3) + 8 * e, lo = 4 * (tid & 7);
+    if (kfast) { x = hi; k = lo; } else { k = hi; x = lo; }
+  };
+  auto fetch_one = [&](const float* P, int64_t sx, int64_t sk, int x0, int X, int k0, int e, bool kfast) {
+    int x, k;
+    place(e, kfast, x, k);
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (x0 + x < X && k0 + k < g.K) v = *reinterpret_cast<const float4*>(kfast ? P + (int64_t)(x0 + x) * sx + (k0 + k) : P + (int64_t)(k0 + k) * sk + (x0 + x));
+    return v;
+  };
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      ra[e] = fetch_one(A, g.sAm, g.sAk, m0, g.M, k0, e, A_KFAST);
+      rb[e] = fetch_one(B, g.sBn, g.sBk, n0, g.N, k0, e, !B_NFAST);
+    }
+  };
+  auto stash_one = [&](float* P, const float4& v, int e, bool kfast) {
+    int x, k;
+    place(e, kfast, x, k);
+    float* q = P + sm_unit(k, x >> 2) + (x & 3);
+    if (kfast) { q[0] = v.x; q[SM_T] = v.y; q[2 * SM_T] = v.z; q[3 * SM_T] = v.w; }    // (the four k share a swizzle)
+    else *reinterpret_cast<float4*>(q) = v;
+  };
+  const int tx = tid & 7, ty = tid >> 3;                  // columns 4 tx .., rows 4 ty ..
+  const int kc = g.K / (g.ksplit > 1 ? g.ksplit : 1);     // a piece of the contraction
+  float acc[4][4] = {}, sum[4][4] = {};
+  int left = kc;
+  bool first = true;
+  fetch(0);
+#pragma unroll 1
+  for (int k0 = 0; k0 < g.K; k0 += MID_K) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) { stash_one(As, ra[e], e, A_KFAST); stash_one(Bs, rb[e], e, !B_NFAST); }
+    __syncthreads();
+    if (k0 + MID_K < g.K) fetch(k0 + MID_K);
+    const int kn = min(MID_K, g.K - k0);
+#pragma unroll 1
+    for (int k = 0; k < kn;) {
+      const int run = min(kn - k, left);                  // a multiple of 16
+#pragma unroll 2
+      for (const int e = k + run; k < e; k += 4) {
+        const float* pa = As + sm_unit(k, ty);            // (four k share a swizzle)
+        const float* pb = Bs + sm_unit(k, tx);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float4 a4 = *reinterpret_cast<const float4*>(pa + t * SM_T), b4 = *reinterpret_cast<const float4*>(pb + t * SM_T);
+          const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+      }
+      left -= run;
+      if (left == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) { sum[i][j] = first ? acc[i][j] : sum[i][j] + acc[i][j]; acc[i][j] = 0.f; }
+        first = false;
+        left = kc;
+      }
+    }
+    __syncthreads();
+  }
+  const int n = n0 + 4 * tx;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int m = m0 + 4 * ty + i;
+    if (m >= g.M || n >= g.N) continue;                   // (N is a multiple of 4)
+    float4 v = make_float4(g.alpha * sum[i][0], g.alpha * sum[i][1], g.alpha * sum[i][2], g.alpha * sum[i][3]);
+    if (g.D) {
+      const float4 d = *reinterpret_cast<const float4*>(g.D + od + (int64_t)m * g.sDm + n);
+      v.x = fmaf(g.beta, d.x, v.x); v.y = fmaf(g.beta, d.y, v.y);
+      v.z = fmaf(g.beta, d.z, v.z); v.w = fmaf(g.beta, d.w, v.w);
+    }
+    *reinterpret_cast<float4*>(g.C + oc + (int64_t)m * g.sCm + n) = v;
+  }
+}
+
+// Tiles per SM from which that kernel takes them: 40 products of 128^3 (4.3 a SM) 14.0 -> 11.4 us; with at most one a SM 256 threads are
+// the faster.
+constexpr int MID_TILES = 2;
+
 // The share of the chip's lanes that 128 x 128 tiles would keep busy: tiles per SM, times the part of a tile that holds
 // elements.  Below a half the small tiles are faster.
 inline bool small_tiles_better(const BGemm& g) {
@@ -398,6 +501,14 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
   if (g.ksplit > 1 && !tile_kernel_ok(g, a_kfast, b_nfast)) g.ksplit = 1;
   if (tile_kernel_ok(g, a_kfast, b_nfast) && small_tiles_better(g)) {
     dim3 grid((g.N + SM_T - 1) / SM_T, (g.M + SM_T - 1) / SM_T, g.batch);
+    if ((int64_t)grid.x * grid.y * grid.z >= (int64_t)MID_TILES * c->n_sm) {
+      if (a_kfast && b_nfast) launch_dependent(bgemm_mid_kernel<true, true>, grid, MID_NT, 0, s, g);
+      else if (a_kfast && !b_nfast) launch_dependent(bgemm_mid_kernel<true, false>, grid, MID_NT, 0, s, g);
+      else if (!a_kfast && b_nfast) launch_dependent(bgemm_mid_kernel<false, true>, grid, MID_NT, 0, s, g);
+      else launch_dependent(bgemm_mid_kernel<false, false>, grid, MID_NT, 0, s, g);
+      c->launches++;
+      return;
+    }
     if (a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<true, true>, grid, NT, 0, s, g);
     else if (a_kfast && !b_nfast) launch_dependent(bgemm_small_kernel<true, false>, grid, NT, 0, s, g);
     else if (!a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<false, true>, grid, NT, 0, s, g);
