@@ -217,7 +217,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
 
 template <int DB, bool SUM>
 __global__ void __launch_bounds__(256)
-fwd_small_kernel(const void* __restrict__ X, int pieces, const __nv_bfloat16* __restrict__ Q, __nv_bfloat16* __restrict__ out,
+fwd_small_kernel(const void* X, int pieces, const __nv_bfloat16* Q, __nv_bfloat16* __restrict__ out,
                  int rows, int64_t d) {
   constexpr int LD = DB * 2 + 64;                     // bytes per staged token: eight lanes of a phase hit eight banks
   __shared__ __align__(16) uint8_t tok[16 * LD];
@@ -225,13 +225,16 @@ fwd_small_kernel(const void* __restrict__ X, int pieces, const __nv_bfloat16* __
   const int64_t n0 = (int64_t)blockIdx.x * 128 + warp * 16;
   const int64_t kbase = (int64_t)blockIdx.x * 128 / DB * DB;   // first column of X of the block these columns belong to
   const int r0 = blockIdx.y * 16;
+  // The first product of a pass waits before anything else and lets the core product in only then: that one fetches the packed core
+  // before its own wait, and what wrote the core may be the kernel before this one.  The last product's weights are there.
+  if (!SUM) grid_dependency_wait();
   grid_launch_dependents();
   uint4 w[2][DB / 32];
 #pragma unroll
   for (int nt = 0; nt < 2; ++nt)
 #pragma unroll
     for (int ch = 0; ch < DB / 32; ++ch)
-      w[nt][ch] = __ldg(reinterpret_cast<const uint4*>(Q + (n0 + 4 * (g >> 1) + 2 * nt + (g & 1)) * DB + ch * 32 + 8 * t));
+      w[nt][ch] = *reinterpret_cast<const uint4*>(Q + (n0 + 4 * (g >> 1) + 2 * nt + (g & 1)) * DB + ch * 32 + 8 * t);
   if (SUM) grid_dependency_wait();
 #pragma unroll
   for (int e = threadIdx.x; e < 16 * DB / 8; e += 256) {
@@ -341,7 +344,7 @@ armor_status launch_fwd_block(armor_ctx* c, const void* X, const void* Q, void* 
 }
 
 // The same for up to ARMOR_SMALL_TOKENS rows.  pieces == 0: X is bf16 [rows][d]; otherwise X holds that many fp32 arrays
-// [rows][d] whose sum, rounded to bf16, is the operand, and the launch may overlap the kernel that writes them.
+// [rows][d] whose sum, rounded to bf16, is the operand.  Either way a dependent launch.
 armor_status launch_fwd_small(armor_ctx* c, const void* X, int pieces, const void* Q, void* out, int64_t rows, int64_t d,
                               cudaStream_t s) {
   if (!fwd_block_ok(c) || rows <= 0 || rows > ARMOR_SMALL_TOKENS || d % 128) return ARMOR_ERR_UNSUPPORTED;
@@ -351,7 +354,7 @@ armor_status launch_fwd_small(armor_ctx* c, const void* X, int pieces, const voi
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = pieces > 0 ? 1 : 0;
+  cfg.attrs = at; cfg.numAttrs = 1;
   const __nv_bfloat16* q = static_cast<const __nv_bfloat16*>(Q);
   __nv_bfloat16* o = static_cast<__nv_bfloat16*>(out);
   const int n = (int)rows;
