@@ -19,9 +19,9 @@
 // Measured and left: pivots eight at a time with every thread factorising the 8 x 8 block (elimination 2 x slower), rows
 // or right-hand sides moving down one register per pivot in a rolled loop (3 x and 1.4 x); two CTAs per SM with fewer right-hand
 // sides each (40 blocks: 59 us a launch against 52).
-// A launch, d_block 128: 32 blocks over 4 CTAs each 48.6 us (62.2 with the panel's elimination unrolled), 40 blocks over 2 to 4 CTAs
-// 51.7 (65.1), 112 and 32 blocks 60.4 on average (74.4); d_block 32, 8 blocks 16 k cycles (22 k); d_block 256, a 28672 x 8192
-// layer's launches of 112 and 32 blocks 480 to 505 us on average.
+// A launch, d_block 128: 32 blocks over 4 CTAs each 46.5 us (62.2 with the panel's elimination unrolled and a row a thread in the last
+// panels' updates), 40 blocks over 2 to 4 CTAs 50.6 (65.1), 112 and 32 blocks 59.4 on average (74.4); d_block 32, 8 blocks 16 k cycles
+// (22 k); d_block 256, a 28672 x 8192 layer's launches of 112 and 32 blocks 449 us on average (505 to 520).
 #include "armor_internal.cuh"
 
 namespace {
@@ -131,9 +131,11 @@ __device__ __noinline__ void eliminate_panel(float* P, float* invd, int below, i
   __syncthreads();
 }
 
-// panel kb (at P, first row c0) -= sum_{p < c0} L(i, p) L(k, p): TR x 4 elements per thread, rows TR*tr.., columns 4*tc..
-template <int TR>
+// panel kb (at P, first row c0) -= sum_{p < c0} L(i, p) L(k, p): 4 x 4 elements per thread, rows TR*tr.., columns 4*tc..  (Also
+// where that leaves most warps without a tile: with one row a thread the panels of 64 and 32 rows of a block of 128 took 6.3 and
+// 4.7 k cycles, what shared memory needs to return five 16-byte accesses per 16 multiply-adds.)
 __device__ __forceinline__ void update_panel(float* Lp, const PanelMap& pm, int kb) {
+  constexpr int TR = 4;
   const int db = pm.db, c0 = NB * kb;
   float* P = Lp + pm.off(kb);
   const int ntiles = ((db - c0) / TR) * (NB / 4);
@@ -393,8 +395,7 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
   // ---- blocked Cholesky
   for (int kb = 0; kb < np; ++kb) {
     if (kb > 0) {
-      // (the last panels have too few 4 x 4 tiles for the CTA's warps)
-      if (db - NB * kb > 64) update_panel<4>(Lp, pm, kb); else update_panel<1>(Lp, pm, kb);
+      update_panel(Lp, pm, kb);
       __syncthreads();
     }
     eliminate_panel(Lp + pm.off(kb), invd + NB * kb, np - 1 - kb, &s_fail);
