@@ -16,7 +16,7 @@
 // Persistent kernel, 320 threads:
 //   warp 0    : TMA producer (raw fp32 chunks of 32 along K; MN-major chunks as four 32 x 32 boxes)
 //   warp 1    : MMA issuer   (tcgen05.mma kind::tf32, 128 x 128 x 8, two accumulators of 128 TMEM columns; dual: four)
-//   warps 2-5 : splitter     (raw chunk -> low part next to it, proxy fence)
+//   warps 2-5 : splitter     (raw chunk -> low part in a ring of its own, proxy fence)
 //   warps 6-9 : epilogue     (D tile prefetched by TMA into swizzled shared memory, tcgen05.ld, alpha / beta
 //                             in place, TMA store: no strided global access)
 // Dual mode: two inputs share the wrapper, A.X1 and A.X2 of a tile go through the pipeline back to back into
@@ -34,11 +34,13 @@ using namespace tc;
 constexpr int TILE = 128, BK = 32;
 constexpr int NTHREADS = 320;
 constexpr int OP_BYTES = TILE * BK * 4;           // 16 KiB: one operand chunk
-// A stage holds the M-side and the N-side chunk, each as its raw words (= high part) followed by its low part.
-constexpr int STAGES = 3, STAGE_BYTES = 4 * OP_BYTES;
+// A stage holds the M-side and the N-side chunk as their raw words (= high parts); the low parts have a ring of their own, so that
+// in the same 192 KiB four raw chunks are under way or in use instead of three.
+constexpr int STAGES = 4, LSTAGES = 2, STAGE_BYTES = 2 * OP_BYTES;
+constexpr size_t LO_OFF = (size_t)STAGES * STAGE_BYTES, EPI_OFF = LO_OFF + (size_t)LSTAGES * STAGE_BYTES;
 constexpr uint32_t TMEM_COLS = 512;               // four accumulators of 128 columns (two in use outside the dual mode)
 constexpr int EPI_BYTES = 32 * 64 * 4;            // per epilogue warp: 32 rows x 64 columns (half a tile row) as two swizzled boxes
-constexpr size_t SMEM_BYTES = (size_t)STAGES * STAGE_BYTES + 4 * EPI_BYTES + 1024;
+constexpr size_t SMEM_BYTES = EPI_OFF + 4 * EPI_BYTES + 1024;
 
 struct OpCoord {
   int mn_major;                     // 0: K-major, 1: MN-major
@@ -104,14 +106,15 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
                 const __grid_constant__ CUtensorMap mapD, const BParams p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ __align__(8) uint64_t bars[3 * STAGES + 12];
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 2 * LSTAGES + 12];
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_flag;
 
   const int warp = (int)uniform(threadIdx.x >> 5), lane = threadIdx.x & 31;
-  const uint32_t full0 = smem_u32(&bars[0]), split0 = smem_u32(&bars[STAGES]), empty0 = smem_u32(&bars[2 * STAGES]);
-  const uint32_t tfull0 = smem_u32(&bars[3 * STAGES]), tempty0 = smem_u32(&bars[3 * STAGES + 4]);
-  const uint32_t dfull0 = smem_u32(&bars[3 * STAGES + 8]);
+  // full / empty of the raw stages, ready / free of the low parts, full / empty of the accumulators, addend slabs
+  const uint32_t full0 = smem_u32(&bars[0]), empty0 = full0 + 8 * STAGES;
+  const uint32_t lready0 = empty0 + 8 * STAGES, lfree0 = lready0 + 8 * LSTAGES;
+  const uint32_t tfull0 = lfree0 + 8 * LSTAGES, tempty0 = tfull0 + 32, dfull0 = tempty0 + 32;
   const int n_items = p.batch * p.m_tiles * p.n_tiles;   // tiles
   const int n_sub = p.dual ? 2 : 1;                                  // passes through the pipeline per tile
   const int n_acc = p.dual ? 2 : 1;                                  // accumulators per tile
@@ -120,9 +123,9 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     abort_flag = 0;
     for (int s = 0; s < STAGES; ++s) {
       mbar_init(full0 + 8 * s, 1);
-      mbar_init(split0 + 8 * s, 4);
       mbar_init(empty0 + 8 * s, 1);
     }
+    for (int s = 0; s < LSTAGES; ++s) { mbar_init(lready0 + 8 * s, 4); mbar_init(lfree0 + 8 * s, 1); }
     for (int s = 0; s < 4; ++s) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 4); }
     for (int s = 0; s < 4; ++s) mbar_init(dfull0 + 8 * s, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -155,7 +158,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
           mbar_expect_tx(fb, 2 * OP_BYTES);
           const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
           load_operand(dst, &mapA, p.a, b, tm, kc, fb);
-          load_operand(dst + 2 * OP_BYTES, sub ? &mapB2 : &mapB, p.b, b, tn, kc, fb);
+          load_operand(dst + OP_BYTES, sub ? &mapB2 : &mapB, p.b, b, tn, kc, fb);
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
@@ -176,10 +179,11 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
       const uint32_t leader = elect_lane();
       const uint32_t idesc = instr_desc_tf32_mn(TILE, TILE, p.a.mn_major, p.b.mn_major);
       const uint64_t da0 = operand_desc(smem_u32(smem), p.a.mn_major, 0);
-      const uint64_t db0 = operand_desc(smem_u32(smem) + 2 * OP_BYTES, p.b.mn_major, 0);
+      const uint64_t db0 = operand_desc(smem_u32(smem) + OP_BYTES, p.b.mn_major, 0);
       const uint64_t kinc_a = p.a.mn_major ? (1024u >> 4) : (32u >> 4);   // one k-step of 8 in the address field
       const uint64_t kinc_b = p.b.mn_major ? (1024u >> 4) : (32u >> 4);
-      int stage = 0; uint32_t phase = 0;
+      int stage = 0;
+      int lst = 0; uint32_t lphase = 0;
       int local = 0;
       bool ok = true;
       for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x)
@@ -191,12 +195,13 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
         tc_fence_after();
         const uint32_t tacc = tmem_base + (uint32_t)(as * TILE);
         for (int kc = 0; kc < p.k_chunks; ++kc) {
-          if (!mbar_wait_warp(split0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+          if (!mbar_wait_warp(lready0 + 8 * lst, lphase, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
           // the descriptors of stage 0 are formed once and only their address field moves
           const uint64_t so = (uint64_t)(uint32_t)(stage * (STAGE_BYTES >> 4));
-          const uint64_t da = da0 + so, dal = da + (OP_BYTES >> 4);
-          const uint64_t dbm = db0 + so, dbl = dbm + (OP_BYTES >> 4);
+          const uint64_t lo = (uint64_t)(uint32_t)((LO_OFF + lst * STAGE_BYTES) >> 4);
+          const uint64_t da = da0 + so, dal = da0 + lo;
+          const uint64_t dbm = db0 + so, dbl = db0 + lo;
           const uint32_t first = (uint32_t)(kc > 0);
           if (p.one_pass) {
             umma_tf32_w(leader, tacc, da, dbm, idesc, first);
@@ -213,8 +218,10 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
               umma_tf32_w(leader, tacc, da + k * kinc_a, dbm + k * kinc_b, idesc, 1u);
             }
           }
-          umma_commit_w(leader, empty0 + 8 * stage);   // frees the stage once these MMAs have read it
-          if (++stage == STAGES) { stage = 0; phase ^= 1; }
+          umma_commit_w(leader, empty0 + 8 * stage);   // frees the chunk and its low parts once these MMAs have read them
+          umma_commit_w(leader, lfree0 + 8 * lst);
+          if (++stage == STAGES) stage = 0;
+          if (++lst == LSTAGES) { lst = 0; lphase ^= 1; }
         }
         if (ok) umma_commit_w(leader, tfull0 + 8 * as);
       }
@@ -223,32 +230,37 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     // ------------------------------------------------------------ splitter warps
     const int t = threadIdx.x - 64;   // 0..127
     int stage = 0; uint32_t phase = 0;
+    int lst = 0; uint32_t lphase = 0;
     bool ok = true;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x) {
       for (int kc = 0; kc < n_sub * p.k_chunks; ++kc) {
         if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
-        float4* base = reinterpret_cast<float4*>(smem + (size_t)stage * STAGE_BYTES);
+        const float4* hi = reinterpret_cast<const float4*>(smem + (size_t)stage * STAGE_BYTES);
+        float4* lo = reinterpret_cast<float4*>(smem + LO_OFF + (size_t)lst * STAGE_BYTES);
+        constexpr int PER = STAGE_BYTES / 16 / 128;
+        float4 v[PER];
+        if (!p.one_pass) {
 #pragma unroll
-        for (int op = 0; op < (p.one_pass ? 0 : 2); ++op) {
-          float4* hi = base + op * (2 * OP_BYTES / 16);
-          float4* lo = hi + OP_BYTES / 16;
+          for (int e = 0; e < PER; ++e) v[e] = hi[t + e * 128];
+        }
+        if (!mbar_wait(lfree0 + 8 * lst, lphase ^ 1, abortp, p.status)) { ok = false; break; }
+        if (!p.one_pass) {
 #pragma unroll
-          for (int e = 0; e < OP_BYTES / 16 / 128; ++e) {
-            const int idx = t + e * 128;
-            const float4 v = hi[idx];
+          for (int e = 0; e < PER; ++e) {
             float4 h;
-            h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
-            h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
-            h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
-            h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
-            lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+            h.x = __uint_as_float(__float_as_uint(v[e].x) & 0xffffe000u);
+            h.y = __uint_as_float(__float_as_uint(v[e].y) & 0xffffe000u);
+            h.z = __uint_as_float(__float_as_uint(v[e].z) & 0xffffe000u);
+            h.w = __uint_as_float(__float_as_uint(v[e].w) & 0xffffe000u);
+            lo[t + e * 128] = make_float4(v[e].x - h.x, v[e].y - h.y, v[e].z - h.z, v[e].w - h.w);
           }
         }
         // make the generic-proxy writes visible to the tensor-core (async proxy) reads
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
-        if (lane == 0) mbar_arrive(split0 + 8 * stage);
+        if (lane == 0) mbar_arrive(lready0 + 8 * lst);
         if (++stage == STAGES) { stage = 0; phase ^= 1; }
+        if (++lst == LSTAGES) { lst = 0; lphase ^= 1; }
       }
     }
   } else {
@@ -257,7 +269,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
     int local = 0;
     uint32_t d_loads = 0;   // D slabs requested so far: parity of their barrier
     bool ok = true;
-    uint8_t* buf = smem + (size_t)STAGES * STAGE_BYTES + (size_t)q * EPI_BYTES;   // two 4 KiB boxes of 32 x 32
+    uint8_t* buf = smem + EPI_OFF + (size_t)q * EPI_BYTES;   // two 4 KiB boxes of 32 x 32
     const uint32_t buf_u32 = smem_u32(buf);
     const uint32_t dbar = dfull0 + 8 * q;
     for (int item = blockIdx.x; item < n_items && ok; item += gridDim.x, ++local) {
