@@ -104,8 +104,8 @@ size_t carve(const armor_config& cfg, armor_ctx* c, char* base) {
     TAKE(rowscale2, float*, (size_t)dmax * sizeof(float));
   }
   if (tc) {
-    TAKE(gemm_slabs, float*, (size_t)160 * 128 * 256 * sizeof(float));
-    if (c) c->gemm_slab_count = 160;
+    TAKE(gemm_slabs, float*, (size_t)ARMOR_GEMM_SLABS * 128 * 256 * sizeof(float));
+    if (c) c->gemm_slab_count = ARMOR_GEMM_SLABS;
     TAKE(Xt_hi, float*, (size_t)cfg.d_in * GRAM_ROWS * sizeof(float));
     // (the fp16 mode keeps both 16-bit parts of the staged chunk in Xt_hi)
     if (cfg.precision == ARMOR_PREC_FP32X3) TAKE(Xt_lo, float*, (size_t)cfg.d_in * GRAM_ROWS * sizeof(float)); else if (c) c->Xt_lo = nullptr;

@@ -59,6 +59,7 @@ struct SelRec {
   float old_val[8];
 };
 
+static const int ARMOR_GEMM_SLABS = 160;  // slabs of partial sums of cut tiles in the workspace
 static const int ARMOR_DOT_BLOCKS = 592;  // 4 x 148 partial sums per reduction
 
 struct armor_ctx {

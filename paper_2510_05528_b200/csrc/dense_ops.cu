@@ -87,6 +87,18 @@ armor_status rmul_H(armor_ctx* c, const float* in, const float* H, float* out, i
   return ARMOR_OK;
 }
 
+// The product of a Gram with more room for the sums of cut tiles: `floats` of scratch at `spare`, where that holds more slabs
+// (128 x 256 sums) than the context's own.  A Gram of 1,024 channels has 10 tiles for 74 pairs of CTAs and 16 segments of 1,024 tokens
+// a launch, 320 slabs: uncut it kept 10 pairs busy (bf16, 30,000 tokens: 188 us).  Same sums in the same order.
+static armor_status gram_product(armor_ctx* c, const TcGemm& g, float* spare, int64_t floats, cudaStream_t s) {
+  float* const own = c->gemm_slabs;
+  const int64_t own_count = c->gemm_slab_count, n = floats / (128 * 256);
+  if (spare && n > own_count) { c->gemm_slabs = spare; c->gemm_slab_count = n; }
+  const armor_status st = launch_tc_gemm(c, g, nullptr, s);
+  c->gemm_slabs = own; c->gemm_slab_count = own_count;
+  return st;
+}
+
 armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t n_rows, int64_t ldx, float* H,
                              cudaStream_t s) {
   const int64_t d_in = c->d_in;
@@ -130,7 +142,7 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
       g.accumulate = 1;
       g.symmetric_lower = 1;
       g.k_segment = K_SEGMENT;
-      const armor_status st = launch_tc_gemm(c, g, nullptr, s);
+      const armor_status st = gram_product(c, g, c->Xt_hi, d_in * c->gram_rows, s);     // (nothing is staged)
       if (st != ARMOR_OK) return st;
     }
     launch_mirror_lower(c, H, d_in, s, Xv, ldx, n_rows, in_range);
@@ -179,7 +191,7 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
       g.accumulate = 1;
       g.symmetric_lower = 1;
       g.k_segment = K_SEGMENT;
-      st = launch_tc_gemm(c, g, nullptr, s);
+      st = gram_product(c, g, overlap ? nullptr : c->Xt_hi2, d_in * c->gram_rows, s);   // (the second staging buffer is idle)
       if (st != ARMOR_OK) return st;
       if (overlap && cudaEventRecord(c->ev_used[b], s) != cudaSuccess) return ARMOR_ERR_CUDA;
     }

@@ -604,8 +604,12 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
       if (per == kt_total && fill > 1 && p.kt_seg < kt_total) per = p.kt_seg;
     }
     const int parts = (kt_total + per - 1) / per;
-    // (a slab holds 128 x 256 sums, a piece writes two)
-    if (parts > 1 && kt_total - per >= worth && (int64_t)rem * parts * 2 <= c->gemm_slab_count) {
+    // (a slab holds 128 x 256 sums, a piece writes two.)  More than the context's own slabs come with a Gram of few channels, whose
+    // pieces may take several rounds of the pairs: 0.8 or 0.25 us a k-tile saved against 0.1 us a piece for its 256 KB and 6 us.
+    const int64_t slabs = (int64_t)rem * parts * 2;
+    const int rounds = (rem * parts + n_pairs - 1) / n_pairs;
+    const bool pays = slabs <= ARMOR_GEMM_SLABS || (kt_total - rounds * per) * (SPLIT ? 32 : 10) > 4 * rem * parts + 240;
+    if (parts > 1 && kt_total - per >= worth && slabs <= c->gemm_slab_count && pays) {
       p.split_kt = per;
       p.split_parts = parts;
       p.split_first = p.n_tiles_total - rem;

@@ -1,4 +1,4 @@
-"""Kernels of the wrapper steps at the edges of their dispatch: per-block Grams, the choice between the two kernels for one-sided
+"""Kernels at the edges of their dispatch: Grams of few channels cut along the tokens, per-block Grams, the choice between the two kernels for one-sided
 products, the two tile sizes of small products, the solves' panels and the joint update of the carried product."""
 import numpy as np
 import pytest
@@ -124,3 +124,23 @@ def test_carried_product_moves_by_both_steps(d_out, d_in, d_block):
         loss = ctx.proxy_loss(st, H).item()
         assert abs(rec["loss_mask"][-1] - loss) <= 1e-5 * rec["loss_start"][0]
         assert np.all(np.diff(rec["loss_mask"]) <= 0)
+
+
+@pytest.mark.parametrize("d_in,tokens", [(768, 16384), (1024, 5000), (1024, 16384), (1024, 16385), (1536, 9000), (2048, 16384)])
+def test_gram_of_few_channels_is_cut_along_the_tokens(d_in, tokens):
+    """Tiles cut at segments of 1,024 tokens add up in the order of an uncut tile: the Gram of bf16 activations, which are not
+    scaled, has the bits of one call per segment; fp32 activations, scaled per call, those of fp64 to the parts' 22 bits."""
+    g = _gen(d_in + tokens)
+    ctx = _ctx(128, d_in, 128)
+    X = torch.randn(tokens, d_in, device=DEV, generator=g)
+    Xb = X.to(torch.bfloat16)
+    H, H1 = ctx.new_gram(), ctx.new_gram()
+    ctx.gram(Xb, H)
+    for r in range(0, tokens, 1024):
+        ctx.gram(Xb[r:r + 1024].contiguous(), H1)
+    assert torch.equal(H, H1) and torch.equal(H, H.t())
+    H.zero_()
+    ctx.gram(X, H)
+    ref = X.double().t() @ X.double()
+    assert (H.double() - ref).norm() <= 3e-5 * ref.norm() and torch.equal(H, H.t())
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
