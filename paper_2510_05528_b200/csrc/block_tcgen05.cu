@@ -476,9 +476,10 @@ inline bool ptr_ok(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15)
 // Tiles of 128 x 128 per SM from which one-sided products (d_block 128) take the wrapper block from tensor memory.  That
 // kernel spends its first 2 to 3 us bringing the block there; a right product's CTAs stay with one column block and read 512
 // bytes of every row, which costs more than the saved shared-memory traffic while there are few tiles.  This kernel / that one:
-// right 1024 x 5120 (2 tiles per SM) 23.4 / 27.0 us, 2048 x 2048 17.2 / 21.0, 4096 x 4096 (7) 36.1 / 35.0, 8195 x 4096 (14) 69 / 62,
-// 14336 x 4096 106 / 97; left 512 x 512 9.3 / 11.9, 2048 x 2048 16.1 / 16.3, 1024 x 5120 22.4 / 22.3, 4096 x 4096 36.6 / 30.8.
-static const int RES_RIGHT = 6, RES_LEFT = 1;
+// right 1024 x 5120 (2.2 tiles per SM) 17.7 / 21.2 us, 4096 x 4096 (6.9) 32.7 / 34.7, 6144 x 4096 (10.4) 48.0 / 50.9, 8192 x 4096 (13.8)
+// 63.7 / 57.9, 14336 x 4096 (24) 98 / 93; left 2048 x 2048 (1.7) 13.9 / 15.2, 1024 x 5120 17.4 / 18.2, 2048 x 4096 (3.5) 23.4 / 20.8, 4096 x 4096
+// 32.9 / 30.7, 14336 x 4096 98 / 89.
+static const int RES_RIGHT = 12, RES_LEFT = 3;
 
 bool tc_block_ok(const armor_ctx* c, int64_t rows, int64_t cols) {
   return c->cfg.precision != ARMOR_PREC_SIMT && c->db % TILE == 0 && rows > 0 && cols % 4 == 0;

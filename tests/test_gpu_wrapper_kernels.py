@@ -19,12 +19,12 @@ def _ctx(d_out, d_in, d_block, **kw):
     return Bd.ArmorContext(d_out, d_in, d_block, device=DEV, **kw)
 
 
-@pytest.mark.parametrize("side,rows,cols", [(0, 128, 128), (0, 1025, 1024), (0, 14200, 1024), (0, 14208, 1024), (1, 128, 132),
-                                            (1, 1024, 2304), (1, 1152, 2100)])
+@pytest.mark.parametrize("side,rows,cols", [(0, 128, 128), (0, 1025, 1024), (0, 28280, 1024), (0, 28416, 1024), (1, 128, 132),
+                                            (1, 1536, 4604), (1, 1536, 4612)])
 @pytest.mark.parametrize("transpose", [0, 1])
 def test_one_sided_products_on_either_side_of_the_choice(side, rows, cols, transpose):
     """The library's choice (path -1) gives the bits of both kernels: one tile, ragged in the free dimension, and the last tile
-    count below and the first above the lines (148 SMs: 888 tiles of a right product, 148 of a left one)."""
+    count below and the first on the lines (148 SMs: 1,776 tiles of a right product, 444 of a left one)."""
     from paper_2510_05528_b200 import binding as Bd
     g = _gen(rows + cols)
     ctx = _ctx(1024, 1024, 128)
