@@ -156,8 +156,8 @@ static const int ARMOR_MAX_TIMED = 8192;
 // the wait made chains of waiting kernels: 3,280 us for 20 iterations of a 256 x 256 layer, 2,996 without any of this, 2,747
 // this way.)  Three rules follow.  grid_begin() stands before the first access to global memory and before any return.  A
 // kernel that takes tensor memory takes it first: the CTAs that grid_begin() lets in may wait for theirs while this one runs.
-// And what a kernel reads is not declared __restrict__ nor read through __ldg (but for data written two or more kernels
-// before: it is there when a kernel starts): a load of data taken for constant may be moved above the wait.
+// And what a kernel reads is not declared __restrict__, const or not, nor read through __ldg (but for data written two or more
+// kernels before: it is there when a kernel starts): a load of data that nothing else is known to write may be moved above the wait.
 __device__ __forceinline__ void grid_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

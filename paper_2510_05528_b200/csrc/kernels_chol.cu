@@ -333,8 +333,8 @@ constexpr int MAX_DB = 256;
 template <int G>
 __global__ void __launch_bounds__(NT, 1)
 chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __restrict__ out,
-                    const float* dotw, float* __restrict__ A, float ridge, int db, double* __restrict__ part,
-                    int32_t* __restrict__ failflag, int32_t* __restrict__ status) {
+                    const float* dotw, float* A, float ridge, int db, double* __restrict__ part,
+                    int32_t* __restrict__ failflag, int32_t* status) {
   grid_begin();
   constexpr int W = 32 * G, LDX = W + 1;                // (odd: neither a row of X nor 8 x 4 floats along a column conflict)
   extern __shared__ __align__(16) float smem[];
@@ -414,24 +414,39 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
   // ---- write back.  Right solves: right-hand side vid is row vid of the result; left solves: column vid.
   double acc = 0.0;
   if (right) {
-#pragma unroll 4
-    for (int e = tid; e < W * q4; e += NT) {
-      const int c8 = e & 7, v = (e >> 3) % W, i = 4 * (c8 + 8 * ((e >> 3) / W));
-      if (v0 + v >= db) continue;
-      const int64_t idx = off + (int64_t)(v0 + v) * db + i;
-      const float4 aold = mode == 0 ? ld4(A + idx) : make_float4(0.f, 0.f, 0.f, 0.f);
-      const float4 gin = ld4((mode == 0 ? rhs : dotw) + idx);
-      float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!fail && !hold) x = make_float4(X[i * LDX + v], X[(i + 1) * LDX + v], X[(i + 2) * LDX + v], X[(i + 3) * LDX + v]);
-      *reinterpret_cast<float4*>(out + idx) = x;
-      if (mode == 0) {
-        *reinterpret_cast<float4*>(A + idx) = make_float4(aold.x + x.x, aold.y + x.y, aold.z + x.z, aold.w + x.w);
-        acc += (double)gin.x * (double)x.x + lam * (double)x.x * (double)x.x;
-        acc += (double)gin.y * (double)x.y + lam * (double)x.y * (double)x.y;
-        acc += (double)gin.z * (double)x.z + lam * (double)x.z * (double)x.z;
-        acc += (double)gin.w * (double)x.w + lam * (double)x.w * (double)x.w;
-      } else {
-        acc += (double)gin.x * (double)x.x + (double)gin.y * (double)x.y + (double)gin.z * (double)x.z + (double)gin.w * (double)x.w;
+    // (four at a time, all loads ahead of the first store: A is read and written)
+    constexpr int U = 4;
+    for (int e0 = tid; e0 < W * q4; e0 += U * NT) {
+      float4 aold[U], gin[U];
+      int64_t idx[U];
+      int cell[U];                                      // first of its four unknowns in X, -1: nothing there
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int e = e0 + u * NT, c8 = e & 7, v = (e >> 3) % W, i = 4 * (c8 + 8 * ((e >> 3) / W));
+        cell[u] = e < W * q4 && v0 + v < db ? i * LDX + v : -1;
+        idx[u] = off + (int64_t)(v0 + v) * db + i;
+        aold[u] = gin[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (cell[u] < 0) continue;
+        if (mode == 0) aold[u] = ld4(A + idx[u]);
+        gin[u] = ld4((mode == 0 ? rhs : dotw) + idx[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (cell[u] < 0) continue;
+        const float* xs = X + cell[u];
+        const float4 g = gin[u], a = aold[u];
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (!fail && !hold) x = make_float4(xs[0], xs[LDX], xs[2 * LDX], xs[3 * LDX]);
+        *reinterpret_cast<float4*>(out + idx[u]) = x;
+        if (mode == 0) {
+          *reinterpret_cast<float4*>(A + idx[u]) = make_float4(a.x + x.x, a.y + x.y, a.z + x.z, a.w + x.w);
+          acc += (double)g.x * (double)x.x + lam * (double)x.x * (double)x.x;
+          acc += (double)g.y * (double)x.y + lam * (double)x.y * (double)x.y;
+          acc += (double)g.z * (double)x.z + lam * (double)x.z * (double)x.z;
+          acc += (double)g.w * (double)x.w + lam * (double)x.w * (double)x.w;
+        } else {
+          acc += (double)g.x * (double)x.x + (double)g.y * (double)x.y + (double)g.z * (double)x.z + (double)g.w * (double)x.w;
+        }
       }
     }
   } else {
@@ -459,9 +474,9 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
 
 // Unblocked variant for block sizes that are not a multiple of 32: thread i owns row i.
 __global__ void chol_kernel(int mode, const float* Gmat, const float* rhs,
-                            float* __restrict__ out, const float* dotw, float* __restrict__ A,
+                            float* __restrict__ out, const float* dotw, float* A,
                             float ridge, int db, double* __restrict__ part,
-                            int32_t* __restrict__ failflag, int32_t* __restrict__ status) {
+                            int32_t* __restrict__ failflag, int32_t* status) {
   grid_begin();
   extern __shared__ float smem[];
   const int ld = db + 1;
@@ -616,7 +631,7 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
 
 namespace {
 
-__global__ void identity_rhs_kernel(float* __restrict__ X, int db) {
+__global__ void identity_rhs_kernel(float* X, int db) {
   grid_begin();
   float* Xb = X + (int64_t)blockIdx.x * db * db;
   for (int e = threadIdx.x; e < db * db; e += blockDim.x) Xb[e] = (e / db == e % db) ? 1.f : 0.f;
@@ -630,7 +645,7 @@ __global__ void save_flags_kernel(const int32_t* failflag, int32_t* __restrict__
 
 // DELTA_PARTS CTAs per block: Delta_j = 0 and failflag[j] = 1 where the inverse does not exist; partial sums of
 // <dotw_j, Delta_j>
-__global__ void __launch_bounds__(NT) delta_finish_kernel(float* __restrict__ Delta, const float* dotw,
+__global__ void __launch_bounds__(NT) delta_finish_kernel(float* Delta, const float* dotw,
                                                           const int32_t* hinv_fail,
                                                           int32_t* __restrict__ failflag, double* __restrict__ part,
                                                           int db) {
@@ -640,12 +655,16 @@ __global__ void __launch_bounds__(NT) delta_finish_kernel(float* __restrict__ De
   const int n4 = db * db / 4, e1 = n4 * (q + 1) / DELTA_PARTS;
   const bool bad = hinv_fail[j] != 0;
   double acc = 0.0;
+  const int e0 = n4 * q / DELTA_PARTS + threadIdx.x;
+  float4* d = reinterpret_cast<float4*>(Delta + off);
+  if (bad) {
+    for (int e = e0; e < e1; e += NT) d[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  } else {
 #pragma unroll 4
-  for (int e = n4 * q / DELTA_PARTS + threadIdx.x; e < e1; e += NT) {
-    float4* d = reinterpret_cast<float4*>(Delta + off) + e;
-    if (bad) { *d = make_float4(0.f, 0.f, 0.f, 0.f); continue; }
-    const float4 w = *(reinterpret_cast<const float4*>(dotw + off) + e), v = *d;
-    acc += (double)w.x * (double)v.x + (double)w.y * (double)v.y + (double)w.z * (double)v.z + (double)w.w * (double)v.w;
+    for (int e = e0; e < e1; e += NT) {
+      const float4 w = *(reinterpret_cast<const float4*>(dotw + off) + e), v = d[e];
+      acc += (double)w.x * (double)v.x + (double)w.y * (double)v.y + (double)w.z * (double)v.z + (double)w.w * (double)v.w;
+    }
   }
   __shared__ double red[NT / 32];
   for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);

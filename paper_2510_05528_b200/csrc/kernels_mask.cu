@@ -129,8 +129,7 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
                                                          int n_keep, int select_mode, uint64_t seed, uint64_t t_base,
                                                          uint64_t t_mul, const int64_t* it_dev,
                                                          uint64_t n_groups_total, int kg_arg,
-                                                         float* __restrict__ tab_key,
-                                                         unsigned long long* __restrict__ tab_g) {
+                                                         float* tab_key, unsigned long long* tab_g) {
   grid_begin();
   const uint64_t t = t_base + t_mul * (uint64_t)(*it_dev);   // selection counter of this run of Algorithm 3
   const int kg = MULTI ? kg_arg : 1;                       // one draw: the loop and the key cache compile away
@@ -471,7 +470,7 @@ __global__ void __launch_bounds__(NT) mask_quad_kernel(const float* Zsel, const 
 
 // A thread per block (one CTA walking 3,584 blocks took 21 us).
 constexpr int COMMIT_NT = 64;
-__global__ void __launch_bounds__(COMMIT_NT) mask_commit_kernel(const SelRec* sel, int nblocks, float* __restrict__ S,
+__global__ void __launch_bounds__(COMMIT_NT) mask_commit_kernel(const SelRec* sel, int nblocks, float* S,
                                                                 uint8_t* __restrict__ M, int64_t d_in, int mg, const double* sc,
                                                                 armor_iter_stats* st_base, const int64_t* it_dev) {
   grid_begin();
@@ -505,7 +504,7 @@ constexpr int CARRY_CTAS = 64;
 constexpr int CARRY_TAB = 2048;                            // picks whose rows are kept in shared memory
 __device__ __forceinline__ int carry_row(const SelRec& rec, int row0) { return rec.valid ? rec.row - row0 : -1; }
 __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* sel, const float* Y,
-                                                        float* __restrict__ P, const double* sc,
+                                                        float* P, const double* sc,
                                                         int64_t d_in, int db, int nbo_pad, int nbv) {
   grid_begin();
   __shared__ int row_of[CARRY_TAB];                        // row inside the block, -1: no group

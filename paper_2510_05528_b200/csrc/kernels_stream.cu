@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(NT) masked_copy_kernel(const float4* gam, cons
 }
 
 // ---- y += sign * sc[slot] * x -------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* __restrict__ y, const float4* x,
+__global__ void __launch_bounds__(NT) axpy_slot_kernel(float4* y, const float4* x,
                                                        int64_t n4, const double* sc, int slot,
                                                        float sign) {
   grid_begin();
@@ -528,7 +528,7 @@ __global__ void __launch_bounds__(NT) screen_count_kernel(const float4* W, int64
     if (zero) atomicAdd(&scr[3], zero);
   }
 }
-__global__ void screen_final_kernel(const int32_t* scr, int32_t* __restrict__ status) {
+__global__ void screen_final_kernel(const int32_t* scr, int32_t* status) {
   grid_begin();
   status[ST_NONFINITE_W] += scr[0];
   status[ST_NONFINITE_H] += scr[1];
@@ -698,8 +698,8 @@ __global__ void __launch_bounds__(NT) block_fro_kernel(const float4* X, int n4_p
 }
 
 // ---- Adam (Kingma & Ba, Algorithm 1, with bias correction) ----------------------------------------------
-__global__ void __launch_bounds__(NT) adam_kernel(float4* __restrict__ theta, const float4* gamma,
-                                                  float4* __restrict__ m, float4* __restrict__ v, int64_t n4,
+__global__ void __launch_bounds__(NT) adam_kernel(float4* theta, const float4* gamma,
+                                                  float4* m, float4* v, int64_t n4,
                                                   const uint8_t* M, int q4, float lr, float b1, float b2,
                                                   float eps, int64_t step_base, const int64_t* it_dev,
                                                   const int32_t* status) {
