@@ -127,8 +127,8 @@ struct armor_ctx {
   int tc_blocks;        // 1, 2, 3: block products and per-block Grams on the tensor cores where the shape allows.
                         // 1: the streaming kernel for every product; 2: with d_block = 128 the kernel that keeps the
                         // wrapper block in tensor memory (products and dual products); 3 (default): that kernel for
-                        // left and dual products and for right products with the column-scaled second output, the
-                        // streaming kernel for other right products, the two-sided kernel where both wrappers apply;
+                        // dual products, right products with the column-scaled second output and other three-pass
+                        // products of many tiles, else the streaming kernel, the two-sided kernel where both wrappers apply;
                         // 0: always the fp32 CUDA-core kernels (exact products with 0 and 1)
   int gram_pairs;       // 1: the two per-block Grams of a step in one launch (shared operand read once)
   armor_status host_err;   // first launch failure inside the running call that no fallback covers

@@ -478,7 +478,8 @@ inline bool ptr_ok(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15)
 // bytes of every row, which costs more than the saved shared-memory traffic while there are few tiles.  This kernel / that one:
 // right 1024 x 5120 (2.2 tiles per SM) 17.7 / 21.2 us, 4096 x 4096 (6.9) 32.7 / 34.7, 6144 x 4096 (10.4) 48.0 / 50.9, 8192 x 4096 (13.8)
 // 63.7 / 57.9, 14336 x 4096 (24) 98 / 93; left 2048 x 2048 (1.7) 13.9 / 15.2, 1024 x 5120 17.4 / 18.2, 2048 x 4096 (3.5) 23.4 / 20.8, 4096 x 4096
-// 32.9 / 30.7, 14336 x 4096 98 / 89.
+// 32.9 / 30.7, 14336 x 4096 98 / 89.  Products of one pass (the bf16 forward) have no low parts to save and stay here: forward of 6144 x 6144,
+// 4,736 tokens, packed core, 443 / 454 us, 8192 x 8192, 8,192 tokens 1,068 / 1,097.
 static const int RES_RIGHT = 12, RES_LEFT = 3;
 
 bool tc_block_ok(const armor_ctx* c, int64_t rows, int64_t cols) {

@@ -71,7 +71,6 @@ struct RParams {
   int tiles, batch;                 // tiles per wrapper block along the free dimension; work = batch * tiles tiles
   float alpha, beta;
   int32_t* status;
-  int one_pass;
   const float* colw;                // one product, right: not null: a second output (through mapX2) = out scaled per
                                     // column by colw
   // dual (left only): the two halves of an instruction are the same tile of two inputs (mapX, mapX2);
@@ -229,11 +228,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
           const uint64_t dx = dx0 + (uint64_t)(uint32_t)(stage * (STAGE_BYTES >> 4));
           const uint64_t dxl = dl0 + (uint64_t)(uint32_t)(lst * (STAGE_BYTES >> 4));
           const uint32_t w_hi = w_hi0 + (uint32_t)(kc * BK), w_lo = w_lo0 + (uint32_t)(kc * BK);
-          if (p.one_pass) {
-            umma_tf32_ta_w(leader, tacc, w_hi, dx, idesc, (uint32_t)(kc > 0));
-#pragma unroll
-            for (int k = 1; k < BK / 8; ++k) umma_tf32_ta_w(leader, tacc, w_hi + 8 * k, dx + k * kinc, idesc, 1u);
-          } else if (p.right) {
+          if (p.right) {
             // low part of X (the M side of the untransposed product) first
             umma_tf32_ta_w(leader, tacc, w_hi, dxl, idesc, (uint32_t)(kc > 0));
             umma_tf32_ta_w(leader, tacc, w_lo, dx, idesc, 1u);
@@ -303,12 +298,10 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
                 for (int i = 0; i < 32; ++i)
                   hi[i] = *reinterpret_cast<const uint32_t*>(colp + (k0 + i) * 128 + (((lane >> 2) ^ (i & 7)) << 4));
                 tmem_st32(tmem_base + W_HI + (uint32_t)k0 + lane_sel, hi);
-                if (!p.one_pass) {
 #pragma unroll
-                  for (int i = 0; i < 32; ++i)
-                    lo[i] = __float_as_uint(__uint_as_float(hi[i]) - __uint_as_float(hi[i] & 0xffffe000u));
-                  tmem_st32(tmem_base + W_LO + (uint32_t)k0 + lane_sel, lo);
-                }
+                for (int i = 0; i < 32; ++i)
+                  lo[i] = __float_as_uint(__uint_as_float(hi[i]) - __uint_as_float(hi[i] & 0xffffe000u));
+                tmem_st32(tmem_base + W_LO + (uint32_t)k0 + lane_sel, lo);
               }
             }
           } else {
@@ -324,12 +317,10 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
                 hi[4 * i] = v.x; hi[4 * i + 1] = v.y; hi[4 * i + 2] = v.z; hi[4 * i + 3] = v.w;
               }
               tmem_st32(tmem_base + W_HI + k0 + lane_sel, hi);
-              if (!p.one_pass) {
 #pragma unroll
-                for (int i = 0; i < 32; ++i)
-                  lo[i] = __float_as_uint(__uint_as_float(hi[i]) - __uint_as_float(hi[i] & 0xffffe000u));
-                tmem_st32(tmem_base + W_LO + k0 + lane_sel, lo);
-              }
+              for (int i = 0; i < 32; ++i)
+                lo[i] = __float_as_uint(__uint_as_float(hi[i]) - __uint_as_float(hi[i] & 0xffffe000u));
+              tmem_st32(tmem_base + W_LO + k0 + lane_sel, lo);
             }
           }
           // the stage goes back to the producer once all four warps have read it (every barrier of a stage
@@ -352,20 +343,18 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       for (int kc = 0; kc < TILE / BK; ++kc) {
         if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
         if (!mbar_wait(lfree0 + 8 * lst, lphase ^ 1, abortp, p.status)) { ok = false; break; }
-        if (!p.one_pass) {
-          const float4* hi = reinterpret_cast<const float4*>(smem + (size_t)stage * STAGE_BYTES);
-          float4* lo = reinterpret_cast<float4*>(smem + LO_OFF + (size_t)lst * STAGE_BYTES);
+        const float4* hi = reinterpret_cast<const float4*>(smem + (size_t)stage * STAGE_BYTES);
+        float4* lo = reinterpret_cast<float4*>(smem + LO_OFF + (size_t)lst * STAGE_BYTES);
 #pragma unroll
-          for (int e = 0; e < CH * (OP_BYTES / 16 / 128); ++e) {
-            const int idx = t + e * 128;
-            const float4 v = hi[idx];
-            float4 h;
-            h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
-            h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
-            h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
-            h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
-            lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
-          }
+        for (int e = 0; e < CH * (OP_BYTES / 16 / 128); ++e) {
+          const int idx = t + e * 128;
+          const float4 v = hi[idx];
+          float4 h;
+          h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
+          h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
+          h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
+          h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
+          lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
         }
         // make the generic-proxy writes visible to the tensor-core (async proxy) reads
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -589,7 +578,6 @@ armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, 
   }
   p.c_rows = rows; p.c_cols = cols;
   p.status = c->status;
-  p.one_pass = c->block_one_pass;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_blockres_kernel<DUAL>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int64_t n_items = (int64_t)p.batch * p.tiles;
@@ -604,7 +592,7 @@ inline bool ptr_ok(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15)
 
 }  // namespace
 
-bool tc_blockres_ok(const armor_ctx* c) { return c->db == TILE; }
+bool tc_blockres_ok(const armor_ctx* c) { return c->db == TILE && !c->block_one_pass; }
 
 // out[:, j-th block] = alpha * in[:, j-th block] * Q_j (+ beta * add[:, j-th block]),  Q_j = Bblk[j] or its transpose; with
 // colw also out2 = out scaled per column by colw

@@ -44,8 +44,8 @@ def test_one_sided_products_on_either_side_of_the_choice(side, rows, cols, trans
 
 @pytest.mark.parametrize("tiles_per_sm", [11.9, 12.0])
 def test_bf16_forward_on_either_side_of_the_choice(tiles_per_sm):
-    """bf16 activations with fp32 wrappers take one tf32 pass per wrapper product: the last count of row tiles below the line of
-    twelve tiles per SM and the first on it, the last tile ragged.  Integer operands, every sum exact in fp32, one rounding to bf16:
+    """bf16 activations with fp32 wrappers take one tf32 pass per wrapper product, on the streaming kernel whatever their number: the last
+    count of row tiles below the three-pass products' line of twelve tiles per SM and the first on it, the last tile ragged.  Integer operands, every sum exact in fp32, one rounding to bf16:
     the bits of fp64."""
     from paper_2510_05528_b200 import binding as Bd
     d, n_sm = 6144, torch.cuda.get_device_properties(0).multi_processor_count
