@@ -766,7 +766,7 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
       yc = static_cast<float*>(d_y) + t0 * d_out;
       if (r1) {
         float* xs = wide ? c->V : c->Tmp;      // (z2 takes its place after z1 is formed)
-        launch_scale_rows_cols(c, xc, r1, nullptr, xs, n, d_in, s);
+        launch_scale_cols(c, xc, r1, xs, n, d_in, s);
         xc = xs;
       }
     }
@@ -780,7 +780,7 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
     bd_right(c, z2, A, true, yc, n, d_out, 1.f, nullptr, 0.f, s);                    // y = z2 A^T
     c->block_one_pass = 0;
     if (bf16) launch_f32_to_bf16(c, yc, r2, static_cast<char*>(d_y) + (size_t)(t0 * d_out) * esz, n, d_out, s);
-    else if (r2) launch_scale_rows_cols(c, yc, r2, nullptr, yc, n, d_out, s);
+    else if (r2) launch_scale_cols(c, yc, r2, yc, n, d_out, s);
   }
   return finish_call(c);
 }

@@ -392,8 +392,7 @@ void launch_block_fro_sum(armor_ctx* c, const float* X, int nblk, const float* h
 void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, int nflag,
                   cudaStream_t s, const double* p1 = nullptr, int n1 = 0, int slot1 = 0, const double* p2 = nullptr,
                   int n2 = 0, int slot2 = 0);
-void launch_scale_rows_cols(armor_ctx* c, const float* in, const float* colscale, const float* rowscale,
-                            float* out, int64_t rows, int64_t cols, cudaStream_t s);
+void launch_scale_cols(armor_ctx* c, const float* in, const float* colscale, float* out, int64_t rows, int64_t cols, cudaStream_t s);
 void launch_split_hilo(armor_ctx* c, const float* in, float* hi, float* lo, int64_t n, cudaStream_t s);
 void launch_transpose_split(armor_ctx* c, const void* X, int x_dtype, int64_t ldx, int64_t rows, int64_t cols,
                             float* Thi, float* Tlo, int64_t ldt, cudaStream_t s);

@@ -60,6 +60,29 @@ __global__ void __launch_bounds__(NT) reduce_final_kernel(const double* part, in
   if (threadIdx.x == 0) *out = acc;
 }
 
+// Grid-stride loop over n elements, four a thread at a time: all four are loaded before the first is stored.  (The compiler makes
+// this of a plain loop only where what is read is __restrict__, which a kernel that waits in grid_begin() may not say: left to
+// it, the bf16 conversions took 59 us for 4,736 x 6,144 elements against 34, the column scales of 4,096 x 4,096 39 against 36.)
+template <typename T, typename Load, typename Store>
+__device__ __forceinline__ void by_fours(int64_t n, Load load, Store store) {
+  const int64_t stride = (int64_t)gridDim.x * NT;
+  int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x;
+  for (; i + 3 * stride < n; i += 4 * stride) {
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = load(i + u * stride);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) store(i + u * stride, v[u]);
+  }
+  T v[3];
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+    if (i + u * stride < n) v[u] = load(i + u * stride);
+#pragma unroll
+  for (int u = 0; u < 3; ++u)
+    if (i + u * stride < n) store(i + u * stride, v[u]);
+}
+
 // ---- column scale: out = in * diag(h) -----------------------------------------------------------
 __global__ void __launch_bounds__(NT) colscale_kernel(const float4* in, const float4* h,
                                                       float4* __restrict__ out, int64_t n4, int cols4) {
@@ -70,17 +93,10 @@ __global__ void __launch_bounds__(NT) colscale_kernel(const float4* in, const fl
   }
 }
 
-__global__ void __launch_bounds__(NT) rowcolscale_kernel(const float* in, const float* cs,
-                                                         const float* rs, float* __restrict__ out,
-                                                         int64_t rows, int64_t cols) {
+// (in and out may be the same array)
+__global__ void __launch_bounds__(NT) scale_cols_kernel(const float* in, const float* cs, float* out, int64_t n, int64_t cols) {
   grid_begin();
-  const int64_t n = rows * cols;
-  for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
-    float v = in[i];
-    if (cs) v *= cs[i % cols];
-    if (rs) v *= rs[i / cols];
-    out[i] = v;
-  }
+  by_fours<float>(n, [&](int64_t i) { return in[i] * cs[i % cols]; }, [&](int64_t i, float v) { out[i] = v; });
 }
 
 // ---- H diagonal and diagonal blocks -------------------------------------------------------------
@@ -331,7 +347,7 @@ __global__ void identity_blocks_kernel(float* __restrict__ A, int db) {
 
 __global__ void copy_kernel(const float4* in, float4* __restrict__ out, int64_t n4) {
   grid_begin();
-  for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) out[i] = in[i];
+  by_fours<float4>(n4, [&](int64_t i) { return in[i]; }, [&](int64_t i, const float4& v) { out[i] = v; });
 }
 
 // ---- scalars and per-iteration bookkeeping ------------------------------------------------------
@@ -543,8 +559,7 @@ __global__ void screen_final_kernel(const int32_t* scr, int32_t* status) {
 __global__ void __launch_bounds__(NT) split_hilo_kernel(const float4* in, float4* __restrict__ hi,
                                                         float4* __restrict__ lo, int64_t n4) {
   grid_begin();
-  for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n4; i += (int64_t)gridDim.x * NT) {
-    float4 v = in[i];
+  by_fours<float4>(n4, [&](int64_t i) { return in[i]; }, [&](int64_t i, const float4& v) {
     float4 h;
     h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
     h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
@@ -552,7 +567,7 @@ __global__ void __launch_bounds__(NT) split_hilo_kernel(const float4* in, float4
     h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
     if (hi) hi[i] = h;
     lo[i] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
-  }
+  });
 }
 
 __device__ __forceinline__ float to_f32(float v) { return v; }
@@ -586,20 +601,14 @@ __global__ void __launch_bounds__(NT) bf16_to_f32_kernel(const __nv_bfloat16* in
                                                          const float* cs, float* __restrict__ out,
                                                          int64_t n, int64_t cols) {
   grid_begin();
-  for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
-    float v = __bfloat162float(in[i]);
-    if (cs) v *= cs[i % cols];
-    out[i] = v;
-  }
+  by_fours<float>(n, [&](int64_t i) { return cs ? __bfloat162float(in[i]) * cs[i % cols] : __bfloat162float(in[i]); },
+                  [&](int64_t i, float v) { out[i] = v; });
 }
 __global__ void __launch_bounds__(NT) f32_to_bf16_kernel(const float* in, const float* cs,
                                                          __nv_bfloat16* __restrict__ out, int64_t n, int64_t cols) {
   grid_begin();
-  for (int64_t i = (int64_t)blockIdx.x * NT + threadIdx.x; i < n; i += (int64_t)gridDim.x * NT) {
-    float v = in[i];
-    if (cs) v *= cs[i % cols];
-    out[i] = __float2bfloat16_rn(v);
-  }
+  by_fours<float>(n, [&](int64_t i) { return cs ? in[i] * cs[i % cols] : in[i]; },
+                  [&](int64_t i, float v) { out[i] = __float2bfloat16_rn(v); });
 }
 
 // H[r][c] = H[c][r] for c > r: the upper triangle from the lower one, 64 x 64 tiles through shared memory, 16 bytes an access
@@ -770,10 +779,9 @@ void launch_colscale(armor_ctx* c, const float* in, const float* h, float* out, 
   c->launches++;
 }
 
-void launch_scale_rows_cols(armor_ctx* c, const float* in, const float* colscale, const float* rowscale, float* out,
-                            int64_t rows, int64_t cols, cudaStream_t s) {
+void launch_scale_cols(armor_ctx* c, const float* in, const float* colscale, float* out, int64_t rows, int64_t cols, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_FORWARD, 8.0 * (double)rows * (double)cols, s);
-  launch_dependent(rowcolscale_kernel, grid_for(rows * cols), NT, 0, s, in, colscale, rowscale, out, rows, cols);
+  launch_dependent(scale_cols_kernel, grid_for(rows * cols), NT, 0, s, in, colscale, out, rows * cols, cols);
   c->launches++;
 }
 

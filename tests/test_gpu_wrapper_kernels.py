@@ -70,6 +70,31 @@ def test_bf16_forward_on_either_side_of_the_choice(tiles_per_sm):
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_conversions_and_scales_of_every_remainder(dtype):
+    """The passes over the activations of a denormalised forward take four elements a thread: token counts at one to five times the
+    2,368 x 256 elements of a round, one token on either side.  Integer operands and scales that are powers of two: the bits of fp64."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(148)
+    d_out, d_in, most = 1024, 4096, 741
+
+    def sparse_ints(hi, density, *shape):
+        return torch.randint(-hi, hi + 1, shape, device=DEV, generator=g).float() * (torch.rand(shape, device=DEV, generator=g) < density)
+    S = sparse_ints(3, 0.25, d_out, d_in)
+    A, B = (sparse_ints(1, 4.0 / 128, d // 128, 128, 128) for d in (d_out, d_in))
+    r1, r2 = (torch.exp2(torch.randint(0, 2, (d,), device=DEV, generator=g).float()) for d in (d_in, d_out))
+    x = sparse_ints(2, 0.25, most, d_in).to(dtype)
+    z1 = torch.einsum("tjk,jmk->tjm", (x.double() * r1).view(most, -1, 128), B.double()).reshape(most, d_in)
+    z2 = z1 @ S.double().t()
+    assert z1.abs().max() < 256 and z2.abs().max() < 2 ** 11
+    y = (torch.einsum("tjk,jmk->tjm", z2.view(most, -1, 128), A.double()).reshape(most, d_out) * r2).to(dtype)
+    ctx = _ctx(d_out, d_in, 128, h_mode=Bd.H_DIAG)
+    st = Bd.LayerState(Wbar=S, A=A, B=B, S=S, M=torch.zeros(d_out, d_in // 4, dtype=torch.uint8, device=DEV), r1=r1, r2=r2)
+    for n in (1, 3, 147, 148, 149, 295, 296, 297, 443, 444, 445, 591, 592, 593, 739, 740, 741):
+        assert torch.equal(ctx.apply(st, x[:n].contiguous(), denormalize=True), y[:n]), n
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
 @pytest.mark.parametrize("d_out,d_in,d_block", [(128, 128, 128), (256, 640, 128), (1024, 5120, 128), (2560, 1152, 128), (256, 256, 256),
                                                 (768, 1280, 256), (2368, 1216, 64), (1216, 2368, 64)])
 @pytest.mark.parametrize("fused", [1, 0])
