@@ -149,7 +149,7 @@ struct armor_ctx {
 static const int ARMOR_MAX_TIMED = 8192;
 
 // ---------------------------------------------------------------- programmatic dependent launches
-// The kernels of an iteration are short (a layer of 256 x 256: 41 launches of 2 to 4 us), so the gap between the end of one and
+// The kernels of an iteration are short (a layer of 256 x 256: 41 launches, most of them of 2 to 4 us, solves 10, contractions of 256 7 to 9), so the gap between the end of one and
 // the start of the next counts.  They open with grid_begin(): launched with the attribute below, a kernel's CTAs are put on the
 // SMs once every CTA of the kernel before it has come past its own grid_begin(), and wait there until that kernel has ended and
 // its writes are visible; everything earlier in the stream has ended by then as well.  (Letting the next kernel in before
@@ -368,10 +368,12 @@ void launch_colscale(armor_ctx* c, const float* in, const float* h, float* out, 
 void launch_extract_hblocks(armor_ctx* c, const float* H, cudaStream_t s);   // hdiag, Hjj (per h_mode)
 void launch_masked_copy(armor_ctx* c, const float* Gam, const uint8_t* M, float* out, double* part,
                         cudaStream_t s);              // out = Gam (.) M; ARMOR_DOT_BLOCKS partial sums of ||out||^2
+// y += sign * sc[slot] * x; for up to three arrays at once, the last may move by sc[slot_before] * x2_before first
 void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slot, float sign,
                       cudaStream_t s);
 void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64_t n0, float* y1, const float* x1, float s1,
-                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s, const float* x2_before = nullptr, int slot_before = 0);                                       // y += sign * sc[slot] * x
+                       int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s,
+                       const float* x2_before = nullptr, int slot_before = 0);
 void launch_init(armor_ctx* c, const float* W, const float* H, float* Wbar, float* r1, float* r2,
                  float* A, float* B, float* S, uint8_t* M, cudaStream_t s);
 // st: base of the iteration records (the kernels add c->it_dev), or null

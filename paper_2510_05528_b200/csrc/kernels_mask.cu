@@ -558,7 +558,7 @@ void launch_mask_carry_P(armor_ctx* c, float* P, cudaStream_t s) {
   const int nbv = c->nbi * c->kg;
   int groups = (nbv + CARRY_PICKS - 1) / CARRY_PICKS;
   if (groups > CARRY_CTAS) groups = CARRY_CTAS;
-  launch_dependent(mask_carry_kernel, dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s, 
+  launch_dependent(mask_carry_kernel, dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s,
       c->sel, c->Ysel, P, c->sc, c->d_in, c->db, c->nbo_pad, nbv);
   c->launches++;
 }
@@ -657,10 +657,11 @@ void launch_mask_select(armor_ctx* c, const float* Gam, const float* S, const ui
       if (smem > 48 * 1024)                                                                                             \
         cudaFuncSetAttribute(mask_select_kernel<MGV, NKV, MULTIV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                              (int)smem);                                                                                \
-      launch_dependent(mask_select_kernel<MGV, NKV, MULTIV, 0>, c->nbo * c->nbi, NT, smem, s, ARMOR_SELECT_ARGS);                     \
+      launch_dependent(mask_select_kernel<MGV, NKV, MULTIV, 0>, c->nbo * c->nbi, NT, smem, s, ARMOR_SELECT_ARGS);       \
     } else {                                                                                                            \
-      launch_dependent(mask_select_kernel<MGV, NKV, false, 1>, c->nbo * c->nbi, NT, 0, s, ARMOR_SELECT_ARGS);                         \
-      launch_dependent(mask_select_kernel<MGV, NKV, false, 2>, c->nbo * c->nbi, MGV == 4 ? 32 : NT, 0, s, ARMOR_SELECT_ARGS);         \
+      launch_dependent(mask_select_kernel<MGV, NKV, false, 1>, c->nbo * c->nbi, NT, 0, s, ARMOR_SELECT_ARGS);           \
+      launch_dependent(mask_select_kernel<MGV, NKV, false, 2>, c->nbo * c->nbi, MGV == 4 ? 32 : NT, 0, s,               \
+                       ARMOR_SELECT_ARGS);                                                                              \
       c->launches++;                                                                                                    \
     }                                                                                                                   \
   } while (0)

@@ -787,7 +787,8 @@ void launch_scale_cols(armor_ctx* c, const float* in, const float* colscale, flo
 
 void launch_extract_hblocks(armor_ctx* c, const float* H, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  launch_dependent(extract_hblocks_kernel, dim3(c->nbi, (c->db + HB_ROWS - 1) / HB_ROWS), NT, 0, s, H, c->hdiag, c->Hjj, c->d_in, c->db, c->cfg.h_mode == ARMOR_H_DIAG);
+  launch_dependent(extract_hblocks_kernel, dim3(c->nbi, (c->db + HB_ROWS - 1) / HB_ROWS), NT, 0, s, H, c->hdiag, c->Hjj, c->d_in, c->db,
+                   c->cfg.h_mode == ARMOR_H_DIAG);
   c->launches++;
 }
 
