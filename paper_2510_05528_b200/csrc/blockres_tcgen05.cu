@@ -10,7 +10,7 @@
 //   one product : 128 x 128 x 8 instructions into two accumulators in turn, four epilogue warps for each, so that the
 //                 MMAs of a tile run while the tile before is stored.  (With one accumulator of 256 columns, two tiles per
 //                 instruction, the MMAs waited for the epilogue and the pass was no faster than the streaming kernel.)
-//                 Left at 4096 x 4096: 31 us, 38 with an addend, against 37 and 44 there and 25 for a copy; with operands formed
+//                 Left at 4096 x 4096, from HBM: 30 us, 39 with an addend, against 33 and 46 there and 25 for a copy; with operands formed
 //                 in front of every MMA by one lane (tc_common.cuh, umma_tf32_ta_w) it took 34 and 40.
 //   dual product: A.X1 and A.X2 of a tile in one 128 x 256 x 8 instruction.
 //   side "left":   out[128 b + m][n]  = alpha * sum_k Qop_b[m][k] * X[128 b + k][n]  (+ beta * add)
