@@ -21,7 +21,7 @@
 // sides each (40 blocks: 59 us a launch against 52).
 // A launch, d_block 128: 32 blocks over 4 CTAs each 46.5 us (62.2 with the panel's elimination unrolled and a row a thread in the last
 // panels' updates), 40 blocks over 2 to 4 CTAs 50.6 (65.1), 112 and 32 blocks 59.4 on average (74.4); d_block 32, 8 blocks 16 k cycles
-// (22 k); d_block 256, a 28672 x 8192 layer's launches of 112 and 32 blocks 449 us on average (505 to 520).
+// (22 k); d_block 256 (chol_ctas_per_block), 40 and 56 blocks 240 us (312 with a CTA per slice), 112 blocks of a 28672 x 8192 layer 630 (956).
 #include "armor_internal.cuh"
 
 namespace {
@@ -346,10 +346,10 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
   __shared__ double red[NT / 32];
   __shared__ int s_fail;
   __shared__ double s_lam;
-  const int b = blockIdx.x, q = blockIdx.y, tid = threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = blockIdx.x, tid = threadIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t off = (int64_t)b * db * db;
   const bool right = (mode != 1);
-  const int v0 = q * W;                                 // first right-hand side of this CTA
+  const int slices = (db + W - 1) / W;                  // of the block's right-hand sides; this CTA takes every gridDim.y-th
   const int q4 = db / 4;                                // 16-byte units per row
 
   // ---- load: the units of G on and below the diagonal, then the right-hand sides
@@ -361,20 +361,23 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
   }
   // A right solve's right-hand side is a row of rhs (eight lanes along it, four rows per warp access), a left solve's a
   // column (lanes along the row of rhs).  Right-hand sides past the end are zeros.
-  if (right) {
+  auto load_rhs = [&](int v0) {
+    if (right) {
 #pragma unroll 4
-    for (int e = tid; e < W * q4; e += NT) {
-      const int c8 = e & 7, v = (e >> 3) % W, i = 4 * (c8 + 8 * ((e >> 3) / W));
-      const float4 x = v0 + v < db ? ld4(rhs + off + (int64_t)(v0 + v) * db + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-      X[i * LDX + v] = x.x; X[(i + 1) * LDX + v] = x.y; X[(i + 2) * LDX + v] = x.z; X[(i + 3) * LDX + v] = x.w;
-    }
-  } else {
+      for (int e = tid; e < W * q4; e += NT) {
+        const int c8 = e & 7, v = (e >> 3) % W, i = 4 * (c8 + 8 * ((e >> 3) / W));
+        const float4 x = v0 + v < db ? ld4(rhs + off + (int64_t)(v0 + v) * db + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+        X[i * LDX + v] = x.x; X[(i + 1) * LDX + v] = x.y; X[(i + 2) * LDX + v] = x.z; X[(i + 3) * LDX + v] = x.w;
+      }
+    } else {
 #pragma unroll 8
-    for (int e = tid; e < W * db; e += NT) {
-      const int v = e % W, i = e / W;
-      X[i * LDX + v] = v0 + v < db ? rhs[off + (int64_t)i * db + v0 + v] : 0.f;
+      for (int e = tid; e < W * db; e += NT) {
+        const int v = e % W, i = e / W;
+        X[i * LDX + v] = v0 + v < db ? rhs[off + (int64_t)i * db + v0 + v] : 0.f;
+      }
     }
-  }
+  };
+  load_rhs((int)blockIdx.y * W);
   asm volatile("cp.async.wait_all;" ::: "memory");
   if (tid == 0) s_fail = 0;
   __syncthreads();
@@ -404,6 +407,13 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
   const bool fail = (s_fail != 0);
   const bool hold = (mode == 0) && status[ST_POISON] != 0;   // unusable inputs: the A-step is withheld (X = 0)
 
+  for (int q = blockIdx.y; q < slices; q += gridDim.y) {
+  const int v0 = q * W;                                 // first right-hand side of the slice
+  if (q != (int)blockIdx.y) {                           // (the first one has come with the factor)
+    __syncthreads();
+    load_rhs(v0);
+    __syncthreads();
+  }
   if (!fail) {
     // ---- forward substitution  L y = r, then backward substitution  L^T x = y
     for (int kb = 0; kb < np; ++kb) solve_block<false, G>(Lp, pm, invd, X, LDX, kb);
@@ -463,10 +473,11 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
     if (tid == 0) {
       double t = 0.0;
       for (int wp = 0; wp < NT / 32; ++wp) t += red[wp];
-      part[(int64_t)b * gridDim.y + q] = t;
+      part[(int64_t)b * slices + q] = t;
     }
   }
-  if (tid == 0 && q == 0 && fail) {
+  }
+  if (tid == 0 && blockIdx.y == 0 && fail) {
     failflag[b] = 1;
     atomicCAS(&status[ST_FIRST_FAIL], 0, b + 1);
   }
@@ -584,6 +595,23 @@ int chol_groups(int db, int nb) {
   return 4;
 }
 
+// CTAs per block, each of which factorises it and then solves for its share of the block's slices of right-hand sides.  A
+// block of up to 128 has a CTA for each slice.  One of 256 fills an SM's shared memory, so that 56 or 112 blocks in four slices came in
+// two and four waves that each repeated the factorisation: the number of CTAs with the shortest chain of waves, a factorisation
+// counted as FACTOR_SLICES slices.
+constexpr double FACTOR_SLICES = 0.8;
+int chol_ctas_per_block(int db, int nb, int n_sm, int slices) {
+  if (db <= 128) return slices;
+  int best = slices;
+  double least = 0.0;
+  for (int y = slices; y >= 1; --y) {
+    const int waves = (nb * y + n_sm - 1) / n_sm;
+    const double t = waves * (FACTOR_SLICES + (slices + y - 1) / y);
+    if (y == slices || t < least) { least = t; best = y; }
+  }
+  return best;
+}
+
 template <int G>
 armor_status launch_blocked(armor_ctx* c, int mode, const float* Gm, const float* rhs, float* out, const float* dotw, float* A,
                             int nb, double* part, cudaStream_t s) {
@@ -594,7 +622,8 @@ armor_status launch_blocked(armor_ctx* c, int mode, const float* Gm, const float
   if (ensure_dynamic_smem(attr, c->device, chol_blocked_kernel<G>,
                           (panel_floats(widest) + (size_t)widest * (32 * G + 1)) * sizeof(float)) != ARMOR_OK)
     return ARMOR_ERR_CUDA;
-  launch_dependent(chol_blocked_kernel<G>, dim3(nb, (db + 32 * G - 1) / (32 * G)), NT, smem, s, mode, Gm, rhs, out, dotw, A, c->cfg.ridge, db,
+  const int slices = (db + 32 * G - 1) / (32 * G);
+  launch_dependent(chol_blocked_kernel<G>, dim3(nb, chol_ctas_per_block(db, nb, c->n_sm, slices)), NT, smem, s, mode, Gm, rhs, out, dotw, A, c->cfg.ridge, db,
                                                                                   part, c->failflag, c->status);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
@@ -602,7 +631,7 @@ armor_status launch_blocked(armor_ctx* c, int mode, const float* Gm, const float
 
 }  // namespace
 
-// The right-hand sides of one block are dealt to this many CTAs (at most four), each of which repeats the factorisation.
+// The right-hand sides of one block come in this many slices (at most four), with a partial sum each.
 int chol_parts_per_block(int db, int nb) {
   if (db % NB) return 1;
   const int w = 32 * chol_groups(db, nb);

@@ -529,3 +529,35 @@ def test_column_grams_with_blocks_of_256(d_out, d_in):
         tau = (got * D).sum() / (D * D).sum()
         assert abs(tau - 1.0) < 1e-3 and (got - tau * D).norm() <= 1e-4 * D.norm()
     assert (moved[1] - moved[0]).norm() <= 1e-5 * moved[1].norm()
+
+
+@pytest.mark.parametrize("nb_out", [37, 38, 75, 112])
+def test_solves_of_256_in_several_slices_a_cta(nb_out):
+    """More blocks of 256 than a wave of CTAs takes in four slices: two slices or four to a CTA, one factorisation each."""
+    test_block_solves(256, nb_out, 1)
+
+
+@pytest.mark.parametrize("nb_in", [37, 38, 75])
+def test_left_solves_of_256_in_several_slices_a_cta(nb_in):
+    """The B-step's solve and the inverse of H_jj with the diagonal weighting: B - I = (S_j^T S_j + lam I)^-1 Gamma_j (D_j + mu I)^-1.
+    fp32 solves of systems whose condition number is below 1e3: 1e-4 of the result."""
+    from paper_2510_05528_b200 import binding as Bd
+    db, d_out = 256, 2048
+    d_in = nb_in * db
+    g = _gen(nb_in)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    h = torch.rand(d_in, device=DEV, generator=g) + 0.5
+    H = torch.diag(h)
+    ctx = _ctx(d_out, d_in, db, h_mode=Bd.H_DIAG, phases=2)   # B-step alone
+    st = ctx.init(W, H)
+    S = st.S.double().view(d_out, nb_in, db).transpose(0, 1)
+    E = (W - st.S).double().view(d_out, nb_in, db).transpose(0, 1)
+    D = h.double().view(nb_in, 1, db)
+    ctx.bcd_step(st, H, 0, 1)
+    eye = torch.eye(db, device=DEV, dtype=torch.float64)
+    C = S.transpose(1, 2) @ S
+    C = C + 1e-6 * C.diagonal(dim1=1, dim2=2).mean(1)[:, None, None] * eye
+    assert torch.linalg.cond(C).max() < 1e3
+    X = torch.linalg.solve(C, S.transpose(1, 2) @ (E * D)) / (D + 1e-6 * D.mean(2, keepdim=True))
+    assert (st.B.double() - eye - X).norm() <= 1e-4 * X.norm()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
