@@ -264,9 +264,9 @@ armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const fl
                           float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s, const uint8_t* mask = nullptr,
                           double* norm_part = nullptr, int* n_norm = nullptr);
 
-// E = add - Ablk in, EH = E diag(colw), partial sums of <E, EH> at part: one launch
+// EH = E diag(colw) with E = add - Ablk in, partial sums of <E, EH> at part: one launch, E stays in the SMs
 armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* in, const float* add, const float* colw,
-                                 float* E, float* EH, int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
+                                 float* EH, int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
 
 // the same with the wrapper block held in tensor memory (blockres_tcgen05.cu); d_block = 128
 bool tc_blockres_ok(const armor_ctx* c);
@@ -274,7 +274,8 @@ armor_status tc_blockres_right(armor_ctx* c, const float* in, const float* Bblk,
                                int64_t cols, float alpha, const float* add, float beta, cudaStream_t s,
                                const float* colw = nullptr, float* out2 = nullptr);
 armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
-                              int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
+                              int64_t cols, float alpha, const float* add, float beta, cudaStream_t s, const float* colw = nullptr,
+                              double* part = nullptr);
 
 armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* out,
                                    int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);

@@ -62,9 +62,11 @@ struct BParams {
   int one_pass;                     // 1: operands as they are, rounded to tf32 by the tensor core; no low parts
   int dual;                         // 1: two B operands per tile (mapB, mapB2); C = alpha * A.B2, dot_part = <A.B1, A.B2>
   double* dot_part;                 // dual, colw: 4 partial sums per tile (one per epilogue warp), in tile order
-  const float* colw;                // not null: a second output C2 (through mapB2) = C scaled per column by colw, and
-                                    // dot_part = sum of C * C2 (the residual, its weighted form and the loss of the
-                                    // diagonal weighting, Eq. 2 with H_w = diag(h), in one pass)
+  const float* colw;                // not null: with E = alpha * A.B + beta * D the output is E scaled per column by colw, and
+                                    // dot_part = sum of E * (E scaled): the weighted residual and the loss of the diagonal
+                                    // weighting (Eq. 2 with H_w = diag(h)) in one pass.  E itself is needed nowhere (written
+                                    // as well it cost 268 MB instead of 201 and a second trip through the boxes: 69 us
+                                    // a launch at 4096 x 4096)
 };
 
 __device__ __forceinline__ void load_operand(uint32_t dst, const CUtensorMap* map, const OpCoord& o, int b, int t, int kc,
@@ -100,6 +102,8 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t base, int mn_major, in
 }
 
 
+// COLW: with column scales (an instantiation of its own: as a branch of the store loop it cost every plain product 10 %)
+template <bool COLW>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CUtensorMap mapB2, const __grid_constant__ CUtensorMap mapC,
@@ -279,7 +283,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
       const uint32_t aphase = (uint32_t)(local >> 1) & 1u;
       const int64_t row_base = p.r_b * b + (int64_t)tm * TILE + q * 32;
       const int64_t col_tile = p.c_b * b + (int64_t)tn * TILE;
-      if (p.dual) {
+      if (!COLW && p.dual) {
         // C = alpha * (A.B2); partial sum of <A.B1, A.B2> over this warp's 32 x 128 slab (rows or columns past the
         // end of the operands were read as zeros and add nothing)
         double dot = 0.0;
@@ -339,6 +343,8 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
         int n_box = 0;
         if (row_base < p.c_rows && tm * TILE + q * 32 < p.m_valid)
           for (int ch = 0; ch < 2; ++ch) n_box += (col_tile + 64 * hf + 32 * ch < p.c_cols) ? 1 : 0;
+        float cw0 = 0.f, cw1 = 0.f;                 // colw: lane l holds the scale of column l of each box (handed round by shuffles)
+        if (COLW) { cw0 = __ldg(p.colw + col_tile + 64 * hf + lane); cw1 = __ldg(p.colw + col_tile + 64 * hf + 32 + lane); }
         if (lane == 0) {
           tma_store_wait_read();                    // the previous stores have read the staging boxes
           if (p.D && n_box > 0) {
@@ -357,6 +363,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
           if (!mbar_wait(dbar, d_loads & 1u, abortp, p.status)) { ok = false; break; }
           ++d_loads;
         }
+        float wpart = 0.f;
 #pragma unroll 1
         for (int ch = 0; ch < 2; ++ch) {
           uint32_t r[32];
@@ -364,6 +371,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
           if (ch >= n_box) continue;                // warp-uniform
           // lane = row of the box; 16-byte chunk c of the row sits at chunk c ^ (row % 8)  (128-byte swizzle)
           uint8_t* rowp = buf + ch * 4096 + lane * 128;
+          const float w = ch ? cw1 : cw0;
 #pragma unroll
           for (int cq = 0; cq < 8; ++cq) {
             float4* cell = reinterpret_cast<float4*>(rowp + ((cq ^ (lane & 7)) << 4));
@@ -374,9 +382,16 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
               v.x = fmaf(p.beta, d.x, v.x); v.y = fmaf(p.beta, d.y, v.y);
               v.z = fmaf(p.beta, d.z, v.z); v.w = fmaf(p.beta, d.w, v.w);
             }
+            if (COLW) {
+              const float4 e = make_float4(v.x * __shfl_sync(0xffffffffu, w, 4 * cq), v.y * __shfl_sync(0xffffffffu, w, 4 * cq + 1),
+                                           v.z * __shfl_sync(0xffffffffu, w, 4 * cq + 2), v.w * __shfl_sync(0xffffffffu, w, 4 * cq + 3));
+              wpart = fmaf(v.x, e.x, wpart); wpart = fmaf(v.y, e.y, wpart); wpart = fmaf(v.z, e.z, wpart); wpart = fmaf(v.w, e.w, wpart);
+              v = e;
+            }
             *cell = v;
           }
         }
+        if (COLW) wdot += (double)wpart;
         if (hf == 1) tc_fence_before();             // all reads of the accumulator are done
         fence_proxy_async();
         __syncwarp();
@@ -386,34 +401,8 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
             tma_store_2d(&mapC, (int)(col_tile + 64 * hf + 32 * ch), (int)row_base, buf_u32 + ch * 4096);
           tma_store_commit();
         }
-        if (p.colw) {
-          // the boxes still hold C: once the store has read them they become C2 = C * colw[column]
-          if (lane == 0) tma_store_wait_read();
-          __syncwarp();
-          float part = 0.f;
-          for (int ch = 0; ch < n_box; ++ch) {
-            const float4* w4 = reinterpret_cast<const float4*>(p.colw + col_tile + 64 * hf + 32 * ch);
-            uint8_t* rowp = buf + ch * 4096 + lane * 128;
-#pragma unroll
-            for (int cq = 0; cq < 8; ++cq) {
-              float4* cell = reinterpret_cast<float4*>(rowp + ((cq ^ (lane & 7)) << 4));
-              const float4 v = *cell, w = __ldg(w4 + cq);
-              const float4 e = make_float4(v.x * w.x, v.y * w.y, v.z * w.z, v.w * w.w);
-              part = fmaf(v.x, e.x, part); part = fmaf(v.y, e.y, part); part = fmaf(v.z, e.z, part); part = fmaf(v.w, e.w, part);
-              *cell = e;
-            }
-          }
-          wdot += (double)part;
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) {
-            for (int ch = 0; ch < n_box; ++ch)
-              tma_store_2d(&mapB2, (int)(col_tile + 64 * hf + 32 * ch), (int)row_base, buf_u32 + ch * 4096);
-            tma_store_commit();
-          }
-        }
       }
-      if (p.colw) {
+      if (COLW) {
         // lanes in a fixed order
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wdot += __shfl_xor_sync(0xffffffffu, wdot, o);
@@ -435,9 +424,10 @@ struct HostOp {
   OpCoord c;
 };
 
-// B2: the second N-side operand (dual); C2: the second output (colw)
+// B2: the second N-side operand (dual)
+template <bool COLW = false>
 armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, int kclass, double kbytes, cudaStream_t s,
-                    const float* B2 = nullptr, float* C2 = nullptr) {
+                    const float* B2 = nullptr) {
   CUtensorMap mA, mB, mB2, mC, mD;
   if (!make_map_2d(&mC, p.C, p.c_cols, p.c_rows, p.ldc, 32, 32)) return ARMOR_ERR_CUDA;
   if (p.D) {
@@ -447,11 +437,7 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, i
   }
   if (!make_map_2d(&mA, A.base, A.inner, A.outer, A.ld, 32, A.c.mn_major ? 32 : TILE, A.c.mn_major != 0)) return ARMOR_ERR_CUDA;
   if (!make_map_2d(&mB, B.base, B.inner, B.outer, B.ld, 32, B.c.mn_major ? 32 : TILE, B.c.mn_major != 0)) return ARMOR_ERR_CUDA;
-  if (p.colw) {
-    // the second output has the geometry of C
-    if (!C2 || p.dual) return ARMOR_ERR_INVALID_ARG;
-    if (!make_map_2d(&mB2, C2, p.c_cols, p.c_rows, p.ldc, 32, 32)) return ARMOR_ERR_CUDA;
-  } else if (B2) {
+  if (B2) {
     if (!make_map_2d(&mB2, B2, B.inner, B.outer, B.ld, 32, B.c.mn_major ? 32 : TILE, B.c.mn_major != 0)) return ARMOR_ERR_CUDA;
   } else {
     mB2 = mB;
@@ -459,12 +445,12 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, i
   p.a = A.c; p.b = B.c;
   p.status = c->status;
   static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_block_kernel, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  if (ensure_dynamic_smem(attr, c->device, tc_block_kernel<COLW>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int n_sm = c->n_sm;
   const int n_items = p.batch * p.m_tiles * p.n_tiles;
   const int grid = n_items < n_sm ? n_items : n_sm;
   KTimer kt(c, kclass, kbytes, s);
-  launch_dependent(tc_block_kernel, grid, NTHREADS, SMEM_BYTES, s, mA, mB, mB2, mC, mD, p);
+  launch_dependent(tc_block_kernel<COLW>, grid, NTHREADS, SMEM_BYTES, s, mA, mB, mB2, mC, mD, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
@@ -478,9 +464,11 @@ inline bool ptr_ok(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15)
 // bytes of every row, which costs more than the saved shared-memory traffic while there are few tiles.  This kernel / that one:
 // right 1024 x 5120 (2.2 tiles per SM) 17.7 / 21.2 us, 4096 x 4096 (6.9) 32.7 / 34.7, 6144 x 4096 (10.4) 48.0 / 50.9, 8192 x 4096 (13.8)
 // 63.7 / 57.9, 14336 x 4096 (24) 98 / 93; left 2048 x 2048 (1.7) 13.9 / 15.2, 1024 x 5120 17.4 / 18.2, 2048 x 4096 (3.5) 23.4 / 20.8, 4096 x 4096
-// 32.9 / 30.7, 14336 x 4096 98 / 89.  Products of one pass (the bf16 forward) have no low parts to save and stay here: forward of 6144 x 6144,
+// 32.9 / 30.7, 14336 x 4096 98 / 89; left with an addend, whose trips through the staging boxes eight epilogue warps share there
+// instead of four, 1024 x 2048 (0.9) 9.6 / 11.0, 2048 x 2048 16.3 / 16.0, 1024 x 5120 22.2 / 20.0, 4096 x 4096 46.2 / 37.7, and scaled per column (the
+// residual of the diagonal weighting) 4096 x 4096 50 / 38, 14336 x 4096 124 there.  Products of one pass (the bf16 forward) have no low parts to save and stay here: forward of 6144 x 6144,
 // 4,736 tokens, packed core, 443 / 454 us, 8192 x 8192, 8,192 tokens 1,068 / 1,097.
-static const int RES_RIGHT = 12, RES_LEFT = 3;
+static const int RES_RIGHT = 12, RES_LEFT = 3, RES_LEFT_ADD = 2;
 
 bool tc_block_ok(const armor_ctx* c, int64_t rows, int64_t cols) {
   return c->cfg.precision != ARMOR_PREC_SIMT && c->db % TILE == 0 && rows > 0 && cols % 4 == 0;
@@ -514,7 +502,7 @@ armor_status tc_bd_right(armor_ctx* c, const float* in, const float* Bblk, bool 
 // out[i-th block, :] = alpha * P_i * in[i-th block, :] (+ beta * add[i-th block, :]),  P_i = Ablk[i] or its transpose
 armor_status tc_bd_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
                         int64_t cols, float alpha, const float* add, float beta, cudaStream_t s) {
-  const bool res = c->tc_blocks == 2 || (c->tc_blocks != 1 && (rows / TILE) * ((cols + TILE - 1) / TILE) >= (int64_t)RES_LEFT * c->n_sm);
+  const bool res = c->tc_blocks == 2 || (c->tc_blocks != 1 && (rows / TILE) * ((cols + TILE - 1) / TILE) >= (int64_t)(add ? RES_LEFT_ADD : RES_LEFT) * c->n_sm);
   if (res && tc_blockres_ok(c)) return tc_blockres_left(c, Ablk, transA, in, out, rows, cols, alpha, add, beta, s);
   if (c->tc_blocks != 1 && tc_blockpair_ok(c, (rows / 256) * ((cols + 255) / 256)))
     return tc_blockpair_left(c, Ablk, transA, in, out, rows, cols, alpha, add, beta, s);
@@ -565,17 +553,22 @@ armor_status tc_bd_left_dual(armor_ctx* c, const float* Ablk, bool transA, const
   return launch(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, 12.0 * (double)rows * (double)cols, s, in2);
 }
 
-// E = add - P_i * in per block row, EH = E scaled per column by colw, and 4 partial sums per 128 x 128 tile of <E, EH> at
-// part (the residual E = W - A T, E diag(h) and the proxy loss of the diagonal weighting in one pass)
+// EH = E scaled per column by colw, E = add - P_i * in per block row, and 4 partial sums per 128 x 128 tile of <E, EH> at
+// part (the residual E = W - A T, E diag(h) and the proxy loss of the diagonal weighting in one pass; E stays in the SMs)
 armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* in, const float* add, const float* colw,
-                                 float* E, float* EH, int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s) {
+                                 float* EH, int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s) {
   const int db = c->db;
   const int nb = (int)(rows / db);
-  if (!ptr_ok(in) || !ptr_ok(Ablk) || !ptr_ok(add) || !ptr_ok(colw) || !ptr_ok(E) || !ptr_ok(EH) || cols % TILE) return ARMOR_ERR_UNSUPPORTED;
+  if (!ptr_ok(in) || !ptr_ok(Ablk) || !ptr_ok(add) || !ptr_ok(colw) || !ptr_ok(EH) || cols % TILE) return ARMOR_ERR_UNSUPPORTED;
+  const bool res = c->tc_blocks == 2 || (c->tc_blocks != 1 && (rows / TILE) * (cols / TILE) >= (int64_t)RES_LEFT_ADD * c->n_sm);
+  if (res && tc_blockres_ok(c)) {
+    *n_part = 4 * (int)((rows / TILE) * (cols / TILE));
+    return tc_blockres_left(c, Ablk, false, in, EH, rows, cols, -1.f, add, 1.f, s, colw, part);
+  }
   HostOp A{Ablk, db, (int64_t)nb * db, db, {0, 0, 0, BK, db, TILE, 0}};
   HostOp B{in, cols, rows, cols, {1, 0, TILE, 0, db, 0, BK}};
   BParams p{};
-  p.C = E; p.D = add; p.ldc = cols; p.ldd = cols; p.c_rows = rows; p.c_cols = cols;
+  p.C = EH; p.D = add; p.ldc = cols; p.ldd = cols; p.c_rows = rows; p.c_cols = cols;
   p.r_b = db; p.c_b = 0;
   p.m_tiles = db / TILE; p.n_tiles = (int)(cols / TILE); p.batch = nb; p.k_chunks = db / BK;
   p.alpha = -1.f; p.beta = 1.f;
@@ -583,8 +576,8 @@ armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* i
   p.one_pass = c->block_one_pass;
   p.colw = colw; p.dot_part = part;
   *n_part = 4 * p.batch * p.m_tiles * p.n_tiles;
-  // two W-shaped reads (in, add), two writes
-  return launch(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, 16.0 * (double)rows * (double)cols, s, nullptr, EH);
+  // two W-shaped reads (in, add), one write
+  return launch<true>(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, 12.0 * (double)rows * (double)cols, s);
 }
 
 namespace {

@@ -71,11 +71,11 @@ struct RParams {
   int tiles, batch;                 // tiles per wrapper block along the free dimension; work = batch * tiles tiles
   float alpha, beta;
   int32_t* status;
-  const float* colw;                // one product, right: not null: a second output (through mapX2) = out scaled per
-                                    // column by colw
+  const float* colw;                // one product, not null: right: a second output (through mapX2) = out scaled per column by
+                                    // colw; left: out itself is scaled per column, dot_part = sum of out * out scaled
   // dual (left only): the two halves of an instruction are the same tile of two inputs (mapX, mapX2);
   // out = alpha * Q.X2, dot_part = <Q.X1, Q.X2>
-  double* dot_part;                 // dual: 8 partial sums per tile (one per epilogue warp), in tile order
+  double* dot_part;                 // dual: 8 partial sums per tile (one per epilogue warp), left with colw: 4, in tile order
 };
 
 // One tile of one wrapper block.
@@ -92,7 +92,8 @@ __device__ __forceinline__ uint64_t x_desc(uint32_t base, int mn_major, int kste
   return mn_major ? smem_desc_mn_sw128_32b(base + kstep * 1024, 4096, 512) : smem_desc_sw128(base + kstep * 32, 16, 1024);
 }
 
-template <bool DUAL>
+// SCALED: left product with column scales (an instantiation of its own, so that plain products stay as they are)
+template <bool DUAL, bool SCALED>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapX2,
                    const __grid_constant__ CUtensorMap mapQ,
@@ -441,9 +442,15 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
         for (int ch = 0; ch < 2; ++ch)
           n_box[hf] += (bx0[hf] + bxs * ch < p.c_cols && by0[hf] + bys * ch < p.c_rows) ? 1 : 0;
       }
+      // left with colw: a half's column scales, lane l holding column l of each box; they travel while the MMAs run or the
+      // addend is waited for, and go round by shuffles
+      float cw0 = 0.f, cw1 = 0.f;
+      if (SCALED) { cw0 = __ldg(p.colw + col_tile + lane); cw1 = __ldg(p.colw + col_tile + 32 + lane); }
+      double wdot = 0.0;
+      float wpart = 0.f;
       // alpha * accumulator (+ beta * addend, which sits in the box already) into staging box ch
-      auto stage_box = [&](int ch, const uint32_t (&r)[32]) {
-        if (p.right) {
+      auto stage_box = [&](int ch, const uint32_t (&r)[32], float w) {
+        if (!SCALED && p.right) {
           // r[i] = out[by + i][bx + lane]: word `lane` of box row i; 16-byte chunk c of a row sits at chunk
           // c ^ (row % 8)  (128-byte swizzle)
           uint8_t* colp = buf + ch * 4096 + (lane & 3) * 4;
@@ -466,6 +473,13 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
               const float4 d = *cell;
               v.x = fmaf(p.beta, d.x, v.x); v.y = fmaf(p.beta, d.y, v.y);
               v.z = fmaf(p.beta, d.z, v.z); v.w = fmaf(p.beta, d.w, v.w);
+            }
+            if (SCALED) {
+              const float4 e4 = make_float4(v.x * __shfl_sync(0xffffffffu, w, 4 * cq), v.y * __shfl_sync(0xffffffffu, w, 4 * cq + 1),
+                                            v.z * __shfl_sync(0xffffffffu, w, 4 * cq + 2), v.w * __shfl_sync(0xffffffffu, w, 4 * cq + 3));
+              wpart = fmaf(v.x, e4.x, wpart); wpart = fmaf(v.y, e4.y, wpart);
+              wpart = fmaf(v.z, e4.z, wpart); wpart = fmaf(v.w, e4.w, wpart);
+              v = e4;
             }
             *cell = v;
           }
@@ -491,7 +505,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
             tma_store_2d(&mapC, (int)(bx0[hf] + bxs * ch), (int)(by0[hf] + bys * ch), buf_u32 + ch * 4096);
           tma_store_commit();
         }
-        if (p.colw) {
+        if (!SCALED && p.colw) {
           // the boxes still hold out (lane = column): once the store has read them they become the second output
           if (lane == 0) tma_store_wait_read();
           __syncwarp();
@@ -526,8 +540,9 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       for (int ch = 0; ch < 2; ++ch) {
         uint32_t r[32];
         tmem_ld32(tacc + (uint32_t)(ch * 32), r);
-        if (ch < n_box[0]) stage_box(ch, r);         // warp-uniform
+        if (ch < n_box[0]) stage_box(ch, r, ch ? cw1 : cw0);         // warp-uniform
       }
+      if (SCALED) { wdot += (double)wpart; wpart = 0.f; }
       store_half(0);
       // the second half is taken into registers at once, so that the accumulator goes back to the MMA issuer
       // before this warp waits for its first store
@@ -538,13 +553,21 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * h);
       open_half(1);
+      if (SCALED) { cw0 = __ldg(p.colw + col_tile + 64 + lane); cw1 = __ldg(p.colw + col_tile + 96 + lane); }
       if (p.D && n_box[1] > 0) {
         if (!__all_sync(0xffffffffu, mbar_wait(dbar, d_loads & 1u, abortp, p.status))) { ok = false; break; }
         ++d_loads;
       }
-      if (0 < n_box[1]) stage_box(0, r2);
-      if (1 < n_box[1]) stage_box(1, r3);
+      if (0 < n_box[1]) stage_box(0, r2, cw0);
+      if (1 < n_box[1]) stage_box(1, r3, cw1);
       store_half(1);
+      if (SCALED) {
+        wdot += (double)wpart;
+        // lanes in a fixed order
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) wdot += __shfl_xor_sync(0xffffffffu, wdot, o);
+        if (lane == 0) p.dot_part[((size_t)u.b * p.tiles + u.t) * 4 + q] = wdot;
+      }
     }
     if (lane == 0) tma_store_wait_read();           // shared memory stays valid until the stores have read it
   }
@@ -556,8 +579,8 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   }
 }
 
-// X2: the second input (DUAL) or the second output (colw)
-template <bool DUAL>
+// X2: the second input (DUAL) or the second output (right with colw)
+template <bool DUAL, bool SCALED = false>
 armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, int64_t cols, RParams p, float* out,
                     cudaStream_t s, const float* X2 = nullptr) {
   CUtensorMap mX, mX2, mQ, mC, mD;
@@ -569,7 +592,7 @@ armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, 
     mD = mC;
   }
   if (!make_map_2d(&mX, X, cols, rows, cols, 32, p.x.mn_major ? 32 : TILE, p.x.mn_major != 0)) return ARMOR_ERR_CUDA;
-  if (p.colw) {
+  if (p.colw && !SCALED) {
     if (!make_map_2d(&mX2, X2, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
   } else if (X2) {
     if (!make_map_2d(&mX2, X2, cols, rows, cols, 32, p.x.mn_major ? 32 : TILE, p.x.mn_major != 0)) return ARMOR_ERR_CUDA;
@@ -579,11 +602,11 @@ armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, 
   p.c_rows = rows; p.c_cols = cols;
   p.status = c->status;
   static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_blockres_kernel<DUAL>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  if (ensure_dynamic_smem(attr, c->device, tc_blockres_kernel<DUAL, SCALED>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int64_t n_items = (int64_t)p.batch * p.tiles;
   const int grid = (int)(n_items < c->n_sm ? n_items : c->n_sm);
   KTimer kt(c, ARMOR_KC_BLOCK_PRODUCT, ((p.D || X2) ? 12.0 : 8.0) * (double)rows * (double)cols, s);
-  launch_dependent(tc_blockres_kernel<DUAL>, grid, NTHREADS, SMEM_BYTES, s, mX, mX2, mQ, mC, mD, p);
+  launch_dependent(tc_blockres_kernel<DUAL, SCALED>, grid, NTHREADS, SMEM_BYTES, s, mX, mX2, mQ, mC, mD, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
@@ -609,16 +632,19 @@ armor_status tc_blockres_right(armor_ctx* c, const float* in, const float* Bblk,
   return launch<false>(c, in, Bblk, rows, cols, p, out, s, out2);
 }
 
-// out[i-th block, :] = alpha * P_i * in[i-th block, :] (+ beta * add[i-th block, :]),  P_i = Ablk[i] or its transpose
+// out[i-th block, :] = alpha * P_i * in[i-th block, :] (+ beta * add[i-th block, :]),  P_i = Ablk[i] or its transpose; with colw
+// scaled per column by colw, and 4 partial sums per 128 x 128 tile of <unscaled, scaled> at part
 armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
-                              int64_t cols, float alpha, const float* add, float beta, cudaStream_t s) {
+                              int64_t cols, float alpha, const float* add, float beta, cudaStream_t s, const float* colw, double* part) {
+  if ((colw == nullptr) != (part == nullptr) || (colw && cols % TILE)) return ARMOR_ERR_UNSUPPORTED;
   if (!ptr_ok(in) || !ptr_ok(Ablk) || !ptr_ok(out) || (add && !ptr_ok(add))) return ARMOR_ERR_UNSUPPORTED;
   RParams p{};
+  p.colw = colw; p.dot_part = part;
   p.x = {1, 0, TILE, 0, TILE, 0, BK};     // N side [n = column of in][k]: x = 128 t, y = 128 i + 32 kc  (N-major)
   p.col_read = transA ? 1 : 0; p.right = 0;
   p.D = add; p.alpha = alpha; p.beta = add ? beta : 0.f;
   p.batch = (int)(rows / TILE); p.tiles = (int)((cols + TILE - 1) / TILE);
-  return launch<false>(c, in, Ablk, rows, cols, p, out, s);
+  return colw ? launch<false, true>(c, in, Ablk, rows, cols, p, out, s) : launch<false>(c, in, Ablk, rows, cols, p, out, s);
 }
 
 // out[i-th block, :] = P_i * in2[i-th block, :] and 8 partial sums per 128 x 128 tile of <P_i * in1, P_i * in2> at part

@@ -244,3 +244,44 @@ def test_gram_of_few_channels_is_cut_along_the_tokens(d_in, tokens):
     ref = X.double().t() @ X.double()
     assert (H.double() - ref).norm() <= 1.2e-5 * ref.norm() and torch.equal(H, H.t())
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("cols", [3068, 3076])
+def test_left_product_with_an_addend_on_either_side_of_its_line(cols):
+    """An addend moves the line between the kernels to two tiles per SM (288 and 300 tiles here, 148 SMs)."""
+    test_one_sided_products_on_either_side_of_the_choice(1, 1536, cols, 0)
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(128, 128, 128), (384, 640, 128), (1536, 3072, 128), (1536, 3200, 128), (2560, 4096, 128),
+                                                (256, 512, 256), (1024, 1280, 256)])
+def test_weighted_residual_of_the_diagonal_weighting(d_out, d_in, d_block):
+    """E = W - A S B is never stored, its weighted form and the loss leave the product's epilogue: one tile, both kernels on either
+    side of their line (two tiles per SM), blocks of 256.  The tensor cores' accumulator truncates: 3 d_block / 8 additions of up to
+    2^-24 each in S B and again in A (S B), and the loss is quadratic in E, hence 4 (3 d_block / 8) 2^-24 (1.2e-5 for 128) of it.
+    The weighted residual comes back through the gradients of an Adam step: compared with the CUDA-core kernels, whose products are fp32."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + d_in)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    h = torch.rand(d_in, device=DEV, generator=g) * 3 + 0.1
+    H = torch.diag(h)
+    got = {}
+    tol = 1.5 * d_block * 2.0 ** -24
+    for precision in (Bd.PREC_FP16X3, Bd.PREC_SIMT):
+        ctx = _ctx(d_out, d_in, d_block, precision=precision, h_mode=Bd.H_DIAG, ab_step=Bd.AB_ADAM, adam_lr=1e-3, seed=5)
+        st = ctx.init(W, H)
+        gen = _gen(3)
+        st.A.add_(torch.randn(st.A.shape, device=DEV, generator=gen), alpha=0.05)
+        st.B.add_(torch.randn(st.B.shape, device=DEV, generator=gen), alpha=0.05)
+        loss = ctx.proxy_loss(st, H).item()
+        T = torch.einsum("rjk,jkn->rjn", st.S.double().view(d_out, -1, d_block), st.B.double()).reshape(d_out, d_in)
+        E = W.double() - torch.einsum("imk,ikn->imn", st.A.double(), T.view(-1, d_block, d_in)).reshape(d_out, d_in)
+        ref = (E * E * h.double()).sum().item()
+        assert abs(loss - ref) <= tol * ref
+        stats = ctx.read_stats(ctx.bcd_step(st, H, 1, 1))
+        got[precision] = (st.A.clone(), st.B.clone(), stats["loss_start"][0], stats["loss_A"][0])
+        assert ctx.device_status()[:4] == [0, 0, 0, 0]
+    a, b = got[Bd.PREC_FP16X3], got[Bd.PREC_SIMT]
+    for k in (0, 1):
+        assert (a[k] - b[k]).double().norm() <= 1e-4 * b[k].double().norm()
+    for k in (2, 3):
+        assert abs(a[k] - b[k]) <= 2 * tol * b[k]
