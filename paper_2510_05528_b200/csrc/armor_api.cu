@@ -143,6 +143,7 @@ size_t carve(const armor_config& cfg, armor_ctx* c, char* base) {
   TAKE(tab_g, unsigned long long*, (size_t)nbo * nbi * sizeof(unsigned long long));
   TAKE(status, int32_t*, ST_COUNT * sizeof(int32_t));
   TAKE(screen, int32_t*, 4 * sizeof(int32_t));
+  TAKE(core_flags, int32_t*, 2 * sizeof(int32_t));
   TAKE(it_dev, int64_t*, sizeof(int64_t));
 #undef TAKE
   if (c) {
@@ -750,7 +751,11 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
   int64_t chunk = d_out < d_in ? d_out : d_in;   // z1 [chunk, d_in] and z2 [chunk, d_out] fit W-shaped scratch
   if (wide) chunk = 4 * chunk < c->gram_rows ? 4 * chunk : c->gram_rows;
   float* const z2 = wide ? c->V : c->E;
-  if (wide) core_f16_split_S(c, S, s);
+  const bool sparse24 = wide && core_f16_sparse(c, n_tokens);
+  if (wide) {
+    const armor_status st = core_f16_split_S(c, S, sparse24, s);
+    if (st != ARMOR_OK) return st;
+  }
   for (int64_t t0 = 0; t0 < n_tokens; t0 += chunk) {
     const int64_t n = (n_tokens - t0 < chunk) ? n_tokens - t0 : chunk;
     const float* xc;
@@ -774,7 +779,7 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
     c->block_one_pass = bf16 ? 1 : 0;
     bd_right(c, xc, B, true, c->T, n, d_in, 1.f, nullptr, 0.f, s);                   // z1 = x B^T
     c->block_one_pass = 0;
-    armor_status st = wide ? core_f16_product(c, c->T, z2, n, s) : apply_core(c, c->T, S, packed, z2, n, bf16, s);   // z2 = z1 S^T
+    armor_status st = wide ? core_f16_product(c, c->T, S, sparse24, z2, n, s) : apply_core(c, c->T, S, packed, z2, n, bf16, s);   // z2 = z1 S^T
     if (st != ARMOR_OK) return st;
     c->block_one_pass = bf16 ? 1 : 0;
     bd_right(c, z2, A, true, yc, n, d_out, 1.f, nullptr, 0.f, s);                    // y = z2 A^T

@@ -109,6 +109,7 @@ struct armor_ctx {
   unsigned long long* tab_g;   // its global group index
   int32_t* status;    // [ST_COUNT]
   int32_t* screen;    // [4] per-call counters of the input screening
+  int32_t* core_flags;   // fp32 forward: [0] the core is not 2:4, [1] activations are not finite
   int64_t* it_dev;    // iteration index inside the running armor_bcd_step call (advanced by the first kernel of an iteration)
   int use_graphs;     // 1: repeated iterations of a call are replayed from a CUDA graph
   cudaStream_t cap_stream;   // the context's own stream, used only to capture that graph
@@ -346,14 +347,18 @@ armor_status apply_core(armor_ctx* c, const float* z1, const float* S, const voi
                         bool bf16, cudaStream_t s);
 
 // the same in the three-pass fp16 mode with S split beforehand (once per call), up to gram_rows tokens at a time
+// (sparse: on the sparse tensor cores, whatever S holds; core_f16_sparse says where that is faster, for calls of so many tokens)
 bool core_f16_ok(const armor_ctx* c);
-void core_f16_split_S(armor_ctx* c, const float* S, cudaStream_t s);
-armor_status core_f16_product(armor_ctx* c, const float* z1, float* z2, int64_t n, cudaStream_t s);
+bool core_f16_sparse(const armor_ctx* c, int64_t n_tokens);
+armor_status core_f16_split_S(armor_ctx* c, const float* S, bool sparse, cudaStream_t s);
+armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, bool sparse, float* z2, int64_t n, cudaStream_t s);
 
 // operand preparation of the three-pass fp16 mode (split_f16.cu)
 void launch_f16_prepare_H(armor_ctx* c, const float* H, cudaStream_t s);   // hpow, scaled H as fp16 hi | lo in Hlo
 void launch_f16_split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t rows, int64_t cols, const float* colscale,
-                           float post, void* hi, void* lo, float* out_scale, cudaStream_t s);
+                           float post, void* hi, void* lo, float* out_scale, cudaStream_t s, int32_t* not_finite = nullptr);
+// the 2:4 core [d_out, d_in] as fp16 parts of its kept entries with their positions, see split_core24_kernel
+void launch_split_core24(armor_ctx* c, const float* S, int layer, void* hi, void* lo, void* E, float* scale, int32_t* flags, cudaStream_t s);
 float f16_H_post_scale();
 armor_status launch_f16_gram_stage(armor_ctx* c, const void* X, int x_dtype, int64_t ldx, int64_t rows, int64_t cols,
                                    void* Thi, void* Tlo, float* gscale, cudaStream_t s);
@@ -466,6 +471,9 @@ size_t tc_sparse_values_bytes(const armor_ctx* c);
 void launch_compress_24(armor_ctx* c, const float* S, const uint8_t* M, void* Sc, void* E, cudaStream_t s);
 armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const void* z1_bf16, void* z2, bool out_bf16,
                               int64_t n, cudaStream_t s);
+bool tc_sparse3_ok(const armor_ctx* c);
+armor_status launch_tc_sparse3(armor_ctx* c, const void* hi, const void* lo, const void* E, const float* row_scale, const void* zhi,
+                               const void* zlo, const float* tok_scale, const int32_t* flags, float* z2, int64_t n, cudaStream_t s);
 // the wrapper products of the bf16 forward (fwd_tcgen05.cu)
 bool fwd_block_ok(const armor_ctx* c);
 void launch_pack_blocks(armor_ctx* c, const float* P, const float* rowscale, const float* colscale, void* Q, int nb,

@@ -229,16 +229,33 @@ armor_status gram_accumulate(armor_ctx* c, const void* Xv, int x_dtype, int64_t 
 bool core_f16_ok(const armor_ctx* c) {
   return c->cfg.precision == ARMOR_PREC_FP16X3 && c->d_out % 32 == 0 && c->d_in % 8 == 0;
 }
-void core_f16_split_S(armor_ctx* c, const float* S, cudaStream_t s) {
-  __half* shi = reinterpret_cast<__half*>(c->U);
-  launch_f16_split_rows(c, S, c->d_in, c->d_out, c->d_in, nullptr, 1.f, shi, shi + c->wn, c->rowscale2, s);
+// On the sparse tensor cores (sparse_tcgen05.cu) once tiles of 64 tokens fill the pairs of CTAs; for fewer the dense product cuts the
+// contraction.  Whole forward, sparse / dense: 4096 x 4096, 200 tokens 90 / 84 us, 400 97 / 103, 1,600 152 / 198; 2048 x 8192, 400 tokens 122 / 105, 800
+// 136 / 146; 14336 x 4096, 100 tokens 160 / 168; 512 x 4096, 1,600 tokens 82 / 78.
+bool core_f16_sparse(const armor_ctx* c, int64_t n_tokens) {
+  return tc_sparse3_ok(c) && n_tokens * (c->d_out / 256) >= (int64_t)c->n_sm / 2 * 64;
 }
-armor_status core_f16_product(armor_ctx* c, const float* z1, float* z2, int64_t n, cudaStream_t s) {
+// sparse: S's parts in U (hi of both layers, then lo), positions in Lo
+armor_status core_f16_split_S(armor_ctx* c, const float* S, bool sparse, cudaStream_t s) {
+  __half* shi = reinterpret_cast<__half*>(c->U);
+  if (sparse) {
+    if (cudaMemsetAsync(c->core_flags, 0, 2 * sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
+    launch_split_core24(c, S, 0, shi, shi + c->wn, c->Lo, c->rowscale2, c->core_flags, s);
+  } else {
+    launch_f16_split_rows(c, S, c->d_in, c->d_out, c->d_in, nullptr, 1.f, shi, shi + c->wn, c->rowscale2, s);
+  }
+  return ARMOR_OK;
+}
+armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, bool sparse, float* z2, int64_t n, cudaStream_t s) {
   const int64_t d_in = c->d_in, d_out = c->d_out;
   __half* ahi = reinterpret_cast<__half*>(c->Xt_hi);
   __half* shi = reinterpret_cast<__half*>(c->U);
   float* scales = reinterpret_cast<float*>(c->colpart);         // 64 d_in doubles
-  launch_f16_split_rows(c, z1, d_in, n, d_in, nullptr, 1.f, ahi, ahi + n * d_in, scales, s);
+  launch_f16_split_rows(c, z1, d_in, n, d_in, nullptr, 1.f, ahi, ahi + n * d_in, scales, s, sparse ? c->core_flags + 1 : nullptr);
+  if (sparse) {
+    launch_split_core24(c, S, 1, shi, shi + c->wn, c->Lo, c->rowscale2, c->core_flags, s);
+    return launch_tc_sparse3(c, shi, shi + c->wn, c->Lo, c->rowscale2, ahi, ahi + n * d_in, scales, c->core_flags, z2, n, s);
+  }
   TcGemm g{};
   g.lda = d_in; g.ldb = d_in; g.ldc = d_out;
   g.M = n; g.N = d_out; g.K = d_in;

@@ -563,6 +563,201 @@ tc_sparse_small_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
   }
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// The fp32-grade product with the 2:4 core (the core product of the fp32 forward): both operands as fp16 high and low parts
+// of rows scaled by powers of two (split_f16.cu), three sparse MMAs lo*hi + hi*lo + hi*hi per 32 of k where the dense product issues
+// six.  Same pairs of CTAs as above; differences:
+//   * 128 k of a stage are 32 KiB of kept values, up to 56 KiB of z1 and 2 KiB of positions, so there are two stages;
+//   * tiles of 256 rows of S by tile_n <= 224 tokens, so that two accumulators and the positions fit tensor memory: the sums of
+//     a segment of the contraction leave for the epilogue warps' registers while the next segment runs.  The host picks the tile_n that
+//     fills the last wave best;
+//   * a core that is not 2:4, or activations that are not finite (0 * inf), take the other two positions of every
+//     group as a second layer of the contraction: flags says so, any S is the sum of two such layers.
+// Segments of 1,024 columns as in the dense product, which are half as many truncating additions here (whole forward 4.0e-6 off fp64
+// sums where the dense core was 5.8e-6; segments of 2,048 6.1e-6, at the same speed).
+// What bounds it: the sparse tensor cores under the power cap, and at the burst clock what L2 delivers (90 KiB per SM and stage).
+// 4096 x 4096, 8,195 tokens: 325 us where the dense product takes 525 (846 TFLOP/s of fp32-grade products, dense-equivalent).
+constexpr int S3_MAX_N = 224, S3_STAGES = 2, S3_THREADS = 320, S3_SEG = 8;      // segment: stages of 128 columns
+constexpr uint32_t S3_META = 2 * S3_MAX_N;
+constexpr int S3_B = 2 * A_BYTES, S3_E = S3_B + 4 * BH_BYTES, S3_STAGE = S3_E + E_BYTES;
+
+struct S3Params {
+  float* Z; int64_t ldz;                            // [tokens][d_out]
+  int64_t N;                                        // tokens
+  int m_rows, m_pairs, n_tiles, k_tiles, tile_n;    // rows of S, tiles of 256 of them, tiles of tile_n tokens, k tiles of 128
+  const float* row_scale;                           // per row of S, per token
+  const float* tok_scale;
+  const int32_t* flags;                             // either of two: both layers
+  int32_t* status;
+};
+
+__global__ void __launch_bounds__(S3_THREADS, 1)
+tc_sparse3_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapAlo,
+                       const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapBlo,
+                       const __grid_constant__ CUtensorMap mapE, const S3Params p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t bars[2 * S3_STAGES + 4];
+  __shared__ uint32_t tmem_base_holder;
+  __shared__ int abort_flag;
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[S3_STAGES]);
+  const uint32_t tfull0 = smem_u32(&bars[2 * S3_STAGES]), tempty0 = smem_u32(&bars[2 * S3_STAGES + 2]);
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int n_tiles_total = p.m_pairs * p.n_tiles;
+  const int k_total = (p.flags[0] | p.flags[1]) ? 2 * p.k_tiles : p.k_tiles;
+  const int half_n = p.tile_n / 2;
+
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int s = 0; s < S3_STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
+    for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 16); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
+                 "r"(TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                                       // both CTAs' barriers exist before anyone signals them
+  tc_fence_after();
+  const uint32_t tmem_base = tmem_base_holder;
+  volatile int* abortp = &abort_flag;
+
+  if (warp == 0) {
+    // ------------------------------------------------------------ TMA producer (both CTAs)
+    if (lane == 0) {
+      int stage = 0; uint32_t phase = 0; long long issued = 0;
+      bool ok = true;
+      const int stage_bytes = 2 * A_BYTES + 4 * half_n * 128 + E_BYTES;
+      for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
+        int mt, nt;
+        tile_to_mn(tile, p.m_pairs, p.n_tiles, mt, nt);
+        const int row0 = mt * 256 + (int)rank * 128, tok0 = nt * p.tile_n + (int)rank * half_n;
+        for (int f = 0; f < k_total; ++f) {
+          if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
+          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * stage_bytes);
+          const int layer = f >= p.k_tiles ? 1 : 0, kt = f - layer * p.k_tiles;
+          const uint32_t fb = map_to_cta(full0 + 8 * stage, 0);
+          const uint32_t dst = smem_u32(smem + (size_t)stage * S3_STAGE);
+          tma_load_2d_pair(dst, &mapA, kt * 64, layer * p.m_rows + row0, fb);
+          tma_load_2d_pair(dst + A_BYTES, &mapAlo, kt * 64, layer * p.m_rows + row0, fb);
+          tma_load_2d_pair(dst + S3_B, &mapB, kt * BKL, tok0, fb);
+          tma_load_2d_pair(dst + S3_B + BH_BYTES, &mapB, kt * BKL + 64, tok0, fb);
+          tma_load_2d_pair(dst + S3_B + 2 * BH_BYTES, &mapBlo, kt * BKL, tok0, fb);
+          tma_load_2d_pair(dst + S3_B + 3 * BH_BYTES, &mapBlo, kt * BKL + 64, tok0, fb);
+          tma_load_2d_pair(dst + S3_E, &mapE, 0, ((layer * 2 * p.m_pairs + 2 * mt + (int)rank) * p.k_tiles + kt) * 128, fb);
+          ++issued;
+          if (++stage == S3_STAGES) { stage = 0; phase ^= 1; }
+        }
+      }
+      // tail: the MMAs that read the stages issued last have finished (their commits reach both CTAs), so
+      // nothing is in flight towards this CTA's shared memory when it leaves
+      for (int back = 1; back <= S3_STAGES && back <= issued; ++back) {
+        int s = stage - back; uint32_t ph = phase;
+        if (s < 0) { s += S3_STAGES; ph ^= 1; }
+        const long long t0 = clock64();
+        while (!mbar_try(empty0 + 8 * s, ph) && clock64() - t0 < (ok ? WAIT_CYCLES : 20000000ll)) {}
+      }
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issuer (even CTA only)
+    if (lane == 0 && rank == 0) {
+      // fp16 operands, fp32 sums, M = 256, N = tile_n, sparse A
+      const uint32_t idesc = (1u << 2) | (1u << 4) | ((uint32_t)(p.tile_n >> 3) << 17) | (uint32_t)(256 >> 4) << 24;
+      const uint64_t d0 = smem_desc_k(smem_u32(smem)), e0 = smem_desc_e(smem_u32(smem) + S3_E);
+      int stage = 0; uint32_t phase = 0;
+      int local = 0;                                        // (tile, segment) items so far: selects the accumulator
+      bool ok = true;
+      for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
+        for (int f0 = 0; f0 < k_total && ok; f0 += S3_SEG, ++local) {
+          const int as = local & 1;
+          if (!mbar_wait_cluster(tempty0 + 8 * as, ((uint32_t)(local >> 1) & 1u) ^ 1u, abortp, p.status)) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t tacc = tmem_base + (uint32_t)(as * S3_MAX_N);
+          const int f1 = min(k_total, f0 + S3_SEG);
+          for (int f = f0; f < f1; ++f) {
+            if (!mbar_wait_cluster(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
+            tc_fence_after();
+            const uint64_t so = (uint64_t)(uint32_t)(stage * (S3_STAGE >> 4));
+            const uint32_t meta = tmem_base + S3_META + (uint32_t)(4 * stage);
+            tmem_cp_e_pair(meta, e0 + so);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint64_t da = d0 + so + j * (32 >> 4), dal = da + (A_BYTES >> 4);
+              const uint64_t dbm = d0 + so + ((S3_B + (j >> 1) * BH_BYTES + (j & 1) * 64) >> 4), dbl = dbm + ((2 * BH_BYTES) >> 4);
+              const uint32_t id = idesc | (uint32_t)(j & 1), ecol = meta + (uint32_t)(j & ~1);
+              umma_bf16_sp_pair(tacc, dal, dbm, ecol, id, (uint32_t)((f > f0) | (j != 0)));
+              umma_bf16_sp_pair(tacc, da, dbl, ecol, id, 1u);
+              umma_bf16_sp_pair(tacc, da, dbm, ecol, id, 1u);
+            }
+            umma_commit_pair(empty0 + 8 * stage);
+            if (++stage == S3_STAGES) { stage = 0; phase ^= 1; }
+          }
+          if (ok) umma_commit_pair(tfull0 + 8 * as);
+        }
+      }
+    }
+  } else {
+    // ------------------------------------------------------------ epilogue warps (both CTAs)
+    // warp w: rows 32 (w % 4) .. of S, one of the two halves of the tile's tokens, one running sum per token and lane
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    int local = 0;
+    bool ok = true;
+    for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
+      int mt, nt;
+      tile_to_mn(tile, p.m_pairs, p.n_tiles, mt, nt);
+      float acc[128];
+#pragma unroll
+      for (int i = 0; i < 128; ++i) acc[i] = 0.f;
+      for (int f0 = 0; f0 < k_total && ok; f0 += S3_SEG, ++local) {
+        const int as = local & 1;
+        if (!mbar_wait(tfull0 + 8 * as, (uint32_t)(local >> 1) & 1u, abortp, p.status)) { ok = false; break; }
+        tc_fence_after();
+#pragma unroll
+        for (int ch = 0; ch < 4; ++ch) {
+          if (ch * 32 >= half_n) continue;                  // uniform; columns past the half are not stored
+          uint32_t r[32];
+          tmem_ld32(tmem_base + (uint32_t)(as * S3_MAX_N + half * half_n + ch * 32) + ((uint32_t)(q * 32) << 16), r);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) acc[ch * 32 + i] += __uint_as_float(r[i]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_to_cta(tempty0 + 8 * as, 0));
+      }
+      if (!ok) break;
+      const int64_t row = (int64_t)mt * 256 + rank * 128 + q * 32 + lane;
+      const int64_t tok0 = (int64_t)nt * p.tile_n + half * half_n;
+      const int left = (int)(p.N - tok0 < half_n ? p.N - tok0 : half_n);
+      const float rs = p.row_scale[row];
+      float* out = p.Z + tok0 * p.ldz + row;
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch) {
+        if (ch * 32 >= left) continue;
+        const float ts = ch * 32 + lane < left ? p.tok_scale[tok0 + ch * 32 + lane] : 0.f;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const float t = __shfl_sync(0xffffffffu, ts, i);
+          if (ch * 32 + i < left) out[(int64_t)(ch * 32 + i) * p.ldz] = acc[ch * 32 + i] * t * rs;
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();                                       // neither CTA leaves while its partner may still signal it
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+  }
+}
+
 // One thread per 32-bit word of positions: 2 rows x 16 k.  Writes the word and the eight pairs of kept values.
 // A group whose mask byte keeps fewer than two positions is padded with unkept positions (their values are
 // written as zeros); more than two kept positions cannot be represented: the first two are taken and the
@@ -612,17 +807,20 @@ compress_24_kernel(const float* __restrict__ S, const uint8_t* __restrict__ Mk, 
   if (bad) atomicAdd(&status[ST_SPARSE_BAD_GROUPS], 1);
 }
 
-bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows = 128) {
+bool make_map_16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows, CUtensorMapDataType type) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
   cuuint32_t box[2] = {64, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
-  CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+  CUresult r = enc(map, type, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int64_t ld, int box_rows = 128) {
+  return make_map_16(map, base, rows, K, ld, box_rows, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16);
 }
 
 bool make_map_e(CUtensorMap* map, const void* base, int64_t rows);
@@ -742,4 +940,48 @@ armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E,
   if (n <= 32) return launch_small<32>(c, Sc, E, z1_bf16, p, *pieces, per, s);
   if (n <= 64) return launch_small<64>(c, Sc, E, z1_bf16, p, *pieces, per, s);
   return launch_small<128>(c, Sc, E, z1_bf16, p, *pieces, per, s);
+}
+
+// Z2[n][d_out] = Z1[n][d_in] * S^T, fp32-grade: the parts of S's two layers (hi: layer 0, layer 1, lo likewise, [d_out][d_in / 2] each)
+// with their positions, z1's parts, the rows' scales and the flags that ask for the second layer.
+bool tc_sparse3_ok(const armor_ctx* c) {
+  return tc_sparse_ok(c) && c->cfg.precision == ARMOR_PREC_FP16X3 && c->d_out % 256 == 0 && c->n_sm >= 2;
+}
+armor_status launch_tc_sparse3(armor_ctx* c, const void* hi, const void* lo, const void* E, const float* row_scale, const void* zhi,
+                               const void* zlo, const float* tok_scale, const int32_t* flags, float* z2, int64_t n, cudaStream_t s) {
+  if (!tc_sparse3_ok(c) || n <= 0) return ARMOR_ERR_UNSUPPORTED;
+  const int pairs = c->n_sm / 2;
+  S3Params p{};
+  p.Z = z2; p.ldz = c->d_out; p.N = n;
+  p.m_rows = (int)c->d_out; p.m_pairs = (int)(c->d_out / 256); p.k_tiles = (int)(c->d_in / BKL);
+  p.row_scale = row_scale; p.tok_scale = tok_scale; p.flags = flags; p.status = c->status;
+  // the width of a tile that costs least: waves of tiles times what a tile takes, its MMAs (proportional to the width) plus what
+  // comes with every tile whatever its width (S's share of the loads, the first stage, the last segment's way out: about 48 tokens' worth)
+  int64_t least = 0;
+  for (int w = S3_MAX_N; w >= 64; w -= 32) {
+    const int64_t tiles = p.m_pairs * ((n + w - 1) / w), cost = (tiles + pairs - 1) / pairs * (w + 48);
+    if (w == S3_MAX_N || cost < least) { least = cost; p.tile_n = w; }
+  }
+  p.n_tiles = (int)((n + p.tile_n - 1) / p.tile_n);
+  CUtensorMap mA, mAlo, mB, mBlo, mE;
+  const CUtensorMapDataType f16 = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+  if (!make_map_16(&mA, hi, 2 * c->d_out, c->d_in / 2, c->d_in / 2, 128, f16)) return ARMOR_ERR_CUDA;
+  if (!make_map_16(&mAlo, lo, 2 * c->d_out, c->d_in / 2, c->d_in / 2, 128, f16)) return ARMOR_ERR_CUDA;
+  if (!make_map_16(&mB, zhi, n, c->d_in, c->d_in, p.tile_n / 2, f16)) return ARMOR_ERR_CUDA;
+  if (!make_map_16(&mBlo, zlo, n, c->d_in, c->d_in, p.tile_n / 2, f16)) return ARMOR_ERR_CUDA;
+  if (!make_map_e(&mE, E, 2 * (c->d_out / 128) * (c->d_in / 128) * 128)) return ARMOR_ERR_CUDA;
+  constexpr size_t SMEM = (size_t)S3_STAGES * S3_STAGE + 1024;
+  static PerDeviceOnce attr;
+  if (ensure_dynamic_smem(attr, c->device, tc_sparse3_pair_kernel, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  const int tiles = p.m_pairs * p.n_tiles;
+  KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)c->d_out * (double)n * (double)c->d_in, s);   // dense-equivalent flops
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(2 * (tiles < pairs ? tiles : pairs)); cfg.blockDim = dim3(S3_THREADS); cfg.dynamicSmemBytes = SMEM; cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, tc_sparse3_pair_kernel, mA, mAlo, mB, mBlo, mE, p) != cudaSuccess) return ARMOR_ERR_CUDA;
+  c->launches++;
+  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }

@@ -561,3 +561,40 @@ def test_left_solves_of_256_in_several_slices_a_cta(nb_in):
     X = torch.linalg.solve(C, S.transpose(1, 2) @ (E * D)) / (D + 1e-6 * D.mean(2, keepdim=True))
     assert (st.B.double() - eye - X).norm() <= 1e-4 * X.norm()
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block,tokens", [(256, 128, 128, 4800), (256, 256, 256, 4737), (512, 384, 128, 2369), (1280, 1152, 128, 1000),
+                                                      (4096, 2048, 128, 297), (2304, 9216, 128, 640), (512, 512, 128, 16384 + 70),
+                                                      (128, 256, 128, 5000), (4096, 2048, 128, 295)])
+@pytest.mark.parametrize("core", ["2of4", "any"])
+def test_fp32_forward_on_the_sparse_tensor_cores(d_out, d_in, d_block, tokens, core):
+    """The core product of many tokens runs on the sparse tensor cores whatever the core holds: rows of one K tile to several
+    segments, ragged tiles of tokens, a second chunk, and the dense product where rows do not come in 256 or tokens are few.  "any": groups
+    with every pattern of entries, two layers.  Truncating additions, 48 in either wrapper product and 96 in a segment of the core's, of up to
+    2^-24: 1.2e-5 of the result.  One token that is not finite spoils its own row and no other."""
+    g = _gen(d_out + d_in + tokens)
+    ctx = _ctx(d_out, d_in, d_block)
+    from paper_2510_05528_b200 import binding as Bd
+    A = torch.eye(d_block, device=DEV) + 0.3 / d_block ** 0.5 * torch.randn(d_out // d_block, d_block, d_block, device=DEV, generator=g)
+    B = torch.eye(d_block, device=DEV) + 0.3 / d_block ** 0.5 * torch.randn(d_in // d_block, d_block, d_block, device=DEV, generator=g)
+    W = torch.randn(d_out, d_in // 4, 4, device=DEV, generator=g)
+    if core == "2of4":
+        keep = torch.zeros_like(W, dtype=torch.bool).scatter_(2, W.abs().topk(2, dim=2).indices, True)
+    else:
+        bits = torch.randint(0, 16, (d_out, d_in // 4, 1), device=DEV, generator=g)
+        keep = ((bits >> torch.arange(4, device=DEV)) & 1).bool()
+    S = (W * keep).view(d_out, d_in)
+    st = Bd.LayerState(Wbar=S, A=A, B=B, S=S, M=torch.zeros(d_out, d_in // 4, dtype=torch.uint8, device=DEV))
+    x = torch.randn(tokens, d_in, device=DEV, generator=g) * torch.exp(torch.randn(d_in, device=DEV, generator=g))
+    y = ctx.apply(st, x)
+    z = torch.einsum("njk,jmk->njm", x.double().view(tokens, -1, d_block), B.double()).reshape(tokens, d_in) @ S.double().t()
+    ref = torch.einsum("njk,jmk->njm", z.view(tokens, -1, d_block), A.double()).reshape(tokens, d_out)
+    assert (y.double() - ref).norm() <= 1.2e-5 * ref.norm()
+    x[tokens - 2, 5] = float("inf")
+    yi = ctx.apply(st, x)
+    assert not torch.isfinite(yi[tokens - 2]).any()
+    others = torch.arange(tokens, device=DEV) != tokens - 2
+    assert (yi[others] - y[others]).norm() <= 1e-6 * y.norm()
+    x[tokens - 2, 5] = 0.0
+    assert torch.isfinite(ctx.apply(st, x)).all()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
