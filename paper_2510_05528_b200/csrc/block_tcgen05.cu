@@ -344,7 +344,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
         if (row_base < p.c_rows && tm * TILE + q * 32 < p.m_valid)
           for (int ch = 0; ch < 2; ++ch) n_box += (col_tile + 64 * hf + 32 * ch < p.c_cols) ? 1 : 0;
         float cw0 = 0.f, cw1 = 0.f;                 // colw: lane l holds the scale of column l of each box (handed round by shuffles)
-        if (COLW) { cw0 = __ldg(p.colw + col_tile + 64 * hf + lane); cw1 = __ldg(p.colw + col_tile + 64 * hf + 32 + lane); }
+        if (COLW) { cw0 = p.colw[col_tile + 64 * hf + lane]; cw1 = p.colw[col_tile + 64 * hf + 32 + lane]; }
         if (lane == 0) {
           tma_store_wait_read();                    // the previous stores have read the staging boxes
           if (p.D && n_box > 0) {

@@ -445,7 +445,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       // left with colw: a half's column scales, lane l holding column l of each box; they travel while the MMAs run or the
       // addend is waited for, and go round by shuffles
       float cw0 = 0.f, cw1 = 0.f;
-      if (SCALED) { cw0 = __ldg(p.colw + col_tile + lane); cw1 = __ldg(p.colw + col_tile + 32 + lane); }
+      if (SCALED) { cw0 = p.colw[col_tile + lane]; cw1 = p.colw[col_tile + 32 + lane]; }
       double wdot = 0.0;
       float wpart = 0.f;
       // alpha * accumulator (+ beta * addend, which sits in the box already) into staging box ch
@@ -553,7 +553,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8 * h);
       open_half(1);
-      if (SCALED) { cw0 = __ldg(p.colw + col_tile + 64 + lane); cw1 = __ldg(p.colw + col_tile + 96 + lane); }
+      if (SCALED) { cw0 = p.colw[col_tile + 64 + lane]; cw1 = p.colw[col_tile + 96 + lane]; }
       if (p.D && n_box[1] > 0) {
         if (!__all_sync(0xffffffffu, mbar_wait(dbar, d_loads & 1u, abortp, p.status))) { ok = false; break; }
         ++d_loads;
