@@ -137,7 +137,8 @@ size_t carve(const armor_config& cfg, armor_ctx* c, char* base) {
   const int64_t nbmax = nbo > nbi ? nbo : nbi;
   TAKE(partblk, double*, (size_t)(4 * nbmax > nbo * nbi * kg ? 4 * nbmax : nbo * nbi * kg) * sizeof(double));
   TAKE(quadpart, double*, (size_t)nbo * nbi * kg * sizeof(double));
-  TAKE(failflag, int32_t*, (size_t)nbmax * sizeof(int32_t));
+  TAKE(partA, double*, (size_t)4 * nbo * sizeof(double));
+  TAKE(failflag, int32_t*, (size_t)2 * nbmax * sizeof(int32_t));
   TAKE(sel, SelRec*, (size_t)nbo * nbi * kg * sizeof(SelRec));
   TAKE(tab_key, float*, (size_t)nbo * nbi * sizeof(float));
   TAKE(tab_g, unsigned long long*, (size_t)nbo * nbi * sizeof(unsigned long long));
@@ -236,7 +237,8 @@ armor_status core_gradient(armor_ctx* c, const float* A, const float* B, cudaStr
 }
 
 armor_status residual_and_loss(armor_ctx* c, const float* W, const float* H, const float* A, const float* B,
-                               const float* S, double* out, cudaStream_t s, bool exact_products = false) {
+                               const float* S, double* out, cudaStream_t s, bool exact_products = false, int* n_left = nullptr) {
+  // n_left: the loss may be left as that many partial sums in c->partials (0: it is in *out)
   // exact_products: the two wrapper products on the fp32 CUDA-core kernel, whose products with 0 and 1 are
   // exact, so that E vanishes exactly where W = A S B term by term (identity wrappers at the initialisation);
   // the three-pass tensor-core product carries 22 bits of each operand
@@ -248,7 +250,8 @@ armor_status residual_and_loss(armor_ctx* c, const float* W, const float* H, con
     int nq = 0;
     if (tc_done(c, tc_bd_left_residual(c, A, c->T, W, c->hdiag, c->EH, c->d_out, c->d_in, c->partials, &nq, s))) {
       c->tc_blocks = saved;
-      reduce_partials_to(c, c->partials, nq, out, s);
+      if (n_left) *n_left = nq;
+      else reduce_partials_to(c, c->partials, nq, out, s);
       return ARMOR_OK;
     }
   }
@@ -470,6 +473,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
   const bool adam = (c->cfg.ab_step == ARMOR_AB_ADAM);
   const int sweeps = c->cfg.mask_sweeps > 0 ? c->cfg.mask_sweeps : 1;
   const bool carry_P = (c->cfg.h_mode == ARMOR_H_FULL) && !adam;
+  const bool late_A = !adam && c->cfg.ab_step == ARMOR_AB_EXACT && (ph & ARMOR_PHASE_A) && (ph & ARMOR_PHASE_B);   // their bookkeeping together
+  const int n_part_A = nbo * chol_parts_per_block(db, nbo);
   const bool late_P = carry_P && (ph & ARMOR_PHASE_B) && (ph & ARMOR_PHASE_S);   // P's moves of the B-step and the S-step together
   if (!adam && c->cfg.ab_step == ARMOR_AB_EXACT && (ph & ARMOR_PHASE_B) && n_iters > 0) {
     st = launch_hjj_inverse(c, s);
@@ -492,9 +497,10 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       // Adam normalises every entry's move, so a gradient that is exactly zero (the kept entries of the core at
       // the initialisation, where E vanishes on them) must come out as zero: E H_w is formed from E itself, not
       // as the difference W H_w - A P, and at t = 0 (identity wrappers) with the exact fp32 products
-      st = residual_and_loss(c, W, H, A, B, S, c->sc + SC_L0, s, t_zero);
+      int n_loss = 0;                                                                // partial sums of the loss, if the stage adds them up
+      st = residual_and_loss(c, W, H, A, B, S, c->sc + SC_L0, s, t_zero, &n_loss);
       if (st != ARMOR_OK) return st;
-      launch_stage(c, is, 0, nullptr, 0, 0, s);
+      launch_stage(c, is, 0, nullptr, 0, s, n_loss ? c->partials : nullptr, n_loss, SC_L0);
     } else {
     if (first || !carry_P) {
       st = bd_right_H(c, S, B, H, c->T, c->P, s);                                    // T = S B, P = T H_w
@@ -506,7 +512,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
     if (fresh_loss) {
       bd_left(c, A, false, c->T, c->E, d_out, d_in, -1.f, W, 1.f, s);                // E = W - A T
       dot_partials(c, c->EH, c->E, c->wn, c->partials, s);                           // L = <E H_w, E>
-      launch_stage(c, is, 0, nullptr, 0, 0, s, c->partials, ARMOR_DOT_BLOCKS, SC_L0);
+      launch_stage(c, is, 0, nullptr, 0, s, c->partials, ARMOR_DOT_BLOCKS, SC_L0);
     }
     }
 
@@ -521,9 +527,10 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       launch_adam(c, B, c->GamB, c->mB, c->vB, nbl, nullptr, t_first + 1, s);
       launch_adam(c, S, c->Gam, c->mS, c->vS, c->wn, M, t_first + 1, s);
       // the new state: residual, E H_w and the loss afresh
-      st = residual_and_loss(c, W, H, A, B, S, c->sc + SC_L0, s);
+      int n_loss = 0;
+      st = residual_and_loss(c, W, H, A, B, S, c->sc + SC_L0, s, false, &n_loss);
       if (st != ARMOR_OK) return st;
-      launch_stage(c, is, 9, nullptr, 0, 0, s);
+      launch_stage(c, is, 9, nullptr, 0, s, n_loss ? c->partials : nullptr, n_loss, SC_L0);
     }
 
     // ---- A-step: A_i += Gamma_i (G_i + lam I)^-1 -------------------------------------------
@@ -538,18 +545,18 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
         dot_to_ptr(c, c->GamA, c->GamA, na, c->sc + SC_TMP0, s);                     // |Gamma|^2
         block_mm(c, c->GamA, false, c->G, false, c->dA, nbo, s);                     // Gamma_i G_i
         dot_to_ptr(c, c->dA, c->GamA, na, c->sc + SC_TMP1, s);                       // sum_i <Gamma_i G_i, Gamma_i>
-        launch_stage(c, is, 7, nullptr, 0, 0, s);
+        launch_stage(c, is, 7, nullptr, 0, s);
         if (cudaMemsetAsync(c->dA, 0, (size_t)na * sizeof(float), s) != cudaSuccess) return ARMOR_ERR_CUDA;
         launch_axpy_slot(c, c->dA, c->GamA, na, SC_TAU_A, 1.f, s);                   // dA = tau Gamma
         launch_axpy_slot(c, A, c->GamA, na, SC_TAU_A, 1.f, s);                       // A += tau Gamma
       } else {
-        st = launch_chol(c, 0, c->G, c->GamA, c->dA, nullptr, A, nbo, c->partblk, s);
+        st = launch_chol(c, 0, c->G, c->GamA, c->dA, nullptr, A, nbo, c->partA, s);
         if (st != ARMOR_OK) return st;
-        launch_stage(c, is, 1, c->partblk, nbo * chol_parts_per_block(db, nbo), nbo, s);
+        if (!late_A) launch_stage(c, is, 1, c->partA, n_part_A, s);
       }
       bd_left(c, c->dA, false, c->P, c->EH, d_out, d_in, -1.f, c->EH, 1.f, s);       // EH -= dA P
     } else if (!adam) {
-      launch_stage(c, is, 1, nullptr, 0, 0, s);
+      launch_stage(c, is, 1, nullptr, 0, s);
     }
 
     // ---- B-step: block-Newton directions, one exact step --------------------------------------
@@ -581,14 +588,16 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       // V H_w = A (R H_w) and q = <V H_w, V> with V = A R (summed by the stage; V itself is needed nowhere else)
       int nq = 0;
       bd_left_dual(c, A, c->Tmp, c->E, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
-      if (b_gd) launch_stage(c, is, 8, nullptr, 0, 0, s, c->partials, nq, SC_Q_B);
-      else launch_stage(c, is, 2, c->partblk, DELTA_PARTS * nbi, nbi, s, c->partials, nq, SC_Q_B);
+      if (b_gd) launch_stage(c, is, 8, nullptr, 0, s, c->partials, nq, SC_Q_B);
+      else if (late_A)
+        launch_stage(c, is, 10, c->partblk, DELTA_PARTS * nbi, s, c->partials, nq, SC_Q_B, c->partA, n_part_A, SC_DEC_A);
+      else launch_stage(c, is, 2, c->partblk, DELTA_PARTS * nbi, s, c->partials, nq, SC_Q_B);
       // B += tau Delta, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch.  (With a core step P moves
       // there by both steps: nothing reads it in between.)
       launch_axpy_multi(c, c->EH, c->VH, -1.f, c->wn, carry_P && !late_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
                         (int64_t)nbi * db * db, SC_TAU_B, s);
     } else if (!adam) {
-      launch_stage(c, is, 2, nullptr, 0, 0, s);
+      launch_stage(c, is, 2, nullptr, 0, s);
     }
 
     // ---- S-step: exact line search along Gamma (.) M ------------------------------------------
@@ -608,8 +617,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       if (st != ARMOR_OK) return st;
       // V H_w = A (R H_w) and q = <V H_w, V> with V = A Gamma_M B
       int nq = 0;
-      bd_left_dual(c, A, c->Tmp, RH, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
       const bool beta_step = (c->cfg.s_step == ARMOR_S_BETA);
+      bd_left_dual(c, A, c->Tmp, RH, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
       if (beta_step) {
         // the paper's step size (Eq. lrWprime): |A^T A|_F and |B H_w B^T|_F  (these dot products reuse the
         // partial-sum buffer, so q is summed first)
@@ -626,13 +635,12 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
           dot_to_ptr(c, c->Kfull, c->Kfull, (int64_t)nbi * db * db, c->sc + SC_BETA_K, s);
         }
       }
-      launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S,
-                   nrm_part, n_nrm, SC_NRM_S);
+      launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S, nrm_part, n_nrm, SC_NRM_S);
       // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
       launch_axpy_multi(c, S, c->U, 1.f, c->wn, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, RH, 1.f, c->wn, SC_TAU_S, s,
                         late_P ? c->E : nullptr, SC_TAU_B);
     } else if (!adam) {
-      launch_stage(c, is, 3, nullptr, 0, 0, s);
+      launch_stage(c, is, 3, nullptr, 0, s);
     }
 
     // ---- sparse-core update (Algorithm 3), mask_sweeps times ------------------------------------
@@ -646,9 +654,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
             st = residual_and_loss(c, W, H, A, B, S, c->sc + SC_TMP0, s);
             if (st != ARMOR_OK) return st;
           } else {
-            if (carry_P) {
-              launch_mask_carry_P(c, c->P, s);                                       // P += dS B H_w (if accepted)
-            } else {
+            if (!carry_P) {
               st = bd_right_H(c, S, B, H, c->T, c->P, s);                            // T = S B, P = T H_w
               if (st != ARMOR_OK) return st;
             }
@@ -656,14 +662,12 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
           }
         }
         core_gradient(c, A, B, s);
-        launch_mask_select(c, c->Gam, S, M, (uint64_t)(t_first * sweeps + sw), (uint64_t)sweeps, s);   // counter (t_first + it) K + k
-        launch_mask_quadratic(c, A, B, H, s);
-        launch_stage(c, is, 4, c->partblk, nbo * nbi * c->kg, 0, s, c->quadpart, nbo * nbi * c->kg, SC_Q_M);
-        launch_mask_commit(c, S, M, is, s);
+        launch_mask_select(c, A, B, c->Gam, S, M, (uint64_t)(t_first * sweeps + sw), (uint64_t)sweeps, s);   // counter (t_first + it) K + k
+        launch_mask_quadratic(c, A, B, H, is, s);                                    // accepted or not
+        launch_mask_commit(c, S, M, carry_P ? c->P : nullptr, is, s);                // if accepted: S, M and P += dS B H_w
       }
-      if (carry_P) launch_mask_carry_P(c, c->P, s);                                  // P += dS B H_w (if accepted)
     } else {
-      launch_stage(c, is, 5, nullptr, 0, 0, s);
+      launch_stage(c, is, 5, nullptr, 0, s);
     }
     return ARMOR_OK;
   };

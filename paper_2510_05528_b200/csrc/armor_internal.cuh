@@ -103,7 +103,8 @@ struct armor_ctx {
   double* partblk;    // [max(4 * nbo, 4 * nbi, nbo * nbi)] per-block partial sums
   double* quadpart;   // [nbo * nbi] per-block terms of the group updates' quadratic form
   double* colpart;    // [64][d_in] column partial sums of the normalisation
-  int32_t* failflag;  // [max(nbo, nbi)]
+  double* partA;      // [4 * nbo] the A-step's decreases, kept until the B-step's bookkeeping
+  int32_t* failflag;  // [2][max(nbo, nbi)] failed solves of the A-step, of the B-step
   SelRec* sel;        // [nbo * nbi]
   float* tab_key;     // [nbo * nbi] winning race key of every block (single draw)
   unsigned long long* tab_g;   // its global group index
@@ -150,7 +151,7 @@ struct armor_ctx {
 static const int ARMOR_MAX_TIMED = 8192;
 
 // ---------------------------------------------------------------- programmatic dependent launches
-// The kernels of an iteration are short (a layer of 256 x 256: 41 launches, most of them of 2 to 4 us, solves 10, contractions of 256 7 to 9), so the gap between the end of one and
+// The kernels of an iteration are short (a layer of 256 x 256: 36 launches, most of them of 2 to 4 us, solves 9, contractions of 256 7 to 9), so the gap between the end of one and
 // the start of the next counts.  They open with grid_begin(): launched with the attribute below, a kernel's CTAs are put on the
 // SMs once every CTA of the kernel before it has come past its own grid_begin(), and wait there until that kernel has ended and
 // its writes are visible; everything earlier in the stream has ended by then as well.  (Letting the next kernel in before
@@ -395,11 +396,10 @@ void launch_adam(armor_ctx* c, float* theta, const float* gamma, float* m, float
 // part[b] = weight_b * || X_b ||_F for the nblk blocks of db x db floats in X; weight_b = 1, or the Euclidean
 // norm of hdiag over the (b % nbi)-th block of columns; out = sum of the parts (fixed order)
 void launch_block_fro_sum(armor_ctx* c, const float* X, int nblk, const float* hdiag, double* out, cudaStream_t s);
-// per-iteration bookkeeping on the device: stage 0 start, 1 after A, 2 after B, 3 after S, 4 mask accept
+// per-iteration bookkeeping on the device: stage 0 start, 1 after A, 2 after B, 10 after both, 3 after S, 4 mask accept
 // (p1, n1, slot1), (p2, n2, slot2): partial sums the stage first adds up into sc[slot] (a preceding dot product)
-void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, int nflag,
-                  cudaStream_t s, const double* p1 = nullptr, int n1 = 0, int slot1 = 0, const double* p2 = nullptr,
-                  int n2 = 0, int slot2 = 0);
+void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, cudaStream_t s, const double* p1 = nullptr,
+                  int n1 = 0, int slot1 = 0, const double* p2 = nullptr, int n2 = 0, int slot2 = 0);
 void launch_scale_cols(armor_ctx* c, const float* in, const float* colscale, float* out, int64_t rows, int64_t cols, cudaStream_t s);
 void launch_split_hilo(armor_ctx* c, const float* in, float* hi, float* lo, int64_t n, cudaStream_t s);
 void launch_transpose_split(armor_ctx* c, const void* X, int x_dtype, int64_t ldx, int64_t rows, int64_t cols,
@@ -433,15 +433,14 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
 void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s);
 // alpha and the m x m diagonal blocks of K_j = Y_j B_j^T (Y = B_j H_jj, [nbi, db, db]) in one launch
 void launch_mask_prep(armor_ctx* c, const float* A, const float* B, const float* Y, cudaStream_t s);
-// selection counter t = t_base + t_mul * (*c->it_dev)
-void launch_mask_select(armor_ctx* c, const float* Gam, const float* S, const uint8_t* M, uint64_t t_base, uint64_t t_mul,
-                        cudaStream_t s);
-// exact loss change of the iteration's group updates without a dense product: fills quadpart with the per-block
-// terms of tr(V H_w V^T), V = A dS B, from the selection records (the stage kernel adds them into sc[SC_Q_M])
-void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const float* H, cudaStream_t s);
-void launch_mask_commit(armor_ctx* c, float* S, uint8_t* M, armor_iter_stats* st, cudaStream_t s);
-// P += dS B H_w for the accepted group updates, from the rows the guard has formed (full weighting only)
-void launch_mask_carry_P(armor_ctx* c, float* P, cudaStream_t s);
+// selection counter t = t_base + t_mul * (*c->it_dev); with one draw per block also the vectors of launch_mask_quadratic
+void launch_mask_select(armor_ctx* c, const float* A, const float* B, const float* Gam, const float* S, const uint8_t* M, uint64_t t_base,
+                        uint64_t t_mul, cudaStream_t s);
+// exact loss change of the iteration's group updates without a dense product: the per-block terms of tr(V H_w V^T), V = A dS B,
+// from the selection records, their sum and the decision (stage 4)
+void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const float* H, armor_iter_stats* st, cudaStream_t s);
+// the accepted group updates: S and M, and with P (full weighting) P += dS B H_w, for which the guard has formed the rows
+void launch_mask_commit(armor_ctx* c, float* S, uint8_t* M, float* P, armor_iter_stats* st, cudaStream_t s);
 
 // tensor-core GEMM (gemm_tcgen05.cu):  C[M][N] (+)= sum_k A[m][k] * B[n][k]  (both K-major, fp32 storage).
 // passes == 3 uses the split operands (A, Alo, B, Blo).  Partial dot products of the output tile with up

@@ -597,8 +597,20 @@ void bd_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float
   if (c->tc_blocks && tc_block_ok(c, rows, cols) &&
       tc_done(c, tc_bd_left_dual(c, Ablk, false, in1, in2, out, rows, cols, part, n_part, s)))
     return;
-  bd_left(c, Ablk, false, in1, tmp, rows, cols, 1.f, nullptr, 0.f, s);
-  bd_left(c, Ablk, false, in2, out, rows, cols, 1.f, nullptr, 0.f, s);
+  if (((in2 - in1) | (out - tmp)) % 4 == 0) {
+    // both products in one launch: the second input and output a fixed distance from the first
+    const int db = c->db;
+    BGemm g{};
+    g.A = Ablk; g.sAb = (int64_t)db * db; g.sAm = db; g.sAk = 1;
+    g.B = in1; g.sBb = (int64_t)db * cols; g.sBk = cols; g.sBn = 1; g.sBb2 = in2 - in1;
+    g.C = tmp; g.sCb = (int64_t)db * cols; g.sCm = cols; g.sCn = 1; g.sCb2 = out - tmp;
+    g.M = db; g.N = (int)cols; g.K = db; g.batch_inner = (int)(rows / db); g.batch = 2 * g.batch_inner;
+    g.alpha = 1.f;
+    launch_bgemm(c, g, s);
+  } else {
+    bd_left(c, Ablk, false, in1, tmp, rows, cols, 1.f, nullptr, 0.f, s);
+    bd_left(c, Ablk, false, in2, out, rows, cols, 1.f, nullptr, 0.f, s);
+  }
   dot_partials(c, out, tmp, rows * cols, part, s);
   *n_part = ARMOR_DOT_BLOCKS;
 }

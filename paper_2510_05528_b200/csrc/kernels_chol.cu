@@ -329,8 +329,8 @@ __device__ __forceinline__ void solve_block(const float* Lp, const PanelMap& pm,
 
 constexpr int MAX_DB = 256;
 
-// G: a CTA takes 32 G right-hand sides
-template <int G>
+// G: a CTA takes 32 G right-hand sides at a time; SLICES: several times (a loop round a single slice costs 5 % of a launch)
+template <int G, bool SLICES>
 __global__ void __launch_bounds__(NT, 1)
 chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __restrict__ out,
                     const float* dotw, float* A, float ridge, int db, double* __restrict__ part,
@@ -407,9 +407,10 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
   const bool fail = (s_fail != 0);
   const bool hold = (mode == 0) && status[ST_POISON] != 0;   // unusable inputs: the A-step is withheld (X = 0)
 
-  for (int q = blockIdx.y; q < slices; q += gridDim.y) {
+  int q = blockIdx.y;
+  do {
   const int v0 = q * W;                                 // first right-hand side of the slice
-  if (q != (int)blockIdx.y) {                           // (the first one has come with the factor)
+  if (SLICES && q != (int)blockIdx.y) {                 // (the first one has come with the factor)
     __syncthreads();
     load_rhs(v0);
     __syncthreads();
@@ -476,7 +477,8 @@ chol_blocked_kernel(int mode, const float* Gmat, const float* rhs, float* __rest
       part[(int64_t)b * slices + q] = t;
     }
   }
-  }
+  q += gridDim.y;
+  } while (SLICES && q < slices);
   if (tid == 0 && blockIdx.y == 0 && fail) {
     failflag[b] = 1;
     atomicCAS(&status[ST_FIRST_FAIL], 0, b + 1);
@@ -612,19 +614,21 @@ int chol_ctas_per_block(int db, int nb, int n_sm, int slices) {
   return best;
 }
 
-template <int G>
+// the A-step's flags, the B-step's
+int32_t* chol_flags(armor_ctx* c, int mode) { return c->failflag + (mode == 0 ? 0 : (c->nbo > c->nbi ? c->nbo : c->nbi)); }
+
+template <int G, bool SLICES = false>
 armor_status launch_blocked(armor_ctx* c, int mode, const float* Gm, const float* rhs, float* out, const float* dotw, float* A,
                             int nb, double* part, cudaStream_t s) {
-  const int db = c->db;
+  const int db = c->db, slices = (db + 32 * G - 1) / (32 * G);
   const size_t smem = (panel_floats(db) + (size_t)db * (32 * G + 1)) * sizeof(float);
   const int widest = G == 2 ? MAX_DB : 128;
   static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, chol_blocked_kernel<G>,
+  if (ensure_dynamic_smem(attr, c->device, chol_blocked_kernel<G, SLICES>,
                           (panel_floats(widest) + (size_t)widest * (32 * G + 1)) * sizeof(float)) != ARMOR_OK)
     return ARMOR_ERR_CUDA;
-  const int slices = (db + 32 * G - 1) / (32 * G);
-  launch_dependent(chol_blocked_kernel<G>, dim3(nb, chol_ctas_per_block(db, nb, c->n_sm, slices)), NT, smem, s, mode, Gm, rhs, out, dotw, A, c->cfg.ridge, db,
-                                                                                  part, c->failflag, c->status);
+  launch_dependent(chol_blocked_kernel<G, SLICES>, dim3(nb, chol_ctas_per_block(db, nb, c->n_sm, slices)), NT, smem, s, mode, Gm, rhs, out, dotw, A,
+                   c->cfg.ridge, db, part, chol_flags(c, mode), c->status);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
@@ -645,6 +649,7 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
   if (db % NB == 0) {
     const int g = chol_groups(db, nb);
     if (g == 1) return launch_blocked<1>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
+    if (db > 128) return launch_blocked<2, true>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
     if (g == 2) return launch_blocked<2>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
     return launch_blocked<4>(c, mode, Gmat, rhs, out, dotw, A, nb, part, s);
   }
@@ -653,7 +658,7 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
   if (ensure_dynamic_smem(attr_set, c->device, chol_kernel, 2 * 128 * 129 * 4) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int nt = ((db + 31) / 32) * 32;
   launch_dependent(chol_kernel, nb, nt < 64 ? 64 : nt, smem, s, mode, Gmat, rhs, out, dotw, A, c->cfg.ridge, db, part,
-                                                 c->failflag, c->status);
+                                                 chol_flags(c, mode), c->status);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
@@ -711,7 +716,7 @@ __global__ void __launch_bounds__(NT) delta_finish_kernel(float* Delta, const fl
 
 armor_status launch_hjj_inverse(armor_ctx* c, cudaStream_t s) {
   const int nbi = c->nbi;
-  if (cudaMemsetAsync(c->failflag, 0, (size_t)nbi * sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
+  if (cudaMemsetAsync(chol_flags(c, 1), 0, (size_t)nbi * sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
   {
     KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
     launch_dependent(identity_rhs_kernel, nbi, NT, 0, s, c->Ktmp, c->db);
@@ -720,14 +725,14 @@ armor_status launch_hjj_inverse(armor_ctx* c, cudaStream_t s) {
   armor_status st = launch_chol(c, 1, c->Hjj, c->Ktmp, c->Hinv, nullptr, nullptr, nbi, nullptr, s);
   if (st != ARMOR_OK) return st;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  launch_dependent(save_flags_kernel, (nbi + 255) / 256, 256, 0, s, c->failflag, c->hinv_fail, nbi);
+  launch_dependent(save_flags_kernel, (nbi + 255) / 256, 256, 0, s, chol_flags(c, 1), c->hinv_fail, nbi);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
 
 void launch_delta_finish(armor_ctx* c, float* Delta, const float* dotw, double* part, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  launch_dependent(delta_finish_kernel, DELTA_PARTS * c->nbi, NT, 0, s, Delta, dotw, c->hinv_fail, c->failflag, part, c->db);
+  launch_dependent(delta_finish_kernel, DELTA_PARTS * c->nbi, NT, 0, s, Delta, dotw, c->hinv_fail, chol_flags(c, 1), part, c->db);
   c->launches++;
 }
 

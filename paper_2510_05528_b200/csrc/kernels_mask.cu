@@ -112,6 +112,37 @@ __device__ __forceinline__ bool chol_small(int n, const double (&Kin)[NKM][NKM],
   return true;
 }
 
+// The group updates of one iteration change the core by dS (one group per (i, j) block) and the
+// reconstruction by V = A dS B.  Block (i, j) of dS has a single non-zero row r, so
+//   tr(V H_w V^T) = sum_i sum_{j, j'} (a_ij . a_ij') * (z_ij H_w[j, j'] z_ij'^T)
+// with a_ij = A_i[:, r_ij] and z_ij = delta_ij^T B_j[rows of the group, :]: row-blocks decouple because A is
+// block diagonal.  a and z are gathered by the CTA that has solved the group (write_vectors; a launch of its own for several draws per
+// block), a batched product forms y_ij = z_ij H_w[j-th block row, :], and mask_quad_kernel sums the pairs in a fixed order.
+// blk: row block bi, virtual column block v = draw * nbi + column block; by threads t0, t0 + step, .. of a CTA.
+struct VectorArgs { const float* A; const float* B; float* Zsel; float* Acol; int nbo_pad; };
+__device__ __forceinline__ void write_vectors(const VectorArgs& w, const SelRec& rec, int bi, int v, int nbi, int nbv, int db, int mg, int t0, int step) {
+  const int rl = rec.row - bi * db, lc = (rec.cgrp % (db / mg)) * mg;
+  const float* Ai = w.A + (int64_t)bi * db * db + rl;
+  const float* Bj = w.B + (int64_t)(v % nbi) * db * db + (int64_t)lc * db;
+#pragma unroll 4
+  for (int k = t0; k < db; k += step) {
+    float a = 0.f, z = 0.f;
+    if (rec.valid) {
+      a = Ai[(int64_t)k * db];
+      for (int p = 0; p < mg; ++p) z = fmaf(rec.new_val[p] - rec.old_val[p], Bj[(int64_t)p * db + k], z);
+    }
+    w.Acol[((int64_t)bi * nbv + v) * db + k] = a;
+    w.Zsel[((int64_t)v * w.nbo_pad + bi) * db + k] = z;
+  }
+}
+
+__global__ void __launch_bounds__(NT) mask_vectors_kernel(VectorArgs w, const SelRec* sel, int db, int nbi, int mg, int nbv) {
+  grid_begin();
+  const int blk = blockIdx.x;
+  const SelRec rec = sel[blk];
+  write_vectors(w, rec, blk / nbv, blk % nbv, nbi, nbv, db, mg, threadIdx.x, NT);
+}
+
 // One CTA per (i, j) block of the core, N:M groups with M = MG (4 or 8) and N = n_keep (<= NKM: 4 for 2:4 and 4:8, 6 for 5:8 and 6:8).
 // Pass 1: every group of the block is scored, keyed and the arg-min found by warp shuffles.
 // Pass 2: thread b < 2^MG evaluates the mask with bit pattern b (if it keeps exactly n_keep positions);
@@ -120,7 +151,7 @@ __device__ __forceinline__ bool chol_small(int n, const double (&Kin)[NKM][NKM],
 // PHASE 0: both passes in one launch (several draws per block).  A single draw runs as two launches, so that the
 // streaming pass keeps few registers and the per-block solves, which are chains of dependent loads, all run
 // side by side: PHASE 1 is pass 1 alone (the block's winner goes to best_key / best_g), PHASE 2 is pass 2
-// alone (one warp per block for groups of four, 256 threads for groups of eight).
+// alone (one warp per block for groups of four, 256 threads for groups of eight) and gathers the block's vectors for the guard.
 template <int MG, int NKM, bool MULTI, int PHASE>
 __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const float* S,
                                                          const uint8_t* M, const float* alpha,
@@ -129,7 +160,7 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
                                                          int n_keep, int select_mode, uint64_t seed, uint64_t t_base,
                                                          uint64_t t_mul, const int64_t* it_dev,
                                                          uint64_t n_groups_total, int kg_arg,
-                                                         float* tab_key, unsigned long long* tab_g) {
+                                                         float* tab_key, unsigned long long* tab_g, VectorArgs vec) {
   grid_begin();
   const uint64_t t = t_base + t_mul * (uint64_t)(*it_dev);   // selection counter of this run of Algorithm 3
   const int kg = MULTI ? kg_arg : 1;                       // one draw: the loop and the key cache compile away
@@ -279,6 +310,10 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
         part[bi * (kg * nbi) + k2 * nbi + bj] = 0.0;
       }
     }
+    if (PHASE == 2) {
+      SelRec none{};
+      write_vectors(vec, none, bi, bj, nbi, nbi, db, MG, threadIdx.x, blockDim.x);
+    }
     return;
   }
   if (MULTI && threadIdx.x == 0) {                          // out of the race for the later draws
@@ -356,6 +391,7 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
   __shared__ double sred[NT / 32];
   __shared__ unsigned stie[NT / 32], scand[NT / 32];
   __shared__ unsigned s_win;
+  __shared__ SelRec s_rec;
   if ((threadIdx.x & 31) == 0) { sred[threadIdx.x >> 5] = b_red; stie[threadIdx.x >> 5] = b_tie; scand[threadIdx.x >> 5] = b_cand; }
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -371,6 +407,7 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
       for (int p = 0; p < 8; ++p) { rec.new_val[p] = 0.f; rec.old_val[p] = 0.f; }
       sel[blk] = rec;
       part[blk] = 0.0;
+      if (PHASE == 2) s_rec = rec;
     }
   }
   __syncthreads();
@@ -395,36 +432,10 @@ __global__ void __launch_bounds__(NT) mask_select_kernel(const float* Gam, const
     ehv += (double)Gam[row * d_in + cg * MG + p] * ((double)rec.new_val[p] - (double)rec.old_val[p]);
   part[blk] = ehv;
   sel[blk] = rec;
+  if (PHASE == 2) s_rec = rec;
   }
   __syncthreads();                                          // the shared scratch is reused by the next draw
-  }
-}
-
-// The group updates of one iteration change the core by dS (one group per (i, j) block) and the
-// reconstruction by V = A dS B.  Block (i, j) of dS has a single non-zero row r, so
-//   tr(V H_w V^T) = sum_i sum_{j, j'} (a_ij . a_ij') * (z_ij H_w[j, j'] z_ij'^T)
-// with a_ij = A_i[:, r_ij] and z_ij = delta_ij^T B_j[rows of the group, :]: row-blocks decouple because A is
-// block diagonal.  mask_vectors_kernel gathers a and z, a batched product forms y_ij = z_ij H_w[j-th block
-// row, :], and mask_quad_kernel sums the pairs in a fixed order.
-__global__ void __launch_bounds__(NT) mask_vectors_kernel(const float* A, const float* B,
-                                                          const SelRec* sel, float* __restrict__ Zsel,
-                                                          float* __restrict__ Acol, int db, int nbo_pad, int nbi, int mg,
-                                                          int nbv) {
-  grid_begin();
-  const int blk = blockIdx.x;                  // (row block, virtual column block v = draw * nbi + column block)
-  const int bi = blk / nbv, v = blk % nbv, bj = v % nbi;
-  const SelRec rec = sel[blk];
-  for (int k = threadIdx.x; k < db; k += NT) {
-    float a = 0.f, z = 0.f;
-    if (rec.valid) {
-      const int rl = rec.row - bi * db;
-      const int lc = (rec.cgrp % (db / mg)) * mg;
-      a = A[(int64_t)bi * db * db + (int64_t)k * db + rl];
-      const float* Bj = B + (int64_t)bj * db * db;
-      for (int p = 0; p < mg; ++p) z = fmaf(rec.new_val[p] - rec.old_val[p], Bj[(int64_t)(lc + p) * db + k], z);
-    }
-    Acol[((int64_t)bi * nbv + v) * db + k] = a;
-    Zsel[((int64_t)v * nbo_pad + bi) * db + k] = z;
+  if (PHASE == 2) write_vectors(vec, s_rec, bi, bj, nbi, nbi, db, MG, threadIdx.x, blockDim.x);
   }
 }
 
@@ -468,28 +479,29 @@ __global__ void __launch_bounds__(NT) mask_quad_kernel(const float* Zsel, const 
   }
 }
 
-// A thread per block (one CTA walking 3,584 blocks took 21 us).
+// The accepted group of a block goes into the core and its mask; returns whether the mask changed.
+struct CommitArgs { float* S; uint8_t* M; armor_iter_stats* st_base; const int64_t* it_dev; int mg; };
+__device__ __forceinline__ bool commit_group(const CommitArgs& w, const SelRec& rec, int64_t d_in) {
+  if (!rec.valid) return false;
+  float* sp = w.S + (int64_t)rec.row * d_in + (int64_t)rec.cgrp * w.mg;
+  for (int h = 0; h < w.mg / 4; ++h)
+    *reinterpret_cast<float4*>(sp + 4 * h) =
+        make_float4(rec.new_val[4 * h], rec.new_val[4 * h + 1], rec.new_val[4 * h + 2], rec.new_val[4 * h + 3]);
+  w.M[(int64_t)rec.row * (d_in / w.mg) + rec.cgrp] = (uint8_t)rec.new_mask;
+  return rec.new_mask != rec.old_mask;
+}
+__device__ __forceinline__ void count_changed(const CommitArgs& w, bool changed) {          // whole warps
+  const int n = __popc(__ballot_sync(0xffffffffu, changed));
+  if (w.st_base && n && (threadIdx.x & 31) == 0) atomicAdd(&w.st_base[*w.it_dev].groups_changed, n);   // summed over the sweeps of the iteration
+}
+
+// Where nothing is carried: a thread per block (one CTA walking 3,584 blocks took 21 us).
 constexpr int COMMIT_NT = 64;
-__global__ void __launch_bounds__(COMMIT_NT) mask_commit_kernel(const SelRec* sel, int nblocks, float* S,
-                                                                uint8_t* __restrict__ M, int64_t d_in, int mg, const double* sc,
-                                                                armor_iter_stats* st_base, const int64_t* it_dev) {
+__global__ void __launch_bounds__(COMMIT_NT) mask_commit_kernel(const SelRec* sel, int nblocks, int64_t d_in, const double* sc, CommitArgs w) {
   grid_begin();
   if (sc[SC_ACCEPT] == 0.0) return;
   const int b = blockIdx.x * COMMIT_NT + threadIdx.x;
-  bool changed = false;
-  if (b < nblocks) {
-    const SelRec rec = sel[b];
-    if (rec.valid) {
-      float* sp = S + (int64_t)rec.row * d_in + (int64_t)rec.cgrp * mg;
-      for (int h = 0; h < mg / 4; ++h)
-        *reinterpret_cast<float4*>(sp + 4 * h) =
-            make_float4(rec.new_val[4 * h], rec.new_val[4 * h + 1], rec.new_val[4 * h + 2], rec.new_val[4 * h + 3]);
-      M[(int64_t)rec.row * (d_in / mg) + rec.cgrp] = (uint8_t)rec.new_mask;
-      changed = rec.new_mask != rec.old_mask;
-    }
-  }
-  const int n = __popc(__ballot_sync(0xffffffffu, changed));
-  if (st_base && n && (threadIdx.x & 31) == 0) atomicAdd(&st_base[*it_dev].groups_changed, n);   // summed over the sweeps of the iteration
+  count_changed(w, b < nblocks && commit_group(w, sel[b], d_in));
 }
 
 // The accepted group updates change T H_w = S B H_w by the rows (delta^T B_j[group rows, :]) H_w[j-th block
@@ -497,7 +509,7 @@ __global__ void __launch_bounds__(COMMIT_NT) mask_commit_kernel(const SelRec* se
 // blocks (deterministic sums), all of them by the CTA that holds the first.  The grid is (row-block, chunk of 1024 columns,
 // CARRY_PICKS column blocks at a time): one CTA walking all column blocks in batches took 20 us for 50 MB, a chain of batches
 // with few CTAs in flight.  Which pick is a row's first and which its last is found once per CTA in a table of the block's
-// rows (d_block <= 256), so that neither shared memory nor, with at most CARRY_CTAS along the picks, the work grows faster
+// rows (d_block <= 256; one CTA of a row-block also commits its groups), so that neither shared memory nor, with at most CARRY_CTAS along the picks, the work grows faster
 // than their number (thousands with small blocks and several draws).
 constexpr int CARRY_PICKS = 4;
 constexpr int CARRY_CTAS = 64;
@@ -505,13 +517,18 @@ constexpr int CARRY_TAB = 2048;                            // picks whose rows a
 __device__ __forceinline__ int carry_row(const SelRec& rec, int row0) { return rec.valid ? rec.row - row0 : -1; }
 __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* sel, const float* Y,
                                                         float* P, const double* sc,
-                                                        int64_t d_in, int db, int nbo_pad, int nbv) {
+                                                        int64_t d_in, int db, int nbo_pad, int nbv, CommitArgs w) {
   grid_begin();
   __shared__ int row_of[CARRY_TAB];                        // row inside the block, -1: no group
   __shared__ int first[256], last[256];                    // picks of a row
   if (sc[SC_ACCEPT] == 0.0) return;
   const int bi = blockIdx.x, row0 = bi * db;
   const SelRec* mine_sel = sel + (int64_t)bi * nbv;
+  if (blockIdx.y == 0 && blockIdx.z == 0)                   // the block row's groups go into the core
+    for (int j0 = 0; j0 < nbv; j0 += NT) {
+      const int j = j0 + threadIdx.x;
+      count_changed(w, j < nbv && commit_group(w, mine_sel[j], d_in));
+    }
   for (int r = threadIdx.x; r < db; r += NT) { first[r] = nbv; last[r] = -1; }
   __syncthreads();
   for (int j = threadIdx.x; j < nbv; j += NT) {
@@ -552,16 +569,6 @@ __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* sel, const
 }
 
 }  // namespace
-
-void launch_mask_carry_P(armor_ctx* c, float* P, cudaStream_t s) {
-  KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  const int nbv = c->nbi * c->kg;
-  int groups = (nbv + CARRY_PICKS - 1) / CARRY_PICKS;
-  if (groups > CARRY_CTAS) groups = CARRY_CTAS;
-  launch_dependent(mask_carry_kernel, dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s,
-      c->sel, c->Ysel, P, c->sc, c->d_in, c->db, c->nbo_pad, nbv);
-  c->launches++;
-}
 
 void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
@@ -643,12 +650,13 @@ void launch_mask_prep(armor_ctx* c, const float* A, const float* B, const float*
   c->launches++;
 }
 
-void launch_mask_select(armor_ctx* c, const float* Gam, const float* S, const uint8_t* M, uint64_t t_base, uint64_t t_mul,
-                        cudaStream_t s) {
+void launch_mask_select(armor_ctx* c, const float* A, const float* B, const float* Gam, const float* S, const uint8_t* M, uint64_t t_base,
+                        uint64_t t_mul, cudaStream_t s) {
   const int mg = c->cfg.m_group;
   const uint64_t n_groups = (uint64_t)(c->d_out * (c->d_in / mg));
+  const VectorArgs vec{A, B, c->Zsel, c->Acol, c->nbo_pad};
 #define ARMOR_SELECT_ARGS Gam, S, M, c->alpha, c->Kfull, c->sel, c->partblk, c->d_in, c->db, c->nbi, c->cfg.n_keep, \
-                          c->cfg.select_mode, c->cfg.seed, t_base, t_mul, c->it_dev, n_groups, c->kg, c->tab_key, c->tab_g
+                          c->cfg.select_mode, c->cfg.seed, t_base, t_mul, c->it_dev, n_groups, c->kg, c->tab_key, c->tab_g, vec
   // kg > 1: the block's keys stay in shared memory between the draws (up to 64 KiB: d_block 256, groups of four)
   const size_t smem = c->kg > 1 ? (size_t)c->db * (c->db / mg) * sizeof(float) : 0;
 #define ARMOR_SELECT_LAUNCH(MGV, NKV, MULTIV)                                                                           \
@@ -675,13 +683,13 @@ void launch_mask_select(armor_ctx* c, const float* Gam, const float* S, const ui
   c->launches++;
 }
 
-void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const float* H, cudaStream_t s) {
+void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const float* H, armor_iter_stats* st, cudaStream_t s) {
   const int db = c->db, nbo = c->nbo, nbi = c->nbi, nbo_pad = c->nbo_pad, kg = c->kg, nbv = nbi * kg;
-  {
+  if (kg > 1) {
     KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-    launch_dependent(mask_vectors_kernel, nbo * nbv, NT, 0, s, A, B, c->sel, c->Zsel, c->Acol, db, nbo_pad, nbi, c->cfg.m_group, nbv);
+    launch_dependent(mask_vectors_kernel, nbo * nbv, NT, 0, s, VectorArgs{A, B, c->Zsel, c->Acol, nbo_pad}, c->sel, db, nbi, c->cfg.m_group, nbv);
+    c->launches++;
   }
-  c->launches++;
   const float* Y = nullptr;
   if (c->cfg.h_mode == ARMOR_H_FULL) {
     // y_v = z_v H[j-th block row, :], batched over the column blocks j, one launch per draw:  [nbo, db] x [db, d_in]
@@ -705,13 +713,20 @@ void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const f
     launch_dependent(mask_quad_kernel, nbo * nbv, NT, 0, s, c->Zsel, c->Acol, Y, c->hdiag, part, c->d_in, db, nbo_pad, nbi, nbv);
   }
   c->launches++;
-  // (the caller's stage kernel adds the nbo * nbv terms up into sc[SC_Q_M])
+  launch_stage(c, st, 4, c->partblk, nbo * nbv, s, part, nbo * nbv, SC_Q_M);     // the sum of the terms and the decision
 }
 
-void launch_mask_commit(armor_ctx* c, float* S, uint8_t* M, armor_iter_stats* st, cudaStream_t s) {
+void launch_mask_commit(armor_ctx* c, float* S, uint8_t* M, float* P, armor_iter_stats* st, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  const int n = c->nbo * c->nbi * c->kg;
-  launch_dependent(mask_commit_kernel, (n + COMMIT_NT - 1) / COMMIT_NT, COMMIT_NT, 0, s, c->sel, n, S, M, c->d_in, c->cfg.m_group, c->sc, st,
-                                       c->it_dev);
+  const int nbv = c->nbi * c->kg, n = c->nbo * nbv;
+  const CommitArgs w{S, M, st, c->it_dev, c->cfg.m_group};
+  if (P) {
+    int groups = (nbv + CARRY_PICKS - 1) / CARRY_PICKS;
+    if (groups > CARRY_CTAS) groups = CARRY_CTAS;
+    launch_dependent(mask_carry_kernel, dim3(c->nbo, (unsigned)((c->d_in + 1023) / 1024), (unsigned)groups), NT, 0, s, c->sel, c->Ysel, P, c->sc,
+                     c->d_in, c->db, c->nbo_pad, nbv, w);
+  } else {
+    launch_dependent(mask_commit_kernel, (n + COMMIT_NT - 1) / COMMIT_NT, COMMIT_NT, 0, s, c->sel, n, c->d_in, c->sc, w);
+  }
   c->launches++;
 }

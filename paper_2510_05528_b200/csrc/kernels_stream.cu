@@ -410,7 +410,11 @@ __device__ __forceinline__ void stage_scalars(double* sc, armor_iter_stats* st, 
     sc[SC_LOSS] -= psum;
     if (st) { st->loss_A = sc[SC_LOSS]; st->chol_failed += nf; }
     if (nf) atomicAdd(&status[ST_CHOL_FAILS], nf);
-  } else if (stage == 2) {
+  } else if (stage == 2 || stage == 10) {
+    if (stage == 10) {       // the A-step's share first, its decrease in sc[SC_DEC_A]
+      sc[SC_LOSS] -= sc[SC_DEC_A];
+      if (st) st->loss_A = sc[SC_LOSS];
+    }
     const double gd = psum;
     sc[SC_GD_B] = gd;
     const double q = sc[SC_Q_B];
@@ -461,14 +465,17 @@ __device__ __forceinline__ void stage_scalars(double* sc, armor_iter_stats* st, 
   }
 }
 
-// stage 0: start, 1: after A, 2: after B, 3 / 6: after S, 4: mask accept, 5: mask phase off.  One CTA of STAGE_NT threads.
+// stage 0: start, 1: after A, 2: after B, 10: after A and B, 3 / 6: after S, 4: mask accept, 5: mask phase off.  One CTA of STAGE_NT threads.
 // Up to two arrays of partial sums (p1, p2) are first added, in a fixed order, into the scalars slot1 / slot2: the
 // reductions of the dot products that precede the stage need no launch of their own.
 // All sums of a call go through one shuffle tree and one barrier; the scalars and the record thread 0 will need are on their
 // way meanwhile (the kernel is nothing but latency: as a chain of separate sums it took 4 to 6 us, four times an iteration).
+// Left to the last CTA of the kernel that writes the partial sums it costs more than this launch: fences, a counter and cold code, dot
+// product and stage of a 256 x 256 layer 8.1 us together against 1.9 and 2.7.
+// flag_a, flag_b: the flags of the A-step's and of the B-step's solves that this stage counts.
 __global__ void __launch_bounds__(STAGE_NT)
-stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* it_dev, int stage, int32_t* failflag,
-             int nflag, int nflag_clear, const double* partA, int nA, int32_t* status, const double* p1, int n1, int slot1,
+stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* it_dev, int stage, const int32_t* flag_a, int n_flag_a,
+             const int32_t* flag_b, int n_flag_b, const double* partA, int nA, int32_t* status, const double* p1, int n1, int slot1,
              const double* p2, int n2, int slot2) {
   grid_begin();
   __shared__ double sc[SC_COUNT];
@@ -486,9 +493,9 @@ stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* it_dev, int
   int nf = 0;
   if (p1) v[0] = stage_thread_sum(p1, n1);
   if (p2) v[1] = stage_thread_sum(p2, n2);
-  if (stage == 1 || stage == 2 || stage == 4) v[2] = stage_thread_sum(partA, nA);
-  if (stage == 1 || stage == 2)
-    for (int i = threadIdx.x; i < nflag; i += STAGE_NT) nf += failflag[i] ? 1 : 0;
+  if (partA) v[2] = stage_thread_sum(partA, nA);
+  for (int i = threadIdx.x; i < n_flag_a; i += STAGE_NT) nf += flag_a[i] ? 1 : 0;
+  for (int i = threadIdx.x; i < n_flag_b; i += STAGE_NT) nf += flag_b[i] ? 1 : 0;
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
     for (int k = 0; k < 3; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
@@ -497,8 +504,6 @@ stage_kernel(double* sc_g, armor_iter_stats* st_base, const int64_t* it_dev, int
   if (threadIdx.x < SC_COUNT) sc[threadIdx.x] = mine;
   if (lane == 0) { sums[0][warp] = v[0]; sums[1][warp] = v[1]; sums[2][warp] = v[2]; flags[warp] = nf; }
   __syncthreads();
-  // (the flags have been counted: the next solves raise them again)
-  for (int i = threadIdx.x; i < nflag_clear; i += STAGE_NT) failflag[i] = 0;
   if (warp != 0) return;
   v[0] = sums[0][lane]; v[1] = sums[1][lane]; v[2] = sums[2][lane]; nf = flags[lane];
   for (int o = 16; o > 0; o >>= 1) {
@@ -872,18 +877,18 @@ armor_status launch_screen_inputs(armor_ctx* c, const float* W, const float* H, 
 }
 
 void launch_zero_scalars(armor_ctx* c, bool advance, bool carry_loss, armor_iter_stats* st, cudaStream_t s) {
-  const int nflag = c->nbo > c->nbi ? c->nbo : c->nbi;
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  launch_dependent(zero_scalars_kernel, 1, NT, 0, s, c->sc, c->failflag, nflag, carry_loss ? 1 : 0, st, c->it_dev, advance ? 1 : 0);
+  launch_dependent(zero_scalars_kernel, 1, NT, 0, s, c->sc, c->failflag, 2 * (c->nbo > c->nbi ? c->nbo : c->nbi), carry_loss ? 1 : 0, st,
+                   c->it_dev, advance ? 1 : 0);
   c->launches++;
 }
 
-void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, int nflag,
-                  cudaStream_t s, const double* p1, int n1, int slot1, const double* p2, int n2, int slot2) {
+void launch_stage(armor_ctx* c, armor_iter_stats* st, int stage, const double* part, int npart, cudaStream_t s, const double* p1, int n1,
+                  int slot1, const double* p2, int n2, int slot2) {
   KTimer kt(c, ARMOR_KC_SMALL, 0.0, s);
-  const int nflag_clear = stage == 1 ? (c->nbo > c->nbi ? c->nbo : c->nbi) : 0;     // the B-step's solves start afresh
-  launch_dependent(stage_kernel, 1, STAGE_NT, 0, s, c->sc, st, c->it_dev, stage, c->failflag, nflag, nflag_clear, part, npart, c->status, p1,
-                                      n1, slot1, p2, n2, slot2);
+  const int32_t* flag_b = c->failflag + (c->nbo > c->nbi ? c->nbo : c->nbi);
+  launch_dependent(stage_kernel, 1, STAGE_NT, 0, s, c->sc, st, c->it_dev, stage, c->failflag, stage == 1 || stage == 10 ? c->nbo : 0, flag_b,
+                   stage == 2 || stage == 10 ? c->nbi : 0, part, npart, c->status, p1, n1, slot1, p2, n2, slot2);
   c->launches++;
 }
 
