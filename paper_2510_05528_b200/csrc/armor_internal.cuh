@@ -279,6 +279,8 @@ armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, cons
                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s, const float* colw = nullptr,
                               double* part = nullptr);
 
+armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s);
+armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s);
 armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* out,
                                    int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
 

@@ -57,12 +57,11 @@ struct P2Params {
 
 
 // chunk kc of a 128 x 128 block operand whose rows start at row0 of the [*, 128] array behind map: K-major as one
-// box of 128 rows x 32 columns, MN-major as four boxes of 32 x 32 (rows 32 kc .., columns 32 q ..)
+// box of 128 rows x 32 columns, MN-major as four boxes of 32 x 32 (rows 32 kc .., columns 32 q ..) by one instruction
 __device__ __forceinline__ void load_block_chunk(uint32_t dst, const CUtensorMap* map, int mn, int row0, int col0, int kc,
                                                  uint32_t bar) {
   if (mn) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tma_load_2d(dst + q * 4096, map, col0 + 32 * q, row0 + BK * kc, bar);
+    tma_load_mn(dst, map, 1, col0, row0 + BK * kc, bar);
   } else {
     tma_load_2d(dst, map, col0 + BK * kc, row0, bar);
   }
@@ -409,9 +408,10 @@ armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const fl
   p.mask = mask; p.m_group = c->cfg.m_group; p.norm_part = norm_part;
   if (n_norm) *n_norm = 4 * p.nbi * p.nbj;
   CUtensorMap mL, mX, mR, mC;
-  if (!make_map_2d(&mL, Lblk, TILE, rows, TILE, 32, p.l_mn ? 32 : TILE, p.l_mn != 0)) return ARMOR_ERR_CUDA;
-  if (!make_map_2d(&mX, X, cols, rows, cols, 32, 32, true)) return ARMOR_ERR_CUDA;
-  if (!make_map_2d(&mR, Rblk, TILE, cols, TILE, 32, p.r_mn ? 32 : TILE, p.r_mn != 0)) return ARMOR_ERR_CUDA;
+  int wide = 0;                                     // (rows of 128 and of whole tiles: always 1)
+  if (p.l_mn ? !make_map_mn(&mL, Lblk, TILE, rows, TILE, &wide) : !make_map_2d(&mL, Lblk, TILE, rows, TILE, 32, TILE)) return ARMOR_ERR_CUDA;
+  if (!make_map_mn(&mX, X, cols, rows, cols, &wide)) return ARMOR_ERR_CUDA;
+  if (p.r_mn ? !make_map_mn(&mR, Rblk, TILE, cols, TILE, &wide) : !make_map_2d(&mR, Rblk, TILE, cols, TILE, 32, TILE)) return ARMOR_ERR_CUDA;
   if (!make_map_2d(&mC, out, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_block2_kernel, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;

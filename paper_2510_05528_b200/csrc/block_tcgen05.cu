@@ -46,6 +46,7 @@ struct OpCoord {
   int mn_major;                     // 0: K-major, 1: MN-major
   int x_b, x_t, x_k;                // TMA x (inner) coordinate = x_b * batch + x_t * tile + x_k * chunk
   int y_b, y_t, y_k;                // TMA y (outer) coordinate likewise
+  int wide;                         // MN-major: see tma_load_mn
 };
 
 struct BParams {
@@ -74,8 +75,7 @@ __device__ __forceinline__ void load_operand(uint32_t dst, const CUtensorMap* ma
   const int x = o.x_b * b + o.x_t * t + o.x_k * kc;
   const int y = o.y_b * b + o.y_t * t + o.y_k * kc;
   if (o.mn_major) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tma_load_2d(dst + q * 4096, map, x + 32 * q, y, bar);
+    tma_load_mn(dst, map, o.wide, x, y, bar);
   } else {
     tma_load_2d(dst, map, x, y, bar);
   }
@@ -435,14 +435,16 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, i
   } else {
     mD = mC;
   }
-  if (!make_map_2d(&mA, A.base, A.inner, A.outer, A.ld, 32, A.c.mn_major ? 32 : TILE, A.c.mn_major != 0)) return ARMOR_ERR_CUDA;
-  if (!make_map_2d(&mB, B.base, B.inner, B.outer, B.ld, 32, B.c.mn_major ? 32 : TILE, B.c.mn_major != 0)) return ARMOR_ERR_CUDA;
+  p.a = A.c; p.b = B.c;
+  auto op_map = [](CUtensorMap* m, const HostOp& o, const float* base, OpCoord& c) {
+    return o.c.mn_major ? make_map_mn(m, base, o.inner, o.outer, o.ld, &c.wide) : make_map_2d(m, base, o.inner, o.outer, o.ld, 32, TILE);
+  };
+  if (!op_map(&mA, A, A.base, p.a) || !op_map(&mB, B, B.base, p.b)) return ARMOR_ERR_CUDA;
   if (B2) {
-    if (!make_map_2d(&mB2, B2, B.inner, B.outer, B.ld, 32, B.c.mn_major ? 32 : TILE, B.c.mn_major != 0)) return ARMOR_ERR_CUDA;
+    if (!op_map(&mB2, B, B2, p.b)) return ARMOR_ERR_CUDA;
   } else {
     mB2 = mB;
   }
-  p.a = A.c; p.b = B.c;
   p.status = c->status;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_block_kernel<COLW>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
@@ -671,6 +673,7 @@ armor_status tc_colblock_gram_self_pair(armor_ctx* c, const float* U, const floa
 armor_status tc_select_rows_times_H(armor_ctx* c, const float* Z, const float* H, float* Y, int nbo_pad, cudaStream_t s) {
   const int db = c->db;
   if (!ptr_ok(Z) || !ptr_ok(H) || !ptr_ok(Y)) return ARMOR_ERR_UNSUPPORTED;
+  if (c->tc_blocks != 1 && tc_blockres_ok(c) && c->nbo <= TILE) return tc_blockres_thin(c, Z, H, Y, c->nbo, nbo_pad, c->nbi, c->d_in, s);
   HostOp A{Z, db, (int64_t)c->nbi * nbo_pad, db, {0, 0, 0, BK, nbo_pad, TILE, 0}};            // Aop[m][k] = Z[j][m][k]
   HostOp B{H, c->d_in, c->d_in, c->d_in, {1, 0, TILE, 0, db, 0, BK}};                         // Bop[n][k] = H[j*db + k][n]
   BParams p{};

@@ -37,6 +37,7 @@ struct OpCoord {
   int mn_major;                     // 0: K-major, 1: MN-major
   int x_b, x_t, x_k;                // TMA x (inner) coordinate = x_b * batch + x_t * (tile of 128) + x_k * chunk
   int y_b, y_t, y_k;
+  int wide;                         // MN-major: see tma_load_mn
 };
 
 struct PParams {
@@ -59,8 +60,7 @@ __device__ __forceinline__ void load_operand(uint32_t dst, const CUtensorMap* ma
   const int x = o.x_b * b + o.x_t * t + o.x_k * kc;
   const int y = o.y_b * b + o.y_t * t + o.y_k * kc;
   if (o.mn_major) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tma_load_2d(dst + q * 4096, map, x + 32 * q, y, bar);
+    tma_load_mn(dst, map, o.wide, x, y, bar);
   } else {
     tma_load_2d(dst, map, x, y, bar);
   }
@@ -343,8 +343,8 @@ struct HostOp {
   OpCoord c;
 };
 
-inline bool map_operand(CUtensorMap* m, const HostOp& o, const float* base) {
-  return make_map_2d(m, base, o.inner, o.outer, o.ld, 32, o.c.mn_major ? 32 : HALF, o.c.mn_major != 0);
+inline bool map_operand(CUtensorMap* m, const HostOp& o, const float* base, OpCoord& c) {
+  return o.c.mn_major ? make_map_mn(m, base, o.inner, o.outer, o.ld, &c.wide) : make_map_2d(m, base, o.inner, o.outer, o.ld, 32, HALF);
 }
 
 // ldc: leading dimension of C and D.  B2: the second N-side operand (dual); A2, C2: the second M-side operand and output (two)
@@ -361,15 +361,15 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, PParams p, f
   } else {
     mD = mC;
   }
-  if (!map_operand(&mA, A, A.base) || !map_operand(&mB, B, B.base)) return ARMOR_ERR_CUDA;
+  p.a = A.c; p.b = B.c;
+  if (!map_operand(&mA, A, A.base, p.a) || !map_operand(&mB, B, B.base, p.b)) return ARMOR_ERR_CUDA;
   if (B2) {
-    if (!map_operand(&mB2, B, B2)) return ARMOR_ERR_CUDA;
+    if (!map_operand(&mB2, B, B2, p.b)) return ARMOR_ERR_CUDA;
   } else if (A2) {
-    if (!map_operand(&mB2, A, A2)) return ARMOR_ERR_CUDA;
+    if (!map_operand(&mB2, A, A2, p.a)) return ARMOR_ERR_CUDA;
   } else {
     mB2 = mB;
   }
-  p.a = A.c; p.b = B.c;
   p.status = c->status;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_blockpair_kernel, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;

@@ -60,6 +60,7 @@ struct XCoord {
   int mn_major;                     // 0: K-major (right), 1: N-major (left)
   int x_b, x_t, x_k;                // TMA x (inner) coordinate = x_b * block + x_t * tile + x_k * chunk
   int y_b, y_t, y_k;
+  int wide;                         // N-major: see tma_load_mn
 };
 
 struct RParams {
@@ -69,6 +70,8 @@ struct RParams {
   const float* D;                   // addend or nullptr
   int64_t c_rows, c_cols;
   int tiles, batch;                 // tiles per wrapper block along the free dimension; work = batch * tiles tiles
+  int q_rows, m_valid;              // left: distance of two blocks in the rows of Q and of out (128 for wrapper blocks), and how many rows
+                                    // of a block exist (a multiple of 32, or whatever lies in the last 32 is stored as well)
   float alpha, beta;
   int32_t* status;
   const float* colw;                // one product, not null: right: a second output (through mapX2) = out scaled per column by
@@ -159,7 +162,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
             const uint32_t fb = full0 + 8 * stage;
             mbar_expect_tx(fb, STAGE_BYTES);
             const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-            for (int g = 0; g < CH; ++g) tma_load_2d(dst + g * OP_BYTES, &mapQ, 32 * (CH * piece + g), TILE * u.b, fb);
+            for (int g = 0; g < CH; ++g) tma_load_2d(dst + g * OP_BYTES, &mapQ, 32 * (CH * piece + g), p.q_rows * u.b, fb);
             ++issued;
             if (++stage == STAGES) { stage = 0; phase ^= 1; }
           }
@@ -176,8 +179,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
             const int x = p.x.x_b * u.b + p.x.x_t * u.t + p.x.x_k * kc;
             const int y = p.x.y_b * u.b + p.x.y_t * u.t + p.x.y_k * kc;
             if (p.x.mn_major) {
-#pragma unroll
-              for (int q = 0; q < 4; ++q) tma_load_2d(dst + (j * 4 + q) * 4096, mx, x + 32 * q, y, fb);
+              tma_load_mn(dst + j * OP_BYTES, mx, p.x.wide, x, y, fb);
             } else {
               tma_load_2d(dst + j * OP_BYTES, mx, x, y, fb);
             }
@@ -343,19 +345,22 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       }
       for (int kc = 0; kc < TILE / BK; ++kc) {
         if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
-        if (!mbar_wait(lfree0 + 8 * lst, lphase ^ 1, abortp, p.status)) { ok = false; break; }
+        // (all loads ahead of the first store: nothing tells the compiler that the two do not overlap)
+        constexpr int PER = CH * (OP_BYTES / 16 / 128);
         const float4* hi = reinterpret_cast<const float4*>(smem + (size_t)stage * STAGE_BYTES);
         float4* lo = reinterpret_cast<float4*>(smem + LO_OFF + (size_t)lst * STAGE_BYTES);
+        float4 v[PER];
 #pragma unroll
-        for (int e = 0; e < CH * (OP_BYTES / 16 / 128); ++e) {
-          const int idx = t + e * 128;
-          const float4 v = hi[idx];
+        for (int e = 0; e < PER; ++e) v[e] = hi[t + e * 128];
+        if (!mbar_wait(lfree0 + 8 * lst, lphase ^ 1, abortp, p.status)) { ok = false; break; }
+#pragma unroll
+        for (int e = 0; e < PER; ++e) {
           float4 h;
-          h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
-          h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
-          h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
-          h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
-          lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
+          h.x = __uint_as_float(__float_as_uint(v[e].x) & 0xffffe000u);
+          h.y = __uint_as_float(__float_as_uint(v[e].y) & 0xffffe000u);
+          h.z = __uint_as_float(__float_as_uint(v[e].z) & 0xffffe000u);
+          h.w = __uint_as_float(__float_as_uint(v[e].w) & 0xffffe000u);
+          lo[t + e * 128] = make_float4(v[e].x - h.x, v[e].y - h.y, v[e].z - h.z, v[e].w - h.w);
         }
         // make the generic-proxy writes visible to the tensor-core (async proxy) reads
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -426,7 +431,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
       if ((local & 1u) != (uint32_t)h) continue;     // tiles alternate between the accumulators
       const uint32_t aphase = (local >> 1) & 1u;
       // origin of the 128 x 128 tile in out
-      const int64_t row_tile = (int64_t)TILE * (p.right ? u.t : u.b);
+      const int64_t row_tile = p.right ? (int64_t)TILE * u.t : (int64_t)p.q_rows * u.b;
       const int64_t col_tile = (int64_t)TILE * (p.right ? u.b : u.t);
       // The warp's share of the tile goes through shared memory in two halves of two 32 x 32 boxes.  Left: the
       // warp holds rows 32 q .. of the tile and box (hf, ch) covers columns 64 hf + 32 ch ..; right: the warp holds
@@ -440,7 +445,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
         by0[hf] = p.right ? row_tile + 64 * hf : row_tile + 32 * q;
         n_box[hf] = 0;
         for (int ch = 0; ch < 2; ++ch)
-          n_box[hf] += (bx0[hf] + bxs * ch < p.c_cols && by0[hf] + bys * ch < p.c_rows) ? 1 : 0;
+          n_box[hf] += (bx0[hf] + bxs * ch < p.c_cols && by0[hf] + bys * ch < p.c_rows && 32 * q < p.m_valid) ? 1 : 0;
       }
       // left with colw: a half's column scales, lane l holding column l of each box; they travel while the MMAs run or the
       // addend is waited for, and go round by shuffles
@@ -582,30 +587,34 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
 // X2: the second input (DUAL) or the second output (right with colw)
 template <bool DUAL, bool SCALED = false>
 armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, int64_t cols, RParams p, float* out,
-                    cudaStream_t s, const float* X2 = nullptr) {
+                    cudaStream_t s, const float* X2 = nullptr, int kclass = ARMOR_KC_BLOCK_PRODUCT, double kbytes = 0.0) {
   CUtensorMap mX, mX2, mQ, mC, mD;
-  if (!make_map_2d(&mQ, Q, TILE, (int64_t)p.batch * TILE, TILE, 32, TILE)) return ARMOR_ERR_CUDA;
-  if (!make_map_2d(&mC, out, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
+  if (p.q_rows == 0) { p.q_rows = TILE; p.m_valid = TILE; }
+  if (!make_map_2d(&mQ, Q, TILE, (int64_t)p.batch * p.q_rows, TILE, 32, TILE)) return ARMOR_ERR_CUDA;
+  if (!make_map_2d(&mC, out, cols, p.right ? rows : (int64_t)p.batch * p.q_rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
   if (p.D) {
     if (!make_map_2d(&mD, p.D, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
   } else {
     mD = mC;
   }
-  if (!make_map_2d(&mX, X, cols, rows, cols, 32, p.x.mn_major ? 32 : TILE, p.x.mn_major != 0)) return ARMOR_ERR_CUDA;
+  auto x_map = [&](CUtensorMap* m, const float* at) {
+    return p.x.mn_major ? make_map_mn(m, at, cols, rows, cols, &p.x.wide) : make_map_2d(m, at, cols, rows, cols, 32, TILE);
+  };
+  if (!x_map(&mX, X)) return ARMOR_ERR_CUDA;
   if (p.colw && !SCALED) {
     if (!make_map_2d(&mX2, X2, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
   } else if (X2) {
-    if (!make_map_2d(&mX2, X2, cols, rows, cols, 32, p.x.mn_major ? 32 : TILE, p.x.mn_major != 0)) return ARMOR_ERR_CUDA;
+    if (!x_map(&mX2, X2)) return ARMOR_ERR_CUDA;
   } else {
     mX2 = mX;
   }
-  p.c_rows = rows; p.c_cols = cols;
+  p.c_rows = p.right ? rows : (int64_t)p.batch * p.q_rows; p.c_cols = cols;
   p.status = c->status;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_blockres_kernel<DUAL, SCALED>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int64_t n_items = (int64_t)p.batch * p.tiles;
   const int grid = (int)(n_items < c->n_sm ? n_items : c->n_sm);
-  KTimer kt(c, ARMOR_KC_BLOCK_PRODUCT, ((p.D || X2) ? 12.0 : 8.0) * (double)rows * (double)cols, s);
+  KTimer kt(c, kclass, kbytes > 0.0 ? kbytes : ((p.D || X2) ? 12.0 : 8.0) * (double)rows * (double)cols, s);
   launch_dependent(tc_blockres_kernel<DUAL, SCALED>, grid, NTHREADS, SMEM_BYTES, s, mX, mX2, mQ, mC, mD, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
@@ -660,4 +669,16 @@ armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float*
   p.dot_part = part;
   *n_part = 8 * p.batch * p.tiles;
   return launch<true>(c, in1, Ablk, rows, cols, p, out, s, in2);
+}
+
+// out[j][i][:] = Z[j][i][:] * X[128 j .. 128 j + 127, :] for i < n (at most 128), Z [blocks][pad][128], out [blocks][pad][cols], X [128 blocks,
+// cols]: a left product whose blocks have few rows (the guard of the group updates)
+armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s) {
+  if (!ptr_ok(Z) || !ptr_ok(X) || !ptr_ok(out) || n > TILE) return ARMOR_ERR_UNSUPPORTED;
+  RParams p{};
+  p.x = {1, 0, TILE, 0, TILE, 0, BK};
+  p.alpha = 1.f;
+  p.q_rows = pad; p.m_valid = n;
+  p.batch = blocks; p.tiles = (int)((cols + TILE - 1) / TILE);
+  return launch<false>(c, X, Z, (int64_t)blocks * TILE, cols, p, out, s, nullptr, ARMOR_KC_MASK_GUARD, 4.0 * (double)blocks * TILE * (double)cols);
 }

@@ -67,8 +67,7 @@ __device__ __forceinline__ void item_decode(const GParams& p, int item, int& tn,
 __device__ __forceinline__ void load_chunk(uint32_t dst, const CUtensorMap* map, const GParams& p, int b, int t, int kc, uint32_t bar) {
   const int mn = p.db * b + TILE * t, k = BK * kc;
   if (p.mn_major) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) tma_load_2d(dst + q * 4096, map, mn + 32 * q, k, bar);
+    tma_load_mn(dst, map, 1, mn, k, bar);
   } else {
     tma_load_2d(dst, map, k, mn, bar);
   }
@@ -335,13 +334,14 @@ template <int MODE>
 armor_status launch(armor_ctx* c, const float* A, const float* A2, const float* B, float* C, float* C2, const GParams& p, cudaStream_t s) {
   using G = Geo<MODE>;
   CUtensorMap mA, mA2, mB, mC, mC2;
-  const int rows = p.mn_major ? 32 : TILE;
-  const bool atom32 = p.mn_major != 0;
-  if (!make_map_2d(&mA, A, c->d_in, c->d_out, c->d_in, 32, rows, atom32) || !make_map_2d(&mB, B, c->d_in, c->d_out, c->d_in, 32, rows, atom32) ||
-      !make_map_2d(&mC, C, p.c_cols, p.c_rows, p.c_cols, 32, 32))
-    return ARMOR_ERR_CUDA;
-  mA2 = mA; mC2 = mC;
-  if (MODE == 1 && !make_map_2d(&mA2, A2, c->d_in, c->d_out, c->d_in, 32, rows, atom32)) return ARMOR_ERR_CUDA;
+  int wide = 0;                                     // (d_in is a multiple of 128: always 1)
+  auto op_map = [&](CUtensorMap* m, const float* at) {
+    return p.mn_major ? make_map_mn(m, at, c->d_in, c->d_out, c->d_in, &wide) : make_map_2d(m, at, c->d_in, c->d_out, c->d_in, 32, TILE);
+  };
+  if (!op_map(&mA, A) || !op_map(&mB, B) || !make_map_2d(&mC, C, p.c_cols, p.c_rows, p.c_cols, 32, 32)) return ARMOR_ERR_CUDA;
+  mA2 = mA;
+  mC2 = mC;
+  if (MODE == 1 && !op_map(&mA2, A2)) return ARMOR_ERR_CUDA;
   if (MODE != 0 && !make_map_2d(&mC2, C2, p.c_cols, p.c_rows, p.c_cols, 32, 32)) return ARMOR_ERR_CUDA;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_gram_kernel<MODE>, G::SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
