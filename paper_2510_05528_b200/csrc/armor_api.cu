@@ -583,11 +583,10 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
         launch_delta_finish(c, c->Delta, c->GamB, c->partblk, s);                    // part_j = <Gamma_j, Delta_j>
       }
       // direction in B: V = A R with R = S Delta; R H_w serves both V H_w = A (R H_w) and the carried P
-      st = bd_right_H(c, S, c->Delta, H, c->Tmp, c->E, s);                           // R = S Delta, R H_w
-      if (st != ARMOR_OK) return st;
-      // V H_w = A (R H_w) and q = <V H_w, V> with V = A R (summed by the stage; V itself is needed nowhere else)
+      // (R H_w, V H_w = A (R H_w) and q = <V H_w, V>, summed by the stage; V itself is needed nowhere else)
       int nq = 0;
-      bd_left_dual(c, A, c->Tmp, c->E, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
+      st = bd_direction(c, S, c->Delta, A, H, c->Tmp, c->E, c->V, c->VH, c->partials, &nq, s);
+      if (st != ARMOR_OK) return st;
       if (b_gd) launch_stage(c, is, 8, nullptr, 0, s, c->partials, nq, SC_Q_B);
       else if (late_A)
         launch_stage(c, is, 10, c->partblk, DELTA_PARTS * nbi, s, c->partials, nq, SC_Q_B, c->partA, n_part_A, SC_DEC_A);
@@ -613,12 +612,11 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       }
       // (the B-step's R H_w stays in E until P has moved by it; T is free from the A-step on)
       float* const RH = late_P ? c->T : c->E;
-      st = bd_right_H(c, c->U, B, H, c->Tmp, RH, s);                                 // R = Gamma_M B, R H_w
-      if (st != ARMOR_OK) return st;
-      // V H_w = A (R H_w) and q = <V H_w, V> with V = A Gamma_M B
+      // R = Gamma_M B, R H_w, V H_w = A (R H_w) and q = <V H_w, V> with V = A Gamma_M B
       int nq = 0;
       const bool beta_step = (c->cfg.s_step == ARMOR_S_BETA);
-      bd_left_dual(c, A, c->Tmp, RH, c->V, c->VH, d_out, d_in, c->partials, &nq, s);
+      st = bd_direction(c, c->U, B, A, H, c->Tmp, RH, c->V, c->VH, c->partials, &nq, s);
+      if (st != ARMOR_OK) return st;
       if (beta_step) {
         // the paper's step size (Eq. lrWprime): |A^T A|_F and |B H_w B^T|_F  (these dot products reuse the
         // partial-sum buffer, so q is summed first)

@@ -249,6 +249,12 @@ void bd_two_sided(armor_ctx* c, const float* Lblk, bool transL, const float* X, 
 void bd_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* tmp, float* out,
                   int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
 
+// R = in Bdiag (into R), out = Ablk (R H_w) and partial sums of <Ablk R, Ablk (R H_w)>: the products behind a line search's step.  RH takes
+// R H_w where a later move needs it (full weighting) or the kernels want it in memory; with the diagonal weighting and d_block 128 it
+// stays in shared memory.  tmp: scratch
+armor_status bd_direction(armor_ctx* c, const float* in, const float* Bblk, const float* Ablk, const float* H, float* R, float* RH, float* tmp,
+                          float* out, double* part, int* n_part, cudaStream_t s);
+
 // the same two products on the tensor cores (block_tcgen05.cu); d_block must be a multiple of 128
 bool tc_block_ok(const armor_ctx* c, int64_t rows, int64_t cols);
 armor_status tc_bd_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
@@ -282,7 +288,7 @@ armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, cons
 armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s);
 armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s);
 armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* out,
-                                   int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s);
+                                   int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s, const float* colw = nullptr);
 
 // products and per-block Grams of 256 x 256 blocks on pairs of CTAs (blockpair_tcgen05.cu)
 bool tc_blockpair_ok(const armor_ctx* c, int64_t tiles);   // tiles of 256 x 256

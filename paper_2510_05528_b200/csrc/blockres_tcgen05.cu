@@ -12,7 +12,8 @@
 //                 instruction, the MMAs waited for the epilogue and the pass was no faster than the streaming kernel.)
 //                 Left at 4096 x 4096, from HBM: 30 us, 39 with an addend, against 33 and 46 there and 25 for a copy; with operands formed
 //                 in front of every MMA by one lane (tc_common.cuh, umma_tf32_ta_w) it took 34 and 40.
-//   dual product: A.X1 and A.X2 of a tile in one 128 x 256 x 8 instruction.
+//   dual product: A.X1 and A.X2 of a tile in one 128 x 256 x 8 instruction.  With the diagonal weighting X2 = X1 diag(h) is formed
+//                 here, next to the low parts, and never exists in memory.
 //   side "left":   out[128 b + m][n]  = alpha * sum_k Qop_b[m][k] * X[128 b + k][n]  (+ beta * add)
 //   side "right":  out[r][128 b + n]  = alpha * sum_k X[r][128 b + k] * Qop_b[k][n]  (+ beta * add)
 //
@@ -91,11 +92,18 @@ __device__ __forceinline__ bool next_unit(int& item, int i1, int tiles, Unit& u)
   return true;
 }
 
+// x - trunc_tf32(x)
+__device__ __forceinline__ float4 low4(const float4 v) {
+  return make_float4(v.x - __uint_as_float(__float_as_uint(v.x) & 0xffffe000u), v.y - __uint_as_float(__float_as_uint(v.y) & 0xffffe000u),
+                     v.z - __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), v.w - __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
+}
+
 __device__ __forceinline__ uint64_t x_desc(uint32_t base, int mn_major, int kstep) {
   return mn_major ? smem_desc_mn_sw128_32b(base + kstep * 1024, 4096, 512) : smem_desc_sw128(base + kstep * 32, 16, 1024);
 }
 
-// SCALED: left product with column scales (an instantiation of its own, so that plain products stay as they are)
+// SCALED: left product with column scales (an instantiation of its own, so that plain products stay as they are); dual: X2 = X1 scaled
+// per column by colw
 template <bool DUAL, bool SCALED>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapX2,
@@ -172,9 +180,10 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
         for (int kc = 0; kc < TILE / BK; ++kc) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
           const uint32_t fb = full0 + 8 * stage;
-          mbar_expect_tx(fb, STAGE_BYTES);
+          constexpr int LOADED = SCALED ? 1 : CH;
+          mbar_expect_tx(fb, LOADED * OP_BYTES);
           const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          for (int j = 0; j < CH; ++j) {
+          for (int j = 0; j < LOADED; ++j) {
             const CUtensorMap* mx = j ? &mapX2 : &mapX;                 // dual: the same tile of the second input
             const int x = p.x.x_b * u.b + p.x.x_t * u.t + p.x.x_k * kc;
             const int y = p.x.y_b * u.b + p.x.y_t * u.t + p.x.y_k * kc;
@@ -343,11 +352,19 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
         ++w_loads;
         cur_b = u.b;
       }
+      // dual with scales: this thread's 16-byte unit of a box row, t % 8 of row t / 8, holds the same four columns of every box (32-byte
+      // atoms of a row change places by row % 4)
+      float4 cw[4];
+      if (DUAL && SCALED) {
+        const float* w = p.colw + (int64_t)TILE * u.t + 8 * (((t & 7) >> 1) ^ ((t >> 3) & 3)) + 4 * (t & 1);
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) cw[q2] = *reinterpret_cast<const float4*>(w + 32 * q2);
+      }
       for (int kc = 0; kc < TILE / BK; ++kc) {
         if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
         // (all loads ahead of the first store: nothing tells the compiler that the two do not overlap)
-        constexpr int PER = CH * (OP_BYTES / 16 / 128);
-        const float4* hi = reinterpret_cast<const float4*>(smem + (size_t)stage * STAGE_BYTES);
+        constexpr int PER = (SCALED ? 1 : CH) * (OP_BYTES / 16 / 128);
+        float4* hi = reinterpret_cast<float4*>(smem + (size_t)stage * STAGE_BYTES);
         float4* lo = reinterpret_cast<float4*>(smem + LO_OFF + (size_t)lst * STAGE_BYTES);
         float4 v[PER];
 #pragma unroll
@@ -355,12 +372,13 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
         if (!mbar_wait(lfree0 + 8 * lst, lphase ^ 1, abortp, p.status)) { ok = false; break; }
 #pragma unroll
         for (int e = 0; e < PER; ++e) {
-          float4 h;
-          h.x = __uint_as_float(__float_as_uint(v[e].x) & 0xffffe000u);
-          h.y = __uint_as_float(__float_as_uint(v[e].y) & 0xffffe000u);
-          h.z = __uint_as_float(__float_as_uint(v[e].z) & 0xffffe000u);
-          h.w = __uint_as_float(__float_as_uint(v[e].w) & 0xffffe000u);
-          lo[t + e * 128] = make_float4(v[e].x - h.x, v[e].y - h.y, v[e].z - h.z, v[e].w - h.w);
+          lo[t + e * 128] = low4(v[e]);
+          if (DUAL && SCALED) {
+            const float4 w = cw[e >> 1];                        // (two 16-row halves of a box)
+            const float4 x2 = make_float4(v[e].x * w.x, v[e].y * w.y, v[e].z * w.z, v[e].w * w.w);
+            hi[OP_BYTES / 16 + t + e * 128] = x2;
+            lo[OP_BYTES / 16 + t + e * 128] = low4(x2);
+          }
         }
         // make the generic-proxy writes visible to the tensor-core (async proxy) reads
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -657,18 +675,21 @@ armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, cons
 }
 
 // out[i-th block, :] = P_i * in2[i-th block, :] and 8 partial sums per 128 x 128 tile of <P_i * in1, P_i * in2> at part
-// (tile order, then the eight 32 x 64 pieces of the tile); the number of partial sums comes back through n_part
+// (tile order, then the eight 32 x 64 pieces of the tile); the number of partial sums comes back through n_part.  in2 null: in1 scaled
+// per column by colw
 armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* out,
-                                   int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s) {
+                                   int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s, const float* colw) {
   if (!ptr_ok(in1) || !ptr_ok(in2) || !ptr_ok(Ablk) || !ptr_ok(out)) return ARMOR_ERR_UNSUPPORTED;
+  if ((in2 == nullptr) != (colw != nullptr) || (colw && (cols % TILE || !ptr_ok(colw)))) return ARMOR_ERR_UNSUPPORTED;
   RParams p{};
+  p.colw = colw;
   p.x = {1, 0, TILE, 0, TILE, 0, BK};
   p.col_read = 0; p.right = 0;
   p.D = nullptr; p.alpha = 1.f; p.beta = 0.f;
   p.batch = (int)(rows / TILE); p.tiles = (int)((cols + TILE - 1) / TILE);
   p.dot_part = part;
   *n_part = 8 * p.batch * p.tiles;
-  return launch<true>(c, in1, Ablk, rows, cols, p, out, s, in2);
+  return colw ? launch<true, true>(c, in1, Ablk, rows, cols, p, out, s) : launch<true>(c, in1, Ablk, rows, cols, p, out, s, in2);
 }
 
 // out[j][i][:] = Z[j][i][:] * X[128 j .. 128 j + 127, :] for i < n (at most 128), Z [blocks][pad][128], out [blocks][pad][cols], X [128 blocks,
