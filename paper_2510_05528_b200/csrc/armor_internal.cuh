@@ -129,7 +129,7 @@ struct armor_ctx {
   int tc_blocks;        // 1, 2, 3: block products and per-block Grams on the tensor cores where the shape allows.
                         // 1: the streaming kernel for every product; 2: with d_block = 128 the kernel that keeps the
                         // wrapper block in tensor memory (products and dual products); 3 (default): that kernel for
-                        // dual products, right products with the column-scaled second output and other three-pass
+                        // dual products and other three-pass
                         // products of many tiles, else the streaming kernel, the two-sided kernel where both wrappers apply;
                         // 0: always the fp32 CUDA-core kernels (exact products with 0 and 1)
   int gram_pairs;       // 1: the two per-block Grams of a step in one launch (shared operand read once)
@@ -259,6 +259,8 @@ armor_status bd_direction(armor_ctx* c, const float* in, const float* Bblk, cons
 bool tc_block_ok(const armor_ctx* c, int64_t rows, int64_t cols);
 armor_status tc_bd_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
                          int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
+armor_status tc_bd_right_scaled(armor_ctx* c, const float* in, const float* Bblk, float* out, const float* colw, float* out2, int64_t rows, int64_t cols,
+                                cudaStream_t s);
 armor_status tc_bd_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
                         int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
 
@@ -279,8 +281,7 @@ armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* i
 // the same with the wrapper block held in tensor memory (blockres_tcgen05.cu); d_block = 128
 bool tc_blockres_ok(const armor_ctx* c);
 armor_status tc_blockres_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
-                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s,
-                               const float* colw = nullptr, float* out2 = nullptr);
+                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s);
 armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, const float* in, float* out, int64_t rows,
                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s, const float* colw = nullptr,
                               double* part = nullptr);

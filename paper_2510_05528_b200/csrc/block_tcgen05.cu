@@ -102,8 +102,9 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t base, int mn_major, in
 }
 
 
-// COLW: with column scales (an instantiation of its own: as a branch of the store loop it cost every plain product 10 %)
-template <bool COLW>
+// COLW: with column scales (instantiations of their own: as a branch of the store loop they cost every plain product 10 %); 1: the output
+// scaled, with its dot product, 2: the output and a scaled second one (through mapB2)
+template <int COLW>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                 const __grid_constant__ CUtensorMap mapB2, const __grid_constant__ CUtensorMap mapC,
@@ -283,7 +284,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
       const uint32_t aphase = (uint32_t)(local >> 1) & 1u;
       const int64_t row_base = p.r_b * b + (int64_t)tm * TILE + q * 32;
       const int64_t col_tile = p.c_b * b + (int64_t)tn * TILE;
-      if (!COLW && p.dual) {
+      if (COLW == 0 && p.dual) {
         // C = alpha * (A.B2); partial sum of <A.B1, A.B2> over this warp's 32 x 128 slab (rows or columns past the
         // end of the operands were read as zeros and add nothing)
         double dot = 0.0;
@@ -334,6 +335,45 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
         if (ok && lane == 0) p.dot_part[(size_t)item * 4 + q] = dot;
         continue;
       }
+      if (COLW == 2) {
+        // the two boxes of a 32 x 32 piece: as it is, and scaled
+        const bool rows_in = row_base < p.c_rows && tm * TILE + q * 32 < p.m_valid;
+        float cw[4];                                // lane l holds the scale of column l of each piece
+#pragma unroll
+        for (int k = 0; k < 4; ++k) cw[k] = p.colw[col_tile + 32 * k + lane];
+        if (!mbar_wait(tfull0 + 8 * as, aphase, abortp, p.status)) { ok = false; break; }
+        tc_fence_after();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          uint32_t r[32];
+          tmem_ld32(tmem_base + (uint32_t)(as * TILE + k * 32) + ((uint32_t)(q * 32) << 16), r);
+          if (k == 3) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(tempty0 + 8 * as);
+          }
+          if (lane == 0) tma_store_wait_read();     // the previous stores have read the boxes
+          __syncwarp();
+          uint8_t* rowp = buf + lane * 128;
+#pragma unroll
+          for (int cq = 0; cq < 8; ++cq) {
+            float4* cell = reinterpret_cast<float4*>(rowp + ((cq ^ (lane & 7)) << 4));
+            const float4 v = make_float4(p.alpha * __uint_as_float(r[4 * cq]), p.alpha * __uint_as_float(r[4 * cq + 1]),
+                                         p.alpha * __uint_as_float(r[4 * cq + 2]), p.alpha * __uint_as_float(r[4 * cq + 3]));
+            cell[0] = v;
+            cell[256] = make_float4(v.x * __shfl_sync(0xffffffffu, cw[k], 4 * cq), v.y * __shfl_sync(0xffffffffu, cw[k], 4 * cq + 1),
+                                    v.z * __shfl_sync(0xffffffffu, cw[k], 4 * cq + 2), v.w * __shfl_sync(0xffffffffu, cw[k], 4 * cq + 3));
+          }
+          fence_proxy_async();
+          __syncwarp();
+          if (lane == 0 && rows_in) {
+            tma_store_2d(&mapC, (int)(col_tile + 32 * k), (int)row_base, buf_u32);
+            tma_store_2d(&mapB2, (int)(col_tile + 32 * k), (int)row_base, buf_u32 + 4096);
+            tma_store_commit();
+          }
+        }
+        continue;
+      }
       // The warp's 32 x 128 slab goes through shared memory in two halves of 64 columns (two 32 x 32 boxes).
       bool waited = false;
       double wdot = 0.0;
@@ -344,7 +384,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
         if (row_base < p.c_rows && tm * TILE + q * 32 < p.m_valid)
           for (int ch = 0; ch < 2; ++ch) n_box += (col_tile + 64 * hf + 32 * ch < p.c_cols) ? 1 : 0;
         float cw0 = 0.f, cw1 = 0.f;                 // colw: lane l holds the scale of column l of each box (handed round by shuffles)
-        if (COLW) { cw0 = p.colw[col_tile + 64 * hf + lane]; cw1 = p.colw[col_tile + 64 * hf + 32 + lane]; }
+        if (COLW == 1) { cw0 = p.colw[col_tile + 64 * hf + lane]; cw1 = p.colw[col_tile + 64 * hf + 32 + lane]; }
         if (lane == 0) {
           tma_store_wait_read();                    // the previous stores have read the staging boxes
           if (p.D && n_box > 0) {
@@ -382,7 +422,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
               v.x = fmaf(p.beta, d.x, v.x); v.y = fmaf(p.beta, d.y, v.y);
               v.z = fmaf(p.beta, d.z, v.z); v.w = fmaf(p.beta, d.w, v.w);
             }
-            if (COLW) {
+            if (COLW == 1) {
               const float4 e = make_float4(v.x * __shfl_sync(0xffffffffu, w, 4 * cq), v.y * __shfl_sync(0xffffffffu, w, 4 * cq + 1),
                                            v.z * __shfl_sync(0xffffffffu, w, 4 * cq + 2), v.w * __shfl_sync(0xffffffffu, w, 4 * cq + 3));
               wpart = fmaf(v.x, e.x, wpart); wpart = fmaf(v.y, e.y, wpart); wpart = fmaf(v.z, e.z, wpart); wpart = fmaf(v.w, e.w, wpart);
@@ -391,7 +431,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
             *cell = v;
           }
         }
-        if (COLW) wdot += (double)wpart;
+        if (COLW == 1) wdot += (double)wpart;
         if (hf == 1) tc_fence_before();             // all reads of the accumulator are done
         fence_proxy_async();
         __syncwarp();
@@ -402,7 +442,7 @@ tc_block_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant_
           tma_store_commit();
         }
       }
-      if (COLW) {
+      if (COLW == 1) {
         // lanes in a fixed order
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wdot += __shfl_xor_sync(0xffffffffu, wdot, o);
@@ -424,10 +464,10 @@ struct HostOp {
   OpCoord c;
 };
 
-// B2: the second N-side operand (dual)
-template <bool COLW = false>
+// B2: the second N-side operand (dual); C2: the second output (COLW 2)
+template <int COLW = 0>
 armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, int kclass, double kbytes, cudaStream_t s,
-                    const float* B2 = nullptr) {
+                    const float* B2 = nullptr, const float* C2 = nullptr) {
   CUtensorMap mA, mB, mB2, mC, mD;
   if (!make_map_2d(&mC, p.C, p.c_cols, p.c_rows, p.ldc, 32, 32)) return ARMOR_ERR_CUDA;
   if (p.D) {
@@ -440,7 +480,9 @@ armor_status launch(armor_ctx* c, const HostOp& A, const HostOp& B, BParams p, i
     return o.c.mn_major ? make_map_mn(m, base, o.inner, o.outer, o.ld, &c.wide) : make_map_2d(m, base, o.inner, o.outer, o.ld, 32, TILE);
   };
   if (!op_map(&mA, A, A.base, p.a) || !op_map(&mB, B, B.base, p.b)) return ARMOR_ERR_CUDA;
-  if (B2) {
+  if (COLW == 2) {
+    if (!make_map_2d(&mB2, C2, p.c_cols, p.c_rows, p.ldc, 32, 32)) return ARMOR_ERR_CUDA;
+  } else if (B2) {
     if (!op_map(&mB2, B, B2, p.b)) return ARMOR_ERR_CUDA;
   } else {
     mB2 = mB;
@@ -499,6 +541,27 @@ armor_status tc_bd_right(armor_ctx* c, const float* in, const float* Bblk, bool 
   p.batch_fastest = 1;   // neighbouring CTAs read neighbouring column blocks of the same rows
   p.one_pass = c->block_one_pass;
   return launch(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, (add ? 12.0 : 8.0) * (double)rows * (double)cols, s);
+}
+
+// out[:, j-th block] = in[:, j-th block] * Bblk[j] and out2 = out scaled per column by colw.  On the streaming kernel at every size: its
+// epilogue holds rows, where the one that keeps the block in tensor memory holds the tile transposed and went over its boxes word by word
+// (1024 x 5120 19 / 42 us, 4096 x 4096 37 / 68, 14336 x 4096 120 / 182); blocks of 256 in two launches (pairs, column scale) 14336 x 4096 189 / 245.
+armor_status tc_bd_right_scaled(armor_ctx* c, const float* in, const float* Bblk, float* out, const float* colw, float* out2, int64_t rows, int64_t cols,
+                                cudaStream_t s) {
+  const int db = c->db, nb = (int)(cols / db);
+  if (!ptr_ok(in) || !ptr_ok(Bblk) || !ptr_ok(out) || !ptr_ok(out2)) return ARMOR_ERR_UNSUPPORTED;
+  HostOp A{in, cols, rows, cols, {0, db, 0, BK, 0, TILE, 0}};
+  HostOp B{Bblk, db, (int64_t)nb * db, db, {1, 0, TILE, 0, db, 0, BK}};
+  BParams p{};
+  p.C = out; p.ldc = cols; p.c_rows = rows; p.c_cols = cols;
+  p.c_b = db;
+  p.m_tiles = (int)((rows + TILE - 1) / TILE); p.n_tiles = db / TILE; p.batch = nb; p.k_chunks = db / BK;
+  p.alpha = 1.f;
+  p.m_valid = 1 << 30;
+  p.batch_fastest = 1;
+  p.one_pass = c->block_one_pass;
+  p.colw = colw;
+  return launch<2>(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, 12.0 * (double)rows * (double)cols, s, nullptr, out2);
 }
 
 // out[i-th block, :] = alpha * P_i * in[i-th block, :] (+ beta * add[i-th block, :]),  P_i = Ablk[i] or its transpose
@@ -579,7 +642,7 @@ armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* i
   p.colw = colw; p.dot_part = part;
   *n_part = 4 * p.batch * p.m_tiles * p.n_tiles;
   // two W-shaped reads (in, add), one write
-  return launch<true>(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, 12.0 * (double)rows * (double)cols, s);
+  return launch<1>(c, A, B, p, ARMOR_KC_BLOCK_PRODUCT, 12.0 * (double)rows * (double)cols, s);
 }
 
 namespace {

@@ -28,8 +28,7 @@
 //   warp 1     : MMA issuer   (tcgen05.mma kind::tf32, A from tensor memory)
 //   warps 2-5  : move the wrapper block from its stages into tensor memory when the block changes (tcgen05.st), then per
 //                chunk write the low part of X into a ring of its own
-//   warps 6-13 : epilogue (addend prefetched by TMA, tcgen05.ld, alpha / beta, TMA store; optionally a second output
-//                scaled per column); the second half of a warp's share is taken into registers before the first half's
+//   warps 6-13 : epilogue (addend prefetched by TMA, tcgen05.ld, alpha / beta, TMA store); the second half of a warp's share is taken into registers before the first half's
 //                store is waited for, so the accumulator is released early
 // The three MMAs per k-step are issued in the same order as in the streaming kernel (low part of the M-side
 // operand of the UNtransposed product first), so both kernels give the same bits.
@@ -75,8 +74,7 @@ struct RParams {
                                     // of a block exist (a multiple of 32, or whatever lies in the last 32 is stored as well)
   float alpha, beta;
   int32_t* status;
-  const float* colw;                // one product, not null: right: a second output (through mapX2) = out scaled per column by
-                                    // colw; left: out itself is scaled per column, dot_part = sum of out * out scaled
+  const float* colw;                // SCALED: the column scales.  One product (left): out is scaled, dot_part = sum of out * out scaled
   // dual (left only): the two halves of an instruction are the same tile of two inputs (mapX, mapX2);
   // out = alpha * Q.X2, dot_part = <Q.X1, Q.X2>
   double* dot_part;                 // dual: 8 partial sums per tile (one per epilogue warp), left with colw: 4, in tile order
@@ -528,27 +526,6 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
             tma_store_2d(&mapC, (int)(bx0[hf] + bxs * ch), (int)(by0[hf] + bys * ch), buf_u32 + ch * 4096);
           tma_store_commit();
         }
-        if (!SCALED && p.colw) {
-          // the boxes still hold out (lane = column): once the store has read them they become the second output
-          if (lane == 0) tma_store_wait_read();
-          __syncwarp();
-          const float w = n_box[hf] > 0 ? __ldg(p.colw + bx0[hf] + lane) : 0.f;
-          for (int ch = 0; ch < n_box[hf]; ++ch) {
-            uint8_t* colp = buf + ch * 4096 + (lane & 3) * 4;
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              float* cell = reinterpret_cast<float*>(colp + i * 128 + (((lane >> 2) ^ (i & 7)) << 4));
-              *cell *= w;
-            }
-          }
-          fence_proxy_async();
-          __syncwarp();
-          if (lane == 0) {
-            for (int ch = 0; ch < n_box[hf]; ++ch)
-              tma_store_2d(&mapX2, (int)(bx0[hf] + bxs * ch), (int)(by0[hf] + bys * ch), buf_u32 + ch * 4096);
-            tma_store_commit();
-          }
-        }
       };
       const uint32_t tacc = tmem_base + (uint32_t)(h * TILE) + ((uint32_t)(q * 32) << 16);
 
@@ -602,7 +579,7 @@ tc_blockres_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_consta
   }
 }
 
-// X2: the second input (DUAL) or the second output (right with colw)
+// X2: the second input (DUAL)
 template <bool DUAL, bool SCALED = false>
 armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, int64_t cols, RParams p, float* out,
                     cudaStream_t s, const float* X2 = nullptr, int kclass = ARMOR_KC_BLOCK_PRODUCT, double kbytes = 0.0) {
@@ -619,9 +596,7 @@ armor_status launch(armor_ctx* c, const float* X, const float* Q, int64_t rows, 
     return p.x.mn_major ? make_map_mn(m, at, cols, rows, cols, &p.x.wide) : make_map_2d(m, at, cols, rows, cols, 32, TILE);
   };
   if (!x_map(&mX, X)) return ARMOR_ERR_CUDA;
-  if (p.colw && !SCALED) {
-    if (!make_map_2d(&mX2, X2, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
-  } else if (X2) {
+  if (X2) {
     if (!x_map(&mX2, X2)) return ARMOR_ERR_CUDA;
   } else {
     mX2 = mX;
@@ -644,19 +619,16 @@ inline bool ptr_ok(const void* q) { return (reinterpret_cast<uintptr_t>(q) & 15)
 
 bool tc_blockres_ok(const armor_ctx* c) { return c->db == TILE && !c->block_one_pass; }
 
-// out[:, j-th block] = alpha * in[:, j-th block] * Q_j (+ beta * add[:, j-th block]),  Q_j = Bblk[j] or its transpose; with
-// colw also out2 = out scaled per column by colw
+// out[:, j-th block] = alpha * in[:, j-th block] * Q_j (+ beta * add[:, j-th block]),  Q_j = Bblk[j] or its transpose
 armor_status tc_blockres_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, float* out, int64_t rows,
-                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s, const float* colw,
-                               float* out2) {
-  if ((colw == nullptr) != (out2 == nullptr) || (out2 && !ptr_ok(out2))) return ARMOR_ERR_UNSUPPORTED;
+                               int64_t cols, float alpha, const float* add, float beta, cudaStream_t s) {
   if (!ptr_ok(in) || !ptr_ok(Bblk) || !ptr_ok(out) || (add && !ptr_ok(add))) return ARMOR_ERR_UNSUPPORTED;
   RParams p{};
   p.x = {0, TILE, 0, BK, 0, TILE, 0};     // N side [n = row of in][k]: x = 128 j + 32 kc, y = 128 t  (K-major)
-  p.col_read = transB ? 0 : 1; p.right = 1; p.colw = colw;
+  p.col_read = transB ? 0 : 1; p.right = 1;
   p.D = add; p.alpha = alpha; p.beta = add ? beta : 0.f;
   p.batch = (int)(cols / TILE); p.tiles = (int)((rows + TILE - 1) / TILE);
-  return launch<false>(c, in, Bblk, rows, cols, p, out, s, out2);
+  return launch<false>(c, in, Bblk, rows, cols, p, out, s);
 }
 
 // out[i-th block, :] = alpha * P_i * in[i-th block, :] (+ beta * add[i-th block, :]),  P_i = Ablk[i] or its transpose; with colw

@@ -559,8 +559,8 @@ void bd_right(armor_ctx* c, const float* in, const float* Bblk, bool transB, flo
 armor_status bd_right_H(armor_ctx* c, const float* in, const float* Bblk, const float* H, float* out, float* outH, cudaStream_t s) {
   const int64_t rows = c->d_out, cols = c->d_in;
   // diagonal weighting: the column scale is a second output of the product's epilogue (same multiplications)
-  if (c->cfg.h_mode == ARMOR_H_DIAG && c->tc_blocks > 1 && tc_block_ok(c, rows, cols) && tc_blockres_ok(c) &&
-      tc_done(c, tc_blockres_right(c, in, Bblk, false, out, rows, cols, 1.f, nullptr, 0.f, s, c->hdiag, outH)))
+  if (c->cfg.h_mode == ARMOR_H_DIAG && c->tc_blocks && tc_block_ok(c, rows, cols) &&
+      tc_done(c, tc_bd_right_scaled(c, in, Bblk, out, c->hdiag, outH, rows, cols, s)))
     return ARMOR_OK;
   bd_right(c, in, Bblk, false, out, rows, cols, 1.f, nullptr, 0.f, s);
   return rmul_H(c, out, H, outH, rows, nullptr, nullptr, nullptr, nullptr, s);

@@ -37,7 +37,6 @@ AHEAD = {
 WRITTEN = {"sum_slabs_kernel": {"out0", "out1"}, "bgemm_tile_kernel": {"part_out"}, "split_rows_kernel": {"hi", "lo"}}
 # Data read through __ldg, and why that is older than the kernel before
 LDG = {
-    ("blockres_tcgen05.cu", "__ldg(p.colw + bx0[hf] + lane)"): "H's diagonal: written once a call, a right product or a scalar kernel in between",
     ("split_f16.cu", "__ldg(reinterpret_cast<const uint4*>(X + r * ldx + col))"): "gram_range_kernel, launched without the attribute",
 }
 

@@ -285,3 +285,33 @@ def test_weighted_residual_of_the_diagonal_weighting(d_out, d_in, d_block):
         assert (a[k] - b[k]).double().norm() <= 1e-4 * b[k].double().norm()
     for k in (2, 3):
         assert abs(a[k] - b[k]) <= 2 * tol * b[k]
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(128, 128, 128), (384, 640, 128), (1536, 3200, 128), (2560, 4096, 128), (256, 512, 256), (1024, 1280, 256)])
+def test_line_search_of_the_core_with_the_diagonal_weighting(d_out, d_in, d_block):
+    """The core's step alone: R = Gamma_M B and R diag(h), which with d_block 128 exists in shared memory only; tau = |Gamma_M|^2 / q with
+    q = <A R, A R diag(h)> and S += tau Gamma_M, against fp64.  Four wrapper products in a row, each with 3 d_block / 8 truncating additions of up
+    to 2^-24; q is quadratic in the last two of them: 6 (3 d_block / 8) 2^-24 of tau, and as much of the move."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + 3 * d_in)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    h = torch.rand(d_in, device=DEV, generator=g) * 3 + 0.1
+    H = torch.diag(h)
+    ctx = _ctx(d_out, d_in, d_block, h_mode=Bd.H_DIAG, phases=4)
+    st = ctx.init(W, H)
+    st.A.add_(torch.randn(st.A.shape, device=DEV, generator=g), alpha=0.05)
+    st.B.add_(torch.randn(st.B.shape, device=DEV, generator=g), alpha=0.05)
+    A, B, S = st.A.double(), st.B.double(), st.S.double()
+    left = lambda P, X: torch.einsum("imk,ikn->imn", P, X.view(-1, d_block, d_in)).reshape(d_out, d_in)
+    right = lambda X, P: torch.einsum("rjk,jkn->rjn", X.view(d_out, -1, d_block), P).reshape(d_out, d_in)
+    EH = (W.double() - left(A, right(S, B))) * h.double()
+    keep = ((st.M.long()[:, :, None] >> torch.arange(4, device=DEV)) & 1).bool().view(d_out, d_in)
+    G = right(left(A.transpose(1, 2), EH), B.transpose(1, 2)) * keep
+    V = left(A, right(G, B))
+    tau = ((G * G).sum() / (V * V * h.double()).sum()).item()
+    stats = ctx.read_stats(ctx.bcd_step(st, H, 0, 1))
+    tol = 6 * 3 * d_block / 8 * 2.0 ** -24
+    assert abs(stats["tau_S"][0] - tau) <= tol * tau
+    move = st.S.double() - S
+    assert (move - tau * G).norm() <= tol * (tau * G).norm() + 2.0 ** -24 * S.norm()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
