@@ -109,21 +109,23 @@ def _check(code: int, where: str) -> None:
         raise ArmorError(code, where)
 
 
-def _ptr(t: torch.Tensor | None, dtype=None, name: str = "tensor") -> C.c_void_p:
+def _ptr(t: torch.Tensor | None, dtype=None, name: str = "tensor") -> int | None:
+    # (a plain address, which ctypes converts as it calls: a pointer object each cost 0.2 us of a call that takes 12)
     if t is None:
-        return C.c_void_p(0)
+        return None
     if not t.is_cuda:
         raise ValueError(f"{name} must be a CUDA tensor (this library has no CPU path)")
     if not t.is_contiguous():
         raise ValueError(f"{name} must be contiguous")
-    if dtype is not None and t.dtype != dtype:
+    if dtype is not None and t.dtype is not dtype:
         raise ValueError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    return C.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
-def _stream() -> C.c_void_p:
-    # the raw handle of torch.cuda.current_stream(), without building a Stream object for it (2 us of a 17 us call)
-    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+def _stream() -> int:
+    # the raw handle of torch.cuda.current_stream(), without building a Stream object for it (2 us of a 17 us call); the tensors of
+    # the call exist, so CUDA is initialised
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def make_config(d_out, d_in, d_block, *, n_keep=2, m_group=4, h_mode=H_FULL, select_mode=SELECT_L1_RANDOM,
@@ -230,10 +232,12 @@ def armor_pack_layer(ctx, A, B, S, M, r1, r2, packed) -> None:
 
 
 def armor_apply_layer(ctx, packed, x, y) -> None:
-    if x.dtype != torch.bfloat16 or y.dtype != torch.bfloat16:
+    bf16 = torch.bfloat16
+    if x.dtype is not bf16 or y.dtype is not bf16:
         raise ValueError("the packed layer takes bf16 x and y")
-    _check(lib().armor_apply_layer(ctx, _ptr(packed, torch.uint8, "packed"), _ptr(x, x.dtype, "x"), _ptr(y, y.dtype, "y"),
-                                   x.shape[0], _stream()), "armor_apply_layer")
+    code = lib().armor_apply_layer(ctx, _ptr(packed, torch.uint8, "packed"), _ptr(x, None, "x"), _ptr(y, None, "y"), x.shape[0], _stream())
+    if code:
+        _check(code, "armor_apply_layer")
 
 
 def armor_get_device_status(ctx, n: int = 16) -> list[int]:
