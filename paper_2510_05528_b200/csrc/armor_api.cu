@@ -210,14 +210,15 @@ void tile_grams(armor_ctx* c, const float* X, const float* Y, bool by_rows, floa
   g.M = db; g.N = db; g.K = db; g.batch = c->nbo * c->nbi; g.batch_inner = c->nbi; g.alpha = 1.f;
   launch_bgemm(c, g, s);
 }
-void block_mm(armor_ctx* c, const float* X, bool tX, const float* Y, bool tY, float* Z, int nb, cudaStream_t s) {
+void block_mm(armor_ctx* c, const float* X, bool tX, const float* Y, bool tY, float* Z, int nb, LaunchStream s) {
   const int db = c->db;
   BGemm g{};
   g.A = X; g.sAb = (int64_t)db * db; g.sAm = tX ? 1 : db; g.sAk = tX ? db : 1;
   g.B = Y; g.sBb = (int64_t)db * db; g.sBk = tY ? 1 : db; g.sBn = tY ? db : 1;
   g.C = Z; g.sCb = (int64_t)db * db; g.sCm = db; g.sCn = 1;
   g.M = db; g.N = db; g.K = db; g.batch = nb; g.alpha = 1.f;
-  launch_bgemm(c, g, s);
+  g.waits = s.waits ? 1 : 0;
+  launch_bgemm(c, g, s.s);
 }
 
 armor_status reset_adam(armor_ctx* c, cudaStream_t s) {
@@ -315,13 +316,17 @@ armor_status armor_create(armor_ctx** out, const armor_config* cfg, void* d_work
   c->cap_split = 0; c->cap_n = 0; c->cap_failed = 0;
   c->cap_stream = nullptr;
   if (cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking) != cudaSuccess) c->cap_stream = nullptr;
-  // a second stream of the context's own and five events: the Gram stages chunk p + 1 there while chunk p is contracted
+  // a second stream of the context's own and its events: the Gram stages chunk p + 1 there while chunk p is contracted, an
+  // iteration forms the group solves' systems there
   c->side_stream = nullptr;
   c->ev_fork = nullptr;
+  c->ev_prep = c->ev_prepared = nullptr;
   for (int k = 0; k < 2; ++k) { c->ev_staged[k] = nullptr; c->ev_used[k] = nullptr; }
   {
     bool ok = cudaStreamCreateWithFlags(&c->side_stream, cudaStreamNonBlocking) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&c->ev_prep, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&c->ev_prepared, cudaEventDisableTiming) == cudaSuccess;
     for (int k = 0; k < 2 && ok; ++k)
       ok = cudaEventCreateWithFlags(&c->ev_staged[k], cudaEventDisableTiming) == cudaSuccess &&
            cudaEventCreateWithFlags(&c->ev_used[k], cudaEventDisableTiming) == cudaSuccess;
@@ -348,6 +353,8 @@ armor_status armor_destroy(armor_ctx* c) {
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
   if (c->side_stream) cudaStreamDestroy(c->side_stream);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
+  if (c->ev_prep) cudaEventDestroy(c->ev_prep);
+  if (c->ev_prepared) cudaEventDestroy(c->ev_prepared);
   for (int k = 0; k < 2; ++k) {
     if (c->ev_staged[k]) cudaEventDestroy(c->ev_staged[k]);
     if (c->ev_used[k]) cudaEventDestroy(c->ev_used[k]);
@@ -492,6 +499,24 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
   armor_iter_stats* const is = d_stats;   // base of the records; the kernels add the device counter
   auto body = [&](bool first, bool fresh_loss, bool t_zero, cudaStream_t s) -> armor_status {
     armor_status st = ARMOR_OK;
+    // What the group solves need of A and B (B_j H_jj, alpha_r, the diagonal blocks of K_j): small products that leave most of
+    // the memory's rate unused, formed on the side stream while the update of the core runs (4096 x 4096: 17 us an iteration, behind
+    // one another in the stream).  Not while launches are timed or captured in pieces.
+    bool prepared = false;
+    const bool fork = (ph & ARMOR_PHASE_MASK) && c->side_stream && c->timing_on == 0;
+    auto prepare_solves = [&](LaunchStream q) {
+      block_mm(c, B, false, c->Hjj, false, c->Ktmp, nbi, q);                         // B_j H_jj
+      launch_mask_prep(c, A, B, c->Ktmp, q.s);               // alpha_r and the m x m diagonal blocks of K_j = B_j H_jj B_j^T
+    };
+    auto prepare_aside = [&]() -> armor_status {
+      if (!fork) return ARMOR_OK;
+      ARMOR_CUDA_OK(cudaEventRecord(c->ev_prep, s));
+      ARMOR_CUDA_OK(cudaStreamWaitEvent(c->side_stream, c->ev_prep, 0));
+      prepare_solves(LaunchStream(c->side_stream, true));
+      ARMOR_CUDA_OK(cudaEventRecord(c->ev_prepared, c->side_stream));
+      prepared = true;
+      return ARMOR_OK;
+    };
     launch_zero_scalars(c, !first, !fresh_loss, is, s);      // with a carried loss this also opens the iteration's record
     if (adam) {
       // Adam normalises every entry's move, so a gradient that is exactly zero (the kept entries of the core at
@@ -525,6 +550,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       core_gradient(c, A, B, s);                                                     // Gamma = A^T E H_w B^T
       launch_adam(c, A, c->GamA, c->mA, c->vA, na, nullptr, t_first + 1, s);      // step number: t_first + 1 + counter
       launch_adam(c, B, c->GamB, c->mB, c->vB, nbl, nullptr, t_first + 1, s);
+      if ((st = prepare_aside()) != ARMOR_OK) return st;
       launch_adam(c, S, c->Gam, c->mS, c->vS, c->wn, M, t_first + 1, s);
       // the new state: residual, E H_w and the loss afresh
       int n_loss = 0;
@@ -634,6 +660,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
         }
       }
       launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S, nrm_part, n_nrm, SC_NRM_S);
+      if ((st = prepare_aside()) != ARMOR_OK) return st;
       // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
       launch_axpy_multi(c, S, c->U, 1.f, c->wn, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, RH, 1.f, c->wn, SC_TAU_S, s,
                         late_P ? c->E : nullptr, SC_TAU_B);
@@ -643,8 +670,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
 
     // ---- sparse-core update (Algorithm 3), mask_sweeps times ------------------------------------
     if (ph & ARMOR_PHASE_MASK) {
-      block_mm(c, B, false, c->Hjj, false, c->Ktmp, nbi, s);                         // B_j H_jj
-      launch_mask_prep(c, A, B, c->Ktmp, s);               // alpha_r and the m x m diagonal blocks of K_j = B_j H_jj B_j^T
+      if (!prepared) prepare_solves(s);
       for (int sw = 0; sw < sweeps; ++sw) {
         if (sw > 0) {
           // E H_w for the state the previous run left
@@ -660,7 +686,9 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
           }
         }
         core_gradient(c, A, B, s);
-        launch_mask_select(c, A, B, c->Gam, S, M, (uint64_t)(t_first * sweeps + sw), (uint64_t)sweeps, s);   // counter (t_first + it) K + k
+        const bool join = prepared && sw == 0;
+        if (join) ARMOR_CUDA_OK(cudaStreamWaitEvent(s, c->ev_prepared, 0));
+        launch_mask_select(c, A, B, c->Gam, S, M, (uint64_t)(t_first * sweeps + sw), (uint64_t)sweeps, LaunchStream(s, join));   // counter (t_first + it) K + k
         launch_mask_quadratic(c, A, B, H, is, s);                                    // accepted or not
         launch_mask_commit(c, S, M, carry_P ? c->P : nullptr, is, s);                // if accepted: S, M and P += dS B H_w
       }

@@ -96,6 +96,7 @@ struct armor_ctx {
   float* Xt_hi2;        // second staging buffer (FP16X3): chunk p + 1 is staged on side_stream while chunk p is contracted
   cudaStream_t side_stream;
   cudaEvent_t ev_fork, ev_staged[2], ev_used[2];
+  cudaEvent_t ev_prep, ev_prepared;   // the group solves' systems are formed on side_stream beside the core's update
   int64_t gram_rows;  // rows of X staged per pass
   double* sc;         // [SC_COUNT]
   double* partials;   // [2][8 * npart] partial sums of the fused / streaming reductions
@@ -169,14 +170,19 @@ __device__ __forceinline__ void grid_begin() {
 // threads 6,561 us, 6,775 without a limit, 6,626 with no dependent launches; limits of 1, 148 and 1,100 CTAs: 256 x 256 layer 2,886,
 // 2,767 and 2,746 us).
 constexpr int64_t DEPENDENT_THREADS = 592 * 256;
+// A stream to launch on; waits: for another stream's event as well, so that what is launched starts behind everything it waits for.
+struct LaunchStream {
+  cudaStream_t s; bool waits;
+  LaunchStream(cudaStream_t s_, bool waits_ = false) : s(s_), waits(waits_) {}
+};
 template <typename... Params, typename... Args>
-inline void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+inline void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, LaunchStream s, Args&&... args) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s.s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = (int64_t)grid.x * grid.y * grid.z * block.x * block.y <= DEPENDENT_THREADS ? 1 : 0;
+  cfg.attrs = at; cfg.numAttrs = !s.waits && (int64_t)grid.x * grid.y * grid.z * block.x * block.y <= DEPENDENT_THREADS ? 1 : 0;
   cudaLaunchKernelEx(&cfg, kernel, Params(args)...);   // (an error is found by the call's cudaGetLastError)
 }
 
@@ -219,6 +225,7 @@ struct BGemm {
   // split of the contraction into ksplit equal chunks whose partial products are summed in a fixed order
   // (needs c->gpart; only without D)
   int ksplit;
+  int waits;             // see LaunchStream
 };
 void launch_bgemm(armor_ctx* c, const BGemm& g, cudaStream_t s);
 // number of chunks a long contraction is cut into so that batch * tiles * chunks fills the GPU about twice
@@ -444,7 +451,7 @@ void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s);
 void launch_mask_prep(armor_ctx* c, const float* A, const float* B, const float* Y, cudaStream_t s);
 // selection counter t = t_base + t_mul * (*c->it_dev); with one draw per block also the vectors of launch_mask_quadratic
 void launch_mask_select(armor_ctx* c, const float* A, const float* B, const float* Gam, const float* S, const uint8_t* M, uint64_t t_base,
-                        uint64_t t_mul, cudaStream_t s);
+                        uint64_t t_mul, LaunchStream s);
 // exact loss change of the iteration's group updates without a dense product: the per-block terms of tr(V H_w V^T), V = A dS B,
 // from the selection records, their sum and the decision (stage 4)
 void launch_mask_quadratic(armor_ctx* c, const float* A, const float* B, const float* H, armor_iter_stats* st, cudaStream_t s);

@@ -497,22 +497,23 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
   BGemm g = g_in;
   if (g.M <= 0 || g.N <= 0 || g.batch <= 0) return;
   if (g.ksplit > 1 && (g.D || !c->gpart || (int64_t)g.ksplit * g.batch * g.M * g.N > c->gpart_floats)) g.ksplit = 1;
+  const LaunchStream at(s, g.waits != 0);
   bool a_kfast = false, b_nfast = false;
   if (g.ksplit > 1 && !tile_kernel_ok(g, a_kfast, b_nfast)) g.ksplit = 1;
   if (tile_kernel_ok(g, a_kfast, b_nfast) && small_tiles_better(g)) {
     dim3 grid((g.N + SM_T - 1) / SM_T, (g.M + SM_T - 1) / SM_T, g.batch);
     if ((int64_t)grid.x * grid.y * grid.z >= (int64_t)MID_TILES * c->n_sm) {
-      if (a_kfast && b_nfast) launch_dependent(bgemm_mid_kernel<true, true>, grid, MID_NT, 0, s, g);
-      else if (a_kfast && !b_nfast) launch_dependent(bgemm_mid_kernel<true, false>, grid, MID_NT, 0, s, g);
-      else if (!a_kfast && b_nfast) launch_dependent(bgemm_mid_kernel<false, true>, grid, MID_NT, 0, s, g);
-      else launch_dependent(bgemm_mid_kernel<false, false>, grid, MID_NT, 0, s, g);
+      if (a_kfast && b_nfast) launch_dependent(bgemm_mid_kernel<true, true>, grid, MID_NT, 0, at, g);
+      else if (a_kfast && !b_nfast) launch_dependent(bgemm_mid_kernel<true, false>, grid, MID_NT, 0, at, g);
+      else if (!a_kfast && b_nfast) launch_dependent(bgemm_mid_kernel<false, true>, grid, MID_NT, 0, at, g);
+      else launch_dependent(bgemm_mid_kernel<false, false>, grid, MID_NT, 0, at, g);
       c->launches++;
       return;
     }
-    if (a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<true, true>, grid, NT, 0, s, g);
-    else if (a_kfast && !b_nfast) launch_dependent(bgemm_small_kernel<true, false>, grid, NT, 0, s, g);
-    else if (!a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<false, true>, grid, NT, 0, s, g);
-    else launch_dependent(bgemm_small_kernel<false, false>, grid, NT, 0, s, g);
+    if (a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<true, true>, grid, NT, 0, at, g);
+    else if (a_kfast && !b_nfast) launch_dependent(bgemm_small_kernel<true, false>, grid, NT, 0, at, g);
+    else if (!a_kfast && b_nfast) launch_dependent(bgemm_small_kernel<false, true>, grid, NT, 0, at, g);
+    else launch_dependent(bgemm_small_kernel<false, false>, grid, NT, 0, at, g);
     c->launches++;
     return;
   }
@@ -520,10 +521,10 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
     const int ks = g.ksplit > 1 ? g.ksplit : 1;
     dim3 grid((g.N + FN - 1) / FN, (g.M + FM - 1) / FM, g.batch * ks);
     const int64_t pstride = (int64_t)g.batch * g.M * g.N;
-    if (a_kfast && b_nfast) launch_dependent(bgemm_tile_kernel<true, true>, grid, NT, 0, s, g, c->gpart, pstride);
-    else if (a_kfast && !b_nfast) launch_dependent(bgemm_tile_kernel<true, false>, grid, NT, 0, s, g, c->gpart, pstride);
-    else if (!a_kfast && b_nfast) launch_dependent(bgemm_tile_kernel<false, true>, grid, NT, 0, s, g, c->gpart, pstride);
-    else launch_dependent(bgemm_tile_kernel<false, false>, grid, NT, 0, s, g, c->gpart, pstride);
+    if (a_kfast && b_nfast) launch_dependent(bgemm_tile_kernel<true, true>, grid, NT, 0, at, g, c->gpart, pstride);
+    else if (a_kfast && !b_nfast) launch_dependent(bgemm_tile_kernel<true, false>, grid, NT, 0, at, g, c->gpart, pstride);
+    else if (!a_kfast && b_nfast) launch_dependent(bgemm_tile_kernel<false, true>, grid, NT, 0, at, g, c->gpart, pstride);
+    else launch_dependent(bgemm_tile_kernel<false, false>, grid, NT, 0, at, g, c->gpart, pstride);
     c->launches++;
     if (ks > 1) {
       const int64_t n4 = pstride / 4;
@@ -535,7 +536,7 @@ void launch_bgemm(armor_ctx* c, const BGemm& g_in, cudaStream_t s) {
     return;
   }
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.batch);
-  launch_dependent(bgemm_kernel, grid, NT, 0, s, g);
+  launch_dependent(bgemm_kernel, grid, NT, 0, at, g);
   c->launches++;
 }
 

@@ -651,7 +651,7 @@ void launch_mask_prep(armor_ctx* c, const float* A, const float* B, const float*
 }
 
 void launch_mask_select(armor_ctx* c, const float* A, const float* B, const float* Gam, const float* S, const uint8_t* M, uint64_t t_base,
-                        uint64_t t_mul, cudaStream_t s) {
+                        uint64_t t_mul, LaunchStream at) {
   const int mg = c->cfg.m_group;
   const uint64_t n_groups = (uint64_t)(c->d_out * (c->d_in / mg));
   const VectorArgs vec{A, B, c->Zsel, c->Acol, c->nbo_pad};
@@ -665,16 +665,16 @@ void launch_mask_select(armor_ctx* c, const float* A, const float* B, const floa
       if (smem > 48 * 1024)                                                                                             \
         cudaFuncSetAttribute(mask_select_kernel<MGV, NKV, MULTIV, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
                              (int)smem);                                                                                \
-      launch_dependent(mask_select_kernel<MGV, NKV, MULTIV, 0>, c->nbo * c->nbi, NT, smem, s, ARMOR_SELECT_ARGS);       \
+      launch_dependent(mask_select_kernel<MGV, NKV, MULTIV, 0>, c->nbo * c->nbi, NT, smem, at, ARMOR_SELECT_ARGS);      \
     } else {                                                                                                            \
-      launch_dependent(mask_select_kernel<MGV, NKV, false, 1>, c->nbo * c->nbi, NT, 0, s, ARMOR_SELECT_ARGS);           \
-      launch_dependent(mask_select_kernel<MGV, NKV, false, 2>, c->nbo * c->nbi, MGV == 4 ? 32 : NT, 0, s,               \
+      launch_dependent(mask_select_kernel<MGV, NKV, false, 1>, c->nbo * c->nbi, NT, 0, at, ARMOR_SELECT_ARGS);          \
+      launch_dependent(mask_select_kernel<MGV, NKV, false, 2>, c->nbo * c->nbi, MGV == 4 ? 32 : NT, 0, at.s,            \
                        ARMOR_SELECT_ARGS);                                                                              \
       c->launches++;                                                                                                    \
     }                                                                                                                   \
   } while (0)
   const bool multi = c->kg > 1;
-  KTimer kt(c, ARMOR_KC_MASK_SELECT, 4.0 * (double)c->wn, s);   // one read of the core gradient
+  KTimer kt(c, ARMOR_KC_MASK_SELECT, 4.0 * (double)c->wn, at.s);   // one read of the core gradient
   if (mg == 8 && c->cfg.n_keep > 4) { if (multi) ARMOR_SELECT_LAUNCH(8, 6, true); else ARMOR_SELECT_LAUNCH(8, 6, false); }
   else if (mg == 8) { if (multi) ARMOR_SELECT_LAUNCH(8, 4, true); else ARMOR_SELECT_LAUNCH(8, 4, false); }
   else { if (multi) ARMOR_SELECT_LAUNCH(4, 4, true); else ARMOR_SELECT_LAUNCH(4, 4, false); }
