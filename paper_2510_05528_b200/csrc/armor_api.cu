@@ -585,6 +585,15 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       launch_stage(c, is, 1, nullptr, 0, s);
     }
 
+    // E H_w's moves by the two line searches are read by the core's gradients only (the next iteration forms it afresh): where the
+    // two-sided product makes them on its way, no update of E H_w reaches memory.
+    Moves eh{};
+    const bool late_EH = !adam && c->tc_blocks == 3 && tc_block2_ok(c, d_out, d_in);
+    auto move_EH = [&]() {                                                           // what has not been made, in memory after all
+      for (int k = 0; k < eh.n; ++k) launch_axpy_slot(c, c->EH, eh.v[k], c->wn, eh.slot[k], -1.f, s);
+      eh = Moves{};
+    };
+
     // ---- B-step: block-Newton directions, one exact step --------------------------------------
     if (!adam && (ph & ARMOR_PHASE_B)) {
       bd_left(c, A, false, S, c->U, d_out, d_in, 1.f, nullptr, 0.f, s);              // U = A S
@@ -611,7 +620,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       // direction in B: V = A R with R = S Delta; R H_w serves both V H_w = A (R H_w) and the carried P
       // (R H_w, V H_w = A (R H_w) and q = <V H_w, V>, summed by the stage; V itself is needed nowhere else)
       int nq = 0;
-      st = bd_direction(c, S, c->Delta, A, H, c->Tmp, c->E, c->V, c->VH, c->partials, &nq, s);
+      float* const VH = late_EH ? c->V : c->VH;                                      // (kept for the second gradient as well)
+      st = bd_direction(c, S, c->Delta, A, H, c->Tmp, c->E, late_EH ? c->VH : c->V, VH, c->partials, &nq, s);
       if (st != ARMOR_OK) return st;
       if (b_gd) launch_stage(c, is, 8, nullptr, 0, s, c->partials, nq, SC_Q_B);
       else if (late_A)
@@ -619,7 +629,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       else launch_stage(c, is, 2, c->partblk, DELTA_PARTS * nbi, s, c->partials, nq, SC_Q_B);
       // B += tau Delta, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch.  (With a core step P moves
       // there by both steps: nothing reads it in between.)
-      launch_axpy_multi(c, c->EH, c->VH, -1.f, c->wn, carry_P && !late_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
+      if (late_EH) eh.add(VH, SC_TAU_B);
+      launch_axpy_multi(c, late_EH ? nullptr : c->EH, VH, -1.f, c->wn, carry_P && !late_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
                         (int64_t)nbi * db * db, SC_TAU_B, s);
     } else if (!adam) {
       launch_stage(c, is, 2, nullptr, 0, s);
@@ -631,7 +642,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       int n_nrm = 0;
       // U = Gamma (.) M, |U|^2: the mask is applied where the gradient leaves tensor memory, or in a pass of its own
       if (!(c->tc_blocks == 3 && tc_block2_ok(c, d_out, d_in) &&
-            tc_done(c, tc_two_sided(c, A, true, c->EH, B, true, c->U, d_out, d_in, 1.f, s, M, nrm_part, &n_nrm)))) {
+            tc_done(c, tc_two_sided(c, A, true, c->EH, B, true, c->U, d_out, d_in, 1.f, s, M, nrm_part, &n_nrm, eh)))) {
+        move_EH();
         core_gradient(c, A, B, s);
         launch_masked_copy(c, c->Gam, M, c->U, nrm_part, s);
         n_nrm = ARMOR_DOT_BLOCKS;
@@ -641,7 +653,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       // R = Gamma_M B, R H_w, V H_w = A (R H_w) and q = <V H_w, V> with V = A Gamma_M B
       int nq = 0;
       const bool beta_step = (c->cfg.s_step == ARMOR_S_BETA);
-      st = bd_direction(c, c->U, B, A, H, c->Tmp, RH, c->V, c->VH, c->partials, &nq, s);
+      st = bd_direction(c, c->U, B, A, H, c->Tmp, RH, late_EH ? c->Gam : c->V, c->VH, c->partials, &nq, s);
       if (st != ARMOR_OK) return st;
       if (beta_step) {
         // the paper's step size (Eq. lrWprime): |A^T A|_F and |B H_w B^T|_F  (these dot products reuse the
@@ -662,7 +674,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S, nrm_part, n_nrm, SC_NRM_S);
       if ((st = prepare_aside()) != ARMOR_OK) return st;
       // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
-      launch_axpy_multi(c, S, c->U, 1.f, c->wn, c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, RH, 1.f, c->wn, SC_TAU_S, s,
+      if (late_EH) eh.add(c->VH, SC_TAU_S);
+      launch_axpy_multi(c, S, c->U, 1.f, c->wn, late_EH ? nullptr : c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, RH, 1.f, c->wn, SC_TAU_S, s,
                         late_P ? c->E : nullptr, SC_TAU_B);
     } else if (!adam) {
       launch_stage(c, is, 3, nullptr, 0, s);
@@ -685,7 +698,11 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
             bd_left(c, A, false, c->P, c->EH, d_out, d_in, -1.f, c->WH, 1.f, s);     // E H_w = W H_w - A P
           }
         }
-        core_gradient(c, A, B, s);
+        if (!(eh.n > 0 && tc_done(c, tc_two_sided(c, A, true, c->EH, B, true, c->Gam, d_out, d_in, 1.f, s, nullptr, nullptr, nullptr, eh)))) {
+          move_EH();
+          core_gradient(c, A, B, s);
+        }
+        eh = Moves{};                                                                // (another sweep starts from E H_w formed afresh)
         const bool join = prepared && sw == 0;
         if (join) ARMOR_CUDA_OK(cudaStreamWaitEvent(s, c->ev_prepared, 0));
         launch_mask_select(c, A, B, c->Gam, S, M, (uint64_t)(t_first * sweeps + sw), (uint64_t)sweeps, LaunchStream(s, join));   // counter (t_first + it) K + k

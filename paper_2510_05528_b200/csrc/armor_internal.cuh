@@ -277,9 +277,14 @@ armor_status tc_bd_left_dual(armor_ctx* c, const float* Ablk, bool transA, const
 
 // both wrappers in one launch (block2_tcgen05.cu); d_block = 128
 bool tc_block2_ok(const armor_ctx* c, int64_t rows, int64_t cols);
+// moves -sc[slot] v that an array still has to make, in this order (v: arrays of the library's own, of the array's shape)
+struct Moves {
+  int n; const float* v[2]; int slot[2];
+  void add(const float* x, int at) { v[n] = x; slot[n] = at; ++n; }
+};
 armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const float* X, const float* Rblk, bool transR,
                           float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s, const uint8_t* mask = nullptr,
-                          double* norm_part = nullptr, int* n_norm = nullptr);
+                          double* norm_part = nullptr, int* n_norm = nullptr, const Moves& moves = Moves{});
 
 // EH = E diag(colw) with E = add - Ablk in, partial sums of <E, EH> at part: one launch, E stays in the SMs
 armor_status tc_bd_left_residual(armor_ctx* c, const float* Ablk, const float* in, const float* add, const float* colw,

@@ -15,7 +15,9 @@
 //   warp 0       : TMA producer.  Per tile four chunks (32 along k) of Lop_i and X_ij (product 1) and four chunks (32
 //                  along l) of Rop_j (product 2)
 //   warp 1       : MMA issuer: product 1 into D1[t % 2]; product 2 (A from tensor memory) into D2
-//   warps 2-5    : low parts of the chunks in shared memory
+//   warps 2-5    : low parts of the chunks in shared memory; with MOVES the chunk of X first moves along one or two directions
+//                  (X + a1 V1 + a2 V2, a line search's update that nothing else reads: it never reaches memory).  The
+//                  directions' chunks land where the low parts will stand.
 //   warps 6-9    : epilogue of D2 (alpha, swizzled staging, TMA store)
 //   warps 10-13  : split of D1 in tensor memory
 // The products are software-pipelined: product 1 of tile t + 1 is issued BEFORE product 2 of tile t
@@ -51,6 +53,7 @@ struct P2Params {
   // not null: only the entries that the N:M mask keeps are written, the others as zeros, and norm_part takes 4 partial sums
   // per tile (one per epilogue warp, in the order of the work items) of their squares
   const uint8_t* mask; int m_group;      // one byte per m_group entries of a row
+  const double* sc; int slot1, slot2;    // MOVES: X + a1 V1 (+ a2 V2) in place of X, a = -sc[slot]
   double* norm_part;
 };
 
@@ -87,9 +90,20 @@ __device__ __forceinline__ uint64_t op_desc(uint32_t base, int mn) {
   return mn ? smem_desc_mn_sw128_32b(base, 4096, 512) : smem_desc_sw128(base, 16, 1024);
 }
 
+__device__ __forceinline__ float4 low4(const float4 v) {
+  return make_float4(v.x - __uint_as_float(__float_as_uint(v.x) & 0xffffe000u), v.y - __uint_as_float(__float_as_uint(v.y) & 0xffffe000u),
+                     v.z - __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), v.w - __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
+}
+// (a step of zero leaves x as it is, whatever v holds, as the update kernels do)
+__device__ __forceinline__ float4 moved(float a, const float4 v, const float4 x) {
+  return a == 0.f ? x : make_float4(fmaf(a, v.x, x.x), fmaf(a, v.y, x.y), fmaf(a, v.z, x.z), fmaf(a, v.w, x.w));
+}
+
+template <int MOVES>
 __global__ void __launch_bounds__(NTHREADS, 1)
 tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant__ CUtensorMap mapX,
-                 const __grid_constant__ CUtensorMap mapR, const __grid_constant__ CUtensorMap mapC, const P2Params p) {
+                 const __grid_constant__ CUtensorMap mapR, const __grid_constant__ CUtensorMap mapC,
+                 const __grid_constant__ CUtensorMap mapV1, const __grid_constant__ CUtensorMap mapV2, const P2Params p) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t bars[3 * STAGES + 5];
@@ -146,9 +160,11 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
           const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
           if (!second) {
             // product 1: Lop_i[:, 32 kc ..] and X_ij[32 kc .., :]
-            mbar_expect_tx(fb, 2 * OP_BYTES);
+            mbar_expect_tx(fb, (2 + MOVES) * OP_BYTES);
             load_block_chunk(dst, &mapL, p.l_mn, TILE * i, 0, kc, fb);
             load_block_chunk(dst + 2 * OP_BYTES, &mapX, 1, TILE * i, TILE * j, kc, fb);
+            if (MOVES > 0) load_block_chunk(dst + 3 * OP_BYTES, &mapV1, 1, TILE * i, TILE * j, kc, fb);
+            if (MOVES > 1) load_block_chunk(dst + OP_BYTES, &mapV2, 1, TILE * i, TILE * j, kc, fb);
           } else {
             // product 2: Rop_j[32 kc .., :]
             mbar_expect_tx(fb, OP_BYTES);
@@ -242,6 +258,7 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
   } else if (warp < 6) {
     // ------------------------------------------------------------ low parts of the chunks
     const int t = threadIdx.x - 64;   // 0..127
+    const float a1 = MOVES > 0 ? -(float)p.sc[p.slot1] : 0.f, a2 = MOVES > 1 ? -(float)p.sc[p.slot2] : 0.f;
     int stage = 0; uint32_t phase = 0;
     bool ok = true;
     for (int o = 0; o < 2 * n_local && ok; ++o) {
@@ -250,22 +267,36 @@ tc_block2_kernel(const __grid_constant__ CUtensorMap mapL, const __grid_constant
       for (int kc = 0; kc < 4; ++kc) {
         if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
         float4* base = reinterpret_cast<float4*>(smem + (size_t)stage * STAGE_BYTES);
+        constexpr int PER = OP_BYTES / 16 / 128, OP4 = OP_BYTES / 16;
+        if (MOVES > 0 && !second) {
+          // (the directions are read before the low parts take their place: the same cells of the same thread)
+#pragma unroll
+          for (int e0 = 0; e0 < PER; e0 += 4) {
+            float4 x[4], v1[4], v2[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int idx = t + (e0 + e) * 128;
+              x[e] = base[2 * OP4 + idx];
+              v1[e] = base[3 * OP4 + idx];
+              if (MOVES > 1) v2[e] = base[OP4 + idx];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int idx = t + (e0 + e) * 128;
+              x[e] = moved(a1, v1[e], x[e]);
+              if (MOVES > 1) x[e] = moved(a2, v2[e], x[e]);
+              base[2 * OP4 + idx] = x[e];
+              base[3 * OP4 + idx] = low4(x[e]);
+            }
+          }
+        }
 #pragma unroll
         for (int op = 0; op < 2; ++op) {
           if (op == 0 && second) continue;        // product 2 has no M-side chunk in shared memory
-          float4* hi = base + op * (2 * OP_BYTES / 16);
-          float4* lo = hi + OP_BYTES / 16;
+          if (op == 1 && MOVES > 0 && !second) continue;
+          float4* hi = base + op * 2 * OP4;
 #pragma unroll
-          for (int e = 0; e < OP_BYTES / 16 / 128; ++e) {
-            const int idx = t + e * 128;
-            const float4 v = hi[idx];
-            float4 h;
-            h.x = __uint_as_float(__float_as_uint(v.x) & 0xffffe000u);
-            h.y = __uint_as_float(__float_as_uint(v.y) & 0xffffe000u);
-            h.z = __uint_as_float(__float_as_uint(v.z) & 0xffffe000u);
-            h.w = __uint_as_float(__float_as_uint(v.w) & 0xffffe000u);
-            lo[idx] = make_float4(v.x - h.x, v.y - h.y, v.z - h.z, v.w - h.w);
-          }
+          for (int e = 0; e < PER; ++e) hi[OP4 + t + e * 128] = low4(hi[t + e * 128]);
         }
         // make the generic-proxy writes visible to the tensor-core (async proxy) reads
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -390,12 +421,29 @@ bool tc_block2_ok(const armor_ctx* c, int64_t rows, int64_t cols) {
          !c->block_one_pass;
 }
 
+namespace {
+template <int MOVES>
+armor_status launch(armor_ctx* c, const CUtensorMap& mL, const CUtensorMap& mX, const CUtensorMap& mR, const CUtensorMap& mC, const CUtensorMap& mV1,
+                    const CUtensorMap& mV2, const P2Params& p, cudaStream_t s) {
+  static PerDeviceOnce attr;
+  if (ensure_dynamic_smem(attr, c->device, tc_block2_kernel<MOVES>, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  const int n_items = p.nbi * p.nbj;
+  const int grid = n_items < c->n_sm ? n_items : c->n_sm;
+  // one W-shaped read, one more per direction, one W-shaped write
+  KTimer kt(c, ARMOR_KC_BLOCK_PRODUCT, (8.0 + 4.0 * MOVES) * (double)p.c_rows * (double)p.c_cols, s);
+  launch_dependent(tc_block2_kernel<MOVES>, grid, NTHREADS, SMEM_BYTES, s, mL, mX, mR, mC, mV1, mV2, p);
+  c->launches++;
+  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+}
+}  // namespace
+
 // out[i-th block row, j-th block column] = alpha * Lop_i * X_ij * Rop_j,  Lop_i = Lblk[i] or its transpose, Rop_j = Rblk[j]
 // or its transpose; X and out are [rows, cols] and must not overlap.  With mask only the kept entries of out are written (the
-// others as zeros), and *n_norm partial sums of their squares go to norm_part.
+// others as zeros), and *n_norm partial sums of their squares go to norm_part.  moves: X - sc[slot] v, one after the other, in
+// place of X.
 armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const float* X, const float* Rblk, bool transR,
                           float* out, int64_t rows, int64_t cols, float alpha, cudaStream_t s, const uint8_t* mask,
-                          double* norm_part, int* n_norm) {
+                          double* norm_part, int* n_norm, const Moves& moves) {
   if (!ptr_ok(Lblk) || !ptr_ok(X) || !ptr_ok(Rblk) || !ptr_ok(out)) return ARMOR_ERR_UNSUPPORTED;
   if (mask && !ptr_ok(mask)) return ARMOR_ERR_UNSUPPORTED;
   P2Params p{};
@@ -406,20 +454,18 @@ armor_status tc_two_sided(armor_ctx* c, const float* Lblk, bool transL, const fl
   p.alpha = alpha;
   p.status = c->status;
   p.mask = mask; p.m_group = c->cfg.m_group; p.norm_part = norm_part;
+  p.sc = c->sc; p.slot1 = moves.slot[0]; p.slot2 = moves.slot[1];
   if (n_norm) *n_norm = 4 * p.nbi * p.nbj;
-  CUtensorMap mL, mX, mR, mC;
+  CUtensorMap mL, mX, mR, mC, mV[2];
   int wide = 0;                                     // (rows of 128 and of whole tiles: always 1)
   if (p.l_mn ? !make_map_mn(&mL, Lblk, TILE, rows, TILE, &wide) : !make_map_2d(&mL, Lblk, TILE, rows, TILE, 32, TILE)) return ARMOR_ERR_CUDA;
   if (!make_map_mn(&mX, X, cols, rows, cols, &wide)) return ARMOR_ERR_CUDA;
   if (p.r_mn ? !make_map_mn(&mR, Rblk, TILE, cols, TILE, &wide) : !make_map_2d(&mR, Rblk, TILE, cols, TILE, 32, TILE)) return ARMOR_ERR_CUDA;
   if (!make_map_2d(&mC, out, cols, rows, cols, 32, 32)) return ARMOR_ERR_CUDA;
-  static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_block2_kernel, SMEM_BYTES) != ARMOR_OK) return ARMOR_ERR_CUDA;
-  const int n_items = p.nbi * p.nbj;
-  const int grid = n_items < c->n_sm ? n_items : c->n_sm;
-  // one W-shaped read, one W-shaped write
-  KTimer kt(c, ARMOR_KC_BLOCK_PRODUCT, 8.0 * (double)rows * (double)cols, s);
-  launch_dependent(tc_block2_kernel, grid, NTHREADS, SMEM_BYTES, s, mL, mX, mR, mC, p);
-  c->launches++;
-  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+  mV[0] = mV[1] = mX;
+  for (int k = 0; k < moves.n; ++k)
+    if (!make_map_mn(&mV[k], moves.v[k], cols, rows, cols, &wide)) return ARMOR_ERR_CUDA;
+  if (moves.n == 2) return launch<2>(c, mL, mX, mR, mC, mV[0], mV[1], p, s);
+  if (moves.n == 1) return launch<1>(c, mL, mX, mR, mC, mV[0], mV[1], p, s);
+  return launch<0>(c, mL, mX, mR, mC, mV[0], mV[1], p, s);
 }

@@ -811,7 +811,7 @@ void launch_axpy_slot(armor_ctx* c, float* y, const float* x, int64_t n, int slo
 }
 
 // y_k += sign_k * sc[slot] * x_k for up to three pairs of lengths n_k (a pair with y == nullptr is skipped); with x2_before the
-// third, which then exists, takes y2 += sc[slot_before] * x2_before first
+// third, which then exists beside at least one other, takes y2 += sc[slot_before] * x2_before first
 void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64_t n0, float* y1, const float* x1, float s1,
                        int64_t n1, float* y2, const float* x2, float s2, int64_t n2, int slot, cudaStream_t s,
                        const float* x2_before, int slot_before) {
@@ -827,7 +827,8 @@ void launch_axpy_multi(armor_ctx* c, float* y0, const float* x0, float s0, int64
   for (int j = k; j < 3; ++j) t[j] = t[0];
   KTimer kt(c, n4 >= (1 << 20) ? ARMOR_KC_AXPY : ARMOR_KC_SMALL, 12.0 * elems + (x2_before ? 4.0 * (double)n2 : 0.0), s);
   const float4* xb = reinterpret_cast<const float4*>(x2_before);
-  if (xb) launch_dependent(axpy_multi_slot_kernel<3, true>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
+  if (xb && k == 3) launch_dependent(axpy_multi_slot_kernel<3, true>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
+  else if (xb) launch_dependent(axpy_multi_slot_kernel<2, true>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
   else if (k == 3) launch_dependent(axpy_multi_slot_kernel<3, false>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
   else if (k == 2) launch_dependent(axpy_multi_slot_kernel<2, false>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
   else launch_dependent(axpy_multi_slot_kernel<1, false>, grid_for(n4), NT, 0, s, t[0], t[1], t[2], n4, c->sc, slot, xb, slot_before);
