@@ -10,10 +10,11 @@
 // Also here: the packing of the wrappers for this kernel (bf16, the normalisation's scales folded in, Section 3.2
 // last paragraph) and the layer forward built from this kernel and the sparse core product.
 //
-// Kernel: persistent, 320 threads: warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue (accumulator ->
-// bf16 -> shared-memory turn -> 128-byte row segments; warps 2-5 take the left 64 columns of the tile, warps 6-9
-// the right 64: with four warps the epilogue, not HBM, set the pace).  Five stages of 32 KiB, two accumulator
-// buffers.  Every wait is bounded.
+// Kernel: persistent, 320 threads: warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue (accumulator -> bf16 -> swizzled
+// staging box of 32 rows x 64 columns -> TMA store).  A CTA works through consecutive row tiles of ONE block, which stays in shared memory
+// (32 or 128 KiB), and takes all its columns in one instruction: X is read once.  (Tiles of 128 columns that fetched their block and
+// their X every time moved four bytes through L2 for each byte written: 28672 columns x 4,096 tokens 104 us, 8192 33 us, 0.66 of the copy
+// bandwidth; now 85 and 27.)  Two accumulators.  Every wait is bounded.
 #include <cuda_bf16.h>
 
 #include "tc_common.cuh"
@@ -22,19 +23,21 @@ namespace {
 
 using namespace tc;
 
-constexpr int BM = 128, BN = 128, BKE = 64;         // BKE bf16 = 128 bytes = one swizzle row
+constexpr int BM = 128, BKE = 64;                   // BKE bf16 = 128 bytes = one swizzle row
 constexpr int NTHREADS = 320;
-constexpr int STAGES = 5;
-constexpr uint32_t TMEM_COLS = 256;                 // two accumulator buffers of BN columns
-constexpr int A_BYTES = BM * BKE * 2;               // 16 KiB
-constexpr int B_BYTES = BN * BKE * 2;               // 16 KiB
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+constexpr int X_BYTES = BM * BKE * 2;               // 16 KiB: a stage
+constexpr int BOX_BYTES = 32 * 64 * 2;              // an epilogue warp's staging box
+template <int DB, int N> struct Geo {               // N: output columns of a tile, a block's or half of them
+  static constexpr int KT = DB / BKE;               // k tiles of a block
+  static constexpr int Q_BYTES = N * DB * 2;
+  static constexpr int STAGES = N == 256 ? 4 : 8;
+  static constexpr uint32_t COLS = 2 * N;           // two accumulators
+  static constexpr size_t SMEM = (size_t)Q_BYTES + (size_t)STAGES * X_BYTES + 8 * BOX_BYTES + 1024;
+};
 
 struct FParams {
-  __nv_bfloat16* out; int64_t ldo;   // [rows][ldo]
-  int64_t rows, d;                   // tokens, output width (= number of rows of the stacked blocks)
-  int db;
-  int m_tiles, n_tiles, k_tiles;     // k_tiles = db / 64
+  int64_t rows;                      // tokens
+  int m_tiles, n_groups;             // groups of N columns
   int32_t* status;
 };
 
@@ -48,12 +51,12 @@ __device__ __forceinline__ uint64_t smem_desc_k(uint32_t addr) {
   return d;
 }
 
-__device__ __forceinline__ uint32_t instr_desc_bf16() {
+__device__ __forceinline__ uint32_t instr_desc_bf16(int n) {
   uint32_t d = 0;
   d |= 1u << 4;                   // D format: F32
   d |= 1u << 7;                   // A format: BF16
   d |= 1u << 10;                  // B format: BF16
-  d |= (uint32_t)(BN >> 3) << 17;
+  d |= (uint32_t)(n >> 3) << 17;
   d |= (uint32_t)(BM >> 4) << 24;
   return d;
 }
@@ -63,57 +66,77 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
+template <int DB, int N>
 __global__ void __launch_bounds__(NTHREADS, 1)
-fwd_block_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapQ, const FParams p) {
+fwd_block_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapC,
+                 const FParams p) {
+  using G = Geo<DB, N>;
+  constexpr int STAGES = G::STAGES, KT = G::KT;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  __shared__ __align__(8) uint64_t bars[2 * STAGES + 4];
+  __shared__ __align__(8) uint64_t bars[2 * STAGES + 6];
   __shared__ uint32_t tmem_base_holder;
   __shared__ int abort_flag;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[STAGES]);
-  const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = smem_u32(&bars[2 * STAGES + 2]);
-  const int n_tiles_total = p.m_tiles * p.n_tiles;
+  const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = tfull0 + 16, qfull = tfull0 + 32, qfree = tfull0 + 40;
+  // the CTA's row tiles: contiguous over all groups, balanced to one tile
+  const int64_t n_items = (int64_t)p.n_groups * p.m_tiles;
+  const int i0 = (int)(n_items * blockIdx.x / gridDim.x), i1 = (int)(n_items * (blockIdx.x + 1) / gridDim.x);
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
     for (int s = 0; s < STAGES; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); }
     for (int s = 0; s < 2; ++s) { mbar_init(tfull0 + 8 * s, 1); mbar_init(tempty0 + 8 * s, 8); }
+    mbar_init(qfull, 1);
+    mbar_init(qfree, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base_holder)),
-                 "r"(TMEM_COLS)
+                 "r"(G::COLS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  grid_begin();                                     // (tensor memory is this CTA's before the next kernel's CTAs start)
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
+  uint8_t* const stage0 = smem + G::Q_BYTES;
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (lane == 0) {
       int stage = 0; uint32_t phase = 0; long long issued = 0;
+      int cur = -1;
+      uint32_t q_loads = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles_total && ok; tile += gridDim.x) {
-        const int mt = tile / p.n_tiles, nt = tile - mt * p.n_tiles;   // the column tile runs fastest
-        const int kx0 = (nt * BN / p.db) * p.db;                       // first column of X of the tile's block
-        for (int kt = 0; kt < p.k_tiles; ++kt) {
+      for (int item = i0; item < i1 && ok; ++item) {
+        const int b = item / p.m_tiles, mt = item - b * p.m_tiles;
+        if (b != cur) {
+          // the MMAs of the block before have read it
+          if (q_loads > 0 && !mbar_wait(qfree, (q_loads - 1) & 1u, abortp, p.status)) { ok = false; break; }
+          mbar_expect_tx(qfull, G::Q_BYTES);
+          for (int kt = 0; kt < KT; ++kt) tma_load_2d(smem_u32(smem) + kt * N * 128, &mapQ, kt * BKE, b * N, qfull);
+          ++q_loads;
+          cur = b;
+        }
+        for (int kt = 0; kt < KT; ++kt) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
           const uint32_t fb = full0 + 8 * stage;
-          mbar_expect_tx(fb, STAGE_BYTES);
-          const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          tma_load_2d(dst, &mapX, kx0 + kt * BKE, mt * BM, fb);
-          tma_load_2d(dst + A_BYTES, &mapQ, kt * BKE, nt * BN, fb);
+          mbar_expect_tx(fb, X_BYTES);
+          tma_load_2d(smem_u32(stage0 + (size_t)stage * X_BYTES), &mapX, b / (DB / N) * DB + kt * BKE, mt * BM, fb);
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
       }
       if (!ok) {
+        // leave no bulk copy in flight: wait (bounded) for the block and the stages armed most recently
+        const long long tq = clock64();
+        while (q_loads > 0 && !mbar_try(qfull, (q_loads - 1) & 1u) && clock64() - tq < 20000000ll) {}
         for (int back = 1; back <= STAGES && back <= issued; ++back) {
           int s = stage - back; uint32_t ph = phase;
           if (s < 0) { s += STAGES; ph ^= 1; }
@@ -125,78 +148,93 @@ fwd_block_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (lane == 0) {
-      const uint32_t idesc = instr_desc_bf16();
+      const uint32_t idesc = instr_desc_bf16(N);
+      const uint64_t dq0 = smem_desc_k(smem_u32(smem)), dx0 = smem_desc_k(smem_u32(stage0));
       int stage = 0; uint32_t phase = 0;
-      int local = 0;
+      int local = 0, cur = -1;
+      uint32_t q_waits = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < n_tiles_total && ok; tile += gridDim.x, ++local) {
+      for (int item = i0; item < i1 && ok; ++item, ++local) {
+        const int b = item / p.m_tiles;
+        if (b != cur) {
+          if (!mbar_wait(qfull, q_waits & 1u, abortp, p.status)) { ok = false; break; }
+          ++q_waits;
+          cur = b;
+        }
         const int as = local & 1;
         const uint32_t aphase = (uint32_t)(local >> 1) & 1u;
         if (!mbar_wait(tempty0 + 8 * as, aphase ^ 1, abortp, p.status)) { ok = false; break; }
         tc_fence_after();
-        const uint32_t tacc = tmem_base + (uint32_t)(as * BN);
-        for (int kt = 0; kt < p.k_tiles; ++kt) {
+        const uint32_t tacc = tmem_base + (uint32_t)(as * N);
+        for (int kt = 0; kt < KT; ++kt) {
           if (!mbar_wait(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          const uint32_t sb = sa + A_BYTES;
+          const uint64_t dx = dx0 + (uint64_t)(uint32_t)(stage * (X_BYTES >> 4)), dq = dq0 + (uint64_t)(uint32_t)(kt * (N * 128 >> 4));
 #pragma unroll
-          for (int k = 0; k < BKE / 16; ++k)
-            umma_bf16(tacc, smem_desc_k(sa + k * 32), smem_desc_k(sb + k * 32), idesc, (uint32_t)((kt > 0) | (k != 0)));
+          for (int k = 0; k < BKE / 16; ++k) umma_bf16(tacc, dx + 2 * k, dq + 2 * k, idesc, (uint32_t)((kt > 0) | (k != 0)));
           umma_commit(empty0 + 8 * stage);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
-        if (ok) umma_commit(tfull0 + 8 * as);
+        if (!ok) break;
+        umma_commit(tfull0 + 8 * as);
+        if (item + 1 < i1 && (item + 1) / p.m_tiles != b) umma_commit(qfree);
       }
     }
   } else {
     // ------------------------------------------------------------ epilogue warps
     const int q = warp & 3;                 // tensor-memory lane quarter this warp may read
-    const int half = (warp - 2) >> 2;       // which 64 columns of the tile
-    uint32_t* tilebuf = reinterpret_cast<uint32_t*>(smem + (size_t)STAGES * STAGE_BYTES) + (warp - 2) * (32 * 33);
+    const int half = (warp - 2) >> 2;       // which half of the tile's columns
+    uint8_t* const box = stage0 + (size_t)STAGES * X_BYTES + (size_t)(warp - 2) * BOX_BYTES;
+    const uint32_t box_u32 = smem_u32(box);
     int local = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < n_tiles_total && ok; tile += gridDim.x, ++local) {
-      const int mt = tile / p.n_tiles, nt = tile - mt * p.n_tiles;
+    for (int item = i0; item < i1 && ok; ++item, ++local) {
+      const int b = item / p.m_tiles, mt = item - b * p.m_tiles;
       const int as = local & 1;
       const uint32_t aphase = (uint32_t)(local >> 1) & 1u;
       if (!mbar_wait(tfull0 + 8 * as, aphase, abortp, p.status)) { ok = false; break; }
       tc_fence_after();
-      const int64_t row_base = (int64_t)mt * BM + q * 32;
-      {
-        const int ch = half;
-        // 64 columns of the lane's row -> 32 words of two bf16; the 32 x 32 words are turned through shared
-        // memory so that one store instruction writes 128 contiguous bytes of one row
+      const int64_t row0 = (int64_t)mt * BM + q * 32;
+#pragma unroll 1
+      for (int ch = 0; ch < N / 128; ++ch) {
+        // 64 columns of the lane's row as bf16: 16-byte unit c of the box's row sits at unit c ^ (row % 8)
+        const int col = half * (N / 2) + ch * 64;
         uint32_t r0[32], r1[32];
-        tmem_ld32(tmem_base + (uint32_t)(as * BN + ch * 64) + ((uint32_t)(q * 32) << 16), r0);
-        tmem_ld32(tmem_base + (uint32_t)(as * BN + ch * 64 + 32) + ((uint32_t)(q * 32) << 16), r1);
+        tmem_ld32(tmem_base + (uint32_t)(as * N + col) + ((uint32_t)(q * 32) << 16), r0);
+        tmem_ld32(tmem_base + (uint32_t)(as * N + col + 32) + ((uint32_t)(q * 32) << 16), r1);
+        if (ch == N / 128 - 1) {                   // all reads of the accumulator are done
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(tempty0 + 8 * as);
+        }
+        if (lane == 0) tma_store_wait_read();       // the previous store has read the box
+        __syncwarp();
 #pragma unroll
-        for (int w = 0; w < 16; ++w) {
-          tilebuf[lane * 33 + w] = pack_bf16(__uint_as_float(r0[2 * w]), __uint_as_float(r0[2 * w + 1]));
-          tilebuf[lane * 33 + 16 + w] = pack_bf16(__uint_as_float(r1[2 * w]), __uint_as_float(r1[2 * w + 1]));
-        }
-        __syncwarp();
-        const int64_t col = (int64_t)nt * BN + ch * 64 + 2 * lane;
-        if (col < p.d) {
-#pragma unroll 8
-          for (int rr = 0; rr < 32; ++rr) {
-            const int64_t grow = row_base + rr;
-            if (grow < p.rows)
-              *reinterpret_cast<uint32_t*>(p.out + grow * p.ldo + col) = tilebuf[rr * 33 + lane];
+        for (int u = 0; u < 4; ++u) {
+          uint32_t w0[4], w1[4];
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            w0[k] = pack_bf16(__uint_as_float(r0[8 * u + 2 * k]), __uint_as_float(r0[8 * u + 2 * k + 1]));
+            w1[k] = pack_bf16(__uint_as_float(r1[8 * u + 2 * k]), __uint_as_float(r1[8 * u + 2 * k + 1]));
           }
+          *reinterpret_cast<uint4*>(box + lane * 128 + ((u ^ (lane & 7)) << 4)) = make_uint4(w0[0], w0[1], w0[2], w0[3]);
+          *reinterpret_cast<uint4*>(box + lane * 128 + (((u + 4) ^ (lane & 7)) << 4)) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
         }
+        fence_proxy_async();
         __syncwarp();
+        if (lane == 0 && row0 < p.rows) {           // (rows past the end are clipped)
+          tma_store_2d(&mapC, b * N + col, (int)row0, box_u32);
+          tma_store_commit();
+        }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty0 + 8 * as);
     }
+    if (lane == 0) tma_store_wait_read();           // shared memory stays valid until the stores have read it
   }
   tc_fence_before();
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(TMEM_COLS) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(G::COLS) : "memory");
   }
 }
 
@@ -292,17 +330,33 @@ pack_blocks_kernel(const float* __restrict__ P, const float* __restrict__ rowsca
   }
 }
 
-bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld) {
+bool make_map_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows) {
   PFN_cuTensorMapEncodeTiled_v12000 enc = get_encode();
   if (!enc) return false;
   cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  cuuint32_t box[2] = {(cuuint32_t)BKE, 128};
+  cuuint32_t box[2] = {(cuuint32_t)BKE, (cuuint32_t)box_rows};
   cuuint32_t estr[2] = {1, 1};
   CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
+}
+
+template <int DB, int N>
+armor_status launch_block(armor_ctx* c, const void* X, const void* Q, void* out, int64_t rows, int64_t d, cudaStream_t s) {
+  CUtensorMap mX, mQ, mC;
+  if (!make_map_bf16(&mX, X, rows, d, d, BM) || !make_map_bf16(&mQ, Q, d, DB, DB, N) || !make_map_bf16(&mC, out, rows, d, d, 32)) return ARMOR_ERR_CUDA;
+  FParams p{};
+  p.rows = rows; p.m_tiles = (int)((rows + BM - 1) / BM); p.n_groups = (int)(d / N);
+  p.status = c->status;
+  static PerDeviceOnce attr;
+  if (ensure_dynamic_smem(attr, c->device, fwd_block_kernel<DB, N>, Geo<DB, N>::SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  const int64_t tiles = (int64_t)p.m_tiles * p.n_groups;
+  KTimer kt(c, ARMOR_KC_FORWARD, 4.0 * (double)rows * (double)d, s);
+  launch_dependent(fwd_block_kernel<DB, N>, (unsigned)(tiles < c->n_sm ? tiles : c->n_sm), NTHREADS, Geo<DB, N>::SMEM, s, mX, mQ, mC, p);
+  c->launches++;
+  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
 
 }  // namespace
@@ -323,24 +377,12 @@ void launch_pack_blocks(armor_ctx* c, const float* P, const float* rowscale, con
 // out[t][n] = sum_k X[t][j*db + k] Q[n][k], j = n / db
 armor_status launch_fwd_block(armor_ctx* c, const void* X, const void* Q, void* out, int64_t rows, int64_t d,
                               cudaStream_t s) {
-  if (!fwd_block_ok(c) || rows <= 0 || d % 128) return ARMOR_ERR_UNSUPPORTED;
-  CUtensorMap mX, mQ;
-  if (!make_map_bf16(&mX, X, rows, d, d)) return ARMOR_ERR_CUDA;
-  if (!make_map_bf16(&mQ, Q, d, c->db, c->db)) return ARMOR_ERR_CUDA;
-  FParams p{};
-  p.out = static_cast<__nv_bfloat16*>(out); p.ldo = d; p.rows = rows; p.d = d; p.db = c->db;
-  p.m_tiles = (int)((rows + BM - 1) / BM); p.n_tiles = (int)(d / BN); p.k_tiles = c->db / BKE;
-  p.status = c->status;
-  constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 + 8 * 32 * 33 * sizeof(uint32_t);
-  static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, fwd_block_kernel, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
-  const int n_sm = c->n_sm;
-  const int64_t tiles = (int64_t)p.m_tiles * p.n_tiles;
-  const int grid = tiles < n_sm ? (int)tiles : n_sm;
-  KTimer kt(c, ARMOR_KC_FORWARD, 4.0 * (double)rows * (double)d, s);
-  fwd_block_kernel<<<grid, NTHREADS, SMEM, s>>>(mX, mQ, p);
-  c->launches++;
-  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+  if (!fwd_block_ok(c) || rows <= 0 || d % c->db) return ARMOR_ERR_UNSUPPORTED;
+  if (c->db == 128) return launch_block<128, 128>(c, X, Q, out, rows, d, s);
+  // a block of 256 in halves while an SM has no more than one: 4096 columns x 400 tokens 28.1 us a forward in halves, 30.4 whole;
+  // x 640 31.8 and 30.9; x 1,000 34.3 and 31.9
+  return 2 * ((rows + BM - 1) / BM) * (d / 256) <= c->n_sm ? launch_block<256, 128>(c, X, Q, out, rows, d, s)
+                                                          : launch_block<256, 256>(c, X, Q, out, rows, d, s);
 }
 
 // The same for up to ARMOR_SMALL_TOKENS rows.  pieces == 0: X is bf16 [rows][d]; otherwise X holds that many fp32 arrays

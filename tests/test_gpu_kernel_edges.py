@@ -91,6 +91,42 @@ def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
     assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
 
 
+@pytest.mark.parametrize("d_out,d_in,d_block,tokens", [
+    (128, 128, 128, (129, 160, 256, 1023)),        # one block, whole and ragged boxes of 32 rows
+    (384, 640, 128, (300,)),                       # a row tile a CTA
+    (19072, 256, 128, (129, 145)),                 # CTAs that go from one block to the next
+    (512, 256, 256, (129, 200)),                   # blocks of 256 in halves
+    (4096, 2304, 256, (129, 513, 1300)),           # on either side of that rule's line; whole blocks over several tiles
+])
+def test_wrapper_products_of_the_packed_forward(d_out, d_in, d_block, tokens):
+    """The products on either side of the core beyond the few-token kernels.  Integer operands: every fp32 sum is exact,
+    so the bf16 outputs are the oracle's; rows past the last one are not written."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + 3 * d_in)
+    ctx = _ctx(d_out, d_in, d_block)
+
+    def ints(lo, hi, *shape):
+        return torch.randint(lo, hi + 1, shape, device=DEV, generator=g).float()
+    S = ints(-1, 1, d_out, d_in)
+    grp = S.view(d_out, d_in // 4, 4)
+    keep = torch.zeros_like(grp, dtype=torch.bool).scatter_(2, torch.rand(grp.shape, device=DEV, generator=g).topk(2, 2).indices, True)
+    grp.mul_(keep)
+    M = (keep * torch.tensor([1, 2, 4, 8], device=DEV)).sum(2).to(torch.uint8)
+    st = Bd.LayerState(Wbar=S, A=ints(-1, 1, d_out // d_block, d_block, d_block), B=ints(-1, 1, d_in // d_block, d_block, d_block),
+                       S=S, M=M)
+    packed = ctx.pack_layer(st)
+    for n in tokens:
+        x = ints(-1, 1, n, d_in).to(torch.bfloat16)
+        z1 = torch.einsum("tjk,jmk->tjm", x.double().view(n, -1, d_block), st.B.double()).reshape(n, d_in).to(torch.bfloat16)
+        z2 = (z1.double() @ S.double().t()).to(torch.bfloat16)
+        y = torch.einsum("tjk,jmk->tjm", z2.double().view(n, -1, d_block), st.A.double()).reshape(n, d_out).float().to(torch.bfloat16)
+        out = torch.full((n + 40, d_out), 7.0, dtype=torch.bfloat16, device=DEV)
+        Bd.armor_apply_layer(ctx.ctx, packed, x, out[:n])
+        assert torch.equal(out[:n], y), n
+        assert (out[n:] == 7.0).all(), n
+    assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
+
+
 @pytest.mark.parametrize("d_out,d_in,d_block", [(32, 64, 32), (96, 256, 32), (256, 256, 32), (320, 128, 64), (120, 200, 8),
                                                 (48, 144, 16), (1024, 512, 64), (160, 96, 32)])
 @pytest.mark.parametrize("side", [0, 1])
