@@ -92,7 +92,8 @@ def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
 
 
 @pytest.mark.parametrize("d_out,d_in,d_block,tokens", [
-    (128, 128, 128, (129, 160, 256, 1023)),        # one block, whole and ragged boxes of 32 rows
+    (128, 128, 128, (129, 160, 1024, 1025, 2200)), # one block, whole and ragged boxes of 32 rows; chunks of 1,024 tokens
+    (128, 384, 128, (1024, 1027)), (384, 128, 128, (1024, 1027)),   # a chunk's z1 and z2 fill their scratch
     (384, 640, 128, (300,)),                       # a row tile a CTA
     (19072, 256, 128, (129, 145)),                 # CTAs that go from one block to the next
     (512, 256, 256, (129, 200)),                   # blocks of 256 in halves
