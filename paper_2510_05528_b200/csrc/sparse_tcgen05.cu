@@ -931,13 +931,25 @@ armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E,
   p.Z = Zp; p.ldz = c->d_out; p.M = c->d_out; p.N = n; p.K = c->d_in;
   p.m_tiles = (int)(c->d_out / BM); p.n_tiles = 1; p.k_tiles = (int)(c->d_in / BKL);
   p.status = c->status;
+  // Pieces of a row tile.  Two CTAs an SM keep most of S in flight, which a large core needs (14336 x 4096, 37 tokens: 224 CTAs
+  // 15.2 us a forward, 112 18.2; 8192 x 8192 256 19.4, 128 25).  A small one is bound by latency, 0.3 us a k tile and 0.1 us a
+  // piece to be written and added: one CTA an SM, one SM in twelve with two, while that leaves a CTA about eight k tiles (4096 x
+  // 4096, 256 -> 160 CTAs: 1 token 8.98 -> 8.2 us, 64 10.9 -> 9.3; 2048 x 2048, 256 -> 128: 7.7 -> 6.5 and 10.4 -> 7.8; beyond 64
+  // tokens, two stages a CTA: five k tiles), and no fewer k tiles than make those two costs alike (512 x 8192, 64 -> 13 pieces:
+  // 14.3 -> 8.2 us).
   int want = 2 * c->n_sm / p.m_tiles;
+  const int one_an_sm = (c->n_sm + c->n_sm / 12) / p.m_tiles;
+  const bool small = one_an_sm >= 2 && (int64_t)p.m_tiles * p.k_tiles <= (int64_t)(n <= 64 ? 8 : 5) * c->n_sm;
+  if (small) want = one_an_sm;
   if (want < 1) want = 1;
   if (want > p.k_tiles) want = p.k_tiles;
-  const int per = (p.k_tiles + want - 1) / want;
+  int per = (p.k_tiles + want - 1) / want;
+  while (3 * per * per < p.k_tiles) ++per;
   *pieces = (p.k_tiles + per - 1) / per;
   if (n <= 16) return launch_small<16>(c, Sc, E, z1_bf16, p, *pieces, per, s);
-  if (n <= 32) return launch_small<32>(c, Sc, E, z1_bf16, p, *pieces, per, s);
+  // (a small core's tile of 32 tokens takes longer than one of 64, 4096 x 4096, 24 tokens 9.4 and 8.9 us; not for its stages nor its
+  // place in tensor memory, and the reverse for a large one, 14336 x 4096 13.8 and 14.3)
+  if (n <= 32 && !small) return launch_small<32>(c, Sc, E, z1_bf16, p, *pieces, per, s);
   if (n <= 64) return launch_small<64>(c, Sc, E, z1_bf16, p, *pieces, per, s);
   return launch_small<128>(c, Sc, E, z1_bf16, p, *pieces, per, s);
 }

@@ -61,7 +61,8 @@ def test_dense_product_with_h_at_tile_edges(d_out, d_in, precision):
 
 
 @pytest.mark.parametrize("d_out,d_in,d_block", [(128, 128, 128), (384, 512, 128), (512, 256, 256), (4096, 1152, 128),
-                                                (19072, 2048, 128)])
+                                                (19072, 2048, 128),
+                                                (256, 3200, 128), (2560, 5120, 128)])   # ragged pieces; one CTA an SM up to 64 tokens
 def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
     """The packed layer at every token tile of the split product (16, 32, 64, 128) and beside its edges, against the rows
     of a batch that takes the persistent kernels.  Integer operands: every fp32 sum is exact in any order, so the
