@@ -172,17 +172,24 @@ __device__ __forceinline__ void grid_begin() {
 constexpr int64_t DEPENDENT_THREADS = 592 * 256;
 // A stream to launch on; waits: for another stream's event as well, so that what is launched starts behind everything it waits for.
 struct LaunchStream {
-  cudaStream_t s; bool waits;
-  LaunchStream(cudaStream_t s_, bool waits_ = false) : s(s_), waits(waits_) {}
+  cudaStream_t s; bool waits; int cluster;            // cluster: CTAs of one along x
+  LaunchStream(cudaStream_t s_, bool waits_ = false, int cluster_ = 1) : s(s_), waits(waits_), cluster(cluster_) {}
 };
 template <typename... Params, typename... Args>
 inline void launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, LaunchStream s, Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s.s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at; cfg.numAttrs = !s.waits && (int64_t)grid.x * grid.y * grid.z * block.x * block.y <= DEPENDENT_THREADS ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (!s.waits && (int64_t)grid.x * grid.y * grid.z * block.x * block.y <= DEPENDENT_THREADS) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (s.cluster > 1) {
+    at[n].id = cudaLaunchAttributeClusterDimension;
+    at[n].val.clusterDim.x = (unsigned)s.cluster; at[n].val.clusterDim.y = 1; at[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = at; cfg.numAttrs = n;
   cudaLaunchKernelEx(&cfg, kernel, Params(args)...);   // (an error is found by the call's cudaGetLastError)
 }
 
