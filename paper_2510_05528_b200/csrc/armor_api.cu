@@ -263,6 +263,17 @@ armor_status residual_and_loss(armor_ctx* c, const float* W, const float* H, con
 
 }  // namespace
 
+// Whether the few-token kernels of the packed forward are the faster ones.  The persistent core product has a pair of SMs for every 256
+// rows x 256 tokens and no split of the contraction; where its tiles leave most of the chip idle, row tiles x token tiles of 128 of the
+// few-token kernel with the contraction cut between CTAs win, until its pieces and the small products that add them cost more:
+// 1024 x 1024, 256 tokens 8.3 and 15.4 us, 1,500 (96 tiles) 16.1 and 16.2, 2,048 (128) 17.6 and 16.7; 4096 x 4096, 129 15.6 and 23.7,
+// 384 (96) 21.4 and 24.5, 512 (128) 24.9 and 25.0; 1024 x 14336, 1,024 (64) 43 and 61; blocks of 256, which those products read
+// more often: 1024 x 1024, 1,024 (64) 17.1 and 17.3, 1,500 (96) 21.8 and 17.7.  The other two terms are what the scratch holds.
+static bool fwd_is_small(const armor_ctx* c, int64_t n) {
+  if (n <= ARMOR_SMALL_TOKENS) return true;
+  return n <= 2048 && n <= 5 * c->d_in && n <= 8 * c->d_out && (n + 127) / 128 * (c->d_out / 128) <= (c->db == 128 ? 96 : 64);
+}
+
 extern "C" {
 
 const char* armor_status_string(armor_status st) {
@@ -926,11 +937,15 @@ armor_status armor_apply_layer(armor_ctx* c, const void* d_packed, const void* d
   cudaStream_t s = cs(stream);
   const char* buf = static_cast<const char*>(d_packed);
   const int64_t d_out = c->d_out, d_in = c->d_in;
-  if (n_tokens <= ARMOR_SMALL_TOKENS) {
+  if (fwd_is_small(c, n_tokens)) {
+    // z1 = (r1 . x) B^T, bf16 in T; from about 2,000 columns x 600 tokens on by the persistent kernel (blocks of 256: half of that):
+    // 1024 x 5120, 200 tokens 13.8 us a forward and 13.9, 1,024 29.2 and 22.6; 512 x 512, 256 6.9 and 8.5
     int pieces = 0;
-    armor_status st = launch_fwd_small(c, d_x, 0, buf + layer_off_B(c), c->T, n_tokens, d_in, s);               // z1 = (r1 . x) B^T
-    if (st == ARMOR_OK) st = launch_tc_sparse_small(c, buf, buf + tc_sparse_values_bytes(c), c->T, c->E, n_tokens, &pieces, s);
-    if (st == ARMOR_OK) st = launch_fwd_small(c, c->E, pieces, buf + layer_off_A(c), d_y, n_tokens, d_out, s);  // y = r2 . (z2 A^T)
+    armor_status st = n_tokens * d_in * c->db > (int64_t)9 << 24 ? launch_fwd_block(c, d_x, buf + layer_off_B(c), c->T, n_tokens, d_in, s)
+                                                                 : launch_fwd_small(c, d_x, 0, buf + layer_off_B(c), c->T, n_tokens, d_in, s);
+    // z2 = z1 S^T as fp32 pieces in the five W-shaped buffers from V
+    if (st == ARMOR_OK) st = launch_tc_sparse_small(c, buf, buf + tc_sparse_values_bytes(c), c->T, c->V, n_tokens, &pieces, s);
+    if (st == ARMOR_OK) st = launch_fwd_small(c, c->V, pieces, buf + layer_off_A(c), d_y, n_tokens, d_out, s);  // y = r2 . (z2 A^T)
     return st == ARMOR_OK ? finish_call(c) : st;
   }
   // A chunk's three launches cost 17 us however few its tokens: the chunk is what the scratch holds.  bf16 z1 [chunk, d_in] in

@@ -507,8 +507,8 @@ void launch_pack_blocks(armor_ctx* c, const float* P, const float* rowscale, con
                         cudaStream_t s);
 armor_status launch_fwd_block(armor_ctx* c, const void* X, const void* Q, void* out, int64_t rows, int64_t d,
                               cudaStream_t s);
-// Few tokens (decoding): up to this many the three products of the bf16 forward run as latency-bound kernels whose
-// contraction over d_in is split over the chip; beyond it the tiles of the persistent kernels fill it themselves.
+// Few tokens (decoding): up to this many, and beyond while the layer is small (fwd_is_small), the three products of the bf16 forward
+// run as latency-bound kernels whose contraction over d_in is split over the chip; the tiles of the persistent kernels fill it themselves.
 static const int64_t ARMOR_SMALL_TOKENS = 128;
 armor_status launch_fwd_small(armor_ctx* c, const void* X, int pieces, const void* Q, void* out, int64_t rows, int64_t d,
                               cudaStream_t s);

@@ -385,11 +385,11 @@ armor_status launch_fwd_block(armor_ctx* c, const void* X, const void* Q, void* 
                                                           : launch_block<256, 256>(c, X, Q, out, rows, d, s);
 }
 
-// The same for up to ARMOR_SMALL_TOKENS rows.  pieces == 0: X is bf16 [rows][d]; otherwise X holds that many fp32 arrays
+// The same for few rows.  pieces == 0: X is bf16 [rows][d]; otherwise X holds that many fp32 arrays
 // [rows][d] whose sum, rounded to bf16, is the operand.  Either way a dependent launch.
 armor_status launch_fwd_small(armor_ctx* c, const void* X, int pieces, const void* Q, void* out, int64_t rows, int64_t d,
                               cudaStream_t s) {
-  if (!fwd_block_ok(c) || rows <= 0 || rows > ARMOR_SMALL_TOKENS || d % 128) return ARMOR_ERR_UNSUPPORTED;
+  if (!fwd_block_ok(c) || rows <= 0 || d % 128) return ARMOR_ERR_UNSUPPORTED;
   KTimer kt(c, ARMOR_KC_FORWARD, 4.0 * (double)rows * (double)d, s);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(d / 128), (unsigned)((rows + 15) / 16)); cfg.blockDim = dim3(256); cfg.stream = s;

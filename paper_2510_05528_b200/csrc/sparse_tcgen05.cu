@@ -431,7 +431,7 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
 }
 
 // ---------------------------------------------------------------------------------------------------------
-// The same product for few tokens (up to 128, one tile of BNS tokens), where reading S is the whole cost and the tiles
+// The same product for few tokens (a tile of BNS, or some of 128), where reading S is the whole cost and the tiles
 // above leave most of the chip idle (one 256 x 256 tile per pair: 32 of 148 SMs at 4096 x 4096, 21 us).  The contraction
 // is cut into pieces so that (row tiles) x (pieces) fills two CTAs per SM; a CTA keeps up to 72 KiB of S in flight, sums
 // its piece in tensor memory and writes it as fp32, and the kernel that multiplies with A adds the pieces in a fixed
@@ -461,6 +461,7 @@ tc_sparse_small_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[T::STAGES]), tfull = smem_u32(&bars[2 * T::STAGES]);
   const int mt = blockIdx.x;
   const int k0 = blockIdx.y * k_per_piece, k1 = min(p.k_tiles, k0 + k_per_piece);
+  const int tok0 = BNS == 128 ? blockIdx.z * BNS : 0;                 // (only a tile of 128 has others beside it)
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -491,8 +492,8 @@ tc_sparse_small_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
       };
       auto load_z = [&](int kt, int stage) {
         const uint32_t dst = smem_u32(smem + (size_t)stage * T::STAGE) + A_BYTES, fb = full0 + 8 * stage;
-        tma_load_2d(dst, &mapB, kt * BKL, 0, fb);
-        tma_load_2d(dst + T::BH, &mapB, kt * BKL + 64, 0, fb);
+        tma_load_2d(dst, &mapB, kt * BKL, tok0, fb);
+        tma_load_2d(dst + T::BH, &mapB, kt * BKL + 64, tok0, fb);
       };
       const int pre = min(T::STAGES, k1 - k0);
       for (int i = 0; i < pre; ++i) load_s(k0 + i, i);
@@ -545,14 +546,14 @@ tc_sparse_small_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
     if (mbar_wait(tfull, 0, abortp, p.status)) {
       tc_fence_after();
       const int64_t row = (int64_t)mt * BM + q * 32 + lane;
-      float* Z = p.Z + (int64_t)blockIdx.y * p.N * p.ldz + row;          // this piece's sums, [tokens][d_out]
+      float* Z = p.Z + ((int64_t)blockIdx.y * p.N + tok0) * p.ldz + row;          // this piece's sums, [tokens][d_out]
 #pragma unroll 1
       for (int ch = 0; ch < BNS / 16; ++ch) {
         uint32_t r[16];
         tmem_ld16(tmem_base + (uint32_t)(ch * 16) + ((uint32_t)(q * 32) << 16), r);
 #pragma unroll
         for (int i = 0; i < 16; ++i)
-          if (ch * 16 + i < p.N) Z[(int64_t)(ch * 16 + i) * p.ldz] = __uint_as_float(r[i]);
+          if (tok0 + ch * 16 + i < p.N) Z[(int64_t)(ch * 16 + i) * p.ldz] = __uint_as_float(r[i]);
       }
     }
   }
@@ -837,7 +838,7 @@ armor_status launch_small(armor_ctx* c, const void* Sc, const void* E, const voi
   if (ensure_dynamic_smem(attr, c->device, tc_sparse_small_kernel<BNS>, SmallN<BNS>::SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
   KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)p.M * (double)p.N * (double)p.K, s);   // dense-equivalent flops
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)p.m_tiles, (unsigned)pieces); cfg.blockDim = dim3(NTHREADS);
+  cfg.gridDim = dim3((unsigned)p.m_tiles, (unsigned)pieces, (unsigned)p.n_tiles); cfg.blockDim = dim3(NTHREADS);
   cfg.dynamicSmemBytes = SmallN<BNS>::SMEM; cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -918,27 +919,28 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
 
-// Zp[piece][n][d_out] = the pieces of Z1[n][d_in] * S^T (bf16 operands, fp32 sums) for n <= ARMOR_SMALL_TOKENS tokens;
-// their number goes to *pieces.  pieces * n <= d_in, so Zp fits a W-shaped fp32 buffer.
+// Zp[piece][n][d_out] = the pieces of Z1[n][d_in] * S^T (bf16 operands, fp32 sums), beyond 64 tokens in tiles of 128; their number
+// goes to *pieces.  pieces * n <= 5 d_in, so Zp fits five W-shaped fp32 buffers.
 armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E, const void* z1_bf16, float* Zp, int64_t n,
                                     int* pieces, cudaStream_t s) {
-  if (!tc_sparse_ok(c) || n <= 0 || n > ARMOR_SMALL_TOKENS) return ARMOR_ERR_UNSUPPORTED;
+  if (!tc_sparse_ok(c) || n <= 0 || n > 5 * c->d_in) return ARMOR_ERR_UNSUPPORTED;
   SParams p{};
   p.Z = Zp; p.ldz = c->d_out; p.M = c->d_out; p.N = n; p.K = c->d_in;
-  p.m_tiles = (int)(c->d_out / BM); p.n_tiles = 1; p.k_tiles = (int)(c->d_in / BKL);
+  p.m_tiles = (int)(c->d_out / BM); p.n_tiles = (int)((n + 127) / 128); p.k_tiles = (int)(c->d_in / BKL);
   p.status = c->status;
-  // Pieces of a row tile.  Two CTAs an SM keep most of S in flight, which a large core needs (14336 x 4096, 37 tokens: 224 CTAs
+  // Pieces of a row (and token) tile.  Two CTAs an SM keep most of S in flight, which a large core needs (14336 x 4096, 37 tokens: 224 CTAs
   // 15.2 us a forward, 112 18.2; 8192 x 8192 256 19.4, 128 25).  A small one is bound by latency, 0.3 us a k tile and 0.1 us a
   // piece to be written and added: one CTA an SM, one SM in twelve with two, while that leaves a CTA about eight k tiles (4096 x
   // 4096, 256 -> 160 CTAs: 1 token 8.98 -> 8.2 us, 64 10.9 -> 9.3; 2048 x 2048, 256 -> 128: 7.7 -> 6.5 and 10.4 -> 7.8; beyond 64
   // tokens, two stages a CTA: five k tiles), and no fewer k tiles than make those two costs alike (512 x 8192, 64 -> 13 pieces:
   // 14.3 -> 8.2 us).
-  int want = 2 * c->n_sm / p.m_tiles;
-  const int one_an_sm = (c->n_sm + c->n_sm / 12) / p.m_tiles;
-  const bool small = one_an_sm >= 2 && (int64_t)p.m_tiles * p.k_tiles <= (int64_t)(n <= 64 ? 8 : 5) * c->n_sm;
+  int want = 2 * c->n_sm / (p.m_tiles * p.n_tiles);
+  const int one_an_sm = (c->n_sm + c->n_sm / 12) / (p.m_tiles * p.n_tiles);
+  const bool small = one_an_sm >= 2 && (int64_t)p.m_tiles * p.n_tiles * p.k_tiles <= (int64_t)(n <= 64 ? 8 : 5) * c->n_sm;
   if (small) want = one_an_sm;
   if (want < 1) want = 1;
   if (want > p.k_tiles) want = p.k_tiles;
+  if (want > 5 * p.K / n) want = (int)(5 * p.K / n);                 // what Zp holds
   int per = (p.k_tiles + want - 1) / want;
   while (3 * per * per < p.k_tiles) ++per;
   *pieces = (p.k_tiles + per - 1) / per;

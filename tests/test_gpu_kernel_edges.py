@@ -93,12 +93,14 @@ def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
 
 
 @pytest.mark.parametrize("d_out,d_in,d_block,tokens", [
-    (128, 128, 128, (129, 160, 1024, 1025, 2200)), # one block, whole and ragged boxes of 32 rows; chunks of 1,024 tokens
+    (128, 128, 128, (129, 640, 641, 1024, 1025, 2200)),             # few-token kernels up to 640; whole and ragged boxes of 32 rows; chunks of 1,024
     (128, 384, 128, (1024, 1027)), (384, 128, 128, (1024, 1027)),   # a chunk's z1 and z2 fill their scratch
-    (384, 640, 128, (300,)),                       # a row tile a CTA
+    (384, 640, 128, (300, 2048, 2049)),            # some token tiles of 128; a row tile a CTA
+    (1024, 384, 128, (256, 1536, 1537)),           # 96 tiles of the few-token core product, and one more
+    (256, 2304, 256, (250, 400)),                  # few tokens with z1 by either kernel
     (19072, 256, 128, (129, 145)),                 # CTAs that go from one block to the next
-    (512, 256, 256, (129, 200)),                   # blocks of 256 in halves
-    (4096, 2304, 256, (129, 513, 1300)),           # on either side of that rule's line; whole blocks over several tiles
+    (512, 256, 256, (129, 200, 2100)),             # blocks of 256 in halves
+    (4096, 2304, 256, (129, 300, 513, 1300)),      # on either side of that rule's line; whole blocks over several tiles
 ])
 def test_wrapper_products_of_the_packed_forward(d_out, d_in, d_block, tokens):
     """The products on either side of the core beyond the few-token kernels.  Integer operands: every fp32 sum is exact,
