@@ -43,7 +43,7 @@ struct SParams {
   float* Z; int64_t ldz;        // [N tokens][ldz], written transposed
   __nv_bfloat16* Zb;            // non-null: the output is written as bf16 here instead
   int64_t M, N, K;              // rows of S, tokens, logical k
-  int m_tiles, n_tiles, k_tiles;
+  int m_tiles, n_tiles, k_tiles, tile_n;
   int32_t* status;
 };
 
@@ -275,8 +275,11 @@ tc_sparse_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant
 //   empty[s], tfull (both CTAs): tcgen05.commit multicast to the pair
 //   tempty    (even CTA): 8 arrivals, one per epilogue warp of either CTA
 // The positions of both CTAs go from their shared to their tensor memory with one tcgen05.cp of the pair.
-// One accumulator buffer of 256 columns (the positions need tensor-memory columns too).
-constexpr int BN2 = 256;
+// One accumulator buffer of 256 columns (the positions need tensor-memory columns too), or two row tiles' of up to 224 that share
+// the stage's tokens: an SM then loads 64 KiB for 256 x 224 outputs and 128 k instead of 50 KiB for 128 x 256, and what L2 delivers
+// (52 bytes a clock and SM) bounds the kernel at the burst clock.  28672 x 8192, 4,096 tokens 898 -> 822 us, 2.34 PFLOP/s of dense-equivalent
+// products.  (Positions copied one stage ahead of their MMAs: 985 us, the stage is held longer; eight epilogue warps with one row tile:
+// 4096 x 4096, 4,096 tokens 94 -> 98.)
 
 __device__ __forceinline__ void umma_bf16_sp_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t tmem_e,
                                                   uint32_t idesc, uint32_t acc) {
@@ -287,19 +290,36 @@ __device__ __forceinline__ void umma_bf16_sp_pair(uint32_t tmem_d, uint64_t ades
       ::"r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(tmem_e), "r"(idesc), "r"(acc)
       : "memory");
 }
-__device__ __forceinline__ uint32_t instr_desc_sp_pair(uint32_t sel) {
-  uint32_t d = sel & 3u;
+__device__ __forceinline__ uint32_t instr_desc_sp_pair(int n) {
+  uint32_t d = 0;
   d |= 1u << 2;
   d |= 1u << 4;
   d |= 1u << 7;
   d |= 1u << 10;
-  d |= (uint32_t)(BN2 >> 3) << 17;
+  d |= (uint32_t)(n >> 3) << 17;
   d |= (uint32_t)(256 >> 4) << 24;
   return d;
 }
-__global__ void __launch_bounds__(NTHREADS, 1)
+// MT: row tiles of 256 that share a stage's tokens
+template <int MT>
+struct PairN {
+  static constexpr int MAX_N = MT == 1 ? 256 : 224;                       // accumulators and positions fit tensor memory
+  static constexpr int STAGES = MT == 1 ? 4 : 3;
+  static constexpr int BH = MAX_N / 2 * 64 * 2;                           // one half (64 k) of the Z1 stage
+  static constexpr int E = MT * A_BYTES + 2 * BH;
+  static constexpr int STAGE = E + MT * E_BYTES;
+  static constexpr uint32_t META = MT * MAX_N;                            // 4 MT columns a stage
+  static constexpr int EPI = MT == 1 ? 4 : 8;                             // epilogue warps
+  static constexpr int THREADS = 64 + 32 * EPI;
+  static constexpr size_t SMEM = (size_t)STAGES * STAGE + 1024;
+};
+
+template <int MT>
+__global__ void __launch_bounds__(PairN<MT>::THREADS, 1)
 tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                       const __grid_constant__ CUtensorMap mapE, const SParams p) {
+  using T = PairN<MT>;
+  constexpr int STAGES = T::STAGES;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t bars[2 * STAGES + 2];
@@ -311,8 +331,9 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[STAGES]);
   const uint32_t tfull = smem_u32(&bars[2 * STAGES]), tempty = smem_u32(&bars[2 * STAGES + 1]);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int m_pairs = p.m_tiles >> 1;                       // 256-row tiles
-  const int n_tiles_total = m_pairs * p.n_tiles;            // p.n_tiles counts 256-token tiles here
+  const int m_groups = p.m_tiles / (2 * MT);
+  const int n_tiles_total = m_groups * p.n_tiles;           // p.n_tiles counts tiles of p.tile_n tokens here
+  const int half_n = p.tile_n / 2;
 
   if (threadIdx.x == 0) {
     abort_flag = 0;
@@ -321,7 +342,7 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
       mbar_init(empty0 + 8 * s, 1);
     }
     mbar_init(tfull, 1);
-    mbar_init(tempty, 8);
+    mbar_init(tempty, 2 * T::EPI);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -345,17 +366,20 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
       bool ok = true;
       for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
         int mt, nt;
-        tile_to_mn(tile, m_pairs, p.n_tiles, mt, nt);
-        const int row0 = mt * 256 + (int)rank * 128, tok0 = nt * BN2 + (int)rank * 128;
+        tile_to_mn(tile, m_groups, p.n_tiles, mt, nt);
+        const int row0 = mt * (256 * MT) + (int)rank * 128, tok0 = nt * p.tile_n + (int)rank * half_n;
         for (int kt = 0; kt < p.k_tiles; ++kt) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * STAGE_BYTES);
+          if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * (MT * (A_BYTES + E_BYTES) + 2 * half_n * 128));
           const uint32_t fb = map_to_cta(full0 + 8 * stage, 0);
-          const uint32_t dst = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          tma_load_2d_pair(dst, &mapA, kt * 64, row0, fb);
-          tma_load_2d_pair(dst + A_BYTES, &mapB, kt * BKL, tok0, fb);
-          tma_load_2d_pair(dst + A_BYTES + BH_BYTES, &mapB, kt * BKL + 64, tok0, fb);
-          tma_load_2d_pair(dst + A_BYTES + 2 * BH_BYTES, &mapE, 0, ((2 * mt + (int)rank) * p.k_tiles + kt) * 128, fb);
+          const uint32_t dst = smem_u32(smem + (size_t)stage * T::STAGE);
+#pragma unroll
+          for (int m = 0; m < MT; ++m) tma_load_2d_pair(dst + m * A_BYTES, &mapA, kt * 64, row0 + 256 * m, fb);
+          tma_load_2d_pair(dst + MT * A_BYTES, &mapB, kt * BKL, tok0, fb);
+          tma_load_2d_pair(dst + MT * A_BYTES + T::BH, &mapB, kt * BKL + 64, tok0, fb);
+#pragma unroll
+          for (int m = 0; m < MT; ++m)
+            tma_load_2d_pair(dst + T::E + m * E_BYTES, &mapE, 0, ((2 * (MT * mt + m) + (int)rank) * p.k_tiles + kt) * 128, fb);
           ++issued;
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
@@ -372,6 +396,8 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (even CTA only)
     if (lane == 0 && rank == 0) {
+      const uint64_t da0 = smem_desc_k(smem_u32(smem)), db0 = smem_desc_k(smem_u32(smem) + MT * A_BYTES), de0 = smem_desc_e(smem_u32(smem) + T::E);
+      const uint32_t idesc = instr_desc_sp_pair(p.tile_n);
       int stage = 0; uint32_t phase = 0;
       int local = 0;
       bool ok = true;
@@ -381,16 +407,17 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
         for (int kt = 0; kt < p.k_tiles; ++kt) {
           if (!mbar_wait_cluster(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t sa = smem_u32(smem + (size_t)stage * STAGE_BYTES);
-          const uint32_t sb = sa + A_BYTES;
-          tmem_cp_e_pair(tmem_base + META_COL0 + (uint32_t)(4 * stage), smem_desc_e(sb + 2 * BH_BYTES));
+          const uint64_t off = (uint64_t)(uint32_t)(stage * (T::STAGE >> 4));
+          const uint32_t meta = tmem_base + T::META + (uint32_t)(4 * MT * stage);
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint64_t da = smem_desc_k(sa + j * 32);
-            const uint64_t dbm = smem_desc_k(sb + (j >> 1) * BH_BYTES + (j & 1) * 64);
-            const uint32_t ecol = tmem_base + META_COL0 + (uint32_t)(4 * stage + j);
-            umma_bf16_sp_pair(tmem_base, da, dbm, ecol & ~1u, instr_desc_sp_pair(ecol & 1u), (uint32_t)((kt > 0) | (j != 0)));
-          }
+          for (int m = 0; m < MT; ++m) tmem_cp_e_pair(meta + 4 * m, de0 + off + (uint64_t)(m * (E_BYTES >> 4)));
+#pragma unroll
+          for (int m = 0; m < MT; ++m)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              umma_bf16_sp_pair(tmem_base + m * T::MAX_N, da0 + off + (uint64_t)(m * (A_BYTES >> 4) + 2 * j),
+                                db0 + off + (uint64_t)((j >> 1) * (T::BH >> 4) + 4 * (j & 1)), meta + 4 * m + (j & 2), idesc | (uint32_t)(j & 1),
+                                (uint32_t)((kt > 0) | (j != 0)));
           umma_commit_pair(empty0 + 8 * stage);
           if (++stage == STAGES) { stage = 0; phase ^= 1; }
         }
@@ -399,22 +426,23 @@ tc_sparse_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_con
     }
   } else {
     // ------------------------------------------------------------ epilogue warps (both CTAs)
-    const int q = warp & 3;
+    const int q = warp & 3, m = (warp - 2) >> 2;                 // lane quarter, row tile
     const uint32_t tempty_lead = map_to_cta(tempty, 0);
     int local = 0;
     bool ok = true;
     for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs, ++local) {
       int mt, nt;
-        tile_to_mn(tile, m_pairs, p.n_tiles, mt, nt);
+        tile_to_mn(tile, m_groups, p.n_tiles, mt, nt);
       if (!mbar_wait(tfull, (uint32_t)local & 1u, abortp, p.status)) { ok = false; break; }
       tc_fence_after();
-      const int64_t row = (int64_t)mt * 256 + rank * 128 + q * 32 + lane;
+      // (trip count and row in constants where they are: with p.tile_n / 32 a tile of 256 took 3 us longer)
+      const int64_t row = (int64_t)(MT * mt + (MT == 1 ? 0 : m)) * 256 + rank * 128 + q * 32 + lane;
 #pragma unroll 1
-      for (int ch = 0; ch < BN2 / 32; ++ch) {
+      for (int ch = 0; ch < T::MAX_N / 32; ++ch) {
+        if (MT > 1 && ch * 32 >= p.tile_n) break;
         uint32_t r[32];
-        tmem_ld32(tmem_base + (uint32_t)(ch * 32) + ((uint32_t)(q * 32) << 16), r);
-        const int64_t tok0 = (int64_t)nt * BN2 + ch * 32;
-        store_chunk(p, r, row, tok0, lane);
+        tmem_ld32(tmem_base + (uint32_t)(m * T::MAX_N + ch * 32) + ((uint32_t)(q * 32) << 16), r);
+        store_chunk(p, r, row, (int64_t)nt * (MT == 1 ? T::MAX_N : p.tile_n) + ch * 32, lane);
       }
       tc_fence_before();
       __syncwarp();
@@ -884,6 +912,21 @@ void launch_compress_24(armor_ctx* c, const float* S, const uint8_t* M, void* Sc
 }
 
 // Z2[n][d_out] = Z1[n][d_in] * S^T with S given compressed (Sc, E); Z1 bf16; Z2 fp32, or bf16 if out_bf16.
+template <int MT>
+static armor_status launch_pairs(armor_ctx* c, const CUtensorMap& mA, const void* z1, const CUtensorMap& mE, SParams p, int tile_n, cudaStream_t s) {
+  CUtensorMap mB;
+  if (!make_map_bf16(&mB, z1, p.N, p.K, p.K, tile_n / 2)) return ARMOR_ERR_CUDA;
+  static PerDeviceOnce attr;
+  if (ensure_dynamic_smem(attr, c->device, tc_sparse_pair_kernel<MT>, PairN<MT>::SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
+  p.tile_n = tile_n;
+  p.n_tiles = (int)((p.N + tile_n - 1) / tile_n);
+  const int tiles = p.m_tiles / (2 * MT) * p.n_tiles, pairs = tiles < c->n_sm / 2 ? tiles : c->n_sm / 2;
+  // (a dependent launch: 4096 x 4096, 400 tokens 26.8 -> 24.9 us a forward)
+  launch_dependent(tc_sparse_pair_kernel<MT>, 2 * pairs, PairN<MT>::THREADS, PairN<MT>::SMEM, LaunchStream(s, false, 2), mA, mB, mE, p);
+  c->launches++;
+  return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
+}
+
 armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const void* z1_bf16, void* z2, bool out_bf16,
                               int64_t n, cudaStream_t s) {
   if (!tc_sparse_ok(c) || n <= 0) return ARMOR_ERR_UNSUPPORTED;
@@ -902,14 +945,21 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
   const int n_sm = c->n_sm;
   KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)p.M * (double)p.N * (double)p.K, s);   // dense-equivalent flops
   if (g_sparse_pairs && c->d_out % 256 == 0 && n_sm >= 2) {
-      static PerDeviceOnce attr2;
-    if (ensure_dynamic_smem(attr2, c->device, tc_sparse_pair_kernel, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
-    p.n_tiles = (int)((n + BN2 - 1) / BN2);
-    const int tiles = (p.m_tiles / 2) * p.n_tiles;
-    int pairs = n_sm / 2;
-    if (tiles < pairs) pairs = tiles;
-    // (a dependent launch: 4096 x 4096, 400 tokens 26.8 -> 24.9 us a forward)
-    launch_dependent(tc_sparse_pair_kernel, 2 * pairs, NTHREADS, SMEM, LaunchStream(s, false, 2), mA, mB, mE, p);
+    // Two row tiles at a time, or one: rounds of the pairs times what a tile takes, its tokens plus, with two, 200 tokens' worth (a tile
+    // of 512 x 224 takes 1.62 times one of 256 x 256, of 512 x 192 1.48 times).  Whole forwards, one and two: 28672 x 8192, 4,096 tokens
+    // (25 rounds and 15) 1,192 and 1,123 us; 8192 x 8192, 640 (2 and 1) 76.5 and 63.2, 2,000 (4 and 2) 156 and 139; 4096 x 4096, 4,096
+    // (4 and 3) 93 and 107: one.
+    int width = 256;
+    if (c->d_out % 512 == 0) {
+      const int pairs = n_sm / 2;
+      int64_t least = (p.m_tiles / 2 * ((n + 255) / 256) + pairs - 1) / pairs * 262;
+      for (int w = PairN<2>::MAX_N; w >= 128; w -= 32) {
+        const int64_t cost = (p.m_tiles / 4 * ((n + w - 1) / w) + pairs - 1) / pairs * (w + 200);
+        if (cost < least) { least = cost; width = w; }
+      }
+    }
+    if (width < 256) return launch_pairs<2>(c, mA, z1_bf16, mE, p, width, s);
+    return launch_pairs<1>(c, mA, z1_bf16, mE, p, 256, s);
   } else {
     const int tiles = p.m_tiles * p.n_tiles;
     const int grid = tiles < n_sm ? tiles : n_sm;

@@ -101,6 +101,8 @@ def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
     (19072, 256, 128, (129, 145)),                 # CTAs that go from one block to the next
     (512, 256, 256, (129, 200, 2100)),             # blocks of 256 in halves
     (4096, 2304, 256, (129, 300, 513, 1300)),      # on either side of that rule's line; whole blocks over several tiles
+    (4096, 512, 128, (1152, 1153, 1500, 2000, 2001)),   # core product: two row tiles by 128, 160, 192, 224 tokens, and one
+    (768, 512, 128, (2050,)), (2560, 640, 128, (1500, 1700)),   # an odd number of row tiles; odd groups of rows
 ])
 def test_wrapper_products_of_the_packed_forward(d_out, d_in, d_block, tokens):
     """The products on either side of the core beyond the few-token kernels.  Integer operands: every fp32 sum is exact,
