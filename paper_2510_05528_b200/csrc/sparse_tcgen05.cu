@@ -945,7 +945,8 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
   const int n_sm = c->n_sm;
   KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)p.M * (double)p.N * (double)p.K, s);   // dense-equivalent flops
   if (g_sparse_pairs && c->d_out % 256 == 0 && n_sm >= 2) {
-    // Two row tiles at a time, or one: rounds of the pairs times what a tile takes, its tokens plus, with two, 200 tokens' worth (a tile
+    // Two row tiles at a time, or one: rounds of the pairs times what a tile takes, its tokens plus, with two, 200 tokens' worth (fp32 out:
+    // 240, 14336 x 2048, 1,459 tokens, 3 rounds or 5, 161 us and 154; a tile
     // of 512 x 224 takes 1.62 times one of 256 x 256, of 512 x 192 1.48 times).  Whole forwards, one and two: 28672 x 8192, 4,096 tokens
     // (25 rounds and 15) 1,192 and 1,123 us; 8192 x 8192, 640 (2 and 1) 76.5 and 63.2, 2,000 (4 and 2) 156 and 139; 4096 x 4096, 4,096
     // (4 and 3) 93 and 107: one.
@@ -954,7 +955,7 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
       const int pairs = n_sm / 2;
       int64_t least = (p.m_tiles / 2 * ((n + 255) / 256) + pairs - 1) / pairs * 262;
       for (int w = PairN<2>::MAX_N; w >= 128; w -= 32) {
-        const int64_t cost = (p.m_tiles / 4 * ((n + w - 1) / w) + pairs - 1) / pairs * (w + 200);
+        const int64_t cost = (p.m_tiles / 4 * ((n + w - 1) / w) + pairs - 1) / pairs * (w + (out_bf16 ? 200 : 240));
         if (cost < least) { least = cost; width = w; }
       }
     }
