@@ -208,6 +208,27 @@ def test_carried_product_moves_by_both_steps(d_out, d_in, d_block):
         assert np.all(np.diff(rec["loss_mask"]) <= 0)
 
 
+@pytest.mark.parametrize("d_out", [128, 640, 4224, 16384, 16512])
+def test_guards_products_of_few_and_many_row_blocks(d_out):
+    """The guard's products with H have a row for every row block: 1, 5, 33 (boxes of 32 rows that are not full), 128 (the most the kernel
+    with the rows in tensor memory takes) and 129; the two line searches move E H_w on its way through the gradients, by both steps,
+    one, or none.  A wrong row, move or sign shows in the tracked loss, which otherwise is the one evaluated from the state (fp32
+    sums: 1e-5 of the start, as above)."""
+    d_in = 256
+    g = _gen(d_out)
+    W = torch.randn(d_out, d_in, device=DEV, generator=g)
+    X = torch.randn(4 * d_in, d_in, device=DEV, generator=g)
+    H = (X.double().t() @ X.double()).float()
+    for phases in (15, 15 - 4, 15 - 2, 9):
+        ctx = _ctx(d_out, d_in, 128, phases=phases)
+        st = ctx.init(W, H)
+        rec = ctx.read_stats(ctx.bcd_step(st, H, 0, 3))
+        loss = ctx.proxy_loss(st, H).item()
+        assert abs(rec["loss_mask"][-1] - loss) <= 1e-5 * rec["loss_start"][0]
+        assert np.all(np.diff(rec["loss_mask"]) <= 0)
+        assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
 @pytest.mark.parametrize("d_in", [768, 1024, 1536])
 def test_cut_and_uncut_grams_have_the_same_bits(d_in):
     """fp32 activations, 16,384 tokens at a time.  One call for two such chunks stages the second beside the contraction of the first:
