@@ -144,7 +144,7 @@ size_t carve(const armor_config& cfg, armor_ctx* c, char* base) {
   TAKE(tab_g, unsigned long long*, (size_t)nbo * nbi * sizeof(unsigned long long));
   TAKE(status, int32_t*, ST_COUNT * sizeof(int32_t));
   TAKE(screen, int32_t*, 4 * sizeof(int32_t));
-  TAKE(core_flags, int32_t*, 2 * sizeof(int32_t));
+  TAKE(core_dense, int32_t*, sizeof(int32_t));
   TAKE(it_dev, int64_t*, sizeof(int64_t));
 #undef TAKE
   if (c) {
@@ -837,7 +837,7 @@ static armor_status apply_impl(armor_ctx* c, const float* A, const float* B, con
     c->block_one_pass = bf16 ? 1 : 0;
     bd_right(c, xc, B, true, c->T, n, d_in, 1.f, nullptr, 0.f, s);                   // z1 = x B^T
     c->block_one_pass = 0;
-    armor_status st = wide ? core_f16_product(c, c->T, S, sparse24, z2, n, s) : apply_core(c, c->T, S, packed, z2, n, bf16, s);   // z2 = z1 S^T
+    armor_status st = wide ? core_f16_product(c, c->T, S, sparse24, t0 == 0, z2, n, s) : apply_core(c, c->T, S, packed, z2, n, bf16, s);   // z2 = z1 S^T
     if (st != ARMOR_OK) return st;
     c->block_one_pass = bf16 ? 1 : 0;
     bd_right(c, z2, A, true, yc, n, d_out, 1.f, nullptr, 0.f, s);                    // y = z2 A^T

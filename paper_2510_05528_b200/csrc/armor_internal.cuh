@@ -111,7 +111,7 @@ struct armor_ctx {
   unsigned long long* tab_g;   // its global group index
   int32_t* status;    // [ST_COUNT]
   int32_t* screen;    // [4] per-call counters of the input screening
-  int32_t* core_flags;   // fp32 forward: [0] the core is not 2:4, [1] activations are not finite
+  int32_t* core_dense;   // fp32 forward: 1 if the core is not 2:4, so that the dense product runs instead of the sparse one
   int64_t* it_dev;    // iteration index inside the running armor_bcd_step call (advanced by the first kernel of an iteration)
   int use_graphs;     // 1: repeated iterations of a call are replayed from a CUDA graph
   cudaStream_t cap_stream;   // the context's own stream, used only to capture that graph
@@ -376,18 +376,22 @@ armor_status apply_core(armor_ctx* c, const float* z1, const float* S, const voi
                         bool bf16, cudaStream_t s);
 
 // the same in the three-pass fp16 mode with S split beforehand (once per call), up to gram_rows tokens at a time
-// (sparse: on the sparse tensor cores, whatever S holds; core_f16_sparse says where that is faster, for calls of so many tokens)
+// (sparse: on the sparse tensor cores unless S is not 2:4; core_f16_sparse says where that is faster, for calls of so many
+// tokens; first: the call's first chunk)
 bool core_f16_ok(const armor_ctx* c);
 bool core_f16_sparse(const armor_ctx* c, int64_t n_tokens);
 armor_status core_f16_split_S(armor_ctx* c, const float* S, bool sparse, cudaStream_t s);
-armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, bool sparse, float* z2, int64_t n, cudaStream_t s);
+armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, bool sparse, bool first, float* z2, int64_t n, cudaStream_t s);
 
 // operand preparation of the three-pass fp16 mode (split_f16.cu)
 void launch_f16_prepare_H(armor_ctx* c, const float* H, cudaStream_t s);   // hpow, scaled H as fp16 hi | lo in Hlo
 void launch_f16_split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t rows, int64_t cols, const float* colscale,
-                           float post, void* hi, void* lo, float* out_scale, cudaStream_t s, int32_t* not_finite = nullptr);
-// the 2:4 core [d_out, d_in] as fp16 parts of its kept entries with their positions, see split_core24_kernel
-void launch_split_core24(armor_ctx* c, const float* S, int layer, void* hi, void* lo, void* E, float* scale, int32_t* flags, cudaStream_t s);
+                           float post, void* hi, void* lo, float* out_scale, cudaStream_t s);
+// the 2:4 core [d_out, d_in] as fp16 parts of its kept entries with their positions, see split_core24_kernel; *dense 1 if it is not 2:4
+void launch_split_core24(armor_ctx* c, const float* S, void* hi, void* lo, void* E, float* scale, int32_t* dense, cudaStream_t s);
+// z1 as launch_f16_split_rows has it, tokens that are not finite with NaN as their scale; with S, and if *dense, S as well
+void launch_split_tokens(armor_ctx* c, const float* z, int64_t tokens, void* hi, void* lo, float* out_scale, const float* S, void* s_hi, void* s_lo,
+                         float* s_scale, const int32_t* dense, cudaStream_t s);
 float f16_H_post_scale();
 armor_status launch_f16_gram_stage(armor_ctx* c, const void* X, int x_dtype, int64_t ldx, int64_t rows, int64_t cols,
                                    void* Thi, void* Tlo, float* gscale, cudaStream_t s);
@@ -489,6 +493,7 @@ struct TcGemm {
   int symmetric_lower;   // only the lower triangle (tiles with n0 <= m0, elements with column <= row) is computed (M == N)
   const float* d1; const float* d2;  // optional dot operands (ld = ldc)
   double* part1; double* part2;      // partial sums, launch_tc_gemm says how many
+  const int32_t* only_if;            // not null: nothing happens where it points to 0 (K-major operands)
 };
 armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStream_t s);
 bool tc_gemm_shape_ok(int64_t M, int64_t N, int64_t K);
@@ -500,7 +505,7 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
                               int64_t n, cudaStream_t s);
 bool tc_sparse3_ok(const armor_ctx* c);
 armor_status launch_tc_sparse3(armor_ctx* c, const void* hi, const void* lo, const void* E, const float* row_scale, const void* zhi,
-                               const void* zlo, const float* tok_scale, const int32_t* flags, float* z2, int64_t n, cudaStream_t s);
+                               const void* zlo, const float* tok_scale, const int32_t* dense, float* z2, int64_t n, cudaStream_t s);
 // the wrapper products of the bf16 forward (fwd_tcgen05.cu)
 bool fwd_block_ok(const armor_ctx* c);
 void launch_pack_blocks(armor_ctx* c, const float* P, const float* rowscale, const float* colscale, void* Q, int nb,

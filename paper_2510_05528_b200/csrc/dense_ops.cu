@@ -235,26 +235,32 @@ bool core_f16_ok(const armor_ctx* c) {
 bool core_f16_sparse(const armor_ctx* c, int64_t n_tokens) {
   return tc_sparse3_ok(c) && n_tokens * (c->d_out / 256) >= (int64_t)c->n_sm / 2 * 64;
 }
-// sparse: S's parts in U (hi of both layers, then lo), positions in Lo
+// S's parts in U (hi, then lo).  sparse: the parts of what a 2:4 core keeps, positions in Lo; if it is not 2:4 core_dense says so, and the first
+// chunk's split puts the parts of the whole of S in their place.
 armor_status core_f16_split_S(armor_ctx* c, const float* S, bool sparse, cudaStream_t s) {
   __half* shi = reinterpret_cast<__half*>(c->U);
   if (sparse) {
-    if (cudaMemsetAsync(c->core_flags, 0, 2 * sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
-    launch_split_core24(c, S, 0, shi, shi + c->wn, c->Lo, c->rowscale2, c->core_flags, s);
+    if (cudaMemsetAsync(c->core_dense, 0, sizeof(int32_t), s) != cudaSuccess) return ARMOR_ERR_CUDA;
+    launch_split_core24(c, S, shi, shi + c->wn, c->Lo, c->rowscale2, c->core_dense, s);
   } else {
     launch_f16_split_rows(c, S, c->d_in, c->d_out, c->d_in, nullptr, 1.f, shi, shi + c->wn, c->rowscale2, s);
   }
   return ARMOR_OK;
 }
-armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, bool sparse, float* z2, int64_t n, cudaStream_t s) {
+armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, bool sparse, bool first, float* z2, int64_t n, cudaStream_t s) {
   const int64_t d_in = c->d_in, d_out = c->d_out;
   __half* ahi = reinterpret_cast<__half*>(c->Xt_hi);
   __half* shi = reinterpret_cast<__half*>(c->U);
   float* scales = reinterpret_cast<float*>(c->colpart);         // 64 d_in doubles
-  launch_f16_split_rows(c, z1, d_in, n, d_in, nullptr, 1.f, ahi, ahi + n * d_in, scales, s, sparse ? c->core_flags + 1 : nullptr);
   if (sparse) {
-    launch_split_core24(c, S, 1, shi, shi + c->wn, c->Lo, c->rowscale2, c->core_flags, s);
-    return launch_tc_sparse3(c, shi, shi + c->wn, c->Lo, c->rowscale2, ahi, ahi + n * d_in, scales, c->core_flags, z2, n, s);
+    // One of the two products does nothing, and which is known on the device only.  For a core that is not 2:4 that costs 10 to 25 us a
+    // call over the dense product alone (14336 x 4096, 2,048 tokens 649 and 656 us, 1024 x 1024, 8,192 134 and 148, 14336 x 1024, 150 82 and
+    // 104), for a 2:4 core up to 1 us.  Two sparse products for the former, of the first and the other two of every four: 1,047, 154, 155.
+    launch_split_tokens(c, z1, n, ahi, ahi + n * d_in, scales, first ? S : nullptr, shi, shi + c->wn, c->rowscale2, c->core_dense, s);
+    const armor_status st = launch_tc_sparse3(c, shi, shi + c->wn, c->Lo, c->rowscale2, ahi, ahi + n * d_in, scales, c->core_dense, z2, n, s);
+    if (st != ARMOR_OK) return st;
+  } else {
+    launch_f16_split_rows(c, z1, d_in, n, d_in, nullptr, 1.f, ahi, ahi + n * d_in, scales, s);
   }
   TcGemm g{};
   g.lda = d_in; g.ldb = d_in; g.ldc = d_out;
@@ -263,6 +269,7 @@ armor_status core_f16_product(armor_ctx* c, const float* z1, const float* S, boo
   g.A = ahi; g.Alo = ahi + n * d_in; g.B = shi; g.Blo = shi + c->wn; g.passes = 6; g.fp16 = 1;
   g.row_scale = scales; g.col_scale = c->rowscale2;
   g.k_segment = K_SEGMENT;
+  g.only_if = sparse ? c->core_dense : nullptr;
   return launch_tc_gemm(c, g, nullptr, s);
 }
 

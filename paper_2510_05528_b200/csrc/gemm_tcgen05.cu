@@ -65,6 +65,7 @@ struct Params {
   const float* row_scale; const float* col_scale;   // optional powers of two the accumulator is multiplied by
   int dependent;         // launched beside the kernel that writes the scales: the epilogue waits for it
   int f16;               // 16-bit operands are fp16 (1) or bf16 (0)
+  const int32_t* only_if;
   int32_t* status;
   // Tail split: tiles [split_first, n_tiles_total) are cut into split_parts pieces of split_kt k-tiles (the last one
   // may be shorter), each piece a work item of its own that writes a 256 x 256 slab of partial sums; a second kernel
@@ -260,6 +261,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__
   const uint32_t tfull0 = smem_u32(&bars[2 * STAGES]), tempty0 = smem_u32(&bars[2 * STAGES + 2]);
   constexpr int BKE = H16 ? 64 : 32;                // elements of K per 128-byte row: 16-bit or fp32
   const int kt_total = (int)((p.K + BKE - 1) / BKE);
+  if (!MN && p.only_if) {
+    grid_dependency_wait();
+    if (*p.only_if == 0) return;                    // (before anything is allocated, both CTAs of the pair alike)
+  }
 
   // full, empty of the stages; tfull, tempty of the accumulator buffers.  full and tempty are used in the even CTA
   // only (both CTAs' loads and epilogue warps signal it there), empty and tfull in both (commits reach the pair).
@@ -487,6 +492,7 @@ constexpr int FIX_NT = BMP / PARTS * BN / 4;
 __global__ void __launch_bounds__(FIX_NT) tc_gemm_fixup_kernel(const Params p) {
   constexpr int FR = BMP / PARTS;                         // rows per CTA
   grid_begin();
+  if (p.only_if && *p.only_if == 0) return;
   const int slots = gridDim.x / (p.n_tiles_total - p.split_first);       // PARTS, or those that hold rows
   const int tile = p.split_first + blockIdx.x / slots, slot = blockIdx.x % slots;
   int mt, nt;
@@ -618,7 +624,7 @@ armor_status launch_impl(armor_ctx* c, const TcGemm& g, Params p, cudaStream_t s
   }
   const int pairs = p.n_items < n_pairs ? p.n_items : n_pairs;
   {
-    KTimer kt(c, ARMOR_KC_GEMM, p.symmetric_lower ? (double)p.M * (double)(p.N + BM) * (double)p.K
+    KTimer kt(c, ARMOR_KC_GEMM, p.only_if ? 0.0 : p.symmetric_lower ? (double)p.M * (double)(p.N + BM) * (double)p.K
                                                   : 2.0 * (double)p.M * (double)p.N * (double)p.K, s);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * pairs); cfg.blockDim = dim3(NTHREADS); cfg.dynamicSmemBytes = SMEM; cfg.stream = s;
@@ -664,6 +670,7 @@ armor_status launch_tc_gemm(armor_ctx* c, const TcGemm& g, int* n_part, cudaStre
   p.accumulate = g.accumulate; p.symmetric_lower = g.symmetric_lower;
   p.d1 = g.d1; p.d2 = g.d2; p.part1 = g.part1; p.part2 = g.part2;
   p.row_scale = g.row_scale; p.col_scale = g.col_scale; p.dependent = g.dependent; p.f16 = g.fp16;
+  p.only_if = g.only_if;
   p.status = c->status;
   p.c_vec = (reinterpret_cast<uintptr_t>(g.C) % 16 == 0) ? 1 : 0;   // (ldc is a multiple of 4)
   const int bke = h16 ? 64 : BK;

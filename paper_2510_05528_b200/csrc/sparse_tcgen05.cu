@@ -601,8 +601,7 @@ tc_sparse_small_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
 //   * tiles of 256 rows of S by tile_n <= 224 tokens, so that two accumulators and the positions fit tensor memory: the sums of
 //     a segment of the contraction leave for the epilogue warps' registers while the next segment runs.  The host picks the tile_n that
 //     fills the last wave best;
-//   * a core that is not 2:4, or activations that are not finite (0 * inf), take the other two positions of every
-//     group as a second layer of the contraction: flags says so, any S is the sum of two such layers.
+//   * a core that is not 2:4 is left to the dense product, which is launched behind this one: *dense says so.
 // Segments of 1,024 columns as in the dense product, which are half as many truncating additions here (whole forward 4.0e-6 off fp64
 // sums where the dense core was 5.8e-6; segments of 2,048 6.1e-6, at the same speed).
 // What bounds it: the sparse tensor cores under the power cap, and at the burst clock what L2 delivers (90 KiB per SM and stage).
@@ -614,10 +613,10 @@ constexpr int S3_B = 2 * A_BYTES, S3_E = S3_B + 4 * BH_BYTES, S3_STAGE = S3_E + 
 struct S3Params {
   float* Z; int64_t ldz;                            // [tokens][d_out]
   int64_t N;                                        // tokens
-  int m_rows, m_pairs, n_tiles, k_tiles, tile_n;    // rows of S, tiles of 256 of them, tiles of tile_n tokens, k tiles of 128
+  int m_pairs, n_tiles, k_tiles, tile_n;            // tiles of 256 rows of S, tiles of tile_n tokens, k tiles of 128
   const float* row_scale;                           // per row of S, per token
   const float* tok_scale;
-  const int32_t* flags;                             // either of two: both layers
+  const int32_t* dense;                             // not 0: the dense product runs instead
   int32_t* status;
 };
 
@@ -636,8 +635,6 @@ tc_sparse3_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
   const uint32_t full0 = smem_u32(&bars[0]), empty0 = smem_u32(&bars[S3_STAGES]);
   const uint32_t tfull0 = smem_u32(&bars[2 * S3_STAGES]), tempty0 = smem_u32(&bars[2 * S3_STAGES + 2]);
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int n_tiles_total = p.m_pairs * p.n_tiles;
-  const int k_total = (p.flags[0] | p.flags[1]) ? 2 * p.k_tiles : p.k_tiles;
   const int half_n = p.tile_n / 2;
 
   if (threadIdx.x == 0) {
@@ -656,6 +653,8 @@ tc_sparse3_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
   __syncthreads();
   cluster_sync_all();                                       // both CTAs' barriers exist before anyone signals them
   tc_fence_after();
+  grid_begin();                                             // (tensor memory is this CTA's before the next kernel's CTAs start)
+  const int n_tiles_total = *p.dense != 0 ? 0 : p.m_pairs * p.n_tiles;
   const uint32_t tmem_base = tmem_base_holder;
   volatile int* abortp = &abort_flag;
 
@@ -669,19 +668,18 @@ tc_sparse3_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
         int mt, nt;
         tile_to_mn(tile, p.m_pairs, p.n_tiles, mt, nt);
         const int row0 = mt * 256 + (int)rank * 128, tok0 = nt * p.tile_n + (int)rank * half_n;
-        for (int f = 0; f < k_total; ++f) {
+        for (int kt = 0; kt < p.k_tiles; ++kt) {
           if (!mbar_wait(empty0 + 8 * stage, phase ^ 1, abortp, p.status)) { ok = false; break; }
           if (rank == 0) mbar_expect_tx(full0 + 8 * stage, 2 * stage_bytes);
-          const int layer = f >= p.k_tiles ? 1 : 0, kt = f - layer * p.k_tiles;
           const uint32_t fb = map_to_cta(full0 + 8 * stage, 0);
           const uint32_t dst = smem_u32(smem + (size_t)stage * S3_STAGE);
-          tma_load_2d_pair(dst, &mapA, kt * 64, layer * p.m_rows + row0, fb);
-          tma_load_2d_pair(dst + A_BYTES, &mapAlo, kt * 64, layer * p.m_rows + row0, fb);
+          tma_load_2d_pair(dst, &mapA, kt * 64, row0, fb);
+          tma_load_2d_pair(dst + A_BYTES, &mapAlo, kt * 64, row0, fb);
           tma_load_2d_pair(dst + S3_B, &mapB, kt * BKL, tok0, fb);
           tma_load_2d_pair(dst + S3_B + BH_BYTES, &mapB, kt * BKL + 64, tok0, fb);
           tma_load_2d_pair(dst + S3_B + 2 * BH_BYTES, &mapBlo, kt * BKL, tok0, fb);
           tma_load_2d_pair(dst + S3_B + 3 * BH_BYTES, &mapBlo, kt * BKL + 64, tok0, fb);
-          tma_load_2d_pair(dst + S3_E, &mapE, 0, ((layer * 2 * p.m_pairs + 2 * mt + (int)rank) * p.k_tiles + kt) * 128, fb);
+          tma_load_2d_pair(dst + S3_E, &mapE, 0, ((2 * mt + (int)rank) * p.k_tiles + kt) * 128, fb);
           ++issued;
           if (++stage == S3_STAGES) { stage = 0; phase ^= 1; }
         }
@@ -705,12 +703,12 @@ tc_sparse3_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
       int local = 0;                                        // (tile, segment) items so far: selects the accumulator
       bool ok = true;
       for (int tile = pair; tile < n_tiles_total && ok; tile += n_pairs) {
-        for (int f0 = 0; f0 < k_total && ok; f0 += S3_SEG, ++local) {
+        for (int f0 = 0; f0 < p.k_tiles && ok; f0 += S3_SEG, ++local) {
           const int as = local & 1;
           if (!mbar_wait_cluster(tempty0 + 8 * as, ((uint32_t)(local >> 1) & 1u) ^ 1u, abortp, p.status)) { ok = false; break; }
           tc_fence_after();
           const uint32_t tacc = tmem_base + (uint32_t)(as * S3_MAX_N);
-          const int f1 = min(k_total, f0 + S3_SEG);
+          const int f1 = min(p.k_tiles, f0 + S3_SEG);
           for (int f = f0; f < f1; ++f) {
             if (!mbar_wait_cluster(full0 + 8 * stage, phase, abortp, p.status)) { ok = false; break; }
             tc_fence_after();
@@ -745,7 +743,7 @@ tc_sparse3_pair_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
       float acc[128];
 #pragma unroll
       for (int i = 0; i < 128; ++i) acc[i] = 0.f;
-      for (int f0 = 0; f0 < k_total && ok; f0 += S3_SEG, ++local) {
+      for (int f0 = 0; f0 < p.k_tiles && ok; f0 += S3_SEG, ++local) {
         const int as = local & 1;
         if (!mbar_wait(tfull0 + 8 * as, (uint32_t)(local >> 1) & 1u, abortp, p.status)) { ok = false; break; }
         tc_fence_after();
@@ -1003,19 +1001,19 @@ armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E,
   return launch_small<128>(c, Sc, E, z1_bf16, p, *pieces, per, s);
 }
 
-// Z2[n][d_out] = Z1[n][d_in] * S^T, fp32-grade: the parts of S's two layers (hi: layer 0, layer 1, lo likewise, [d_out][d_in / 2] each)
-// with their positions, z1's parts, the rows' scales and the flags that ask for the second layer.
+// Z2[n][d_out] = Z1[n][d_in] * S^T, fp32-grade: the parts of what S keeps (hi, lo, [d_out][d_in / 2] each) with their positions, z1's
+// parts and the rows' scales; nothing if *dense.
 bool tc_sparse3_ok(const armor_ctx* c) {
   return tc_sparse_ok(c) && c->cfg.precision == ARMOR_PREC_FP16X3 && c->d_out % 256 == 0 && c->n_sm >= 2;
 }
 armor_status launch_tc_sparse3(armor_ctx* c, const void* hi, const void* lo, const void* E, const float* row_scale, const void* zhi,
-                               const void* zlo, const float* tok_scale, const int32_t* flags, float* z2, int64_t n, cudaStream_t s) {
+                               const void* zlo, const float* tok_scale, const int32_t* dense, float* z2, int64_t n, cudaStream_t s) {
   if (!tc_sparse3_ok(c) || n <= 0) return ARMOR_ERR_UNSUPPORTED;
   const int pairs = c->n_sm / 2;
   S3Params p{};
   p.Z = z2; p.ldz = c->d_out; p.N = n;
-  p.m_rows = (int)c->d_out; p.m_pairs = (int)(c->d_out / 256); p.k_tiles = (int)(c->d_in / BKL);
-  p.row_scale = row_scale; p.tok_scale = tok_scale; p.flags = flags; p.status = c->status;
+  p.m_pairs = (int)(c->d_out / 256); p.k_tiles = (int)(c->d_in / BKL);
+  p.row_scale = row_scale; p.tok_scale = tok_scale; p.dense = dense; p.status = c->status;
   // the width of a tile that costs least: waves of tiles times what a tile takes, its MMAs (proportional to the width) plus what
   // comes with every tile whatever its width (S's share of the loads, the first stage, the last segment's way out: about 48 tokens' worth)
   int64_t least = 0;
@@ -1026,23 +1024,17 @@ armor_status launch_tc_sparse3(armor_ctx* c, const void* hi, const void* lo, con
   p.n_tiles = (int)((n + p.tile_n - 1) / p.tile_n);
   CUtensorMap mA, mAlo, mB, mBlo, mE;
   const CUtensorMapDataType f16 = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-  if (!make_map_16(&mA, hi, 2 * c->d_out, c->d_in / 2, c->d_in / 2, 128, f16)) return ARMOR_ERR_CUDA;
-  if (!make_map_16(&mAlo, lo, 2 * c->d_out, c->d_in / 2, c->d_in / 2, 128, f16)) return ARMOR_ERR_CUDA;
+  if (!make_map_16(&mA, hi, c->d_out, c->d_in / 2, c->d_in / 2, 128, f16)) return ARMOR_ERR_CUDA;
+  if (!make_map_16(&mAlo, lo, c->d_out, c->d_in / 2, c->d_in / 2, 128, f16)) return ARMOR_ERR_CUDA;
   if (!make_map_16(&mB, zhi, n, c->d_in, c->d_in, p.tile_n / 2, f16)) return ARMOR_ERR_CUDA;
   if (!make_map_16(&mBlo, zlo, n, c->d_in, c->d_in, p.tile_n / 2, f16)) return ARMOR_ERR_CUDA;
-  if (!make_map_e(&mE, E, 2 * (c->d_out / 128) * (c->d_in / 128) * 128)) return ARMOR_ERR_CUDA;
+  if (!make_map_e(&mE, E, (c->d_out / 128) * (c->d_in / 128) * 128)) return ARMOR_ERR_CUDA;
   constexpr size_t SMEM = (size_t)S3_STAGES * S3_STAGE + 1024;
   static PerDeviceOnce attr;
   if (ensure_dynamic_smem(attr, c->device, tc_sparse3_pair_kernel, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int tiles = p.m_pairs * p.n_tiles;
   KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)c->d_out * (double)n * (double)c->d_in, s);   // dense-equivalent flops
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(2 * (tiles < pairs ? tiles : pairs)); cfg.blockDim = dim3(S3_THREADS); cfg.dynamicSmemBytes = SMEM; cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, tc_sparse3_pair_kernel, mA, mAlo, mB, mBlo, mE, p) != cudaSuccess) return ARMOR_ERR_CUDA;
+  launch_dependent(tc_sparse3_pair_kernel, 2 * (tiles < pairs ? tiles : pairs), S3_THREADS, SMEM, LaunchStream(s, false, 2), mA, mAlo, mB, mBlo, mE, p);
   c->launches++;
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }

@@ -106,14 +106,12 @@ __global__ void __launch_bounds__(NT) split_H_kernel(const float4* H, const floa
 // range by a power of two of its own; out_scale[row] = post / that power.  KEEP float4 per thread stay in registers between
 // the maximum and the split (0: the row is read again).  The scaling is a product with a power of two: exact, or rounded
 // once where the result is subnormal.
-// FINITE: *not_finite becomes 1 if an entry is not finite.
+// FINITE: a row with an entry that is not finite gets NaN as its scale, and with it a result of nothing but NaN.  (The dense
+// product has that without help: the low part of infinity is NaN, times whatever the other operand holds.  The sparse
+// one leaves out half of it.)
 template <int KEEP, bool FINITE>
-__global__ void __launch_bounds__(NT) split_rows_kernel(const float* in, int64_t ld, int64_t cols,
-                                                        const float* colscale, float post,
-                                                        __half2* __restrict__ hi, __half2* __restrict__ lo,
-                                                        float* __restrict__ out_scale, int32_t* __restrict__ not_finite) {
-  grid_begin();
-  const int64_t row = blockIdx.x;
+__device__ __forceinline__ void split_row(const float* in, int64_t ld, int64_t cols, const float* colscale, float post, int64_t row,
+                                          __half2* __restrict__ hi, __half2* __restrict__ lo, float* __restrict__ out_scale) {
   const float4* src = reinterpret_cast<const float4*>(in + row * ld);
   const float4* cs4 = reinterpret_cast<const float4*>(colscale);
   const int64_t c4n = cols / 4;
@@ -139,7 +137,7 @@ __global__ void __launch_bounds__(NT) split_rows_kernel(const float* in, int64_t
   mx = block_max(mx);
   const int e = scale_exp(mx);
   const float p = scalbnf(1.f, e);
-  if (threadIdx.x == 0) out_scale[row] = scalbnf(post, -e);
+  if (!FINITE && threadIdx.x == 0) out_scale[row] = scalbnf(post, -e);
   uint2* dh = reinterpret_cast<uint2*>(hi + row * (cols / 2));
   uint2* dl = reinterpret_cast<uint2*>(lo + row * (cols / 2));
   bool odd = false;
@@ -162,98 +160,112 @@ __global__ void __launch_bounds__(NT) split_rows_kernel(const float* in, int64_t
   } else {
     for (int64_t i = threadIdx.x; i < c4n; i += NT) put(i, fetch(i));
   }
-  if (FINITE && odd) *not_finite = 1;
+  if (FINITE) {
+    odd = __syncthreads_or(odd) != 0;
+    if (threadIdx.x == 0) out_scale[row] = odd ? __uint_as_float(0x7fc00000u) : scalbnf(post, -e);
+  }
+}
+
+template <int KEEP>
+__global__ void __launch_bounds__(NT) split_rows_kernel(const float* in, int64_t ld, int64_t cols, const float* colscale, float post,
+                                                        __half2* __restrict__ hi, __half2* __restrict__ lo, float* __restrict__ out_scale) {
+  grid_begin();
+  split_row<KEEP, false>(in, ld, cols, colscale, post, blockIdx.x, hi, lo, out_scale);
+}
+
+// The activations of the fp32 forward, `tokens` rows of z.  The CTAs behind the first `tokens` split the rows of the core S as the dense
+// product wants them, in turn, if *dense says that it will run: work for a core that is not 2:4, nothing otherwise.
+template <int KEEP>
+__global__ void __launch_bounds__(NT) split_tokens_kernel(const float* z, int64_t cols, int64_t tokens, __half2* __restrict__ hi,
+                                                          __half2* __restrict__ lo, float* __restrict__ out_scale, const float* S, int64_t rows,
+                                                          __half2* __restrict__ s_hi, __half2* __restrict__ s_lo, float* __restrict__ s_scale,
+                                                          const int32_t* dense) {
+  grid_begin();
+  if ((int64_t)blockIdx.x < tokens) {
+    split_row<KEEP, true>(z, cols, cols, nullptr, 1.f, blockIdx.x, hi, lo, out_scale);
+    return;
+  }
+  if (*dense == 0) return;
+  // (a warp per row instead: 4096 x 4096, 400 tokens 114 -> 132 us a forward)
+  for (int64_t row = blockIdx.x - tokens; row < rows; row += gridDim.x - tokens)
+    split_row<KEEP, false>(S, cols, cols, nullptr, 1.f, row, s_hi, s_lo, s_scale);
 }
 
 // A row of the 2:4 core for the sparse tensor cores: scaled by a power of two of its own as in split_rows_kernel, two of every
-// four entries (the first two that are not zero, else whatever fills them up) as fp16 parts, their positions in the order
-// that sparse_tcgen05.cu describes.  The other two of every four make up a second layer of the same form; for a 2:4 core it holds
-// zeros, and flags[0] becomes 1 where it does not.  LAYER 0 writes the first layer, the scale and the flag, one CTA per row, KEEP
-// float4 per thread in registers as in split_rows_kernel; LAYER 1 the second layer, unless both flags say that nobody will read it (few
-// CTAs, rows in turn).  Bound by issue: 4096 x 4096, 67 MB in
+// four entries (those that are not zero, else whatever fills them up) as fp16 parts, their positions in the order
+// that sparse_tcgen05.cu describes.  *dense becomes 1 where a group holds more than two.  One CTA per row, KEEP float4 per thread in
+// registers as in split_row.  Bound by issue: 4096 x 4096, 67 MB in
 // and 36 out, 28 us (31 with the positions found by branches instead of the table, 33 with two reads of a row)
 // The two positions (lower in bits 0-1, higher in bits 2-3) for every pattern of entries that are not zero, four bits each
-constexpr unsigned long long pick24(bool rest) {
+constexpr unsigned long long pick24() {
   unsigned long long table = 0;
   for (int nz = 0; nz < 16; ++nz) {
     int pos[4] = {0, 0, 0, 0}, n = 0;
-    for (int k = 0; k < 4; ++k) if (nz >> k & 1) { pos[n] = k; ++n; }
+    for (int k = 0; k < 4 && n < 2; ++k) if (nz >> k & 1) { pos[n] = k; ++n; }
     if (n == 0) { pos[0] = 0; pos[1] = 1; }
     if (n == 1 && pos[0] < 3) pos[1] = pos[0] + 1;
     if (n == 1 && pos[0] == 3) { pos[0] = 2; pos[1] = 3; }
-    if (rest) {
-      const int taken = 1 << pos[0] | 1 << pos[1];
-      n = 0;
-      for (int k = 0; k < 4; ++k) if (!(taken >> k & 1)) { pos[n] = k; ++n; }
-    }
     table |= (unsigned long long)(pos[0] | pos[1] << 2) << 4 * nz;
   }
   return table;
 }
-constexpr unsigned long long PICK_FIRST = pick24(false), PICK_REST = pick24(true);
-template <int LAYER, int KEEP>
-__global__ void __launch_bounds__(NT) split_core24_kernel(const float* S, int64_t rows, int64_t cols, __half2* __restrict__ hi,
-                                                          __half2* __restrict__ lo, uint16_t* __restrict__ E, float* scale, int32_t* flags) {
+constexpr unsigned long long PICK24 = pick24();
+template <int KEEP>
+__global__ void __launch_bounds__(NT) split_core24_kernel(const float* S, int64_t cols, __half2* __restrict__ hi, __half2* __restrict__ lo,
+                                                          uint16_t* __restrict__ E, float* __restrict__ scale, int32_t* dense) {
   grid_begin();
-  if (LAYER == 1 && !(flags[0] | flags[1])) return;
-  const int64_t c4n = cols / 4, k_tiles = cols / 128;
-  for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    const float4* src = reinterpret_cast<const float4*>(S + row * cols);
-    float4 kept[KEEP > 0 ? KEEP : 1];
-    float p;
-    if (LAYER == 0) {
-      float mx = 0.f;
-      auto larger = [&](const float4& v) { mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
-      if (KEEP > 0) {
+  if (__syncthreads_or(threadIdx.x == 0 && __ldcg(dense) != 0)) return;        // nobody will read it
+  const int64_t row = blockIdx.x, c4n = cols / 4, k_tiles = cols / 128;
+  const float4* src = reinterpret_cast<const float4*>(S + row * cols);
+  float4 kept[KEEP > 0 ? KEEP : 1];
+  float mx = 0.f;
+  auto larger = [&](const float4& v) { mx = fmaxf(mx, fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)))); };
+  if (KEEP > 0) {
 #pragma unroll
-        for (int u = 0; u < KEEP; ++u) {
-          const int64_t i = threadIdx.x + (int64_t)u * NT;
-          kept[u] = i < c4n ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-#pragma unroll
-        for (int u = 0; u < KEEP; ++u) larger(kept[u]);
-      } else {
-        for (int64_t i = threadIdx.x; i < c4n; i += NT) larger(src[i]);
-      }
-      const int e = scale_exp(block_max(mx));
-      p = scalbnf(1.f, e);
-      if (threadIdx.x == 0) scale[row] = scalbnf(1.f, -e);
-    } else {
-      p = 1.f / scale[row];                                    // (a power of two)
+    for (int u = 0; u < KEEP; ++u) {
+      const int64_t i = threadIdx.x + (int64_t)u * NT;
+      kept[u] = i < c4n ? src[i] : make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    bool more = false;
-    const int m0 = row & 7, hf = (row >> 3) & 1, m2 = (row >> 4) & 7;
-    const int64_t mt = row >> 7;
-    auto put = [&](int64_t i, const float4& x) {               // (c4n is a multiple of 32: whole warps)
-      constexpr unsigned long long table = LAYER == 1 ? PICK_REST : PICK_FIRST;
-      const unsigned nz = (x.x != 0.f ? 1u : 0u) | (x.y != 0.f ? 2u : 0u) | (x.z != 0.f ? 4u : 0u) | (x.w != 0.f ? 8u : 0u);
-      if (LAYER == 0) more |= __popc(nz) > 2;
-      const unsigned pos = (unsigned)(table >> (4 * nz)) & 15u, i0 = pos & 3u, i1 = pos >> 2;
-      const float a = i0 == 0 ? x.x : (i0 == 1 ? x.y : x.z), b = i1 == 1 ? x.y : (i1 == 2 ? x.z : x.w);
-      __half2 h, l;
-      split2(a * p, h.x, l.x);
-      split2(b * p, h.y, l.y);
-      hi[row * (cols / 4) + i] = h;
-      lo[row * (cols / 4) + i] = l;
-      // four neighbouring groups are the 16 bits of one position word's half
-      uint32_t nib = pos << (4 * (i & 3));
-      nib |= __shfl_xor_sync(0xffffffffu, nib, 1);
-      nib |= __shfl_xor_sync(0xffffffffu, nib, 2);
-      if ((i & 3) == 0) {
-        const int64_t kt = i >> 5;                              // 32 groups to 128 columns
-        const int k2 = (int)(i >> 3) & 3, k1 = (int)(i >> 2) & 1;
-        E[2 * ((mt * k_tiles + kt) * 512 + (m0 + 8 * k1 + 16 * m2) * 4 + k2) + hf] = (uint16_t)nib;
-      }
-    };
-    if (KEEP > 0) {
 #pragma unroll
-      for (int u = 0; u < KEEP; ++u)
-        if (threadIdx.x + (int64_t)u * NT < c4n) put(threadIdx.x + (int64_t)u * NT, kept[u]);
-    } else {
-      for (int64_t i = threadIdx.x; i < c4n; i += NT) put(i, src[i]);
-    }
-    if (LAYER == 0 && more) flags[0] = 1;
+    for (int u = 0; u < KEEP; ++u) larger(kept[u]);
+  } else {
+    for (int64_t i = threadIdx.x; i < c4n; i += NT) larger(src[i]);
   }
+  const int e = scale_exp(block_max(mx));
+  const float p = scalbnf(1.f, e);
+  if (threadIdx.x == 0) scale[row] = scalbnf(1.f, -e);
+  bool more = false;
+  const int m0 = row & 7, hf = (row >> 3) & 1, m2 = (row >> 4) & 7;
+  const int64_t mt = row >> 7;
+  auto put = [&](int64_t i, const float4& x) {               // (c4n is a multiple of 32: whole warps)
+    const unsigned nz = (x.x != 0.f ? 1u : 0u) | (x.y != 0.f ? 2u : 0u) | (x.z != 0.f ? 4u : 0u) | (x.w != 0.f ? 8u : 0u);
+    more |= __popc(nz) > 2;
+    const unsigned pos = (unsigned)(PICK24 >> (4 * nz)) & 15u, i0 = pos & 3u, i1 = pos >> 2;
+    const float a = i0 == 0 ? x.x : (i0 == 1 ? x.y : x.z), b = i1 == 1 ? x.y : (i1 == 2 ? x.z : x.w);
+    __half2 h, l;
+    split2(a * p, h.x, l.x);
+    split2(b * p, h.y, l.y);
+    hi[row * (cols / 4) + i] = h;
+    lo[row * (cols / 4) + i] = l;
+    // four neighbouring groups are the 16 bits of one position word's half
+    uint32_t nib = pos << (4 * (i & 3));
+    nib |= __shfl_xor_sync(0xffffffffu, nib, 1);
+    nib |= __shfl_xor_sync(0xffffffffu, nib, 2);
+    if ((i & 3) == 0) {
+      const int64_t kt = i >> 5;                              // 32 groups to 128 columns
+      const int k2 = (int)(i >> 3) & 3, k1 = (int)(i >> 2) & 1;
+      E[2 * ((mt * k_tiles + kt) * 512 + (m0 + 8 * k1 + 16 * m2) * 4 + k2) + hf] = (uint16_t)nib;
+    }
+  };
+  if (KEEP > 0) {
+#pragma unroll
+    for (int u = 0; u < KEEP; ++u)
+      if (threadIdx.x + (int64_t)u * NT < c4n) put(threadIdx.x + (int64_t)u * NT, kept[u]);
+  } else {
+    for (int64_t i = threadIdx.x; i < c4n; i += NT) put(i, src[i]);
+  }
+  // (one store a CTA: with one from every thread that found a group a core of nothing else took 296 us)
+  if (__syncthreads_or(more) && threadIdx.x == 0) atomicOr(dense, 1);
 }
 
 __device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
@@ -388,40 +400,44 @@ void launch_f16_prepare_H(armor_ctx* c, const float* H, cudaStream_t s) {
   c->launches += 2;
 }
 
-namespace {
-template <int KEEP>
-void split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t rows, int64_t cols, const float* colscale, float post, __half2* h, __half2* l,
-                float* out_scale, int32_t* not_finite, cudaStream_t s) {
-  if (not_finite)
-    launch_dependent(split_rows_kernel<KEEP, true>, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale, not_finite);
-  else
-    launch_dependent(split_rows_kernel<KEEP, false>, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale, not_finite);
-}
-}  // namespace
-
 void launch_f16_split_rows(armor_ctx* c, const float* in, int64_t ld, int64_t rows, int64_t cols, const float* colscale,
-                           float post, void* hi, void* lo, float* out_scale, cudaStream_t s, int32_t* not_finite) {
+                           float post, void* hi, void* lo, float* out_scale, cudaStream_t s) {
   KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 8.0 * (double)rows * (double)cols, s);
   __half2 *h = static_cast<__half2*>(hi), *l = static_cast<__half2*>(lo);
+  auto launch = [&](auto kernel) { launch_dependent(kernel, (unsigned)rows, NT, 0, s, in, ld, cols, colscale, post, h, l, out_scale); };
   // a row in registers up to 8,192 columns: one read of it instead of two (from L1 or L2)
-  if (cols <= 4 * NT) split_rows<1>(c, in, ld, rows, cols, colscale, post, h, l, out_scale, not_finite, s);
-  else if (cols <= 16 * NT) split_rows<4>(c, in, ld, rows, cols, colscale, post, h, l, out_scale, not_finite, s);
-  else if (cols <= 32 * NT) split_rows<8>(c, in, ld, rows, cols, colscale, post, h, l, out_scale, not_finite, s);
-  else split_rows<0>(c, in, ld, rows, cols, colscale, post, h, l, out_scale, not_finite, s);
+  if (cols <= 4 * NT) launch(split_rows_kernel<1>);
+  else if (cols <= 16 * NT) launch(split_rows_kernel<4>);
+  else if (cols <= 32 * NT) launch(split_rows_kernel<8>);
+  else launch(split_rows_kernel<0>);
   c->launches++;
 }
 
-void launch_split_core24(armor_ctx* c, const float* S, int layer, void* hi, void* lo, void* E, float* scale, int32_t* flags, cudaStream_t s) {
+void launch_split_tokens(armor_ctx* c, const float* z, int64_t tokens, void* hi, void* lo, float* out_scale, const float* S, void* s_hi, void* s_lo,
+                         float* s_scale, const int32_t* dense, cudaStream_t s) {
   const int64_t rows = c->d_out, cols = c->d_in;
-  KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, layer ? 0.0 : 6.125 * (double)c->wn, s);
-  __half2* h = reinterpret_cast<__half2*>(hi) + (layer ? c->wn / 4 : 0);
-  __half2* l = reinterpret_cast<__half2*>(lo) + (layer ? c->wn / 4 : 0);
-  uint16_t* e = static_cast<uint16_t*>(E) + (layer ? c->wn / 16 : 0);
-  if (layer == 0 && cols <= 4 * NT) launch_dependent(split_core24_kernel<0, 1>, (unsigned)rows, NT, 0, s, S, rows, cols, h, l, e, scale, flags);
-  else if (layer == 0 && cols <= 16 * NT) launch_dependent(split_core24_kernel<0, 4>, (unsigned)rows, NT, 0, s, S, rows, cols, h, l, e, scale, flags);
-  else if (layer == 0 && cols <= 32 * NT) launch_dependent(split_core24_kernel<0, 8>, (unsigned)rows, NT, 0, s, S, rows, cols, h, l, e, scale, flags);
-  else if (layer == 0) launch_dependent(split_core24_kernel<0, 0>, (unsigned)rows, NT, 0, s, S, rows, cols, h, l, e, scale, flags);
-  else launch_dependent(split_core24_kernel<1, 0>, (unsigned)(rows < 4 * c->n_sm ? rows : 4 * c->n_sm), NT, 0, s, S, rows, cols, h, l, e, scale, flags);
+  const int64_t more = !S ? 0 : (rows < 8 * c->n_sm ? rows : 8 * c->n_sm);
+  KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 8.0 * (double)tokens * (double)cols, s);
+  __half2 *h = static_cast<__half2*>(hi), *l = static_cast<__half2*>(lo), *sh = static_cast<__half2*>(s_hi), *sl = static_cast<__half2*>(s_lo);
+  auto launch = [&](auto kernel) {
+    launch_dependent(kernel, (unsigned)(tokens + more), NT, 0, s, z, cols, tokens, h, l, out_scale, S, rows, sh, sl, s_scale, dense);
+  };
+  if (cols <= 4 * NT) launch(split_tokens_kernel<1>);
+  else if (cols <= 16 * NT) launch(split_tokens_kernel<4>);
+  else if (cols <= 32 * NT) launch(split_tokens_kernel<8>);
+  else launch(split_tokens_kernel<0>);
+  c->launches++;
+}
+
+void launch_split_core24(armor_ctx* c, const float* S, void* hi, void* lo, void* E, float* scale, int32_t* dense, cudaStream_t s) {
+  const int64_t cols = c->d_in;
+  KTimer kt(c, ARMOR_KC_OPERAND_SPLIT, 6.125 * (double)c->wn, s);
+  __half2 *h = static_cast<__half2*>(hi), *l = static_cast<__half2*>(lo);
+  auto launch = [&](auto kernel) { launch_dependent(kernel, (unsigned)c->d_out, NT, 0, s, S, cols, h, l, static_cast<uint16_t*>(E), scale, dense); };
+  if (cols <= 4 * NT) launch(split_core24_kernel<1>);
+  else if (cols <= 16 * NT) launch(split_core24_kernel<4>);
+  else if (cols <= 32 * NT) launch(split_core24_kernel<8>);
+  else launch(split_core24_kernel<0>);
   c->launches++;
 }
 

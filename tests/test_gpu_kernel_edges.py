@@ -610,9 +610,9 @@ def test_left_solves_of_256_in_several_slices_a_cta(nb_in):
                                                       (128, 256, 128, 5000), (4096, 2048, 128, 295)])
 @pytest.mark.parametrize("core", ["2of4", "any"])
 def test_fp32_forward_on_the_sparse_tensor_cores(d_out, d_in, d_block, tokens, core):
-    """The core product of many tokens runs on the sparse tensor cores whatever the core holds: rows of one K tile to several
+    """The core product of many tokens runs on the sparse tensor cores: rows of one K tile to several
     segments, ragged tiles of tokens, a second chunk, and the dense product where rows do not come in 256 or tokens are few.  "any": groups
-    with every pattern of entries, two layers.  Truncating additions, 48 in either wrapper product and 96 in a segment of the core's, of up to
+    with every pattern of entries, the dense product again.  Truncating additions, 48 in either wrapper product and 96 in a segment of the core's, of up to
     2^-24: 1.2e-5 of the result.  One token that is not finite spoils its own row and no other."""
     g = _gen(d_out + d_in + tokens)
     ctx = _ctx(d_out, d_in, d_block)
@@ -639,4 +639,49 @@ def test_fp32_forward_on_the_sparse_tensor_cores(d_out, d_in, d_block, tokens, c
     assert (yi[others] - y[others]).norm() <= 1e-6 * y.norm()
     x[tokens - 2, 5] = 0.0
     assert torch.isfinite(ctx.apply(st, x)).all()
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block,tokens", [(256, 128, 128, 4800), (256, 256, 256, 4737), (512, 512, 128, 16384 + 70)])
+@pytest.mark.parametrize("at", [0, -1])
+def test_fp32_forward_of_a_core_with_one_group_that_is_not_2_of_4(d_out, d_in, d_block, tokens, at):
+    """One group of three entries, in the first or the last row, sends the call to the dense product: the bits of calls of 2,000 tokens,
+    which run there anyway (up to 1,024 columns a sum is one segment however the call is cut).  The call after it is sparse again."""
+    g = _gen(d_out + d_in)
+    ctx = _ctx(d_out, d_in, d_block)
+    from paper_2510_05528_b200 import binding as Bd
+    A = torch.randn(d_out // d_block, d_block, d_block, device=DEV, generator=g)
+    B = torch.randn(d_in // d_block, d_block, d_block, device=DEV, generator=g)
+    W = torch.randn(d_out, d_in // 4, 4, device=DEV, generator=g)
+    W[:, :, 2:] = 0.0
+    x = torch.randn(tokens, d_in, device=DEV, generator=g)
+    st = Bd.LayerState(Wbar=W.view(d_out, d_in), A=A, B=B, S=W.view(d_out, d_in), M=torch.zeros(d_out, d_in // 4, dtype=torch.uint8, device=DEV))
+    sparse = ctx.apply(st, x)
+    W[at, at, 3] = 1.0
+    assert torch.equal(ctx.apply(st, x), torch.cat([ctx.apply(st, t) for t in x.split(2000)]))
+    W[at, at, 3] = 0.0
+    assert torch.equal(ctx.apply(st, x), sparse)
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_in", [128, 1152, 4224, 8320])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_fp32_forward_with_tokens_that_are_not_finite(d_in, bad):
+    """Rows of every form of the split: a token that is not finite comes out as NaN throughout, the others keep their bits."""
+    g = _gen(d_in)
+    ctx = _ctx(256, d_in, 128)
+    from paper_2510_05528_b200 import binding as Bd
+    W = torch.randn(256, d_in // 4, 4, device=DEV, generator=g)
+    W[:, :, 1:3] = 0.0
+    st = Bd.LayerState(Wbar=W.view(256, d_in), A=torch.randn(2, 128, 128, device=DEV, generator=g), B=torch.randn(d_in // 128, 128, 128, device=DEV, generator=g),
+                       S=W.view(256, d_in), M=torch.zeros(256, d_in // 4, dtype=torch.uint8, device=DEV))
+    x = torch.randn(4800, d_in, device=DEV, generator=g)
+    y = ctx.apply(st, x)
+    spoiled = [0, 223, 4799]
+    x[spoiled, d_in - 1] = bad
+    yi = ctx.apply(st, x)
+    assert torch.isnan(yi[spoiled]).all()
+    rest = torch.ones(4800, dtype=torch.bool, device=DEV)
+    rest[spoiled] = False
+    assert torch.equal(yi[rest], y[rest])
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
