@@ -982,10 +982,14 @@ armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E,
   // piece to be written and added: one CTA an SM, one SM in twelve with two, while that leaves a CTA about eight k tiles (4096 x
   // 4096, 256 -> 160 CTAs: 1 token 8.98 -> 8.2 us, 64 10.9 -> 9.3; 2048 x 2048, 256 -> 128: 7.7 -> 6.5 and 10.4 -> 7.8; beyond 64
   // tokens, two stages a CTA: five k tiles), and no fewer k tiles than make those two costs alike (512 x 8192, 64 -> 13 pieces:
-  // 14.3 -> 8.2 us).
+  // 14.3 -> 8.2 us).  From 40 row tiles on fewer pieces are worth their longer chains only where the pieces are large, from 25 tokens
+  // on (6144 x 2048, two CTAs an SM and one: 1 token 7.7 and 8.0 us, 17 9.1 and 9.7, 64 9.7 and 8.8; 5120 x 2560, 8 tokens 7.8 and 8.2,
+  // 64 10.3 and 9.4).  Below 40 the one size seen to lose is 4096 x 2048, 1 token: 7.2 and 7.4.  The twelfth is for 32 row tiles (five
+  // pieces; four of them, 128 CTAs, 8.7 us for 1 token at 4096 x 4096); 20 row tiles do without (2560 x 5120, 1 token 8.5, with seven pieces
+  // for eight 8.2).
   int want = 2 * c->n_sm / (p.m_tiles * p.n_tiles);
   const int one_an_sm = (c->n_sm + c->n_sm / 12) / (p.m_tiles * p.n_tiles);
-  const bool small = one_an_sm >= 2 && (int64_t)p.m_tiles * p.n_tiles * p.k_tiles <= (int64_t)(n <= 64 ? 8 : 5) * c->n_sm;
+  const bool small = one_an_sm >= 2 && (n > 24 || p.m_tiles < 40) && (int64_t)p.m_tiles * p.n_tiles * p.k_tiles <= (int64_t)(n <= 64 ? 8 : 5) * c->n_sm;
   if (small) want = one_an_sm;
   if (want < 1) want = 1;
   if (want > p.k_tiles) want = p.k_tiles;
