@@ -126,7 +126,9 @@ armor_status armor_workspace_bytes(const armor_config* cfg, size_t* bytes);
 /* Creates a context over caller-owned device scratch (256-byte aligned, at
  * least armor_workspace_bytes).  The context holds the configuration and the
  * carve-up of the workspace only, plus two non-blocking streams and a few events of its own (graph capture of the
- * iterations, staging of the Gram).  Must be called with the device current. */
+ * iterations; staging of the Gram and a branch of every iteration, which is joined
+ * again before the call returns and becomes a branch of the caller's graph where the
+ * caller captures).  Must be called with the device current. */
 armor_status armor_create(armor_ctx** ctx, const armor_config* cfg, void* d_workspace, size_t bytes);
 armor_status armor_destroy(armor_ctx* ctx);
 

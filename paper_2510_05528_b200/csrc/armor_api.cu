@@ -512,8 +512,18 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
     armor_status st = ARMOR_OK;
     // What the group solves need of A and B (B_j H_jj, alpha_r, the diagonal blocks of K_j): small products that leave most of
     // the memory's rate unused, formed on the side stream while the update of the core runs (4096 x 4096: 17 us an iteration, behind
-    // one another in the stream).  Not while launches are timed or captured in pieces.
-    bool prepared = false;
+    // one another in the stream).  Not while launches are timed or captured in pieces.  Whatever way the iteration ends, `s` goes on behind
+    // the side stream: a capture is not left with an open branch, nor work in flight behind an error.
+    struct Aside {
+      armor_ctx* c; cudaStream_t s; bool open;
+      armor_status join() {
+        open = false;
+        ARMOR_CUDA_OK(cudaEventRecord(c->ev_prepared, c->side_stream));
+        ARMOR_CUDA_OK(cudaStreamWaitEvent(s, c->ev_prepared, 0));
+        return ARMOR_OK;
+      }
+      ~Aside() { if (open) (void)join(); }
+    } aside{c, s, false};
     const bool fork = (ph & ARMOR_PHASE_MASK) && c->side_stream && c->timing_on == 0;
     auto prepare_solves = [&](LaunchStream q) {
       block_mm(c, B, false, c->Hjj, false, c->Ktmp, nbi, q);                         // B_j H_jj
@@ -523,9 +533,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       if (!fork) return ARMOR_OK;
       ARMOR_CUDA_OK(cudaEventRecord(c->ev_prep, s));
       ARMOR_CUDA_OK(cudaStreamWaitEvent(c->side_stream, c->ev_prep, 0));
+      aside.open = true;
       prepare_solves(LaunchStream(c->side_stream, true));
-      ARMOR_CUDA_OK(cudaEventRecord(c->ev_prepared, c->side_stream));
-      prepared = true;
       return ARMOR_OK;
     };
     launch_zero_scalars(c, !first, !fresh_loss, is, s);      // with a carried loss this also opens the iteration's record
@@ -694,7 +703,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
 
     // ---- sparse-core update (Algorithm 3), mask_sweeps times ------------------------------------
     if (ph & ARMOR_PHASE_MASK) {
-      if (!prepared) prepare_solves(s);
+      if (!aside.open) prepare_solves(s);
       for (int sw = 0; sw < sweeps; ++sw) {
         if (sw > 0) {
           // E H_w for the state the previous run left
@@ -714,8 +723,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
           core_gradient(c, A, B, s);
         }
         eh = Moves{};                                                                // (another sweep starts from E H_w formed afresh)
-        const bool join = prepared && sw == 0;
-        if (join) ARMOR_CUDA_OK(cudaStreamWaitEvent(s, c->ev_prepared, 0));
+        const bool join = aside.open;
+        if (join && (st = aside.join()) != ARMOR_OK) return st;
         launch_mask_select(c, A, B, c->Gam, S, M, (uint64_t)(t_first * sweeps + sw), (uint64_t)sweeps, LaunchStream(s, join));   // counter (t_first + it) K + k
         launch_mask_quadratic(c, A, B, H, is, s);                                    // accepted or not
         launch_mask_commit(c, S, M, carry_P ? c->P : nullptr, is, s);                // if accepted: S, M and P += dS B H_w

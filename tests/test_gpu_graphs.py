@@ -72,6 +72,41 @@ def test_a_captured_call_and_timing_fall_back_to_direct_launches():
     assert t["gemm"][0] >= 2 * 6 and t["block_product"][0] > 0 and t["cholesky"][0] == 2 * 6 + 1
 
 
+@pytest.mark.parametrize("mode", ["full-exact", "full-adam", "full-2-sweeps", "diag-exact", "diag-adam"])
+@pytest.mark.parametrize("cfg,prec", [(TINY, Bd.PREC_SIMT), (MID, Bd.PREC_FP16X3)], ids=["tiny-simt", "mid-fp16x3"])
+def test_a_call_in_a_callers_graph_is_bit_identical_to_direct_launches(cfg, prec, mode):
+    """A call captured by its caller: the branch on the context's side stream becomes part of the caller's graph and is joined again,
+    so the capture ends, every replay gives what direct launches give, and the context works on afterwards."""
+    W = inputs.make_weight(cfg)
+    Hd, Wd = dev(O.gram(inputs.make_activations(cfg)).astype(np.float32)), dev(W)
+    ctx = make(cfg, prec, **MODES[mode])
+    Bd.armor_use_graphs(ctx.ctx, False)
+    st = ctx.init(Wd, Hd)
+    fresh = [t.clone() for t in (st.A, st.B, st.S, st.M)]
+    stats = ctx.read_stats(ctx.bcd_step(st, Hd, 0, 5)).copy()
+    ref = [t.clone() for t in (st.A, st.B, st.S, st.M)]
+    assert stats["loss_mask"][-1] < stats["loss_start"][0]
+
+    def back():
+        for t, f in zip((st.A, st.B, st.S, st.M), fresh):
+            t.copy_(f)
+
+    back()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=torch.cuda.Stream()):
+        records = ctx.bcd_step(st, Hd, 0, 5)
+    for _ in range(2):
+        back()
+        g.replay()
+        assert all(torch.equal(t, r) for t, r in zip((st.A, st.B, st.S, st.M), ref))
+        assert ctx.read_stats(records).tobytes() == stats.tobytes()
+    back()
+    assert ctx.read_stats(ctx.bcd_step(st, Hd, 0, 5)).tobytes() == stats.tobytes()
+    assert all(torch.equal(t, r) for t, r in zip((st.A, st.B, st.S, st.M), ref))
+    assert ctx.device_status()[:4] == [0, 0, 0, 0]
+
+
 @pytest.mark.parametrize("mode", ["full-exact", "full-adam", "full-2-sweeps", "diag-exact"])
 def test_replay_in_pieces_around_timed_products_is_bit_identical(mode):
     """With events around the dense products only, the iteration is replayed as graph pieces with the products launched
