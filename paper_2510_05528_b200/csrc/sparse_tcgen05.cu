@@ -984,7 +984,8 @@ armor_status launch_tc_sparse_small(armor_ctx* c, const void* Sc, const void* E,
   // tokens, two stages a CTA: five k tiles), and no fewer k tiles than make those two costs alike (512 x 8192, 64 -> 13 pieces:
   // 14.3 -> 8.2 us).  From 40 row tiles on fewer pieces are worth their longer chains only where the pieces are large, from 25 tokens
   // on (6144 x 2048, two CTAs an SM and one: 1 token 7.7 and 8.0 us, 17 9.1 and 9.7, 64 9.7 and 8.8; 5120 x 2560, 8 tokens 7.8 and 8.2,
-  // 64 10.3 and 9.4).  Below 40 the one size seen to lose is 4096 x 2048, 1 token: 7.2 and 7.4.  The twelfth is for 32 row tiles (five
+  // 64 10.3 and 9.4; 7168 x 2048 in blocks of 256 33 10.6 and 10.9, 64 11.7 and 10.7).  Below 40 the one size seen to lose is 4096 x 2048, 1
+  // token: 7.2 and 7.4.  The twelfth is for 32 row tiles (five
   // pieces; four of them, 128 CTAs, 8.7 us for 1 token at 4096 x 4096); 20 row tiles do without (2560 x 5120, 1 token 8.5, with seven pieces
   // for eight 8.2).
   int want = 2 * c->n_sm / (p.m_tiles * p.n_tiles);
