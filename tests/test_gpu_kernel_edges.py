@@ -133,6 +133,41 @@ def test_wrapper_products_of_the_packed_forward(d_out, d_in, d_block, tokens):
     assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
 
 
+@pytest.mark.parametrize("d_out,d_in,d_block,tokens", [
+    (4096, 2048, 128, (1024, 1025, 1152, 1153, 1441, 1729, 2016, 2017)),   # one row tile, two by 128, 160, 192, 224 tokens, one
+    (2560, 2304, 256, (1793, 2000, 2241)),         # an odd number of groups of rows; 160 and 192 tokens
+    (5120, 2048, 128, (769, 1345, 1568)),
+])
+def test_packed_core_with_fp32_wrappers_at_every_width_of_a_tile(d_out, d_in, d_block, tokens):
+    """The core product on the sparse tensor cores with its output in fp32, one and two row tiles to a stage's tokens, ragged.  Integers
+    small enough for the wrappers' one tf32 pass (11 bits) and every sum: the outputs are the oracle's, rows past the last are not written."""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + d_in)
+    ctx = _ctx(d_out, d_in, d_block)
+
+    def turned(n):
+        # one entry in every row and column of a block, -2 .. 2 without 0
+        v = (torch.randint(1, 3, (n // d_block, d_block), device=DEV, generator=g) * (2 * torch.randint(0, 2, (n // d_block, d_block), device=DEV, generator=g) - 1)).float()
+        at = torch.rand(n // d_block, d_block, device=DEV, generator=g).argsort(1)
+        return torch.zeros(n // d_block, d_block, d_block, device=DEV).scatter_(2, at[:, :, None], v[:, :, None])
+    grp = torch.randint(-1, 2, (d_out, d_in // 4, 4), device=DEV, generator=g).float()
+    keep = torch.zeros_like(grp, dtype=torch.bool).scatter_(2, torch.rand(grp.shape, device=DEV, generator=g).topk(2, 2).indices, True)
+    S = (grp * keep).view(d_out, d_in)
+    M = (keep * torch.tensor([1, 2, 4, 8], device=DEV)).sum(2).to(torch.uint8)
+    st = Bd.LayerState(Wbar=S, A=turned(d_out), B=turned(d_in), S=S, M=M)
+    packed = ctx.pack_core(st)
+    for n in tokens:
+        x = (torch.randint(-1, 2, (n, d_in), device=DEV, generator=g) * (torch.rand(n, d_in, device=DEV, generator=g) < 0.2)).to(torch.bfloat16)
+        z = torch.einsum("tjk,jmk->tjm", x.double().view(n, -1, d_block), st.B.double()).reshape(n, d_in) @ S.double().t()
+        assert z.abs().max() < 2048
+        y = torch.einsum("tjk,jmk->tjm", z.view(n, -1, d_block), st.A.double()).reshape(n, d_out).float().to(torch.bfloat16)
+        out = torch.full((n + 40, d_out), 7.0, dtype=torch.bfloat16, device=DEV)
+        Bd.armor_apply_packed(ctx.ctx, st.A, st.B, packed, None, None, x, out[:n])
+        assert torch.equal(out[:n], y), n
+        assert (out[n:] == 7.0).all(), n
+    assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
+
+
 @pytest.mark.parametrize("d_out,d_in,d_block", [(32, 64, 32), (96, 256, 32), (256, 256, 32), (320, 128, 64), (120, 200, 8),
                                                 (48, 144, 16), (1024, 512, 64), (160, 96, 32)])
 @pytest.mark.parametrize("side", [0, 1])
