@@ -909,7 +909,7 @@ void launch_compress_24(armor_ctx* c, const float* S, const uint8_t* M, void* Sc
   c->launches++;
 }
 
-// Z2[n][d_out] = Z1[n][d_in] * S^T with S given compressed (Sc, E); Z1 bf16; Z2 fp32, or bf16 if out_bf16.
+// The product on pairs of CTAs, MT row tiles of 256 to a stage's tokens, tiles of tile_n tokens
 template <int MT>
 static armor_status launch_pairs(armor_ctx* c, const CUtensorMap& mA, const void* z1, const CUtensorMap& mE, SParams p, int tile_n, cudaStream_t s) {
   CUtensorMap mB;
@@ -925,27 +925,24 @@ static armor_status launch_pairs(armor_ctx* c, const CUtensorMap& mA, const void
   return cudaGetLastError() == cudaSuccess ? ARMOR_OK : ARMOR_ERR_CUDA;
 }
 
+// Z2[n][d_out] = Z1[n][d_in] * S^T with S given compressed (Sc, E); Z1 bf16; Z2 fp32, or bf16 if out_bf16.
 armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const void* z1_bf16, void* z2, bool out_bf16,
                               int64_t n, cudaStream_t s) {
   if (!tc_sparse_ok(c) || n <= 0) return ARMOR_ERR_UNSUPPORTED;
-  CUtensorMap mA, mB, mE;
+  CUtensorMap mA, mE;
   if (!make_map_bf16(&mA, Sc, c->d_out, c->d_in / 2, c->d_in / 2)) return ARMOR_ERR_CUDA;
-  if (!make_map_bf16(&mB, z1_bf16, n, c->d_in, c->d_in)) return ARMOR_ERR_CUDA;
   if (!make_map_e(&mE, E, (c->d_out / 128) * (c->d_in / 128) * 128)) return ARMOR_ERR_CUDA;
   SParams p{};
   p.Z = out_bf16 ? nullptr : static_cast<float*>(z2); p.Zb = out_bf16 ? static_cast<__nv_bfloat16*>(z2) : nullptr;
   p.ldz = c->d_out; p.M = c->d_out; p.N = n; p.K = c->d_in;
   p.m_tiles = (int)(c->d_out / BM); p.n_tiles = (int)((n + BN - 1) / BN); p.k_tiles = (int)(c->d_in / BKL);
   p.status = c->status;
-  constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024;
-  static PerDeviceOnce attr;
-  if (ensure_dynamic_smem(attr, c->device, tc_sparse_kernel, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
   const int n_sm = c->n_sm;
   KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)p.M * (double)p.N * (double)p.K, s);   // dense-equivalent flops
   if (g_sparse_pairs && c->d_out % 256 == 0 && n_sm >= 2) {
-    // Two row tiles at a time, or one: rounds of the pairs times what a tile takes, its tokens plus, with two, 200 tokens' worth (fp32 out:
-    // 240, 14336 x 2048, 1,459 tokens, 3 rounds or 5, 161 us and 154; a tile
-    // of 512 x 224 takes 1.62 times one of 256 x 256, of 512 x 192 1.48 times).  Whole forwards, one and two: 28672 x 8192, 4,096 tokens
+    // Two row tiles at a time, or one: rounds of the pairs times what a tile takes, its tokens plus, with two, 200 tokens' worth (a tile
+    // of 512 x 224 takes 1.62 times one of 256 x 256, of 512 x 192 1.48 times), 240 with the output in fp32: 14336 x 2048, 1,459 tokens, 3
+    // rounds of two or 5 of one, 149 us and 144 a forward with fp32 wrappers.  Whole forwards, one and two: 28672 x 8192, 4,096 tokens
     // (25 rounds and 15) 1,192 and 1,123 us; 8192 x 8192, 640 (2 and 1) 76.5 and 63.2, 2,000 (4 and 2) 156 and 139; 4096 x 4096, 4,096
     // (4 and 3) 93 and 107: one.
     int width = 256;
@@ -960,6 +957,11 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
     if (width < 256) return launch_pairs<2>(c, mA, z1_bf16, mE, p, width, s);
     return launch_pairs<1>(c, mA, z1_bf16, mE, p, 256, s);
   } else {
+    CUtensorMap mB;
+    if (!make_map_bf16(&mB, z1_bf16, n, c->d_in, c->d_in)) return ARMOR_ERR_CUDA;
+    constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024;
+    static PerDeviceOnce attr;
+    if (ensure_dynamic_smem(attr, c->device, tc_sparse_kernel, SMEM) != ARMOR_OK) return ARMOR_ERR_CUDA;
     const int tiles = p.m_tiles * p.n_tiles;
     const int grid = tiles < n_sm ? tiles : n_sm;
     tc_sparse_kernel<<<grid, NTHREADS, SMEM, s>>>(mA, mB, mE, p);
