@@ -647,8 +647,8 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       else if (late_A)
         launch_stage(c, is, 10, c->partblk, DELTA_PARTS * nbi, s, c->partials, nq, SC_Q_B, c->partA, n_part_A, SC_DEC_A);
       else launch_stage(c, is, 2, c->partblk, DELTA_PARTS * nbi, s, c->partials, nq, SC_Q_B);
-      // B += tau Delta, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch.  (With a core step P moves
-      // there by both steps: nothing reads it in between.)
+      // B += tau Delta, EH -= tau V H_w unless that is left to the gradients (late_EH) and, where T H_w is carried, P += tau R H_w: one
+      // launch.  (With a core step P moves there by both steps: nothing reads it in between.)
       if (late_EH) eh.add(VH, SC_TAU_B);
       launch_axpy_multi(c, late_EH ? nullptr : c->EH, VH, -1.f, c->wn, carry_P && !late_P ? c->P : nullptr, c->E, 1.f, c->wn, B, c->Delta, 1.f,
                         (int64_t)nbi * db * db, SC_TAU_B, s);
@@ -693,7 +693,7 @@ armor_status armor_bcd_step(armor_ctx* c, const float* W, const float* H, float*
       }
       launch_stage(c, is, beta_step ? 6 : 3, nullptr, 0, s, beta_step ? nullptr : c->partials, nq, SC_Q_S, nrm_part, n_nrm, SC_NRM_S);
       if ((st = prepare_aside()) != ARMOR_OK) return st;
-      // S += tau Gamma_M, EH -= tau V H_w and, where T H_w is carried, P += tau R H_w: one launch
+      // S += tau Gamma_M, EH -= tau V H_w unless that is left to the gradient and, where T H_w is carried, P += tau R H_w: one launch
       if (late_EH) eh.add(c->VH, SC_TAU_S);
       launch_axpy_multi(c, S, c->U, 1.f, c->wn, late_EH ? nullptr : c->EH, c->VH, -1.f, c->wn, carry_P ? c->P : nullptr, RH, 1.f, c->wn, SC_TAU_S, s,
                         late_P ? c->E : nullptr, SC_TAU_B);

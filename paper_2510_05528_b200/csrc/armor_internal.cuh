@@ -306,7 +306,6 @@ armor_status tc_blockres_left(armor_ctx* c, const float* Ablk, bool transA, cons
                               double* part = nullptr);
 
 armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s);
-armor_status tc_blockres_thin(armor_ctx* c, const float* Z, const float* X, float* out, int n, int pad, int blocks, int64_t cols, cudaStream_t s);
 armor_status tc_blockres_left_dual(armor_ctx* c, const float* Ablk, const float* in1, const float* in2, float* out,
                                    int64_t rows, int64_t cols, double* part, int* n_part, cudaStream_t s, const float* colw = nullptr);
 
@@ -462,7 +461,6 @@ armor_status launch_chol(armor_ctx* c, int mode, const float* Gmat, const float*
                          float* A, int nb, double* part, cudaStream_t s);
 
 // sparse-core update (kernels_mask.cu)
-void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s);
 // alpha and the m x m diagonal blocks of K_j = Y_j B_j^T (Y = B_j H_jj, [nbi, db, db]) in one launch
 void launch_mask_prep(armor_ctx* c, const float* A, const float* B, const float* Y, cudaStream_t s);
 // selection counter t = t_base + t_mul * (*c->it_dev); with one draw per block also the vectors of launch_mask_quadratic

@@ -90,10 +90,6 @@ __device__ __forceinline__ uint64_t op_desc(uint32_t base, int mn) {
   return mn ? smem_desc_mn_sw128_32b(base, 4096, 512) : smem_desc_sw128(base, 16, 1024);
 }
 
-__device__ __forceinline__ float4 low4(const float4 v) {
-  return make_float4(v.x - __uint_as_float(__float_as_uint(v.x) & 0xffffe000u), v.y - __uint_as_float(__float_as_uint(v.y) & 0xffffe000u),
-                     v.z - __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), v.w - __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
-}
 // (a step of zero leaves x as it is, whatever v holds, as the update kernels do)
 __device__ __forceinline__ float4 moved(float a, const float4 v, const float4 x) {
   return a == 0.f ? x : make_float4(fmaf(a, v.x, x.x), fmaf(a, v.y, x.y), fmaf(a, v.z, x.z), fmaf(a, v.w, x.w));

@@ -90,12 +90,6 @@ __device__ __forceinline__ bool next_unit(int& item, int i1, int tiles, Unit& u)
   return true;
 }
 
-// x - trunc_tf32(x)
-__device__ __forceinline__ float4 low4(const float4 v) {
-  return make_float4(v.x - __uint_as_float(__float_as_uint(v.x) & 0xffffe000u), v.y - __uint_as_float(__float_as_uint(v.y) & 0xffffe000u),
-                     v.z - __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), v.w - __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
-}
-
 __device__ __forceinline__ uint64_t x_desc(uint32_t base, int mn_major, int kstep) {
   return mn_major ? smem_desc_mn_sw128_32b(base + kstep * 1024, 4096, 512) : smem_desc_sw128(base + kstep * 32, 16, 1024);
 }

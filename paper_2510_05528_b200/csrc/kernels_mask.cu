@@ -23,29 +23,6 @@ __device__ __forceinline__ float neg_log_uniform(uint32_t k24) {
   return -log1pf(-(float)(2u * ((1u << 24) - k24) - 1u) * 2.98023223876953125e-8f);
 }
 
-// alpha[r] = || A[:, r] ||^2 : column r of the block that owns row r of the core.
-// blockDim = (32 columns, 8 row slices); grid = (nbo, db / 32).
-__global__ void alpha_kernel(const float* A, float* __restrict__ alpha, int db) {
-  grid_begin();
-  const int i = blockIdx.x;
-  const int r = blockIdx.y * 32 + threadIdx.x;
-  const float* Ai = A + (int64_t)i * db * db;
-  double acc = 0.0;
-  if (r < db)
-    for (int o = threadIdx.y; o < db; o += 8) {
-      const double v = Ai[(int64_t)o * db + r];
-      acc += v * v;
-    }
-  __shared__ double part[8][33];
-  part[threadIdx.y][threadIdx.x] = acc;
-  __syncthreads();
-  if (threadIdx.y == 0 && r < db) {
-    double t = 0.0;
-    for (int k = 0; k < 8; ++k) t += part[k][threadIdx.x];
-    alpha[i * db + r] = (float)t;
-  }
-}
-
 // 2x2 PSD solve with the pseudo-inverse rule: w = K^+ z, red = z^T K^+ z.
 __device__ __forceinline__ void pinv2(double k11, double k12, double k22, double z1, double z2, double& w1,
                                       double& w2, double& red) {
@@ -570,13 +547,7 @@ __global__ void __launch_bounds__(NT) mask_carry_kernel(const SelRec* sel, const
 
 }  // namespace
 
-void launch_alpha(armor_ctx* c, const float* A, cudaStream_t s) {
-  KTimer kt(c, ARMOR_KC_MASK_GUARD, 0.0, s);
-  launch_dependent(alpha_kernel, dim3(c->nbo, (c->db + 31) / 32), dim3(32, 8), 0, s, A, c->alpha, c->db);
-  c->launches++;
-}
-
-// alpha (column norms of the blocks of A) and the m x m diagonal blocks of K_j = (B_j H_jj) B_j^T, the only entries
+// alpha (alpha[r] = || A[:, r] ||^2, column r of the block that owns row r of the core) and the m x m diagonal blocks of K_j = (B_j H_jj) B_j^T, the only entries
 // of K_j the group solves read (Appendix B.1: B' D B'^T for the m rows of one group), in one launch.
 // Y = B_j H_jj comes from a block product.  CTAs [0, n_kc): one warp per group, lane l takes columns l, l + 32, ..;
 // the remaining CTAs compute alpha.

@@ -891,8 +891,6 @@ bool make_map_e(CUtensorMap* map, const void* base, int64_t rows) {
 
 }  // namespace
 
-int g_sparse_pairs = 1;   // 0: the one-CTA kernel only (tests compare the two)
-
 bool tc_sparse_ok(const armor_ctx* c) {
   return c->cfg.n_keep == 2 && c->cfg.m_group == 4 && c->d_out % 128 == 0 && c->d_in % 128 == 0 &&
          c->cfg.precision != ARMOR_PREC_SIMT;
@@ -939,7 +937,7 @@ armor_status launch_tc_sparse(armor_ctx* c, const void* Sc, const void* E, const
   p.status = c->status;
   const int n_sm = c->n_sm;
   KTimer kt(c, ARMOR_KC_GEMM, 2.0 * (double)p.M * (double)p.N * (double)p.K, s);   // dense-equivalent flops
-  if (g_sparse_pairs && c->d_out % 256 == 0 && n_sm >= 2) {
+  if (c->d_out % 256 == 0 && n_sm >= 2) {
     // Two row tiles at a time, or one: rounds of the pairs times what a tile takes, its tokens plus, with two, 200 tokens' worth (a tile
     // of 512 x 224 takes 1.62 times one of 256 x 256, of 512 x 192 1.48 times), 240 with the output in fp32: 14336 x 2048, 1,459 tokens, 3
     // rounds of two or 5 of one, 149 us and 144 a forward with fp32 wrappers.  Whole forwards, one and two: 28672 x 8192, 4,096 tokens

@@ -77,6 +77,12 @@ __device__ __forceinline__ void tma_load_mn(uint32_t dst, const CUtensorMap* map
   }
 }
 
+// x - trunc_tf32(x)
+__device__ __forceinline__ float4 low4(const float4 v) {
+  return make_float4(v.x - __uint_as_float(__float_as_uint(v.x) & 0xffffe000u), v.y - __uint_as_float(__float_as_uint(v.y) & 0xffffe000u),
+                     v.z - __uint_as_float(__float_as_uint(v.z) & 0xffffe000u), v.w - __uint_as_float(__float_as_uint(v.w) & 0xffffe000u));
+}
+
 // shared -> global tile store (bulk group completion)
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int c0, int c1, uint32_t src) {
   asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"

@@ -638,7 +638,7 @@ def test_packed_layer_forward_with_d_block_256():
     Hd = dev(H32)
     st = ctx.init(dev(W), Hd)
     ctx.bcd_step(st, Hd, 0, 2, want_stats=False)
-    xb = dev(inputs.make_tokens(BIG_BLOCK, 1000)).to(torch.bfloat16)     # two chunks of 512 tokens, the second ragged
+    xb = dev(inputs.make_tokens(BIG_BLOCK, 1000)).to(torch.bfloat16)     # more tokens than rows or columns, ragged
     A, B, S = (host(t).astype(np.float64) for t in (st.A, st.B, st.S))
     r1, r2 = host(st.r1).astype(np.float64), host(st.r2).astype(np.float64)
     yo = O.apply(A, B, S, xb.float().cpu().numpy(), r1, r2)
