@@ -81,14 +81,40 @@ def test_few_token_forward_equals_the_large_batch(d_out, d_in, d_block):
     st = Bd.LayerState(Wbar=S, A=ints(-1, 1, d_out // d_block, d_block, d_block), B=ints(-1, 1, d_in // d_block, d_block, d_block),
                        S=S, M=M)
     packed = ctx.pack_layer(st)
-    x = ints(-1, 1, 300, d_in).to(torch.bfloat16)
+    x = ints(-1, 1, 2100, d_in).to(torch.bfloat16)                     # (more than 2,048 tokens: the persistent kernels whatever the size)
     big = ctx.apply_layer(packed, x)
-    z1 = torch.einsum("tjk,jmk->tjm", x.float().view(300, -1, d_block), st.B).reshape(300, d_in).to(torch.bfloat16)
+    z1 = torch.einsum("tjk,jmk->tjm", x.float().view(2100, -1, d_block), st.B).reshape(2100, d_in).to(torch.bfloat16)
     z2 = (z1.double() @ S.double().t()).to(torch.bfloat16)
-    y = torch.einsum("tjk,jmk->tjm", z2.double().view(300, -1, d_block), st.A.double()).reshape(300, d_out).float().to(torch.bfloat16)
+    y = torch.einsum("tjk,jmk->tjm", z2.double().view(2100, -1, d_block), st.A.double()).reshape(2100, d_out).float().to(torch.bfloat16)
     assert torch.equal(big, y)
-    for n in (1, 15, 16, 17, 32, 33, 63, 64, 65, 127, 128, 129):
+    for n in (1, 15, 16, 17, 24, 25, 32, 33, 63, 64, 65, 127, 128, 129, 300):
         assert torch.equal(ctx.apply_layer(packed, x[:n].contiguous()), big[:n]), n
+    assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
+
+
+@pytest.mark.parametrize("d_out,d_in,d_block", [(512, 2048, 128), (4096, 2048, 128), (5120, 1024, 128), (1024, 2048, 256)])
+def test_few_token_forward_of_real_numbers_against_fp64(d_out, d_in, d_block):
+    """The sums of the packed forward are fp32 however the core's contraction is cut, and z1, z2 and y are rounded to bf16 once.  At most 64
+    truncating additions put a sum off by 64 * 2^-24 of itself, so that at most 2 * 64 * 2^-24 / 2^-8 = 2e-3 of the values
+    are rounded the other way, by 2^-7 of themselves at most: sqrt(3 * 2e-3) * 2^-7 = 6e-4 in the norm after three roundings.  (Pieces rounded
+    to bf16 before they are added: 1.1e-3 and more.)"""
+    from paper_2510_05528_b200 import binding as Bd
+    g = _gen(d_out + d_in + d_block)
+    ctx = _ctx(d_out, d_in, d_block)
+    W = torch.randn(d_out, d_in // 4, 4, device=DEV, generator=g)
+    keep = torch.zeros_like(W, dtype=torch.bool).scatter_(2, W.abs().topk(2, dim=2).indices, True)
+    S = (W * keep).view(d_out, d_in)
+    M = (keep * torch.tensor([1, 2, 4, 8], device=DEV)).sum(2).to(torch.uint8)
+    A = torch.eye(d_block, device=DEV) + 0.3 / d_block ** 0.5 * torch.randn(d_out // d_block, d_block, d_block, device=DEV, generator=g)
+    B = torch.eye(d_block, device=DEV) + 0.3 / d_block ** 0.5 * torch.randn(d_in // d_block, d_block, d_block, device=DEV, generator=g)
+    packed = ctx.pack_layer(Bd.LayerState(Wbar=S, A=A, B=B, S=S, M=M))
+    A, B, S = (t.to(torch.bfloat16).double() for t in (A, B, S))
+    x = (torch.randn(2100, d_in, device=DEV, generator=g) * torch.exp(torch.randn(d_in, device=DEV, generator=g))).to(torch.bfloat16)
+    z1 = torch.einsum("tjk,jmk->tjm", x.double().view(2100, -1, d_block), B).reshape(2100, d_in).to(torch.bfloat16)
+    z2 = (z1.double() @ S.t()).to(torch.bfloat16)
+    y = torch.einsum("tjk,jmk->tjm", z2.double().view(2100, -1, d_block), A).reshape(2100, d_out).to(torch.bfloat16).double()
+    for n in (1, 16, 24, 25, 64, 128, 129, 300, 768, 2048, 2100):
+        assert (ctx.apply_layer(packed, x[:n].contiguous()).double() - y[:n]).norm() <= 6e-4 * y[:n].norm(), n
     assert ctx.device_status()[:5] == [0, 0, 0, 0, 0]
 
 
