@@ -722,6 +722,14 @@ def test_fp32_forward_of_a_core_with_one_group_that_is_not_2_of_4(d_out, d_in, d
     assert torch.equal(ctx.apply(st, x), torch.cat([ctx.apply(st, t) for t in x.split(2000)]))
     W[at, at, 3] = 0.0
     assert torch.equal(ctx.apply(st, x), sparse)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()                                       # which product runs is decided as the graph runs
+    with torch.cuda.graph(graph, stream=torch.cuda.Stream()):
+        y = ctx.apply(st, x)
+    for entry in (1.0, 0.0, 1.0):
+        W[at, at, 3] = entry
+        graph.replay()
+        assert torch.equal(y, ctx.apply(st, x)) and torch.equal(y, sparse) == (entry == 0.0)
     assert ctx.device_status()[:4] == [0, 0, 0, 0]
 
 
